@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import math
+import operator
 import os
 from dataclasses import dataclass
 from typing import Optional
@@ -102,6 +103,30 @@ class Params:
         return cp
 
 
+# A call's C struct depends on the parameter fields and the tensors' strides alone, so the structs of the last few
+# hundred distinct calls are kept: building one takes about 8 us of Python, as long as the kernels of a small call run,
+# finding it again 1 us.  The library only reads them.
+_FIELDS = operator.attrgetter("n_units", "n_q_heads", "n_kv_heads", "head_dim", "seq_len", "window", "n_keep", "dtype",
+                              "softmax_scale", "theta", "tau", "tau_mode", "flow_mode", "merge_mode", "keep_window", "path")
+_MAX_STRUCTS = 512
+_structs = {}
+
+
+def _keep_struct(key, cp):
+    if len(_structs) >= _MAX_STRUCTS:
+        _structs.clear()
+    _structs[key] = cp
+    return cp
+
+
+def _params(p: Params, q=None, k=None, v=None, ko=None, vo=None) -> _CParams:
+    """p.c(...), out of the kept structs where the same fields and strides have been seen."""
+    key = (_FIELDS(p), q is None or q.stride(), k is None or k.stride(), v is None or v.stride(), ko is None or ko.stride(),
+           vo is None or vo.stride())
+    cp = _structs.get(key)
+    return cp if cp is not None else _keep_struct(key, p.c(q=q, k=k, v=v, ko=ko, vo=vo))
+
+
 _lib = None
 
 
@@ -133,6 +158,15 @@ def load() -> ctypes.CDLL:
         lib.flowmm_decode_attention.restype = ctypes.c_int
         lib.flowmm_full_flow_workspace_bytes.restype = ctypes.c_int
         lib.flowmm_full_flow.restype = ctypes.c_int
+        # device pointers, the workspace size and the stream go in as plain integers (None: NULL)
+        P, N = ctypes.c_void_p, ctypes.c_size_t
+        for name, types in (("flowmm_score", [P] * 7 + [N, P]), ("flowmm_layer_flow", [P] * 5), ("flowmm_select", [P] * 5 + [N, P]),
+                            ("flowmm_match", [P] * 10 + [N, P]), ("flowmm_merge", [P] * 10 + [N, P]), ("flowmm_merge_static", [P] * 10),
+                            ("flowmm_compress_layer", [P] * 15 + [N, P]), ("flowmm_recompress", [P] * 16 + [N, P]),
+                            ("flowmm_full_flow", [P] * 9 + [N, P]), ("flowmm_decode_attention", [P] * 6 + [N, P]),
+                            ("flowmm_last_device_status", [P] * 2), ("flowmm_selftest_wait_timeout", [P] * 2),
+                            ("flowmm_merge_static_status", [P]), ("flowmm_merge_static_poke_status", [ctypes.c_int32, P])):
+            getattr(lib, name).argtypes = types
         _lib = lib
     return _lib
 
@@ -146,16 +180,17 @@ def _check(code: int, where: str):
         raise FlowmmError(code, where)
 
 
-def _p(t: Optional[torch.Tensor]):
+def _p(t: Optional[torch.Tensor]) -> Optional[int]:
     if t is None:
-        return ctypes.c_void_p(0)
+        return None
     if not t.is_cuda:
         raise ValueError("flowmm takes CUDA tensors")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+def _stream() -> int:
+    """The current stream's handle, without the Stream object around it (3 us of Python)."""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def torch_dtype(code: int):
@@ -177,9 +212,9 @@ def alloc_workspace(p: Params, device="cuda") -> torch.Tensor:
 
 
 def flowmm_score(p: Params, q_win, k, modality, importance, cross_mass, ws):
-    cp = p.c(q=q_win, k=k)
+    cp = _params(p, q=q_win, k=k)
     _check(load().flowmm_score(ctypes.byref(cp), _p(q_win), _p(k), _p(modality), _p(importance), _p(cross_mass),
-                               _p(ws), ctypes.c_size_t(ws.numel()), _stream()), "flowmm_score")
+                               _p(ws), ws.numel(), _stream()), "flowmm_score")
 
 
 def flowmm_full_flow_workspace_bytes(p: Params) -> int:
@@ -193,42 +228,42 @@ def flowmm_full_flow(p: Params, q_full, k, modality, cross_mass, rho, strategy, 
     """Eq. 6 and Eq. 7 over every query row of the prefill: q_full [units, q_heads, seq_len, head_dim]."""
     if q_full.dim() != 4 or q_full.stride(3) != 1:
         raise ValueError("expected a [units, heads, tokens, head_dim] tensor with contiguous head_dim")
-    cp = p.c(k=k)
+    cp = _params(p, k=k)
     qs = (ctypes.c_int64 * 3)(q_full.stride(0), q_full.stride(1), q_full.stride(2))
-    _check(load().flowmm_full_flow(ctypes.byref(cp), _p(q_full), qs, _p(k), _p(modality), _p(cross_mass), _p(rho),
-                                   _p(strategy), _p(ws), ctypes.c_size_t(ws.numel()), _stream()), "flowmm_full_flow")
+    _check(load().flowmm_full_flow(ctypes.byref(cp), _p(q_full), ctypes.byref(qs), _p(k), _p(modality), _p(cross_mass), _p(rho),
+                                   _p(strategy), _p(ws), ws.numel(), _stream()), "flowmm_full_flow")
 
 
 def flowmm_layer_flow(p: Params, cross_mass, rho, strategy):
-    cp = p.c()
+    cp = _params(p)
     _check(load().flowmm_layer_flow(ctypes.byref(cp), _p(cross_mass), _p(rho), _p(strategy), _stream()),
            "flowmm_layer_flow")
 
 
 def flowmm_select(p: Params, importance, retained_idx, evicted_idx, ws):
-    cp = p.c()
+    cp = _params(p)
     _check(load().flowmm_select(ctypes.byref(cp), _p(importance), _p(retained_idx), _p(evicted_idx), _p(ws),
-                                ctypes.c_size_t(ws.numel()), _stream()), "flowmm_select")
+                                ws.numel(), _stream()), "flowmm_select")
 
 
 def flowmm_match(p: Params, k, importance, modality, retained_idx, evicted_idx, strategy, match, match_sim, ws):
-    cp = p.c(k=k)
+    cp = _params(p, k=k)
     _check(load().flowmm_match(ctypes.byref(cp), _p(k), _p(importance), _p(modality), _p(retained_idx),
                                _p(evicted_idx), _p(strategy), _p(match), _p(match_sim), _p(ws),
-                               ctypes.c_size_t(ws.numel()), _stream()), "flowmm_match")
+                               ws.numel(), _stream()), "flowmm_match")
 
 
 def flowmm_merge(p: Params, k, v, retained_idx, evicted_idx, match, match_sim, k_out, v_out, ws):
-    cp = p.c(k=k, v=v, ko=k_out, vo=v_out)
+    cp = _params(p, k=k, v=v, ko=k_out, vo=v_out)
     _check(load().flowmm_merge(ctypes.byref(cp), _p(k), _p(v), _p(retained_idx), _p(evicted_idx), _p(match),
-                               _p(match_sim), _p(k_out), _p(v_out), _p(ws), ctypes.c_size_t(ws.numel()), _stream()),
+                               _p(match_sim), _p(k_out), _p(v_out), _p(ws), ws.numel(), _stream()),
            "flowmm_merge")
 
 
 def flowmm_merge_static(p: Params, k, v, retained_idx, evicted_idx, match, match_sim, k_out, v_out):
     """flowmm_merge for callers that cannot allocate: no workspace argument, the scratch is a
     fixed array inside the library (see include/flowmm.h for its size limit and sharing rules)."""
-    cp = p.c(k=k, v=v, ko=k_out, vo=v_out)
+    cp = _params(p, k=k, v=v, ko=k_out, vo=v_out)
     _check(load().flowmm_merge_static(ctypes.byref(cp), _p(k), _p(v), _p(retained_idx), _p(evicted_idx), _p(match),
                                       _p(match_sim), _p(k_out), _p(v_out), _stream()), "flowmm_merge_static")
 
@@ -239,16 +274,16 @@ def flowmm_merge_static_status() -> int:
 
 
 def flowmm_merge_static_poke_status(word: int):
-    _check(load().flowmm_merge_static_poke_status(ctypes.c_int32(word), _stream()), "flowmm_merge_static_poke_status")
+    _check(load().flowmm_merge_static_poke_status(word, _stream()), "flowmm_merge_static_poke_status")
 
 
 def flowmm_compress_layer(p: Params, q_win, k, v, modality, k_out, v_out, ws, importance=None, rho=None,
                           strategy=None, retained_idx=None, evicted_idx=None, match=None, match_sim=None):
-    cp = p.c(q=q_win, k=k, v=v, ko=k_out, vo=v_out)
+    cp = _params(p, q=q_win, k=k, v=v, ko=k_out, vo=v_out)
     _check(load().flowmm_compress_layer(ctypes.byref(cp), _p(q_win), _p(k), _p(v), _p(modality), _p(k_out),
                                         _p(v_out), _p(importance), _p(rho), _p(strategy), _p(retained_idx),
                                         _p(evicted_idx), _p(match), _p(match_sim), _p(ws),
-                                        ctypes.c_size_t(ws.numel()), _stream()), "flowmm_compress_layer")
+                                        ws.numel(), _stream()), "flowmm_compress_layer")
 
 
 def flowmm_recompress_workspace_bytes(p: Params) -> int:
@@ -262,11 +297,11 @@ def flowmm_recompress(p: Params, q_win, k_cache, v_cache, row_modality, k_out, v
                       importance=None, rho=None, strategy=None, retained_idx=None, evicted_idx=None, match=None,
                       match_sim=None):
     """Section 3.3 again on a cache that grew during decoding; row_modality [units, kv_heads, rows] uint8."""
-    cp = p.c(q=q_win, k=k_cache, v=v_cache, ko=k_out, vo=v_out)
+    cp = _params(p, q=q_win, k=k_cache, v=v_cache, ko=k_out, vo=v_out)
     _check(load().flowmm_recompress(ctypes.byref(cp), _p(q_win), _p(k_cache), _p(v_cache), _p(row_modality), _p(k_out),
                                     _p(v_out), _p(row_modality_out), _p(importance), _p(rho), _p(strategy),
                                     _p(retained_idx), _p(evicted_idx), _p(match), _p(match_sim), _p(ws),
-                                    ctypes.c_size_t(ws.numel()), _stream()), "flowmm_recompress")
+                                    ws.numel(), _stream()), "flowmm_recompress")
 
 
 def flowmm_last_device_status(ws) -> int:
@@ -283,6 +318,10 @@ class _CDecodeParams(ctypes.Structure):
 
 
 def _decode_params(q, k, v, softmax_scale: float, path: int) -> _CDecodeParams:
+    key = (q.shape, q.stride(), q.dtype, k.shape, k.stride(), v.shape, v.stride(), softmax_scale, path)
+    cp = _structs.get(key)
+    if cp is not None:
+        return cp
     if q.dim() != 3 or not q.is_contiguous():
         raise ValueError("q must be a contiguous [units, q_heads, head_dim] tensor")
     if k.dim() != 4 or v.dim() != 4 or k.stride(3) != 1 or v.stride(3) != 1 or k.shape != v.shape:
@@ -291,7 +330,7 @@ def _decode_params(q, k, v, softmax_scale: float, path: int) -> _CDecodeParams:
     cp = _CDecodeParams(q.shape[0], q.shape[1], k.shape[1], q.shape[2], k.shape[2], dtype, softmax_scale, path)
     cp.k_stride = (ctypes.c_int64 * 3)(k.stride(0), k.stride(1), k.stride(2))
     cp.v_stride = (ctypes.c_int64 * 3)(v.stride(0), v.stride(1), v.stride(2))
-    return cp
+    return _keep_struct(key, cp)
 
 
 def flowmm_decode_workspace_bytes(q, k, v, softmax_scale: float = 0.0, path: int = PATH_AUTO) -> int:
@@ -305,7 +344,7 @@ def flowmm_decode_attention(q, k, v, out, ws, softmax_scale: float = 0.0, path: 
     """Eq. 4 for one new query per head over the cache rows of k, v; out [units, q_heads, head_dim] float32."""
     cp = _decode_params(q, k, v, softmax_scale, path)
     _check(load().flowmm_decode_attention(ctypes.byref(cp), _p(q), _p(k), _p(v), _p(out), _p(ws),
-                                          ctypes.c_size_t(ws.numel()), _stream()), "flowmm_decode_attention")
+                                          ws.numel(), _stream()), "flowmm_decode_attention")
 
 
 def flowmm_selftest_wait_timeout(ws):

@@ -32,6 +32,7 @@ template <typename T, int D, int GP>
 __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const DecodeArgs A) {
     constexpr int V = Elem<T>::kVec, LPR = D / V, GROUPS = kDecThreads / LPR;
     extern __shared__ float dec_smem[];                              // [GROUPS][GP][D + 2]
+    predecessor_done();
     const int tid = threadIdx.x, sub = tid % LPR, grp = tid / LPR;
     const int uh = blockIdx.x, u = uh / A.Hkv, h = uh % A.Hkv;
     const int lo = blockIdx.y * A.keys_per_split, hi = min(A.N, lo + A.keys_per_split);
@@ -137,6 +138,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const Decod
 // grid = U*Hq, block = D: joins the key ranges of one query head and normalises.
 template <int D>
 __global__ void __launch_bounds__(D) decode_combine_kernel(const DecodeArgs A) {
+    predecessor_done();
     const int ug = blockIdx.x, u = ug / A.Hq, gq = ug % A.Hq, h = gq / A.G, g = gq % A.G, d = threadIdx.x;
     const int uh = u * A.Hkv + h;
     float mx = kNegBig;

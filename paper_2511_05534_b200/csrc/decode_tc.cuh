@@ -102,6 +102,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    predecessor_done();
 
     const int uh = blockIdx.x, u = uh / A.Hkv, h = uh % A.Hkv, split = blockIdx.y;
     const int tiles_total = (A.N + kTile - 1) / kTile;

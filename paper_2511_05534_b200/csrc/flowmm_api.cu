@@ -49,6 +49,21 @@ inline void profile_mark(const char *name, cudaStream_t st) {
     }
 }
 
+// Launches a kernel as a programmatic dependent of the one before it in the stream: its blocks are set up while that
+// kernel drains, and predecessor_done() in the kernel holds them back from the data (common.cuh).  A launch boundary
+// costs 2 us less than with a plain launch (13 launches of a re-compression: 163 to 135 us) and the host no more.  An
+// error stays in cudaGetLastError() for FLOWMM_LAUNCHED.
+template <typename... Params, typename... Args>
+void launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 #define FLOWMM_LAUNCHED(name)                                          \
     do {                                                               \
         ++g_launches;                                                  \
@@ -225,6 +240,7 @@ float tau_effective(const flowmm_params &p) {
 // One block per (unit, head): pivots and non-pivots inside [0, L) and strictly ascending, matches inside [-1, B).
 __global__ void debug_check_lists_kernel(const int32_t *retained, const int32_t *evicted, const int32_t *match,
                                          int L, int B, int E, int *status) {
+    predecessor_done();
     const int uh = blockIdx.x;
     bool bad = false;
     if (retained)
@@ -248,7 +264,7 @@ __global__ void debug_check_lists_kernel(const int32_t *retained, const int32_t 
 // Runs the check, waits for it and reports: the entry point launches nothing else when a list is bad.
 flowmm_status debug_check_lists(const flowmm_params &p, const int32_t *retained, const int32_t *evicted,
                                 const int32_t *match, int *status, cudaStream_t st) {
-    debug_check_lists_kernel<<<p.n_units * p.n_kv_heads, 256, 0, st>>>(retained, evicted, match, p.seq_len, p.n_keep,
+    launch(debug_check_lists_kernel, p.n_units * p.n_kv_heads, 256, 0, st, retained, evicted, match, p.seq_len, p.n_keep,
                                                                         p.seq_len - p.n_keep, status);
     if (cudaGetLastError() != cudaSuccess) return FLOWMM_ERR_CUDA;
     int32_t word = 0;
@@ -308,19 +324,19 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
                              (int)tcs::Small::kSmemBytes) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
     const int sms = tc::sm_count();
-    score_stats_tc_kernel<tcs::Big><<<a.n_items1 < sms ? a.n_items1 : sms, tcs::kThreads, tcs::Big::kSmemBytes, st>>>(qa, k256, a);
+    launch(score_stats_tc_kernel<tcs::Big>, a.n_items1 < sms ? a.n_items1 : sms, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
     FLOWMM_LAUNCHED("score_stats_tc");
     const int n_negc = UH * a.GWpad;
-    score_combine_kernel<<<(n_negc + 255) / 256, 256, 0, st>>>(a.row_part, 4 * a.n_chunk, a.GW, a.GWpad, UH, a.negc);
+    launch(score_combine_kernel, (n_negc + 255) / 256, 256, 0, st, a.row_part, 4 * a.n_chunk, a.GW, a.GWpad, UH, a.negc);
     FLOWMM_LAUNCHED("score_combine");
     if (small2)
-        score_colsum_tc_kernel<tcs::Small><<<a.n_items2 < sms ? a.n_items2 : sms, tcs::kThreads, tcs::Small::kSmemBytes, st>>>(k128, qb, a);
+        launch(score_colsum_tc_kernel<tcs::Small>, a.n_items2 < sms ? a.n_items2 : sms, tcs::kThreads, tcs::Small::kSmemBytes, st, k128, qb, a);
     else
-        score_colsum_tc_kernel<tcs::Big><<<a.n_items2 < sms ? a.n_items2 : sms, tcs::kThreads, tcs::Big::kSmemBytes, st>>>(k128, qb, a);
+        launch(score_colsum_tc_kernel<tcs::Big>, a.n_items2 < sms ? a.n_items2 : sms, tcs::kThreads, tcs::Big::kSmemBytes, st, k128, qb, a);
     FLOWMM_LAUNCHED("score_colsum_tc");
     if (parts_out) { *parts_out = a.n_rt * 8; return FLOWMM_OK; }     // the caller reduces the partial masses itself
     const int n = p.n_units * p.n_q_heads;
-    cross_mass_reduce<<<(n + 7) / 8, 256, 0, st>>>(a.cross_part, a.n_rt * 8, n, cross_mass);
+    launch(cross_mass_reduce, (n + 7) / 8, 256, 0, st, a.cross_part, a.n_rt * 8, n, cross_mass);
     FLOWMM_LAUNCHED("cross_mass_reduce");
     return FLOWMM_OK;
 }
@@ -350,7 +366,7 @@ flowmm_status run_score_fused(const flowmm_params &p, const Layout &y, const voi
                              (int)sft::kSmemBytes) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
     const int grid = UH < tc::sm_count() ? UH : tc::sm_count();
-    sft::score_fused_tc_kernel<<<grid, sft::kThreads, sft::kSmemBytes, st>>>(qmap, kmap, a);
+    launch(sft::score_fused_tc_kernel, grid, sft::kThreads, sft::kSmemBytes, st, qmap, kmap, a);
     FLOWMM_LAUNCHED("score_fused_tc");
     return FLOWMM_OK;
 }
@@ -378,26 +394,26 @@ flowmm_status run_score(const flowmm_params &p, const Layout &y, const void *q, 
     const dim3 g1(UH, (GW + kTile - 1) / kTile, y.n_chunk1), g2(UH, y.n_chunk2);
     const size_t dyn = (size_t)3 * GW * sizeof(float);
     if (p.dtype == FLOWMM_BF16) {
-        score_stats_simt<__nv_bfloat16><<<g1, kSimtThreads, 0, st>>>(a);
+        launch(score_stats_simt<__nv_bfloat16>, g1, kSimtThreads, 0, st, a);
         FLOWMM_LAUNCHED("score_stats_simt");
-        score_colsum_simt<__nv_bfloat16><<<g2, kSimtThreads, dyn, st>>>(a);
+        launch(score_colsum_simt<__nv_bfloat16>, g2, kSimtThreads, dyn, st, a);
         FLOWMM_LAUNCHED("score_colsum_simt");
     } else {
-        score_stats_simt<float><<<g1, kSimtThreads, 0, st>>>(a);
+        launch(score_stats_simt<float>, g1, kSimtThreads, 0, st, a);
         FLOWMM_LAUNCHED("score_stats_simt");
-        score_colsum_simt<float><<<g2, kSimtThreads, dyn, st>>>(a);
+        launch(score_colsum_simt<float>, g2, kSimtThreads, dyn, st, a);
         FLOWMM_LAUNCHED("score_colsum_simt");
     }
     if (parts_out) { *parts_out = y.n_chunk2; return FLOWMM_OK; }
     const int n = p.n_units * p.n_q_heads;
-    cross_mass_reduce<<<(n + 7) / 8, 256, 0, st>>>(a.cross_part, y.n_chunk2, n, cross_mass);
+    launch(cross_mass_reduce, (n + 7) / 8, 256, 0, st, a.cross_part, y.n_chunk2, n, cross_mass);
     FLOWMM_LAUNCHED("cross_mass_reduce");
     return FLOWMM_OK;
 }
 
 flowmm_status run_layer_flow(const flowmm_params &p, const float *cross_mass, float *rho, int32_t *strategy,
                              cudaStream_t st) {
-    layer_flow_kernel<<<(p.n_units + 127) / 128, 128, 0, st>>>(cross_mass, p.n_units, p.n_q_heads, p.window, p.theta,
+    launch(layer_flow_kernel, (p.n_units + 127) / 128, 128, 0, st, cross_mass, p.n_units, p.n_q_heads, p.window, p.theta,
                                                                 p.flow_mode, rho, strategy);
     FLOWMM_LAUNCHED("layer_flow");
     return FLOWMM_OK;
@@ -432,7 +448,7 @@ flowmm_status run_select(const flowmm_params &p, const float *importance, int32_
     f.cross_part = cross_part; f.n_parts = n_parts; f.cross_mass = cross_mass; f.rho = rho; f.strategy = strategy; f.Hq = p.n_q_heads; f.Hkv = p.n_kv_heads;
     f.theta = p.theta; f.flow_mode = p.flow_mode;
     MatchPrepArgs none = {};
-    select_topb_kernel<<<p.n_units * p.n_kv_heads, threads, 0, st>>>(importance, p.seq_len, p.n_keep, p.window,
+    launch(select_topb_kernel, p.n_units * p.n_kv_heads, threads, 0, st, importance, p.seq_len, p.n_keep, p.window,
                                                                            p.keep_window, retained, evicted, f,
                                                                            prep ? *prep : none, prep ? 1 : 0);
     FLOWMM_LAUNCHED("select_topb");
@@ -449,11 +465,11 @@ flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *
     if (!prepared) {                                 // (the fused call's selection launch has done it already)
         // few heads: a head's lists are walked by more threads, the GPU is not full either way
         const int prep_threads = UH >= 4 * tc::sm_count() ? 256 : UH >= 2 * tc::sm_count() ? 512 : 1024;
-        match_prepare_kernel<<<UH, prep_threads, 0, st>>>(g);
+        launch(match_prepare_kernel, UH, prep_threads, 0, st, g);
         FLOWMM_LAUNCHED("match_prepare");
     }
     if (!g.copy_here) {
-        match_gather_kernel<<<dim3(UH, (y.c_tot + 63) / 64), 256, 0, st>>>(g);
+        launch(match_gather_kernel, dim3(UH, (y.c_tot + 63) / 64), 256, 0, st, g);
         FLOWMM_LAUNCHED("match_gather");
     }
 
@@ -475,7 +491,7 @@ flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *
         if (cudaFuncSetAttribute(mst::match_small_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)mst::kSmemBytes) != cudaSuccess)
             return FLOWMM_ERR_CUDA;
-        mst::match_small_tc_kernel<<<UH < tc::sm_count() ? UH : tc::sm_count(), mst::kThreads, mst::kSmemBytes, st>>>(k_map, cand_map, a);
+        launch(mst::match_small_tc_kernel, UH < tc::sm_count() ? UH : tc::sm_count(), mst::kThreads, mst::kSmemBytes, st, k_map, cand_map, a);
         FLOWMM_LAUNCHED("match_small_tc");
         return FLOWMM_OK;
     }
@@ -497,8 +513,8 @@ flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *
                              (int)tcs::Small::kSmemBytes) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
     const int grid = a.n_items < tc::sm_count() ? a.n_items : tc::sm_count();
-    if (small) match_tc_kernel<tcs::Small><<<grid, tcs::kThreads, tcs::Small::kSmemBytes, st>>>(k_map, cand_map, a);
-    else match_tc_kernel<tcs::Big><<<grid, tcs::kThreads, tcs::Big::kSmemBytes, st>>>(k_map, cand_map, a);
+    if (small) launch(match_tc_kernel<tcs::Small>, grid, tcs::kThreads, tcs::Small::kSmemBytes, st, k_map, cand_map, a);
+    else launch(match_tc_kernel<tcs::Big>, grid, tcs::kThreads, tcs::Big::kSmemBytes, st, k_map, cand_map, a);
     FLOWMM_LAUNCHED("match_tc");
     return FLOWMM_OK;
 }
@@ -517,10 +533,10 @@ flowmm_status run_match(const flowmm_params &p, const Layout &y, const void *k, 
     const int64_t threads = rows * lanes;
     const unsigned blocks = (unsigned)((threads + 255) / 256);
     if (p.dtype == FLOWMM_BF16)
-        inv_norm_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(k, rows, p.n_kv_heads, p.seq_len, p.head_dim,
+        launch(inv_norm_kernel<__nv_bfloat16>, blocks, 256, 0, st, k, rows, p.n_kv_heads, p.seq_len, p.head_dim,
                                                                p.k_stride[0], p.k_stride[1], p.k_stride[2], rn);
     else
-        inv_norm_kernel<float><<<blocks, 256, 0, st>>>(k, rows, p.n_kv_heads, p.seq_len, p.head_dim, p.k_stride[0],
+        launch(inv_norm_kernel<float>, blocks, 256, 0, st, k, rows, p.n_kv_heads, p.seq_len, p.head_dim, p.k_stride[0],
                                                        p.k_stride[1], p.k_stride[2], rn);
     FLOWMM_LAUNCHED("inv_norm");
     MatchArgs a;
@@ -530,8 +546,8 @@ flowmm_status run_match(const flowmm_params &p, const Layout &y, const void *k, 
     a.tau_eff = tau_effective(p);
     for (int i = 0; i < 3; ++i) a.ks[i] = p.k_stride[i];
     const dim3 grid(p.n_units * p.n_kv_heads, (E + kTile - 1) / kTile);
-    if (p.dtype == FLOWMM_BF16) match_simt<__nv_bfloat16><<<grid, kSimtThreads, 0, st>>>(a);
-    else match_simt<float><<<grid, kSimtThreads, 0, st>>>(a);
+    if (p.dtype == FLOWMM_BF16) launch(match_simt<__nv_bfloat16>, grid, kSimtThreads, 0, st, a);
+    else launch(match_simt<float>, grid, kSimtThreads, 0, st, a);
     FLOWMM_LAUNCHED("match_simt");
     return FLOWMM_OK;
 }
@@ -564,7 +580,7 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         ma.tokmap = at<int2>(ws, y.tokmap); ma.L = p.seq_len; ma.B = p.n_keep; ma.E = E; ma.merge_mode = p.merge_mode;
         const int longest = E > p.n_keep ? E : p.n_keep;
         if (!map_ready) {
-            mtc::merge_map_kernel<<<dim3(UH, (longest + 255) / 256), 256, 0, st>>>(ma);
+            launch(mtc::merge_map_kernel, dim3(UH, (longest + 255) / 256), 256, 0, st, ma);
             FLOWMM_LAUNCHED("merge_map");
         }
         CUtensorMap kmap, vmap;
@@ -582,7 +598,7 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         if (cudaFuncSetAttribute(mtc::merge_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return FLOWMM_ERR_CUDA;
         const int grid = UH < tc::sm_count() ? UH : tc::sm_count();
-        mtc::merge_tc_kernel<<<grid, mtc::kThreads, smem, st>>>(kmap, vmap, a);
+        launch(mtc::merge_tc_kernel, grid, mtc::kThreads, smem, st, kmap, vmap, a);
         FLOWMM_LAUNCHED("merge_tc");
         return FLOWMM_OK;
     }
@@ -600,13 +616,13 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         if (staged) {
             if (E <= 4096) {
                 if (cudaFuncSetAttribute(build_csr_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csr_smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
-                build_csr_kernel<8, true><<<UH, 256, csr_smem, st>>>(c);
+                launch(build_csr_kernel<8, true>, UH, 256, csr_smem, st, c);
             } else {
                 if (cudaFuncSetAttribute(build_csr_kernel<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csr_smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
-                build_csr_kernel<32, true><<<UH, 1024, csr_smem, st>>>(c);
+                launch(build_csr_kernel<32, true>, UH, 1024, csr_smem, st, c);
             }
-        } else if (E <= 4096) build_csr_kernel<8, false><<<UH, 256, 0, st>>>(c);
-        else build_csr_kernel<32, false><<<UH, 1024, 0, st>>>(c);
+        } else if (E <= 4096) launch(build_csr_kernel<8, false>, UH, 256, 0, st, c);
+        else launch(build_csr_kernel<32, false>, UH, 1024, 0, st, c);
         FLOWMM_LAUNCHED("build_csr");
         m.mem_tok = c.mem_tok; m.mem_w = c.mem_w; m.piece_desc = c.piece_desc;
         m.piece_off = c.piece_off; m.part_off = c.part_off; m.ticket = c.ticket; m.slot_done = c.slot_done;
@@ -621,14 +637,14 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
                                  (int)mstg::kSmemBytes) != cudaSuccess)
             return FLOWMM_ERR_CUDA;
         const int gs = (int)(want_blocks < 3 * tc::sm_count() ? want_blocks : 3 * tc::sm_count());
-        mstg::merge_staged_kernel<__nv_bfloat16><<<gs, mstg::kThreads, mstg::kSmemBytes, st>>>(
+        launch(mstg::merge_staged_kernel<__nv_bfloat16>, gs, mstg::kThreads, mstg::kSmemBytes, st, 
             m, UH, at<int>(ws, y.merge_status), make_fastdiv((uint32_t)m.max_pieces), make_fastdiv((uint32_t)p.n_kv_heads));
         FLOWMM_LAUNCHED("merge_staged");
     } else if (p.dtype == FLOWMM_BF16) {
-        merge_pieces_kernel<__nv_bfloat16><<<gp, 256, 0, st>>>(m, UH);
+        launch(merge_pieces_kernel<__nv_bfloat16>, gp, 256, 0, st, m, UH);
         FLOWMM_LAUNCHED("merge_pieces");
     } else {
-        merge_pieces_kernel<float><<<gp, 256, 0, st>>>(m, UH);
+        launch(merge_pieces_kernel<float>, gp, 256, 0, st, m, UH);
         FLOWMM_LAUNCHED("merge_pieces");
     }
     return FLOWMM_OK;
@@ -871,10 +887,10 @@ flowmm_status run_flow_tile_tc(const flowmm_params &tp, const Layout &y, const v
                              (int)tcs::Big::kSmemBytes) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
     const int sms = tc::sm_count();
-    score_stats_tc_kernel<tcs::Big, true><<<a.n_items1 < sms ? a.n_items1 : sms, tcs::kThreads, tcs::Big::kSmemBytes, st>>>(qa, k256, a);
+    launch(score_stats_tc_kernel<tcs::Big, true>, a.n_items1 < sms ? a.n_items1 : sms, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
     FLOWMM_LAUNCHED("flow_stats_tc");
     const int n_heads = tp.n_units * tp.n_q_heads;
-    flow_combine_kernel<<<(n_heads + 7) / 8, 256, 0, st>>>(a.row_part, a.row_cross, 4 * a.n_chunk, G, W, tp.n_kv_heads, n_heads, cross_out);
+    launch(flow_combine_kernel, (n_heads + 7) / 8, 256, 0, st, a.row_part, a.row_cross, 4 * a.n_chunk, G, W, tp.n_kv_heads, n_heads, cross_out);
     FLOWMM_LAUNCHED("flow_combine");
     return FLOWMM_OK;
 }
@@ -935,7 +951,7 @@ extern "C" flowmm_status flowmm_full_flow(const flowmm_params *p, const void *q_
     uint32_t *bits = at<uint32_t>(ws, f.bits);
     const int mod_words = (p->seq_len + 31) / 32 + 8;                  // + slack: whole 256-key tiles are indexed
     if (use_tc(*p)) {
-        pack_modality_kernel<<<dim3(p->n_units, (mod_words + 7) / 8), 256, 0, st>>>(modality, p->seq_len, mod_words, bits);
+        launch(pack_modality_kernel, dim3(p->n_units, (mod_words + 7) / 8), 256, 0, st, modality, p->seq_len, mod_words, bits);
         FLOWMM_LAUNCHED("pack_modality");
     }
     for (int t = 0; t < n_tiles; ++t) {
@@ -955,7 +971,7 @@ extern "C" flowmm_status flowmm_full_flow(const flowmm_params *p, const void *q_
         const char *q_tile = static_cast<const char *>(q_full) + (size_t)lo * (size_t)q_full_stride[2] * esize;
         FLOWMM_TRY(run_score(tp, y, q_tile, k, mod, imp, parts + (size_t)t * n, ws, st));
     }
-    full_flow_reduce_kernel<<<p->n_units, 64, 0, st>>>(parts, n_tiles, n, p->n_q_heads, p->seq_len, p->theta, p->flow_mode,
+    launch(full_flow_reduce_kernel, p->n_units, 64, 0, st, parts, n_tiles, n, p->n_q_heads, p->seq_len, p->theta, p->flow_mode,
                                                        cross_mass, rho, strategy);
     FLOWMM_LAUNCHED("full_flow_reduce");
     return FLOWMM_OK;
@@ -1024,13 +1040,13 @@ flowmm_status launch_decode(const DecodeArgs &a, int uh, int n_q, cudaStream_t s
     const int gp = a.G <= 1 ? 1 : a.G <= 2 ? 2 : a.G <= 4 ? 4 : 8;
     const size_t smem = (size_t)groups * gp * (D + 2) * sizeof(float);
     switch (gp) {
-        case 1: decode_partial_kernel<T, D, 1><<<grid, kDecThreads, smem, st>>>(a); break;
-        case 2: decode_partial_kernel<T, D, 2><<<grid, kDecThreads, smem, st>>>(a); break;
-        case 4: decode_partial_kernel<T, D, 4><<<grid, kDecThreads, smem, st>>>(a); break;
-        default: decode_partial_kernel<T, D, 8><<<grid, kDecThreads, smem, st>>>(a); break;
+        case 1: launch(decode_partial_kernel<T, D, 1>, grid, kDecThreads, smem, st, a); break;
+        case 2: launch(decode_partial_kernel<T, D, 2>, grid, kDecThreads, smem, st, a); break;
+        case 4: launch(decode_partial_kernel<T, D, 4>, grid, kDecThreads, smem, st, a); break;
+        default: launch(decode_partial_kernel<T, D, 8>, grid, kDecThreads, smem, st, a); break;
     }
     FLOWMM_LAUNCHED("decode_partial");
-    decode_combine_kernel<D><<<n_q, D, 0, st>>>(a);
+    launch(decode_combine_kernel<D>, n_q, D, 0, st, a);
     FLOWMM_LAUNCHED("decode_combine");
     return FLOWMM_OK;
 }
@@ -1054,7 +1070,7 @@ flowmm_status launch_decode_tc(const flowmm_decode_params &p, const DecodeArgs &
     t.tickets = status + 64;
     t.Hq = a.Hq; t.Hkv = a.Hkv; t.G = a.G; t.N = a.N; t.n_split = a.n_split; t.tiles_per_split = a.keys_per_split;
     t.scale_log2 = a.scale_log2;
-    dtc::decode_tc_kernel<<<dim3(uh, a.n_split), dtc::kThreads, dtc::kSmemBytes, st>>>(kmap, vmap, t);
+    launch(dtc::decode_tc_kernel, dim3(uh, a.n_split), dtc::kThreads, dtc::kSmemBytes, st, kmap, vmap, t);
     FLOWMM_LAUNCHED("decode_tc");
     return FLOWMM_OK;
 }
@@ -1101,6 +1117,7 @@ namespace {
 
 // strategy of a unit copied to each of its KV heads (the per-head problems below take one strategy each)
 __global__ void expand_strategy_kernel(const int32_t *strategy, int n_units, int n_kv_heads, int32_t *per_head) {
+    predecessor_done();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n_units * n_kv_heads) per_head[i] = strategy[i / n_kv_heads];
 }
@@ -1108,6 +1125,7 @@ __global__ void expand_strategy_kernel(const int32_t *strategy, int n_units, int
 // modality of the rows that were kept: out[uh, s] = row_modality[uh, retained[uh, s]]
 __global__ void gather_row_modality_kernel(const uint8_t *row_modality, const int32_t *retained, int64_t n, int L, int B,
                                            uint8_t *out) {
+    predecessor_done();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[i] = row_modality[(i / B) * L + retained[i]];
 }
@@ -1183,13 +1201,13 @@ extern "C" flowmm_status flowmm_recompress(const flowmm_params *p, const void *q
     // scoring per (unit, KV head) against that head's own row modalities; Eq. 6 over all query heads of the layer
     FLOWMM_TRY(run_score(ph, y, q_win, k_cache, row_modality, importance, cross_mass, ws, st));
     FLOWMM_TRY(run_layer_flow(*p, cross_mass, rho, strategy, st));
-    expand_strategy_kernel<<<(ph.n_units + 255) / 256, 256, 0, st>>>(strategy, p->n_units, p->n_kv_heads, strategy_h);
+    launch(expand_strategy_kernel, (ph.n_units + 255) / 256, 256, 0, st, strategy, p->n_units, p->n_kv_heads, strategy_h);
     FLOWMM_LAUNCHED("expand_strategy");
     FLOWMM_TRY(run_select(ph, importance, retained_idx, evicted_idx, st));
     FLOWMM_TRY(run_match(ph, y, k_cache, importance, row_modality, retained_idx, evicted_idx, strategy_h, match, match_sim, ws, st));
     FLOWMM_TRY(run_merge(ph, y, k_cache, v_cache, retained_idx, evicted_idx, match, match_sim, k_out, v_out, ws, st));
     const int64_t n = (int64_t)ph.n_units * p->n_keep;
-    gather_row_modality_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(row_modality, retained_idx, n, p->seq_len, p->n_keep,
+    launch(gather_row_modality_kernel, (unsigned)((n + 255) / 256), 256, 0, st, row_modality, retained_idx, n, p->seq_len, p->n_keep,
                                                                             row_modality_out);
     FLOWMM_LAUNCHED("gather_row_modality");
     return FLOWMM_OK;
@@ -1203,6 +1221,7 @@ namespace {
 __global__ void wait_timeout_selftest_kernel(int *status) {
     __shared__ __align__(8) unsigned long long bar;
     __shared__ int abort_flag;
+    predecessor_done();
     if (threadIdx.x == 0) {
         abort_flag = 0;
         tc::mbar_init(tc::smem_u32(&bar), 1);
@@ -1218,7 +1237,7 @@ extern "C" flowmm_status flowmm_selftest_wait_timeout(void *ws, void *cuda_strea
     if (!ws) return FLOWMM_ERR_NULL;
     FLOWMM_TRY(check_device());
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    wait_timeout_selftest_kernel<<<1, 64, 0, st>>>(static_cast<int *>(ws));
+    launch(wait_timeout_selftest_kernel, 1, 64, 0, st, static_cast<int *>(ws));
     FLOWMM_LAUNCHED("wait_timeout_selftest");
     return FLOWMM_OK;
 }

@@ -81,6 +81,7 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    predecessor_done();
 
     if (warp == 0) {
         if (lane == 0) {

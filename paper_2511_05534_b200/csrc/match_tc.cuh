@@ -129,12 +129,14 @@ __device__ __forceinline__ void match_prepare_head(const MatchPrepArgs &A, int u
 __global__ void __launch_bounds__(1024) match_prepare_kernel(const MatchPrepArgs A) {
     __shared__ int scratch[33];
     __shared__ int s_ntext;
+    predecessor_done();
     match_prepare_head(A, blockIdx.x, scratch, &s_ntext);
 }
 
 // The gather step of the preparation as a kernel of its own for long candidate lists, so that many
 // CTAs share a head's rows.  grid = (U*Hkv, ceil(Ctot / 64)), block = 256.
 __global__ void __launch_bounds__(256) match_gather_kernel(const MatchPrepArgs A) {
+    predecessor_done();
     const int lo = blockIdx.y * 64;
     match_gather_rows(A, blockIdx.x, lo, min(A.Ctot, lo + 64), threadIdx.x, blockDim.x);
 }

@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(kThreads, 3) merge_staged_kernel(const MergeAr
         tc::mbar_init_fence();
     }
     __syncthreads();
+    predecessor_done();
     const unsigned total = (unsigned)n_uh * (unsigned)A.max_pieces;
     const bool is_v = lane >= 16;                             // lanes 0-15: the K row, 16-31: the V row, 16 bytes each
     const int c0 = (lane & 15) * V;

@@ -67,6 +67,7 @@ struct MapArgs {
 
 // grid = (UH, ceil(max(E, B) / 256))
 __global__ void __launch_bounds__(256) merge_map_kernel(const MapArgs A) {
+    predecessor_done();
     const int uh = blockIdx.x, i = blockIdx.y * 256 + threadIdx.x;
     int2 *map = A.tokmap + (int64_t)uh * A.L;
     if (i < A.E) {
@@ -117,6 +118,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    predecessor_done();
     const int n_chunk = (A.L + kTile - 1) / kTile;
 
     if (warp == 0) {

@@ -95,6 +95,7 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    predecessor_done();
     const int nt = (A.L + kTile - 1) / kTile;
 
     if (warp == 0) {

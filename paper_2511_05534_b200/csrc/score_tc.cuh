@@ -197,6 +197,7 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
 __global__ void flow_combine_kernel(const float2 *row_part, const float *row_cross, int n_part, int G, int W, int Hkv, int n_heads,
                                     float *cross_mass) {
     const int head = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    predecessor_done();
     if (head >= n_heads) return;                                         // head = (u * Hkv + h) * G + g
     const int uh = head / G, g = head % G;
     float s = 0.f;
@@ -219,6 +220,7 @@ __global__ void flow_combine_kernel(const float2 *row_part, const float *row_cro
 // Packs the modality map: word w of a unit holds keys 32 w .. 32 w + 31 (bit set = visual; keys past the prompt: 0).
 __global__ void pack_modality_kernel(const uint8_t *modality, int L, int n_words, uint32_t *bits) {
     const int u = blockIdx.x, w = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    predecessor_done();
     if (w >= n_words) return;
     const int key = 32 * w + lane;
     const uint32_t word = __ballot_sync(0xFFFFFFFFu, key < L && modality[(int64_t)u * L + key] != 0);
@@ -229,6 +231,7 @@ __global__ void pack_modality_kernel(const uint8_t *modality, int L, int n_words
 // probability; padding rows get a constant that makes every probability 0.
 __global__ void score_combine_kernel(const float2 *row_part, int n_chunk, int GW, int GWpad, int n_uh, float *negc) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    predecessor_done();
     if (i >= n_uh * GWpad) return;
     const int uh = i / GWpad, r = i % GWpad;
     float out = kNegBig;

@@ -41,6 +41,7 @@ select_topb_kernel(const float *importance, int L, int B, int W, int keep_window
     __shared__ int scratch[33];
     __shared__ uint32_t s_prefix;
     __shared__ int s_need;
+    predecessor_done();
     const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31;
     const float *imp = importance + (int64_t)blockIdx.x * L;
     int *ret = retained + (int64_t)blockIdx.x * B;
@@ -220,6 +221,7 @@ __global__ void __launch_bounds__(32 * NW) build_csr_kernel(const CsrArgs A) {
     __shared__ int scratch[33];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int uh = blockIdx.x;
+    predecessor_done();
     if (uh == 0 && tid == 0) *A.ticket = 0u;
     const int *match = A.match + (int64_t)uh * A.E;
     const int Ep = (A.E + 7) & ~7;
@@ -439,6 +441,7 @@ constexpr int kMergeBatch = 8;        // member rows a warp keeps in flight
 template <typename T>
 __global__ void __launch_bounds__(256) merge_pieces_kernel(const MergeArgs A, int n_uh) {
     constexpr int V = Elem<T>::kVec;
+    predecessor_done();
     const int lane = lane_id();
     const unsigned n_warps = gridDim.x * (blockDim.x >> 5);
     const unsigned total = (unsigned)n_uh * (unsigned)A.max_pieces;

@@ -82,6 +82,7 @@ struct ScoreArgs {
 // chunk of keys.  grid = (U*Hkv, row tiles of G*W, n_chunk1).
 template <typename T>
 __global__ void __launch_bounds__(kSimtThreads) score_stats_simt(const ScoreArgs A) {
+    predecessor_done();
     __shared__ SimtTiles sm;
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
     const int uh = blockIdx.x, u = uh / A.Hkv, h = uh % A.Hkv;
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(kSimtThreads) score_stats_simt(const ScoreArgs
 // 3*G*W floats.
 template <typename T>
 __global__ void __launch_bounds__(kSimtThreads) score_colsum_simt(const ScoreArgs A) {
+    predecessor_done();
     __shared__ SimtTiles sm;
     __shared__ float colpart[16][kTile];
     extern __shared__ float dyn[];
@@ -241,6 +243,7 @@ __global__ void __launch_bounds__(kSimtThreads) score_colsum_simt(const ScoreArg
 // cross_mass[u, g] = sum of the per-chunk partial masses; one warp per head.
 __global__ void cross_mass_reduce(const float *cross_part, int n_chunk, int n, float *cross_mass) {
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    predecessor_done();
     if (i >= n) return;
     const float s = head_mass(cross_part + (int64_t)i * n_chunk, n_chunk);
     if (lane_id() == 0) cross_mass[i] = s;
@@ -250,6 +253,7 @@ __global__ void cross_mass_reduce(const float *cross_part, int n_chunk, int n, f
 __global__ void layer_flow_kernel(const float *cross_mass, int U, int Hq, int W, float theta, int flow_mode,
                                   float *rho, int *strategy) {
     const int u = blockIdx.x * blockDim.x + threadIdx.x;
+    predecessor_done();
     if (u >= U) return;
     float s = 0.f;
     for (int g = 0; g < Hq; ++g) s += cross_mass[(int64_t)u * Hq + g] / (float)W;   // a head's total mass is W
@@ -262,6 +266,7 @@ __global__ void layer_flow_kernel(const float *cross_mass, int U, int Hq, int W,
 // and the theta rule.  parts [n_tiles][U * Hq]; one block per unit, one thread per query head.
 __global__ void full_flow_reduce_kernel(const float *parts, int n_tiles, int n, int Hq, int L, float theta, int flow_mode,
                                         float *cross_mass, float *rho, int *strategy) {
+    predecessor_done();
     const int u = blockIdx.x;
     for (int g = threadIdx.x; g < Hq; g += blockDim.x) {
         float s = 0.f;
@@ -283,6 +288,7 @@ template <typename T>
 __global__ void inv_norm_kernel(const void *k_, int64_t n_rows, int Hkv, int L, int D, int64_t s0, int64_t s1,
                                 int64_t s2, float *rn) {
     constexpr int V = Elem<T>::kVec;
+    predecessor_done();
     const int lanes = D / V;                               // 8, 16 or 32
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t row = gid / lanes;
@@ -318,6 +324,7 @@ struct MatchArgs {
 // grid = (U*Hkv, ceil(E / 64)).
 template <typename T>
 __global__ void __launch_bounds__(kSimtThreads) match_simt(const MatchArgs A) {
+    predecessor_done();
     __shared__ SimtTiles sm;
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
     const int uh = blockIdx.x, u = uh / A.Hkv, h = uh % A.Hkv;

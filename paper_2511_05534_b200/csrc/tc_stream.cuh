@@ -17,6 +17,7 @@
 // stages) and Skel<128, 2> for problems whose items have few B columns, where the A operand is
 // the stream: two A stages per half let the next item's rows load while this item is computed.
 #pragma once
+#include "common.cuh"
 #include "tc_common.cuh"
 
 namespace flowmm {
@@ -123,6 +124,7 @@ struct Skel {
         __syncthreads();
         tc::tc_fence_after();
         c.tmem_base = *tmem_slot;
+        predecessor_done();
         return c;
     }
 
