@@ -16,8 +16,9 @@
 #include "merge_tc.cuh"
 #include "score_fused_tc.cuh"
 #include "match_tc.cuh"
+#include "merge_lists.cuh"
 #include "score_tc.cuh"
-#include "select_merge.cuh"
+#include "select.cuh"
 #include "simt_kernels.cuh"
 #include "tc_host.cuh"
 
@@ -132,7 +133,7 @@ void layout_merge(Layout &y, const flowmm_params &p, Take take) {
 Layout make_layout(const flowmm_params &p) {
     Layout y;
     const size_t U = p.n_units, Hq = p.n_q_heads, Hkv = p.n_kv_heads, L = p.seq_len, W = p.window;
-    const size_t B = p.n_keep, E = L - B, D = p.head_dim, G = Hq / Hkv;
+    const size_t B = p.n_keep, E = L - B, G = Hq / Hkv;
     const int row_tiles = (int)((G * W + kTile - 1) / kTile);
     y.n_chunk1 = chunks_for((int)L, (int)(U * Hkv) * row_tiles, y.chunk1);
     y.n_chunk2 = chunks_for((int)L, (int)(U * Hkv), y.chunk2);
@@ -436,25 +437,38 @@ MatchPrepArgs match_prep_args(const flowmm_params &p, const Layout &y, const voi
     return g;
 }
 
-// cross_mass != nullptr: the launch also applies Eq. 6 and the theta rule to the final masses (rho may be nullptr)
-// prep != nullptr: each block goes on to prepare its head's matching candidates (the fused call, tensor-core matching)
-flowmm_status run_select(const flowmm_params &p, const float *importance, int32_t *retained, int32_t *evicted,
-                         cudaStream_t st, float *cross_mass = nullptr, float *rho = nullptr,
-                         int32_t *strategy = nullptr, const float *cross_part = nullptr, int n_parts = 0,
-                         const MatchPrepArgs *prep = nullptr) {
-    const int few = p.n_units * p.n_kv_heads < 2 * tc::sm_count();       // few heads: more threads per head
-    const int threads = few ? (p.seq_len <= 512 ? 256 : kSelectThreads) : p.seq_len <= 2048 ? 256 : p.seq_len <= 8192 ? 512 : kSelectThreads;
-    SelectFlow f;
-    f.cross_part = cross_part; f.n_parts = n_parts; f.cross_mass = cross_mass; f.rho = rho; f.strategy = strategy; f.Hq = p.n_q_heads; f.Hkv = p.n_kv_heads;
-    f.theta = p.theta; f.flow_mode = p.flow_mode;
-    MatchPrepArgs none = {};
-    launch(select_topb_kernel, p.n_units * p.n_kv_heads, threads, 0, st, importance, p.seq_len, p.n_keep, p.window,
-                                                                           p.keep_window, retained, evicted, f,
-                                                                           prep ? *prep : none, prep ? 1 : 0);
+template <int kThreads, bool kOneChunk>
+flowmm_status launch_select(const SelectArgs &a, const SelectFlow &f, const MatchPrepArgs &g, int with_prepare, cudaStream_t st) {
+    const size_t smem = select_smem(a.chunk);
+    if (cudaFuncSetAttribute(select_topb_kernel<kThreads, kOneChunk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return FLOWMM_ERR_CUDA;
+    launch(select_topb_kernel<kThreads, kOneChunk>, a.n_heads + f.n_units, kThreads, smem, st, a, f, g, with_prepare);
     FLOWMM_LAUNCHED("select_topb");
     return FLOWMM_OK;
 }
 
+// flow != nullptr: the launch also applies Eq. 6 and the theta rule (SelectFlow's comments).
+// prep != nullptr: each block goes on to prepare its head's matching candidates (tensor-core matching).
+// row_mod, row_mod_out: the pivots' modalities are written as well, from one modality map per head.
+flowmm_status run_select(const flowmm_params &p, const float *importance, int32_t *retained, int32_t *evicted,
+                         cudaStream_t st, const SelectFlow *flow = nullptr, const MatchPrepArgs *prep = nullptr,
+                         const uint8_t *row_mod = nullptr, uint8_t *row_mod_out = nullptr) {
+    SelectArgs a;
+    a.importance = importance; a.retained = retained; a.evicted = evicted; a.row_mod_out = row_mod_out;
+    a.n_heads = p.n_units * p.n_kv_heads; a.L = p.seq_len; a.B = p.n_keep; a.W = p.window; a.keep_window = p.keep_window;
+    a.chunk = p.seq_len <= kSelMaxChunk ? (p.seq_len + 31) / 32 * 32 : kSelMaxChunk;
+    const SelectFlow no_flow = {};
+    MatchPrepArgs g = {};
+    g.Hkv = 1; g.modality = row_mod;
+    if (prep) g = *prep;
+    const SelectFlow &f = flow ? *flow : no_flow;
+    // Warps per head: a block's latency is its rounds of shared-memory work, which shrink with more warps until the
+    // barriers outweigh them (640 tokens) or other heads' blocks no longer fit beside it
+    if (p.seq_len <= 1024) return launch_select<256, true>(a, f, g, prep != nullptr, st);
+    if (p.seq_len <= 4096) return launch_select<512, true>(a, f, g, prep != nullptr, st);
+    if (p.seq_len <= kSelMaxChunk) return launch_select<1024, true>(a, f, g, prep != nullptr, st);
+    return launch_select<1024, false>(a, f, g, prep != nullptr, st);
+}
 
 flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *k, const float *importance,
                            const uint8_t *mod, const int32_t *retained, const int32_t *evicted,
@@ -463,9 +477,8 @@ flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *
     const int UH = p.n_units * p.n_kv_heads, E = p.seq_len - p.n_keep;
     const MatchPrepArgs g = match_prep_args(p, y, k, importance, mod, retained, evicted, ws);
     if (!prepared) {                                 // (the fused call's selection launch has done it already)
-        // few heads: a head's lists are walked by more threads, the GPU is not full either way
-        const int prep_threads = UH >= 4 * tc::sm_count() ? 256 : UH >= 2 * tc::sm_count() ? 512 : 1024;
-        launch(match_prepare_kernel, UH, prep_threads, 0, st, g);
+        const int slices = (p.seq_len + kPrepSlice - 1) / kPrepSlice;
+        launch(match_prepare_kernel, dim3(UH, 1 + (slices < 64 ? slices : 64)), kPrepThreads, 0, st, g);
         FLOWMM_LAUNCHED("match_prepare");
     }
     if (!g.copy_here) {
@@ -762,8 +775,11 @@ flowmm_status flowmm_compress_layer(const flowmm_params *p, const void *q_win, c
     // ... and so does the candidate layout of the tensor-core matching step
     const bool prep_in_select = p->seq_len > p->n_keep && use_tc(*p);
     const MatchPrepArgs prep = match_prep_args(*p, y, k, importance, modality, retained_idx, evicted_idx, ws);
-    FLOWMM_TRY(run_select(*p, importance, retained_idx, evicted_idx, st, cross_mass, rho, strategy,
-                          n_parts > 0 ? at<float>(ws, y.cross_part) : nullptr, n_parts, prep_in_select ? &prep : nullptr));
+    SelectFlow flow = {};
+    flow.cross_part = n_parts > 0 ? at<float>(ws, y.cross_part) : nullptr; flow.n_parts = n_parts; flow.cross_mass = cross_mass;
+    flow.rho = rho; flow.strategy = strategy; flow.n_units = p->n_units; flow.Hq = p->n_q_heads;
+    flow.theta = p->theta; flow.flow_mode = p->flow_mode;
+    FLOWMM_TRY(run_select(*p, importance, retained_idx, evicted_idx, st, &flow, prep_in_select ? &prep : nullptr));
     // when both the short-list matching kernel and the tensor-core merge apply, the former writes the latter's table
     const bool map_in_match = p->seq_len > p->n_keep && use_tc(*p) && y.c_tot <= mst::kMaxCols && merge_is_tc(*p);
     FLOWMM_TRY(run_match(*p, y, k, importance, modality, retained_idx, evicted_idx, strategy, match, match_sim, ws, st,
@@ -1115,21 +1131,6 @@ extern "C" flowmm_status flowmm_decode_attention(const flowmm_decode_params *p, 
 // ---- re-compression of a cache that grew during decoding ----------------------------------------
 namespace {
 
-// strategy of a unit copied to each of its KV heads (the per-head problems below take one strategy each)
-__global__ void expand_strategy_kernel(const int32_t *strategy, int n_units, int n_kv_heads, int32_t *per_head) {
-    predecessor_done();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_units * n_kv_heads) per_head[i] = strategy[i / n_kv_heads];
-}
-
-// modality of the rows that were kept: out[uh, s] = row_modality[uh, retained[uh, s]]
-__global__ void gather_row_modality_kernel(const uint8_t *row_modality, const int32_t *retained, int64_t n, int L, int B,
-                                           uint8_t *out) {
-    predecessor_done();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = row_modality[(i / B) * L + retained[i]];
-}
-
 // Every (unit, KV head) of the cache as a problem of its own: one KV head, its G query heads, its own row modalities.
 // Needs the unit stride of every tensor to be heads x head stride (one stride then steps through units and heads).
 bool per_head_params(const flowmm_params &p, flowmm_params &ph) {
@@ -1198,19 +1199,22 @@ extern "C" flowmm_status flowmm_recompress(const flowmm_params *p, const void *q
     if (!match_sim) match_sim = at<float>(ws, y.match_sim);
     float *cross_mass = at<float>(ws, y.cross_mass);             // [U * Hkv, G] = [U, Hq]
     int32_t *strategy_h = at<int32_t>(ws, r.strategy_h);
-    // scoring per (unit, KV head) against that head's own row modalities; Eq. 6 over all query heads of the layer
-    FLOWMM_TRY(run_score(ph, y, q_win, k_cache, row_modality, importance, cross_mass, ws, st));
-    FLOWMM_TRY(run_layer_flow(*p, cross_mass, rho, strategy, st));
-    launch(expand_strategy_kernel, (ph.n_units + 255) / 256, 256, 0, st, strategy, p->n_units, p->n_kv_heads, strategy_h);
-    FLOWMM_LAUNCHED("expand_strategy");
-    FLOWMM_TRY(run_select(ph, importance, retained_idx, evicted_idx, st));
-    FLOWMM_TRY(run_match(ph, y, k_cache, importance, row_modality, retained_idx, evicted_idx, strategy_h, match, match_sim, ws, st));
-    FLOWMM_TRY(run_merge(ph, y, k_cache, v_cache, retained_idx, evicted_idx, match, match_sim, k_out, v_out, ws, st));
-    const int64_t n = (int64_t)ph.n_units * p->n_keep;
-    launch(gather_row_modality_kernel, (unsigned)((n + 255) / 256), 256, 0, st, row_modality, retained_idx, n, p->seq_len, p->n_keep,
-                                                                            row_modality_out);
-    FLOWMM_LAUNCHED("gather_row_modality");
-    return FLOWMM_OK;
+    // scoring per (unit, KV head) against that head's own row modalities; Eq. 6 over all query heads of the layer rides along
+    // with the selection, which hands the unit's strategy to each of its heads and notes the kept rows' modalities
+    int n_parts = 0;
+    FLOWMM_TRY(run_score(ph, y, q_win, k_cache, row_modality, importance, cross_mass, ws, st, &n_parts));
+    const bool prep_in_select = p->seq_len > p->n_keep && use_tc(ph);
+    const MatchPrepArgs prep = match_prep_args(ph, y, k_cache, importance, row_modality, retained_idx, evicted_idx, ws);
+    SelectFlow flow = {};
+    flow.cross_part = n_parts > 0 ? at<float>(ws, y.cross_part) : nullptr; flow.n_parts = n_parts; flow.cross_mass = cross_mass;
+    flow.rho = rho; flow.strategy = strategy; flow.strategy_h = strategy_h; flow.n_units = p->n_units; flow.Hq = p->n_q_heads;
+    flow.n_rep = p->n_kv_heads; flow.theta = p->theta; flow.flow_mode = p->flow_mode;
+    FLOWMM_TRY(run_select(ph, importance, retained_idx, evicted_idx, st, &flow, prep_in_select ? &prep : nullptr, row_modality,
+                          row_modality_out));
+    const bool map_in_match = prep_in_select && y.c_tot <= mst::kMaxCols && merge_is_tc(ph);
+    FLOWMM_TRY(run_match(ph, y, k_cache, importance, row_modality, retained_idx, evicted_idx, strategy_h, match, match_sim, ws, st,
+                         map_in_match ? at<int2>(ws, y.tokmap) : nullptr, prep_in_select));
+    return run_merge(ph, y, k_cache, v_cache, retained_idx, evicted_idx, match, match_sim, k_out, v_out, ws, st, map_in_match);
 }
 
 // ---- bounded-wait self-test ----------------------------------------------------------------------

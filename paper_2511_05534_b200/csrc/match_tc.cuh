@@ -40,57 +40,64 @@ struct MatchPrepArgs {
 
 // Copies the candidate key rows (256 bytes each) of positions [lo, hi) of one head's candidate
 // list, 16 lanes per row, and takes each row's reciprocal norm on the way (0 for a zero row: its
-// similarity to anything is 0).  lo, hi multiples of 16; every thread of the block takes part.
-__device__ __forceinline__ void match_gather_rows(const MatchPrepArgs &A, int uh, int lo, int hi, int tid, int nthreads) {
+// similarity to anything is 0).  lo, hi multiples of 32; every thread of the block takes part.
+// cand_tok: the positions' tokens (-1: no candidate), or nullptr: found through the slots and the pivot list.
+// kRows rows per lane are in flight together: a row is one dependent chain of loads.
+template <int kRows>
+__device__ __forceinline__ void match_gather_rows(const MatchPrepArgs &A, int uh, const int *cand_tok, int lo, int hi, int tid, int nthreads) {
     const int u = uh / A.Hkv, h = uh % A.Hkv;
     const int *ret = A.retained + (int64_t)uh * A.B;
     const int *slot_out = A.cand_slot + (int64_t)uh * A.Ctot;
     float *scale_out = A.cand_scale + (int64_t)uh * A.Ctot;
     const __nv_bfloat16 *kb = static_cast<const __nv_bfloat16 *>(A.k) + u * A.ks[0] + h * A.ks[1];
     uint4 *dst = reinterpret_cast<uint4 *>(A.cand_k + (int64_t)uh * A.Ctot * 128);
-    const int sub = tid & 15;
-    for (int pos = lo + (tid >> 4); pos < hi; pos += nthreads >> 4) {       // uniform trip count within a warp
-        const int s = slot_out[pos];
-        uint4 val = make_uint4(0, 0, 0, 0);
-        if (s >= 0 && index_ok(s, A.B, A.status) && index_ok(ret[s], A.L, A.status))
-            val = *reinterpret_cast<const uint4 *>(kb + (int64_t)ret[s] * A.ks[2] + sub * 8);
-        dst[(int64_t)pos * 16 + sub] = val;
-        float x[8], ssq = 0.f;
-        Elem<__nv_bfloat16>::unpack(val, x);
+    const int sub = tid & 15, stride = nthreads >> 4;
+    for (int p0 = lo + (tid >> 4); p0 < hi; p0 += kRows * stride) {         // uniform trip count within a warp
+        int tok[kRows];
+        uint4 val[kRows];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) ssq = fmaf(x[e], x[e], ssq);
+        for (int q = 0; q < kRows; ++q) {
+            const int pos = p0 + q * stride;
+            tok[q] = -1;
+            if (pos < hi) {
+                if (cand_tok) tok[q] = cand_tok[pos];
+                else {
+                    const int s = slot_out[pos];
+                    if (s >= 0 && index_ok(s, A.B, A.status)) tok[q] = ret[s];
+                }
+            }
+        }
 #pragma unroll
-        for (int o = 8; o > 0; o >>= 1) ssq += __shfl_xor_sync(0xFFFFFFFFu, ssq, o);
-        if (sub == 0 && s >= 0) scale_out[pos] = ssq > 0.f ? rsqrtf(ssq) : 0.f;
+        for (int q = 0; q < kRows; ++q) {
+            val[q] = make_uint4(0, 0, 0, 0);
+            if (tok[q] >= 0 && index_ok(tok[q], A.L, A.status))
+                val[q] = *reinterpret_cast<const uint4 *>(kb + (int64_t)tok[q] * A.ks[2] + sub * 8);
+        }
+#pragma unroll
+        for (int q = 0; q < kRows; ++q) {
+            const int pos = p0 + q * stride;
+            if (pos >= hi) break;                                           // (the same for both rows of a warp)
+            dst[(int64_t)pos * 16 + sub] = val[q];
+            float x[8], ssq = 0.f;
+            Elem<__nv_bfloat16>::unpack(val[q], x);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) ssq = fmaf(x[e], x[e], ssq);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) ssq += __shfl_xor_sync(0xFFFFFFFFu, ssq, o);
+            if (sub == 0 && tok[q] >= 0) scale_out[pos] = ssq > 0.f ? rsqrtf(ssq) : 0.f;
+        }
     }
 }
 
-// The preparation of one (unit, head) by its whole block (256 to 1024 threads, a multiple of 32); `scratch` = 33 ints
-// and `s_ntext` = one int of shared memory.  Also called at the end of the selection kernel, which has just written
-// this head's index lists.
-__device__ __forceinline__ void match_prepare_head(const MatchPrepArgs &A, int uh, int *scratch, int *s_ntext) {
-    const int tid = threadIdx.x, u = uh / A.Hkv, h = uh % A.Hkv;
+// The candidate layout of one head from its pivot list, by a whole block (`scratch`: 33 ints of shared memory).
+__device__ __forceinline__ void match_lay_out_candidates(const MatchPrepArgs &A, int uh, int *scratch) {
+    const int tid = threadIdx.x, u = uh / A.Hkv;
     const int *ret = A.retained + (int64_t)uh * A.B;
-    const int *evi = A.evicted + (int64_t)uh * A.E;
     const float *imp = A.importance + (int64_t)uh * A.L;
     const uint8_t *mod = A.modality + (int64_t)u * A.L;
-    int *rank = A.rank + (int64_t)uh * A.L;
     int *slot_out = A.cand_slot + (int64_t)uh * A.Ctot;
     float *scale_out = A.cand_scale + (int64_t)uh * A.Ctot;
-
     for (int i = tid; i < A.Ctot; i += blockDim.x) { slot_out[i] = -1; scale_out[i] = __int_as_float(0x7FC00000); }   // NaN: no candidate here
-    for (int s = tid; s < A.B; s += blockDim.x)
-        if (index_ok(ret[s], A.L, A.status)) rank[ret[s]] = -(s + 2);
-    for (int j = tid; j < A.E; j += blockDim.x)
-        if (index_ok(evi[j], A.L, A.status)) rank[evi[j]] = j;
-    if (h == 0) {
-        for (int t = tid; t < A.n_rt; t += blockDim.x) {
-            int bits = 0;
-            const int hi = min(A.L, (t + 1) * kMtItemRows);
-            for (int i = t * kMtItemRows; i < hi; ++i) bits |= mod[i] ? 2 : 1;
-            A.tile_mod[(int64_t)u * A.n_rt + t] = (uint8_t)bits;
-        }
-    }
     // admissible text pivots first: count them to know where the visual group starts
     int n_text = 0;
     for (int s = tid; s < A.B; s += blockDim.x) {
@@ -99,9 +106,7 @@ __device__ __forceinline__ void match_prepare_head(const MatchPrepArgs &A, int u
     }
     int total;
     block_exclusive_scan(n_text, scratch, total);
-    if (tid == 0) *s_ntext = total;
-    __syncthreads();
-    const int t0 = (*s_ntext + 31) & ~31;
+    const int t0 = (total + 31) & ~31;
     int seen_t = 0, seen_v = 0;
     for (int base = 0; base < A.B; base += blockDim.x) {
         const int s = base + tid;
@@ -112,25 +117,59 @@ __device__ __forceinline__ void match_prepare_head(const MatchPrepArgs &A, int u
             ft = adm && mod[r] == 0;
             fv = adm && mod[r] != 0;
         }
-        int tot_t, tot_v;
-        const int pt = seen_t + block_exclusive_scan(ft, scratch, tot_t);
-        const int pv = seen_v + block_exclusive_scan(fv, scratch, tot_v);
-        if (ft) slot_out[pt] = s;
-        if (fv) slot_out[t0 + pv] = s;
-        seen_t += tot_t;
-        seen_v += tot_v;
+        int tot;                                               // (both counts in one scan: text in the low half, at most 1024 each)
+        const int both = block_exclusive_scan(ft | fv << 16, scratch, tot);
+        if (ft) slot_out[seen_t + (both & 0xFFFF)] = s;
+        if (fv) slot_out[t0 + seen_v + (both >> 16)] = s;
+        seen_t += tot & 0xFFFF;
+        seen_v += tot >> 16;
     }
     if (tid == 0) { A.cand_count[2 * uh] = seen_t; A.cand_count[2 * uh + 1] = seen_v; }
     __syncthreads();
-    if (A.copy_here) match_gather_rows(A, uh, 0, A.Ctot, tid, blockDim.x);
+    if (A.copy_here) match_gather_rows<4>(A, uh, nullptr, 0, A.Ctot, tid, blockDim.x);
 }
 
-// grid = U*Hkv, block = 256 to 1024 (a multiple of 32).
-__global__ void __launch_bounds__(1024) match_prepare_kernel(const MatchPrepArgs A) {
+// The preparation of flowmm_match, which is handed the index lists (inside flowmm_compress_layer and flowmm_recompress the
+// selection kernel lays everything out itself).  grid = (U*Hkv, 1 + parts), block = 512: blocks y = 0 lay out a head's
+// candidates, the others write the rank of every token and the tiles' modalities, a slice each.
+constexpr int kPrepThreads = 512;
+constexpr int kPrepSlice = 8 * kPrepThreads;                   // list entries of a rank block: eight loads in flight per thread
+__global__ void __launch_bounds__(kPrepThreads) match_prepare_kernel(const MatchPrepArgs A) {
     __shared__ int scratch[33];
-    __shared__ int s_ntext;
     predecessor_done();
-    match_prepare_head(A, blockIdx.x, scratch, &s_ntext);
+    const int uh = blockIdx.x, tid = threadIdx.x;
+    if (blockIdx.y == 0) { match_lay_out_candidates(A, uh, scratch); return; }
+    const int part = blockIdx.y - 1, parts = gridDim.y - 1;
+    const int *ret = A.retained + (int64_t)uh * A.B;
+    const int *evi = A.evicted + (int64_t)uh * A.E;
+    int *rank = A.rank + (int64_t)uh * A.L;
+    for (int i0 = part * kPrepSlice; i0 < A.L; i0 += parts * kPrepSlice) {   // entries of the two lists, pivots first
+        int tok[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int i = i0 + e * kPrepThreads + tid;
+            tok[e] = i < A.B ? ret[i] : i < A.L ? evi[i - A.B] : -1;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int i = i0 + e * kPrepThreads + tid;
+            if (i < A.L && index_ok(tok[e], A.L, A.status)) rank[tok[e]] = i < A.B ? -(i + 2) : i - A.B;
+        }
+    }
+    if (uh % A.Hkv == 0) {
+        const int u = uh / A.Hkv, lane = tid & 31, n_warps = kPrepThreads / 32;
+        const uint8_t *mod = A.modality + (int64_t)u * A.L;
+        for (int t = part * n_warps + (tid >> 5); t < A.n_rt; t += parts * n_warps) {
+            bool any_t = false, any_v = false;
+#pragma unroll
+            for (int q = 0; q < kMtItemRows / 32; ++q) {
+                const int i = t * kMtItemRows + q * 32 + lane;
+                if (i < A.L) { if (mod[i]) any_v = true; else any_t = true; }
+            }
+            any_t = __any_sync(0xFFFFFFFFu, any_t); any_v = __any_sync(0xFFFFFFFFu, any_v);
+            if (lane == 0) A.tile_mod[(int64_t)u * A.n_rt + t] = (uint8_t)((any_t ? 1 : 0) | (any_v ? 2 : 0));
+        }
+    }
 }
 
 // The gather step of the preparation as a kernel of its own for long candidate lists, so that many
@@ -138,7 +177,7 @@ __global__ void __launch_bounds__(1024) match_prepare_kernel(const MatchPrepArgs
 __global__ void __launch_bounds__(256) match_gather_kernel(const MatchPrepArgs A) {
     predecessor_done();
     const int lo = blockIdx.y * 64;
-    match_gather_rows(A, blockIdx.x, lo, min(A.Ctot, lo + 64), threadIdx.x, blockDim.x);
+    match_gather_rows<4>(A, blockIdx.x, nullptr, lo, min(A.Ctot, lo + 64), threadIdx.x, blockDim.x);
 }
 
 struct MatchTcArgs {

@@ -1,169 +1,9 @@
-// Pivot selection (top-B per KV head) and the merge / compaction stage.
+// The merge / compaction stage.
 #pragma once
 #include <type_traits>
 #include "common.cuh"
-#include "match_tc.cuh"
 
 namespace flowmm {
-
-constexpr int kSelectThreads = 1024;
-
-// Order-preserving integer key of an importance (a non-negative float); window tokens forced
-// into the pivot set get the largest key.
-__device__ __forceinline__ uint32_t select_key(float v, bool forced) {
-    if (forced) return 0xFFFFFFFFu;
-    const uint32_t b = __float_as_uint(v);
-    return (b & 0x80000000u) ? 0u : b;        // -0 and (never expected) negatives sort lowest
-}
-
-// Section 3.3.1 pivot selection: a radix select finds the B-th largest key, then one ordered
-// sweep writes the pivot positions and the non-pivot positions, both ascending.  Ties at the
-// threshold go to the lower positions.  grid = U*Hkv, block = any multiple of 32 up to 1024.
-// Eq. 6 and the theta rule riding along with the selection (cross_mass == nullptr: not asked for): the block of a
-// unit's first KV head applies them, one thread, same arithmetic as layer_flow_kernel.
-struct SelectFlow {
-    const float *cross_part;     // nullptr, or [U * Hq, n_parts] partial masses that are first added up into cross_mass
-    int n_parts;
-    float *cross_mass;           // [U, Hq] per-head masses (read; written first when cross_part is given)
-    float *rho;                  // [U] or nullptr
-    int *strategy;               // [U]
-    int Hq, Hkv;
-    float theta;
-    int flow_mode;
-};
-
-// with_prepare: the block goes on to lay out the head's matching candidates (match_prepare_head) from the lists it has
-// just written, which saves the short-context workloads a launch and a second pass over the same few kilobytes.
-__global__ void __launch_bounds__(kSelectThreads)
-select_topb_kernel(const float *importance, int L, int B, int W, int keep_window, int *retained, int *evicted,
-                   const SelectFlow F, const MatchPrepArgs P, int with_prepare) {
-    __shared__ int hist[256];
-    __shared__ int scratch[33];
-    __shared__ uint32_t s_prefix;
-    __shared__ int s_need;
-    predecessor_done();
-    const int tid = threadIdx.x, nthreads = blockDim.x, lane = tid & 31;
-    const float *imp = importance + (int64_t)blockIdx.x * L;
-    int *ret = retained + (int64_t)blockIdx.x * B;
-    int *evi = evicted + (int64_t)blockIdx.x * (L - B);
-    const int first_forced = keep_window ? L - W : L;
-    if (F.cross_part && blockIdx.x % F.Hkv == 0) {                   // (the same for every thread of the block)
-        const int u = blockIdx.x / F.Hkv;
-        for (int g = tid >> 5; g < F.Hq; g += nthreads >> 5) {      // same sums in the same order as cross_mass_reduce
-            const int64_t i = (int64_t)u * F.Hq + g;
-            const float s = head_mass(F.cross_part + i * F.n_parts, F.n_parts);
-            if (lane == 0) F.cross_mass[i] = s;
-        }
-        __syncthreads();
-    }
-    if (F.cross_mass && blockIdx.x % F.Hkv == 0 && tid == nthreads - 1) {
-        const int u = blockIdx.x / F.Hkv;
-        float s = 0.f;
-        for (int g = 0; g < F.Hq; ++g) s += F.cross_mass[(int64_t)u * F.Hq + g] / (float)W;   // a head's total mass is W
-        const float r = s / (float)F.Hq;
-        if (F.rho) F.rho[u] = r;
-        F.strategy[u] = F.flow_mode == 1 ? 0 : F.flow_mode == 2 ? 1 : ((r > F.theta) != (F.flow_mode == 3) ? 1 : 0);
-    }
-
-    // radix select, most significant byte first: after the loop `prefix` is the B-th largest key
-    uint32_t prefix = 0, mask = 0;
-    int need = B;                                    // how many keys to take among those matching prefix
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int i = tid; i < 256; i += nthreads) hist[i] = 0;
-        __syncthreads();
-        // Eight keys per thread are in flight at a time, and a thread adds runs of equal digits at once: the first
-        // digits (sign and exponent) are nearly the same for all keys, which would put every thread's every add on one counter.
-        {
-            int run_bin = -1, run_cnt = 0;
-            for (int base = 0; base < L; base += 8 * nthreads) {
-                uint32_t keys[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int i = base + e * nthreads + tid;
-                    keys[e] = i < L ? select_key(imp[i], i >= first_forced) : 0u;
-                }
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const int i = base + e * nthreads + tid;
-                    if (i < L && (keys[e] & mask) == prefix) {
-                        const int bin = (keys[e] >> shift) & 255;
-                        if (bin != run_bin) {
-                            if (run_cnt > 0) atomicAdd(&hist[run_bin], run_cnt);
-                            run_bin = bin; run_cnt = 0;
-                        }
-                        ++run_cnt;
-                    }
-                }
-            }
-            if (run_cnt > 0) atomicAdd(&hist[run_bin], run_cnt);
-        }
-        __syncthreads();
-        if (tid < 32) {                              // walk down from the largest digit, 8 digits per lane
-            int local[8], lsum = 0;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) { local[e] = hist[255 - (lane * 8 + e)]; lsum += local[e]; }
-            int incl = lsum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                if (lane >= o) incl += t;
-            }
-            int acc = incl - lsum;                   // keys with a larger digit than this lane's first
-            if (acc < need && need <= incl) {        // the B-th largest key has one of this lane's digits
-                int e = 0;
-                for (; e < 7; ++e) {
-                    if (acc + local[e] >= need) break;
-                    acc += local[e];
-                }
-                s_prefix = prefix | ((uint32_t)(255 - (lane * 8 + e)) << shift);
-                s_need = need - acc;
-            }
-        }
-        __syncthreads();
-        prefix = s_prefix;
-        need = s_need;
-        mask |= 0xFFu << shift;
-    }
-    // keys > prefix are all kept; of the keys == prefix the first `need` (by position) are kept
-    // (four consecutive positions per thread and iteration: a quarter of the block-wide scans)
-    int eq_seen = 0, kept_seen = 0;
-    for (int base = 0; base < L; base += 4 * nthreads) {
-        const int i0 = base + 4 * tid;
-        uint32_t key[4];
-        int n_eq = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            key[e] = i0 + e < L ? select_key(imp[i0 + e], i0 + e >= first_forced) : 0u;
-            n_eq += i0 + e < L && key[e] == prefix;
-        }
-        int total_eq;
-        int eq_rank = eq_seen + block_exclusive_scan(n_eq, scratch, total_eq);
-        int keep[4], n_keep = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const bool valid = i0 + e < L, is_eq = valid && key[e] == prefix;
-            keep[e] = valid && (key[e] > prefix || (is_eq && eq_rank < need));
-            eq_rank += is_eq;
-            n_keep += keep[e];
-        }
-        int total_keep;
-        int pos = kept_seen + block_exclusive_scan(n_keep, scratch, total_keep);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (i0 + e < L) {
-                if (keep[e]) ret[pos] = i0 + e;
-                else evi[i0 + e - pos] = i0 + e;
-            }
-            pos += keep[e];
-        }
-        eq_seen += total_eq;
-        kept_seen += total_keep;
-    }
-    if (with_prepare) {
-        __syncthreads();                                 // this block's lists are complete and visible to all its threads
-        match_prepare_head(P, blockIdx.x, scratch, &s_need);
-    }
-}
 
 // ---------------------------------------------------------------------------------------------
 // Merge stage.  The match array maps non-pivot j to a slot (or -1).  The members of every slot

@@ -10,7 +10,7 @@
 // eight warps fit an SM and each warp keeps up to 9 KB coming.
 #pragma once
 #include "common.cuh"
-#include "select_merge.cuh"
+#include "merge_lists.cuh"
 #include "tc_common.cuh"
 
 namespace flowmm {

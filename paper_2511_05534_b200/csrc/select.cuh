@@ -1,0 +1,347 @@
+// Pivot selection (top-B per KV head, Section 3.3.1) with what rides along with it: the layer flow of Eq. 6, the theta
+// rule, and the candidate layout of the tensor-core matching step.
+#pragma once
+#include "common.cuh"
+#include "match_tc.cuh"
+
+namespace flowmm {
+
+// Order-preserving integer key of an importance (a non-negative float); window tokens forced
+// into the pivot set get the largest key.  31 bits: bit 31 of a staged word holds the token's modality.
+constexpr uint32_t kKeyMask = 0x7FFFFFFFu;
+__device__ __forceinline__ uint32_t select_key(float v, bool forced) {
+    if (forced) return kKeyMask;
+    const uint32_t b = __float_as_uint(v);
+    return (b & 0x80000000u) ? 0u : b;        // -0 and (never expected) negatives sort lowest
+}
+
+// Eq. 6 and the theta rule riding along with the selection: one extra block per unit, behind those of the heads.
+struct SelectFlow {
+    const float *cross_part;     // nullptr, or [n_units * Hq, n_parts] partial masses that are first added up into cross_mass
+    int n_parts;
+    float *cross_mass;           // [n_units, Hq] per-head masses (read; written first when cross_part is given)
+    float *rho;                  // [n_units] or nullptr
+    int *strategy;               // [n_units]
+    int *strategy_h;             // nullptr, or [n_units, n_rep]: the unit's strategy once more for each of its KV heads
+    int n_units, Hq, n_rep;
+    float theta;
+    int flow_mode;
+};
+
+struct SelectArgs {
+    const float *importance;     // [n_heads, L]
+    int *retained, *evicted;     // [n_heads, B], [n_heads, L - B]
+    uint8_t *row_mod_out;        // nullptr, or [n_heads, B]: the pivots' modalities (one modality map per head: P.Hkv == 1)
+    int n_heads, L, B, W, keep_window;
+    int chunk;                   // positions handled at a time, a multiple of 32: the whole context if it fits in shared memory
+};
+
+// The extra block of unit u.  Sums as in cross_mass_reduce and layer_flow_kernel, term for term.
+__device__ __forceinline__ void select_flow_block(const SelectFlow &F, int u, int W, float *masses) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    if (F.cross_part) {
+        for (int g = warp; g < F.Hq; g += nwarps) {
+            const int64_t i = (int64_t)u * F.Hq + g;
+            const float s = head_mass(F.cross_part + i * F.n_parts, F.n_parts);
+            if (lane == 0) F.cross_mass[i] = s;
+        }
+        __syncthreads();
+    }
+    float s = 0.f;
+    for (int g0 = 0; g0 < F.Hq; g0 += blockDim.x) {              // (one round unless a unit has more heads than threads)
+        const int g = g0 + threadIdx.x;
+        if (g < F.Hq) masses[threadIdx.x] = F.cross_mass[(int64_t)u * F.Hq + g] / (float)W;   // a head's total mass is W
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int j = 0; j < min((int)blockDim.x, F.Hq - g0); ++j) s += masses[j];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const float r = s / (float)F.Hq;
+        const int st = F.flow_mode == 1 ? 0 : F.flow_mode == 2 ? 1 : ((r > F.theta) != (F.flow_mode == 3) ? 1 : 0);
+        if (F.rho) F.rho[u] = r;
+        F.strategy[u] = st;
+        if (F.strategy_h)
+            for (int h = 0; h < F.n_rep; ++h) F.strategy_h[(int64_t)u * F.n_rep + h] = st;
+    }
+}
+
+constexpr int kSelBits = 11, kSelBins = 1 << kSelBits;           // digit width of the radix select
+// dynamic shared memory: two sets of counters; the chunk's words; six values per 32 positions
+__host__ __device__ constexpr size_t select_smem(int chunk) { return 4 * (2 * (size_t)kSelBins + chunk + 6 * (size_t)(chunk / 32)); }
+constexpr int kSelMaxChunk = 45248;
+static_assert(select_smem(kSelMaxChunk) <= 232448 - 1024, "shared memory budget");
+
+
+// The block of one head (blocks below n_heads).
+//   1. The importances are staged in shared memory as 31-bit keys with the token's modality in the top bit, and counted
+//      by their 11 highest key bits on the way.
+//   2. The digit that holds the B-th largest key is found from the counts; the next 11 (then 9) bits are only counted
+//      among the keys that share it.  Two digits decide nearly always: as soon as all keys of the last digit belong to
+//      the B, its lower bits do not matter.
+//   3. Warps mark the pivots (and, of those, the matching candidates by modality) of 32 positions at a time, one prefix
+//      sum over the words of marks numbers them, warps write the lists, all ascending.  Ties at the threshold go to the
+//      lower positions.
+// Bound by latency: one block per head, a few dependent rounds over shared memory.  The marks and
+// one prefix sum replace block-wide scans per 1024 to 4096 positions, four counting passes over global memory and a separate
+// preparation pass over the lists: 128 heads of 33 792 tokens 118 -> 42 us, 32 heads of 640 tokens 20 -> 10 us.
+template <int kThreads, bool kOneChunk>
+__global__ void __launch_bounds__(kThreads)
+select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P, int with_prepare) {
+    constexpr int kWarps = kThreads / 32, kPer = kSelBins / kThreads;
+    extern __shared__ __align__(16) int sel_smem[];
+    __shared__ int wtot[kWarps], res[3];
+    __shared__ unsigned long long wsum[kWarps];
+    int *hist = sel_smem;
+    uint32_t *words = reinterpret_cast<uint32_t *>(sel_smem + 2 * kSelBins);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int head = blockIdx.x, L = A.L;
+    for (int i = tid; i < 2 * kSelBins / 4; i += kThreads) reinterpret_cast<int4 *>(hist)[i] = make_int4(0, 0, 0, 0);
+    __syncthreads();
+    predecessor_done();
+    if (head >= A.n_heads) {
+        select_flow_block(F, head - A.n_heads, A.W, reinterpret_cast<float *>(hist));
+        return;
+    }
+    const float *imp = A.importance + (int64_t)head * L;
+    const uint8_t *mod = P.modality + (int64_t)(head / P.Hkv) * L;   // (not read unless with_prepare)
+    const int first_forced = A.keep_window ? L - A.W : L;
+    auto word = [&](int i) -> uint32_t {
+        if (kOneChunk) return words[i];
+        return select_key(imp[i], i >= first_forced) | (with_prepare && mod[i] ? 0x80000000u : 0u);
+    };
+
+    // keys that agree with `prefix` in the bits of `mask`, counted by the `width` bits at `shift`
+    uint32_t prefix = 0, mask = 0;
+    auto count = [&](uint32_t key, int *h, int shift, int width) {
+        if ((key & mask) == prefix) atomicAdd(h + ((int)(key >> shift) & ((1 << width) - 1)), 1);
+    };
+    for (int base = 0; base < L; base += 8 * kThreads) {
+        float v[8];
+        uint8_t m[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int i = base + e * kThreads + tid;
+            v[e] = i < L ? imp[i] : 0.f;
+            m[e] = with_prepare && i < L ? mod[i] : 0;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            if (base + e * kThreads >= L) break;                     // (the same for the whole block)
+            const int i = base + e * kThreads + tid;
+            if (i < L) {
+                const uint32_t key = select_key(v[e], i >= first_forced);
+                if (kOneChunk) words[i] = key | (m[e] ? 0x80000000u : 0u);
+                count(key, hist, 20, 11);
+            }
+        }
+    }
+    int need = A.B, n_eq = 0;                                        // keys still to take among those that match the prefix; their number
+#pragma unroll 1
+    for (int pass = 0; pass < 3; ++pass) {
+        const int shift = pass == 0 ? 20 : pass == 1 ? 9 : 0, width = pass == 2 ? 9 : 11;
+        int *h = hist + (pass & 1) * kSelBins;
+        if (pass > 0) {
+            for (int i = tid; i < L; i += kThreads) count(word(i) & kKeyMask, h, shift, width);
+        }
+        __syncthreads();
+        // counters from the largest digit down, kPer per thread; thread t holds digits hi - kPer + 1 .. hi
+        const int hi = kSelBins - 1 - tid * kPer;
+        int c[kPer], sum = 0;
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) { c[e] = h[hi - e]; sum += c[e]; }
+        int incl = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) wtot[warp] = incl;
+        __syncthreads();
+        int w = lane < kWarps && lane < warp ? wtot[lane] : 0;       // totals of the warps before this one
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xFFFFFFFFu, w, o);
+        int acc = w + incl - sum;                                    // keys with a larger digit than this thread's first
+        if (acc < need && need <= acc + sum) {
+            int e = 0;
+#pragma unroll
+            for (int q = 0; q < kPer - 1; ++q)
+                if (e == q && acc + c[q] < need) { acc += c[q]; ++e; }
+            int ce = c[0];
+#pragma unroll
+            for (int q = 1; q < kPer; ++q) ce = e == q ? c[q] : ce;
+            res[0] = hi - e; res[1] = need - acc; res[2] = ce;
+        }
+        __syncthreads();
+        prefix |= (uint32_t)res[0] << shift;
+        need = res[1];
+        n_eq = res[2];
+        mask |= ((1u << width) - 1u) << shift;
+        if (need == n_eq) break;                                     // all of them are kept: lower bits do not matter
+        if (pass == 1)                                               // the third digit takes the first one's counters
+            for (int i = tid; i < kSelBins; i += kThreads) hist[i] = 0;
+        __syncthreads();
+    }
+    const bool all_eq = need == n_eq;
+
+    // 3. the positions of a chunk in ascending order, 32 to a word
+    const int chunk_w = A.chunk >> 5;
+    uint32_t *keep_w = words + A.chunk;                              // which of a word's 32 positions are pivots,
+    uint32_t *text_w = keep_w + chunk_w, *vis_w = text_w + chunk_w;  // which of those are candidates, by modality,
+    int *pos_w = reinterpret_cast<int *>(vis_w + chunk_w);           // how many pivots come before the word,
+    int *pt_w = pos_w + chunk_w, *pv_w = pt_w + chunk_w;             // and how many candidates
+    const uint32_t lt = lanemask_lt();
+    int *ret = A.retained + (int64_t)head * A.B;
+    int *evi = A.evicted + (int64_t)head * (L - A.B);
+    int *rank = P.rank + (int64_t)head * L;
+    int *cand_tok = hist;                                            // token of every candidate column (copy_here: up to 256)
+    int *slot_out = P.cand_slot + (int64_t)head * P.Ctot;
+    float *scale_out = P.cand_scale + (int64_t)head * P.Ctot;
+    const bool copy_here = with_prepare && P.copy_here;
+    auto block_sum = [&](unsigned long long v, unsigned long long &total) -> unsigned long long {   // exclusive prefix sum
+        unsigned long long incl_v = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, incl_v, o);
+            if (lane >= o) incl_v += t;
+        }
+        __syncthreads();                                             // the totals of the call before have been read
+        if (lane == 31) wsum[warp] = incl_v;
+        __syncthreads();
+        const unsigned long long mine = lane < kWarps ? wsum[lane] : 0ull;
+        unsigned long long b = lane < warp ? mine : 0ull, all = mine;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            b += __shfl_xor_sync(0xFFFFFFFFu, b, o);
+            all += __shfl_xor_sync(0xFFFFFFFFu, all, o);
+        }
+        total = all;
+        return b + incl_v - v;
+    };
+    int t0 = 0;                                                      // first column of the visual candidates
+    // (a context longer than a chunk is walked once more beforehand, for the number of its text candidates)
+    for (int walk = kOneChunk || !with_prepare ? 1 : 0; walk < 2; ++walk) {
+        int seen = 0, seen_t = 0, seen_v = 0, seen_eq = 0;
+        for (int c0 = 0; c0 < L; c0 += A.chunk) {
+            const int n_w = (min(A.chunk, L - c0) + 31) >> 5, per = (n_w + kThreads - 1) / kThreads;
+            if (!all_eq) {                                           // ties at the threshold go to the lower positions:
+                for (int w = warp; w < n_w; w += kWarps) {           // mark the equal keys, then number them
+                    const int i = c0 + 32 * w + lane;
+                    const uint32_t eq = __ballot_sync(0xFFFFFFFFu, i < L && (word(i) & kKeyMask) == prefix);
+                    if (lane == 0) text_w[w] = eq;
+                }
+                __syncthreads();
+                const int w_lo = min(n_w, tid * per), w_hi = min(n_w, w_lo + per);   // words whose counts this thread adds up
+                unsigned long long n_mine = 0, tot;
+                for (int w = w_lo; w < w_hi; ++w) n_mine += __popc(text_w[w]);
+                int r = seen_eq + (int)block_sum(n_mine, tot);
+                for (int w = w_lo; w < w_hi; ++w) { pos_w[w] = r; r += __popc(text_w[w]); }
+                seen_eq += (int)tot;
+                __syncthreads();
+            }
+#pragma unroll 4
+            for (int w = warp; w < n_w; w += kWarps) {               // marks, a word per warp and step
+                const int i = c0 + 32 * w + lane;
+                const uint32_t wd = i < L ? word(i) : 0u, mk = wd & kKeyMask & mask;
+                bool take = i < L && mk >= prefix;
+                if (!all_eq && take && mk == prefix) take = pos_w[w] + __popc(text_w[w] & lt) < need;
+                const uint32_t keep = __ballot_sync(0xFFFFFFFFu, take);
+                uint32_t text = 0, vis = 0;
+                if (with_prepare) {                                  // Eq. 10: pivots above tau are kept out of merging
+                    const bool adm = take && (i < first_forced ? __uint_as_float(wd & kKeyMask) : imp[i]) <= P.tau_eff;
+                    const uint32_t cand = __ballot_sync(0xFFFFFFFFu, adm), seen_vis = __ballot_sync(0xFFFFFFFFu, wd >> 31);
+                    text = cand & ~seen_vis; vis = cand & seen_vis;
+                }
+                __syncwarp();
+                if (lane == 0) { keep_w[w] = keep; text_w[w] = text; vis_w[w] = vis; }
+            }
+            __syncthreads();
+            // Pivots (24 bits), admissible text pivots (20) and admissible visual ones (20) before each word: one prefix sum
+            // for all three.  Up to 128 words every warp takes it for itself, four words to a lane, without a barrier.
+            auto counts = [&](int w) -> unsigned long long {
+                return (unsigned long long)__popc(keep_w[w]) | (unsigned long long)__popc(text_w[w]) << 24 | (unsigned long long)__popc(vis_w[w]) << 44;
+            };
+            const bool few = kOneChunk && n_w <= 128;
+            const int w_lo = min(n_w, few ? 4 * lane : tid * per), w_hi = min(n_w, w_lo + (few ? 4 : per));
+            unsigned long long mine = 0, all, before;
+            for (int w = w_lo; w < w_hi; ++w) mine += counts(w);
+            if (few) {
+                before = mine;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, before, o);
+                    if (lane >= o) before += t;
+                }
+                all = __shfl_sync(0xFFFFFFFFu, before, 31);
+                before -= mine;
+            } else before = block_sum(mine, all);
+            const int n_text = (int)(all >> 24) & 0xFFFFF, n_vis = (int)(all >> 44);
+            if (kOneChunk) t0 = (n_text + 31) & ~31;                 // text group first, visual group from the next multiple of 32
+            if (walk == 1) {
+                int s = seen + (int)(before & 0xFFFFFF), pt = seen_t + ((int)(before >> 24) & 0xFFFFF), pv = t0 + seen_v + (int)(before >> 44);
+                for (int w = w_lo; w < w_hi; ++w) {                  // (few: every warp writes the same values, and reads its own)
+                    pos_w[w] = s; pt_w[w] = pt; pv_w[w] = pv;
+                    const unsigned long long c = counts(w);
+                    s += (int)(c & 0xFFFFFF); pt += (int)(c >> 24) & 0xFFFFF; pv += (int)(c >> 44);
+                }
+                if (few) __syncwarp(); else __syncthreads();
+#pragma unroll 4
+                for (int w = warp; w < n_w; w += kWarps) {           // the lists, a word per warp and step: coalesced
+                    const uint32_t keep = keep_w[w];
+                    const int i = c0 + 32 * w + lane, sl = pos_w[w] + __popc(keep & lt);
+                    if (i >= L) continue;
+                    if (!((keep >> lane) & 1u)) {
+                        evi[i - sl] = i;
+                        if (with_prepare) rank[i] = i - sl;
+                        continue;
+                    }
+                    ret[sl] = i;
+                    if (A.row_mod_out) A.row_mod_out[(int64_t)head * A.B + sl] = mod[i];
+                    if (with_prepare) {
+                        rank[i] = -(sl + 2);
+                        const uint32_t text = text_w[w], vis = vis_w[w];
+                        const int c = ((text >> lane) & 1u) ? pt_w[w] + __popc(text & lt) : ((vis >> lane) & 1u) ? pv_w[w] + __popc(vis & lt) : -1;
+                        if (c >= 0 && index_ok(c, P.Ctot, P.status)) {
+                            slot_out[c] = sl;
+                            if (copy_here) cand_tok[c] = i;
+                        }
+                    }
+                }
+                if (!kOneChunk) __syncthreads();                     // (the next chunk's words go into the same place)
+            }
+            seen += (int)(all & 0xFFFFFF); seen_t += n_text; seen_v += n_vis;
+        }
+        if (walk == 0) t0 = (seen_t + 31) & ~31;
+        else if (with_prepare) {
+            // columns without a candidate: between the groups and behind them
+            for (int c = seen_t + tid; c < P.Ctot; c += kThreads)
+                if (c < t0 || c >= t0 + seen_v) {
+                    slot_out[c] = -1;
+                    scale_out[c] = __int_as_float(0x7FC00000);       // NaN: no candidate here
+                    if (copy_here) cand_tok[c] = -1;
+                }
+            if (tid == 0) { P.cand_count[2 * head] = seen_t; P.cand_count[2 * head + 1] = seen_v; }
+        }
+    }
+    if (!with_prepare) return;
+    if (head % P.Hkv == 0) {                                         // modalities in every tile of 256 tokens
+        const int u = head / P.Hkv;
+        for (int tl = warp; tl < P.n_rt; tl += kWarps) {
+            uint32_t any_v = 0, any_t = 0;
+#pragma unroll
+            for (int q = 0; q < kMtItemRows / 32; ++q) {
+                const int i = tl * kMtItemRows + q * 32 + lane;
+                const bool in = i < L, vis = in && word(i) >> 31;
+                any_v |= vis; any_t |= in && !vis;
+            }
+            any_v = __any_sync(0xFFFFFFFFu, any_v); any_t = __any_sync(0xFFFFFFFFu, any_t);
+            if (lane == 0) P.tile_mod[(int64_t)u * P.n_rt + tl] = (uint8_t)((any_t ? 1 : 0) | (any_v ? 2 : 0));
+        }
+    }
+    if (copy_here) {
+        __syncthreads();
+        match_gather_rows<8>(P, head, cand_tok, 0, P.Ctot, tid, kThreads);
+    }
+}
+
+}  // namespace flowmm

@@ -1,0 +1,52 @@
+"""Selection kernel at the edges of its shapes: words of 32 positions, the block sizes (1024, 4096 tokens), contexts that
+exceed what fits in shared memory at once (45248 tokens), ties at the threshold, forced windows."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import flowmm_oracle as O
+from paper_2511_05534_b200 import binding as F
+
+from gpu_util import gpu_params, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("L,B", [(1, 1), (33, 32), (640, 64), (1024, 1), (1025, 1024), (4096, 400), (4097, 211), (33792, 1690),
+                                 (45248, 5000), (45249, 77), (100003, 9000)])
+@pytest.mark.parametrize("kind", ["spread", "ties", "equal", "window"])
+def test_select_against_oracle(L, B, kind):
+    rng = np.random.default_rng(L + B)
+    imp = np.exp(rng.standard_normal((3, 2, L)) * 2).astype(np.float32)
+    if kind == "ties":                                              # few distinct values: the threshold is shared by many
+        imp = np.round(imp * 2) / 2
+    elif kind == "equal":
+        imp[:] = 0.125
+    W = min(L, B, 16) if kind == "window" else 1
+    p = O.OracleParams(3, 4, 2, 64, L, W, B, keep_window=int(kind == "window"))
+    ref_r, ref_e = O.select(p, imp.astype(np.float64))
+    fp = gpu_params(p, F.F32)
+    r = torch.full((3, 2, B), -9, dtype=torch.int32, device="cuda")
+    e = torch.full((3, 2, L - B), -9, dtype=torch.int32, device="cuda")
+    F.flowmm_select(fp, torch.from_numpy(imp).cuda(), r, e, F.alloc_workspace(fp))
+    assert np.array_equal(r.cpu().numpy(), ref_r)
+    assert np.array_equal(e.cpu().numpy(), ref_e)
+
+
+@pytest.mark.parametrize("L,B", [(290, 193), (2000, 225), (46000, 300)])
+def test_fused_preparation_equals_the_steps(L, B):
+    """The candidate layout written by the selection launch of flowmm_compress_layer against the one flowmm_match makes
+    from the lists: same matches, bit for bit (short lists, long lists, a context of more than one chunk)."""
+    rng = np.random.default_rng(L)
+    p = O.OracleParams(2, 2, 1, 128, L, 32, B, theta=0.3, tau=2.0, tau_mode=O.TAU_REL)
+    q, k, v = (rng.standard_normal(s).astype(np.float32) for s in ((2, 2, 32, 128), (2, 1, L, 128), (2, 1, L, 128)))
+    m = (np.arange(L) % 700 < 500).astype(np.uint8)[None].repeat(2, 0)
+    got = run_gpu(p, q, k, v, m, F.BF16)
+    fp = gpu_params(p, F.BF16)
+    dev = lambda key, dt: torch.from_numpy(got[key]).to(dt).cuda()
+    match = torch.full((2, 1, L - B), -9, dtype=torch.int32, device="cuda")
+    sim = torch.zeros((2, 1, L - B), device="cuda")
+    F.flowmm_match(fp, torch.from_numpy(k).cuda().bfloat16(), dev("importance", torch.float32), torch.from_numpy(m).cuda(),
+                   dev("retained", torch.int32), dev("evicted", torch.int32), dev("strategy", torch.int32), match, sim, F.alloc_workspace(fp))
+    assert np.array_equal(match.cpu().numpy(), got["match"])
+    assert np.array_equal(sim.cpu().numpy().astype(np.float64), got["match_sim"])
