@@ -1,0 +1,175 @@
+// Full-prefill information flow (Eq. 6 and Eq. 7 over every query row) on the tensor cores, for bf16 inputs with
+// head_dim 128: one launch for the whole call.
+//
+// An item is 256 consecutive query rows of one query head (two accumulator halves of 128) against the keys up to its last
+// row.  Per row the softmax statistics are kept as in the first scoring pass, with the part of the exp-sum that falls on
+// keys of the other modality beside it (a word of 32 keys is of one modality nearly always: then it costs one comparison;
+// only mixed words go element by element).  At the end of an item the four column quarters of a row meet in shared memory
+// and a row's share cross / total is added up per warp, so nothing but four floats per half leaves the CTA.
+//
+// Bound by the epilogue: Hq L^2 / 2 exponentials per unit, a quarter of them as a polynomial on the FMA pipe, with four
+// warps per scheduler to cover the latencies (half of the issue slots used; TMA and MMA alone take half the time).  The
+// form before launched the statistics once per 128 query rows, with a join of all partial statistics after each: launches
+// of a few hundred items in one to three uneven rounds, 1190 us for 28 layers of 28 heads and 2176 tokens against 693 us.
+#pragma once
+#include "common.cuh"
+#include "score_tc.cuh"
+#include "tc_stream.cuh"
+
+namespace flowmm {
+
+struct FlowTcArgs {
+    const uint32_t *modbits;     // [U, mod_words] key modality, 32 keys per word
+    float *parts;                // [8 n_rp][U * Hq]: shares of (256-row block, half, 32-row quarter)
+    int *status;
+    int Hq, G, Hkv, L, n_rp, n_heads, mod_words, n_items;
+    int group_heads;             // query heads of a group of KV heads whose keys stay in L2 together
+    FastDiv by_group_items, by_group_heads, by_last_heads, by_g, by_hkv;   // exact divisions of item and head numbers
+    float scale_log2;
+};
+
+struct FlowItem { int u, h, head, rp; };       // head: query head of the unit
+// Item numbers run through the groups of KV heads; inside a group from the longest block of rows to the shortest.
+__device__ __forceinline__ FlowItem flow_item(const FlowTcArgs &A, int item) {
+    const int grp = (int)A.by_group_items.div(item), in = item - grp * (int)A.by_group_items.d;
+    const bool last = (grp + 1) * A.group_heads > A.n_heads;               // a last group of fewer heads
+    const int back = (int)(last ? A.by_last_heads.div(in) : A.by_group_heads.div(in));
+    const int hg = grp * A.group_heads + in - back * (int)(last ? A.by_last_heads.d : A.by_group_heads.d);
+    FlowItem f;
+    f.rp = A.n_rp - 1 - back;
+    const int uh = (int)A.by_g.div(hg);
+    f.u = (int)A.by_hkv.div(uh);
+    f.h = uh - f.u * A.Hkv;
+    f.head = hg - f.u * A.Hq;
+    return f;
+}
+
+__global__ void __launch_bounds__(tcs::kThreads, 1)
+flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, const FlowTcArgs A) {
+    using S = tcs::Big;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const S::Ctx c = S::setup(smem_raw, &q_map, &k_map, A.status, 0, 16);
+    if (!c.ok) return;
+    auto plan_of = [&](const FlowItem &f) {
+        tcs::TilePlan p;
+        const int lo = f.rp * tcs::kItemRows;
+        p.a1 = lo; p.a2 = f.head; p.a3 = f.u;
+        p.h1 = tcs::kRows; p.h2 = 0;
+        p.n_halves = lo + tcs::kRows < A.L ? 2 : 1;
+        p.b1 = 0; p.b2 = f.h; p.b3 = f.u; p.step1 = S::kCols; p.step2 = 0;
+        p.cols_total = min(A.L, lo + tcs::kItemRows);
+        p.cols_first = min(A.L, lo + tcs::kRows);            // the first half's rows end 128 keys earlier
+        p.n_tiles = f.rp + 1;
+        p.extra = nullptr;
+        return p;
+    };
+    auto plan = [&](int item) { return plan_of(flow_item(A, item)); };
+    if (c.warp == 0) {
+        if (c.lane == 0) S::producer(c, &q_map, &k_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
+    } else if (c.warp == 1) {
+        if (c.lane == 0) S::mma_issuer(c, A.n_items, plan, A.status);
+    } else {
+        // all sixteen warps drain one accumulator at a time: a warp owns 32 lanes x a quarter of the columns of both halves
+        const int row_in_half = c.quarter * 32 + c.lane, colq = (c.warp - 2) >> 2;
+        float *xch = reinterpret_cast<float *>(smem_raw + S::kSmemEpi);      // [3 values][2 halves][4 column quarters][128 rows]
+        int kh[2] = {0, 0};
+        bool ok = true;
+        FlowItem f_next;
+        uint32_t flip_next[2];                                       // modality words of this warp's 32 rows of each half
+        auto fetch_next = [&](int item) {
+            if (item >= A.n_items) return;
+            f_next = flow_item(A, item);
+            const uint32_t *w = A.modbits + (int64_t)f_next.u * A.mod_words + f_next.rp * (tcs::kItemRows / 32) + c.quarter;
+            flip_next[0] = w[0]; flip_next[1] = w[tcs::kRows / 32];
+        };
+        fetch_next(blockIdx.x);
+        for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x) {
+            const FlowItem f = f_next;
+            const tcs::TilePlan p = plan_of(f);
+            const int lo = f.rp * tcs::kItemRows;
+            const uint32_t *bits = A.modbits + (int64_t)f.u * A.mod_words;
+            float m[2] = {kNegBig, kNegBig}, l[2] = {0.f, 0.f}, lc[2] = {0.f, 0.f};
+            // all ones for a row of a visual token, whose other modality is the complement; fetched an item ahead
+            const uint32_t flip[2] = {((flip_next[0] >> c.lane) & 1u) ? 0xFFFFFFFFu : 0u, ((flip_next[1] >> c.lane) & 1u) ? 0xFFFFFFFFu : 0u};
+            fetch_next(item + gridDim.x);
+            for (int t = 0; ok && t < p.n_tiles; ++t) {
+                const int kb = t * S::kCols;
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    if (hf >= p.n_halves || !ok) continue;
+                    ok = S::acc_wait_h(c, hf, kh[hf]++, A.status);
+                    if (!ok) continue;
+                    // this warp's rows r0 .. r0 + 31 see the keys up to themselves: chunks past r0 + 31 are left out and
+                    // only the one on the diagonal is masked
+                    const int r0 = lo + hf * tcs::kRows + c.quarter * 32;
+                    const int ncols = min(S::kCols, min(r0 + 32, A.L) - kb);
+                    S::for_each_chunk_q(c, hf, colq, (ncols + 31) >> 5, [&](int ch, uint32_t (&acc)[32]) {
+                        const int k0 = kb + ch * 32;
+                        const uint32_t other = bits[k0 >> 5] ^ flip[hf];                 // keys of the other modality than the row's token
+                        float mx, add, addc = 0.f;
+                        if (k0 < r0) {                               // all 32 keys come before all 32 rows
+                            float raw[32];
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) raw[j] = __uint_as_float(acc[j]);
+                            mx = fmaxf(max32(raw) * A.scale_log2, m[hf]);
+                            add = exp_sum32(raw, A.scale_log2, mx);
+                            if (other == 0xFFFFFFFFu) addc = add;
+                            else if (other != 0u) {
+#pragma unroll
+                                for (int j = 0; j < 32; ++j)
+                                    addc += ((other >> j) & 1u) ? tc::ex2(fmaf(raw[j], A.scale_log2, -mx)) : 0.f;
+                            }
+                        } else {
+                            float s[32], add4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                            for (int j = 0; j < 32; ++j)
+                                s[j] = (j <= c.lane) ? __uint_as_float(acc[j]) * A.scale_log2 : kNegBig;
+                            mx = fmaxf(max32(s), m[hf]);
+#pragma unroll
+                            for (int j = 0; j < 32; ++j) {           // masked entries sit ~1e30 below: exp2 gives 0
+                                const float e = tc::ex2(s[j] - mx);
+                                add4[j & 3] += e;
+                                addc += ((other >> j) & 1u) ? e : 0.f;
+                            }
+                            add = (add4[0] + add4[1]) + (add4[2] + add4[3]);
+                        }
+                        const float carry = tc::ex2(m[hf] - mx);
+                        l[hf] = l[hf] * carry + add;
+                        lc[hf] = lc[hf] * carry + addc;
+                        m[hf] = mx;
+                    });
+                    S::acc_release_h(c, hf);
+                }
+            }
+            // The four column quarters of every row meet.  (After a wait that ran out the barriers are still kept, by all
+            // sixteen warps: the vote ends the loop for all of them together.)
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                float *x = xch + (hf * 4 + colq) * tcs::kRows + row_in_half;
+                x[0] = m[hf]; x[1024] = l[hf]; x[2048] = lc[hf];
+            }
+            ok = !S::epi_meet(!ok);
+            if (ok && colq < p.n_halves) {                           // column quarter 0 joins half 0, column quarter 1 half 1
+                const float *x = xch + colq * 4 * tcs::kRows + row_in_half;
+                const float mx = fmaxf(fmaxf(x[0], x[128]), fmaxf(x[256], x[384]));
+                float z = 0.f, zc = 0.f;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float w = tc::ex2(x[q * 128] - mx);
+                    z = fmaf(x[1024 + q * 128], w, z);
+                    zc = fmaf(x[2048 + q * 128], w, zc);
+                }
+                const bool row_on = lo + colq * tcs::kRows + row_in_half < A.L;
+                const float share = warp_sum(row_on && z > 0.f ? zc / z : 0.f);
+                if (c.lane == 0)
+                    A.parts[((int64_t)(f.rp * 2 + colq) * 4 + c.quarter) * (int64_t)A.n_heads + (int64_t)f.u * A.Hq + f.head] = share;
+            }
+            if (ok && p.n_halves == 1 && colq == 1 && c.lane == 0)   // no rows in the second half
+                A.parts[((int64_t)(f.rp * 2 + 1) * 4 + c.quarter) * (int64_t)A.n_heads + (int64_t)f.u * A.Hq + f.head] = 0.f;
+            S::epi_sync();                                           // the exchange may be overwritten again
+        }
+    }
+    S::teardown(c);
+}
+
+}  // namespace flowmm

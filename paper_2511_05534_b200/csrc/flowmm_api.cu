@@ -11,6 +11,7 @@
 #include "common.cuh"
 #include "decode.cuh"
 #include "decode_tc.cuh"
+#include "flow_tc.cuh"
 #include "match_small_tc.cuh"
 #include "merge_staged.cuh"
 #include "merge_tc.cuh"
@@ -87,7 +88,6 @@ constexpr int64_t kMaxHeadsPerCall = 1 << 22;
 // Where everything lives inside the caller's workspace.  One layout serves every entry point.
 struct Layout {
     size_t status, importance, cross_mass, rho, strategy, retained, evicted, match, match_sim;
-    size_t row_cross;          // flow-only statistics pass: the other-modality part of every partial row sum
     size_t row_part, cross_part, rn, sort_a, sort_b, mem_tok, mem_w, piece_desc, off, piece_off, part_off, partial, ticket, slot_done;
     size_t cand_k, cand_scale, cand_slot, cand_count, rank, tile_mod, negc;
     size_t tokmap;             // [UH, L] (slot, weight) of every token position, for the tensor-core merge
@@ -169,7 +169,6 @@ Layout make_layout(const flowmm_params &p) {
     const size_t max_chunk1 = (size_t)(y.n_chunk1 > 4 * y.tc_n_chunk ? y.n_chunk1 : 4 * y.tc_n_chunk);
     const size_t max_chunk2 = (size_t)(y.n_chunk2 > 8 * y.n_rt ? y.n_chunk2 : 8 * y.n_rt);
     y.row_part = take(U * Hq * W * max_chunk1 * 8);
-    y.row_cross = take(U * Hq * W * max_chunk1 * 4);
     y.cross_part = take(U * Hq * max_chunk2 * 4);
     y.negc = take(U * Hkv * (size_t)y.gw_pad * 4);
     y.rn = take(U * Hkv * L * 4);
@@ -875,45 +874,52 @@ flowmm_params flow_tile_params(const flowmm_params &p, const int64_t qs[3], int 
     return t;
 }
 
+int flow_parts_tc(int L) { return (L + tcs::kItemRows - 1) / tcs::kItemRows * 8; }
+
 struct FlowLayout { size_t std_bytes, mod, imp, parts, bits, total; };
 
-// One query tile of the full-prefill flow on the tensor cores: the statistics pass alone, with the row sums split by
-// key modality, then the per-head join.  `tp` is the tile's scoring problem (prompt cut after the tile, tile = window).
-flowmm_status run_flow_tile_tc(const flowmm_params &tp, const Layout &y, const void *q_tile, const void *k,
-                               const uint8_t *modality, int mod_pitch, const uint32_t *modbits, int mod_words,
-                               float *cross_out, void *ws, cudaStream_t st) {
-    const int UH = tp.n_units * tp.n_kv_heads, G = tp.n_q_heads / tp.n_kv_heads, W = tp.window;
-    ScoreTcArgs a = {};
-    a.row_part = at<float2>(ws, y.row_part); a.row_cross = at<float>(ws, y.row_cross); a.modality = modality;
-    a.modbits = modbits; a.mod_words = mod_words; a.mod_pitch = mod_pitch; a.status = at<int>(ws, y.status);
-    a.Hq = tp.n_q_heads; a.Hkv = tp.n_kv_heads; a.G = G; a.W = W; a.L = tp.seq_len; a.GW = G * W; a.GWpad = y.gw_pad;
-    a.n_qt = y.tc_n_qt; a.n_chunk = y.tc_n_chunk; a.tiles_per_chunk = y.tc_tiles_per_chunk; a.n_rt = y.n_rt;
-    a.a_heads = G < tcs::kRows / W ? G : tcs::kRows / W;
-    a.n_items1 = UH * a.n_qt * a.n_chunk;
-    const float scale = tp.softmax_scale != 0.f ? tp.softmax_scale : 1.f / sqrtf((float)tp.head_dim);
+// bf16 at head_dim 128: every query row in one launch (flow_tc.cuh).
+flowmm_status run_flow_tc(const flowmm_params &p, const void *q, const int64_t q_stride[3], const void *k, const uint32_t *modbits,
+                          int mod_words, float *parts, int *status, cudaStream_t st) {
+    FlowTcArgs a = {};
+    a.modbits = modbits; a.parts = parts; a.status = status;
+    a.Hq = p.n_q_heads; a.Hkv = p.n_kv_heads; a.G = p.n_q_heads / p.n_kv_heads; a.L = p.seq_len;
+    a.n_rp = (p.seq_len + tcs::kItemRows - 1) / tcs::kItemRows; a.n_heads = p.n_units * p.n_q_heads; a.mod_words = mod_words;
+    a.n_items = a.n_heads * a.n_rp;
+    const float scale = p.softmax_scale != 0.f ? p.softmax_scale : 1.f / sqrtf((float)p.head_dim);
     a.scale_log2 = scale * kLog2e;
+    // every block of rows reads its head's keys again: the keys of a group of heads take at most 48 MB of the 126 MB L2
+    const int64_t head_bytes = (int64_t)p.seq_len * 256, fit = (48ll << 20) / head_bytes;
+    const int n_uh = p.n_units * p.n_kv_heads, group = fit < 1 ? 1 : fit > n_uh ? n_uh : (int)fit;
+    a.group_heads = group * a.G;
+    a.by_group_items = make_fastdiv((uint32_t)(a.group_heads * a.n_rp)); a.by_group_heads = make_fastdiv((uint32_t)a.group_heads);
+    a.by_last_heads = make_fastdiv((uint32_t)(n_uh % group ? n_uh % group * a.G : a.group_heads));
+    a.by_g = make_fastdiv((uint32_t)a.G); a.by_hkv = make_fastdiv((uint32_t)p.n_kv_heads);
     CUtensorMap qa, k256;
-    const uint64_t qd[4] = {128, (uint64_t)W, (uint64_t)tp.n_q_heads, (uint64_t)tp.n_units};
-    const uint64_t qs[3] = {(uint64_t)tp.q_stride[2] * 2, (uint64_t)tp.q_stride[1] * 2, (uint64_t)tp.q_stride[0] * 2};
-    const uint64_t kd[4] = {128, (uint64_t)tp.seq_len, (uint64_t)tp.n_kv_heads, (uint64_t)tp.n_units};
-    const uint64_t ks[3] = {(uint64_t)tp.k_stride[2] * 2, (uint64_t)tp.k_stride[1] * 2, (uint64_t)tp.k_stride[0] * 2};
-    const uint32_t bqa[4] = {64, (uint32_t)W, (uint32_t)a.a_heads, 1}, bk256[4] = {64, tcs::Big::kCols, 1, 1};
-    if (!tc::make_bf16_map(&qa, q_tile, 4, qd, qs, bqa) || !tc::make_bf16_map(&k256, k, 4, kd, ks, bk256)) return FLOWMM_ERR_CUDA;
-    if (cudaFuncSetAttribute(score_stats_tc_kernel<tcs::Big, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tcs::Big::kSmemBytes) != cudaSuccess)
+    const uint64_t qd[4] = {128, (uint64_t)p.seq_len, (uint64_t)p.n_q_heads, (uint64_t)p.n_units};
+    const uint64_t qs[3] = {(uint64_t)q_stride[2] * 2, (uint64_t)q_stride[1] * 2, (uint64_t)q_stride[0] * 2};
+    const uint64_t kd[4] = {128, (uint64_t)p.seq_len, (uint64_t)p.n_kv_heads, (uint64_t)p.n_units};
+    const uint64_t ks[3] = {(uint64_t)p.k_stride[2] * 2, (uint64_t)p.k_stride[1] * 2, (uint64_t)p.k_stride[0] * 2};
+    const uint32_t bqa[4] = {64, tcs::kRows, 1, 1}, bk256[4] = {64, tcs::Big::kCols, 1, 1};
+    if (!tc::make_bf16_map(&qa, q, 4, qd, qs, bqa) || !tc::make_bf16_map(&k256, k, 4, kd, ks, bk256)) return FLOWMM_ERR_CUDA;
+    if (cudaFuncSetAttribute(flow_stats_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcs::Big::kSmemBytes) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
     const int sms = tc::sm_count();
-    launch(score_stats_tc_kernel<tcs::Big, true>, a.n_items1 < sms ? a.n_items1 : sms, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
+    launch(flow_stats_tc_kernel, a.n_items < sms ? a.n_items : sms, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
     FLOWMM_LAUNCHED("flow_stats_tc");
-    const int n_heads = tp.n_units * tp.n_q_heads;
-    launch(flow_combine_kernel, (n_heads + 7) / 8, 256, 0, st, a.row_part, a.row_cross, 4 * a.n_chunk, G, W, tp.n_kv_heads, n_heads, cross_out);
-    FLOWMM_LAUNCHED("flow_combine");
     return FLOWMM_OK;
 }
 
 FlowLayout flow_layout(const flowmm_params &p, const int64_t qs[3]) {
     FlowLayout f = {};
     const int n = flow_tiles(p.seq_len);
+    if (use_tc(p)) {
+        f.std_bytes = 256;                                               // the status word
+        f.parts = align256(f.std_bytes);
+        f.bits = f.parts + align256((size_t)flow_parts_tc(p.seq_len) * p.n_units * p.n_q_heads * 4);
+        f.total = f.bits + align256((size_t)p.n_units * ((p.seq_len + 31) / 32 + 8) * 4);
+        return f;
+    }
     for (int t = 0; t < n; ++t) {
         int lo, hi;
         flow_tile(p.seq_len, t, lo, hi);
@@ -924,7 +930,6 @@ FlowLayout flow_layout(const flowmm_params &p, const int64_t qs[3]) {
     f.mod = o; o += align256((size_t)p.n_units * p.seq_len);
     f.imp = o; o += align256((size_t)p.n_units * p.n_kv_heads * p.seq_len * 4);
     f.parts = o; o += align256((size_t)n * p.n_units * p.n_q_heads * 4);
-    f.bits = o; o += align256((size_t)p.n_units * ((p.seq_len + 31) / 32 + 8) * 4);
     f.total = o;
     return f;
 }
@@ -960,34 +965,34 @@ extern "C" flowmm_status flowmm_full_flow(const flowmm_params *p, const void *q_
     if (ws_bytes < f.total) return FLOWMM_ERR_WORKSPACE;
     FLOWMM_TRY(check_device());
     if (cudaMemsetAsync(ws, 0, 4, st) != cudaSuccess) return FLOWMM_ERR_CUDA;       // the status word
-    const int n_tiles = flow_tiles(p->seq_len), n = p->n_units * p->n_q_heads;
-    const size_t esize = p->dtype == FLOWMM_BF16 ? 2 : 4;
-    uint8_t *mod = at<uint8_t>(ws, f.mod);
-    float *imp = at<float>(ws, f.imp), *parts = at<float>(ws, f.parts);
-    uint32_t *bits = at<uint32_t>(ws, f.bits);
-    const int mod_words = (p->seq_len + 31) / 32 + 8;                  // + slack: whole 256-key tiles are indexed
+    int n_tiles = flow_tiles(p->seq_len);
+    const int n = p->n_units * p->n_q_heads;
+    float *parts = at<float>(ws, f.parts);
     if (use_tc(*p)) {
+        const int mod_words = (p->seq_len + 31) / 32 + 8;              // + slack: whole 256-key tiles are indexed
+        uint32_t *bits = at<uint32_t>(ws, f.bits);
         launch(pack_modality_kernel, dim3(p->n_units, (mod_words + 7) / 8), 256, 0, st, modality, p->seq_len, mod_words, bits);
         FLOWMM_LAUNCHED("pack_modality");
-    }
-    for (int t = 0; t < n_tiles; ++t) {
-        int lo, hi;
-        flow_tile(p->seq_len, t, lo, hi);
-        const flowmm_params tp = flow_tile_params(*p, q_full_stride, lo, hi);
-        const Layout y = make_layout(tp);
-        const char *q_tile_tc = static_cast<const char *>(q_full) + (size_t)lo * (size_t)q_full_stride[2] * esize;
-        if (use_tc_score(tp)) {            // full tiles on the tensor cores: one pass, no importance
-            FLOWMM_TRY(run_flow_tile_tc(tp, y, q_tile_tc, k, modality, p->seq_len, bits, mod_words, parts + (size_t)t * n, ws, st));
-            continue;
+        FLOWMM_TRY(run_flow_tc(*p, q_full, q_full_stride, k, bits, mod_words, parts, static_cast<int *>(ws), st));
+        n_tiles = flow_parts_tc(p->seq_len);
+    } else {
+        const size_t esize = p->dtype == FLOWMM_BF16 ? 2 : 4;
+        uint8_t *mod = at<uint8_t>(ws, f.mod);
+        float *imp = at<float>(ws, f.imp);
+        for (int t = 0; t < n_tiles; ++t) {
+            int lo, hi;
+            flow_tile(p->seq_len, t, lo, hi);
+            const flowmm_params tp = flow_tile_params(*p, q_full_stride, lo, hi);
+            const Layout y = make_layout(tp);
+            // the scoring kernels index the modality map with the cut prompt's length as the row pitch
+            if (cudaMemcpy2DAsync(mod, (size_t)hi, modality, (size_t)p->seq_len, (size_t)hi, (size_t)p->n_units,
+                                  cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+                return FLOWMM_ERR_CUDA;
+            const char *q_tile = static_cast<const char *>(q_full) + (size_t)lo * (size_t)q_full_stride[2] * esize;
+            FLOWMM_TRY(run_score(tp, y, q_tile, k, mod, imp, parts + (size_t)t * n, ws, st));
         }
-        // the scoring kernels index the modality map with the cut prompt's length as the row pitch
-        if (cudaMemcpy2DAsync(mod, (size_t)hi, modality, (size_t)p->seq_len, (size_t)hi, (size_t)p->n_units,
-                              cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-            return FLOWMM_ERR_CUDA;
-        const char *q_tile = static_cast<const char *>(q_full) + (size_t)lo * (size_t)q_full_stride[2] * esize;
-        FLOWMM_TRY(run_score(tp, y, q_tile, k, mod, imp, parts + (size_t)t * n, ws, st));
     }
-    launch(full_flow_reduce_kernel, p->n_units, 64, 0, st, parts, n_tiles, n, p->n_q_heads, p->seq_len, p->theta, p->flow_mode,
+    launch(full_flow_reduce_kernel, p->n_units, 1024, 0, st, parts, n_tiles, n, p->n_q_heads, p->seq_len, p->theta, p->flow_mode,
                                                        cross_mass, rho, strategy);
     FLOWMM_LAUNCHED("full_flow_reduce");
     return FLOWMM_OK;

@@ -262,24 +262,27 @@ __global__ void layer_flow_kernel(const float *cross_mass, int U, int Hq, int W,
     strategy[u] = flow_mode == 1 ? 0 : flow_mode == 2 ? 1 : ((r > theta) != (flow_mode == 3) ? 1 : 0);
 }
 
-// Full-prefill flow: per-head masses of the query tiles added up in tile order, then Eq. 6 over all L rows
-// and the theta rule.  parts [n_tiles][U * Hq]; one block per unit, one thread per query head.
-__global__ void full_flow_reduce_kernel(const float *parts, int n_tiles, int n, int Hq, int L, float theta, int flow_mode,
+// Full-prefill flow: the parts of every head's mass added up (lanes take parts with a stride of 32, then a shuffle tree:
+// a fixed order), then Eq. 6 over all L rows and the theta rule.  parts [n_parts][U * Hq]; one block per unit, a warp per head.
+__global__ void full_flow_reduce_kernel(const float *parts, int n_parts, int n, int Hq, int L, float theta, int flow_mode,
                                         float *cross_mass, float *rho, int *strategy) {
     predecessor_done();
-    const int u = blockIdx.x;
-    for (int g = threadIdx.x; g < Hq; g += blockDim.x) {
+    const int u = blockIdx.x, lane = lane_id();
+    for (int g = threadIdx.x >> 5; g < Hq; g += blockDim.x >> 5) {
         float s = 0.f;
-        for (int t = 0; t < n_tiles; ++t) s += parts[(int64_t)t * n + (int64_t)u * Hq + g];
-        cross_mass[(int64_t)u * Hq + g] = s;
+        for (int t = lane; t < n_parts; t += 32) s += parts[(int64_t)t * n + (int64_t)u * Hq + g];
+        s = warp_sum(s);
+        if (lane == 0) cross_mass[(int64_t)u * Hq + g] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
         float s = 0.f;
-        for (int g = 0; g < Hq; ++g) s += cross_mass[(int64_t)u * Hq + g] / (float)L;   // a head's total mass is L
-        const float r = s / (float)Hq;
-        if (rho) rho[u] = r;
-        strategy[u] = flow_mode == 1 ? 0 : flow_mode == 2 ? 1 : ((r > theta) != (flow_mode == 3) ? 1 : 0);
+        for (int g = lane; g < Hq; g += 32) s += cross_mass[(int64_t)u * Hq + g] / (float)L;   // a head's total mass is L
+        const float r = warp_sum(s) / (float)Hq;
+        if (lane == 0) {
+            if (rho) rho[u] = r;
+            strategy[u] = flow_mode == 1 ? 0 : flow_mode == 2 ? 1 : ((r > theta) != (flow_mode == 3) ? 1 : 0);
+        }
     }
 }
 

@@ -41,6 +41,7 @@ struct TilePlan {
     int step1, step2;          // B origin advance per tile along c1 / c2
     int n_tiles;               // 0: every role skips the item
     int cols_total;            // valid B rows over all tiles (tile t has min(NB, cols_total - NB t))
+    int cols_first = 0;        // ... for A half 0, where it needs fewer in the last tile (0: the same)
     const float *extra;        // nullptr, or NB fp32 per-column constants per tile: tile t reads extra + NB t
     __device__ __forceinline__ bool empty() const { return n_tiles == 0 || n_halves == 0; }
 };
@@ -194,7 +195,7 @@ struct Skel {
                 ok = tc::mbar_wait(c.bar(kBarBFull + sb), (bt >> 1) & 1, c.abort_flag, status);
                 if (!ok) break;
                 const int ncols = min(NB, p.cols_total - t * NB);
-                const uint32_t idesc = tc::idesc_bf16(kRows, (uint32_t)((ncols + 15) & ~15));
+                const int ncols0 = p.cols_first ? min(NB, p.cols_first - t * NB) : ncols;
                 const uint32_t b_base = c.base + kSmemB + sb * kBStage;
                 for (int h = 0; ok && h < p.n_halves; ++h) {
                     const int st = ia[h] % AST;
@@ -203,6 +204,7 @@ struct Skel {
                     if (!ok) break;
                     tc::tc_fence_after();
                     const uint32_t a_base = c.base + kSmemA + (uint32_t)(st * 2 + h) * kAHalf;
+                    const uint32_t idesc = tc::idesc_bf16(kRows, (uint32_t)(((h == 0 ? ncols0 : ncols) + 15) & ~15));
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks) {                     // head_dim 128 = 8 K slices of 16
                         const uint32_t a_off = (ks >> 2) * (kAHalf / 2) + (ks & 3) * 32;
@@ -301,7 +303,21 @@ struct Skel {
             f(ch, a);
         }
     }
-    // The same meeting point with a vote: returns whether either warp has given up on a wait, so that both leave
+    // Meeting points of all sixteen epilogue warps; the first with a vote: whether any of them has given up on a wait.
+    static __device__ __forceinline__ bool epi_meet(bool gave_up) {
+        uint32_t any;
+        asm volatile(
+            "{\n\t.reg .pred p, q;\n\t"
+            "setp.ne.u32 q, %1, 0;\n\t"
+            "barrier.cta.red.or.pred p, 1, %2, q;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(any)
+            : "r"((uint32_t)gave_up), "n"(32 * kEpiWarps)
+            : "memory");
+        return any != 0;
+    }
+    static __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory"); }
+    // Meeting point of the two warps that share rows, with a vote: returns whether either warp has given up on a wait, so that both leave
     // the item loop together and neither is left alone at the next meeting.
     static __device__ __forceinline__ bool pair_meet(const Ctx &c, bool gave_up) {
         uint32_t any;

@@ -91,3 +91,28 @@ def test_video_shaped_prompt_at_full_length():
     assert np.allclose(g_rho, rho, atol=1e-4)
     if abs(rho[0] - wl.theta) > 1e-4:
         assert g_strat[0] == strat[0]
+
+
+@pytest.mark.parametrize("L", [8200, 8448])
+def test_heads_in_several_groups_equal_the_units_alone(L):
+    """26 KV heads of this length do not share the L2 at once: the items go by groups of heads, the last one smaller.
+    Every unit must come out as in a call of its own, bit for bit."""
+    U, Hq, Hkv, D = 13, 4, 2, 128
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(L)
+    q = torch.randn((U, Hq, L, D), generator=gen, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn((U, Hkv, L, D), generator=gen, device="cuda", dtype=torch.bfloat16)
+    m = (torch.rand((U, L), generator=gen, device="cuda") < 0.5).to(torch.uint8)
+
+    def run(lo, hi):
+        fp = F.Params(hi - lo, Hq, Hkv, D, L, 1, 1, theta=0.4)
+        cross, rho = torch.zeros((hi - lo, Hq), device="cuda"), torch.zeros((hi - lo,), device="cuda")
+        strat = torch.zeros((hi - lo,), dtype=torch.int32, device="cuda")
+        ws = torch.zeros(F.flowmm_full_flow_workspace_bytes(fp), dtype=torch.uint8, device="cuda")
+        F.flowmm_full_flow(fp, q[lo:hi], k[lo:hi], m[lo:hi], cross, rho, strat, ws)
+        assert F.flowmm_last_device_status(ws) == 0
+        return cross, rho
+    cross, rho = run(0, U)
+    for u in (0, 10, 11, 12):
+        c1, r1 = run(u, u + 1)
+        assert torch.equal(cross[u], c1[0]) and torch.equal(rho[u], r1[0])
