@@ -14,6 +14,7 @@ struct DecodeArgs {
     const void *q, *k, *v;       // q [U, Hq, D] dense
     float *part;                 // [UH, n_split, G, D + 2]: unnormalised output, running max (log2), exp-sum
     float *out;                  // [U, Hq, D]
+    int *status;                 // device status word, cleared here
     int Hq, Hkv, G, N, n_split, keys_per_split;
     float scale_log2;
     int64_t ks[3], vs[3];
@@ -34,6 +35,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const Decod
     extern __shared__ float dec_smem[];                              // [GROUPS][GP][D + 2]
     predecessor_done();
     const int tid = threadIdx.x, sub = tid % LPR, grp = tid / LPR;
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *A.status = 0;
     const int uh = blockIdx.x, u = uh / A.Hkv, h = uh % A.Hkv;
     const int lo = blockIdx.y * A.keys_per_split, hi = min(A.N, lo + A.keys_per_split);
     const T *kb = static_cast<const T *>(A.k) + u * A.ks[0] + h * A.ks[1] + sub * V;
@@ -135,23 +137,38 @@ __global__ void __launch_bounds__(kDecThreads) decode_partial_kernel(const Decod
     }
 }
 
-// grid = U*Hq, block = D: joins the key ranges of one query head and normalises.
+// grid = U*Hq, block = 4 D: joins the key ranges of one query head and normalises.  Each quarter of the block takes a
+// quarter of the ranges, so that a long cache's few hundred records are read 4 x 8 at a time.
+constexpr int kCombineParts = 4;
 template <int D>
-__global__ void __launch_bounds__(D) decode_combine_kernel(const DecodeArgs A) {
+__global__ void __launch_bounds__(kCombineParts * D) decode_combine_kernel(const DecodeArgs A) {
+    __shared__ float red[kCombineParts * D / 32], acc[kCombineParts][D], sums[kCombineParts];
+    const int ug = blockIdx.x, u = ug / A.Hq, gq = ug % A.Hq, h = gq / A.G, g = gq % A.G;
+    const int d = threadIdx.x % D, part = threadIdx.x / D;
+    const int64_t step = (int64_t)A.G * (D + 2);
+    const float *rec = A.part + (((int64_t)u * A.Hkv + h) * A.n_split * A.G + g) * (D + 2);
     predecessor_done();
-    const int ug = blockIdx.x, u = ug / A.Hq, gq = ug % A.Hq, h = gq / A.G, g = gq % A.G, d = threadIdx.x;
-    const int uh = u * A.Hkv + h;
     float mx = kNegBig;
-    for (int sp = 0; sp < A.n_split; ++sp)
-        mx = fmaxf(mx, A.part[(((int64_t)uh * A.n_split + sp) * A.G + g) * (D + 2) + D]);
+    for (int sp = threadIdx.x; sp < A.n_split; sp += kCombineParts * D) mx = fmaxf(mx, rec[sp * step + D]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    if (lane_id() == 0) red[threadIdx.x >> 5] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kCombineParts * D / 32; ++w) mx = fmaxf(mx, red[w]);
+    const int per = (A.n_split + kCombineParts - 1) / kCombineParts, lo = part * per, hi = min(A.n_split, lo + per);
     float o = 0.f, ls = 0.f;
-    for (int sp = 0; sp < A.n_split; ++sp) {
-        const float *rec = A.part + (((int64_t)uh * A.n_split + sp) * A.G + g) * (D + 2);
-        const float w = dec_ex2(rec[D] - mx);
-        o = fmaf(rec[d], w, o);
-        ls = fmaf(rec[D + 1], w, ls);
+#pragma unroll 8
+    for (int sp = lo; sp < hi; ++sp) {
+        const float w = dec_ex2(rec[sp * step + D] - mx);
+        o = fmaf(rec[sp * step + d], w, o);
+        ls = fmaf(rec[sp * step + D + 1], w, ls);
     }
-    A.out[(int64_t)ug * D + d] = o / ls;
+    acc[part][d] = o;
+    if (d == 0) sums[part] = ls;
+    __syncthreads();
+    if (part != 0) return;
+    A.out[(int64_t)ug * D + d] = (acc[0][d] + acc[1][d] + acc[2][d] + acc[3][d]) / (sums[0] + sums[1] + sums[2] + sums[3]);
 }
 
 }  // namespace flowmm

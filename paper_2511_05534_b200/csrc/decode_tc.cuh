@@ -11,9 +11,11 @@
 //             contraction over the tile's keys; a head's output is the sum of its two columns.  The V tile is the same swizzled
 //             shared-memory tile a K tile is, read the other way round (MN-major operand), so V needs no
 //             transposition.  O never needs rescaling because the maximum is already final.
-// A head with one range is normalised and written at once.  Otherwise the CTA writes its unnormalised
-// output, its maximum and its sum of weights, and whichever range of a head finishes last (a ticket per
-// head) joins them all; the records it reads are L2-resident.
+// A head with one range is normalised and written at once.  Two to eight ranges are a cluster: every CTA leaves its
+// unnormalised output, maximum and sum of weights in its shared memory, and after a cluster barrier the CTAs join a share
+// of the heads each.  With more ranges the CTA writes its record to global memory and decode_combine_kernel joins them, a
+// block per query head.  (One layer of 4 KV heads: 218 keys 12.4 us when the range that finished last joined all of them,
+// found by tickets that a memset had to clear first, 6.2 us as clusters of two.)
 // Roles: warp 0 lane 0 streams K tiles then V tiles through a three-stage TMA ring, warp 1 lane 0 issues
 // the MMAs, warps 2-5 (one thread per key of a tile / per output dim) do the softmax and the output.
 // Two CTAs fit an SM (256 TMEM columns, about 109 KB of shared memory each), so one streams while the
@@ -31,14 +33,13 @@ constexpr int kHeads = 16;                  // N of both contractions
 constexpr int kMaxHeads = 8;                // query heads per KV head this kernel serves
 constexpr int kMaxTiles = 15;               // 16 TMEM columns for O + 16 per score tile = 256
 constexpr int kTmemCols = 256;
-constexpr int kMaxJoin = 8192;               // (range, head) records the joining CTA can stage: ranges per head x heads
 constexpr int kThreads = 192;
 constexpr uint32_t kStageBytes = kTile * 128 * 2;            // both 64-element panels of a 128-row tile
 constexpr uint32_t kPanel = kStageBytes / 2;
 constexpr uint32_t kSmallPanel = kHeads * 128;               // 16 rows x 128 bytes
 constexpr uint32_t kSmemQ = kStages * kStageBytes;           // Q operand: two panels of 16 rows
 constexpr uint32_t kSmemP = kSmemQ + 2 * kSmallPanel;        // two P buffers of the same shape
-constexpr uint32_t kSmemRed = kSmemP + 4 * kSmallPanel;      // float [4 warps][8 heads], then the last-range flag
+constexpr uint32_t kSmemRed = kSmemP + 4 * kSmallPanel;      // float [4 warps][8 heads]
 constexpr uint32_t kSmemBar = kSmemRed + 256;
 constexpr int kBarFull = 0, kBarEmpty = kStages, kBarQ = 2 * kStages, kBarS = kBarQ + 1 /* one per score tile */,
               kBarPFull = kBarS + kMaxTiles, kBarPEmpty = kBarPFull + 2, kBarO = kBarPEmpty + 2, kNumBars = kBarO + 1;
@@ -48,11 +49,23 @@ struct Args {
     const __nv_bfloat16 *q;     // [U, Hq, 128] dense
     float *part;                // [UH, n_split, G, 130]: unnormalised output, maximum (log2 domain), sum of weights
     float *out;                 // [U, Hq, 128]
-    int *tickets;               // [UH], zero on entry and on exit: how many ranges of the head have finished
     int *status;
     int Hq, Hkv, G, N, n_split, tiles_per_split;
     float scale_log2;
+    int clustered;              // the ranges of a head are one cluster
 };
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// a float in the shared memory of the cluster's CTA `rank`, at this CTA's shared address `addr`
+__device__ __forceinline__ float ld_cluster(uint32_t addr, int rank) {
+    uint32_t remote;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(remote) : "memory");
+    return v;
+}
 
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
@@ -103,6 +116,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     predecessor_done();
+    // the status word starts at zero (a wait that runs out reports two seconds after this at the earliest)
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *A.status = 0;
 
     const int uh = blockIdx.x, u = uh / A.Hkv, h = uh % A.Hkv, split = blockIdx.y;
     const int tiles_total = (A.N + kTile - 1) / kTile;
@@ -249,6 +264,16 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
                 if (g < G && ok)
                     out[g * 128] = (__uint_as_float(r[g]) + __uint_as_float(r[kMaxHeads + g])) /
                                    (red[g] + red[kMaxHeads + g] + red[2 * kMaxHeads + g] + red[3 * kMaxHeads + g]);
+        } else if (A.clustered) {                                    // record: output [8][128], then maxima, sums (the tile stages are idle by now)
+            float *rec = reinterpret_cast<float *>(dtc_smem);
+#pragma unroll
+            for (int g = 0; g < kMaxHeads; ++g) {
+                if (g < G) rec[g * 128 + row] = __uint_as_float(r[g]) + __uint_as_float(r[kMaxHeads + g]);
+                if (e == g && g < G) {
+                    rec[kMaxHeads * 128 + g] = mref[g];
+                    rec[kMaxHeads * 128 + kMaxHeads + g] = red[g] + red[kMaxHeads + g] + red[2 * kMaxHeads + g] + red[3 * kMaxHeads + g];
+                }
+            }
         } else {
             float *dst = A.part + ((int64_t)uh * A.n_split + split) * G * 130;
 #pragma unroll
@@ -259,55 +284,31 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
                     dst[g * 130 + 129] = red[g] + red[kMaxHeads + g] + red[2 * kMaxHeads + g] + red[3 * kMaxHeads + g];
                 }
             }
-            // the range that finishes last joins all ranges of its head
-            __threadfence();
-            epi_sync();
-            int *last = reinterpret_cast<int *>(red + 4 * kMaxHeads);
-            if (e == 0) {
-                const int done = atomicAdd(A.tickets + uh, 1);
-                *last = done == A.n_split - 1;
-                if (*last) A.tickets[uh] = 0;                        // ready for the next call
-            }
-            epi_sync();
-            if (*last && *abort_flag == 0) {        // both the same for all 128 threads: the barrier below is safe
-                __threadfence();
-                // maxima and sums of every (range, head) go through shared memory (the tile stages are idle by
-                // now), so that the long loop below is over independent loads only
-                const float *rec0 = A.part + (int64_t)uh * A.n_split * G * 130;
-                float *sm_m = reinterpret_cast<float *>(dtc_smem), *sm_l = sm_m + kMaxJoin;
-                const int n_rec = A.n_split * G;
-                for (int i = e; i < n_rec; i += 128) {
-                    sm_m[i] = __ldcg(rec0 + (int64_t)i * 130 + 128);
-                    sm_l[i] = __ldcg(rec0 + (int64_t)i * 130 + 129);
-                }
-                epi_sync();
-                float m[kMaxHeads], o[kMaxHeads], ls[kMaxHeads];
-#pragma unroll
-                for (int g = 0; g < kMaxHeads; ++g) {
-                    m[g] = kNegBig; o[g] = 0.f; ls[g] = 0.f;
-                    if (g < G)
-                        for (int sp = 0; sp < A.n_split; ++sp) m[g] = fmaxf(m[g], sm_m[sp * G + g]);
-                }
-#pragma unroll 2
-                for (int sp = 0; sp < A.n_split; ++sp) {             // all heads of two ranges in flight at a time
-#pragma unroll
-                    for (int g = 0; g < kMaxHeads; ++g)
-                        if (g < G) {
-                            const float w = tc::ex2(sm_m[sp * G + g] - m[g]);
-                            o[g] = fmaf(__ldcg(rec0 + ((int64_t)sp * G + g) * 130 + row), w, o[g]);
-                            ls[g] = fmaf(sm_l[sp * G + g], w, ls[g]);
-                        }
-                }
-#pragma unroll
-                for (int g = 0; g < kMaxHeads; ++g)
-                    if (g < G) out[g * 128] = o[g] / ls[g];
-            }
         }
     }
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     if (warp == 1) tc::tmem_dealloc(tmem, kTmemCols);
+    if (A.clustered) {                                               // (also after a wait that ran out: every thread of the cluster comes here)
+        __syncwarp();
+        cluster_sync();
+        if (threadIdx.x >= 64 && *abort_flag == 0) {
+            const int d = threadIdx.x - 64;
+            for (int g = split; g < A.G; g += A.n_split) {           // this CTA's share of the heads, thread = output dim
+                float mx = kNegBig, o = 0.f, ls = 0.f;
+                for (int sp = 0; sp < A.n_split; ++sp) mx = fmaxf(mx, ld_cluster(base + 4 * (kMaxHeads * 128 + g), sp));
+                for (int sp = 0; sp < A.n_split; ++sp) {
+                    const float w = tc::ex2(ld_cluster(base + 4 * (kMaxHeads * 128 + g), sp) - mx);
+                    o = fmaf(ld_cluster(base + 4 * (g * 128 + d), sp), w, o);
+                    ls = fmaf(ld_cluster(base + 4 * (kMaxHeads * 128 + kMaxHeads + g), sp), w, ls);
+                }
+                A.out[((int64_t)u * A.Hq + h * A.G + g) * 128 + d] = o / ls;
+            }
+        }
+        __syncwarp();
+        cluster_sync();                                              // nobody's shared memory goes away while it is read
+    }
 }
 
 }  // namespace dtc

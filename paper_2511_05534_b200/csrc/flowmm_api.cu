@@ -56,14 +56,20 @@ inline void profile_mark(const char *name, cudaStream_t st) {
 // costs 2 us less than with a plain launch (13 launches of a re-compression: 163 to 135 us) and the host no more.  An
 // error stays in cudaGetLastError() for FLOWMM_LAUNCHED.
 template <typename... Params, typename... Args>
-void launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
+void launch_cluster(dim3 cluster, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster.x; attr[1].val.clusterDim.y = cluster.y; attr[1].val.clusterDim.z = cluster.z;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cfg.attrs = &attr; cfg.numAttrs = 1;
+    cfg.attrs = attr; cfg.numAttrs = cluster.x * cluster.y * cluster.z > 1 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+template <typename... Params, typename... Args>
+void launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
+    launch_cluster(dim3(1), kernel, grid, block, smem, st, args...);
 }
 
 #define FLOWMM_LAUNCHED(name)                                          \
@@ -1014,32 +1020,36 @@ flowmm_status validate_decode(const flowmm_decode_params *p) {
 }
 
 // How a call is cut into key ranges, and where its scratch lives:
-// [status word, 256 bytes][one ticket per (unit, KV head)][partial records].
+// [status word, 256 bytes][partial records].
 struct DecodePlan {
     bool tc;                 // tensor-core kernel (bf16, head_dim 128) or the SIMT one
     int n_split, per_split;  // ranges per (unit, KV head); keys (SIMT) or 128-key tiles (tensor core) per range
     size_t part_off, bytes;
 };
 
+constexpr int kMaxDecodeCluster = 8;         // ranges of a head that are joined as one cluster (the portable cluster size)
+
 DecodePlan decode_plan(const flowmm_decode_params &p) {
     DecodePlan d;
     const int uh = p.n_units * p.n_kv_heads, g = p.n_q_heads / p.n_kv_heads;
     d.tc = p.dtype == FLOWMM_BF16 && p.head_dim == 128 && p.path != FLOWMM_PATH_SIMT;
     if (d.tc) {
-        // Two CTAs share an SM.  Of the range lengths TMEM allows, take the one with the least work per CTA
-        // slot when the CTAs run in rounds; a CTA's fixed cost (set-up, the pause between its two phases)
-        // counts like a tile and a half.
+        // Two CTAs share an SM.  Of the range lengths TMEM allows, take the one with the least work per CTA slot: rounds of
+        // CTAs (a last one that is nearly empty counts half when there are several) times a CTA's tiles and its fixed cost
+        // (set-up, the pause between its two phases: like a tile and a half), and for joining the ranges a tile and a half
+        // as a cluster or two and a half as a launch of its own.  Measured over 16 shapes from 4 heads of 218 keys to 640
+        // of 1690 the choice is within 11 % of the best length.
         const int tiles = (p.n_keys + dtc::kTile - 1) / dtc::kTile;
-        const int64_t slots = 2 * (int64_t)tc::sm_count();
+        const double slots = 2.0 * tc::sm_count();
         double best = 0.0;
         d.per_split = 1;
         for (int per = 1; per <= dtc::kMaxTiles && per <= tiles; ++per) {
-            const int64_t ctas = (int64_t)uh * ((tiles + per - 1) / per);
-            const double cost = (double)((ctas + slots - 1) / slots) * (per + 1.5);
+            const int64_t splits = (tiles + per - 1) / per;
+            const double full = (double)(uh * splits) / slots, rounds = fmax(1.0, fmin(ceil(full), full + 0.5));
+            const double cost = rounds * (per + 1.5) + (splits == 1 ? 0.0 : splits <= kMaxDecodeCluster ? 1.5 : 2.5);
             if (per == 1 || cost < best) { best = cost; d.per_split = per; }
         }
         d.n_split = (tiles + d.per_split - 1) / d.per_split;
-        if ((int64_t)d.n_split * g > dtc::kMaxJoin) d.tc = false;      // more ranges than the joining CTA can stage
     }
     if (!d.tc) {
         // enough CTAs for about four per SM, at least 64 keys each
@@ -1049,7 +1059,7 @@ DecodePlan decode_plan(const flowmm_decode_params &p) {
         d.per_split = (p.n_keys + want - 1) / want;
         d.n_split = (p.n_keys + d.per_split - 1) / d.per_split;
     }
-    d.part_off = 256 + align256((size_t)uh * sizeof(int));
+    d.part_off = 256;
     d.bytes = d.part_off + align256((size_t)uh * d.n_split * g * (p.head_dim + 2) * sizeof(float));
     return d;
 }
@@ -1067,7 +1077,7 @@ flowmm_status launch_decode(const DecodeArgs &a, int uh, int n_q, cudaStream_t s
         default: launch(decode_partial_kernel<T, D, 8>, grid, kDecThreads, smem, st, a); break;
     }
     FLOWMM_LAUNCHED("decode_partial");
-    launch(decode_combine_kernel<D>, n_q, D, 0, st, a);
+    launch(decode_combine_kernel<D>, n_q, kCombineParts * D, 0, st, a);
     FLOWMM_LAUNCHED("decode_combine");
     return FLOWMM_OK;
 }
@@ -1088,11 +1098,14 @@ flowmm_status launch_decode_tc(const flowmm_decode_params &p, const DecodeArgs &
         return FLOWMM_ERR_CUDA;
     dtc::Args t;
     t.q = static_cast<const __nv_bfloat16 *>(a.q); t.part = a.part; t.out = a.out; t.status = status;
-    t.tickets = status + 64;
     t.Hq = a.Hq; t.Hkv = a.Hkv; t.G = a.G; t.N = a.N; t.n_split = a.n_split; t.tiles_per_split = a.keys_per_split;
     t.scale_log2 = a.scale_log2;
-    launch(dtc::decode_tc_kernel, dim3(uh, a.n_split), dtc::kThreads, dtc::kSmemBytes, st, kmap, vmap, t);
+    t.clustered = a.n_split > 1 && a.n_split <= kMaxDecodeCluster;
+    launch_cluster(dim3(1, t.clustered ? a.n_split : 1), dtc::decode_tc_kernel, dim3(uh, a.n_split), dtc::kThreads, dtc::kSmemBytes, st, kmap, vmap, t);
     FLOWMM_LAUNCHED("decode_tc");
+    if (a.n_split <= kMaxDecodeCluster) return FLOWMM_OK;
+    launch(decode_combine_kernel<128>, p.n_units * p.n_q_heads, kCombineParts * 128, 0, st, a);
+    FLOWMM_LAUNCHED("decode_combine");
     return FLOWMM_OK;
 }
 
@@ -1118,8 +1131,8 @@ extern "C" flowmm_status flowmm_decode_attention(const flowmm_decode_params *p, 
     const DecodePlan plan = decode_plan(*p);
     if (ws_bytes < plan.bytes) return FLOWMM_ERR_WORKSPACE;
     FLOWMM_TRY(check_device());
-    if (cudaMemsetAsync(ws, 0, plan.part_off, st) != cudaSuccess) return FLOWMM_ERR_CUDA;   // status word and tickets
     DecodeArgs a;
+    a.status = static_cast<int *>(ws);                               // (cleared by the kernel)
     a.q = q; a.k = k; a.v = v; a.part = reinterpret_cast<float *>(static_cast<char *>(ws) + plan.part_off); a.out = out;
     a.Hq = p->n_q_heads; a.Hkv = p->n_kv_heads; a.G = p->n_q_heads / p->n_kv_heads; a.N = p->n_keys;
     a.n_split = plan.n_split; a.keys_per_split = plan.per_split;

@@ -110,3 +110,23 @@ def test_whole_stack_in_the_timed_configuration(name, permille):
                                  v[u:u + 1].float().cpu().numpy())
         got = out[u:u + 1].cpu().numpy()
         assert np.allclose(got, ref, rtol=RTOL, atol=ATOL), (u, np.abs(got - ref).max())
+
+
+@pytest.mark.parametrize("U,Hq,Hkv,N", [(1, 28, 4, 128), (1, 28, 4, 129), (1, 7, 1, 1024), (1, 8, 1, 1025), (1, 6, 2, 1153), (1, 4, 4, 3000),
+                                        (1, 8, 1, 15361), (1, 8, 1, 16000), (60, 5, 5, 300), (40, 64, 8, 1000)])
+def test_one_range_cluster_and_tickets(U, Hq, Hkv, N):
+    """Key counts around the switch points of how a head's ranges are joined: one range, a cluster of two to eight, tickets.
+    Called twice on one workspace that starts with garbage."""
+    rng = np.random.default_rng(N)
+    q = inputs.round_to_bf16(rng.standard_normal((U, Hq, 128)).astype(np.float32))
+    k = inputs.round_to_bf16(rng.standard_normal((U, Hkv, N, 128)).astype(np.float32))
+    v = inputs.round_to_bf16(rng.standard_normal((U, Hkv, N, 128)).astype(np.float32))
+    qd, kd, vd = to_dev(q, F.BF16), to_dev(k, F.BF16), to_dev(v, F.BF16)
+    ws = torch.full((F.flowmm_decode_workspace_bytes(qd, kd, vd),), 77, dtype=torch.uint8, device="cuda")
+    ref = O.decode_attention(q, k, v)
+    for _ in range(2):
+        out = torch.full(q.shape, float("nan"), dtype=torch.float32, device="cuda")
+        F.flowmm_decode_attention(qd, kd, vd, out, ws)
+        assert F.flowmm_last_device_status(ws) == 0
+        got = out.cpu().numpy().astype(np.float64)
+        assert np.allclose(got, ref, rtol=RTOL, atol=ATOL), np.abs(got - ref).max()
