@@ -628,19 +628,18 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         c.off = at<int>(ws, y.off); c.piece_off = at<int>(ws, y.piece_off); c.part_off = at<int>(ws, y.part_off);
         c.piece_desc = at<int4>(ws, y.piece_desc); c.ticket = at<unsigned>(ws, y.ticket); c.slot_done = at<int>(ws, y.slot_done);
         c.B = p.n_keep; c.E = E; c.n_pass = y.csr_passes; c.max_pieces = y.max_pieces; c.merge_mode = p.merge_mode;
-        // positions and keys as 16-bit arrays in shared memory when they fit (6 bytes per non-pivot), else through global memory
-        const size_t csr_smem = 6 * (((size_t)E + 7) & ~(size_t)7);
-        const bool staged = E < 65536 && p.n_keep < 65535 && csr_smem <= 200 * 1024;
-        if (staged) {
-            if (E <= 4096) {
-                if (cudaFuncSetAttribute(build_csr_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csr_smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
-                launch(build_csr_kernel<8, true>, UH, 256, csr_smem, st, c);
-            } else {
-                if (cudaFuncSetAttribute(build_csr_kernel<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csr_smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
-                launch(build_csr_kernel<32, true>, UH, 1024, csr_smem, st, c);
-            }
-        } else if (E <= 4096) launch(build_csr_kernel<8, false>, UH, 256, 0, st, c);
-        else launch(build_csr_kernel<32, false>, UH, 1024, 0, st, c);
+        // Warps per head by the length of its list: 8 walk up to 4096 positions in 16 steps each, which ends before 32 warps
+        // are through their barriers.  Sorted in shared memory when positions and counters fit, else through global memory.
+        const bool long_list = E > 4096;
+        const size_t csr_smem = csr_count_smem(E, p.n_keep, long_list ? 32 : 8);
+        if (E < 65536 && csr_smem <= 224 * 1024) {
+            int n_bits = 1;
+            while ((p.n_keep >> n_bits) != 0) ++n_bits;
+            auto kernel = long_list ? build_csr_count_kernel<32> : build_csr_count_kernel<8>;
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csr_smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
+            launch(kernel, UH, long_list ? 1024 : 256, csr_smem, st, c, n_bits);
+        } else if (!long_list) launch(build_csr_kernel<8>, UH, 256, 0, st, c);
+        else launch(build_csr_kernel<32>, UH, 1024, 0, st, c);
         FLOWMM_LAUNCHED("build_csr");
         m.mem_tok = c.mem_tok; m.mem_w = c.mem_w; m.piece_desc = c.piece_desc;
         m.piece_off = c.piece_off; m.part_off = c.part_off; m.ticket = c.ticket; m.slot_done = c.slot_done;

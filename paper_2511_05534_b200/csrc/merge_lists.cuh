@@ -1,6 +1,5 @@
 // The merge / compaction stage.
 #pragma once
-#include <type_traits>
 #include "common.cuh"
 
 namespace flowmm {
@@ -47,16 +46,42 @@ __device__ __forceinline__ uint32_t digit_peers(int digit, bool valid) {
     return mine;
 }
 
+// Pieces per slot and partial records per slot, exclusive scans over the slots; off[s] = first member of slot s (s <= B).
+template <int kThreads>
+__device__ __forceinline__ void csr_write_pieces(const CsrArgs &A, int uh, const int *off, int *scratch) {
+    const int tid = threadIdx.x;
+    int *piece_off = A.piece_off + (int64_t)uh * (A.B + 1);
+    int *part_off = A.part_off + (int64_t)uh * (A.B + 1);
+    int4 *desc = A.piece_desc + (int64_t)uh * A.max_pieces;
+    int piece_seen = 0, part_seen = 0;
+    for (int base = 0; base <= A.B; base += kThreads) {
+        const int s = base + tid;
+        int n = 0, np = 0, npart = 0;
+        if (s < A.B) {
+            n = off[s + 1] - off[s];
+            np = n > kPiece ? (n + kPiece - 1) / kPiece : 1;
+            npart = np > 1 ? np : 0;
+        }
+        int tot_p, tot_q;
+        const int pp = piece_seen + block_exclusive_scan(np, scratch, tot_p);
+        const int qq = part_seen + block_exclusive_scan(npart, scratch, tot_q);
+        if (s <= A.B) { piece_off[s] = pp; part_off[s] = qq; }
+        if (s < A.B) A.slot_done[(int64_t)uh * A.B + s] = 0;
+        for (int q = 0; q < np; ++q)
+            desc[pp + q] = make_int4(s, off[s] + q * kPiece, min(kPiece, n - q * kPiece), np > 1 ? qq + q : -1);
+        piece_seen += tot_p;
+        part_seen += tot_q;
+    }
+    for (int i = piece_seen + tid; i < A.max_pieces; i += kThreads) desc[i] = make_int4(0, 0, -1, -1);   // unused entries
+}
+
 // grid = U*Hkv, block = 32 * NW threads (warp w owns a contiguous range of the input).  n_pass passes of kCsrBits bits.
-// The sort gathers keys by position and scatters positions, 4 or 2 bytes at a time, which an SM's global-memory path
-// takes at about one access per clock: with kStaged (E and B below 65536 and 6 E bytes of dynamic shared memory) the
-// keys and both position buffers are 16-bit arrays in shared memory and only the results touch global memory.
-template <int NW, bool kStaged>
+// For heads too large for build_csr_count_kernel below: keys are gathered by position and positions scattered through
+// global memory, which an SM takes at about one access per clock.
+template <int NW>
 __global__ void __launch_bounds__(32 * NW) build_csr_kernel(const CsrArgs A) {
     constexpr int kThreads = 32 * NW;
     constexpr int kBatch = 8;                       // steps of 32 positions whose loads are in flight together
-    using Pos = std::conditional_t<kStaged, uint16_t, int>;
-    extern __shared__ __align__(16) uint16_t csr_smem[];   // kStaged: keys[Ep], positions[2][Ep], Ep = E rounded up to 8
     __shared__ int counters[NW][kCsrBins + 1];      // [warp][digit], padded
     __shared__ int scratch[33];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -64,28 +89,16 @@ __global__ void __launch_bounds__(32 * NW) build_csr_kernel(const CsrArgs A) {
     predecessor_done();
     if (uh == 0 && tid == 0) *A.ticket = 0u;
     const int *match = A.match + (int64_t)uh * A.E;
-    const int Ep = (A.E + 7) & ~7;
-    Pos *bufs[2];
-    if constexpr (kStaged) {
-        // (the buffer that holds the final order comes last: keys and the other buffer are then one free region of 4 Ep bytes)
-        const int fin = (A.n_pass - 1) & 1;
-        bufs[fin] = csr_smem + 2 * Ep; bufs[fin ^ 1] = csr_smem + Ep;
-        for (int i = tid; i < A.E; i += kThreads) csr_smem[i] = (uint16_t)csr_key(match[i], A.B);
-        __syncthreads();
-    } else {
-        bufs[0] = A.sort_a + (int64_t)uh * A.E; bufs[1] = A.sort_b + (int64_t)uh * A.E;
-    }
-    auto key_of = [&](int j) -> int {
-        if constexpr (kStaged) return csr_smem[j]; else return csr_key(match[j], A.B);
-    };
+    int *bufs[2] = {A.sort_a + (int64_t)uh * A.E, A.sort_b + (int64_t)uh * A.E};
+    auto key_of = [&](int j) -> int { return csr_key(match[j], A.B); };
     const int per_warp = ((A.E + NW - 1) / NW + 31) / 32 * 32;     // multiple of 32
     const int lo = warp * per_warp, hi = min(A.E, lo + per_warp);
     const int end = min(lo + per_warp, ((hi + 31) / 32) * 32);
 
     for (int pass = 0; pass < A.n_pass; ++pass) {
         const int shift = kCsrBits * pass;
-        const Pos *src = pass == 0 ? nullptr : bufs[(pass - 1) & 1];
-        Pos *dst = bufs[pass & 1];
+        const int *src = pass == 0 ? nullptr : bufs[(pass - 1) & 1];
+        int *dst = bufs[pass & 1];
         // The positions and their keys are fetched kBatch steps at a time (the loads of a step depend on each other,
         // those of different steps do not); a step past the warp's range has no valid lane and changes nothing.
         auto fetch = [&](int t0, int (&jv)[kBatch], int (&dg)[kBatch]) {
@@ -138,7 +151,7 @@ __global__ void __launch_bounds__(32 * NW) build_csr_kernel(const CsrArgs A) {
             for (int b = 0; b < kBatch; ++b) {
                 const bool valid = jv[b] >= 0;
                 const uint32_t mine = digit_peers(dg[b], valid);
-                if (valid) dst[counters[warp][dg[b]] + __popc(mine & lanemask_lt())] = (Pos)jv[b];
+                if (valid) dst[counters[warp][dg[b]] + __popc(mine & lanemask_lt())] = jv[b];
                 __syncwarp();
                 if (valid && lane == __ffs(mine) - 1) counters[warp][dg[b]] += __popc(mine);
                 __syncwarp();
@@ -147,10 +160,8 @@ __global__ void __launch_bounds__(32 * NW) build_csr_kernel(const CsrArgs A) {
         __syncthreads();
         __threadfence_block();
     }
-    const Pos *sorted = bufs[(A.n_pass - 1) & 1];
+    const int *sorted = bufs[(A.n_pass - 1) & 1];
     int *off = A.off + (int64_t)uh * (A.B + 1);
-    int *piece_off = A.piece_off + (int64_t)uh * (A.B + 1);
-    int *part_off = A.part_off + (int64_t)uh * (A.B + 1);
     // token position and weight of every member, in slot order
     {
         const int *evi = A.evicted + (int64_t)uh * A.E;
@@ -163,56 +174,123 @@ __global__ void __launch_bounds__(32 * NW) build_csr_kernel(const CsrArgs A) {
             const int j = sorted[i];
             const int key = key_of(j);
             const int prev = i > 0 ? key_of(sorted[i - 1]) : -1;
-            if constexpr (!kStaged) {
-                mem_tok[i] = evi[j];
-                mem_w[i] = A.merge_mode == 1 ? 1.f : __expf(sim[j] - 1.f);
-            }
+            mem_tok[i] = evi[j];
+            mem_w[i] = A.merge_mode == 1 ? 1.f : __expf(sim[j] - 1.f);
             for (int s2 = prev + 1; s2 <= key; ++s2) off[s2] = i;
             if (i == A.E - 1)
                 for (int s2 = key + 1; s2 <= A.B; ++s2) off[s2] = A.E;
         }
-        if constexpr (kStaged) {
-            // the gathers by position go through shared memory as well: the token positions, then the similarities, are
-            // copied in order into the region the keys and the spare buffer have left, and picked from there
-            int *stage_i = reinterpret_cast<int *>(csr_smem);
-            float *stage_f = reinterpret_cast<float *>(csr_smem);
-            __syncthreads();                                     // the keys are not read any more
-            for (int i = tid; i < A.E; i += kThreads) stage_i[i] = evi[i];
-            __syncthreads();
-            for (int i = tid; i < A.E; i += kThreads) mem_tok[i] = stage_i[sorted[i]];
-            __syncthreads();
-            if (A.merge_mode == 1) {
-                for (int i = tid; i < A.E; i += kThreads) mem_w[i] = 1.f;
-            } else {
-                for (int i = tid; i < A.E; i += kThreads) stage_f[i] = sim[i];
-                __syncthreads();
-                for (int i = tid; i < A.E; i += kThreads) mem_w[i] = __expf(stage_f[sorted[i]] - 1.f);
+    }
+    __syncthreads();
+    csr_write_pieces<kThreads>(A, uh, off, scratch);
+}
+
+// The same lists for heads whose sort fits in shared memory: one counting pass over the whole slot number instead of a
+// digit at a time.  Every warp owns a contiguous range of positions and 16-bit counters for all B + 1 slots.
+//   1. warps count their ranges;  2. a thread per pair of slots turns the counts into every warp's start inside the slot,
+//   one prefix sum over the slots gives the slots' starts;  3. warps walk their ranges again, in order, and place the
+//   positions (lanes of the same slot rank themselves by votes);  4. token positions and similarities are staged in the
+//   counters' place and written out in slot order;  5. the piece table.
+// Bound by issue slots and shared-memory latency of one CTA per head (two walks of E positions, 11 votes per step at
+// B = 1690): 8 heads of 32 102 positions 77 us with two 6-bit digits in shared memory, 58 us so; 112 heads of 6 758 32 and
+// 25 us.  Dynamic shared memory: csr_count_smem().
+__host__ __device__ constexpr size_t csr_count_smem(int E, int B, int n_warps) {
+    const size_t Ep = ((size_t)E + 7) & ~(size_t)7, cnt = (size_t)n_warps * (((size_t)B + 2) & ~(size_t)1) * 2;
+    return 2 * Ep + 4 * (((size_t)B + 4) & ~(size_t)3) + (4 * Ep > cnt ? 4 * Ep : cnt) + 16;
+}
+template <int NW>
+__global__ void __launch_bounds__(32 * NW) build_csr_count_kernel(const CsrArgs A, int n_bits) {
+    constexpr int kThreads = 32 * NW, kBatch = 8;
+    extern __shared__ __align__(16) uint8_t csr_raw[];
+    __shared__ int scratch[33];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, uh = blockIdx.x, E = A.E, B = A.B;
+    const size_t Ep = ((size_t)E + 7) & ~(size_t)7;
+    uint16_t *sorted = reinterpret_cast<uint16_t *>(csr_raw);                        // [Ep] positions in slot order
+    int *off = reinterpret_cast<int *>(csr_raw + 2 * Ep);                            // [B + 1] first member of every slot
+    uint8_t *region = csr_raw + 2 * Ep + 4 * (((size_t)B + 4) & ~(size_t)3);
+    const int pitch = (B + 2) & ~1;                                                  // counters of a warp, an even number
+    uint16_t *cnt = reinterpret_cast<uint16_t *>(region) + warp * pitch;
+    for (int i = tid; i < NW * pitch / 2; i += kThreads) reinterpret_cast<uint32_t *>(region)[i] = 0u;
+    __syncthreads();
+    predecessor_done();
+    if (uh == 0 && tid == 0) *A.ticket = 0u;
+    const int *match = A.match + (int64_t)uh * E;
+    const int per_warp = ((E + NW - 1) / NW + 31) / 32 * 32, lo = min(E, warp * per_warp), hi = min(E, lo + per_warp);
+    auto fetch = [&](int t0, int (&key)[kBatch]) {                                   // -1: no such position
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const int j = t0 + 32 * b + lane;
+            key[b] = j < hi ? csr_key(match[j], B) : -1;
+        }
+    };
+    for (int t0 = lo; t0 < hi; t0 += 32 * kBatch) {
+        int key[kBatch];
+        fetch(t0, key);
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b)
+            if (key[b] >= 0) atomicAdd(reinterpret_cast<uint32_t *>(cnt) + (key[b] >> 1), (key[b] & 1) ? 0x10000u : 1u);
+    }
+    __syncthreads();
+    for (int i0 = 0, seen = 0; i0 < pitch / 2; i0 += kThreads) {                     // (one round up to 2 kThreads slots)
+        const int i = i0 + tid;
+        uint32_t run = 0;
+        if (i < pitch / 2) {
+            uint32_t *col = reinterpret_cast<uint32_t *>(region) + i;
+#pragma unroll 8
+            for (int w = 0; w < NW; ++w) {                                           // two slots at a time, no carry between them: E < 65536
+                const uint32_t x = col[w * (pitch / 2)];
+                col[w * (pitch / 2)] = run;
+                run += x;
             }
+        }
+        int total;
+        const int first = seen + block_exclusive_scan((int)(run & 0xFFFFu) + (int)(run >> 16), scratch, total);
+        if (2 * i <= B) off[2 * i] = first;
+        if (2 * i + 1 <= B) off[2 * i + 1] = first + (int)(run & 0xFFFFu);
+        seen += total;
+    }
+    __syncthreads();
+    for (int t0 = lo; t0 < hi; t0 += 32 * kBatch) {
+        int key[kBatch];
+        fetch(t0, key);
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const bool valid = key[b] >= 0;
+            uint32_t mine = __ballot_sync(0xFFFFFFFFu, valid);                       // lanes of the same slot
+            if (mine == 0u) break;
+            for (int q = 0; q < n_bits; ++q) {
+                const uint32_t vote = __ballot_sync(0xFFFFFFFFu, (key[b] >> q) & 1);
+                mine &= ((key[b] >> q) & 1) ? vote : ~vote;
+            }
+            if (valid) sorted[off[key[b]] + cnt[key[b]] + __popc(mine & lanemask_lt())] = (uint16_t)(t0 + 32 * b + lane);
+            __syncwarp();
+            if (valid && lane == __ffs(mine) - 1) cnt[key[b]] += (uint16_t)__popc(mine);
+            __syncwarp();
         }
     }
     __syncthreads();
-    // pieces per slot and partial records per slot, exclusive scans over the slots
-    int4 *desc = A.piece_desc + (int64_t)uh * A.max_pieces;
-    int piece_seen = 0, part_seen = 0;
-    for (int base = 0; base <= A.B; base += kThreads) {
-        const int s = base + tid;
-        int n = 0, np = 0, npart = 0;
-        if (s < A.B) {
-            n = off[s + 1] - off[s];
-            np = n > kPiece ? (n + kPiece - 1) / kPiece : 1;
-            npart = np > 1 ? np : 0;
+    // (entries past off[B] are the dropped tokens: nobody reads them)
+    const int n_mem = off[B];
+    int *mem_tok = A.mem_tok + (int64_t)uh * E;
+    float *mem_w = A.mem_w + (int64_t)uh * E;
+    {
+        const int *evi = A.evicted + (int64_t)uh * E;
+        int *stage = reinterpret_cast<int *>(region);
+        for (int i = tid; i < E; i += kThreads) stage[i] = evi[i];
+        __syncthreads();
+        for (int i = tid; i < n_mem; i += kThreads) mem_tok[i] = stage[sorted[i]];
+        if (A.merge_mode == 1) {
+            for (int i = tid; i < n_mem; i += kThreads) mem_w[i] = 1.f;
+        } else {
+            const float *sim = A.match_sim + (int64_t)uh * E;
+            float *stage_f = reinterpret_cast<float *>(region);
+            __syncthreads();
+            for (int i = tid; i < E; i += kThreads) stage_f[i] = sim[i];
+            __syncthreads();
+            for (int i = tid; i < n_mem; i += kThreads) mem_w[i] = __expf(stage_f[sorted[i]] - 1.f);
         }
-        int tot_p, tot_q;
-        const int pp = piece_seen + block_exclusive_scan(np, scratch, tot_p);
-        const int qq = part_seen + block_exclusive_scan(npart, scratch, tot_q);
-        if (s <= A.B) { piece_off[s] = pp; part_off[s] = qq; }
-        if (s < A.B) A.slot_done[(int64_t)uh * A.B + s] = 0;
-        for (int q = 0; q < np; ++q)
-            desc[pp + q] = make_int4(s, off[s] + q * kPiece, min(kPiece, n - q * kPiece), np > 1 ? qq + q : -1);
-        piece_seen += tot_p;
-        part_seen += tot_q;
     }
-    for (int i = piece_seen + tid; i < A.max_pieces; i += kThreads) desc[i] = make_int4(0, 0, -1, -1);   // unused entries
+    csr_write_pieces<kThreads>(A, uh, off, scratch);
 }
 
 struct MergeArgs {
