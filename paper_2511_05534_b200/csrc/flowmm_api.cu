@@ -506,10 +506,13 @@ flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *
         a.tokmap = tokmap; a.merge_mode = p.merge_mode;
         a.status = at<int>(ws, y.status);
         a.Hkv = p.n_kv_heads; a.L = p.seq_len; a.E = E; a.Ctot = y.c_tot; a.n_heads = UH;
+        const int tiles = (p.seq_len + mst::kTile - 1) / mst::kTile;
+        a.by_nt = make_fastdiv((uint32_t)tiles); a.by_hkv = make_fastdiv((uint32_t)p.n_kv_heads);
+        const int64_t n_tiles = (int64_t)UH * tiles;
         if (cudaFuncSetAttribute(mst::match_small_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)mst::kSmemBytes) != cudaSuccess)
             return FLOWMM_ERR_CUDA;
-        launch(mst::match_small_tc_kernel, UH < tc::sm_count() ? UH : tc::sm_count(), mst::kThreads, mst::kSmemBytes, st, k_map, cand_map, a);
+        launch(mst::match_small_tc_kernel, n_tiles < tc::sm_count() ? (int)n_tiles : tc::sm_count(), mst::kThreads, mst::kSmemBytes, st, k_map, cand_map, a);
         FLOWMM_LAUNCHED("match_small_tc");
         return FLOWMM_OK;
     }
@@ -610,12 +613,15 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
             return FLOWMM_ERR_CUDA;
         mtc::Args a;
         a.tokmap = ma.tokmap; a.k_out = k_out; a.v_out = v_out; a.status = at<int>(ws, y.merge_status);
-        a.Hkv = p.n_kv_heads; a.L = p.seq_len; a.B = p.n_keep; a.n_items = UH; a.n_stages = p.n_keep <= 128 ? mtc::kMaxStages : 3;
+        a.Hkv = p.n_kv_heads; a.L = p.seq_len; a.B = p.n_keep; a.n_stages = p.n_keep <= 128 ? mtc::kMaxStages : 3;
+        // few heads: K and V of a head on an SM each
+        a.per_item = 2 * UH <= tc::sm_count() ? 1 : 2;
+        a.n_items = a.per_item == 1 ? 2 * UH : UH;
         for (int i = 0; i < 3; ++i) { a.kos[i] = p.ko_stride[i]; a.vos[i] = p.vo_stride[i]; }
         const uint32_t smem = mtc::smem_bytes(p.n_keep, a.n_stages);
         if (cudaFuncSetAttribute(mtc::merge_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return FLOWMM_ERR_CUDA;
-        const int grid = UH < tc::sm_count() ? UH : tc::sm_count();
+        const int grid = a.n_items < tc::sm_count() ? a.n_items : tc::sm_count();
         launch(mtc::merge_tc_kernel, grid, mtc::kThreads, smem, st, kmap, vmap, a);
         FLOWMM_LAUNCHED("merge_tc");
         return FLOWMM_OK;

@@ -13,9 +13,14 @@
 //       out^T[dim, slot] += X_step^T W_step^T as tcgen05.mma with M = 128 dims, N = slots, contraction
 //       over the step's tokens; the X tile is the swizzled TMA tile read as an MN-major operand, for K
 //       and for V against the same W slice;
-//       after the last step four reader warps take out^T from TMEM, scale by 1 / (1 + sum of weights)
-//       and store bf16 rows, while the next head's steps already run into a second set of sums and (up to
-//       128 slots) a second set of accumulators.
+//       after the last step eight reader warps (four for K, four for V) take out^T from TMEM, scale by
+//       1 / (1 + sum of weights), transpose 4 x 4 blocks between lanes and store bf16 rows, while the next head's steps
+//       already run into a second set of sums and (up to 128 slots) a second set of accumulators.
+// When the heads fill at most half of the SMs a CTA takes one head's K or V only, with its own copy of W.
+// Bound by the products: a step of 128 tokens takes the tensor core about 1000 clocks per tensor whatever the slots (the X
+// operand is read MN-major).  With four readers storing two bytes per lane the readout took 9 000 (64 slots) to 30 000
+// clocks (218) per head on top: 8 heads of 1471 tokens, 148 slots 32 -> 18 us, 112 of 2176, 218 slots 47 -> 36 us, 32 of 640,
+// 64 slots 18 -> 12 us, 1024 of 640 68 -> 63 us.
 // The weights enter rounded to bf16 (relative error <= 2^-9) in numerator and denominator alike, so every
 // output row is still a weighted mean of its members with weights within 0.2 % of Eq. 5's; the change of
 // the result is below the bf16 rounding of the output itself.
@@ -32,14 +37,14 @@ namespace mtc {
 
 constexpr int kTile = 128;                       // tokens per step
 constexpr int kMaxSlots = 240;                   // N <= 240: two 60 KB weight slices and three tile stages fit in shared memory
-constexpr int kThreads = 320;                    // TMA warp, MMA warp, four builder warps, four reader warps
+constexpr int kThreads = 448;                    // TMA warp, MMA warp, four builder warps, eight reader warps
 constexpr int kPivotFlag = 1 << 30;              // in the table's slot word: the token is the slot's pivot
 constexpr uint32_t kStageBytes = kTile * 128 * 2, kPanel = kStageBytes / 2;
 constexpr int kMaxStages = 4;
 constexpr int kBarFull = 0, kBarEmpty = kMaxStages, kBarWFull = 2 * kMaxStages, kBarWEmpty = kBarWFull + 2,
               kBarOutFull = kBarWEmpty + 2, kBarSumFull = kBarOutFull + 2, kBarOutEmpty = kBarSumFull + 2,
-              kNumBars = kBarOutEmpty + 2;               // from kBarSumFull on: 128 arrivals each
-constexpr uint32_t kTailData = 2 * kMaxSlots * 4 + kMaxSlots * 4;     // weight sums of two heads, reciprocal normalisers
+              kNumBars = kBarOutEmpty + 2;               // sums: 128 arrivals; accumulators read out: 256
+constexpr uint32_t kTailData = 2 * kMaxSlots * 4 + 256 * 4;           // weight sums of two heads, reciprocal normalisers (whole blocks of 32 are read)
 constexpr float kSumScale = 65536.f;             // weights in [2^-3, 1] rounded to bf16 are whole multiples of 2^-10
 
 struct Args {
@@ -47,6 +52,7 @@ struct Args {
     void *k_out, *v_out;
     int *status;
     int Hkv, L, B, n_items, n_stages;
+    int per_item;                // 2: an item is a head; 1: an item is a head's K (even items) or V (odd items)
     int64_t kos[3], vos[3];
 };
 
@@ -56,7 +62,29 @@ __host__ __device__ inline uint32_t smem_bytes(int B, int n_stages) {
     return (uint32_t)n_stages * kStageBytes + 2 * w_bytes(B) + kTailData + 8 * kNumBars + 16;
 }
 
-__device__ __forceinline__ void reader_sync() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
+__device__ __forceinline__ void reader_sync() { asm volatile("bar.sync 2, 256;" ::: "memory"); }
+
+// 32 output columns (slots s0 ..) of this thread's row (dim) scaled, rounded and stored.  Lanes of four exchange so that each
+// holds four consecutive dims of one slot: 8-byte stores, 64 contiguous bytes per slot and warp.
+__device__ __forceinline__ void store_slots32(const uint32_t (&acc)[32], const float *inv, __nv_bfloat16 *out, int64_t stride, int s0, int B,
+                                              int lane) {
+    const int sub = lane & 3;
+    __nv_bfloat16 *dst = out + (int64_t)(s0 + sub) * stride;
+#pragma unroll
+    for (int q = 0; q < 32; q += 4) {
+        const float4 f = *reinterpret_cast<const float4 *>(inv + s0 + q);
+        const __nv_bfloat162 p01 = __floats2bfloat162_rn(__uint_as_float(acc[q]) * f.x, __uint_as_float(acc[q + 1]) * f.y);
+        const __nv_bfloat162 p23 = __floats2bfloat162_rn(__uint_as_float(acc[q + 2]) * f.z, __uint_as_float(acc[q + 3]) * f.w);
+        const uint32_t w01 = *reinterpret_cast<const uint32_t *>(&p01), w23 = *reinterpret_cast<const uint32_t *>(&p23);
+        const uint32_t r01 = __shfl_xor_sync(0xFFFFFFFFu, w01, 1), r23 = __shfl_xor_sync(0xFFFFFFFFu, w23, 1);
+        // even lanes: the pair's first slot, dims (d, d + 1); odd lanes: its second slot, dims (d - 1, d)
+        const uint32_t a = (lane & 1) ? __byte_perm(r01, w01, 0x7632) : __byte_perm(w01, r01, 0x5410);
+        const uint32_t b = (lane & 1) ? __byte_perm(r23, w23, 0x7632) : __byte_perm(w23, r23, 0x5410);
+        const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, (lane & 2) ? a : b, 2);
+        if (s0 + q + sub < B)
+            *reinterpret_cast<uint2 *>(dst + (int64_t)q * stride) = (lane & 2) ? make_uint2(got, b) : make_uint2(a, got);
+    }
+}
 
 struct MapArgs {
     const int *retained, *evicted, *match;
@@ -93,7 +121,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     const uint32_t w0 = base + (uint32_t)A.n_stages * kStageBytes;
     uint8_t *tail = mtc_smem + (size_t)A.n_stages * kStageBytes + 2 * (size_t)wsize;
     unsigned *wsum = reinterpret_cast<unsigned *>(tail);                                  // [2][kMaxSlots], units of 1 / kSumScale
-    float *inv_s = reinterpret_cast<float *>(tail + 2 * kMaxSlots * 4);                   // [kMaxSlots]
+    float *inv_s = reinterpret_cast<float *>(tail + 2 * kMaxSlots * 4);                   // [256]
     const uint32_t bars = tc::smem_u32(tail + kTailData);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tail + kTailData + 8 * kNumBars);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tail + kTailData + 8 * kNumBars + 4);
@@ -105,7 +133,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     auto bar = [&](int i) { return bars + 8u * i; };
     if (threadIdx.x == 0) {
         for (int i = 0; i < kNumBars; ++i)
-            tc::mbar_init(bar(i), (i >= kBarWFull && i < kBarWFull + 2) || i >= kBarSumFull ? 128 : 1);
+            tc::mbar_init(bar(i), i >= kBarOutEmpty ? 256 : (i >= kBarWFull && i < kBarWFull + 2) || i >= kBarSumFull ? 128 : 1);
         *abort_flag = 0;
         tc::mbar_init_fence();
         tc::tma_prefetch_desc(&kmap);
@@ -120,22 +148,26 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     const uint32_t tmem = *tmem_slot;
     predecessor_done();
     const int n_chunk = (A.L + kTile - 1) / kTile;
+    const int per_item = A.per_item;                             // tensors of an item; the first (only) one:
+    auto first_tensor = [&](int item) { return per_item == 2 ? 0 : item & 1; };
+    auto head_of = [&](int item) { return per_item == 2 ? item : item >> 1; };
 
     if (warp == 0) {
         if (lane == 0) {
             bool ok = true;
             int i = 0;
             for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x) {
-                const int u = item / A.Hkv, h = item % A.Hkv;
-                for (int c = 0; ok && c < 2 * n_chunk; ++c, ++i) {   // per step the K tile, then the V tile
+                const int u = head_of(item) / A.Hkv, h = head_of(item) % A.Hkv, t0 = first_tensor(item);
+                for (int c = 0; ok && c < per_item * n_chunk; ++c, ++i) {   // per step the K tile, then the V tile
                     const int st = i % A.n_stages;
                     ok = tc::mbar_wait(bar(kBarEmpty + st), ((i / A.n_stages) & 1) ^ 1, abort_flag, A.status);
                     if (!ok) break;
-                    const CUtensorMap *m = (c & 1) ? &vmap : &kmap;
+                    const int step = per_item == 2 ? c >> 1 : c;
+                    const CUtensorMap *m = (per_item == 2 ? c & 1 : t0) ? &vmap : &kmap;
                     const uint32_t dst = base + st * kStageBytes;
                     tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
-                    tc::tma_load_4d(dst, m, bar(kBarFull + st), 0, (c >> 1) * kTile, h, u);
-                    tc::tma_load_4d(dst + kPanel, m, bar(kBarFull + st), 64, (c >> 1) * kTile, h, u);
+                    tc::tma_load_4d(dst, m, bar(kBarFull + st), 0, step * kTile, h, u);
+                    tc::tma_load_4d(dst + kPanel, m, bar(kBarFull + st), 64, step * kTile, h, u);
                 }
             }
             if (!ok)         // winding down after a timeout: give copies already issued a moment to land
@@ -155,7 +187,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                     const int wb = j & 1;
                     ok = tc::mbar_wait(bar(kBarWFull + wb), (j >> 1) & 1, abort_flag, A.status);
                     const uint32_t w = w0 + wb * wsize;
-                    for (int t = 0; ok && t < 2; ++t, ++i) {
+                    for (int t = 0; ok && t < per_item; ++t, ++i) {
                         const int st = i % A.n_stages;
                         ok = tc::mbar_wait(bar(kBarFull + st), (i / A.n_stages) & 1, abort_flag, A.status);
                         if (!ok) break;
@@ -181,9 +213,9 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
         // position of this thread's token inside a W panel row: 64 tokens per 128-byte row, 16-byte groups swizzled by row
         const uint32_t tok_off = (uint32_t)(e >> 6) * wpanel + (uint32_t)((e & 7) << 1);
         const int tok_grp = (e & 63) >> 3;
-        int2 first = (int)blockIdx.x < A.n_items && e < A.L ? A.tokmap[(int64_t)blockIdx.x * A.L + e] : make_int2(-1, 0);
+        int2 first = (int)blockIdx.x < A.n_items && e < A.L ? A.tokmap[(int64_t)head_of(blockIdx.x) * A.L + e] : make_int2(-1, 0);
         for (int item = blockIdx.x; item < A.n_items; item += gridDim.x, ++it) {
-            const int2 *map = A.tokmap + (int64_t)item * A.L;
+            const int2 *map = A.tokmap + (int64_t)head_of(item) * A.L;
             const int set = it % n_sets, use = it / n_sets;
             unsigned *sums = wsum + set * kMaxSlots;
             // the set's sums are zero again once its previous head has been read out
@@ -193,7 +225,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                 const int2 cur = nxt;
                 const int t_next = (c + 1) * kTile + e;
                 if (c + 1 < n_chunk) nxt = t_next < A.L ? map[t_next] : make_int2(-1, 0);
-                else first = item + (int)gridDim.x < A.n_items && e < A.L ? map[(int64_t)gridDim.x * A.L + e] : make_int2(-1, 0);
+                else first = item + (int)gridDim.x < A.n_items && e < A.L ? A.tokmap[(int64_t)head_of(item + gridDim.x) * A.L + e] : make_int2(-1, 0);
                 const int wb = j & 1;
                 ok = ok && tc::mbar_wait(bar(kBarWEmpty + wb), ((j >> 1) & 1) ^ 1, abort_flag, A.status);
                 const uint32_t w = w0 + wb * wsize;
@@ -215,18 +247,17 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
             tc::mbar_arrive(bar(kBarSumFull + set));                 // this head's weight sums are complete
         }
     } else {
-        // readers: thread = output dim; columns = slots
-        const int e = threadIdx.x - 192;
-        const int row = 32 * (warp & 3) + lane;
+        // readers: thread = output dim; columns = slots; the first four warps take K, the others V
+        const int e = threadIdx.x - 192, t = e >> 7;
         const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
         bool ok = true;
         int it = 0;
         for (int item = blockIdx.x; item < A.n_items; item += gridDim.x, ++it) {
-            const int u = item / A.Hkv, h = item % A.Hkv;
+            const int u = head_of(item) / A.Hkv, h = head_of(item) % A.Hkv;
             const int set = it % n_sets, use = it / n_sets;
             unsigned *sums = wsum + set * kMaxSlots;
             ok = ok && tc::mbar_wait(bar(kBarSumFull + set), use & 1, abort_flag, A.status);
-            for (int sl = e; sl < N; sl += 128) {
+            for (int sl = e; sl < N; sl += 256) {
                 inv_s[sl] = 1.f / (1.f + (float)sums[sl] * (1.f / kSumScale));
                 sums[sl] = 0u;
             }
@@ -234,22 +265,18 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
             ok = ok && tc::mbar_wait(bar(kBarOutFull + set), use & 1, abort_flag, A.status);
             tc::tc_fence_after();
             if (*abort_flag == 0) {
+                // a single tensor's slots go to the two quads in turn, 32 at a time
+                const int which = per_item == 2 ? t : first_tensor(item);
+                __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(which ? A.v_out : A.k_out) +
+                                     (which ? u * A.vos[0] + h * A.vos[1] : u * A.kos[0] + h * A.kos[1]) + 32 * (warp & 3) + (lane & ~3);
+                const int64_t stride = which ? A.vos[2] : A.kos[2];
+                const uint32_t tcol = trow + set * set_cols + (per_item == 2 ? t * v_col : 0u);
 #pragma unroll 1
-                for (int t = 0; t < 2; ++t) {
-                    __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(t ? A.v_out : A.k_out) +
-                                         (t ? u * A.vos[0] + h * A.vos[1] : u * A.kos[0] + h * A.kos[1]) + row;
-                    const int64_t stride = t ? A.vos[2] : A.kos[2];
-                    const uint32_t tcol = trow + set * set_cols + t * v_col;
-#pragma unroll 1
-                    for (int s0 = 0; s0 < A.B; s0 += 16) {
-                        uint32_t acc[16];
-                        tc::tmem_ld16(tcol + s0, acc);
-                        tc::tmem_ld_wait(acc);
-#pragma unroll
-                        for (int q = 0; q < 16; ++q)
-                            if (s0 + q < A.B)
-                                out[(int64_t)(s0 + q) * stride] = __float2bfloat16_rn(__uint_as_float(acc[q]) * inv_s[s0 + q]);
-                    }
+                for (int s0 = per_item == 2 ? 0 : 32 * t; s0 < A.B; s0 += per_item == 2 ? 32 : 64) {
+                    uint32_t acc[32];
+                    tc::tmem_ld32(tcol + s0, acc);
+                    tc::tmem_ld_wait(acc);
+                    store_slots32(acc, inv_s, out, stride, s0, A.B, lane);
                 }
             }
             tc::tc_fence_before();

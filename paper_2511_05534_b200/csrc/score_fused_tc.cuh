@@ -240,15 +240,15 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
                 const int c = cb + q;
                 lt[q] = 1.f / (red[4 * kRows + c] + red[5 * kRows + c] + red[6 * kRows + c] + red[7 * kRows + c]);
             }
-            if (e < A.G && ok) {                                     // Eq. 7 for query head e of the group: sum over its rows
-                float s = 0.f;
-                for (int a = 0; a < A.W; ++a) {
-                    const int c = e * A.W + a;
-                    const float tot = red[4 * kRows + c] + red[5 * kRows + c] + red[6 * kRows + c] + red[7 * kRows + c];
-                    const float cr = red[8 * kRows + c] + red[9 * kRows + c] + red[10 * kRows + c] + red[11 * kRows + c];
-                    s += cr / tot;
+            if (tw == 0 && ok) {                                     // Eq. 7: a lane per proxy row, summed per query head as a tree
+                const float tot = red[4 * kRows + lane] + red[5 * kRows + lane] + red[6 * kRows + lane] + red[7 * kRows + lane];
+                const float cr = red[8 * kRows + lane] + red[9 * kRows + lane] + red[10 * kRows + lane] + red[11 * kRows + lane];
+                float share = cr / tot;
+                for (int o = 1; o < A.W; o <<= 1) {                  // (W divides 32: lanes g W .. g W + W - 1 are head g's)
+                    const float other = __shfl_down_sync(0xFFFFFFFFu, share, o);
+                    if ((lane & (2 * o - 1)) == 0) share += other;
                 }
-                A.cross_mass[(int64_t)u * A.Hq + h * A.G + e] = s;
+                if (lane % A.W == 0) A.cross_mass[(int64_t)u * A.Hq + h * A.G + lane / A.W] = share;
             }
             float imp[kMaxTiles];                                    // sweep C: this thread's share of every key's importance
 #pragma unroll

@@ -171,3 +171,23 @@ def test_strided_inputs():
     g = {key: (t.float().cpu().numpy().astype(np.float64) if t.is_floating_point() else t.cpu().numpy())
          for key, t in out.items() if key != "ws"}
     C.compare(p, q, k, v, m, g, bf16_out=True)
+
+
+def test_short_lists_over_runs_of_tiles():
+    """The short-list matching kernel gives every CTA an equal run of the 128-token tiles of all heads: heads of one tile, runs
+    that begin and end inside a head, one and two units of candidate columns, many heads per run; and the tensor-core merge
+    with a head per CTA, with K and V apart, and with budgets at the edges of its 32-slot blocks."""
+    rng = np.random.default_rng(31)
+    for (U, Hq, Hkv, L, W, B, kw) in [
+        (1, 160, 160, 100, 8, 30, {}),                              # one tile per head, more heads than CTAs: K and V together
+        (3, 75, 75, 128, 32, 33, dict(flow_mode=O.FLOW_FORCE_INTRA)),
+        (2, 80, 80, 260, 16, 97, {}),                               # two units (129 to 256 candidate columns), three tiles per head
+        (1, 90, 90, 513, 8, 128, dict(flow_mode=O.FLOW_FORCE_INTRA)),
+        (1, 4, 4, 1300, 32, 225 - 1, dict(vis_frac=0.1)),
+        (1, 3, 3, 900, 32, 160, dict(vis_frac=0.95)),
+        (1, 2, 2, 300, 32, 64, dict(tau=0.0)),                      # no candidate at all
+        (1, 1, 1, 4000, 32, 1, {}),
+    ]:
+        args = dict(tau=4.0, tau_mode=O.TAU_REL, theta=0.5)
+        args.update(kw)
+        _random_case(rng, U, Hq, Hkv, 128, L, W, B, F.BF16, **args)
