@@ -33,6 +33,20 @@ __device__ __forceinline__ constexpr bool index_ok(long long, long long, int *) 
 // memory that a block of the running kernel has yet to allocate.
 __device__ __forceinline__ void predecessor_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// ---- thread-block clusters ----------------------------------------------------------------------
+// (every thread of the cluster calls these, converged warps)
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
+// a 32-bit word in the shared memory of the cluster's CTA `rank`, at this CTA's shared address `addr`
+__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr, int rank) {
+    uint32_t remote, v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t addr, int rank) { return __uint_as_float(ld_cluster_u32(addr, rank)); }
+
 // ---- element access -------------------------------------------------------------------------
 template <typename T> struct Elem;
 template <> struct Elem<float> {

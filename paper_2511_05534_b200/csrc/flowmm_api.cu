@@ -637,10 +637,18 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         // Warps per head by the length of its list: 8 walk up to 4096 positions in 16 steps each, which ends before 32 warps
         // are through their barriers.  Sorted in shared memory when positions and counters fit, else through global memory.
         const bool long_list = E > 4096;
+        int n_bits = 1;
+        while ((p.n_keep >> n_bits) != 0) ++n_bits;
+        // Few heads: a head's list is shared among 2, 4 or 8 CTAs, at least 1024 positions each, as long as every CTA has an
+        // SM (with four per SM 128 heads of 33 792 tokens took 89 instead of 68 us: the scattered writes then set the pace)
+        int ctas = 8;
+        while (ctas > 1 && (ctas * UH > tc::sm_count() || E < 1024 * ctas)) ctas >>= 1;
         const size_t csr_smem = csr_count_smem(E, p.n_keep, long_list ? 32 : 8);
-        if (E < 65536 && csr_smem <= 224 * 1024) {
-            int n_bits = 1;
-            while ((p.n_keep >> n_bits) != 0) ++n_bits;
+        if (ctas > 1 && E < 65536 && csr_cluster_smem(p.n_keep) <= 96 * 1024) {
+            const size_t smem = csr_cluster_smem(p.n_keep);
+            if (cudaFuncSetAttribute(build_csr_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
+            launch_cluster(dim3(ctas), build_csr_cluster_kernel, UH * ctas, 32 * kCsrClusterWarps, smem, st, c, n_bits, ctas);
+        } else if (E < 65536 && csr_smem <= 224 * 1024) {
             auto kernel = long_list ? build_csr_count_kernel<32> : build_csr_count_kernel<8>;
             if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csr_smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
             launch(kernel, UH, long_list ? 1024 : 256, csr_smem, st, c, n_bits);

@@ -293,6 +293,111 @@ __global__ void __launch_bounds__(32 * NW) build_csr_count_kernel(const CsrArgs 
     csr_write_pieces<kThreads>(A, uh, off, scratch);
 }
 
+// The counting sort with a head's positions shared among the CTAs of a cluster, for calls whose heads do not fill the GPU.
+// As above, but every CTA counts its part of the positions, reads the other CTAs' totals per slot out of their shared
+// memory, and writes its members' token positions and weights straight to their places (8 heads of 32 102 positions:
+// 59 -> 22 us).
+// grid = (U*Hkv * ctas), cluster = ctas along x.  Dynamic shared memory: csr_cluster_smem().
+constexpr int kCsrClusterWarps = 16;
+__host__ __device__ constexpr size_t csr_cluster_smem(int B) {
+    const size_t pitch = ((size_t)B + 2) & ~(size_t)1;
+    return kCsrClusterWarps * pitch * 2 + pitch * 2 + 2 * pitch * 4 + 16;
+}
+__global__ void __launch_bounds__(32 * kCsrClusterWarps) build_csr_cluster_kernel(const CsrArgs A, int n_bits, int ctas) {
+    constexpr int NW = kCsrClusterWarps, kThreads = 32 * NW, kBatch = 8;
+    extern __shared__ __align__(16) uint8_t csr_raw[];
+    __shared__ int scratch[33];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, E = A.E, B = A.B;
+    const int uh = blockIdx.x / ctas, rank = blockIdx.x % ctas;
+    const int pitch = (B + 2) & ~1;                                                  // counters of a warp, an even number
+    uint32_t *words = reinterpret_cast<uint32_t *>(csr_raw);                         // [NW][pitch / 2] pairs of 16-bit counters
+    uint32_t *totals = words + NW * pitch / 2;                                       // [pitch / 2] this CTA's counts
+    int *off = reinterpret_cast<int *>(totals + pitch / 2);                          // [B + 1] first member of every slot
+    int *base = off + pitch;                                                         // ... of this CTA's part of it
+    uint16_t *cnt = reinterpret_cast<uint16_t *>(csr_raw) + warp * pitch;
+    for (int i = tid; i < NW * pitch / 2; i += kThreads) words[i] = 0u;
+    __syncthreads();
+    predecessor_done();
+    if (blockIdx.x == 0 && tid == 0) *A.ticket = 0u;
+    const int *match = A.match + (int64_t)uh * E;
+    const int per_warp = ((E + ctas * NW - 1) / (ctas * NW) + 31) / 32 * 32;
+    const int lo = min(E, (rank * NW + warp) * per_warp), hi = min(E, lo + per_warp);
+    for (int t0 = lo; t0 < hi; t0 += 32 * kBatch) {
+        int key[kBatch];
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) key[b] = t0 + 32 * b + lane < hi ? csr_key(match[t0 + 32 * b + lane], B) : -1;
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b)
+            if (key[b] >= 0) atomicAdd(reinterpret_cast<uint32_t *>(cnt) + (key[b] >> 1), (key[b] & 1) ? 0x10000u : 1u);
+    }
+    __syncthreads();
+    for (int i = tid; i < pitch / 2; i += kThreads) {                                // two slots at a time, no carry between them: E < 65536
+        uint32_t run = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const uint32_t x = words[w * (pitch / 2) + i];
+            words[w * (pitch / 2) + i] = run;
+            run += x;
+        }
+        totals[i] = run;
+    }
+    cluster_sync();
+    const uint32_t totals_at = (uint32_t)__cvta_generic_to_shared(totals);
+    for (int i0 = 0, seen = 0; i0 < pitch / 2; i0 += kThreads) {
+        const int i = i0 + tid;
+        uint32_t all = 0, before = 0;
+        if (i < pitch / 2)
+            for (int r = 0; r < ctas; ++r) {
+                if (r == rank) before = all;
+                all += ld_cluster_u32(totals_at + 4 * i, r);
+            }
+        int total;
+        const int first = seen + block_exclusive_scan((int)(all & 0xFFFFu) + (int)(all >> 16), scratch, total);
+        const int second = first + (int)(all & 0xFFFFu);
+        if (2 * i <= B) { off[2 * i] = first; base[2 * i] = first + (int)(before & 0xFFFFu); }
+        if (2 * i + 1 <= B) { off[2 * i + 1] = second; base[2 * i + 1] = second + (int)(before >> 16); }
+        seen += total;
+    }
+    __syncthreads();
+    cluster_arrive();                                                                // the other CTAs' totals have been read
+    const int *evi = A.evicted + (int64_t)uh * E;
+    const float *sim = A.match_sim + (int64_t)uh * E;
+    int *mem_tok = A.mem_tok + (int64_t)uh * E;
+    float *mem_w = A.mem_w + (int64_t)uh * E;
+    for (int t0 = lo; t0 < hi; t0 += 32 * kBatch) {
+        int key[kBatch], tok[kBatch];
+        float w[kBatch];
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const int j = t0 + 32 * b + lane;
+            key[b] = j < hi ? csr_key(match[j], B) : -1;
+            tok[b] = j < hi ? evi[j] : 0;
+            w[b] = j < hi ? sim[j] : 0.f;
+        }
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b) {
+            const bool valid = key[b] >= 0;
+            uint32_t mine = __ballot_sync(0xFFFFFFFFu, valid);                       // lanes of the same slot
+            if (mine == 0u) break;
+            for (int q = 0; q < n_bits; ++q) {
+                const uint32_t vote = __ballot_sync(0xFFFFFFFFu, (key[b] >> q) & 1);
+                mine &= ((key[b] >> q) & 1) ? vote : ~vote;
+            }
+            if (valid && key[b] < B) {                                               // (dropped tokens have no place)
+                const int at = base[key[b]] + cnt[key[b]] + __popc(mine & lanemask_lt());
+                mem_tok[at] = tok[b];
+                mem_w[at] = A.merge_mode == 1 ? 1.f : __expf(w[b] - 1.f);
+            }
+            __syncwarp();
+            if (valid && lane == __ffs(mine) - 1) cnt[key[b]] += (uint16_t)__popc(mine);
+            __syncwarp();
+        }
+    }
+    if (rank == ctas - 1) csr_write_pieces<kThreads>(A, uh, off, scratch);           // (the last CTA has the fewest positions)
+    __syncwarp();
+    cluster_wait();                                                                  // nobody's totals go away while they are read
+}
+
 struct MergeArgs {
     const void *k, *v;
     void *k_out, *v_out;

@@ -32,8 +32,8 @@ constexpr int kThreads = 64 + 2 * kTeam;
 constexpr uint32_t kStageBytes = kTile * 128 * 2, kPanel = kStageBytes / 2;
 constexpr uint32_t kQBytes = kRows * 256;                          // Q operand of one head: two panels of 32 rows
 constexpr uint32_t kSmemQ = kStages * kStageBytes;                 // two Q operands
-constexpr uint32_t kSmemRed = kSmemQ + 2 * kQBytes;                // per team: float [3][4][kRows], int [kRows] mask limits
-constexpr uint32_t kRedBytes = 13 * kRows * 4;
+constexpr uint32_t kSmemRed = kSmemQ + 2 * kQBytes;                // per team: float [3][4][kRows], int [kRows] mask limits, float [2][kRows] row maxima and 1 / row sums
+constexpr uint32_t kRedBytes = 15 * kRows * 4;
 constexpr uint32_t kSmemImp = kSmemRed + 2 * kRedBytes;            // per team: float [kMaxTiles][128] partial importances
 constexpr uint32_t kImpBytes = kMaxTiles * kTile * 4;
 constexpr uint32_t kSmemBar = kSmemImp + 2 * kImpBytes;
@@ -164,6 +164,7 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
         float *red = reinterpret_cast<float *>(sft_smem + kSmemRed + team * kRedBytes);    // [3][4][kRows]
         float *impx = reinterpret_cast<float *>(sft_smem + kSmemImp + team * kImpBytes);   // [nt][128]
         int *lim = reinterpret_cast<int *>(red + 12 * kRows);
+        float *row_max = red + 13 * kRows, *row_inv = red + 14 * kRows;
         const int first_proxy = A.L - A.W;
         // a (key, proxy row c) pair counts if key <= lim[c] = first_proxy + c % W (which also keeps key < L)
         if (e < GW) lim[e] = first_proxy + e % A.W;
@@ -206,26 +207,41 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
             warp_reduce16(mx, [](float a, float b) { return fmaxf(a, b); });
             if (!(lane & 1)) red[wq * kRows + cb + (lane >> 1)] = mx[0];
             team_sync(team);
+            if (tw == 0)                                             // the row's maximum in the log2 domain
+                row_max[lane] = A.scale_log2 * fmaxf(fmaxf(red[lane], red[kRows + lane]), fmaxf(red[2 * kRows + lane], red[3 * kRows + lane]));
+            team_sync(team);
+            auto load_rows = [&](const float *from, float (&v)[HC]) {
 #pragma unroll
-            for (int q = 0; q < HC; ++q) {   // from here on: the row's maximum in the log2 domain
-                const int c = cb + q;
-                mx[q] = A.scale_log2 * fmaxf(fmaxf(red[c], red[kRows + c]), fmaxf(red[2 * kRows + c], red[3 * kRows + c]));
-            }
+                for (int q = 0; q < HC; q += 4) {
+                    const float4 f = *reinterpret_cast<const float4 *>(from + cb + q);
+                    v[q] = f.x; v[q + 1] = f.y; v[q + 2] = f.z; v[q + 3] = f.w;
+                }
+            };
+            load_rows(row_max, mx);
 
             float lt[HC], lc[HC];                                    // sweep B: row sums, total and other-modality keys
 #pragma unroll
             for (int q = 0; q < HC; ++q) { lt[q] = 0.f; lc[q] = 0.f; }
+            const bool one_kind = qvis == 0u || qvis == (1u << HC) - 1u;   // this warp's proxy rows are of one modality
             for (int t = 0; t < nt; ++t) {
-                const int key = t * kTile + row;
                 const unsigned oth = ((vis_bits >> t) & 1u) ? ~qvis : qvis;   // proxy rows of the other modality than this key's
                 uint32_t r[HC];
                 load(t, r);
+                float p[HC];
 #pragma unroll
-                for (int q = 0; q < HC; ++q) {
-                    float p = tc::ex2(fmaf(__uint_as_float(r[q]), A.scale_log2, -mx[q]));
-                    if (t >= n_plain && key > lim[cb + q]) p = 0.f;
-                    lt[q] += p;
-                    lc[q] += ((oth >> q) & 1u) ? p : 0.f;
+                for (int q = 0; q < HC; ++q) p[q] = tc::ex2(fmaf(__uint_as_float(r[q]), A.scale_log2, -mx[q]));
+                if (t >= n_plain) {
+                    const int key = t * kTile + row;
+#pragma unroll
+                    for (int q = 0; q < HC; ++q) p[q] = key > lim[cb + q] ? 0.f : p[q];
+                }
+                if (one_kind) {
+                    const float o = (oth & 1u) ? 1.f : 0.f;
+#pragma unroll
+                    for (int q = 0; q < HC; ++q) { lt[q] += p[q]; lc[q] = fmaf(o, p[q], lc[q]); }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < HC; ++q) { lt[q] += p[q]; lc[q] += ((oth >> q) & 1u) ? p[q] : 0.f; }
                 }
             }
             warp_reduce16(lt, [](float a, float b) { return a + b; });
@@ -235,21 +251,19 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
                 red[(8 + wq) * kRows + cb + (lane >> 1)] = lc[0];
             }
             team_sync(team);
-#pragma unroll
-            for (int q = 0; q < HC; ++q) {   // from here on: 1 / row sum
-                const int c = cb + q;
-                lt[q] = 1.f / (red[4 * kRows + c] + red[5 * kRows + c] + red[6 * kRows + c] + red[7 * kRows + c]);
-            }
-            if (tw == 0 && ok) {                                     // Eq. 7: a lane per proxy row, summed per query head as a tree
+            if (tw == 0) {                                           // Eq. 7: a lane per proxy row, summed per query head as a tree
                 const float tot = red[4 * kRows + lane] + red[5 * kRows + lane] + red[6 * kRows + lane] + red[7 * kRows + lane];
                 const float cr = red[8 * kRows + lane] + red[9 * kRows + lane] + red[10 * kRows + lane] + red[11 * kRows + lane];
+                row_inv[lane] = 1.f / tot;
                 float share = cr / tot;
                 for (int o = 1; o < A.W; o <<= 1) {                  // (W divides 32: lanes g W .. g W + W - 1 are head g's)
                     const float other = __shfl_down_sync(0xFFFFFFFFu, share, o);
                     if ((lane & (2 * o - 1)) == 0) share += other;
                 }
-                if (lane % A.W == 0) A.cross_mass[(int64_t)u * A.Hq + h * A.G + lane / A.W] = share;
+                if (ok && lane % A.W == 0) A.cross_mass[(int64_t)u * A.Hq + h * A.G + lane / A.W] = share;
             }
+            team_sync(team);
+            load_rows(row_inv, lt);
             float imp[kMaxTiles];                                    // sweep C: this thread's share of every key's importance
 #pragma unroll
             for (int t = 0; t < kMaxTiles; ++t) {
