@@ -4,7 +4,7 @@
 // An item is 256 consecutive query rows of one query head (two accumulator halves of 128) against the keys up to its last
 // row.  Per row the softmax statistics are kept as in the first scoring pass, with the part of the exp-sum that falls on
 // keys of the other modality beside it (a word of 32 keys is of one modality nearly always: then it costs one comparison;
-// only mixed words go element by element).  At the end of an item the four column quarters of a row meet in shared memory
+// only mixed words go element by element).  At the end of an item the two column halves of a row meet in shared memory
 // and a row's share cross / total is added up per warp, so nothing but four floats per half leaves the CTA.
 //
 // Bound by the epilogue: Hq L^2 / 2 exponentials per unit, a quarter of them as a polynomial on the FMA pipe, with four
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(tcs::kThreads, 1)
 flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, const FlowTcArgs A) {
     using S = tcs::Big;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    const S::Ctx c = S::setup(smem_raw, &q_map, &k_map, A.status, 0, 16);
+    const S::Ctx c = S::setup(smem_raw, &q_map, &k_map, A.status, 0, 4);
     if (!c.ok) return;
     auto plan_of = [&](const FlowItem &f) {
         tcs::TilePlan p;
@@ -67,20 +67,18 @@ flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
     if (c.warp == 0) {
         if (c.lane == 0) S::producer(c, &q_map, &k_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
-        if (c.lane == 0) S::mma_issuer(c, A.n_items, plan, A.status);
+        if (c.lane == 0) S::mma_issuer<true>(c, A.n_items, plan, A.status);
     } else {
-        // all sixteen warps drain one accumulator at a time: a warp owns 32 lanes x a quarter of the columns of both halves
-        const int row_in_half = c.quarter * 32 + c.lane, colq = (c.warp - 2) >> 2;
-        float *xch = reinterpret_cast<float *>(smem_raw + S::kSmemEpi);      // [3 values][2 halves][4 column quarters][128 rows]
-        int kh[2] = {0, 0};
+        const int row = c.quarter * 32 + c.lane;                     // row of the half
+        const uint32_t xch = c.epi_addr() + row * 16, pxch = c.partner_addr() + row * 16;   // hand-over slot of this row, the other column half's
+        int k = 0;
         bool ok = true;
         FlowItem f_next;
-        uint32_t flip_next[2];                                       // modality words of this warp's 32 rows of each half
+        uint32_t flip_next = 0;                                      // modality word of this warp's 32 rows
         auto fetch_next = [&](int item) {
             if (item >= A.n_items) return;
             f_next = flow_item(A, item);
-            const uint32_t *w = A.modbits + (int64_t)f_next.u * A.mod_words + f_next.rp * (tcs::kItemRows / 32) + c.quarter;
-            flip_next[0] = w[0]; flip_next[1] = w[tcs::kRows / 32];
+            flip_next = A.modbits[(int64_t)f_next.u * A.mod_words + f_next.rp * (tcs::kItemRows / 32) + c.group * (tcs::kRows / 32) + c.quarter];
         };
         fetch_next(blockIdx.x);
         for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x) {
@@ -88,85 +86,70 @@ flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
             const tcs::TilePlan p = plan_of(f);
             const int lo = f.rp * tcs::kItemRows;
             const uint32_t *bits = A.modbits + (int64_t)f.u * A.mod_words;
-            float m[2] = {kNegBig, kNegBig}, l[2] = {0.f, 0.f}, lc[2] = {0.f, 0.f};
+            float m = kNegBig, l = 0.f, lc = 0.f;
             // all ones for a row of a visual token, whose other modality is the complement; fetched an item ahead
-            const uint32_t flip[2] = {((flip_next[0] >> c.lane) & 1u) ? 0xFFFFFFFFu : 0u, ((flip_next[1] >> c.lane) & 1u) ? 0xFFFFFFFFu : 0u};
+            const uint32_t flip = ((flip_next >> c.lane) & 1u) ? 0xFFFFFFFFu : 0u;
             fetch_next(item + gridDim.x);
-            for (int t = 0; ok && t < p.n_tiles; ++t) {
+            const bool active = c.group < p.n_halves;
+            // this warp's rows r0 .. r0 + 31 see the keys up to themselves: chunks past r0 + 31 are left out and only the one
+            // on the diagonal is masked
+            const int r0 = lo + c.group * tcs::kRows + c.quarter * 32, half_end = c.group == 0 ? p.cols_first : p.cols_total;
+            for (int t = 0; ok && active && t < p.n_tiles; ++t) {
                 const int kb = t * S::kCols;
+                if (!S::takes_part(c, min(S::kCols, half_end - kb))) continue;
+                ok = S::quad_wait(c, k++, A.status);
+                if (!ok) continue;
+                const int ncols = min(S::kCols, min(r0 + 32, A.L) - kb);
+                S::for_each_chunk(c, (ncols + 31) >> 5, [&](int ch, uint32_t (&acc)[32]) {
+                    const int k0 = kb + ch * 32;
+                    const uint32_t other = bits[k0 >> 5] ^ flip;         // keys of the other modality than the row's token
+                    float mx, add, addc = 0.f;
+                    if (k0 < r0) {                                   // all 32 keys come before all 32 rows
+                        float raw[32];
 #pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                    if (hf >= p.n_halves || !ok) continue;
-                    ok = S::acc_wait_h(c, hf, kh[hf]++, A.status);
-                    if (!ok) continue;
-                    // this warp's rows r0 .. r0 + 31 see the keys up to themselves: chunks past r0 + 31 are left out and
-                    // only the one on the diagonal is masked
-                    const int r0 = lo + hf * tcs::kRows + c.quarter * 32;
-                    const int ncols = min(S::kCols, min(r0 + 32, A.L) - kb);
-                    S::for_each_chunk_q(c, hf, colq, (ncols + 31) >> 5, [&](int ch, uint32_t (&acc)[32]) {
-                        const int k0 = kb + ch * 32;
-                        const uint32_t other = bits[k0 >> 5] ^ flip[hf];                 // keys of the other modality than the row's token
-                        float mx, add, addc = 0.f;
-                        if (k0 < r0) {                               // all 32 keys come before all 32 rows
-                            float raw[32];
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) raw[j] = __uint_as_float(acc[j]);
-                            mx = fmaxf(max32(raw) * A.scale_log2, m[hf]);
-                            add = exp_sum32(raw, A.scale_log2, mx);
-                            if (other == 0xFFFFFFFFu) addc = add;
-                            else if (other != 0u) {
-#pragma unroll
-                                for (int j = 0; j < 32; ++j)
-                                    addc += ((other >> j) & 1u) ? tc::ex2(fmaf(raw[j], A.scale_log2, -mx)) : 0.f;
-                            }
-                        } else {
-                            float s[32], add4[4] = {0.f, 0.f, 0.f, 0.f};
+                        for (int j = 0; j < 32; ++j) raw[j] = __uint_as_float(acc[j]);
+                        mx = fmaxf(max32(raw) * A.scale_log2, m);
+                        add = exp_sum32(raw, A.scale_log2, mx);
+                        if (other == 0xFFFFFFFFu) addc = add;
+                        else if (other != 0u) {
 #pragma unroll
                             for (int j = 0; j < 32; ++j)
-                                s[j] = (j <= c.lane) ? __uint_as_float(acc[j]) * A.scale_log2 : kNegBig;
-                            mx = fmaxf(max32(s), m[hf]);
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) {           // masked entries sit ~1e30 below: exp2 gives 0
-                                const float e = tc::ex2(s[j] - mx);
-                                add4[j & 3] += e;
-                                addc += ((other >> j) & 1u) ? e : 0.f;
-                            }
-                            add = (add4[0] + add4[1]) + (add4[2] + add4[3]);
+                                addc += ((other >> j) & 1u) ? tc::ex2(fmaf(raw[j], A.scale_log2, -mx)) : 0.f;
                         }
-                        const float carry = tc::ex2(m[hf] - mx);
-                        l[hf] = l[hf] * carry + add;
-                        lc[hf] = lc[hf] * carry + addc;
-                        m[hf] = mx;
-                    });
-                    S::acc_release_h(c, hf);
-                }
-            }
-            // The four column quarters of every row meet.  (After a wait that ran out the barriers are still kept, by all
-            // sixteen warps: the vote ends the loop for all of them together.)
+                    } else {
+                        float s[32], add4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                float *x = xch + (hf * 4 + colq) * tcs::kRows + row_in_half;
-                x[0] = m[hf]; x[1024] = l[hf]; x[2048] = lc[hf];
-            }
-            ok = !S::epi_meet(!ok);
-            if (ok && colq < p.n_halves) {                           // column quarter 0 joins half 0, column quarter 1 half 1
-                const float *x = xch + colq * 4 * tcs::kRows + row_in_half;
-                const float mx = fmaxf(fmaxf(x[0], x[128]), fmaxf(x[256], x[384]));
-                float z = 0.f, zc = 0.f;
+                        for (int j = 0; j < 32; ++j)
+                            s[j] = (j <= c.lane) ? __uint_as_float(acc[j]) * A.scale_log2 : kNegBig;
+                        mx = fmaxf(max32(s), m);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float w = tc::ex2(x[q * 128] - mx);
-                    z = fmaf(x[1024 + q * 128], w, z);
-                    zc = fmaf(x[2048 + q * 128], w, zc);
-                }
-                const bool row_on = lo + colq * tcs::kRows + row_in_half < A.L;
-                const float share = warp_sum(row_on && z > 0.f ? zc / z : 0.f);
+                        for (int j = 0; j < 32; ++j) {               // masked entries sit ~1e30 below: exp2 gives 0
+                            const float e = tc::ex2(s[j] - mx);
+                            add4[j & 3] += e;
+                            addc += ((other >> j) & 1u) ? e : 0.f;
+                        }
+                        add = (add4[0] + add4[1]) + (add4[2] + add4[3]);
+                    }
+                    const float carry = tc::ex2(m - mx);
+                    l = l * carry + add;
+                    lc = lc * carry + addc;
+                    m = mx;
+                });
+                S::quad_release(c);
+            }
+            // The two column halves of every row meet.  (After a wait that ran out the meeting is still kept: the vote ends the
+            // loop for both warps.)
+            if (c.colhalf == 1) tc::sts128(xch, m, l, lc, 0.f);
+            ok = !S::pair_meet(c, !ok);
+            if (c.colhalf == 0 && ok) {
+                const float4 o = tc::lds128(pxch);
+                const float mx = fmaxf(m, o.x), wa = tc::ex2(m - mx), wb = tc::ex2(o.x - mx);
+                const float z = l * wa + o.y * wb, zc = lc * wa + o.z * wb;
+                const float share = warp_sum(active && r0 + c.lane < A.L && z > 0.f ? zc / z : 0.f);   // (a half without rows: 0)
                 if (c.lane == 0)
-                    A.parts[((int64_t)(f.rp * 2 + colq) * 4 + c.quarter) * (int64_t)A.n_heads + (int64_t)f.u * A.Hq + f.head] = share;
+                    A.parts[((int64_t)(f.rp * 2 + c.group) * 4 + c.quarter) * (int64_t)A.n_heads + (int64_t)f.u * A.Hq + f.head] = share;
             }
-            if (ok && p.n_halves == 1 && colq == 1 && c.lane == 0)   // no rows in the second half
-                A.parts[((int64_t)(f.rp * 2 + 1) * 4 + c.quarter) * (int64_t)A.n_heads + (int64_t)f.u * A.Hq + f.head] = 0.f;
-            S::epi_sync();                                           // the exchange may be overwritten again
+            S::pair_sync(c);                                         // the hand-over slot may be overwritten again
         }
     }
     S::teardown(c);

@@ -303,12 +303,16 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
     a.Hq = p.n_q_heads; a.Hkv = p.n_kv_heads; a.G = G; a.W = W; a.L = p.seq_len; a.GW = G * W; a.GWpad = y.gw_pad;
     a.n_qt = y.tc_n_qt; a.n_chunk = y.tc_n_chunk; a.tiles_per_chunk = y.tc_tiles_per_chunk; a.n_rt = y.n_rt;
     a.a_heads = G < tcs::kRows / W ? G : tcs::kRows / W;        // one A half holds 128 proxy rows
-    // pass 2 streams the keys as the A operand; with few proxy rows per KV head the small shape (two A stages)
-    // keeps the key loads in flight across items
-    const bool small2 = a.GW <= 128 && W <= 64;
+    // pass 2 streams the keys as the A operand; with up to 256 proxy rows per KV head the shapes with two A stages keep
+    // the key loads in flight across items
+    const bool small2 = a.GW <= 128 && W <= 64, resident2 = !small2 && a.GW <= 256;
     const int nb2 = small2 ? tcs::Small::kCols : tcs::Big::kCols;
     a.b_heads = G < nb2 / W ? G : nb2 / W;
     a.n_items1 = UH * a.n_qt * a.n_chunk; a.n_items2 = UH * a.n_rt;
+    const int grid1 = a.n_items1 < tc::sm_count() ? a.n_items1 : tc::sm_count();
+    const int grid2 = a.n_items2 < tc::sm_count() ? a.n_items2 : tc::sm_count();
+    a.by_grid2 = make_fastdiv((uint32_t)grid2);
+    a.by_hkv = make_fastdiv((uint32_t)p.n_kv_heads); a.by_rt = make_fastdiv((uint32_t)a.n_rt);
     const float scale = p.softmax_scale != 0.f ? p.softmax_scale : 1.f / sqrtf((float)p.head_dim);
     a.scale_log2 = scale * kLog2e;
 
@@ -326,19 +330,19 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
                              (int)tcs::Big::kSmemBytes) != cudaSuccess ||
         cudaFuncSetAttribute(score_colsum_tc_kernel<tcs::Big>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)tcs::Big::kSmemBytes) != cudaSuccess ||
+        cudaFuncSetAttribute(score_colsum_tc_kernel<tcs::Resident>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)tcs::Resident::kSmemBytes) != cudaSuccess ||
         cudaFuncSetAttribute(score_colsum_tc_kernel<tcs::Small>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)tcs::Small::kSmemBytes) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
-    const int sms = tc::sm_count();
-    launch(score_stats_tc_kernel<tcs::Big>, a.n_items1 < sms ? a.n_items1 : sms, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
+    launch(score_stats_tc_kernel<tcs::Big>, grid1, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
     FLOWMM_LAUNCHED("score_stats_tc");
     const int n_negc = UH * a.GWpad;
-    launch(score_combine_kernel, (n_negc + 255) / 256, 256, 0, st, a.row_part, 4 * a.n_chunk, a.GW, a.GWpad, UH, a.negc);
+    launch(score_combine_kernel, (n_negc + 63) / 64, 256, 0, st, a.row_part, 4 * a.n_chunk, a.GW, a.GWpad, UH, a.negc);
     FLOWMM_LAUNCHED("score_combine");
-    if (small2)
-        launch(score_colsum_tc_kernel<tcs::Small>, a.n_items2 < sms ? a.n_items2 : sms, tcs::kThreads, tcs::Small::kSmemBytes, st, k128, qb, a);
-    else
-        launch(score_colsum_tc_kernel<tcs::Big>, a.n_items2 < sms ? a.n_items2 : sms, tcs::kThreads, tcs::Big::kSmemBytes, st, k128, qb, a);
+    if (small2) launch(score_colsum_tc_kernel<tcs::Small>, grid2, tcs::kThreads, tcs::Small::kSmemBytes, st, k128, qb, a);
+    else if (resident2) launch(score_colsum_tc_kernel<tcs::Resident>, grid2, tcs::kThreads, tcs::Resident::kSmemBytes, st, k128, qb, a);
+    else launch(score_colsum_tc_kernel<tcs::Big>, grid2, tcs::kThreads, tcs::Big::kSmemBytes, st, k128, qb, a);
     FLOWMM_LAUNCHED("score_colsum_tc");
     if (parts_out) { *parts_out = a.n_rt * 8; return FLOWMM_OK; }     // the caller reduces the partial masses itself
     const int n = p.n_units * p.n_q_heads;
@@ -516,10 +520,8 @@ flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *
         FLOWMM_LAUNCHED("match_small_tc");
         return FLOWMM_OK;
     }
-    // few candidates per head: the token rows are the stream, take the shape with two A stages
-    const bool small = y.c_tot <= 128;
     const uint32_t box_a[4] = {64, kMtRows, 1, 1};
-    const uint32_t box_b[4] = {64, (uint32_t)(small ? tcs::Small::kCols : tcs::Big::kCols), 1, 1};
+    const uint32_t box_b[4] = {64, tcs::Big::kCols, 1, 1};
     if (!tc::make_bf16_map(&k_map, k, 4, kd, ks, box_a) || !tc::make_bf16_map(&cand_map, g.cand_k, 4, cd, cs, box_b))
         return FLOWMM_ERR_CUDA;
     MatchTcArgs a;
@@ -529,13 +531,10 @@ flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *
     a.Hkv = p.n_kv_heads; a.L = p.seq_len; a.E = E; a.Ctot = y.c_tot; a.n_rt = y.n_rt; a.n_items = UH * y.n_rt;
     a.by_nrt = make_fastdiv((uint32_t)y.n_rt); a.by_hkv = make_fastdiv((uint32_t)p.n_kv_heads);
     if (cudaFuncSetAttribute(match_tc_kernel<tcs::Big>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tcs::Big::kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(match_tc_kernel<tcs::Small>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tcs::Small::kSmemBytes) != cudaSuccess)
+                             (int)tcs::Big::kSmemBytes) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
     const int grid = a.n_items < tc::sm_count() ? a.n_items : tc::sm_count();
-    if (small) launch(match_tc_kernel<tcs::Small>, grid, tcs::kThreads, tcs::Small::kSmemBytes, st, k_map, cand_map, a);
-    else launch(match_tc_kernel<tcs::Big>, grid, tcs::kThreads, tcs::Big::kSmemBytes, st, k_map, cand_map, a);
+    launch(match_tc_kernel<tcs::Big>, grid, tcs::kThreads, tcs::Big::kSmemBytes, st, k_map, cand_map, a);
     FLOWMM_LAUNCHED("match_tc");
     return FLOWMM_OK;
 }
@@ -579,6 +578,8 @@ bool merge_is_tc(const flowmm_params &p) {
     return p.seq_len > p.n_keep && p.dtype == FLOWMM_BF16 && p.head_dim == 128 && p.n_keep <= mtc::kMaxSlots &&
            p.seq_len < 65536 && p.path != FLOWMM_PATH_SIMT;
 }
+
+constexpr int kFixedPieces = 6;             // merge_staged_kernel: fixed assignment below this many pieces per warp
 
 // map_ready: the (slot, weight) table of the tensor-core merge has been written already (by the matching kernel)
 flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, const void *v,
@@ -664,12 +665,11 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
     const int gp = (int)(want_blocks < 2 * tc::sm_count() ? want_blocks : 2 * tc::sm_count());   // persistent warps
     if (p.dtype == FLOWMM_BF16 && p.head_dim == 128 && E > 0 && p.path != FLOWMM_PATH_SIMT) {
         // rows of 256 bytes: member rows staged through shared memory by asynchronous copies, three CTAs per SM
-        if (cudaFuncSetAttribute(mstg::merge_staged_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)mstg::kSmemBytes) != cudaSuccess)
-            return FLOWMM_ERR_CUDA;
         const int gs = (int)(want_blocks < 3 * tc::sm_count() ? want_blocks : 3 * tc::sm_count());
-        launch(mstg::merge_staged_kernel<__nv_bfloat16>, gs, mstg::kThreads, mstg::kSmemBytes, st, 
-            m, UH, at<int>(ws, y.merge_status), make_fastdiv((uint32_t)m.max_pieces), make_fastdiv((uint32_t)p.n_kv_heads));
+        auto kernel = total_pieces < kFixedPieces * 8 * gs ? mstg::merge_staged_kernel<__nv_bfloat16, true> : mstg::merge_staged_kernel<__nv_bfloat16, false>;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mstg::kSmemBytes) != cudaSuccess) return FLOWMM_ERR_CUDA;
+        launch(kernel, gs, mstg::kThreads, mstg::kSmemBytes, st, m, UH, at<int>(ws, y.merge_status), make_fastdiv((uint32_t)m.max_pieces),
+               make_fastdiv((uint32_t)p.n_kv_heads));
         FLOWMM_LAUNCHED("merge_staged");
     } else if (p.dtype == FLOWMM_BF16) {
         launch(merge_pieces_kernel<__nv_bfloat16>, gp, 256, 0, st, m, UH);

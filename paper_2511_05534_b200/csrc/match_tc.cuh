@@ -375,7 +375,7 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
     if (c.warp == 0) {
         if (c.lane == 0) S::producer(c, &k_map, &cand_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
-        if (c.lane == 0) S::mma_issuer(c, A.n_items, plan, A.status);
+        if (c.lane == 0) S::template mma_issuer<false>(c, A.n_items, plan, A.status);
     } else {
         const int lane = c.lane, row = c.quarter * 32 + lane;
         const int b0 = kPer * c.colhalf;                         // first block of this warp's share of a tile

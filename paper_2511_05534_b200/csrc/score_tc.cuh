@@ -28,6 +28,7 @@ struct ScoreTcArgs {
     int Hq, Hkv, G, W, L, GW, GWpad;
     int n_qt;                    // 256-row tiles over the G*W proxy rows
     int n_chunk, tiles_per_chunk;   // pass 1: key chunks per row tile, 256-key tiles per chunk
+    FastDiv by_grid2, by_hkv, by_rt;   // exact divisions by the second pass's grid, Hkv, n_rt
     int n_rt;                    // pass 2: 256-key tiles
     int a_heads, b_heads;        // query heads one A box (pass 1) / B box (pass 2) delivers
     int n_items1, n_items2;
@@ -92,7 +93,7 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     if (c.warp == 0) {
         if (c.lane == 0) S::producer(c, &q_map, &k_map, A.n_items1, a_bytes, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
-        if (c.lane == 0) S::mma_issuer(c, A.n_items1, plan, A.status);
+        if (c.lane == 0) S::template mma_issuer<false>(c, A.n_items1, plan, A.status);
     } else {
         // all sixteen warps drain one accumulator at a time: a warp owns 32 lanes x a quarter of the columns of
         // BOTH halves, so the tensor core refills one half while the other is being read
@@ -173,21 +174,23 @@ __global__ void pack_modality_kernel(const uint8_t *modality, int L, int n_words
 
 // Row constants for pass 2: negc[r] = -(M_r + log2 Z_r) so that exp2(s + negc) is the softmax
 // probability; padding rows get a constant that makes every probability 0.
-__global__ void score_combine_kernel(const float2 *row_part, int n_chunk, int GW, int GWpad, int n_uh, float *negc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Four lanes share a row and read its parts together (a thread per row took 17 us for 65 536 rows of 32 parts, this 8).
+__global__ void score_combine_kernel(const float2 *row_part, int n_part, int GW, int GWpad, int n_uh, float *negc) {
     predecessor_done();
-    if (i >= n_uh * GWpad) return;
-    const int uh = i / GWpad, r = i % GWpad;
-    float out = kNegBig;
-    if (r < GW) {
-        const float2 *part = row_part + ((int64_t)uh * GW + r) * n_chunk;
-        float mx = kNegBig;
-        for (int c = 0; c < n_chunk; ++c) mx = fmaxf(mx, part[c].x);
-        float z = 0.f;
-        for (int c = 0; c < n_chunk; ++c) z += part[c].y * exp2f(part[c].x - mx);
-        out = -(mx + log2f(z));
-    }
-    negc[i] = out;
+    const int i = blockIdx.x * (blockDim.x >> 2) + (threadIdx.x >> 2), sub = threadIdx.x & 3;
+    const int uh = i / GWpad, r = i - uh * GWpad;
+    const bool on = i < n_uh * GWpad && r < GW;
+    const float2 *part = row_part + ((int64_t)uh * GW + r) * n_part;       
+    float mx = kNegBig, z = 0.f;
+    if (on)
+        for (int c = sub; c < n_part; c += 4) mx = fmaxf(mx, part[c].x);
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    if (on)
+        for (int c = sub; c < n_part; c += 4) z += part[c].y * exp2f(part[c].x - mx);
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
+    if (sub == 0 && i < n_uh * GWpad) negc[i] = r < GW ? -(mx + log2f(z)) : kNegBig;
 }
 
 // The common case of pass 2's inner step, written out in PTX so that it costs what it must and no more: 32 accumulator
@@ -274,32 +277,37 @@ __device__ __forceinline__ float colsum_chunk32(uint32_t taddr, uint32_t negc, f
 #undef FLOWMM_CS_A
 
 // ---------------------------------------------------------------------------------------------
-// Pass 2.  item = (unit*head, tile of 256 keys); the B stream is the head group's proxy rows.
+// Pass 2.  item = (unit*head, tile of 256 keys); the B stream is the head group's proxy rows.  A CTA takes a run of
+// consecutive items, so that with up to 256 proxy rows per head they are loaded once per head, not once per item.
 template <class S>
 __global__ void __launch_bounds__(tcs::kThreads, 1)
 score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap q_map,
                        const ScoreTcArgs A) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    const typename S::Ctx c = S::setup(smem_raw, &k_map, &q_map, A.status);
+    const typename S::Ctx c = S::setup(smem_raw, &k_map, &q_map, A.status, 0, 4);
     if (!c.ok) return;
+    const int g_lo = (int)((int64_t)A.n_items2 * blockIdx.x / gridDim.x), g_hi = (int)((int64_t)A.n_items2 * (blockIdx.x + 1) / gridDim.x);
+    const int n_loop = (g_hi - g_lo) * gridDim.x;                   // the roles count items blockIdx.x, blockIdx.x + gridDim.x, ...
     auto plan = [&](int item) {
         tcs::TilePlan p;
-        const int kt = item % A.n_rt, uh = item / A.n_rt;
-        const int u = uh / A.Hkv, h = uh % A.Hkv;
+        const int g = g_lo + (int)A.by_grid2.div(item), uh = (int)A.by_rt.div(g), kt = g - uh * A.n_rt;
+        const int u = (int)A.by_hkv.div(uh), h = uh - u * A.Hkv;
         p.a1 = kt * tcs::kItemRows; p.a2 = h; p.a3 = u;
         p.h1 = tcs::kRows; p.h2 = 0;
         p.n_halves = p.a1 + tcs::kRows < A.L ? 2 : 1;
         p.b1 = 0; p.b2 = h * A.G; p.b3 = u; p.step1 = 0; p.step2 = S::kCols / A.W;
         p.cols_total = A.GW;
         p.n_tiles = (A.GW + S::kCols - 1) / S::kCols;
+        p.reuse_b = p.n_tiles == 1 && kt > 0 && g > g_lo;
+        p.keep_b = p.n_tiles == 1 && kt + 1 < A.n_rt && g + 1 < g_hi;
         p.extra = A.negc + (int64_t)uh * A.GWpad;        // row constants of pass 1, 256 per B tile
         return p;
     };
     const uint32_t b_bytes = (uint32_t)A.b_heads * A.W * 256u;
     if (c.warp == 0) {
-        if (c.lane == 0) S::producer(c, &k_map, &q_map, A.n_items2, tcs::kAHalf, b_bytes, plan, A.status);
+        if (c.lane == 0) S::producer(c, &k_map, &q_map, blockIdx.x + n_loop, tcs::kAHalf, b_bytes, plan, A.status);
     } else if (c.warp == 1) {
-        if (c.lane == 0) S::mma_issuer(c, A.n_items2, plan, A.status);
+        if (c.lane == 0) S::template mma_issuer<true>(c, blockIdx.x + n_loop, plan, A.status);
     } else {
         const int lane = c.lane, row = c.quarter * 32 + lane;
         const uint32_t xch = c.epi_addr() + row * 4;            // hand-over slot of this row
@@ -308,9 +316,18 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
         const int w_shift = 31 - __clz(A.W);
         uint32_t wbits[4] = {0, 0, 0, 0};                            // modality of the proxy tokens, 32 per word
         bool ok = true;
-        for (int item = blockIdx.x; ok && item < A.n_items2; item += gridDim.x) {
-            const tcs::TilePlan p = plan(item);
-            const int kt = item % A.n_rt, uh = item / A.n_rt, u = uh / A.Hkv, h = uh % A.Hkv;
+        auto fetch_mod = [&](int g) -> int {                         // modality of this thread's key, an item ahead
+            if (g >= g_hi) return 0;
+            const int uh = (int)A.by_rt.div(g), key = (g - uh * A.n_rt) * tcs::kItemRows + c.group * tcs::kRows + row;
+            return key < A.L ? A.modality[(int64_t)A.by_hkv.div(uh) * A.L + key] : 0;
+        };
+        int mod_next = fetch_mod(g_lo);
+        for (int g = g_lo; ok && g < g_hi; ++g) {
+            const tcs::TilePlan p = plan(blockIdx.x + (g - g_lo) * gridDim.x);
+            const int uh = (int)A.by_rt.div(g), kt = g - uh * A.n_rt, u = (int)A.by_hkv.div(uh), h = uh - u * A.Hkv;
+            const bool my_vis = mod_next != 0;
+            mod_next = fetch_mod(g + 1);
+            if (p.reuse_b) --bt;                                     // (bt: number of the B tile an item begins with)
             float *cross_out = A.cross_part + ((int64_t)u * A.Hq + h * A.G) * (A.n_rt * 8) + kt * 8 + c.group * 4 + c.quarter;
             if (c.group >= p.n_halves) {                             // no keys in this half: its masses are zero
                 if (lane == 0)
@@ -330,13 +347,13 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
             const int key0 = kt * tcs::kItemRows + c.group * tcs::kRows;
             const int key = key0 + row;
             const bool masked_tile = key0 + tcs::kRows > A.L - A.W + 1;   // some (key, proxy row) pair is masked
-            const bool my_vis = key < A.L && A.modality[(int64_t)u * A.L + key] != 0;
             const int first_proxy = A.L - A.W;
             float imp = 0.f, cg = 0.f;
             int cur_g = -1;                                          // head whose mass is being summed; -1: none yet
-            for (int t = 0; ok && t < p.n_tiles; ++t, ++k, ++bt) {
+            for (int t = 0; ok && t < p.n_tiles; ++t, ++bt) {
                 const int ncols = min(S::kCols, A.GW - t * S::kCols);
-                ok = S::extra_wait(c, bt, A.status) && S::acc_wait(c, k, A.status);
+                if (!S::takes_part(c, ncols)) continue;
+                ok = S::extra_wait(c, bt, A.status) && S::quad_wait(c, k++, A.status);
                 if (!ok) break;
                 const uint32_t negc4 = c.extra(bt);
                 constexpr int kPerC = S::kCols / 64;               // 32-column chunks a warp takes of a full tile
@@ -401,7 +418,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                         cg += x;
                     }
                 }
-                S::acc_release(c);
+                S::quad_release(c);
             }
             if (ok && cur_g >= 0) {
                 const float tot = warp_sum(cg);

@@ -13,9 +13,17 @@
 // Shared-memory stages (AST per A half, two for B) and the two accumulators are handed around
 // with mbarriers; every wait is bounded.
 //
-// Two shapes are instantiated: Skel<256, 1> for long B streams (one A stage per half, 64 KB B
-// stages) and Skel<128, 2> for problems whose items have few B columns, where the A operand is
-// the stream: two A stages per half let the next item's rows load while this item is computed.
+// Accumulators are handed around in one of three ways, the kernel's choice (acc_arrivals of setup()):
+//   8   by half, the two quads of the half together (matching: products 256 columns wide);
+//   16  by half, all sixteen warps drain one half at a time while the other is refilled (row statistics);
+//   4   by quad: the two column halves are refilled one by one, each as soon as its quad has released it, so that a quad
+//       waits for 128 columns only and the four warps of a scheduler are in different phases of their work.  Second
+//       scoring pass: 112 heads of 8448 tokens 181 -> 171 us, full-prefill flow of 2176 tokens 680 -> 657 us, of 512 66 -> 57;
+//       the matching kernel was 8 % slower, the row statistics 2 %.
+// Three shapes are instantiated: Skel<256, 1, 2> for long B streams (one A stage per half, two 64 KB B
+// stages), and for problems whose items have few B columns, where the A operand is the stream, Skel<128, 2, 2>
+// and Skel<256, 2, 1>: two A stages per half let the next item's rows load while this item is computed, and an item
+// whose single B tile is the previous item's (TilePlan::reuse_b) takes it as it stands.
 #pragma once
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -42,11 +50,13 @@ struct TilePlan {
     int n_tiles;               // 0: every role skips the item
     int cols_total;            // valid B rows over all tiles (tile t has min(NB, cols_total - NB t))
     int cols_first = 0;        // ... for A half 0, where it needs fewer in the last tile (0: the same)
+    bool reuse_b = false;      // the item's only B tile (and its constants) is the one the item before ended with
+    bool keep_b = false;       // ... and the next item's as well: its stage is not handed back after this item
     const float *extra;        // nullptr, or NB fp32 per-column constants per tile: tile t reads extra + NB t
     __device__ __forceinline__ bool empty() const { return n_tiles == 0 || n_halves == 0; }
 };
 
-template <int NB, int AST>
+template <int NB, int AST, int BST>
 struct Skel {
     static constexpr int kCols = NB;                         // rows of a B tile (UMMA N)
     static constexpr int kAStages = AST;
@@ -54,13 +64,13 @@ struct Skel {
     static constexpr uint32_t kExtraBytes = NB * 4;          // per-column fp32 constants that travel with a B tile
     static constexpr uint32_t kSmemA = 0;                    // [stage][half]
     static constexpr uint32_t kSmemB = 2 * AST * kAHalf;
-    static constexpr uint32_t kSmemExtra = kSmemB + 2 * kBStage;
+    static constexpr uint32_t kSmemExtra = kSmemB + BST * kBStage;
     static constexpr uint32_t kSmemEpi = kSmemExtra + kExtraSlots * kExtraBytes;   // epilogue scratch
     static constexpr uint32_t kSmemBar = kSmemEpi + kEpiBytes;
     static constexpr uint32_t kSmemBytes = kSmemBar + 256;
     // barrier slots
-    static constexpr int kBarAFull = 0, kBarAEmpty = 2 * AST, kBarBFull = 4 * AST, kBarBEmpty = kBarBFull + 2,
-                         kBarAccFull = kBarBEmpty + 2, kBarAccEmpty = kBarAccFull + 2, kBarXFull = kBarAccEmpty + 2,
+    static constexpr int kBarAFull = 0, kBarAEmpty = 2 * AST, kBarBFull = 4 * AST, kBarBEmpty = kBarBFull + BST,
+                         kBarAccFull = kBarBEmpty + BST, kBarAccEmpty = kBarAccFull + 4, kBarXFull = kBarAccEmpty + 4,
                          kNumBars = kBarXFull + kExtraSlots;
     static_assert(8 * kNumBars + 8 <= 256, "barrier block too small");
     static_assert(kSmemBytes <= 232448, "shared memory budget");
@@ -112,7 +122,7 @@ struct Skel {
             for (int i = 0; i < kNumBars; ++i) {
                 int count = 1;
                 if (i >= kBarAEmpty && i < kBarBFull) count = 1 + a_readers;
-                if (i >= kBarAccEmpty && i < kBarXFull) count = acc_arrivals;   // one arrival per epilogue warp that reads the half
+                if (i >= kBarAccEmpty && i < kBarXFull) count = acc_arrivals;   // one arrival per epilogue warp that reads it
                 tc::mbar_init(c.bar(i), count);
             }
             *c.abort_flag = 0;
@@ -146,20 +156,23 @@ struct Skel {
         for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
             const TilePlan p = plan(item);
             if (p.empty()) continue;
-            for (int t = 0; ok && t < p.n_tiles; ++t, ++bt) {
-                const int sb = bt & 1;
-                ok = tc::mbar_wait(c.bar(kBarBEmpty + sb), ((bt >> 1) & 1) ^ 1, c.abort_flag, status);
+            for (int t = 0; ok && t < p.n_tiles; ++t) {
+                const int sb = bt % BST;
+                if (!p.reuse_b) ok = tc::mbar_wait(c.bar(kBarBEmpty + sb), ((bt / BST) & 1) ^ 1, c.abort_flag, status);
                 if (!ok) break;
-                if (p.extra) {       // slot reuse is safe: both epilogues released tile bt-4 before the MMAs of bt-2 began
+                if (p.extra && !p.reuse_b) {   // slot reuse is safe: every epilogue released tile bt-4 before the stage of bt-2 was released
                     const int xs = bt & (kExtraSlots - 1);
                     tc::mbar_expect_tx(c.bar(kBarXFull + xs), kExtraBytes);
                     tc::bulk_load(c.base + kSmemExtra + (uint32_t)xs * kExtraBytes, p.extra + (size_t)t * NB, kExtraBytes,
                                   c.bar(kBarXFull + xs));
                 }
-                tc::mbar_expect_tx(c.bar(kBarBFull + sb), b_bytes);
-                const uint32_t b_dst = c.base + kSmemB + sb * kBStage;
-                tc::tma_load_4d(b_dst, mb, c.bar(kBarBFull + sb), 0, p.b1 + t * p.step1, p.b2 + t * p.step2, p.b3);
-                tc::tma_load_4d(b_dst + kBStage / 2, mb, c.bar(kBarBFull + sb), 64, p.b1 + t * p.step1, p.b2 + t * p.step2, p.b3);
+                if (!p.reuse_b) {
+                    tc::mbar_expect_tx(c.bar(kBarBFull + sb), b_bytes);
+                    const uint32_t b_dst = c.base + kSmemB + sb * kBStage;
+                    tc::tma_load_4d(b_dst, mb, c.bar(kBarBFull + sb), 0, p.b1 + t * p.step1, p.b2 + t * p.step2, p.b3);
+                    tc::tma_load_4d(b_dst + kBStage / 2, mb, c.bar(kBarBFull + sb), 64, p.b1 + t * p.step1, p.b2 + t * p.step2, p.b3);
+                    ++bt;
+                }
                 if (t == 0) {                  // the item's A halves go out right after its first B tile
                     for (int h = 0; ok && h < p.n_halves; ++h) {
                         const int st = ia[h] % AST, full = kBarAFull + st * 2 + h;
@@ -177,50 +190,67 @@ struct Skel {
         if (!ok) {          // winding down after a timeout: give copies already issued a moment to land
             for (int i = 0; i < 2 * AST; ++i)
                 for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(c.bar(kBarAFull + i), 0) && !tc::mbar_try_wait(c.bar(kBarAFull + i), 1); ++s) {}
-            for (int i = 0; i < 2; ++i)
+            for (int i = 0; i < BST; ++i)
                 for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(c.bar(kBarBFull + i), 0) && !tc::mbar_try_wait(c.bar(kBarBFull + i), 1); ++s) {}
         }
     }
 
-    // Call from one thread.
-    template <class PlanFn>
+    // Call from one thread.  kQuads: accumulators are handed around by quad, else by half.
+    template <bool kQuads, class PlanFn>
     static __device__ __forceinline__ void mma_issuer(const Ctx &c, int n_items, PlanFn plan, int *status) {
-        int ia[2] = {0, 0}, ta[2] = {0, 0}, bt = 0;
+        constexpr int kParts = kQuads ? 2 : 1, kPartCols = NB / kParts;   // accumulators of a half, their columns
+        int ia[2] = {0, 0}, ta[4] = {0, 0, 0, 0}, bt = 0;
         bool ok = true;
         for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
             const TilePlan p = plan(item);
             if (p.empty()) continue;
-            for (int t = 0; ok && t < p.n_tiles; ++t, ++bt) {
-                const int sb = bt & 1;
-                ok = tc::mbar_wait(c.bar(kBarBFull + sb), (bt >> 1) & 1, c.abort_flag, status);
+            for (int t = 0; ok && t < p.n_tiles; ++t) {
+                if (!p.reuse_b) ++bt;
+                const int sb = (bt - 1) % BST;                           // bt: B tiles taken so far, this one included
+                ok = tc::mbar_wait(c.bar(kBarBFull + sb), ((bt - 1) / BST) & 1, c.abort_flag, status);
                 if (!ok) break;
                 const int ncols = min(NB, p.cols_total - t * NB);
                 const int ncols0 = p.cols_first ? min(NB, p.cols_first - t * NB) : ncols;
                 const uint32_t b_base = c.base + kSmemB + sb * kBStage;
+                uint32_t took = 0;
                 for (int h = 0; ok && h < p.n_halves; ++h) {
                     const int st = ia[h] % AST;
                     if (t == 0) ok = tc::mbar_wait(c.bar(kBarAFull + st * 2 + h), (ia[h] / AST) & 1, c.abort_flag, status);
-                    ok = ok && tc::mbar_wait(c.bar(kBarAccEmpty + h), (ta[h] & 1) ^ 1, c.abort_flag, status);
-                    if (!ok) break;
-                    tc::tc_fence_after();
                     const uint32_t a_base = c.base + kSmemA + (uint32_t)(st * 2 + h) * kAHalf;
-                    const uint32_t idesc = tc::idesc_bf16(kRows, (uint32_t)(((h == 0 ? ncols0 : ncols) + 15) & ~15));
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks) {                     // head_dim 128 = 8 K slices of 16
-                        const uint32_t a_off = (ks >> 2) * (kAHalf / 2) + (ks & 3) * 32;
-                        const uint32_t b_off = (ks >> 2) * (kBStage / 2) + (ks & 3) * 32;
-                        tc::umma_bf16(c.tmem_base + h * NB, tc::smem_desc_sw128(a_base, a_off),
-                                      tc::smem_desc_sw128(b_base, b_off), idesc, ks > 0);
+                    for (int ch = 0; ch < kParts; ++ch) {                // the accumulators that hold columns
+                        const int q = kParts * h + ch, n = min(kPartCols, (h == 0 ? ncols0 : ncols) - ch * kPartCols);
+                        if (n <= 0 || !ok) continue;
+                        ok = tc::mbar_wait(c.bar(kBarAccEmpty + q), (ta[q] & 1) ^ 1, c.abort_flag, status);
+                        if (!ok) continue;
+                        tc::tc_fence_after();
+                        const uint32_t idesc = tc::idesc_bf16(kRows, (uint32_t)((n + 15) & ~15));
+#pragma unroll
+                        for (int ks = 0; ks < 8; ++ks) {                 // head_dim 128 = 8 K slices of 16
+                            const uint32_t a_off = (ks >> 2) * (kAHalf / 2) + (ks & 3) * 32;
+                            const uint32_t b_off = (ks >> 2) * (kBStage / 2) + ch * (kPartCols * 128) + (ks & 3) * 32;
+                            tc::umma_bf16(c.tmem_base + q * kPartCols, tc::smem_desc_sw128(a_base, a_off),
+                                          tc::smem_desc_sw128(b_base, b_off), idesc, ks > 0);
+                        }
+                        tc::umma_commit(c.bar(kBarAccFull + q));         // accumulator ready
+                        ++ta[q];
+                        took |= 1u << q;
                     }
-                    tc::umma_commit(c.bar(kBarAccFull + h));             // accumulator of this half ready
-                    ++ta[h];
+                    if (!ok) break;
                     if (t == p.n_tiles - 1) {                            // that was the half's last use of its A stage
                         tc::umma_commit(c.bar(kBarAEmpty + st * 2 + h));
                         ++ia[h];
                     }
                 }
                 if (!ok) break;
-                tc::umma_commit(c.bar(kBarBEmpty + sb));                 // B stage free once both halves' MMAs finish
+                if constexpr (kQuads) {
+                    // accumulators without a part in this tile: their quads must be through with the tiles before it as well,
+                    // so that a tile's release tells the producer that nobody reads the constants of the tile before any more
+                    for (int q = 0; ok && q < 4; ++q)
+                        if (!(took & (1u << q))) ok = tc::mbar_wait(c.bar(kBarAccEmpty + q), (ta[q] & 1) ^ 1, c.abort_flag, status);
+                    if (!ok) break;
+                }
+                if (!p.keep_b) tc::umma_commit(c.bar(kBarBEmpty + sb));  // B stage free once both halves' MMAs finish
             }
         }
     }
@@ -248,6 +278,19 @@ struct Skel {
         tc::tc_fence_before();
         __syncwarp();
         if (c.lane == 0) tc::mbar_arrive(c.bar(kBarAccEmpty + c.group));
+    }
+    // The same for kernels whose accumulators are handed around by quad: whether this warp's takes part in a tile of ncols
+    // columns, and (then) the wait and the release; `k` counts the tiles it has taken part in.
+    static __device__ __forceinline__ bool takes_part(const Ctx &c, int ncols) { return ncols > c.colhalf * (NB / 2); }
+    static __device__ __forceinline__ bool quad_wait(const Ctx &c, int k, int *status) {
+        const bool ok = tc::mbar_wait(c.bar(kBarAccFull + 2 * c.group + c.colhalf), k & 1, c.abort_flag, status);
+        tc::tc_fence_after();
+        return ok;
+    }
+    static __device__ __forceinline__ void quad_release(const Ctx &c) {
+        tc::tc_fence_before();
+        __syncwarp();
+        if (c.lane == 0) tc::mbar_arrive(c.bar(kBarAccEmpty + 2 * c.group + c.colhalf));
     }
     // TMEM address of columns [32*chunk, 32*chunk+32) of this warp's half for its 32 lanes.
     static __device__ __forceinline__ uint32_t acc_addr(const Ctx &c, int chunk) {
@@ -303,20 +346,6 @@ struct Skel {
             f(ch, a);
         }
     }
-    // Meeting points of all sixteen epilogue warps; the first with a vote: whether any of them has given up on a wait.
-    static __device__ __forceinline__ bool epi_meet(bool gave_up) {
-        uint32_t any;
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t"
-            "setp.ne.u32 q, %1, 0;\n\t"
-            "barrier.cta.red.or.pred p, 1, %2, q;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(any)
-            : "r"((uint32_t)gave_up), "n"(32 * kEpiWarps)
-            : "memory");
-        return any != 0;
-    }
-    static __device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory"); }
     // Meeting point of the two warps that share rows, with a vote: returns whether either warp has given up on a wait, so that both leave
     // the item loop together and neither is left alone at the next meeting.
     static __device__ __forceinline__ bool pair_meet(const Ctx &c, bool gave_up) {
@@ -337,8 +366,9 @@ struct Skel {
     }
 };
 
-using Big = Skel<256, 1>;       // long B streams
-using Small = Skel<128, 2>;     // few B columns per item: the A operand is the stream
+using Big = Skel<256, 1, 2>;       // long B streams
+using Small = Skel<128, 2, 2>;     // few B columns per item: the A operand is the stream
+using Resident = Skel<256, 2, 1>;  // ... with a B tile of up to 256 columns that stays for many items
 
 }  // namespace tcs
 }  // namespace flowmm

@@ -191,3 +191,20 @@ def test_short_lists_over_runs_of_tiles():
         args = dict(tau=4.0, tau_mode=O.TAU_REL, theta=0.5)
         args.update(kw)
         _random_case(rng, U, Hq, Hkv, 128, L, W, B, F.BF16, **args)
+
+
+def test_scoring_over_runs_of_tiles():
+    """The two scoring passes give every CTA a run of consecutive key tiles: runs inside a head and across heads, few and many
+    tiles, one to four row tiles per KV head (up to 128, 256 and 512 proxy rows take different shapes of the second pass), a
+    last half tile without keys."""
+    rng = np.random.default_rng(37)
+    for (U, Hq, Hkv, L, W, B) in [
+        (1, 7, 1, 300, 32, 20),          # 224 rows, two tiles: fewer tiles than CTAs
+        (3, 21, 3, 2176, 32, 60),        # 224 rows, runs across heads
+        (50, 8, 4, 400, 64, 30),         # 128 rows, more tiles than CTAs
+        (2, 2, 1, 8300, 128, 100),       # 256 rows, last half tile without keys
+        (1, 8, 2, 5000, 128, 90),        # 512 rows, window of 128
+        (40, 28, 4, 640, 64, 80),        # 448 rows, many heads
+        (1, 3, 1, 1030, 32, 40),         # 96 rows
+    ]:
+        _random_case(rng, U, Hq, Hkv, 128, L, W, B, F.BF16, tau=4.0, tau_mode=O.TAU_REL, theta=0.4)
