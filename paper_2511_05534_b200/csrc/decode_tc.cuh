@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap, const Args A) {
     extern __shared__ __align__(1024) uint8_t dtc_smem[];
     const uint32_t base = tc::smem_u32(dtc_smem), bars = base + kSmemBar;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tc::warp_number(), lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(dtc_smem + kSmemBar + 8 * kNumBars + 4);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(dtc_smem + kSmemBar + 8 * kNumBars);
     if ((base & 1023u) != 0) {                      // the swizzled tiles need a 1024-byte aligned base
@@ -131,37 +131,44 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
                     for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + i), 0) && !tc::mbar_try_wait(bar(kBarFull + i), 1); ++s) {}
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            bool ok = tc::mbar_wait(bar(kBarQ), 0, abort_flag, A.status);
-            for (int t = 0; ok && t < nt; ++t) {
-                const int st = t % kStages;
-                ok = tc::mbar_wait(bar(kBarFull + st), (t / kStages) & 1, abort_flag, A.status);
-                if (!ok) break;
-                tc::tc_fence_after();
-                const uint32_t a = base + st * kStageBytes;
+        const uint32_t q_lo = tc::desc_lo(base + kSmemQ), v_lead = (kPanel >> 4) << 16;
+        bool ok = tc::mbar_wait_warp(bar(kBarQ), 0, abort_flag, A.status);
+        int st = 0, phase = 0;
+        auto next = [&]() { if (++st == kStages) { st = 0; phase ^= 1; } };
+        for (int t = 0; ok && t < nt; ++t, next()) {
+            ok = tc::mbar_wait_warp(bar(kBarFull + st), phase, abort_flag, A.status);
+            if (!ok) break;
+            tc::tc_fence_after();
+            const uint32_t a_lo = tc::desc_lo(base + st * kStageBytes);
+            if (tc::elect_one()) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
-                    tc::umma_bf16(tmem + kHeads + kHeads * t, tc::smem_desc_sw128(a + (j >> 2) * kPanel, (j & 3) * 32),
-                                  tc::smem_desc_sw128(base + kSmemQ + (j >> 2) * kSmallPanel, (j & 3) * 32), kIdescQK, j > 0);
+                    tc::umma_bf16(tmem + kHeads + kHeads * t, a_lo + (j >> 2) * (kPanel >> 4) + (j & 3) * 2, tc::kDescSw128Hi,
+                                  q_lo + (j >> 2) * (kSmallPanel >> 4) + (j & 3) * 2, tc::kDescSw128Hi, kIdescQK, j > 0);
                 tc::umma_commit(bar(kBarEmpty + st));
                 tc::umma_commit(bar(kBarS + t));
             }
-            for (int t = 0; ok && t < nt; ++t) {
-                const int i = nt + t, st = i % kStages, pb = t & 1;
-                ok = tc::mbar_wait(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status) &&
-                     tc::mbar_wait(bar(kBarPFull + pb), (t >> 1) & 1, abort_flag, A.status);
-                if (!ok) break;
-                tc::tc_fence_after();
-                const uint32_t a = base + st * kStageBytes, p = base + kSmemP + pb * 2 * kSmallPanel;
+            __syncwarp();
+        }
+        for (int t = 0; ok && t < nt; ++t, next()) {
+            const int pb = t & 1;
+            ok = tc::mbar_wait_warp(bar(kBarFull + st), phase, abort_flag, A.status) &&
+                 tc::mbar_wait_warp(bar(kBarPFull + pb), (t >> 1) & 1, abort_flag, A.status);
+            if (!ok) break;
+            tc::tc_fence_after();
+            const uint32_t a_lo = tc::desc_lo(base + st * kStageBytes) | v_lead, p_lo = tc::desc_lo(base + kSmemP + pb * 2 * kSmallPanel);
+            if (tc::elect_one()) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
-                    tc::umma_bf16(tmem, smem_desc_sw128_mn(a, j * 2048),
-                                  tc::smem_desc_sw128(p + (j >> 2) * kSmallPanel, (j & 3) * 32), kIdescPV, (t | j) != 0);
+                    tc::umma_bf16(tmem, a_lo + j * 128, tc::kDescSw128Hi, p_lo + (j >> 2) * (kSmallPanel >> 4) + (j & 3) * 2, tc::kDescSw128Hi,
+                                  kIdescPV, (t | j) != 0);
                 tc::umma_commit(bar(kBarEmpty + st));
                 tc::umma_commit(bar(kBarPEmpty + pb));
             }
-            if (ok) tc::umma_commit(bar(kBarO));
+            __syncwarp();
         }
+        if (ok && tc::elect_one()) tc::umma_commit(bar(kBarO));
+        __syncwarp();
     } else {
         const int e = threadIdx.x - 64;                              // 0 .. 127
         const int row = 32 * (warp & 3) + lane;                      // TMEM lane this thread reads: key of a tile / output dim
@@ -183,7 +190,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
 #pragma unroll
         for (int g = 0; g < kMaxHeads; ++g) mx[g] = kNegBig;
         for (int t = 0; t < nt; ++t) {                               // running maxima while the K tiles stream
-            ok = ok && tc::mbar_wait(bar(kBarS + t), 0, abort_flag, A.status);
+            ok = ok && tc::mbar_wait_warp(bar(kBarS + t), 0, abort_flag, A.status);
+            if (!ok) continue;
             tc::tc_fence_after();
             uint32_t r[16];
             tc::tmem_ld16(trow + kHeads + kHeads * t, r);
@@ -210,7 +218,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
         epi_sync();                                                  // red is reused for the sums below
         for (int t = 0; t < nt; ++t) {
             const int pb = t & 1;
-            ok = ok && tc::mbar_wait(bar(kBarPEmpty + pb), ((t >> 1) & 1) ^ 1, abort_flag, A.status);
+            ok = ok && tc::mbar_wait_warp(bar(kBarPEmpty + pb), ((t >> 1) & 1) ^ 1, abort_flag, A.status);
+            if (!ok) continue;
             uint32_t r[16];
             tc::tmem_ld16(trow + kHeads + kHeads * t, r);
             tc::tmem_ld_wait(r);
@@ -240,11 +249,13 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
             if (lane == 0) red[(warp & 3) * kMaxHeads + g] = l[g];
         }
         epi_sync();
-        ok = ok && tc::mbar_wait(bar(kBarO), 0, abort_flag, A.status);
+        ok = ok && tc::mbar_wait_warp(bar(kBarO), 0, abort_flag, A.status);
         tc::tc_fence_after();
-        uint32_t r[16];
-        tc::tmem_ld16(trow, r);
-        tc::tmem_ld_wait(r);
+        uint32_t r[16] = {};
+        if (ok) {
+            tc::tmem_ld16(trow, r);
+            tc::tmem_ld_wait(r);
+        }
         float *out = A.out + ((int64_t)u * A.Hq + h * G) * 128 + row;
         if (A.n_split == 1) {                                        // the only range of its head: normalise and finish
 #pragma unroll

@@ -67,7 +67,7 @@ flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
     if (c.warp == 0) {
         if (c.lane == 0) S::producer(c, &q_map, &k_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
-        if (c.lane == 0) S::mma_issuer<true>(c, A.n_items, plan, A.status);
+        S::mma_issuer<true>(c, A.n_items, plan, A.status);
     } else {
         const int row = c.quarter * 32 + c.lane;                     // row of the half
         const uint32_t xch = c.epi_addr() + row * 16, pxch = c.partner_addr() + row * 16;   // hand-over slot of this row, the other column half's

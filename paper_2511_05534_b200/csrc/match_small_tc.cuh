@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap cand_map, const Args A) {
     extern __shared__ __align__(1024) uint8_t mst_smem[];
     const uint32_t base = tc::smem_u32(mst_smem), bars = base + kSmemBar;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tc::warp_number(), lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(mst_smem + kSmemBar + 8 * kNumBars + 4);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mst_smem + kSmemBar + 8 * kNumBars);
     if ((base & 1023u) != 0) {
@@ -128,36 +128,44 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             bool ok = true;
             int hc = 0;
+            int n_text_next = A.cand_count[2 * A.by_nt.div(g_lo)], n_vis_next = A.cand_count[2 * A.by_nt.div(g_lo) + 1];   // a head ahead
             for (int g = g_lo; ok && g < g_hi; ++hc) {
                 const int uh = (int)A.by_nt.div(g), hp = hc % n_bbuf;
-                const int n_text = A.cand_count[2 * uh], n_vis = A.cand_count[2 * uh + 1];
+                const int n_text = n_text_next, n_vis = n_vis_next;
+                if (uh + 1 < A.n_heads) { n_text_next = A.cand_count[2 * uh + 2]; n_vis_next = A.cand_count[2 * uh + 3]; }
                 const int cols = n_vis > 0 ? ((n_text + 31) & ~31) + n_vis : n_text;         // columns up to the last candidate
-                ok = tc::mbar_wait(bar(kBarBFull + hp), (hc / n_bbuf) & 1, abort_flag, A.status);
+                ok = tc::mbar_wait_warp(bar(kBarBFull + hp), (hc / n_bbuf) & 1, abort_flag, A.status);
                 const uint32_t bd = base + kSmemB + hp * b_stride;
                 for (const int end = min(g_hi, (uh + 1) * nt); ok && g < end; ++g) {
                     const int i = g - g_lo, st = i % kStages;
-                    ok = tc::mbar_wait(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
+                    ok = tc::mbar_wait_warp(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
                     const uint32_t a = base + st * kStageBytes;
                     for (int q = 0; ok && q < units; ++q) {          // unit number k goes to accumulator and team k mod 4
                         const int k = i * units + q, set = k & (kTeams - 1), n = min(kUnitCols, cols - q * kUnitCols);
-                        ok = tc::mbar_wait(bar(kBarSetFree + set), ((k / kTeams) & 1) ^ 1, abort_flag, A.status);
+                        ok = tc::mbar_wait_warp(bar(kBarSetFree + set), ((k / kTeams) & 1) ^ 1, abort_flag, A.status);
                         if (!ok) break;
                         tc::tc_fence_after();
-                        if (n > 0) {
-                            const uint32_t idesc = tc::idesc_bf16(kTile, (uint32_t)((n + 15) & ~15));
+                        const uint32_t idesc = tc::idesc_bf16(kTile, (uint32_t)((n + 15) & ~15));
+                        const uint32_t a_lo = tc::desc_lo(a), b_lo = tc::desc_lo(bd + q * (kUnitCols * 128u));
+                        if (tc::elect_one()) {
+                            if (n > 0) {
 #pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                tc::umma_bf16(tmem + kUnitCols * set, tc::smem_desc_sw128(a + (j >> 2) * kPanel, (j & 3) * 32),
-                                              tc::smem_desc_sw128(bd + q * (kUnitCols * 128u) + (j >> 2) * b_panel, (j & 3) * 32), idesc, j > 0);
+                                for (int j = 0; j < 8; ++j)
+                                    tc::umma_bf16(tmem + kUnitCols * set, a_lo + (j >> 2) * (kPanel >> 4) + (j & 3) * 2, tc::kDescSw128Hi,
+                                                  b_lo + (j >> 2) * (b_panel >> 4) + (j & 3) * 2, tc::kDescSw128Hi, idesc, j > 0);
+                            }
+                            tc::umma_commit(bar(kBarAccFull + set));
                         }
-                        tc::umma_commit(bar(kBarAccFull + set));
+                        __syncwarp();
                     }
-                    if (ok) tc::umma_commit(bar(kBarEmpty + st));
+                    if (ok && tc::elect_one()) tc::umma_commit(bar(kBarEmpty + st));
+                    __syncwarp();
                 }
-                if (ok) tc::umma_commit(bar(kBarBEmpty + hp));
+                if (ok && tc::elect_one()) tc::umma_commit(bar(kBarBEmpty + hp));
+                __syncwarp();
             }
         }
     } else {
@@ -169,11 +177,29 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
         const uint32_t prow = base + kSmemStash + (team ^ 1) * 4096 + row * 32;      // the other unit's team
         bool ok = true;
         int hc = 0;
+        // what a tile needs from global memory is fetched a tile of this team ahead, what a head needs a head ahead
+        const int step = kTeams / units;                             // tiles between two of this team
+        auto fetch_mod = [&](int g) -> int {
+            const int uh = (int)A.by_nt.div(g), token = (g - uh * nt) * kTile + row;
+            return g < g_hi && token < A.L ? A.modality[(int64_t)A.by_hkv.div(uh) * A.L + token] : 0;
+        };
+        auto fetch_rank = [&](int g) -> int {
+            const int uh = (int)A.by_nt.div(g), token = (g - uh * nt) * kTile + row;
+            return g < g_hi && token < A.L ? A.rank[(int64_t)uh * A.L + token] : -1;
+        };
+        int mod_next = fetch_mod(g_lo + team / units), rank_next = fetch_rank(g_lo + team / units);
+        struct Head { int n_text, n_vis, strategy; };
+        auto fetch_head = [&](int uh) -> Head {
+            if (uh >= A.n_heads) return Head{0, 0, 0};
+            return Head{A.cand_count[2 * uh], A.cand_count[2 * uh + 1], A.strategy[A.by_hkv.div(uh)]};
+        };
+        Head head_next = fetch_head((int)A.by_nt.div(g_lo));
         for (int g = g_lo; g < g_hi; ++hc) {
-            const int uh = (int)A.by_nt.div(g), u = (int)A.by_hkv.div(uh), hp = hc % n_bbuf;
+            const int uh = (int)A.by_nt.div(g), hp = hc % n_bbuf;
             const uint32_t md = base + kSmemMeta + hp * m_stride;
-            const int n_text = A.cand_count[2 * uh], n_vis = A.cand_count[2 * uh + 1];
-            const bool intra = A.strategy[u] == 0;
+            const int n_text = head_next.n_text, n_vis = head_next.n_vis;
+            const bool intra = head_next.strategy == 0;
+            head_next = fetch_head(uh + 1);
             // blocks of 16 columns, text group [0, tb) and visual group [vb, ve), and this unit's share of them
             const int t0 = (n_text + 31) & ~31, c0 = hf * kUnitCols, blk0 = c0 >> 4;
             const int tb = min((n_text + 15) >> 4, blk0 + kUnitCols / 16);
@@ -184,21 +210,25 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 if ((k & (kTeams - 1)) != team) continue;            // (the parity of a tile's two units picks the pair of teams)
                 const int token = t * kTile + row;
                 const bool in_range = token < A.L;
-                const int my_mod = in_range ? A.modality[(int64_t)u * A.L + token] : 0;
-                const int my_rank = in_range ? A.rank[(int64_t)uh * A.L + token] : -1;
+                const int my_mod = mod_next, my_rank = rank_next;
+                mod_next = fetch_mod(g + step);
+                rank_next = fetch_rank(g + step);
                 const bool want_text = in_range && (!intra || my_mod == 0), want_vis = in_range && (!intra || my_mod != 0);
                 // the token's key row sits in the A stage (128-byte rows, 16-byte units XOR-swizzled by the row index)
-                ok = ok && tc::mbar_wait(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
+                ok = ok && tc::mbar_wait_warp(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
                 const uint32_t a_row = base + st * kStageBytes + row * 128;
-                float ssq = row_half_ssq(a_row + hf * kPanel, row);
-                if (units == 1) ssq += row_half_ssq(a_row + kPanel, row);
+                float ssq = 0.f;
+                if (ok) {
+                    ssq = row_half_ssq(a_row + hf * kPanel, row);
+                    if (units == 1) ssq += row_half_ssq(a_row + kPanel, row);
+                }
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(bar(kBarEmpty + st));
                 if (!b_ready) {                                      // scales and slots of this head have landed
-                    ok = ok && tc::mbar_wait(bar(kBarBFull + hp), (hc / n_bbuf) & 1, abort_flag, A.status);
+                    ok = ok && tc::mbar_wait_warp(bar(kBarBFull + hp), (hc / n_bbuf) & 1, abort_flag, A.status);
                     b_ready = true;
                 }
-                ok = ok && tc::mbar_wait(bar(kBarAccFull + team), (k / kTeams) & 1, abort_flag, A.status);
+                ok = ok && tc::mbar_wait_warp(bar(kBarAccFull + team), (k / kTeams) & 1, abort_flag, A.status);
                 tc::tc_fence_after();
                 // Candidates are laid out text group first, each group by ascending slot, so the first maximum of a group is
                 // its lowest slot; the groups' winners meet by (similarity, slot), so that equal similarities go to the lower.
@@ -257,15 +287,22 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                     }
                     return w;
                 };
-                const Winner wt = walk(blk0, tb, want_text);
-                float best = wt.best;
-                int slot = slot_of(wt);
-                const Winner wv = walk(vb, ve, want_vis);
+                float best = -INFINITY;
+                int slot = -1;
+                Winner wv = {-INFINITY, -1};
+                if (ok) {
+                    const Winner wt = walk(blk0, tb, want_text);
+                    best = wt.best;
+                    slot = slot_of(wt);
+                    wv = walk(vb, ve, want_vis);
+                }
                 tc::tc_fence_before();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(bar(kBarSetFree + team));   // this warp has read the accumulator
-                const int slot_v = slot_of(wv);
-                if (match_better(wv.best, slot_v, best, slot)) { best = wv.best; slot = slot_v; }
+                if (ok) {
+                    const int slot_v = slot_of(wv);
+                    if (match_better(wv.best, slot_v, best, slot)) { best = wv.best; slot = slot_v; }
+                }
                 if (units == 2) {
                     // the upper unit hands its result and its half of the norm to the lower one, which owns the row's output;
                     // (kept also after a wait that ran out, so that the partner warp is never left waiting)
@@ -293,7 +330,7 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
             }
             // done with this head's scales and slots (a warp without a tile of the head waits for them all the same: it must
             // not arrive for a later head while the buffer still belongs to an earlier one)
-            if (!b_ready) ok = ok && tc::mbar_wait(bar(kBarBFull + hp), (hc / n_bbuf) & 1, abort_flag, A.status);
+            if (!b_ready) ok = ok && tc::mbar_wait_warp(bar(kBarBFull + hp), (hc / n_bbuf) & 1, abort_flag, A.status);
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(bar(kBarBEmpty + hp));
         }

@@ -375,7 +375,7 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
     if (c.warp == 0) {
         if (c.lane == 0) S::producer(c, &k_map, &cand_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
-        if (c.lane == 0) S::template mma_issuer<false>(c, A.n_items, plan, A.status);
+        S::template mma_issuer<false>(c, A.n_items, plan, A.status);
     } else {
         const int lane = c.lane, row = c.quarter * 32 + lane;
         const int b0 = kPer * c.colhalf;                         // first block of this warp's share of a tile
@@ -439,7 +439,7 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 {   // the token's key row sits in this half's A stage: each of the row's two warps reads one 64-element
                     // half of it for the norm while the first MMAs run, then hands the stage back
                     ok = S::a_wait(c, n_mine, A.status);
-                    ssq = row_half_ssq(c.a_addr(n_mine) + c.colhalf * (tcs::kAHalf / 2) + row * 128, row);
+                    if (ok) ssq = row_half_ssq(c.a_addr(n_mine) + c.colhalf * (tcs::kAHalf / 2) + row * 128, row);
                     S::a_release(c, n_mine++);
                 }
                 for (int t = 0; ok && t < p.tp.n_tiles; ++t, ++k, ++bt) {

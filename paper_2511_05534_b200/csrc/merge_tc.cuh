@@ -125,7 +125,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     const uint32_t bars = tc::smem_u32(tail + kTailData);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tail + kTailData + 8 * kNumBars);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tail + kTailData + 8 * kNumBars + 4);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tc::warp_number(), lane = threadIdx.x & 31;
     if ((base & 1023u) != 0) {
         if (threadIdx.x == 0) atomicCAS(A.status, 0, 6);
         return;
@@ -175,34 +175,37 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                     for (int n = 0; n < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + s), 0) && !tc::mbar_try_wait(bar(kBarFull + s), 1); ++n) {}
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = tc::idesc_bf16(128, (uint32_t)N) | (1u << 15);       // A operand MN-major
-            bool ok = true;
-            int i = 0, j = 0, it = 0;
-            for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x, ++it) {
-                const int set = it % n_sets, use = it / n_sets;
-                ok = tc::mbar_wait(bar(kBarOutEmpty + set), (use & 1) ^ 1, abort_flag, A.status);   // the set's previous head is read out
-                tc::tc_fence_after();
-                for (int c = 0; ok && c < n_chunk; ++c, ++j) {
-                    const int wb = j & 1;
-                    ok = tc::mbar_wait(bar(kBarWFull + wb), (j >> 1) & 1, abort_flag, A.status);
-                    const uint32_t w = w0 + wb * wsize;
-                    for (int t = 0; ok && t < per_item; ++t, ++i) {
-                        const int st = i % A.n_stages;
-                        ok = tc::mbar_wait(bar(kBarFull + st), (i / A.n_stages) & 1, abort_flag, A.status);
-                        if (!ok) break;
-                        tc::tc_fence_after();
-                        const uint32_t a = base + st * kStageBytes;
+        const uint32_t idesc = tc::idesc_bf16(128, (uint32_t)N) | (1u << 15);           // A operand MN-major
+        const uint32_t a_hi = tc::kDescSw128Hi, a_lead = (kPanel >> 4) << 16;            // (and the stride between its panels)
+        bool ok = true;
+        int st = 0, st_phase = 0, wb = 0, w_phase = 0, it = 0;
+        for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x, ++it) {
+            const int set = it % n_sets, use = it / n_sets;
+            ok = tc::mbar_wait_warp(bar(kBarOutEmpty + set), (use & 1) ^ 1, abort_flag, A.status);   // the set's previous head is read out
+            tc::tc_fence_after();
+            for (int c = 0; ok && c < n_chunk; ++c) {
+                ok = tc::mbar_wait_warp(bar(kBarWFull + wb), w_phase, abort_flag, A.status);
+                const uint32_t w_lo = tc::desc_lo(w0 + wb * wsize);
+                for (int t = 0; ok && t < per_item; ++t) {
+                    ok = tc::mbar_wait_warp(bar(kBarFull + st), st_phase, abort_flag, A.status);
+                    if (!ok) break;
+                    tc::tc_fence_after();
+                    const uint32_t a_lo = tc::desc_lo(base + st * kStageBytes) | a_lead, d = tmem + set * set_cols + t * v_col;
+                    if (tc::elect_one()) {
 #pragma unroll
                         for (int q = 0; q < 8; ++q)
-                            tc::umma_bf16(tmem + set * set_cols + t * v_col, dtc::smem_desc_sw128_mn(a, q * 2048),
-                                          tc::smem_desc_sw128(w + (q >> 2) * wpanel, (q & 3) * 32), idesc, (c | q) != 0);
+                            tc::umma_bf16(d, a_lo + q * 128, a_hi, w_lo + (q >> 2) * (wpanel >> 4) + (q & 3) * 2, tc::kDescSw128Hi, idesc, (c | q) != 0);
                         tc::umma_commit(bar(kBarEmpty + st));
+                        if (t == per_item - 1) tc::umma_commit(bar(kBarWEmpty + wb));
                     }
-                    if (ok) tc::umma_commit(bar(kBarWEmpty + wb));
+                    __syncwarp();
+                    if (++st == A.n_stages) { st = 0; st_phase ^= 1; }
                 }
-                if (ok) tc::umma_commit(bar(kBarOutFull + set));
+                wb ^= 1;
+                w_phase ^= wb == 0;
             }
+            if (ok && tc::elect_one()) tc::umma_commit(bar(kBarOutFull + set));
+            __syncwarp();
         }
     } else if (warp < 6) {
         // builders: thread = token of a step
@@ -231,9 +234,9 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                 const uint32_t w = w0 + wb * wsize;
                 const uint32_t prev = wb ? wr1 : wr0;
                 uint32_t mine = 0;
-                if (prev) dtc::sts16(prev, 0);                       // take back what this thread wrote two steps ago
+                if (ok && prev) dtc::sts16(prev, 0);                 // take back what this thread wrote two steps ago
                 const int slot = cur.x & ~kPivotFlag;
-                if (cur.x >= 0 && slot < A.B) {
+                if (ok && cur.x >= 0 && slot < A.B) {
                     const __nv_bfloat16 wt = __float2bfloat16_rn(__int_as_float(cur.y));
                     const uint32_t at = w + tok_off + (uint32_t)slot * 128u + (uint32_t)((tok_grp ^ (slot & 7)) << 4);
                     dtc::sts16(at, __bfloat16_as_ushort(wt));
@@ -256,15 +259,15 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
             const int u = head_of(item) / A.Hkv, h = head_of(item) % A.Hkv;
             const int set = it % n_sets, use = it / n_sets;
             unsigned *sums = wsum + set * kMaxSlots;
-            ok = ok && tc::mbar_wait(bar(kBarSumFull + set), use & 1, abort_flag, A.status);
-            for (int sl = e; sl < N; sl += 256) {
+            ok = ok && tc::mbar_wait_warp(bar(kBarSumFull + set), use & 1, abort_flag, A.status);
+            for (int sl = e; ok && sl < N; sl += 256) {
                 inv_s[sl] = 1.f / (1.f + (float)sums[sl] * (1.f / kSumScale));
                 sums[sl] = 0u;
             }
             reader_sync();
-            ok = ok && tc::mbar_wait(bar(kBarOutFull + set), use & 1, abort_flag, A.status);
+            ok = ok && tc::mbar_wait_warp(bar(kBarOutFull + set), use & 1, abort_flag, A.status);
             tc::tc_fence_after();
-            if (*abort_flag == 0) {
+            if (ok) {
                 // a single tensor's slots go to the two quads in turn, 32 at a time
                 const int which = per_item == 2 ? t : first_tensor(item);
                 __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(which ? A.v_out : A.k_out) +

@@ -75,7 +75,7 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
     constexpr int GW = kRows, HC = GW / 2;
     extern __shared__ __align__(1024) uint8_t sft_smem[];
     const uint32_t base = tc::smem_u32(sft_smem), bars = base + kSmemBar;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tc::warp_number(), lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sft_smem + kSmemBar + 8 * kNumBars + 4);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sft_smem + kSmemBar + 8 * kNumBars);
     if ((base & 1023u) != 0) {
@@ -128,30 +128,35 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             constexpr uint32_t idesc = tc::idesc_bf16(kTile, GW);
             bool ok = true;
             int i = 0, it = 0;
             for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x, ++it) {
                 const int set = it & 1, use = it >> 1;
-                ok = tc::mbar_wait(bar(kBarQFull + set), use & 1, abort_flag, A.status) &&
-                     tc::mbar_wait(bar(kBarSetFree + set), (use & 1) ^ 1, abort_flag, A.status);   // the half's previous head is swept
+                ok = tc::mbar_wait_warp(bar(kBarQFull + set), use & 1, abort_flag, A.status) &&
+                     tc::mbar_wait_warp(bar(kBarSetFree + set), (use & 1) ^ 1, abort_flag, A.status);   // the half's previous head is swept
                 tc::tc_fence_after();
                 const uint32_t qd = base + kSmemQ + set * kQBytes;
                 for (int t = 0; ok && t < nt; ++t, ++i) {
                     const int st = i % kStages;
-                    ok = tc::mbar_wait(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
+                    ok = tc::mbar_wait_warp(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
                     if (!ok) break;
                     tc::tc_fence_after();
                     const uint32_t a = base + st * kStageBytes;
+                    const uint32_t a_lo = tc::desc_lo(a), b_lo = tc::desc_lo(qd), d = tmem + 256 * set + GW * t;
+                    if (tc::elect_one()) {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
-                        tc::umma_bf16(tmem + 256 * set + GW * t, tc::smem_desc_sw128(a + (j >> 2) * kPanel, (j & 3) * 32),
-                                      tc::smem_desc_sw128(qd + (j >> 2) * (kQBytes / 2), (j & 3) * 32), idesc, j > 0);
-                    tc::umma_commit(bar(kBarEmpty + st));
-                    tc::umma_commit(bar(kBarS + set * kMaxTiles + t));
+                        for (int j = 0; j < 8; ++j)
+                            tc::umma_bf16(d, a_lo + (j >> 2) * (kPanel >> 4) + (j & 3) * 2, tc::kDescSw128Hi,
+                                          b_lo + (j >> 2) * (kQBytes / 32) + (j & 3) * 2, tc::kDescSw128Hi, idesc, j > 0);
+                        tc::umma_commit(bar(kBarEmpty + st));
+                        tc::umma_commit(bar(kBarS + set * kMaxTiles + t));
+                    }
+                    __syncwarp();
                 }
-                if (ok) tc::umma_commit(bar(kBarQEmpty + set));
+                if (ok && tc::elect_one()) tc::umma_commit(bar(kBarQEmpty + set));
+                __syncwarp();
             }
         }
     } else {
@@ -175,22 +180,32 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
         };
         bool ok = true;
         int it = team;
+        uint8_t proxy_next = 0, key_next[kMaxTiles];
+        auto fetch_modality = [&](int item) {                        // (independent loads: nothing waits in between)
+            const uint8_t *mod = A.modality + (int64_t)(item / A.Hkv) * A.L;
+            const bool on = item < A.n_items;
+            proxy_next = on && lane < HC ? mod[first_proxy + (cb + lane) % A.W] : (uint8_t)0;
+#pragma unroll
+            for (int t = 0; t < kMaxTiles; ++t) key_next[t] = on && t * kTile + row < A.L ? mod[t * kTile + row] : (uint8_t)0;
+        };
+        fetch_modality(blockIdx.x + team * gridDim.x);
         for (int item = blockIdx.x + team * gridDim.x; item < A.n_items; item += 2 * gridDim.x, it += 2) {
             const int uh = item, u = item / A.Hkv, h = item % A.Hkv, use = it >> 1;
-            const uint8_t *mod = A.modality + (int64_t)u * A.L;
-            // which of this thread's proxy rows belong to visual tokens: bit q for row cb + q = g W + a, token first_proxy + a
-            const unsigned qvis = __ballot_sync(0xFFFFFFFFu, lane < HC && mod[first_proxy + (cb + lane) % A.W] != 0);
-            unsigned vis_bits = 0;                                   // bit t: this thread's key of tile t is a visual token
+            // modalities, fetched an item ahead: `qvis` bit q: this thread's proxy row cb + q = g W + a belongs to a visual token
+            // (token first_proxy + a); `vis_bits` bit t: its key of tile t is one
+            const unsigned qvis = __ballot_sync(0xFFFFFFFFu, proxy_next != 0);
+            unsigned vis_bits = 0;
 #pragma unroll
-            for (int t = 0; t < kMaxTiles; ++t)
-                if (t < nt && t * kTile + row < A.L && mod[t * kTile + row] != 0) vis_bits |= 1u << t;
+            for (int t = 0; t < kMaxTiles; ++t) vis_bits |= key_next[t] != 0 ? 1u << t : 0u;
+            fetch_modality(item + 2 * gridDim.x);
             team_sync(team);                                         // lim is written; the previous item's scratch is free
 
             float mx[HC];
 #pragma unroll
             for (int q = 0; q < HC; ++q) mx[q] = kNegBig;
             for (int t = 0; t < nt; ++t) {                           // sweep A, under the K stream
-                ok = ok && tc::mbar_wait(bar(kBarS + team * kMaxTiles + t), use & 1, abort_flag, A.status);
+                ok = ok && tc::mbar_wait_warp(bar(kBarS + team * kMaxTiles + t), use & 1, abort_flag, A.status);
+                if (!ok) continue;
                 tc::tc_fence_after();
                 const int key = t * kTile + row;
                 uint32_t r[HC];

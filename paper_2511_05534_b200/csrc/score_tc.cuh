@@ -93,7 +93,7 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     if (c.warp == 0) {
         if (c.lane == 0) S::producer(c, &q_map, &k_map, A.n_items1, a_bytes, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
-        if (c.lane == 0) S::template mma_issuer<false>(c, A.n_items1, plan, A.status);
+        S::template mma_issuer<false>(c, A.n_items1, plan, A.status);
     } else {
         // all sixteen warps drain one accumulator at a time: a warp owns 32 lanes x a quarter of the columns of
         // BOTH halves, so the tensor core refills one half while the other is being read
@@ -307,7 +307,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
     if (c.warp == 0) {
         if (c.lane == 0) S::producer(c, &k_map, &q_map, blockIdx.x + n_loop, tcs::kAHalf, b_bytes, plan, A.status);
     } else if (c.warp == 1) {
-        if (c.lane == 0) S::template mma_issuer<true>(c, blockIdx.x + n_loop, plan, A.status);
+        S::template mma_issuer<true>(c, blockIdx.x + n_loop, plan, A.status);
     } else {
         const int lane = c.lane, row = c.quarter * 32 + lane;
         const uint32_t xch = c.epi_addr() + row * 4;            // hand-over slot of this row

@@ -61,6 +61,8 @@ __device__ __forceinline__ bool mbar_try_wait_for(uint32_t bar, uint32_t parity,
 }
 constexpr uint32_t kWaitSuspendNs = 2000;
 
+// What a wait was for - reads of shared or tensor memory, overwriting a buffer - must depend on its result (`if (ok)`), not
+// just follow it: code that goes on regardless of a give-up was compiled to shared-memory reads ahead of the wait.
 // Bounded wait.  `abort_flag` (shared memory) is raised by whichever thread of the CTA runs out
 // of time first; every other waiter sees it and gives up too.  Returns false on give-up.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status_word) {
@@ -80,6 +82,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
             }
         }
     }
+}
+
+// The same for a whole converged warp, which stays together whatever its lanes saw.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status_word) {
+    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, status_word));
 }
 
 // ---- TMA ---------------------------------------------------------------------------------------
@@ -149,6 +156,33 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint6
         ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
+// The same with descriptors given as their lower words, the upper words being constants of the operand's layout.
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                          uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}"
+        ::"r"(tmem_d), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+// One thread of the (converged) warp: true for it alone.  The roles that issue MMAs run with their whole warp and elect the
+// issuing thread, so that addresses, descriptors and loop control are known to be the same for the warp and stay in uniform
+// registers; run by lane 0 in a divergent branch, every MMA cost a few dozen clocks of moves and a tile of eight 600 to
+// 1200, more than the products themselves.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t is;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xFFFFFFFF;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(is));
+    return is != 0;
+}
+// The warp's number, as a value the compiler knows to be uniform.
+__device__ __forceinline__ int warp_number() { return __shfl_sync(0xFFFFFFFFu, (int)(threadIdx.x >> 5), 0); }
 // The mbarrier gets one arrival when every MMA this thread issued so far has completed.
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
@@ -214,6 +248,8 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t tile_base, uint32_t
     d |= (uint64_t)2 << 61;                                              // 128-byte swizzle
     return d;
 }
+constexpr uint32_t kDescSw128Hi = (1024u >> 4) | (1u << 14) | (2u << 29);      // upper word of smem_desc_sw128
+__device__ __forceinline__ uint32_t desc_lo(uint32_t tile_base) { return (tile_base & 0x3FFFFu) >> 4; }   // its lower word
 // kind::f16 instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, tile M x N.
 __host__ __device__ constexpr uint32_t idesc_bf16(uint32_t M, uint32_t N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);

@@ -105,7 +105,7 @@ struct Skel {
         Ctx c;
         c.base = tc::smem_u32(smem_raw);
         c.bars = c.base + kSmemBar;
-        c.warp = threadIdx.x >> 5;
+        c.warp = tc::warp_number();
         c.lane = threadIdx.x & 31;
         c.group = ((c.warp - 2) >> 2) & 1;
         c.quarter = c.warp & 3;
@@ -195,7 +195,7 @@ struct Skel {
         }
     }
 
-    // Call from one thread.  kQuads: accumulators are handed around by quad, else by half.
+    // Call from a whole warp.  kQuads: accumulators are handed around by quad, else by half.
     template <bool kQuads, class PlanFn>
     static __device__ __forceinline__ void mma_issuer(const Ctx &c, int n_items, PlanFn plan, int *status) {
         constexpr int kParts = kQuads ? 2 : 1, kPartCols = NB / kParts;   // accumulators of a half, their columns
@@ -207,7 +207,7 @@ struct Skel {
             for (int t = 0; ok && t < p.n_tiles; ++t) {
                 if (!p.reuse_b) ++bt;
                 const int sb = (bt - 1) % BST;                           // bt: B tiles taken so far, this one included
-                ok = tc::mbar_wait(c.bar(kBarBFull + sb), ((bt - 1) / BST) & 1, c.abort_flag, status);
+                ok = tc::mbar_wait_warp(c.bar(kBarBFull + sb), ((bt - 1) / BST) & 1, c.abort_flag, status);
                 if (!ok) break;
                 const int ncols = min(NB, p.cols_total - t * NB);
                 const int ncols0 = p.cols_first ? min(NB, p.cols_first - t * NB) : ncols;
@@ -215,30 +215,32 @@ struct Skel {
                 uint32_t took = 0;
                 for (int h = 0; ok && h < p.n_halves; ++h) {
                     const int st = ia[h] % AST;
-                    if (t == 0) ok = tc::mbar_wait(c.bar(kBarAFull + st * 2 + h), (ia[h] / AST) & 1, c.abort_flag, status);
+                    if (t == 0) ok = tc::mbar_wait_warp(c.bar(kBarAFull + st * 2 + h), (ia[h] / AST) & 1, c.abort_flag, status);
                     const uint32_t a_base = c.base + kSmemA + (uint32_t)(st * 2 + h) * kAHalf;
 #pragma unroll
                     for (int ch = 0; ch < kParts; ++ch) {                // the accumulators that hold columns
                         const int q = kParts * h + ch, n = min(kPartCols, (h == 0 ? ncols0 : ncols) - ch * kPartCols);
                         if (n <= 0 || !ok) continue;
-                        ok = tc::mbar_wait(c.bar(kBarAccEmpty + q), (ta[q] & 1) ^ 1, c.abort_flag, status);
+                        ok = tc::mbar_wait_warp(c.bar(kBarAccEmpty + q), (ta[q] & 1) ^ 1, c.abort_flag, status);
                         if (!ok) continue;
                         tc::tc_fence_after();
                         const uint32_t idesc = tc::idesc_bf16(kRows, (uint32_t)((n + 15) & ~15));
+                        const uint32_t a_lo = tc::desc_lo(a_base), b_lo = tc::desc_lo(b_base + ch * (kPartCols * 128)), d = c.tmem_base + q * kPartCols;
+                        if (tc::elect_one()) {
 #pragma unroll
-                        for (int ks = 0; ks < 8; ++ks) {                 // head_dim 128 = 8 K slices of 16
-                            const uint32_t a_off = (ks >> 2) * (kAHalf / 2) + (ks & 3) * 32;
-                            const uint32_t b_off = (ks >> 2) * (kBStage / 2) + ch * (kPartCols * 128) + (ks & 3) * 32;
-                            tc::umma_bf16(c.tmem_base + q * kPartCols, tc::smem_desc_sw128(a_base, a_off),
-                                          tc::smem_desc_sw128(b_base, b_off), idesc, ks > 0);
+                            for (int ks = 0; ks < 8; ++ks)               // head_dim 128 = 8 K slices of 16
+                                tc::umma_bf16(d, a_lo + (ks >> 2) * (kAHalf / 32) + (ks & 3) * 2, tc::kDescSw128Hi,
+                                              b_lo + (ks >> 2) * (kBStage / 32) + (ks & 3) * 2, tc::kDescSw128Hi, idesc, ks > 0);
+                            tc::umma_commit(c.bar(kBarAccFull + q));     // accumulator ready
                         }
-                        tc::umma_commit(c.bar(kBarAccFull + q));         // accumulator ready
+                        __syncwarp();
                         ++ta[q];
                         took |= 1u << q;
                     }
                     if (!ok) break;
                     if (t == p.n_tiles - 1) {                            // that was the half's last use of its A stage
-                        tc::umma_commit(c.bar(kBarAEmpty + st * 2 + h));
+                        if (tc::elect_one()) tc::umma_commit(c.bar(kBarAEmpty + st * 2 + h));
+                        __syncwarp();
                         ++ia[h];
                     }
                 }
@@ -247,10 +249,11 @@ struct Skel {
                     // accumulators without a part in this tile: their quads must be through with the tiles before it as well,
                     // so that a tile's release tells the producer that nobody reads the constants of the tile before any more
                     for (int q = 0; ok && q < 4; ++q)
-                        if (!(took & (1u << q))) ok = tc::mbar_wait(c.bar(kBarAccEmpty + q), (ta[q] & 1) ^ 1, c.abort_flag, status);
+                        if (!(took & (1u << q))) ok = tc::mbar_wait_warp(c.bar(kBarAccEmpty + q), (ta[q] & 1) ^ 1, c.abort_flag, status);
                     if (!ok) break;
                 }
-                if (!p.keep_b) tc::umma_commit(c.bar(kBarBEmpty + sb));  // B stage free once both halves' MMAs finish
+                if (!p.keep_b && tc::elect_one()) tc::umma_commit(c.bar(kBarBEmpty + sb));   // B stage free once both halves' MMAs finish
+                __syncwarp();
             }
         }
     }
@@ -264,7 +267,7 @@ struct Skel {
     // For kernels whose epilogue reads its A half from shared memory: wait until the half of the
     // n-th item this group takes part in has landed (at Ctx::a_addr(n)) / hand it back (one arrival per warp).
     static __device__ __forceinline__ bool a_wait(const Ctx &c, int n, int *status) {
-        return tc::mbar_wait(c.bar(kBarAFull + (n % AST) * 2 + c.group), (n / AST) & 1, c.abort_flag, status);
+        return tc::mbar_wait_warp(c.bar(kBarAFull + (n % AST) * 2 + c.group), (n / AST) & 1, c.abort_flag, status);
     }
     static __device__ __forceinline__ void a_release(const Ctx &c, int n) {
         __syncwarp();
