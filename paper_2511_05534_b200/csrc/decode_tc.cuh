@@ -113,23 +113,25 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
     const int key0 = t0 * kTile;
 
     if (warp == 0) {
-        if (lane == 0) {
-            bool ok = true;
-            for (int i = 0; ok && i < 2 * nt; ++i) {                 // the K tiles, then the V tiles
-                const int st = i % kStages;
-                ok = tc::mbar_wait(bar(kBarEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag, A.status);
-                if (!ok) break;
-                const CUtensorMap *m = i < nt ? &kmap : &vmap;
-                const int row = key0 + (i < nt ? i : i - nt) * kTile;
-                const uint32_t dst = base + st * kStageBytes;
+        bool ok = true;
+        int st = 0, phase = 0;
+        for (int i = 0; ok && i < 2 * nt; ++i) {                     // the K tiles, then the V tiles
+            ok = tc::mbar_wait_warp(bar(kBarEmpty + st), phase ^ 1, abort_flag, A.status);
+            if (!ok) break;
+            const CUtensorMap *m = i < nt ? &kmap : &vmap;
+            const int row = key0 + (i < nt ? i : i - nt) * kTile;
+            const uint32_t dst = base + st * kStageBytes;
+            if (tc::elect_one()) {
                 tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
                 tc::tma_load_4d(dst, m, bar(kBarFull + st), 0, row, h, u);
                 tc::tma_load_4d(dst + kPanel, m, bar(kBarFull + st), 64, row, h, u);
             }
-            if (!ok)         // winding down after a timeout: give copies already issued a moment to land
-                for (int i = 0; i < kStages; ++i)
-                    for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + i), 0) && !tc::mbar_try_wait(bar(kBarFull + i), 1); ++s) {}
+            __syncwarp();
+            if (++st == kStages) { st = 0; phase ^= 1; }
         }
+        if (!ok)         // winding down after a timeout: give copies already issued a moment to land
+            for (int i = 0; i < kStages; ++i)
+                for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + i), 0) && !tc::mbar_try_wait(bar(kBarFull + i), 1); ++s) {}
     } else if (warp == 1) {
         const uint32_t q_lo = tc::desc_lo(base + kSmemQ), v_lead = (kPanel >> 4) << 16;
         bool ok = tc::mbar_wait_warp(bar(kBarQ), 0, abort_flag, A.status);

@@ -65,7 +65,7 @@ flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
     };
     auto plan = [&](int item) { return plan_of(flow_item(A, item)); };
     if (c.warp == 0) {
-        if (c.lane == 0) S::producer(c, &q_map, &k_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
+        S::producer(c, &q_map, &k_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
         S::mma_issuer<true>(c, A.n_items, plan, A.status);
     } else {

@@ -97,27 +97,33 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
 
     // every role walks the heads of the run: tiles [t_lo, t_hi) of head uh, hc heads before it, tile number i of the run
     if (warp == 0) {
-        if (lane == 0) {
+        {
             bool ok = true;
             int hc = 0;
             for (int g = g_lo; ok && g < g_hi; ++hc) {
                 const int uh = (int)A.by_nt.div(g), u = (int)A.by_hkv.div(uh), h = uh - u * A.Hkv, hp = hc % n_bbuf;
-                ok = tc::mbar_wait(bar(kBarBEmpty + hp), ((hc / n_bbuf) & 1) ^ 1, abort_flag, A.status);
+                ok = tc::mbar_wait_warp(bar(kBarBEmpty + hp), ((hc / n_bbuf) & 1) ^ 1, abort_flag, A.status);
                 if (!ok) break;
                 const uint32_t bd = base + kSmemB + hp * b_stride, md = base + kSmemMeta + hp * m_stride;
-                tc::mbar_expect_tx(bar(kBarBFull + hp), b_bytes + 8u * (uint32_t)N);
-                tc::tma_load_4d(bd, &cand_map, bar(kBarBFull + hp), 0, 0, uh, 0);
-                tc::tma_load_4d(bd + b_panel, &cand_map, bar(kBarBFull + hp), 64, 0, uh, 0);
-                tc::bulk_load(md, A.cand_scale + (int64_t)uh * N, 4u * (uint32_t)N, bar(kBarBFull + hp));
-                tc::bulk_load(md + slot_off, A.cand_slot + (int64_t)uh * N, 4u * (uint32_t)N, bar(kBarBFull + hp));
+                if (tc::elect_one()) {
+                    tc::mbar_expect_tx(bar(kBarBFull + hp), b_bytes + 8u * (uint32_t)N);
+                    tc::tma_load_4d(bd, &cand_map, bar(kBarBFull + hp), 0, 0, uh, 0);
+                    tc::tma_load_4d(bd + b_panel, &cand_map, bar(kBarBFull + hp), 64, 0, uh, 0);
+                    tc::bulk_load(md, A.cand_scale + (int64_t)uh * N, 4u * (uint32_t)N, bar(kBarBFull + hp));
+                    tc::bulk_load(md + slot_off, A.cand_slot + (int64_t)uh * N, 4u * (uint32_t)N, bar(kBarBFull + hp));
+                }
+                __syncwarp();
                 for (const int end = min(g_hi, (uh + 1) * nt); ok && g < end; ++g) {
                     const int i = g - g_lo, t = g - uh * nt, st = i % kStages;
-                    ok = tc::mbar_wait(bar(kBarEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag, A.status);
+                    ok = tc::mbar_wait_warp(bar(kBarEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag, A.status);
                     if (!ok) break;
                     const uint32_t dst = base + st * kStageBytes;
-                    tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
-                    tc::tma_load_4d(dst, &k_map, bar(kBarFull + st), 0, t * kTile, h, u);
-                    tc::tma_load_4d(dst + kPanel, &k_map, bar(kBarFull + st), 64, t * kTile, h, u);
+                    if (tc::elect_one()) {
+                        tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
+                        tc::tma_load_4d(dst, &k_map, bar(kBarFull + st), 0, t * kTile, h, u);
+                        tc::tma_load_4d(dst + kPanel, &k_map, bar(kBarFull + st), 64, t * kTile, h, u);
+                    }
+                    __syncwarp();
                 }
             }
             if (!ok) {       // winding down after a timeout: give copies already issued a moment to land

@@ -373,7 +373,7 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
     if (!c.ok) return;
     auto plan = [&](int item) { return match_plan<S>(A, item).tp; };
     if (c.warp == 0) {
-        if (c.lane == 0) S::producer(c, &k_map, &cand_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
+        S::producer(c, &k_map, &cand_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
         S::template mma_issuer<false>(c, A.n_items, plan, A.status);
     } else {

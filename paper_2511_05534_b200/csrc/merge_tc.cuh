@@ -153,27 +153,28 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     auto head_of = [&](int item) { return per_item == 2 ? item : item >> 1; };
 
     if (warp == 0) {
-        if (lane == 0) {
-            bool ok = true;
-            int i = 0;
-            for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x) {
-                const int u = head_of(item) / A.Hkv, h = head_of(item) % A.Hkv, t0 = first_tensor(item);
-                for (int c = 0; ok && c < per_item * n_chunk; ++c, ++i) {   // per step the K tile, then the V tile
-                    const int st = i % A.n_stages;
-                    ok = tc::mbar_wait(bar(kBarEmpty + st), ((i / A.n_stages) & 1) ^ 1, abort_flag, A.status);
+        bool ok = true;
+        int st = 0, phase = 0;
+        for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x) {
+            const int u = head_of(item) / A.Hkv, h = head_of(item) % A.Hkv, t0 = first_tensor(item);
+            for (int c = 0; ok && c < n_chunk; ++c)
+                for (int t = 0; t < per_item; ++t) {             // per step the K tile, then the V tile
+                    ok = tc::mbar_wait_warp(bar(kBarEmpty + st), phase ^ 1, abort_flag, A.status);
                     if (!ok) break;
-                    const int step = per_item == 2 ? c >> 1 : c;
-                    const CUtensorMap *m = (per_item == 2 ? c & 1 : t0) ? &vmap : &kmap;
+                    const CUtensorMap *m = (per_item == 2 ? t : t0) ? &vmap : &kmap;
                     const uint32_t dst = base + st * kStageBytes;
-                    tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
-                    tc::tma_load_4d(dst, m, bar(kBarFull + st), 0, step * kTile, h, u);
-                    tc::tma_load_4d(dst + kPanel, m, bar(kBarFull + st), 64, step * kTile, h, u);
+                    if (tc::elect_one()) {
+                        tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
+                        tc::tma_load_4d(dst, m, bar(kBarFull + st), 0, c * kTile, h, u);
+                        tc::tma_load_4d(dst + kPanel, m, bar(kBarFull + st), 64, c * kTile, h, u);
+                    }
+                    __syncwarp();
+                    if (++st == A.n_stages) { st = 0; phase ^= 1; }
                 }
-            }
-            if (!ok)         // winding down after a timeout: give copies already issued a moment to land
-                for (int s = 0; s < A.n_stages; ++s)
-                    for (int n = 0; n < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + s), 0) && !tc::mbar_try_wait(bar(kBarFull + s), 1); ++n) {}
         }
+        if (!ok)         // winding down after a timeout: give copies already issued a moment to land
+            for (int i = 0; i < A.n_stages; ++i)
+                for (int n = 0; n < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + i), 0) && !tc::mbar_try_wait(bar(kBarFull + i), 1); ++n) {}
     } else if (warp == 1) {
         const uint32_t idesc = tc::idesc_bf16(128, (uint32_t)N) | (1u << 15);           // A operand MN-major
         const uint32_t a_hi = tc::kDescSw128Hi, a_lead = (kPanel >> 4) << 16;            // (and the stride between its panels)

@@ -99,25 +99,31 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
     const int nt = (A.L + kTile - 1) / kTile;
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             bool ok = true;
             int i = 0, it = 0;
             for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x, ++it) {
                 const int u = item / A.Hkv, h = item % A.Hkv, set = it & 1;
-                ok = tc::mbar_wait(bar(kBarQEmpty + set), ((it >> 1) & 1) ^ 1, abort_flag, A.status);
+                ok = tc::mbar_wait_warp(bar(kBarQEmpty + set), ((it >> 1) & 1) ^ 1, abort_flag, A.status);
                 if (!ok) break;
                 const uint32_t qd = base + kSmemQ + set * kQBytes;
-                tc::mbar_expect_tx(bar(kBarQFull + set), kQBytes);
-                tc::tma_load_4d(qd, &qmap, bar(kBarQFull + set), 0, 0, h * A.G, u);
-                tc::tma_load_4d(qd + kQBytes / 2, &qmap, bar(kBarQFull + set), 64, 0, h * A.G, u);
+                if (tc::elect_one()) {
+                    tc::mbar_expect_tx(bar(kBarQFull + set), kQBytes);
+                    tc::tma_load_4d(qd, &qmap, bar(kBarQFull + set), 0, 0, h * A.G, u);
+                    tc::tma_load_4d(qd + kQBytes / 2, &qmap, bar(kBarQFull + set), 64, 0, h * A.G, u);
+                }
+                __syncwarp();
                 for (int t = 0; ok && t < nt; ++t, ++i) {
                     const int st = i % kStages;
-                    ok = tc::mbar_wait(bar(kBarEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag, A.status);
+                    ok = tc::mbar_wait_warp(bar(kBarEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag, A.status);
                     if (!ok) break;
                     const uint32_t dst = base + st * kStageBytes;
-                    tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
-                    tc::tma_load_4d(dst, &kmap, bar(kBarFull + st), 0, t * kTile, h, u);
-                    tc::tma_load_4d(dst + kPanel, &kmap, bar(kBarFull + st), 64, t * kTile, h, u);
+                    if (tc::elect_one()) {
+                        tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
+                        tc::tma_load_4d(dst, &kmap, bar(kBarFull + st), 0, t * kTile, h, u);
+                        tc::tma_load_4d(dst + kPanel, &kmap, bar(kBarFull + st), 64, t * kTile, h, u);
+                    }
+                    __syncwarp();
                 }
             }
             if (!ok) {       // winding down after a timeout: give copies already issued a moment to land

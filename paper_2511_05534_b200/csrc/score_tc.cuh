@@ -91,7 +91,7 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     };
     const uint32_t a_bytes = (uint32_t)A.a_heads * A.W * 256u;
     if (c.warp == 0) {
-        if (c.lane == 0) S::producer(c, &q_map, &k_map, A.n_items1, a_bytes, S::kBStage, plan, A.status);
+        S::producer(c, &q_map, &k_map, A.n_items1, a_bytes, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
         S::template mma_issuer<false>(c, A.n_items1, plan, A.status);
     } else {
@@ -305,7 +305,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
     };
     const uint32_t b_bytes = (uint32_t)A.b_heads * A.W * 256u;
     if (c.warp == 0) {
-        if (c.lane == 0) S::producer(c, &k_map, &q_map, blockIdx.x + n_loop, tcs::kAHalf, b_bytes, plan, A.status);
+        S::producer(c, &k_map, &q_map, blockIdx.x + n_loop, tcs::kAHalf, b_bytes, plan, A.status);
     } else if (c.warp == 1) {
         S::template mma_issuer<true>(c, blockIdx.x + n_loop, plan, A.status);
     } else {

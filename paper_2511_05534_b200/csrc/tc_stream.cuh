@@ -147,7 +147,7 @@ struct Skel {
         if (c.warp == 1) tc::tmem_dealloc(c.tmem_base, 512);
     }
 
-    // Call from one thread.  a_bytes / b_bytes: bytes one A-half / B box pair delivers (both K halves).
+    // Call from a whole warp.  a_bytes / b_bytes: bytes one A-half / B box pair delivers (both K halves).
     template <class PlanFn>
     static __device__ __forceinline__ void producer(const Ctx &c, const CUtensorMap *ma, const CUtensorMap *mb, int n_items,
                                                     uint32_t a_bytes, uint32_t b_bytes, PlanFn plan, int *status) {
@@ -158,30 +158,39 @@ struct Skel {
             if (p.empty()) continue;
             for (int t = 0; ok && t < p.n_tiles; ++t) {
                 const int sb = bt % BST;
-                if (!p.reuse_b) ok = tc::mbar_wait(c.bar(kBarBEmpty + sb), ((bt / BST) & 1) ^ 1, c.abort_flag, status);
+                if (!p.reuse_b) ok = tc::mbar_wait_warp(c.bar(kBarBEmpty + sb), ((bt / BST) & 1) ^ 1, c.abort_flag, status);
                 if (!ok) break;
                 if (p.extra && !p.reuse_b) {   // slot reuse is safe: every epilogue released tile bt-4 before the stage of bt-2 was released
                     const int xs = bt & (kExtraSlots - 1);
-                    tc::mbar_expect_tx(c.bar(kBarXFull + xs), kExtraBytes);
-                    tc::bulk_load(c.base + kSmemExtra + (uint32_t)xs * kExtraBytes, p.extra + (size_t)t * NB, kExtraBytes,
-                                  c.bar(kBarXFull + xs));
+                    if (tc::elect_one()) {
+                        tc::mbar_expect_tx(c.bar(kBarXFull + xs), kExtraBytes);
+                        tc::bulk_load(c.base + kSmemExtra + (uint32_t)xs * kExtraBytes, p.extra + (size_t)t * NB, kExtraBytes,
+                                      c.bar(kBarXFull + xs));
+                    }
+                    __syncwarp();
                 }
                 if (!p.reuse_b) {
-                    tc::mbar_expect_tx(c.bar(kBarBFull + sb), b_bytes);
                     const uint32_t b_dst = c.base + kSmemB + sb * kBStage;
-                    tc::tma_load_4d(b_dst, mb, c.bar(kBarBFull + sb), 0, p.b1 + t * p.step1, p.b2 + t * p.step2, p.b3);
-                    tc::tma_load_4d(b_dst + kBStage / 2, mb, c.bar(kBarBFull + sb), 64, p.b1 + t * p.step1, p.b2 + t * p.step2, p.b3);
+                    if (tc::elect_one()) {
+                        tc::mbar_expect_tx(c.bar(kBarBFull + sb), b_bytes);
+                        tc::tma_load_4d(b_dst, mb, c.bar(kBarBFull + sb), 0, p.b1 + t * p.step1, p.b2 + t * p.step2, p.b3);
+                        tc::tma_load_4d(b_dst + kBStage / 2, mb, c.bar(kBarBFull + sb), 64, p.b1 + t * p.step1, p.b2 + t * p.step2, p.b3);
+                    }
+                    __syncwarp();
                     ++bt;
                 }
                 if (t == 0) {                  // the item's A halves go out right after its first B tile
                     for (int h = 0; ok && h < p.n_halves; ++h) {
                         const int st = ia[h] % AST, full = kBarAFull + st * 2 + h;
-                        ok = tc::mbar_wait(c.bar(kBarAEmpty + st * 2 + h), ((ia[h] / AST) & 1) ^ 1, c.abort_flag, status);
+                        ok = tc::mbar_wait_warp(c.bar(kBarAEmpty + st * 2 + h), ((ia[h] / AST) & 1) ^ 1, c.abort_flag, status);
                         if (!ok) break;
-                        tc::mbar_expect_tx(c.bar(full), a_bytes);
                         const uint32_t a_dst = c.base + kSmemA + (uint32_t)(st * 2 + h) * kAHalf;
-                        tc::tma_load_4d(a_dst, ma, c.bar(full), 0, p.a1 + h * p.h1, p.a2 + h * p.h2, p.a3);
-                        tc::tma_load_4d(a_dst + kAHalf / 2, ma, c.bar(full), 64, p.a1 + h * p.h1, p.a2 + h * p.h2, p.a3);
+                        if (tc::elect_one()) {
+                            tc::mbar_expect_tx(c.bar(full), a_bytes);
+                            tc::tma_load_4d(a_dst, ma, c.bar(full), 0, p.a1 + h * p.h1, p.a2 + h * p.h2, p.a3);
+                            tc::tma_load_4d(a_dst + kAHalf / 2, ma, c.bar(full), 64, p.a1 + h * p.h1, p.a2 + h * p.h2, p.a3);
+                        }
+                        __syncwarp();
                         ++ia[h];
                     }
                 }
