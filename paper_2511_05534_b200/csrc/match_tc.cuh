@@ -412,14 +412,16 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             // Running winner of this row among the warp's columns: its similarity (still times the row's norm, four
             // lowest mantissa bits cleared), the tile it came from, and in `win` the block of 16 columns inside the warp's
             // share of that tile (x 16) with 15 - column inside the block.  Candidates are laid out text group first, each group by ascending
-            // slot, so within a group the first maximum is the lowest slot; where a row sees both groups (a cross-modal
-            // layer) the text group's winner is set aside when the first visual column comes up, and the two meet by
-            // (similarity, slot).
+            // slot, so within a group the first maximum is the lowest slot; where a tile visits both groups the text group's
+            // winner is set aside when the first visual column comes up: in a cross-modal layer the two meet by
+            // (similarity, slot), in an intra-modal one, whose tile then holds tokens of both modalities, the row's modality
+            // picks one.  (Masking such a row's columns one by one took half of all epilogue time where a tenth of the tiles
+            // were mixed: 28 units x 4 heads of 8448 tokens against 1690 pivots 441 us, this 330.)
             float best = -INFINITY, before = -INFINITY;
             int win = -1, best_tile = 0;
             float val_a = -INFINITY;                                 // the winner set aside
             int slot_a = -1;
-            bool parked = p.intra;                                   // (an intra-modal row sees one group only)
+            bool parked = p.intra && !row_masked;                    // (one group only)
             float ssq = 0.f;                                         // squared norm of this row's key, this warp's half of it
             auto resolve = [&]() -> int {                            // slot of the running winner
                 if (win < 0) return -1;
@@ -449,64 +451,32 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     if (!ok) break;
                     const uint32_t scale4 = c.extra(bt);             // reciprocal norms of this tile's candidates
                     const int n_blocks = (ncols + 15) >> 4;
-                    if (row_masked) {
-                        // intra-modal layer, tile with tokens of both modalities: rows differ in which columns they may take
-                        S::for_each_block16(c, n_blocks, [&](int bl, uint32_t (&acc)[16]) {
-                            const int cc = col0 + bl * 16;
-                            float v[16];
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4) {     // a column that is no candidate has scale NaN and never wins
-                                const float4 s4 = tc::lds128(scale4 + (bl * 4 + q4) * 16);
-                                v[4 * q4 + 0] = __uint_as_float(acc[4 * q4 + 0]) * s4.x;
-                                v[4 * q4 + 1] = __uint_as_float(acc[4 * q4 + 1]) * s4.y;
-                                v[4 * q4 + 2] = __uint_as_float(acc[4 * q4 + 2]) * s4.z;
-                                v[4 * q4 + 3] = __uint_as_float(acc[4 * q4 + 3]) * s4.w;
-                            }
-                            int r1hi = p.n_text, r2lo = p.t0, r2hi = p.t0 + p.n_vis;   // admissible columns of this row
-                            if (my_mod == 0) r2hi = r2lo; else r1hi = 0;
-                            float q = -INFINITY;
-                            int qj = 0;
-#pragma unroll
-                            for (int j = 0; j < 16; ++j) {           // columns in ascending order; NaN never wins
-                                const int col = cc + j;
-                                const bool valid = (col < r1hi) || (col >= r2lo && col < r2hi);
-                                const float x = __uint_as_float(__float_as_uint(v[j]) & 0xFFFFFFF0u);   // as the unmasked path rounds it
-                                if (valid && x > q) { q = x; qj = j; }
-                            }
-                            if (q > best) {                          // strict: an earlier block keeps a tie
-                                best = q;
-                                win = (bl - b0) * 16 + 15 - qj;
-                                best_tile = t;
-                            }
-                        });
+                    const int nb = min(n_blocks - b0, kPer);     // blocks of this warp in this tile (may be <= 0)
+                    // block before which the text group's winner is set aside (>= nb: not in this tile)
+                    // (splitting a ragged last tile evenly between the row's two warps was measured and is no faster:
+                    // the tile's arithmetic, not the longer of its two shares, is what takes the time)
+                    const int pk = parked ? kPer : max(0, (p.t0 - (col0 + b0 * 16)) >> 4);
+                    const uint32_t sc = scale4 + b0 * 64, tl = t_lane;
+                    before = best;
+                    if (nb == kPer && pk >= kPer) {
+                        match_blocks<kPer>(tl, sc, best, win);
                     } else {
-                        const int nb = min(n_blocks - b0, kPer);     // blocks of this warp in this tile (may be <= 0)
-                        // block before which the text group's winner is set aside (>= nb: not in this tile)
-                        // (splitting a ragged last tile evenly between the row's two warps was measured and is no faster:
-                        // the tile's arithmetic, not the longer of its two shares, is what takes the time)
-                        const int pk = parked ? kPer : max(0, (p.t0 - (col0 + b0 * 16)) >> 4);
-                        const uint32_t sc = scale4 + b0 * 64, tl = t_lane;
-                        before = best;
-                        if (nb == kPer && pk >= kPer) {
-                            match_blocks<kPer>(tl, sc, best, win);
-                        } else {
-                            // (the group boundary is a multiple of 32 columns, the warp's share starts at one: pairs of blocks)
+                        // (the group boundary is a multiple of 32 columns, the warp's share starts at one: pairs of blocks)
 #pragma unroll
-                            for (int i = 0; i < kPer; i += 2) {
-                                if (i < nb) {
-                                    if (i == pk) park(t);
-                                    const bool two = i + 1 < nb;
-                                    switch (i) {                     // (the block's number is a compile-time constant)
-                                        case 0: if (two) match_block32<0>(tl, sc, best, win); else match_block16<0>(tl, sc, best, win); break;
-                                        case 2: if (two) match_block32<2>(tl + 32, sc + 128, best, win); else match_block16<2>(tl + 32, sc + 128, best, win); break;
-                                        case 4: if (two) match_block32<4>(tl + 64, sc + 256, best, win); else match_block16<4>(tl + 64, sc + 256, best, win); break;
-                                        default: if (two) match_block32<6>(tl + 96, sc + 384, best, win); else match_block16<6>(tl + 96, sc + 384, best, win); break;
-                                    }
+                        for (int i = 0; i < kPer; i += 2) {
+                            if (i < nb) {
+                                if (i == pk) park(t);
+                                const bool two = i + 1 < nb;
+                                switch (i) {                     // (the block's number is a compile-time constant)
+                                    case 0: if (two) match_block32<0>(tl, sc, best, win); else match_block16<0>(tl, sc, best, win); break;
+                                    case 2: if (two) match_block32<2>(tl + 32, sc + 128, best, win); else match_block16<2>(tl + 32, sc + 128, best, win); break;
+                                    case 4: if (two) match_block32<4>(tl + 64, sc + 256, best, win); else match_block16<4>(tl + 64, sc + 256, best, win); break;
+                                    default: if (two) match_block32<6>(tl + 96, sc + 384, best, win); else match_block16<6>(tl + 96, sc + 384, best, win); break;
                                 }
                             }
                         }
-                        if (best > before) best_tile = t;            // the winner moved into this tile
                     }
+                    if (best > before) best_tile = t;                // the winner moved into this tile
                     S::acc_release(c);
                 }
             }
@@ -517,7 +487,10 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
             int slot = -1;
             if (ok && active) {
                 slot = resolve();
-                if (match_better(val_a, slot_a, best, slot)) { best = val_a; slot = slot_a; }
+                if (row_masked) {                                        // the group of the row's own modality counts
+                    if (my_mod == 0 && parked) { best = val_a; slot = slot_a; }
+                    if (my_mod != 0 && !parked) slot = -1;
+                } else if (match_better(val_a, slot_a, best, slot)) { best = val_a; slot = slot_a; }
             }
             // the upper column half hands its result and its half of the norm to the lower one, which owns the row's output
             if (c.colhalf == 1) tc::sts128(wrow, best, __int_as_float(slot), ssq, 0.f);

@@ -322,19 +322,6 @@ struct Skel {
             f(ch, a);
         }
     }
-    // The same walk in blocks of 16 columns (for epilogues that are short of registers): f(block, values)
-    // for the blocks of this warp's column half below n_blocks = ceil(columns of the tile / 16).
-    template <class F>
-    static __device__ __forceinline__ void for_each_block16(const Ctx &c, int n_blocks, F &&f) {
-        constexpr int kPer = NB / 32;
-        const int hi = min(n_blocks, kPer * c.colhalf + kPer);
-        for (int b = kPer * c.colhalf; b < hi; ++b) {
-            uint32_t a[16];
-            tc::tmem_ld16(c.tmem_base + c.group * NB + b * 16 + ((uint32_t)(c.quarter * 32) << 16), a);
-            tc::tmem_ld_wait(a);
-            f(b, a);
-        }
-    }
     // The same for epilogues in which all sixteen warps drain one accumulator at a time (warp = 32 lanes x
     // a quarter of the columns, both halves in turn): explicit half index, `k` = tiles of that half so far.
     static __device__ __forceinline__ bool acc_wait_h(const Ctx &c, int h, int k, int *status) {

@@ -208,3 +208,11 @@ def test_scoring_over_runs_of_tiles():
         (1, 3, 1, 1030, 32, 40),         # 96 rows
     ]:
         _random_case(rng, U, Hq, Hkv, 128, L, W, B, F.BF16, tau=4.0, tau_mode=O.TAU_REL, theta=0.4)
+
+
+@pytest.mark.parametrize("L,B,vis", [(1500, 300, 0.5), (1100, 257, 0.03), (1100, 400, 0.97), (700, 290, 1.0), (700, 290, 0.0), (2304, 600, 0.2)])
+def test_intra_modal_tiles_of_both_modalities(L, B, vis):
+    """Long pivot lists in an intra-modal layer whose tiles hold tokens of both modalities: the boundary of the two candidate
+    groups inside the first tile of columns, in a later one, at the end, or with one of the groups empty."""
+    _random_case(np.random.default_rng(41), 2, 8, 2, 128, L, 32, B, F.BF16, vis_frac=vis, tau=4.0, tau_mode=O.TAU_REL, theta=0.5,
+                 flow_mode=O.FLOW_FORCE_INTRA)
