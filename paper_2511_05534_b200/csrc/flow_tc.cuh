@@ -70,7 +70,8 @@ flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
         S::mma_issuer<true>(c, A.n_items, plan, A.status);
     } else {
         const int row = c.quarter * 32 + c.lane;                     // row of the half
-        const uint32_t xch = c.epi_addr() + row * 16, pxch = c.partner_addr() + row * 16;   // hand-over slot of this row, the other column half's
+        const uint32_t xch = c.epi_addr() + row * 16, pxch = c.partner_addr() + row * 16;   // hand-over slots of this row, the other column half's
+        uint32_t turn = 0;                                           // two slots by turns: the next meeting keeps the upper half from one still being read
         int k = 0;
         bool ok = true;
         FlowItem f_next;
@@ -139,17 +140,17 @@ flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
             }
             // The two column halves of every row meet.  (After a wait that ran out the meeting is still kept: the vote ends the
             // loop for both warps.)
-            if (c.colhalf == 1) tc::sts128(xch, m, l, lc, 0.f);
+            if (c.colhalf == 1) tc::sts128(xch + turn, m, l, lc, 0.f);
             ok = !S::pair_meet(c, !ok);
             if (c.colhalf == 0 && ok) {
-                const float4 o = tc::lds128(pxch);
+                const float4 o = tc::lds128(pxch + turn);
                 const float mx = fmaxf(m, o.x), wa = tc::ex2(m - mx), wb = tc::ex2(o.x - mx);
                 const float z = l * wa + o.y * wb, zc = lc * wa + o.z * wb;
                 const float share = warp_sum(active && r0 + c.lane < A.L && z > 0.f ? zc / z : 0.f);   // (a half without rows: 0)
                 if (c.lane == 0)
                     A.parts[((int64_t)(f.rp * 2 + c.group) * 4 + c.quarter) * (int64_t)A.n_heads + (int64_t)f.u * A.Hq + f.head] = share;
             }
-            S::pair_sync(c);                                         // the hand-over slot may be overwritten again
+            turn ^= tcs::kRows * 16;
         }
     }
     S::teardown(c);

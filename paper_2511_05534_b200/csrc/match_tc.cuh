@@ -199,26 +199,25 @@ struct MatchItem {
 
 // What an item's plan reads from global memory; kept apart so that a role can fetch the next item's
 // values while it works on the current one.
-struct MatchRaw { int n_text, n_vis, strategy, tile_mod; };
+struct MatchRaw { int uh, u, rt, n_text, n_vis, strategy, tile_mod; };
 
 __device__ __forceinline__ MatchRaw match_raw(const MatchTcArgs &A, int item) {
-    MatchRaw r = {0, 0, 1, 0};
+    MatchRaw r = {0, 0, 0, 0, 0, 1, 0};
     if (item >= A.n_items) return r;
-    const int uh = (int)A.by_nrt.div(item), rt = item - uh * A.n_rt, u = (int)A.by_hkv.div(uh);
-    r.n_text = A.cand_count[2 * uh]; r.n_vis = A.cand_count[2 * uh + 1];
-    r.strategy = A.strategy[u];
-    r.tile_mod = A.tile_mod[(int64_t)u * A.n_rt + rt];
+    r.uh = (int)A.by_nrt.div(item); r.rt = item - r.uh * A.n_rt; r.u = (int)A.by_hkv.div(r.uh);
+    r.n_text = A.cand_count[2 * r.uh]; r.n_vis = A.cand_count[2 * r.uh + 1];
+    r.strategy = A.strategy[r.u];
+    r.tile_mod = A.tile_mod[(int64_t)r.u * A.n_rt + r.rt];
     return r;
 }
 
 // Which candidate columns a tile of 256 tokens has to visit: everything in a cross-modal layer or
 // when the tile mixes modalities, otherwise only the group of the tile's modality.
 template <class S>
-__device__ __forceinline__ MatchItem match_plan(const MatchTcArgs &A, int item, const MatchRaw &raw) {
+__device__ __forceinline__ MatchItem match_plan(const MatchTcArgs &A, const MatchRaw &raw) {
     constexpr int kMtCols = S::kCols;        // candidates per column tile
     MatchItem p;
-    p.uh = (int)A.by_nrt.div(item); p.rt = item - p.uh * A.n_rt;
-    p.u = (int)A.by_hkv.div(p.uh); p.h = p.uh - p.u * A.Hkv;
+    p.uh = raw.uh; p.rt = raw.rt; p.u = raw.u; p.h = p.uh - p.u * A.Hkv;
     p.n_text = raw.n_text; p.n_vis = raw.n_vis;
     p.t0 = (p.n_text + 31) & ~31;
     p.intra = raw.strategy == 0;
@@ -241,7 +240,7 @@ __device__ __forceinline__ MatchItem match_plan(const MatchTcArgs &A, int item, 
 }
 template <class S>
 __device__ __forceinline__ MatchItem match_plan(const MatchTcArgs &A, int item) {
-    return match_plan<S>(A, item, match_raw(A, item));
+    return match_plan<S>(A, match_raw(A, item));
 }
 
 // The inner step of the epilogue, written out in PTX so that it stays inside what the tensor core leaves room for:
@@ -379,31 +378,31 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
     } else {
         const int lane = c.lane, row = c.quarter * 32 + lane;
         const int b0 = kPer * c.colhalf;                         // first block of this warp's share of a tile
-        const uint32_t wrow = c.epi_addr() + row * 16;          // hand-over slot of this row
+        const uint32_t wrow = c.epi_addr() + row * 16;          // hand-over slots of this row, by turns
         const uint32_t prow = c.partner_addr() + row * 16;      // the other column half's
+        uint32_t turn = 0;
         const uint32_t t_lane = c.tmem_base + c.group * kMtCols + b0 * 16 + ((uint32_t)(c.quarter * 32) << 16);
         int k = 0, bt = 0, n_mine = 0;
         bool ok = true;
         // what an item needs from global memory is fetched one item ahead: its plan values, the token's
         // modality and its place in the non-pivot list
-        auto token_of = [&](int item) { return (item - (int)A.by_nrt.div(item) * A.n_rt) * kMtItemRows + c.group * kMtRows + row; };
-        auto fetch_mod = [&](int item) -> int {
-            const int token = token_of(item);
-            return item < A.n_items && token < A.L ? A.modality[(int64_t)A.by_hkv.div(A.by_nrt.div(item)) * A.L + token] : 0;
+        auto fetch_mod = [&](const MatchRaw &r, int item) -> int {
+            const int token = r.rt * kMtItemRows + c.group * kMtRows + row;
+            return item < A.n_items && token < A.L ? A.modality[(int64_t)r.u * A.L + token] : 0;
         };
-        auto fetch_rank = [&](int item) -> int {
-            const int token = token_of(item);
-            return item < A.n_items && token < A.L ? A.rank[(int64_t)A.by_nrt.div(item) * A.L + token] : -1;
+        auto fetch_rank = [&](const MatchRaw &r, int item) -> int {
+            const int token = r.rt * kMtItemRows + c.group * kMtRows + row;
+            return item < A.n_items && token < A.L ? A.rank[(int64_t)r.uh * A.L + token] : -1;
         };
         MatchRaw raw_next = match_raw(A, blockIdx.x);
-        int mod_next = fetch_mod(blockIdx.x), rank_next = fetch_rank(blockIdx.x);
+        int mod_next = fetch_mod(raw_next, blockIdx.x), rank_next = fetch_rank(raw_next, blockIdx.x);
         for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x) {
             const MatchRaw raw = raw_next;
             const int my_mod = mod_next, my_rank = rank_next;
             raw_next = match_raw(A, item + gridDim.x);
-            mod_next = fetch_mod(item + gridDim.x);
-            rank_next = fetch_rank(item + gridDim.x);
-            const MatchItem p = match_plan<S>(A, item, raw);
+            mod_next = fetch_mod(raw_next, item + gridDim.x);
+            rank_next = fetch_rank(raw_next, item + gridDim.x);
+            const MatchItem p = match_plan<S>(A, raw);
             const bool active = !p.tp.empty() && c.group < p.tp.n_halves;
             const int token = p.rt * kMtItemRows + c.group * kMtRows + row;
             const bool in_range = token < A.L;
@@ -493,10 +492,10 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 } else if (match_better(val_a, slot_a, best, slot)) { best = val_a; slot = slot_a; }
             }
             // the upper column half hands its result and its half of the norm to the lower one, which owns the row's output
-            if (c.colhalf == 1) tc::sts128(wrow, best, __int_as_float(slot), ssq, 0.f);
+            if (c.colhalf == 1) tc::sts128(wrow + turn, best, __int_as_float(slot), ssq, 0.f);
             ok = !S::pair_meet(c, !ok);                            // (both warps of a row go on, or neither)
             if (c.colhalf == 0 && ok) {
-                const float4 other = tc::lds128(prow);
+                const float4 other = tc::lds128(prow + turn);
                 if (match_better(other.x, __float_as_int(other.y), best, slot)) { best = other.x; slot = __float_as_int(other.y); }
                 ssq += other.z;
                 if (in_range) {
@@ -509,7 +508,7 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                     }
                 }
             }
-            S::pair_sync(c);                                       // the hand-over slot may be overwritten again
+            turn ^= kMtRows * 16;                                  // (the next meeting keeps the upper half from a slot that is still being read)
         }
     }
     S::teardown(c);

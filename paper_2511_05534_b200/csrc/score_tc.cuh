@@ -278,7 +278,11 @@ __device__ __forceinline__ float colsum_chunk32(uint32_t taddr, uint32_t negc, f
 
 // ---------------------------------------------------------------------------------------------
 // Pass 2.  item = (unit*head, tile of 256 keys); the B stream is the head group's proxy rows.  A CTA takes a run of
-// consecutive items, so that with up to 256 proxy rows per head they are loaded once per head, not once per item.
+// consecutive items, so that proxy rows that fit the B stages (up to 512) are loaded once per head, not once per item.
+// Bound by the epilogue (four warps per scheduler, exp2 at half of its rate): what an item costs besides its exponentials
+// counts.  Its place in the run is stepped, not divided out, the two column halves of a key meet once per item, and two
+// heads' masses are summed over the warp together: 112 heads of 8448 tokens, 448 rows each, 158 -> 148 us; 128 heads of 33792,
+// 512 rows, 861 -> 812 us; 112 of 2176, 224 rows, 34.5 -> 30.8 us.
 template <class S>
 __global__ void __launch_bounds__(tcs::kThreads, 1)
 score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap q_map,
@@ -298,8 +302,8 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
         p.b1 = 0; p.b2 = h * A.G; p.b3 = u; p.step1 = 0; p.step2 = S::kCols / A.W;
         p.cols_total = A.GW;
         p.n_tiles = (A.GW + S::kCols - 1) / S::kCols;
-        p.reuse_b = p.n_tiles == 1 && kt > 0 && g > g_lo;
-        p.keep_b = p.n_tiles == 1 && kt + 1 < A.n_rt && g + 1 < g_hi;
+        p.reuse_b = p.n_tiles <= S::kBStages && kt > 0 && g > g_lo;
+        p.keep_b = p.n_tiles <= S::kBStages && kt + 1 < A.n_rt && g + 1 < g_hi;
         p.extra = A.negc + (int64_t)uh * A.GWpad;        // row constants of pass 1, 256 per B tile
         return p;
     };
@@ -316,41 +320,60 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
         const int w_shift = 31 - __clz(A.W);
         uint32_t wbits[4] = {0, 0, 0, 0};                            // modality of the proxy tokens, 32 per word
         bool ok = true;
-        auto fetch_mod = [&](int g) -> int {                         // modality of this thread's key, an item ahead
-            if (g >= g_hi) return 0;
-            const int uh = (int)A.by_rt.div(g), key = (g - uh * A.n_rt) * tcs::kItemRows + c.group * tcs::kRows + row;
-            return key < A.L ? A.modality[(int64_t)A.by_hkv.div(uh) * A.L + key] : 0;
+        // the run's items one after the other: (unit u, KV head uh, its tile kt) step by step instead of by divisions, which
+        // together with the rest of an item's start took a tenth of the epilogue's time
+        const int n_tiles = (A.GW + S::kCols - 1) / S::kCols;
+        int uh = (int)A.by_rt.div(g_lo), kt = g_lo - uh * A.n_rt, u = (int)A.by_hkv.div(uh), hk = uh - u * A.Hkv;
+        const int key_in_item = c.group * tcs::kRows + row;
+        auto fetch_mod = [&](int u, int kt) -> int {                 // modality of this thread's key, an item ahead
+            const int key = kt * tcs::kItemRows + key_in_item;
+            return key < A.L ? A.modality[(int64_t)u * A.L + key] : 0;
         };
-        int mod_next = fetch_mod(g_lo);
+        int mod_next = g_lo < g_hi ? fetch_mod(u, kt) : 0;
+        uint32_t slot = 0;                                           // hand-over slots by turns
         for (int g = g_lo; ok && g < g_hi; ++g) {
-            const tcs::TilePlan p = plan(blockIdx.x + (g - g_lo) * gridDim.x);
-            const int uh = (int)A.by_rt.div(g), kt = g - uh * A.n_rt, u = (int)A.by_hkv.div(uh), h = uh - u * A.Hkv;
+            const int uh0 = uh, kt0 = kt, u0 = u, h0 = hk;           // this item
+            if (++kt == A.n_rt) {                                    // the next one
+                kt = 0; ++uh;
+                if (++hk == A.Hkv) { hk = 0; ++u; }
+            }
             const bool my_vis = mod_next != 0;
-            mod_next = fetch_mod(g + 1);
-            if (p.reuse_b) --bt;                                     // (bt: number of the B tile an item begins with)
-            float *cross_out = A.cross_part + ((int64_t)u * A.Hq + h * A.G) * (A.n_rt * 8) + kt * 8 + c.group * 4 + c.quarter;
-            if (c.group >= p.n_halves) {                             // no keys in this half: its masses are zero
+            mod_next = g + 1 < g_hi ? fetch_mod(u, kt) : 0;
+            if (n_tiles <= S::kBStages && kt0 > 0 && g > g_lo) bt -= n_tiles;   // TilePlan::reuse_b (bt: number of the B tile an item begins with)
+            const int key0 = kt0 * tcs::kItemRows + c.group * tcs::kRows;
+            float *cross_out = A.cross_part + ((int64_t)u0 * A.Hq + h0 * A.G) * (A.n_rt * 8) + kt0 * 8 + c.group * 4 + c.quarter;
+            if (key0 >= A.L) {                                       // no keys in this half: its masses are zero
                 if (lane == 0)
-                    for (int g = 0; g < A.G; ++g) cross_out[(int64_t)g * (A.n_rt * 8)] = 0.f;
-                bt += p.n_tiles;                                     // keep the B-tile count in step
+                    for (int j = 0; j < A.G; ++j) cross_out[(int64_t)j * (A.n_rt * 8)] = 0.f;
+                bt += n_tiles;                                       // keep the B-tile count in step
                 continue;
             }
-            if (u != cached_u) {
+            if (u0 != cached_u) {
 #pragma unroll
                 for (int w = 0; w < 4; ++w) {
                     const int a = w * 32 + lane;
-                    const bool vis = a < A.W && A.modality[(int64_t)u * A.L + A.L - A.W + a] != 0;
+                    const bool vis = a < A.W && A.modality[(int64_t)u0 * A.L + A.L - A.W + a] != 0;
                     wbits[w] = __ballot_sync(0xFFFFFFFFu, vis);
                 }
-                cached_u = u;
+                cached_u = u0;
             }
-            const int key0 = kt * tcs::kItemRows + c.group * tcs::kRows;
             const int key = key0 + row;
             const bool masked_tile = key0 + tcs::kRows > A.L - A.W + 1;   // some (key, proxy row) pair is masked
             const int first_proxy = A.L - A.W;
             float imp = 0.f, cg = 0.f;
             int cur_g = -1;                                          // head whose mass is being summed; -1: none yet
-            for (int t = 0; ok && t < p.n_tiles; ++t, ++bt) {
+            float held = 0.f;                                        // a complete head's mass that waits for the next one's:
+            int held_g = -1;                                         // two are summed over the warp together
+            auto publish = [&]() {
+                if (held_g < 0) { held = cg; held_g = cur_g; return; }
+                const bool up = lane & 16;                           // the held head goes to the lower lanes, this one to the upper
+                float x = (up ? cg : held) + __shfl_xor_sync(0xFFFFFFFFu, up ? held : cg, 16);
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
+                if ((lane & 15) == 0) cross_out[(int64_t)(up ? cur_g : held_g) * (A.n_rt * 8)] = x;
+                held_g = -1;
+            };
+            for (int t = 0; ok && t < n_tiles; ++t, ++bt) {
                 const int ncols = min(S::kCols, A.GW - t * S::kCols);
                 if (!S::takes_part(c, ncols)) continue;
                 ok = S::extra_wait(c, bt, A.status) && S::quad_wait(c, k++, A.status);
@@ -362,10 +385,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                     const int col = t * S::kCols + ch * 32;        // proxy row index r = g_local * W + a
                     const int g_local = col >> w_shift, a0 = col & (A.W - 1);   // (the window is 32, 64 or 128 rows)
                     if (g_local != cur_g) {                          // a head is complete: publish its mass
-                        if (cur_g >= 0) {
-                            const float tot = warp_sum(cg);
-                            if (lane == 0) cross_out[(int64_t)cur_g * (A.n_rt * 8)] = tot;
-                        }
+                        if (cur_g >= 0) publish();
                         cg = 0.f;
                         cur_g = g_local;
                     }
@@ -421,15 +441,19 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                 S::quad_release(c);
             }
             if (ok && cur_g >= 0) {
-                const float tot = warp_sum(cg);
-                if (lane == 0) cross_out[(int64_t)cur_g * (A.n_rt * 8)] = tot;
+                publish();
+                if (held_g >= 0) {
+                    const float tot = warp_sum(held);
+                    if (lane == 0) cross_out[(int64_t)held_g * (A.n_rt * 8)] = tot;
+                }
             }
             // the two column halves of a key meet: the upper one hands its partial sum over (kept even after a
-            // wait ran out, so that the partner warp is never left waiting)
-            if (c.colhalf == 1) tc::sts32(xch, imp);
+            // wait ran out, so that the partner warp is never left waiting).  Two slots by turns: the next meeting keeps the
+            // upper half from a slot that is still being read.
+            if (c.colhalf == 1) tc::sts32(xch + slot, imp);
             ok = !S::pair_meet(c, !ok);                            // (both warps of a key go on, or neither)
-            if (c.colhalf == 0 && ok && key < A.L) A.importance[(int64_t)uh * A.L + key] = (imp + tc::lds32(pxch)) / (float)A.G;   // group mean
-            S::pair_sync(c);
+            if (c.colhalf == 0 && ok && key < A.L) A.importance[(int64_t)uh0 * A.L + key] = (imp + tc::lds32(pxch + slot)) / (float)A.G;   // group mean
+            slot ^= tcs::kRows * 4;
         }
     }
     S::teardown(c);

@@ -23,7 +23,7 @@
 // Three shapes are instantiated: Skel<256, 1, 2> for long B streams (one A stage per half, two 64 KB B
 // stages), and for problems whose items have few B columns, where the A operand is the stream, Skel<128, 2, 2>
 // and Skel<256, 2, 1>: two A stages per half let the next item's rows load while this item is computed, and an item
-// whose single B tile is the previous item's (TilePlan::reuse_b) takes it as it stands.
+// whose B tiles are the previous item's and still in their stages (TilePlan::reuse_b) takes them as they stand.
 #pragma once
 #include "common.cuh"
 #include "tc_common.cuh"
@@ -50,8 +50,8 @@ struct TilePlan {
     int n_tiles;               // 0: every role skips the item
     int cols_total;            // valid B rows over all tiles (tile t has min(NB, cols_total - NB t))
     int cols_first = 0;        // ... for A half 0, where it needs fewer in the last tile (0: the same)
-    bool reuse_b = false;      // the item's only B tile (and its constants) is the one the item before ended with
-    bool keep_b = false;       // ... and the next item's as well: its stage is not handed back after this item
+    bool reuse_b = false;      // the item's B tiles (and their constants), at most as many as there are stages, are those of the item before
+    bool keep_b = false;       // ... and the next item's as well: their stages are not handed back after this item
     const float *extra;        // nullptr, or NB fp32 per-column constants per tile: tile t reads extra + NB t
     __device__ __forceinline__ bool empty() const { return n_tiles == 0 || n_halves == 0; }
 };
@@ -59,7 +59,7 @@ struct TilePlan {
 template <int NB, int AST, int BST>
 struct Skel {
     static constexpr int kCols = NB;                         // rows of a B tile (UMMA N)
-    static constexpr int kAStages = AST;
+    static constexpr int kAStages = AST, kBStages = BST;
     static constexpr uint32_t kBStage = NB * 128 * 2;
     static constexpr uint32_t kExtraBytes = NB * 4;          // per-column fp32 constants that travel with a B tile
     static constexpr uint32_t kSmemA = 0;                    // [stage][half]
@@ -213,10 +213,10 @@ struct Skel {
         for (int item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
             const TilePlan p = plan(item);
             if (p.empty()) continue;
-            for (int t = 0; ok && t < p.n_tiles; ++t) {
-                if (!p.reuse_b) ++bt;
-                const int sb = (bt - 1) % BST;                           // bt: B tiles taken so far, this one included
-                ok = tc::mbar_wait_warp(c.bar(kBarBFull + sb), ((bt - 1) / BST) & 1, c.abort_flag, status);
+            if (p.reuse_b) bt -= p.n_tiles;                              // bt: number of the B tile
+            for (int t = 0; ok && t < p.n_tiles; ++t, ++bt) {
+                const int sb = bt % BST;
+                ok = tc::mbar_wait_warp(c.bar(kBarBFull + sb), (bt / BST) & 1, c.abort_flag, status);
                 if (!ok) break;
                 const int ncols = min(NB, p.cols_total - t * NB);
                 const int ncols0 = p.cols_first ? min(NB, p.cols_first - t * NB) : ncols;
@@ -358,10 +358,6 @@ struct Skel {
             : "r"((uint32_t)gave_up), "r"(1 + c.group * 4 + c.quarter)
             : "memory");
         return any != 0;
-    }
-    // Meeting point of the two warps that share rows (same half, same lanes, other columns).
-    static __device__ __forceinline__ void pair_sync(const Ctx &c) {
-        asm volatile("bar.sync %0, 64;" ::"r"(1 + c.group * 4 + c.quarter) : "memory");
     }
 };
 
