@@ -34,9 +34,9 @@ __device__ __forceinline__ constexpr bool index_ok(long long, long long, int *) 
 __device__ __forceinline__ void predecessor_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---- thread-block clusters ----------------------------------------------------------------------
-// (every thread of the cluster calls these, converged warps)
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// (every thread of the cluster calls these)
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
 // a 32-bit word in the shared memory of the cluster's CTA `rank`, at this CTA's shared address `addr`
 __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr, int rank) {
@@ -44,6 +44,18 @@ __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t addr, int rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
     asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(remote) : "memory");
     return v;
+}
+__device__ __forceinline__ uint4 ld_cluster_u128(uint32_t addr, int rank) {
+    uint32_t remote;
+    uint4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(remote) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, int rank, uint32_t v) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(v) : "memory");
 }
 __device__ __forceinline__ float ld_cluster(uint32_t addr, int rank) { return __uint_as_float(ld_cluster_u32(addr, rank)); }
 

@@ -446,12 +446,12 @@ MatchPrepArgs match_prep_args(const flowmm_params &p, const Layout &y, const voi
     return g;
 }
 
-template <int kThreads, bool kOneChunk>
+template <int kThreads, bool kOneChunk, int kCtas = 1>
 flowmm_status launch_select(const SelectArgs &a, const SelectFlow &f, const MatchPrepArgs &g, int with_prepare, cudaStream_t st) {
     const size_t smem = select_smem(a.chunk);
-    if (cudaFuncSetAttribute(select_topb_kernel<kThreads, kOneChunk>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(select_topb_kernel<kThreads, kOneChunk, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
-    launch(select_topb_kernel<kThreads, kOneChunk>, a.n_heads + f.n_units, kThreads, smem, st, a, f, g, with_prepare);
+    launch_cluster(dim3(kCtas), select_topb_kernel<kThreads, kOneChunk, kCtas>, (a.n_heads + f.n_units) * kCtas, kThreads, smem, st, a, f, g, with_prepare);
     FLOWMM_LAUNCHED("select_topb");
     return FLOWMM_OK;
 }
@@ -473,6 +473,13 @@ flowmm_status run_select(const flowmm_params &p, const float *importance, int32_
     const SelectFlow &f = flow ? *flow : no_flow;
     // Warps per head: a block's latency is its rounds of shared-memory work, which shrink with more warps until the
     // barriers outweigh them (640 tokens) or other heads' blocks no longer fit beside it
+    // Long contexts of few heads: four CTAs for each (from about 6000 positions on their shares outweigh the cluster's
+    // barriers; two save less, eight no more)
+    const int part = (p.seq_len + 1023) / 1024 * 256;
+    if (p.seq_len >= 6144 && part <= kSelMaxChunk && 4 * a.n_heads <= tc::sm_count()) {
+        a.chunk = part;
+        return launch_select<512, true, 4>(a, f, g, prep != nullptr, st);
+    }
     if (p.seq_len <= 1024) return launch_select<256, true>(a, f, g, prep != nullptr, st);
     if (p.seq_len <= 4096) return launch_select<512, true>(a, f, g, prep != nullptr, st);
     if (p.seq_len <= kSelMaxChunk) return launch_select<1024, true>(a, f, g, prep != nullptr, st);

@@ -33,7 +33,7 @@ struct SelectArgs {
     int *retained, *evicted;     // [n_heads, B], [n_heads, L - B]
     uint8_t *row_mod_out;        // nullptr, or [n_heads, B]: the pivots' modalities (one modality map per head: P.Hkv == 1)
     int n_heads, L, B, W, keep_window;
-    int chunk;                   // positions handled at a time, a multiple of 32: the whole context if it fits in shared memory
+    int chunk;                   // positions handled at a time, a multiple of 32: the whole context if it fits in shared memory, or a CTA's part of it
 };
 
 // The extra block of unit u.  Sums as in cross_mass_reduce and layer_flow_kernel, term for term.
@@ -85,27 +85,34 @@ static_assert(select_smem(kSelMaxChunk) <= 232448 - 1024, "shared memory budget"
 // Bound by latency: one block per head, a few dependent rounds over shared memory.  The marks and
 // one prefix sum replace block-wide scans per 1024 to 4096 positions, four counting passes over global memory and a separate
 // preparation pass over the lists: 128 heads of 33 792 tokens 118 -> 42 us, 32 heads of 640 tokens 20 -> 10 us.
-template <int kThreads, bool kOneChunk>
+// kCtas > 1: the CTAs of a cluster share a head, A.chunk positions each (a multiple of 256).  The counts of all of them are
+// added up through distributed shared memory in every pass, their totals before the lists are written.  For calls of few
+// heads, whose blocks would leave most SMs idle: 8 heads of 33 792 tokens 31 -> 18 us, 4 heads of 8448 14 -> 12.
+template <int kThreads, bool kOneChunk, int kCtas>
 __global__ void __launch_bounds__(kThreads)
 select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P, int with_prepare) {
+    static_assert(kCtas == 1 || (kOneChunk && kThreads == 512), "a CTA's part is one chunk; four counters per thread");
     constexpr int kWarps = kThreads / 32, kPer = kSelBins / kThreads;
     extern __shared__ __align__(16) int sel_smem[];
     __shared__ int wtot[kWarps], res[3];
     __shared__ unsigned long long wsum[kWarps];
+    __shared__ uint32_t xtot[3];                                     // a CTA's totals, for the others of the cluster
     int *hist = sel_smem;
     uint32_t *words = reinterpret_cast<uint32_t *>(sel_smem + 2 * kSelBins);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int head = blockIdx.x, L = A.L;
+    const int head = blockIdx.x / kCtas, rank_c = kCtas > 1 ? (int)(blockIdx.x % kCtas) : 0;
+    const int i0 = rank_c * A.chunk;                                 // first position of this CTA's part (kCtas == 1: 0)
+    const int L = kCtas > 1 ? max(0, min(A.chunk, A.L - i0)) : A.L;  // positions this CTA looks at; counted from i0 below
     for (int i = tid; i < 2 * kSelBins / 4; i += kThreads) reinterpret_cast<int4 *>(hist)[i] = make_int4(0, 0, 0, 0);
     __syncthreads();
     predecessor_done();
     if (head >= A.n_heads) {
-        select_flow_block(F, head - A.n_heads, A.W, reinterpret_cast<float *>(hist));
+        if (rank_c == 0) select_flow_block(F, head - A.n_heads, A.W, reinterpret_cast<float *>(hist));
         return;
     }
-    const float *imp = A.importance + (int64_t)head * L;
-    const uint8_t *mod = P.modality + (int64_t)(head / P.Hkv) * L;   // (not read unless with_prepare)
-    const int first_forced = A.keep_window ? L - A.W : L;
+    const float *imp = A.importance + (int64_t)head * A.L + i0;
+    const uint8_t *mod = P.modality + (int64_t)(head / P.Hkv) * A.L + i0;   // (not read unless with_prepare or row_mod_out)
+    const int first_forced = (A.keep_window ? A.L - A.W : A.L) - i0;
     auto word = [&](int i) -> uint32_t {
         if (kOneChunk) return words[i];
         return select_key(imp[i], i >= first_forced) | (with_prepare && mod[i] ? 0x80000000u : 0u);
@@ -144,12 +151,23 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
         if (pass > 0) {
             for (int i = tid; i < L; i += kThreads) count(word(i) & kKeyMask, h, shift, width);
         }
-        __syncthreads();
+        if (kCtas > 1) cluster_sync(); else __syncthreads();
         // counters from the largest digit down, kPer per thread; thread t holds digits hi - kPer + 1 .. hi
         const int hi = kSelBins - 1 - tid * kPer;
         int c[kPer], sum = 0;
+        if constexpr (kCtas > 1) {
+            const uint32_t at = (uint32_t)__cvta_generic_to_shared(h + hi - (kPer - 1));
+            uint4 part[kCtas];
 #pragma unroll
-        for (int e = 0; e < kPer; ++e) { c[e] = h[hi - e]; sum += c[e]; }
+            for (int q = 0; q < kCtas; ++q) part[q] = ld_cluster_u128(at, q);   // (scalar reads took four times as long)
+            c[0] = c[1] = c[2] = c[3] = 0;
+#pragma unroll
+            for (int q = 0; q < kCtas; ++q) { c[0] += (int)part[q].w; c[1] += (int)part[q].z; c[2] += (int)part[q].y; c[3] += (int)part[q].x; }
+            sum = (c[0] + c[1]) + (c[2] + c[3]);
+        } else {
+#pragma unroll
+            for (int e = 0; e < kPer; ++e) { c[e] = h[hi - e]; sum += c[e]; }
+        }
         int incl = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -178,7 +196,7 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
         n_eq = res[2];
         mask |= ((1u << width) - 1u) << shift;
         if (need == n_eq) break;                                     // all of them are kept: lower bits do not matter
-        if (pass == 1)                                               // the third digit takes the first one's counters
+        if (pass == 1)                                               // the third digit takes the first one's counters, which every CTA has read
             for (int i = tid; i < kSelBins; i += kThreads) hist[i] = 0;
         __syncthreads();
     }
@@ -192,8 +210,8 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
     int *pt_w = pos_w + chunk_w, *pv_w = pt_w + chunk_w;             // and how many candidates
     const uint32_t lt = lanemask_lt();
     int *ret = A.retained + (int64_t)head * A.B;
-    int *evi = A.evicted + (int64_t)head * (L - A.B);
-    int *rank = P.rank + (int64_t)head * L;
+    int *evi = A.evicted + (int64_t)head * (A.L - A.B) + i0;
+    int *rank = P.rank + (int64_t)head * A.L + i0;
     int *cand_tok = hist;                                            // token of every candidate column (copy_here: up to 256)
     int *slot_out = P.cand_slot + (int64_t)head * P.Ctot;
     float *scale_out = P.cand_scale + (int64_t)head * P.Ctot;
@@ -218,11 +236,26 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
         total = all;
         return b + incl_v - v;
     };
+    // the same across the cluster: what the CTAs before this one hold, and all of them together
+    auto cluster_sum = [&](unsigned long long v, unsigned long long &total) -> unsigned long long {
+        if (tid == 0) { xtot[0] = (uint32_t)v; xtot[1] = (uint32_t)(v >> 32); }
+        cluster_sync();
+        const uint32_t at = (uint32_t)__cvta_generic_to_shared(xtot);
+        unsigned long long b = 0, all = 0;
+#pragma unroll
+        for (int q = 0; q < kCtas; ++q) {
+            const unsigned long long x = (unsigned long long)ld_cluster_u32(at, q) | (unsigned long long)ld_cluster_u32(at + 4, q) << 32;
+            if (q < rank_c) b += x;
+            all += x;
+        }
+        total = all;
+        return b;
+    };
     int t0 = 0;                                                      // first column of the visual candidates
     // (a context longer than a chunk is walked once more beforehand, for the number of its text candidates)
     for (int walk = kOneChunk || !with_prepare ? 1 : 0; walk < 2; ++walk) {
-        int seen = 0, seen_t = 0, seen_v = 0, seen_eq = 0;
-        for (int c0 = 0; c0 < L; c0 += A.chunk) {
+        int seen = 0, seen_t = 0, seen_v = 0, seen_eq = 0;           // before the chunk (kCtas > 1: in the CTAs before this one)
+        for (int c0 = 0; c0 < L || (kCtas > 1 && c0 == 0); c0 += A.chunk) {   // (a CTA without positions takes part all the same)
             const int n_w = (min(A.chunk, L - c0) + 31) >> 5, per = (n_w + kThreads - 1) / kThreads;
             if (!all_eq) {                                           // ties at the threshold go to the lower positions:
                 for (int w = warp; w < n_w; w += kWarps) {           // mark the equal keys, then number them
@@ -234,7 +267,14 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
                 const int w_lo = min(n_w, tid * per), w_hi = min(n_w, w_lo + per);   // words whose counts this thread adds up
                 unsigned long long n_mine = 0, tot;
                 for (int w = w_lo; w < w_hi; ++w) n_mine += __popc(text_w[w]);
-                int r = seen_eq + (int)block_sum(n_mine, tot);
+                int r = (int)block_sum(n_mine, tot);
+                if (kCtas > 1) {
+                    if (tid == 0) xtot[2] = (uint32_t)tot;
+                    cluster_sync();
+                    const uint32_t at = (uint32_t)__cvta_generic_to_shared(xtot + 2);
+                    for (int q = 0; q < rank_c; ++q) seen_eq += (int)ld_cluster_u32(at, q);
+                }
+                r += seen_eq;
                 for (int w = w_lo; w < w_hi; ++w) { pos_w[w] = r; r += __popc(text_w[w]); }
                 seen_eq += (int)tot;
                 __syncthreads();
@@ -275,6 +315,11 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
                 all = __shfl_sync(0xFFFFFFFFu, before, 31);
                 before -= mine;
             } else before = block_sum(mine, all);
+            if (kCtas > 1) {                                         // (from here on `all` is the head's)
+                const unsigned long long ahead = cluster_sum(all, all);
+                seen = (int)(ahead & 0xFFFFFF); seen_t = (int)(ahead >> 24) & 0xFFFFF; seen_v = (int)(ahead >> 44);
+                if (!copy_here) cluster_arrive();                    // the other CTAs' words have been read
+            }
             const int n_text = (int)(all >> 24) & 0xFFFFF, n_vis = (int)(all >> 44);
             if (kOneChunk) t0 = (n_text + 31) & ~31;                 // text group first, visual group from the next multiple of 32
             if (walk == 1) {
@@ -291,11 +336,11 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
                     const int i = c0 + 32 * w + lane, sl = pos_w[w] + __popc(keep & lt);
                     if (i >= L) continue;
                     if (!((keep >> lane) & 1u)) {
-                        evi[i - sl] = i;
-                        if (with_prepare) rank[i] = i - sl;
+                        evi[i - sl] = i0 + i;
+                        if (with_prepare) rank[i] = i0 + i - sl;
                         continue;
                     }
-                    ret[sl] = i;
+                    ret[sl] = i0 + i;
                     if (A.row_mod_out) A.row_mod_out[(int64_t)head * A.B + sl] = mod[i];
                     if (with_prepare) {
                         rank[i] = -(sl + 2);
@@ -303,30 +348,38 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
                         const int c = ((text >> lane) & 1u) ? pt_w[w] + __popc(text & lt) : ((vis >> lane) & 1u) ? pv_w[w] + __popc(vis & lt) : -1;
                         if (c >= 0 && index_ok(c, P.Ctot, P.status)) {
                             slot_out[c] = sl;
-                            if (copy_here) cand_tok[c] = i;
+                            if (copy_here) {
+                                if (kCtas > 1) {
+                                    const uint32_t at = (uint32_t)__cvta_generic_to_shared(cand_tok + c);
+#pragma unroll
+                                    for (int q = 0; q < kCtas; ++q) st_cluster_u32(at, q, (uint32_t)(i0 + i));
+                                } else cand_tok[c] = i;
+                            }
                         }
                     }
                 }
                 if (!kOneChunk) __syncthreads();                     // (the next chunk's words go into the same place)
             }
-            seen += (int)(all & 0xFFFFFF); seen_t += n_text; seen_v += n_vis;
+            if (kCtas > 1) { seen_t = n_text; seen_v = n_vis; }
+            else { seen += (int)(all & 0xFFFFFF); seen_t += n_text; seen_v += n_vis; }
         }
         if (walk == 0) t0 = (seen_t + 31) & ~31;
         else if (with_prepare) {
             // columns without a candidate: between the groups and behind them
             for (int c = seen_t + tid; c < P.Ctot; c += kThreads)
                 if (c < t0 || c >= t0 + seen_v) {
-                    slot_out[c] = -1;
-                    scale_out[c] = __int_as_float(0x7FC00000);       // NaN: no candidate here
+                    if (rank_c == 0) {
+                        slot_out[c] = -1;
+                        scale_out[c] = __int_as_float(0x7FC00000);   // NaN: no candidate here
+                    }
                     if (copy_here) cand_tok[c] = -1;
                 }
-            if (tid == 0) { P.cand_count[2 * head] = seen_t; P.cand_count[2 * head + 1] = seen_v; }
+            if (tid == 0 && rank_c == 0) { P.cand_count[2 * head] = seen_t; P.cand_count[2 * head + 1] = seen_v; }
         }
     }
-    if (!with_prepare) return;
-    if (head % P.Hkv == 0) {                                         // modalities in every tile of 256 tokens
-        const int u = head / P.Hkv;
-        for (int tl = warp; tl < P.n_rt; tl += kWarps) {
+    if (with_prepare && head % P.Hkv == 0) {                         // modalities in every tile of 256 tokens
+        const int u = head / P.Hkv, n_tiles = (L + kMtItemRows - 1) / kMtItemRows;
+        for (int tl = warp; tl < n_tiles; tl += kWarps) {
             uint32_t any_v = 0, any_t = 0;
 #pragma unroll
             for (int q = 0; q < kMtItemRows / 32; ++q) {
@@ -335,13 +388,14 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
                 any_v |= vis; any_t |= in && !vis;
             }
             any_v = __any_sync(0xFFFFFFFFu, any_v); any_t = __any_sync(0xFFFFFFFFu, any_t);
-            if (lane == 0) P.tile_mod[(int64_t)u * P.n_rt + tl] = (uint8_t)((any_t ? 1 : 0) | (any_v ? 2 : 0));
+            if (lane == 0) P.tile_mod[(int64_t)u * P.n_rt + i0 / kMtItemRows + tl] = (uint8_t)((any_t ? 1 : 0) | (any_v ? 2 : 0));
         }
     }
     if (copy_here) {
-        __syncthreads();
-        match_gather_rows<8>(P, head, cand_tok, 0, P.Ctot, tid, kThreads);
-    }
+        if (kCtas > 1) cluster_sync(); else __syncthreads();         // every candidate's token is in place, in every CTA
+        const int lo = P.Ctot / 32 * rank_c / kCtas * 32, hi = P.Ctot / 32 * (rank_c + 1) / kCtas * 32;
+        match_gather_rows<8>(P, head, cand_tok, lo, hi, tid, kThreads);
+    } else if (kCtas > 1) cluster_wait();                            // nobody's words go away while they are read
 }
 
 }  // namespace flowmm

@@ -33,7 +33,26 @@ def test_select_against_oracle(L, B, kind):
     assert np.array_equal(e.cpu().numpy(), ref_e)
 
 
-@pytest.mark.parametrize("L,B", [(290, 193), (2000, 225), (46000, 300)])
+@pytest.mark.parametrize("L,B", [(6143, 600), (6144, 600), (6145, 601), (8192, 8000), (33792, 1690), (45249, 77)])
+@pytest.mark.parametrize("U", [1, 18, 20])
+@pytest.mark.parametrize("kind", ["spread", "ties"])
+def test_select_by_clusters_and_by_blocks(L, B, U, kind):
+    """Long contexts with few heads (a cluster of CTAs for each, the last CTA's part short or empty) and with many (one block)."""
+    rng = np.random.default_rng(L + U)
+    imp = np.exp(rng.standard_normal((U, 2, L)) * 2).astype(np.float32)
+    if kind == "ties":
+        imp = np.round(imp * 2) / 2
+    p = O.OracleParams(U, 4, 2, 64, L, 16, B, keep_window=1)
+    ref_r, ref_e = O.select(p, imp.astype(np.float64))
+    fp = gpu_params(p, F.F32)
+    r = torch.full((U, 2, B), -9, dtype=torch.int32, device="cuda")
+    e = torch.full((U, 2, L - B), -9, dtype=torch.int32, device="cuda")
+    F.flowmm_select(fp, torch.from_numpy(imp).cuda(), r, e, F.alloc_workspace(fp))
+    assert np.array_equal(r.cpu().numpy(), ref_r)
+    assert np.array_equal(e.cpu().numpy(), ref_e)
+
+
+@pytest.mark.parametrize("L,B", [(290, 193), (7000, 130), (9000, 700), (2000, 225), (46000, 300)])
 def test_fused_preparation_equals_the_steps(L, B):
     """The candidate layout written by the selection launch of flowmm_compress_layer against the one flowmm_match makes
     from the lists: same matches, bit for bit (short lists, long lists, a context of more than one chunk)."""
