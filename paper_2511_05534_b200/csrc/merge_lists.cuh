@@ -598,4 +598,140 @@ __global__ void __launch_bounds__(256) merge_pieces_kernel(const MergeArgs A, in
     }
 }
 
+// Short lists (up to kShortList non-pivots per head): no member lists and no piece table.  A block holds the head's matches,
+// tokens and weights in shared memory, a warp finds the members of its slot by ballots over them, in ascending order, and
+// sums their rows as merge_pieces_kernel sums a piece (8 on their way at a time).  A slot of more than kSoloMembers is shared
+// by the block's warps, each with an eighth of the members; the parts are added in order.
+// Bound by latency: a chain of three loads, where the sort of the lists and the tables around it took a launch of its own.  The
+// call of 4 heads of 192 tokens (fp32) 40.6 -> 31.4 us, 8 of 950 62 -> 50, 112 of 640 with 423 slots (bf16) 110 -> 102.
+constexpr int kShortList = 1024, kSoloMembers = 64;
+
+// grid = (UH, slots / (8 * per_warp)), 256 threads
+template <typename T>
+__global__ void __launch_bounds__(256, 4) merge_short_kernel(const MergeArgs A, const int *match, const int *evicted, const float *match_sim,
+                                                             int merge_mode, int per_warp) {
+    constexpr int V = Elem<T>::kVec, kWarps = 8;
+    __shared__ int e_slot[kShortList], e_tok[kShortList];
+    __shared__ float e_w[kShortList];
+    __shared__ uint16_t members[kWarps][kSoloMembers];
+    __shared__ float part[kWarps][32][V + 1];
+    __shared__ int popular;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int uh = blockIdx.x, u = uh / A.Hkv, h = uh % A.Hkv, s0 = blockIdx.y * kWarps * per_warp, s1 = min(A.B, s0 + kWarps * per_warp);
+    const int rv = A.D / V, n_vec = 2 * rv;                              // 16-byte vectors of a row, of a K row and its V row
+    const T *kb = static_cast<const T *>(A.k) + u * A.ks[0] + h * A.ks[1], *vb = static_cast<const T *>(A.v) + u * A.vs[0] + h * A.vs[1];
+    const int *ret = A.retained + (int64_t)uh * A.B;
+    if (tid == 0) popular = 0;
+    predecessor_done();
+    for (int j = tid; j < A.E; j += 256) {
+        const int64_t i = (int64_t)uh * A.E + j;
+        const float sim = merge_mode == 1 ? 1.f : match_sim[i];
+        e_slot[j] = match[i];
+        e_tok[j] = evicted[i];
+        e_w[j] = merge_mode == 1 ? 1.f : __expf(sim - 1.f);
+    }
+    __syncthreads();
+    auto finish = [&](int slot, bool is_v, int c0, const uint4 &pivot, const float (&acc)[V], float wsum, int count) {
+        T *dst = (is_v ? static_cast<T *>(A.v_out) + u * A.vos[0] + h * A.vos[1] + (int64_t)slot * A.vos[2]
+                       : static_cast<T *>(A.k_out) + u * A.kos[0] + h * A.kos[1] + (int64_t)slot * A.kos[2]) + c0;
+        if (count == 0) { *reinterpret_cast<uint4 *>(dst) = pivot; return; }   // nothing merged in: the pivot row, bit for bit
+        const float inv = 1.f / (1.f + wsum);
+        float xf[V], o[V];
+        Elem<T>::unpack(pivot, xf);
+#pragma unroll
+        for (int e = 0; e < V; ++e) o[e] = (xf[e] + acc[e]) * inv;
+        Elem<T>::store16(dst, o);
+    };
+    for (int slot = s0 + warp; slot < s1; slot += kWarps) {
+        const int r = ret[slot];
+        int count = 0;
+#pragma unroll 4
+        for (int b = 0; b < A.E; b += 32) {
+            const bool hit = b + lane < A.E && e_slot[b + lane] == slot;
+            const uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit);
+            const int at = count + __popc(hits & lanemask_lt());
+            if (hit && at < kSoloMembers) members[warp][at] = (uint16_t)(b + lane);
+            count += __popc(hits);
+        }
+        __syncwarp();
+        if (count > kSoloMembers) {
+            if (lane == 0) popular = 1;
+        } else {
+            for (int vec = lane; vec < n_vec; vec += 32) {
+                const bool is_v = vec >= rv;
+                const int c0 = (is_v ? vec - rv : vec) * V;
+                const T *src = (is_v ? vb : kb) + c0;
+                const int64_t stride = is_v ? A.vs[2] : A.ks[2];
+                const uint4 pivot = load_raw16(src + (int64_t)r * stride);
+                float acc[V], wsum = 0.f;
+#pragma unroll
+                for (int e = 0; e < V; ++e) acc[e] = 0.f;
+                for (int t0 = 0; t0 < count; t0 += kMergeBatch) {
+                    uint4 x[kMergeBatch];
+#pragma unroll
+                    for (int q = 0; q < kMergeBatch; ++q)                // the batch's row loads, back to back
+                        x[q] = t0 + q < count ? load_raw16(src + (int64_t)e_tok[members[warp][t0 + q]] * stride) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                    for (int q = 0; q < kMergeBatch; ++q)                // fixed order: ascending member index
+                        if (t0 + q < count) {
+                            const float w = e_w[members[warp][t0 + q]];
+                            float xf[V];
+                            Elem<T>::unpack(x[q], xf);
+                            wsum += w;
+#pragma unroll
+                            for (int e = 0; e < V; ++e) acc[e] = fmaf(w, xf[e], acc[e]);
+                        }
+                }
+                finish(slot, is_v, c0, pivot, acc, wsum, count);
+            }
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    if (!popular) return;
+    for (int slot = s0; slot < s1; ++slot) {                             // the popular slots, by all warps
+        int count = 0;
+        for (int b = 0; b < A.E; b += 32) count += __popc(__ballot_sync(0xFFFFFFFFu, b + lane < A.E && e_slot[b + lane] == slot));
+        if (count <= kSoloMembers) continue;                             // (the same for the whole block)
+        const int first = count * warp / kWarps, last = count * (warp + 1) / kWarps;
+        for (int vec0 = 0; vec0 < n_vec; vec0 += 32) {
+            const int vec = vec0 + lane;
+            const bool on = vec < n_vec, is_v = vec >= rv;
+            const int c0 = on ? (is_v ? vec - rv : vec) * V : 0;
+            const T *src = (is_v ? vb : kb) + c0;
+            const int64_t stride = is_v ? A.vs[2] : A.ks[2];
+            float acc[V], wsum = 0.f;
+#pragma unroll
+            for (int e = 0; e < V; ++e) acc[e] = 0.f;
+            int seen = 0;
+            for (int b = 0; b < A.E && seen < last; b += 32) {
+                uint32_t hits = __ballot_sync(0xFFFFFFFFu, b + lane < A.E && e_slot[b + lane] == slot);
+                for (; hits != 0u && seen < last; hits &= hits - 1, ++seen) {
+                    if (seen < first) continue;
+                    const int i = b + __ffs(hits) - 1;
+                    const float w = e_w[i];
+                    float xf[V];
+                    Elem<T>::unpack(load_raw16(src + (int64_t)e_tok[i] * stride), xf);
+                    wsum += w;
+#pragma unroll
+                    for (int e = 0; e < V; ++e) acc[e] = fmaf(w, xf[e], acc[e]);
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < V; ++e) part[warp][lane][e] = acc[e];
+            part[warp][lane][V] = wsum;
+            __syncthreads();
+            if (warp == 0) {
+                for (int w = 1; w < kWarps; ++w) {
+#pragma unroll
+                    for (int e = 0; e < V; ++e) acc[e] += part[w][lane][e];
+                    wsum += part[w][lane][V];
+                }
+                if (on) finish(slot, is_v, c0, load_raw16(src + (int64_t)ret[slot] * stride), acc, wsum, count);
+            }
+            __syncthreads();
+        }
+    }
+}
+
 }  // namespace flowmm

@@ -49,3 +49,36 @@ def test_merge_of_hand_made_matches(E, B, heads, kind):
         assert np.all(np.abs(got[:, last].float().cpu().numpy() - ref) <= 2e-2 + 1e-2 * np.abs(ref))
         if Hkv > n and kind != "dropped":
             assert torch.equal(got[:, :n], got[:, last])
+
+
+@pytest.mark.parametrize("dtype,D", [(F.F32, 64), (F.F32, 128), (F.BF16, 64), (F.BF16, 128)])
+@pytest.mark.parametrize("E,B,heads", [(1, 300, 1), (32, 257, 2), (33, 249, 40), (1023, 248, 1), (1024, 300, 30), (1025, 300, 2)])
+@pytest.mark.parametrize("kind", ["spread", "popular"])
+def test_short_lists(dtype, D, E, B, heads, kind):
+    """Lists up to 1024 non-pivots are merged straight from the matches: one slot or four per warp, slots of up to 64 members and
+    of more, rows of one to two 16-byte vectors per lane."""
+    rng = np.random.default_rng(E + B + D)
+    L = E + B
+    p = O.OracleParams(1, heads, heads, D, L, 1, B)
+    k, v = (rng.standard_normal((1, heads, L, D)).astype(np.float32) for _ in range(2))
+    if dtype == F.BF16:
+        k, v = inputs.round_to_bf16(k), inputs.round_to_bf16(v)
+    ret = np.stack([np.sort(rng.choice(L, B, replace=False)) for _ in range(heads)])[None].astype(np.int32)
+    evi = np.stack([np.setdiff1d(np.arange(L), r) for r in ret[0]])[None].astype(np.int32)
+    match = rng.integers(-1, B, (1, heads, E)).astype(np.int32)
+    if kind == "popular":                                           # a few slots of 64, 65 and many members
+        match[..., : E // 2] = 7
+        match[..., E // 2: E // 2 + 65] = B - 1
+        match[..., E // 2 + 65: E // 2 + 129] = 0
+    sim = np.where(match >= 0, rng.random((1, heads, E)), 0).astype(np.float32)
+    ko, vo = O.merge(p, k, v, ret, evi, match, sim.astype(np.float64))[:2]
+    g = [torch.zeros((1, heads, B, D), dtype=torch.bfloat16 if dtype == F.BF16 else torch.float32, device="cuda") for _ in range(2)]
+    fp = gpu_params(p, dtype)
+    ws = F.alloc_workspace(fp)
+    t = lambda x: torch.from_numpy(x).cuda()
+    F.flowmm_merge(fp, to_dev(k, dtype), to_dev(v, dtype), t(ret), t(evi), t(match), t(sim), g[0], g[1], ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    tol = 1e-2 if dtype == F.BF16 else 1e-5
+    for got, ref in zip(g, (ko, vo)):
+        ref = np.asarray(ref, dtype=np.float64).reshape(1, heads, B, D)
+        assert np.all(np.abs(got.float().cpu().numpy() - ref) <= tol + tol * np.abs(ref))
