@@ -94,7 +94,7 @@ constexpr int64_t kMaxHeadsPerCall = 1 << 22;
 // Where everything lives inside the caller's workspace.  One layout serves every entry point.
 struct Layout {
     size_t status, importance, cross_mass, rho, strategy, retained, evicted, match, match_sim;
-    size_t row_part, cross_part, rn, sort_a, sort_b, mem_tok, mem_w, piece_desc, off, piece_off, part_off, partial, ticket, slot_done;
+    size_t row_part, cross_part, sort_a, sort_b, mem_tok, mem_w, piece_desc, off, piece_off, part_off, partial, ticket, slot_done;
     size_t cand_k, cand_scale, cand_slot, cand_count, rank, tile_mod, negc;
     size_t tokmap;             // [UH, L] (slot, weight) of every token position, for the tensor-core merge
     size_t merge_status;       // status word the merge kernels report to (the workspace's own, or one of the merge scratch)
@@ -177,7 +177,6 @@ Layout make_layout(const flowmm_params &p) {
     y.row_part = take(U * Hq * W * max_chunk1 * 8);
     y.cross_part = take(U * Hq * max_chunk2 * 4);
     y.negc = take(U * Hkv * (size_t)y.gw_pad * 4);
-    y.rn = take(U * Hkv * L * 4);
     layout_merge(y, p, take);
     y.merge_status = y.status;
     y.c_tot = (int)((B + 31) / 32 * 32 + 32);
@@ -554,21 +553,9 @@ flowmm_status run_match(const flowmm_params &p, const Layout &y, const void *k, 
     const int E = p.seq_len - p.n_keep;
     if (E == 0) return FLOWMM_OK;
     if (use_tc(p)) return run_match_tc(p, y, k, importance, mod, retained, evicted, strategy, match, match_sim, ws, st, tokmap, prepared);
-    float *rn = at<float>(ws, y.rn);
-    const int64_t rows = (int64_t)p.n_units * p.n_kv_heads * p.seq_len;
-    const int lanes = p.head_dim / (p.dtype == FLOWMM_BF16 ? 8 : 4);
-    const int64_t threads = rows * lanes;
-    const unsigned blocks = (unsigned)((threads + 255) / 256);
-    if (p.dtype == FLOWMM_BF16)
-        launch(inv_norm_kernel<__nv_bfloat16>, blocks, 256, 0, st, k, rows, p.n_kv_heads, p.seq_len, p.head_dim,
-                                                               p.k_stride[0], p.k_stride[1], p.k_stride[2], rn);
-    else
-        launch(inv_norm_kernel<float>, blocks, 256, 0, st, k, rows, p.n_kv_heads, p.seq_len, p.head_dim, p.k_stride[0],
-                                                       p.k_stride[1], p.k_stride[2], rn);
-    FLOWMM_LAUNCHED("inv_norm");
     MatchArgs a;
     a.k = k; a.importance = importance; a.modality = mod; a.retained = retained; a.evicted = evicted;
-    a.strategy = strategy; a.rn = rn; a.match = match; a.match_sim = match_sim;
+    a.strategy = strategy; a.match = match; a.match_sim = match_sim;
     a.Hkv = p.n_kv_heads; a.D = p.head_dim; a.L = p.seq_len; a.B = p.n_keep; a.E = E;
     a.tau_eff = tau_effective(p);
     for (int i = 0; i < 3; ++i) a.ks[i] = p.k_stride[i];

@@ -14,11 +14,15 @@ constexpr int kSimtThreads = 256;
 struct SimtTiles {
     float a[kDChunk][kPitch];
     float b[kDChunk][kPitch];
+    float norm_a[kTile], norm_b[kTile];      // kNorms: reciprocal norms of the tile's rows (0 for a zero row)
 };
 
 // acc[i][j] = sum_d A[ty*4+i][d] * B[tx*4+j][d] for a 64x64 tile; rowA(r) / rowB(r) give the
 // address of tile row r (nullptr: a row of zeros).  All 256 threads of the CTA take part.
-template <typename T, typename FA, typename FB>
+// Small calls wait for their loads more than they compute: a slice of the head dimension is fetched while the one before it
+// is multiplied, and with kNorms the threads that bring the rows in take their norms on the way (left in sm.norm_a / norm_b
+// at the function's end, behind a barrier).
+template <typename T, bool kNorms = false, typename FA, typename FB>
 __device__ __forceinline__ void simt_tile_dot(SimtTiles &sm, int D, FA rowA, FB rowB, float (&acc)[4][4]) {
     constexpr int V = Elem<T>::kVec;
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
@@ -29,28 +33,33 @@ __device__ __forceinline__ void simt_tile_dot(SimtTiles &sm, int D, FA rowA, FB 
     const int lr = tid >> 2, ld = (tid & 3) * 8;       // this thread loads 8 elements of row lr
     const T *pa = rowA(lr);
     const T *pb = rowB(lr);
+    float va[8 / V][V], vb[8 / V][V], na = 0.f, nb = 0.f;
+    auto fetch = [&](int d0) {
+#pragma unroll
+        for (int half = 0; half < 8 / V; ++half) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) va[half][e] = vb[half][e] = 0.f;
+            if (pa) Elem<T>::load16(pa + d0 + ld + half * V, va[half]);
+            if (pb) Elem<T>::load16(pb + d0 + ld + half * V, vb[half]);
+        }
+    };
+    fetch(0);
     for (int d0 = 0; d0 < D; d0 += kDChunk) {
         __syncthreads();
 #pragma unroll
         for (int half = 0; half < 8 / V; ++half) {
-            float va[V], vb[V];
-            if (pa) Elem<T>::load16(pa + d0 + ld + half * V, va);
-            else {
-#pragma unroll
-                for (int e = 0; e < V; ++e) va[e] = 0.f;
-            }
-            if (pb) Elem<T>::load16(pb + d0 + ld + half * V, vb);
-            else {
-#pragma unroll
-                for (int e = 0; e < V; ++e) vb[e] = 0.f;
-            }
 #pragma unroll
             for (int e = 0; e < V; ++e) {
-                sm.a[ld + half * V + e][lr] = va[e];
-                sm.b[ld + half * V + e][lr] = vb[e];
+                sm.a[ld + half * V + e][lr] = va[half][e];
+                sm.b[ld + half * V + e][lr] = vb[half][e];
+                if (kNorms) {
+                    na = fmaf(va[half][e], va[half][e], na);
+                    nb = fmaf(vb[half][e], vb[half][e], nb);
+                }
             }
         }
         __syncthreads();
+        if (d0 + kDChunk < D) fetch(d0 + kDChunk);
 #pragma unroll 8
         for (int d = 0; d < kDChunk; ++d) {
             const float4 a4 = *reinterpret_cast<const float4 *>(&sm.a[d][ty * 4]);
@@ -62,6 +71,18 @@ __device__ __forceinline__ void simt_tile_dot(SimtTiles &sm, int D, FA rowA, FB 
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
+    }
+    if (kNorms) {                                      // the four threads of a row sit side by side
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+            na += __shfl_xor_sync(0xFFFFFFFFu, na, o);
+            nb += __shfl_xor_sync(0xFFFFFFFFu, nb, o);
+        }
+        if ((tid & 3) == 0) {
+            sm.norm_a[lr] = na > 0.f ? rsqrtf(na) : 0.f;
+            sm.norm_b[lr] = nb > 0.f ? rsqrtf(nb) : 0.f;
+        }
+        __syncthreads();
     }
 }
 
@@ -195,6 +216,12 @@ __global__ void __launch_bounds__(kSimtThreads) score_colsum_simt(const ScoreArg
                 if (r >= GW) return nullptr;
                 return q + (int64_t)(h * A.G + r / A.W) * A.qs[1] + (int64_t)(r % A.W) * A.qs[2];
             };
+            uint8_t mqs[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {                        // (fetched along with the rows)
+                const int r = row0 + ty * 4 + i;
+                mqs[i] = r < GW ? mod[A.L - A.W + (r % A.W)] : 0;
+            }
             float acc[4][4];
             simt_tile_dot<T>(sm, A.D, rowA, rowB, acc);
 #pragma unroll
@@ -203,7 +230,7 @@ __global__ void __launch_bounds__(kSimtThreads) score_colsum_simt(const ScoreArg
                 float cr = 0.f;
                 if (r < GW) {
                     const int pa = A.L - A.W + (r % A.W);
-                    const uint8_t mq = mod[pa];
+                    const uint8_t mq = mqs[i];
                     const float mx = row_max[r], inv = row_inv[r];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -286,36 +313,11 @@ __global__ void full_flow_reduce_kernel(const float *parts, int n_parts, int n, 
     }
 }
 
-// Reciprocal Euclidean norm of every key row (0 for a zero row).  One group of D/kVec lanes per row.
-template <typename T>
-__global__ void inv_norm_kernel(const void *k_, int64_t n_rows, int Hkv, int L, int D, int64_t s0, int64_t s1,
-                                int64_t s2, float *rn) {
-    constexpr int V = Elem<T>::kVec;
-    predecessor_done();
-    const int lanes = D / V;                               // 8, 16 or 32
-    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t row = gid / lanes;
-    const int sub = (int)(gid % lanes);
-    float s = 0.f;
-    if (row < n_rows) {
-        const int64_t u = row / ((int64_t)Hkv * L);
-        const int64_t rem = row % ((int64_t)Hkv * L);
-        const T *p = static_cast<const T *>(k_) + u * s0 + (rem / L) * s1 + (rem % L) * s2 + sub * V;
-        float v[V];
-        Elem<T>::load16(p, v);
-#pragma unroll
-        for (int e = 0; e < V; ++e) s = fmaf(v[e], v[e], s);
-    }
-    for (int o = lanes >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-    if (row < n_rows && sub == 0) rn[row] = s > 0.f ? rsqrtf(s) : 0.f;
-}
-
 struct MatchArgs {
     const void *k;
     const float *importance;      // [U, Hkv, L]
     const uint8_t *modality;      // [U, L]
     const int *retained, *evicted, *strategy;
-    const float *rn;              // [U, Hkv, L] reciprocal key norms
     int *match;
     float *match_sim;
     int Hkv, D, L, B, E;
@@ -335,19 +337,17 @@ __global__ void __launch_bounds__(kSimtThreads) match_simt(const MatchArgs A) {
     const int *ret = A.retained + (int64_t)uh * A.B;
     const int *evi = A.evicted + (int64_t)uh * A.E;
     const float *imp = A.importance + (int64_t)uh * A.L;
-    const float *rn = A.rn + (int64_t)uh * A.L;
     const uint8_t *mod = A.modality + (int64_t)u * A.L;
     const bool intra = A.strategy[u] == 0;
     const int j0 = blockIdx.y * kTile;
 
-    float rne[4], best[4];
+    float best[4];
     int bests[4];
     uint8_t me[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int j = j0 + ty * 4 + i;
         const int e = j < A.E ? evi[j] : -1;
-        rne[i] = e >= 0 ? rn[e] : 0.f;
         me[i] = e >= 0 ? mod[e] : 0;
         best[i] = -INFINITY;
         bests[i] = 0x7FFFFFFF;
@@ -361,20 +361,25 @@ __global__ void __launch_bounds__(kSimtThreads) match_simt(const MatchArgs A) {
             const int s = s0 + lr;
             return s < A.B ? k + (int64_t)ret[s] * A.ks[2] : nullptr;
         };
+        bool adm[4];
+        uint8_t mr[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {                        // (fetched along with the rows)
+            const int s = s0 + tx * 4 + j, r = s < A.B ? ret[s] : -1;
+            adm[j] = r >= 0 && imp[r] <= A.tau_eff;          // a highly sensitive pivot is never a merge target
+            mr[j] = r >= 0 ? mod[r] : 0;
+        }
         float acc[4][4];
-        simt_tile_dot<T>(sm, A.D, rowA, rowB, acc);
+        simt_tile_dot<T, true>(sm, A.D, rowA, rowB, acc);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int s = s0 + tx * 4 + j;
-            if (s >= A.B) continue;
-            const int r = ret[s];
-            if (!(imp[r] <= A.tau_eff)) continue;            // highly sensitive pivot: never a merge target
-            const float rnr = rn[r];
-            const uint8_t mr = mod[r];
+            if (!adm[j]) continue;
+            const float rnr = sm.norm_b[tx * 4 + j];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                if (intra && mr != me[i]) continue;
-                const float uval = acc[i][j] * rne[i] * rnr;
+                if (intra && mr[j] != me[i]) continue;
+                const float uval = acc[i][j] * sm.norm_a[ty * 4 + i] * rnr;
                 if (uval > best[i] || (uval == best[i] && s < bests[i])) { best[i] = uval; bests[i] = s; }
             }
         }
