@@ -400,22 +400,33 @@ flowmm_status run_score(const flowmm_params &p, const Layout &y, const void *q, 
     for (int i = 0; i < 3; ++i) { a.qs[i] = p.q_stride[i]; a.ks[i] = p.k_stride[i]; }
     const int GW = a.G * a.W;
     const int UH = p.n_units * p.n_kv_heads;
-    const dim3 g1(UH, (GW + kTile - 1) / kTile, y.n_chunk1), g2(UH, y.n_chunk2);
-    const size_t dyn = (size_t)3 * GW * sizeof(float);
-    if (p.dtype == FLOWMM_BF16) {
-        launch(score_stats_simt<__nv_bfloat16>, g1, kSimtThreads, 0, st, a);
-        FLOWMM_LAUNCHED("score_stats_simt");
-        launch(score_colsum_simt<__nv_bfloat16>, g2, kSimtThreads, dyn, st, a);
-        FLOWMM_LAUNCHED("score_colsum_simt");
+    const int key_tiles = (p.seq_len + kTile - 1) / kTile;
+    int n_parts = y.n_chunk2;
+    if (GW <= kTile && key_tiles <= kClusterScoreTiles) {    // the logits fit the registers of a cluster
+        const int ctas = key_tiles <= 8 ? key_tiles : (key_tiles + 1) / 2;
+        n_parts = ctas;                                      // (8 parts per head always have room)
+        auto kernel = p.dtype == FLOWMM_BF16 ? (key_tiles <= 8 ? score_cluster_simt<__nv_bfloat16, 1> : score_cluster_simt<__nv_bfloat16, 2>)
+                                             : (key_tiles <= 8 ? score_cluster_simt<float, 1> : score_cluster_simt<float, 2>);
+        launch_cluster(dim3(ctas), kernel, UH * ctas, kSimtThreads, 0, st, a, ctas);
+        FLOWMM_LAUNCHED("score_cluster_simt");
     } else {
-        launch(score_stats_simt<float>, g1, kSimtThreads, 0, st, a);
-        FLOWMM_LAUNCHED("score_stats_simt");
-        launch(score_colsum_simt<float>, g2, kSimtThreads, dyn, st, a);
-        FLOWMM_LAUNCHED("score_colsum_simt");
+        const dim3 g1(UH, (GW + kTile - 1) / kTile, y.n_chunk1), g2(UH, y.n_chunk2);
+        const size_t dyn = (size_t)3 * GW * sizeof(float);
+        if (p.dtype == FLOWMM_BF16) {
+            launch(score_stats_simt<__nv_bfloat16>, g1, kSimtThreads, 0, st, a);
+            FLOWMM_LAUNCHED("score_stats_simt");
+            launch(score_colsum_simt<__nv_bfloat16>, g2, kSimtThreads, dyn, st, a);
+            FLOWMM_LAUNCHED("score_colsum_simt");
+        } else {
+            launch(score_stats_simt<float>, g1, kSimtThreads, 0, st, a);
+            FLOWMM_LAUNCHED("score_stats_simt");
+            launch(score_colsum_simt<float>, g2, kSimtThreads, dyn, st, a);
+            FLOWMM_LAUNCHED("score_colsum_simt");
+        }
     }
-    if (parts_out) { *parts_out = y.n_chunk2; return FLOWMM_OK; }
+    if (parts_out) { *parts_out = n_parts; return FLOWMM_OK; }
     const int n = p.n_units * p.n_q_heads;
-    launch(cross_mass_reduce, (n + 7) / 8, 256, 0, st, a.cross_part, y.n_chunk2, n, cross_mass);
+    launch(cross_mass_reduce, (n + 7) / 8, 256, 0, st, a.cross_part, n_parts, n, cross_mass);
     FLOWMM_LAUNCHED("cross_mass_reduce");
     return FLOWMM_OK;
 }

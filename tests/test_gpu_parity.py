@@ -216,3 +216,11 @@ def test_intra_modal_tiles_of_both_modalities(L, B, vis):
     groups inside the first tile of columns, in a later one, at the end, or with one of the groups empty."""
     _random_case(np.random.default_rng(41), 2, 8, 2, 128, L, 32, B, F.BF16, vis_frac=vis, tau=4.0, tau_mode=O.TAU_REL, theta=0.5,
                  flow_mode=O.FLOW_FORCE_INTRA)
+
+
+@pytest.mark.parametrize("L", [17, 64, 65, 511, 512, 513, 1024, 1025])
+@pytest.mark.parametrize("Hq,Hkv,W,D", [(4, 4, 16, 64), (6, 2, 16, 128), (3, 1, 17, 64)])
+def test_fp32_scoring_by_clusters(L, Hq, Hkv, W, D):
+    """Key tiles of a head shared by one to eight CTAs, one tile or two each, a last tile with few keys, up to 64 proxy rows;
+    beyond that two launches."""
+    _random_case(np.random.default_rng(L + D), 2, Hq, Hkv, D, L, W, max(W, L // 5), F.F32, tau=3.0, tau_mode=O.TAU_REL, theta=0.4)
