@@ -627,8 +627,13 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         const uint32_t smem = mtc::smem_bytes(p.n_keep, a.n_stages);
         if (cudaFuncSetAttribute(mtc::merge_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return FLOWMM_ERR_CUDA;
-        const int grid = a.n_items < tc::sm_count() ? a.n_items : tc::sm_count();
-        launch(mtc::merge_tc_kernel, grid, mtc::kThreads, smem, st, kmap, vmap, a);
+        // ... and, while SMs are left, the steps of such an item on two or four (three steps each, or adding the parts up costs
+        // what the split saves: 5 steps of 32 heads took 12 instead of 10 us; clusters of eight with this much shared memory start late)
+        const int steps = (p.seq_len + mtc::kTile - 1) / mtc::kTile;
+        a.ctas = 1;
+        while (a.per_item == 1 && a.ctas < 4 && 2 * a.ctas * a.n_items <= tc::sm_count() && steps >= 6 * a.ctas) a.ctas *= 2;
+        const int grid = a.ctas > 1 ? a.n_items * a.ctas : a.n_items < tc::sm_count() ? a.n_items : tc::sm_count();
+        launch_cluster(dim3(a.ctas), mtc::merge_tc_kernel, grid, mtc::kThreads, smem, st, kmap, vmap, a);
         FLOWMM_LAUNCHED("merge_tc");
         return FLOWMM_OK;
     }

@@ -17,6 +17,9 @@
 //       1 / (1 + sum of weights), transpose 4 x 4 blocks between lanes and store bf16 rows, while the next head's steps
 //       already run into a second set of sums and (up to 128 slots) a second set of accumulators.
 // When the heads fill at most half of the SMs a CTA takes one head's K or V only, with its own copy of W.
+// When SMs are left over even so, a cluster of two or four CTAs shares the steps: each leaves its part of out^T in fp32 in its
+// shared memory (where W was) and they add the parts up in a fixed order through distributed shared memory, a slice of the
+// slots each: calls of 8 heads of 1471 tokens 42.0 -> 39.8 us, 4 of 2176 47.4 -> 43.0, 4 of 4528 65.6 -> 52.5.
 // Bound by the products: a step of 128 tokens takes the tensor core about 1000 clocks per tensor whatever the slots (the X
 // operand is read MN-major).  With four readers storing two bytes per lane the readout took 9 000 (64 slots) to 30 000
 // clocks (218) per head on top: 8 heads of 1471 tokens, 148 slots 32 -> 18 us, 112 of 2176, 218 slots 47 -> 36 us, 32 of 640,
@@ -53,6 +56,7 @@ struct Args {
     int *status;
     int Hkv, L, B, n_items, n_stages;
     int per_item;                // 2: an item is a head; 1: an item is a head's K (even items) or V (odd items)
+    int ctas;                    // > 1 (per_item == 1): the steps of an item are shared by the CTAs of a cluster
     int64_t kos[3], vos[3];
 };
 
@@ -147,7 +151,9 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     predecessor_done();
-    const int n_chunk = (A.L + kTile - 1) / kTile;
+    const int ctas = A.ctas, rank = ctas > 1 ? (int)(blockIdx.x % (unsigned)ctas) : 0;
+    const int first_item = ctas > 1 ? (int)(blockIdx.x / (unsigned)ctas) : (int)blockIdx.x, item_step = ctas > 1 ? A.n_items : (int)gridDim.x;
+    const int n_steps = (A.L + kTile - 1) / kTile, c_lo = n_steps * rank / ctas, n_chunk = n_steps * (rank + 1) / ctas;   // steps c_lo .. n_chunk - 1
     const int per_item = A.per_item;                             // tensors of an item; the first (only) one:
     auto first_tensor = [&](int item) { return per_item == 2 ? 0 : item & 1; };
     auto head_of = [&](int item) { return per_item == 2 ? item : item >> 1; };
@@ -155,9 +161,9 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     if (warp == 0) {
         bool ok = true;
         int st = 0, phase = 0;
-        for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x) {
+        for (int item = first_item; ok && item < A.n_items; item += item_step) {
             const int u = head_of(item) / A.Hkv, h = head_of(item) % A.Hkv, t0 = first_tensor(item);
-            for (int c = 0; ok && c < n_chunk; ++c)
+            for (int c = c_lo; ok && c < n_chunk; ++c)
                 for (int t = 0; t < per_item; ++t) {             // per step the K tile, then the V tile
                     ok = tc::mbar_wait_warp(bar(kBarEmpty + st), phase ^ 1, abort_flag, A.status);
                     if (!ok) break;
@@ -180,11 +186,11 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
         const uint32_t a_hi = tc::kDescSw128Hi, a_lead = (kPanel >> 4) << 16;            // (and the stride between its panels)
         bool ok = true;
         int st = 0, st_phase = 0, wb = 0, w_phase = 0, it = 0;
-        for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x, ++it) {
+        for (int item = first_item; ok && item < A.n_items; item += item_step, ++it) {
             const int set = it % n_sets, use = it / n_sets;
             ok = tc::mbar_wait_warp(bar(kBarOutEmpty + set), (use & 1) ^ 1, abort_flag, A.status);   // the set's previous head is read out
             tc::tc_fence_after();
-            for (int c = 0; ok && c < n_chunk; ++c) {
+            for (int c = c_lo; ok && c < n_chunk; ++c) {
                 ok = tc::mbar_wait_warp(bar(kBarWFull + wb), w_phase, abort_flag, A.status);
                 const uint32_t w_lo = tc::desc_lo(w0 + wb * wsize);
                 for (int t = 0; ok && t < per_item; ++t) {
@@ -195,7 +201,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                     if (tc::elect_one()) {
 #pragma unroll
                         for (int q = 0; q < 8; ++q)
-                            tc::umma_bf16(d, a_lo + q * 128, a_hi, w_lo + (q >> 2) * (wpanel >> 4) + (q & 3) * 2, tc::kDescSw128Hi, idesc, (c | q) != 0);
+                            tc::umma_bf16(d, a_lo + q * 128, a_hi, w_lo + (q >> 2) * (wpanel >> 4) + (q & 3) * 2, tc::kDescSw128Hi, idesc, c > c_lo || q > 0);
                         tc::umma_commit(bar(kBarEmpty + st));
                         if (t == per_item - 1) tc::umma_commit(bar(kBarWEmpty + wb));
                     }
@@ -217,19 +223,20 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
         // position of this thread's token inside a W panel row: 64 tokens per 128-byte row, 16-byte groups swizzled by row
         const uint32_t tok_off = (uint32_t)(e >> 6) * wpanel + (uint32_t)((e & 7) << 1);
         const int tok_grp = (e & 63) >> 3;
-        int2 first = (int)blockIdx.x < A.n_items && e < A.L ? A.tokmap[(int64_t)head_of(blockIdx.x) * A.L + e] : make_int2(-1, 0);
-        for (int item = blockIdx.x; item < A.n_items; item += gridDim.x, ++it) {
+        const int e0 = c_lo * kTile + e;                             // this thread's first token
+        int2 first = first_item < A.n_items && e0 < A.L ? A.tokmap[(int64_t)head_of(first_item) * A.L + e0] : make_int2(-1, 0);
+        for (int item = first_item; item < A.n_items; item += item_step, ++it) {
             const int2 *map = A.tokmap + (int64_t)head_of(item) * A.L;
             const int set = it % n_sets, use = it / n_sets;
             unsigned *sums = wsum + set * kMaxSlots;
             // the set's sums are zero again once its previous head has been read out
             ok = ok && tc::mbar_wait(bar(kBarOutEmpty + set), (use & 1) ^ 1, abort_flag, A.status);
             int2 nxt = first;
-            for (int c = 0; c < n_chunk; ++c, ++j) {
+            for (int c = c_lo; c < n_chunk; ++c, ++j) {
                 const int2 cur = nxt;
                 const int t_next = (c + 1) * kTile + e;
                 if (c + 1 < n_chunk) nxt = t_next < A.L ? map[t_next] : make_int2(-1, 0);
-                else first = item + (int)gridDim.x < A.n_items && e < A.L ? A.tokmap[(int64_t)head_of(item + gridDim.x) * A.L + e] : make_int2(-1, 0);
+                else first = item + item_step < A.n_items && e0 < A.L ? A.tokmap[(int64_t)head_of(item + item_step) * A.L + e0] : make_int2(-1, 0);
                 const int wb = j & 1;
                 ok = ok && tc::mbar_wait(bar(kBarWEmpty + wb), ((j >> 1) & 1) ^ 1, abort_flag, A.status);
                 const uint32_t w = w0 + wb * wsize;
@@ -256,11 +263,27 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
         const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
         bool ok = true;
         int it = 0;
-        for (int item = blockIdx.x; item < A.n_items; item += gridDim.x, ++it) {
+        for (int item = first_item; item < A.n_items; item += item_step, ++it) {
             const int u = head_of(item) / A.Hkv, h = head_of(item) % A.Hkv;
             const int set = it % n_sets, use = it / n_sets;
             unsigned *sums = wsum + set * kMaxSlots;
             ok = ok && tc::mbar_wait_warp(bar(kBarSumFull + set), use & 1, abort_flag, A.status);
+            if (ctas > 1) {
+                // this CTA's part of the product, slot by slot, over the weight slices (whose products are complete)
+                ok = ok && tc::mbar_wait_warp(bar(kBarOutFull + set), use & 1, abort_flag, A.status);
+                tc::tc_fence_after();
+                if (ok) {
+                    for (int s0 = 32 * t; s0 < N; s0 += 64) {
+                        uint32_t acc[32];
+                        tc::tmem_ld32(trow + set * set_cols + s0, acc);
+                        tc::tmem_ld_wait(acc);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i)
+                            if (s0 + i < N) tc::sts32(w0 + ((uint32_t)(s0 + i) * 128u + (uint32_t)(32 * (warp & 3) + lane)) * 4u, __uint_as_float(acc[i]));
+                    }
+                }
+                break;                                               // (one item per cluster)
+            }
             for (int sl = e; ok && sl < N; sl += 256) {
                 inv_s[sl] = 1.f / (1.f + (float)sums[sl] * (1.f / kSumScale));
                 sums[sl] = 0u;
@@ -287,6 +310,29 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
             reader_sync();                                           // inv_s may be rewritten, the set reused
             tc::mbar_arrive(bar(kBarOutEmpty + set));
         }
+    }
+    if (ctas > 1) {
+        // the parts of all CTAs added up in their order, a slice of the slots per CTA, a slot per warp
+        cluster_sync();
+        const int item = first_item, u = head_of(item) / A.Hkv, h = head_of(item) % A.Hkv, which = first_tensor(item);
+        __nv_bfloat16 *out = static_cast<__nv_bfloat16 *>(which ? A.v_out : A.k_out) +
+                             (which ? u * A.vos[0] + h * A.vos[1] : u * A.kos[0] + h * A.kos[1]) + 4 * lane;
+        const int64_t stride = which ? A.vos[2] : A.kos[2];
+        const uint32_t sums_at = tc::smem_u32(wsum);
+        for (int sl = A.B * rank / ctas + warp; sl < A.B * (rank + 1) / ctas; sl += kThreads / 32) {
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            unsigned total = 0;
+#pragma unroll 4
+            for (int q = 0; q < ctas; ++q) {
+                const uint4 v = ld_cluster_u128(w0 + (uint32_t)sl * 512u + (uint32_t)lane * 16u, q);
+                total += ld_cluster_u32(sums_at + 4u * (uint32_t)sl, q);
+                x.x += __uint_as_float(v.x); x.y += __uint_as_float(v.y); x.z += __uint_as_float(v.z); x.w += __uint_as_float(v.w);
+            }
+            const float inv = 1.f / (1.f + (float)total * (1.f / kSumScale));
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(x.x * inv, x.y * inv), hi = __floats2bfloat162_rn(x.z * inv, x.w * inv);
+            *reinterpret_cast<uint2 *>(out + (int64_t)sl * stride) = make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+        }
+        cluster_sync();                                              // nobody's part goes away while it is read
     }
     tc::tc_fence_before();
     __syncthreads();

@@ -224,3 +224,10 @@ def test_fp32_scoring_by_clusters(L, Hq, Hkv, W, D):
     """Key tiles of a head shared by one to eight CTAs, one tile or two each, a last tile with few keys, up to 64 proxy rows;
     beyond that two launches."""
     _random_case(np.random.default_rng(L + D), 2, Hq, Hkv, D, L, W, max(W, L // 5), F.F32, tau=3.0, tau_mode=O.TAU_REL, theta=0.4)
+
+
+@pytest.mark.parametrize("heads,L,B", [(2, 768, 100), (2, 767, 33), (2, 1536, 240), (2, 1537, 16), (2, 640, 64), (30, 1000, 97), (40, 900, 64)])
+def test_merge_steps_shared_by_clusters(heads, L, B):
+    """The tensor-core merge with few heads: two or four CTAs share the steps of 128 tokens of a head's K or V (from 6 and 12
+    steps on), or one takes them all; slots in uneven slices."""
+    _random_case(np.random.default_rng(L + B), 1, heads, heads, 128, L, 16, B, F.BF16, tau=4.0, tau_mode=O.TAU_REL, theta=0.4)
