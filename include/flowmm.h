@@ -245,8 +245,8 @@ flowmm_status flowmm_recompress(const flowmm_params *p, const void *q_win, const
  *   k      [U, Hkv, L, D] with p->k_stride
  *   cross_mass [U, Hq] f32 out;  rho [U] f32 out (may be NULL);  strategy [U] int32 out
  * Of p, the fields n_units, n_q_heads, n_kv_heads, head_dim, seq_len, dtype, softmax_scale, theta,
- * flow_mode, k_stride and path are used (window, n_keep, tau, q_stride are not).  The work is the
- * scoring step applied to query tiles of 128 rows, each against the keys up to its last row, so it
+ * flow_mode, k_stride and path are used (window, n_keep, tau, q_stride are not).  Every query row
+ * is scored against the keys up to itself, so the call
  * costs O(L^2 D) per head.  Scratch: flowmm_full_flow_workspace_bytes; its first word is the device status.
  */
 flowmm_status flowmm_full_flow_workspace_bytes(const flowmm_params *p, size_t *bytes);
