@@ -10,7 +10,7 @@
 // Bound by the epilogue: Hq L^2 / 2 exponentials per unit, a quarter of them as a polynomial on the FMA pipe, with four
 // warps per scheduler to cover the latencies (half of the issue slots used; TMA and MMA alone take half the time).  The
 // form before launched the statistics once per 128 query rows, with a join of all partial statistics after each: launches
-// of a few hundred items in one to three uneven rounds, 1190 us for 28 layers of 28 heads and 2176 tokens against 693 us.
+// of a few hundred items in one to three uneven rounds, 1190 us for 28 layers of 28 heads and 2176 tokens against 595 us.
 #pragma once
 #include "common.cuh"
 #include "score_tc.cuh"
