@@ -644,8 +644,9 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         // a slot per warp while the blocks fit the SMs together, else four, which share the block's copy of the list
         const int per = slot_blocks <= 4 * tc::sm_count() ? 1 : 4;
         const dim3 grid(UH, (p.n_keep + 8 * per - 1) / (8 * per));
-        if (p.dtype == FLOWMM_BF16) launch(merge_short_kernel<__nv_bfloat16>, grid, 256, 0, st, m, match, evicted, match_sim, p.merge_mode, per);
-        else launch(merge_short_kernel<float>, grid, 256, 0, st, m, match, evicted, match_sim, p.merge_mode, per);
+        auto kernel = p.dtype == FLOWMM_BF16 ? (per == 1 ? merge_short_kernel<__nv_bfloat16, 1> : merge_short_kernel<__nv_bfloat16, 4>)
+                                             : (per == 1 ? merge_short_kernel<float, 1> : merge_short_kernel<float, 4>);
+        launch(kernel, grid, 256, 0, st, m, match, evicted, match_sim, p.merge_mode);
         FLOWMM_LAUNCHED("merge_short");
         return FLOWMM_OK;
     }
