@@ -23,7 +23,7 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
 
 // ---- mbarrier ---------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
 __device__ __forceinline__ void mbar_init_fence() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -116,10 +116,12 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
 }
 
 // Explicit shared-memory accesses by 32-bit shared address (a generic pointer would make the
-// compiler emit generic loads, which take the slower global-memory path through L1).
+// compiler emit generic loads, which take the slower global-memory path through L1).  The reads name memory as clobbered:
+// what they read is written by copies and other warps, and nothing may be moved across them.
 __device__ __forceinline__ float4 lds128(uint32_t addr) {
     float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr)
+                 : "memory");
     return v;
 }
 __device__ __forceinline__ void sts128(uint32_t addr, float a, float b, float c, float d) {
@@ -127,7 +129,7 @@ __device__ __forceinline__ void sts128(uint32_t addr, float a, float b, float c,
 }
 __device__ __forceinline__ float lds32(uint32_t addr) {
     float v;
-    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
     return v;
 }
 __device__ __forceinline__ void sts32(uint32_t addr, float v) {
