@@ -446,7 +446,7 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 for (int t = 0; ok && t < p.tp.n_tiles; ++t, ++k, ++bt) {
                     const int col0 = p.lo + t * kMtCols;
                     const int ncols = min(kMtCols, p.hi - col0);
-                    ok = S::extra_wait(c, bt, A.status) && S::acc_wait(c, k, A.status);
+                    ok = S::acc_extra_wait(c, k, bt, A.status);
                     if (!ok) break;
                     const uint32_t scale4 = c.extra(bt);             // reciprocal norms of this tile's candidates
                     const int n_blocks = (ncols + 15) >> 4;

@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 3) merge_staged_kernel(const MergeAr
                 // the next batch starts before this one is worked on: of this piece, else the next piece's first
                 if (b + 1 < nb) { issue(cur, g, b + 1, j); ++j; }
                 else if (g_nxt < total && nxt.d.z >= 0) { issue(nxt, g_nxt, 0, j); ++j; next_started = true; }
-                ok = tc::mbar_wait(bar0 + (jc & 1) * 8, (jc >> 1) & 1, abort_flag, status);
+                ok = tc::mbar_wait_warp(bar0 + (jc & 1) * 8, (jc >> 1) & 1, abort_flag, status);
                 if (!ok) break;
                 const uint32_t buf = bufs + (jc & 1) * kBufBytes + lane * 16;
                 ++jc;

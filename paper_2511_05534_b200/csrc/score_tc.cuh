@@ -376,7 +376,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
             for (int t = 0; ok && t < n_tiles; ++t, ++bt) {
                 const int ncols = min(S::kCols, A.GW - t * S::kCols);
                 if (!S::takes_part(c, ncols)) continue;
-                ok = S::extra_wait(c, bt, A.status) && S::quad_wait(c, k++, A.status);
+                ok = S::quad_extra_wait(c, k++, bt, A.status);
                 if (!ok) break;
                 const uint32_t negc4 = c.extra(bt);
                 constexpr int kPerC = S::kCols / 64;               // 32-column chunks a warp takes of a full tile

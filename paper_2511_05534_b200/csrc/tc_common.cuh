@@ -84,9 +84,34 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
-// The same for a whole converged warp, which stays together whatever its lanes saw.
+// The same for a whole converged warp: all lanes go on, or all give up.  The vote is the branch's condition (a vote on what the
+// lanes' own waits had returned cost the scoring and matching kernels 1 %.)
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag, int *status_word) {
-    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity, abort_flag, status_word));
+    if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
+    unsigned long long t0 = 0;
+    for (uint32_t spins = 1;; ++spins) {
+        if (__all_sync(0xFFFFFFFFu, mbar_try_wait_for(bar, parity, kWaitSuspendNs))) return true;
+        if ((spins & 15u) != 0) continue;
+        bool give_up = *abort_flag != 0;
+        if ((spins & 1023u) == 0) {
+            const unsigned long long now = global_timer_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > kWaitLimitNs) {
+                *abort_flag = 1;
+                atomicCAS(status_word, 0, kStatusTimeout);
+                give_up = true;
+            }
+        }
+        if (__any_sync(0xFFFFFFFFu, give_up)) return false;
+    }
+}
+
+// Two of them, both looked at before the one vote.
+__device__ __forceinline__ bool mbar_wait_both_warp(uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1, volatile int *abort_flag,
+                                                    int *status_word) {
+    const bool there = mbar_try_wait(bar0, parity0), too = mbar_try_wait(bar1, parity1);
+    if (__all_sync(0xFFFFFFFFu, there && too)) return true;
+    return mbar_wait_warp(bar0, parity0, abort_flag, status_word) && mbar_wait_warp(bar1, parity1, abort_flag, status_word);
 }
 
 // ---- TMA ---------------------------------------------------------------------------------------

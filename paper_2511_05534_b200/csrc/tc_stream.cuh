@@ -84,7 +84,7 @@ struct Skel {
         bool ok;                   // false: shared memory was not 1024-byte aligned; nothing may run
         __device__ __forceinline__ uint32_t bar(int i) const { return bars + 8u * i; }
         // shared address of the per-column constants of the bt-th B tile this CTA streams (valid from the tile's
-        // extra_wait to its release)
+        // acc_extra_wait or quad_extra_wait to its release)
         __device__ __forceinline__ uint32_t extra(int bt) const {
             return base + kSmemExtra + (uint32_t)(bt & (kExtraSlots - 1)) * kExtraBytes;
         }
@@ -267,9 +267,12 @@ struct Skel {
         }
     }
 
-    // Epilogue side.  `k` counts the accumulator tiles this warp's half has consumed.
-    static __device__ __forceinline__ bool acc_wait(const Ctx &c, int k, int *status) {
-        const bool ok = tc::mbar_wait(c.bar(kBarAccFull + c.group), k & 1, c.abort_flag, status);
+    // Epilogue side.  `k` counts the accumulator tiles this warp's half has consumed.  (All waits of the epilogue are the whole
+    // warp's: votes, shuffles and tensor-memory reads follow, which the warp must reach, or give up on, as one.)
+    // Waits for the accumulator and for the per-column constants of the bt-th B tile.
+    static __device__ __forceinline__ bool acc_extra_wait(const Ctx &c, int k, int bt, int *status) {
+        const bool ok = tc::mbar_wait_both_warp(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1,
+                                                c.bar(kBarAccFull + c.group), k & 1, c.abort_flag, status);
         tc::tc_fence_after();
         return ok;
     }
@@ -282,10 +285,6 @@ struct Skel {
         __syncwarp();
         if (c.lane == 0) tc::mbar_arrive(c.bar(kBarAEmpty + (n % AST) * 2 + c.group));
     }
-    // Waits until the per-column constants of the bt-th B tile are in shared memory.
-    static __device__ __forceinline__ bool extra_wait(const Ctx &c, int bt, int *status) {
-        return tc::mbar_wait(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1, c.abort_flag, status);
-    }
     static __device__ __forceinline__ void acc_release(const Ctx &c) {
         tc::tc_fence_before();
         __syncwarp();
@@ -295,7 +294,13 @@ struct Skel {
     // columns, and (then) the wait and the release; `k` counts the tiles it has taken part in.
     static __device__ __forceinline__ bool takes_part(const Ctx &c, int ncols) { return ncols > c.colhalf * (NB / 2); }
     static __device__ __forceinline__ bool quad_wait(const Ctx &c, int k, int *status) {
-        const bool ok = tc::mbar_wait(c.bar(kBarAccFull + 2 * c.group + c.colhalf), k & 1, c.abort_flag, status);
+        const bool ok = tc::mbar_wait_warp(c.bar(kBarAccFull + 2 * c.group + c.colhalf), k & 1, c.abort_flag, status);
+        tc::tc_fence_after();
+        return ok;
+    }
+    static __device__ __forceinline__ bool quad_extra_wait(const Ctx &c, int k, int bt, int *status) {
+        const bool ok = tc::mbar_wait_both_warp(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1,
+                                                c.bar(kBarAccFull + 2 * c.group + c.colhalf), k & 1, c.abort_flag, status);
         tc::tc_fence_after();
         return ok;
     }
@@ -325,7 +330,7 @@ struct Skel {
     // The same for epilogues in which all sixteen warps drain one accumulator at a time (warp = 32 lanes x
     // a quarter of the columns, both halves in turn): explicit half index, `k` = tiles of that half so far.
     static __device__ __forceinline__ bool acc_wait_h(const Ctx &c, int h, int k, int *status) {
-        const bool ok = tc::mbar_wait(c.bar(kBarAccFull + h), k & 1, c.abort_flag, status);
+        const bool ok = tc::mbar_wait_warp(c.bar(kBarAccFull + h), k & 1, c.abort_flag, status);
         tc::tc_fence_after();
         return ok;
     }

@@ -1,5 +1,5 @@
-"""Inline assembly that touches memory says so: without the "memory" clobber the compiler may move other accesses across the
-statement - a read of shared memory ahead of the wait that it depends on, for instance."""
+"""Rules of the device code that no run can show to be kept: what a broken one does depends on the compiler or on a wait that
+runs out at the wrong moment."""
 import os
 import re
 
@@ -18,6 +18,8 @@ def _asm_statements(text):
 
 
 def test_every_statement_that_touches_memory_names_it():
+    """Without the "memory" clobber the compiler may move other accesses across the statement: a read of shared memory ahead of
+    the wait that it depends on, for instance."""
     seen, bad = 0, []
     for name in sorted(os.listdir(CSRC)):
         for line, stmt in _asm_statements(open(os.path.join(CSRC, name)).read()):
@@ -28,3 +30,15 @@ def test_every_statement_that_touches_memory_names_it():
             if '"memory"' not in stmt or "volatile" not in stmt:
                 bad.append("%s:%d" % (name, line))
     assert seen > 30 and not bad, (seen, bad)
+
+
+def test_waits_before_warp_wide_operations_are_the_whole_warps():
+    """A wait of each lane for itself may end differently for the lanes of a warp when it runs out; votes, shuffles and
+    tensor-memory reads would then wait for lanes that have left.  Such waits are for threads that do none of these: the weight
+    builders of the tensor-core merge and the self-test."""
+    per_lane = {}
+    for name in sorted(os.listdir(CSRC)):
+        n = len(re.findall(r"(?<!bool )\bmbar_wait\(", open(os.path.join(CSRC, name)).read()))
+        if n:
+            per_lane[name] = n
+    assert per_lane == {"flowmm_api.cu": 1, "merge_tc.cuh": 2}, per_lane
