@@ -264,6 +264,8 @@ flowmm_status flowmm_full_flow(const flowmm_params *p, const void *q_full, const
  *   out [U, Hq, D]  f32
  * n_q_heads / n_kv_heads must be at most 8; head_dim 64 or 128.  Scratch: flowmm_decode_workspace_bytes
  * (its first word is a device status like the compression workspace's, see flowmm_last_device_status).
+ * Every call starts the status at FLOWMM_OK by itself, so the scratch may hold anything beforehand; only replays of one
+ * captured graph keep an error of an earlier replay until it is read.
  * `path` as in flowmm_params: AUTO runs both contractions on the tensor cores (tcgen05) when dtype is
  * bf16 and head_dim is 128, and SIMT fp32 kernels otherwise; SIMT forces the latter.
  * Same conventions as above (device pointers, caller-owned memory, asynchronous on the stream).

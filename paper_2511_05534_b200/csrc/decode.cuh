@@ -14,7 +14,7 @@ struct DecodeArgs {
     const void *q, *k, *v;       // q [U, Hq, D] dense
     float *part;                 // [UH, n_split, G, D + 2]: unnormalised output, running max (log2), exp-sum
     float *out;                  // [U, Hq, D]
-    int *status;                 // device status word, cleared here
+    int *status;                 // device status word, cleared here (nothing in this kernel reports to it)
     int Hq, Hkv, G, N, n_split, keys_per_split;
     float scale_log2;
     int64_t ks[3], vs[3];

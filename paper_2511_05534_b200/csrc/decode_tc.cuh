@@ -22,6 +22,7 @@
 // other is between its phases.  Every wait is bounded.
 #pragma once
 #include "common.cuh"
+#include "status_word.cuh"
 #include "tc_common.cuh"
 
 namespace flowmm {
@@ -43,13 +44,14 @@ constexpr uint32_t kSmemRed = kSmemP + 4 * kSmallPanel;      // float [4 warps][
 constexpr uint32_t kSmemBar = kSmemRed + 256;
 constexpr int kBarFull = 0, kBarEmpty = kStages, kBarQ = 2 * kStages, kBarS = kBarQ + 1 /* one per score tile */,
               kBarPFull = kBarS + kMaxTiles, kBarPEmpty = kBarPFull + 2, kBarO = kBarPEmpty + 2, kNumBars = kBarO + 1;
-constexpr uint32_t kSmemBytes = kSmemBar + 8 * kNumBars + 16;
+constexpr uint32_t kSmemBytes = kSmemBar + 8 * kNumBars + 16;   // (+ TMEM address, abort flag, status)
 
 struct Args {
     const __nv_bfloat16 *q;     // [U, Hq, 128] dense
     float *part;                // [UH, n_split, G, 130]: unnormalised output, maximum (log2 domain), sum of weights
     float *out;                 // [U, Hq, 128]
-    int *status;
+    int *status;                // the call's status word (status_word.cuh)
+    uint32_t call;
     int Hq, Hkv, G, N, n_split, tiles_per_split;
     float scale_log2;
     int clustered;              // the ranges of a head are one cluster
@@ -85,8 +87,11 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
     const int warp = tc::warp_number(), lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(dtc_smem + kSmemBar + 8 * kNumBars + 4);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(dtc_smem + kSmemBar + 8 * kNumBars);
+    // what the waits report, until the CTA hands it to the call's status word
+    int *cta_status = reinterpret_cast<int *>(dtc_smem + kSmemBar + 8 * kNumBars + 8);
     if ((base & 1023u) != 0) {                      // the swizzled tiles need a 1024-byte aligned base
-        if (threadIdx.x == 0) atomicCAS(A.status, 0, 6);
+        predecessor_done();
+        if (threadIdx.x == 0) status_write(A.status, A.call, 6);
         return;
     }
     auto bar = [&](int i) { return bars + 8u * i; };
@@ -94,6 +99,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
         for (int i = 0; i < kNumBars; ++i)
             tc::mbar_init(bar(i), (i == kBarQ || i == kBarPFull || i == kBarPFull + 1) ? 128 : 1);
         *abort_flag = 0;
+        *cta_status = 0;
         tc::mbar_init_fence();
         tc::tma_prefetch_desc(&kmap);
         tc::tma_prefetch_desc(&vmap);
@@ -104,8 +110,6 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     predecessor_done();
-    // the status word starts at zero (a wait that runs out reports two seconds after this at the earliest)
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *A.status = 0;
 
     const int uh = blockIdx.x, u = uh / A.Hkv, h = uh % A.Hkv, split = blockIdx.y;
     const int tiles_total = (A.N + kTile - 1) / kTile;
@@ -116,7 +120,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
         bool ok = true;
         int st = 0, phase = 0;
         for (int i = 0; ok && i < 2 * nt; ++i) {                     // the K tiles, then the V tiles
-            ok = tc::mbar_wait_warp(bar(kBarEmpty + st), phase ^ 1, abort_flag, A.status);
+            ok = tc::mbar_wait_warp(bar(kBarEmpty + st), phase ^ 1, abort_flag, cta_status);
             if (!ok) break;
             const CUtensorMap *m = i < nt ? &kmap : &vmap;
             const int row = key0 + (i < nt ? i : i - nt) * kTile;
@@ -132,13 +136,15 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
         if (!ok)         // winding down after a timeout: give copies already issued a moment to land
             for (int i = 0; i < kStages; ++i)
                 for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + i), 0) && !tc::mbar_try_wait(bar(kBarFull + i), 1); ++s) {}
+        // the call's status word starts at zero; here, because this warp has nothing left to do (other CTAs may have reported already)
+        if (blockIdx.x == 0 && blockIdx.y == 0 && tc::elect_one()) status_write(A.status, A.call, 0);
     } else if (warp == 1) {
         const uint32_t q_lo = tc::desc_lo(base + kSmemQ), v_lead = (kPanel >> 4) << 16;
-        bool ok = tc::mbar_wait_warp(bar(kBarQ), 0, abort_flag, A.status);
+        bool ok = tc::mbar_wait_warp(bar(kBarQ), 0, abort_flag, cta_status);
         int st = 0, phase = 0;
         auto next = [&]() { if (++st == kStages) { st = 0; phase ^= 1; } };
         for (int t = 0; ok && t < nt; ++t, next()) {
-            ok = tc::mbar_wait_warp(bar(kBarFull + st), phase, abort_flag, A.status);
+            ok = tc::mbar_wait_warp(bar(kBarFull + st), phase, abort_flag, cta_status);
             if (!ok) break;
             tc::tc_fence_after();
             const uint32_t a_lo = tc::desc_lo(base + st * kStageBytes);
@@ -154,8 +160,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
         }
         for (int t = 0; ok && t < nt; ++t, next()) {
             const int pb = t & 1;
-            ok = tc::mbar_wait_warp(bar(kBarFull + st), phase, abort_flag, A.status) &&
-                 tc::mbar_wait_warp(bar(kBarPFull + pb), (t >> 1) & 1, abort_flag, A.status);
+            ok = tc::mbar_wait_warp(bar(kBarFull + st), phase, abort_flag, cta_status) &&
+                 tc::mbar_wait_warp(bar(kBarPFull + pb), (t >> 1) & 1, abort_flag, cta_status);
             if (!ok) break;
             tc::tc_fence_after();
             const uint32_t a_lo = tc::desc_lo(base + st * kStageBytes) | v_lead, p_lo = tc::desc_lo(base + kSmemP + pb * 2 * kSmallPanel);
@@ -192,7 +198,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
 #pragma unroll
         for (int g = 0; g < kMaxHeads; ++g) mx[g] = kNegBig;
         for (int t = 0; t < nt; ++t) {                               // running maxima while the K tiles stream
-            ok = ok && tc::mbar_wait_warp(bar(kBarS + t), 0, abort_flag, A.status);
+            ok = ok && tc::mbar_wait_warp(bar(kBarS + t), 0, abort_flag, cta_status);
             if (!ok) continue;
             tc::tc_fence_after();
             uint32_t r[16];
@@ -220,7 +226,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
         epi_sync();                                                  // red is reused for the sums below
         for (int t = 0; t < nt; ++t) {
             const int pb = t & 1;
-            ok = ok && tc::mbar_wait_warp(bar(kBarPEmpty + pb), ((t >> 1) & 1) ^ 1, abort_flag, A.status);
+            ok = ok && tc::mbar_wait_warp(bar(kBarPEmpty + pb), ((t >> 1) & 1) ^ 1, abort_flag, cta_status);
             if (!ok) continue;
             uint32_t r[16];
             tc::tmem_ld16(trow + kHeads + kHeads * t, r);
@@ -251,7 +257,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
             if (lane == 0) red[(warp & 3) * kMaxHeads + g] = l[g];
         }
         epi_sync();
-        ok = ok && tc::mbar_wait_warp(bar(kBarO), 0, abort_flag, A.status);
+        ok = ok && tc::mbar_wait_warp(bar(kBarO), 0, abort_flag, cta_status);
         tc::tc_fence_after();
         uint32_t r[16] = {};
         if (ok) {
@@ -291,6 +297,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
     __syncthreads();
     tc::tc_fence_after();
     if (warp == 1) tc::tmem_dealloc(tmem, kTmemCols);
+    if (threadIdx.x == 0 && *abort_flag != 0) status_write(A.status, A.call, *cta_status);
     if (A.clustered) {                                               // (also after a wait that ran out: every thread of the cluster comes here)
         __syncwarp();
         cluster_sync();

@@ -6,6 +6,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -1118,6 +1119,15 @@ flowmm_status launch_decode(const DecodeArgs &a, int uh, int n_q, cudaStream_t s
     return FLOWMM_OK;
 }
 
+// Numbers of the calls that clear their own status word (status_word.cuh): consecutive calls differ, and none is a number
+// that memory is likely to hold by itself (0, small integers).
+uint32_t status_call_number() {
+    static std::atomic<uint32_t> n{0};
+    uint32_t call = 0;
+    while (call == 0) call = (n.fetch_add(1, std::memory_order_relaxed) + 1) * 0x9E3779B1u;
+    return call;
+}
+
 flowmm_status launch_decode_tc(const flowmm_decode_params &p, const DecodeArgs &a, int *status, int uh, cudaStream_t st) {
     CUtensorMap kmap, vmap;
     const uint64_t dims[4] = {128, (uint64_t)p.n_keys, (uint64_t)p.n_kv_heads, (uint64_t)p.n_units};
@@ -1133,7 +1143,7 @@ flowmm_status launch_decode_tc(const flowmm_decode_params &p, const DecodeArgs &
                              cudaSharedmemCarveoutMaxShared) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
     dtc::Args t;
-    t.q = static_cast<const __nv_bfloat16 *>(a.q); t.part = a.part; t.out = a.out; t.status = status;
+    t.q = static_cast<const __nv_bfloat16 *>(a.q); t.part = a.part; t.out = a.out; t.status = status; t.call = status_call_number();
     t.Hq = a.Hq; t.Hkv = a.Hkv; t.G = a.G; t.N = a.N; t.n_split = a.n_split; t.tiles_per_split = a.keys_per_split;
     t.scale_log2 = a.scale_log2;
     t.clustered = a.n_split > 1 && a.n_split <= kMaxDecodeCluster;
