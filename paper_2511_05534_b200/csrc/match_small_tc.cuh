@@ -65,6 +65,7 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     volatile int *abort_flag = reinterpret_cast<volatile int *>(mst_smem + kSmemBar + 8 * kNumBars + 4);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(mst_smem + kSmemBar + 8 * kNumBars);
     if ((base & 1023u) != 0) {
+        predecessor_done();
         if (threadIdx.x == 0) atomicCAS(A.status, 0, 6);
         return;
     }

@@ -131,6 +131,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tail + kTailData + 8 * kNumBars + 4);
     const int warp = tc::warp_number(), lane = threadIdx.x & 31;
     if ((base & 1023u) != 0) {
+        predecessor_done();
         if (threadIdx.x == 0) atomicCAS(A.status, 0, 6);
         return;
     }

@@ -79,6 +79,7 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
     volatile int *abort_flag = reinterpret_cast<volatile int *>(sft_smem + kSmemBar + 8 * kNumBars + 4);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sft_smem + kSmemBar + 8 * kNumBars);
     if ((base & 1023u) != 0) {
+        predecessor_done();
         if (threadIdx.x == 0) atomicCAS(A.status, 0, 6);
         return;
     }

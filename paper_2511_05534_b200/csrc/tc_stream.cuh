@@ -114,6 +114,7 @@ struct Skel {
         c.abort_flag = reinterpret_cast<volatile int *>(smem_raw + kSmemBar + 8 * kNumBars + 4);
         c.ok = (c.base & 1023u) == 0;              // the swizzled operand tiles need a 1024-byte aligned base
         if (!c.ok) {
+            predecessor_done();
             if (threadIdx.x == 0) atomicCAS(status, 0, kStatusAlign);
             return c;
         }

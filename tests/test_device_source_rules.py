@@ -42,3 +42,19 @@ def test_waits_before_warp_wide_operations_are_the_whole_warps():
         if n:
             per_lane[name] = n
     assert per_lane == {"flowmm_api.cu": 1, "merge_tc.cuh": 2}, per_lane
+
+
+def test_no_block_leaves_or_reports_before_its_predecessor_is_done():
+    """Kernels are launched as programmatic dependents: a block that returned without waiting would let the kernel after it start
+    before the kernel in front has ended, and a status word may still be the predecessor's."""
+    bad = []
+    for name in sorted(os.listdir(CSRC)):
+        text = open(os.path.join(CSRC, name)).read()
+        for m in re.finditer(r"__global__[^;{]*\{", text):
+            body = text[m.end():]
+            body = body[:re.search(r"\n}", body).start()]
+            wait = min((body.find(w) for w in ("predecessor_done()", "::setup(") if w in body), default=-1)
+            early = re.search(r"\breturn\b|atomicCAS|status_write|atomicAdd", re.sub(r"\[&\][^{]*\{[^}]*\}", lambda l: " " * len(l.group()), body))
+            if wait < 0 or (early and early.start() < wait):
+                bad.append("%s:%d" % (name, text.count("\n", 0, m.start()) + 1))
+    assert not bad, bad
