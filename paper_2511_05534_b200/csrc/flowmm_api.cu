@@ -641,10 +641,11 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
     // Short lists: straight from the matches.  Every slot reads its head's whole list, so beyond 256 entries this is for few
     // slots only (28 units x 4 heads of 1270 tokens, 254 slots: 105 us sorted, 115 so; one of those units: 46 and 40).
     const int64_t slot_blocks = (int64_t)UH * ((p.n_keep + 7) / 8);
-    if (E > 0 && (E <= 256 || (E <= kShortList && slot_blocks <= 2048))) {
-        // a slot per warp while the blocks fit the SMs together, else four, which share the block's copy of the list
-        const int per = slot_blocks <= 4 * tc::sm_count() ? 1 : 4;
-        const dim3 grid(UH, (p.n_keep + 8 * per - 1) / (8 * per));
+    // a slot per warp while the blocks fit the SMs together, else four, which share the block's copy of the list
+    const int per = slot_blocks <= 4 * tc::sm_count() ? 1 : 4, grid_y = (p.n_keep + 8 * per - 1) / (8 * per);
+    // (more slots than a grid has room for: the persistent kernels below take any number)
+    if (E > 0 && grid_y <= 65535 && (E <= 256 || (E <= kShortList && slot_blocks <= 2048))) {
+        const dim3 grid(UH, grid_y);
         auto kernel = p.dtype == FLOWMM_BF16 ? (per == 1 ? merge_short_kernel<__nv_bfloat16, 1> : merge_short_kernel<__nv_bfloat16, 4>)
                                              : (per == 1 ? merge_short_kernel<float, 1> : merge_short_kernel<float, 4>);
         launch(kernel, grid, 256, 0, st, m, match, evicted, match_sim, p.merge_mode);

@@ -82,3 +82,42 @@ def test_short_lists(dtype, D, E, B, heads, kind):
     for got, ref in zip(g, (ko, vo)):
         ref = np.asarray(ref, dtype=np.float64).reshape(1, heads, B, D)
         assert np.all(np.abs(got.float().cpu().numpy() - ref) <= tol + tol * np.abs(ref))
+
+
+@pytest.mark.parametrize("B", [65535 * 32, 65535 * 32 + 1])
+def test_short_list_with_more_slots_than_a_grid_has_rows(B):
+    """256 non-pivots and budgets around two million: the last one that a grid of short-list blocks covers and the first that
+    goes to the persistent kernels.  Pivots without members come back bit for bit; the others as the sum says."""
+    E, D, H = 256, 64, 1
+    L = E + B
+    gen = torch.Generator(device="cuda").manual_seed(B)
+    k, v = (torch.randn((1, H, L, D), device="cuda", generator=gen).bfloat16() for _ in range(2))
+    rng = np.random.default_rng(1)
+    evi = torch.from_numpy(np.sort(rng.choice(L, E, replace=False))).cuda()
+    keep = torch.ones(L, dtype=torch.bool, device="cuda")
+    keep[evi] = False
+    ret = keep.nonzero()[:, 0]
+    match = torch.from_numpy(rng.integers(0, B, E)).cuda()
+    match[0], match[1:70], match[70] = -1, B - 1, 0
+    sim = torch.rand(E, device="cuda", generator=gen)
+    p = O.OracleParams(1, H, H, D, L, 1, B)
+    fp = gpu_params(p, F.BF16)
+    g = [torch.zeros((1, H, B, D), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    ws = F.alloc_workspace(fp)
+    i32 = lambda x: x.to(torch.int32).view(1, H, -1).contiguous()
+    F.flowmm_merge(fp, k, v, i32(ret), i32(evi), i32(match), sim.view(1, H, E), g[0], g[1], ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    slots = match[1:].unique()
+    w = torch.exp(sim.double() - 1)[1:, None]
+    for got, x in zip(g, (k, v)):
+        x = x[0, 0]
+        plain = torch.ones(B, dtype=torch.bool, device="cuda")
+        plain[slots] = False
+        assert torch.equal(got[0, 0][plain], x[ret[plain]])
+        num, den = torch.zeros((B, D), dtype=torch.float64, device="cuda"), torch.ones((B, 1), dtype=torch.float64, device="cuda")
+        num.index_add_(0, match[1:], w * x[evi[1:]].double())
+        den.index_add_(0, match[1:], w)
+        ref = ((num + x[ret].double()) / den)[slots]
+        # the output's rounding to bf16 (8 bits: 2^-8 of the value), and below it fp32 sums of up to 69 members: (69 + 16) 2^-24
+        # of the mean magnitude, which is below 8
+        assert torch.all((got[0, 0][slots].double() - ref).abs() <= ref.abs() * 2 ** -8 + 2 ** -14)
