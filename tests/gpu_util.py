@@ -32,6 +32,26 @@ def run_gpu(p: O.OracleParams, q, k, v, modality, dtype: int, path: int = F.PATH
     return res
 
 
+def small_integers(rng, shape) -> np.ndarray:
+    """Values -3 .. 3: exact in bf16, and sums of up to five million of them exact in fp32."""
+    return rng.integers(-3, 4, shape).astype(np.float32)
+
+
+def merge_reference(p: O.OracleParams, k, v, ret, evi, match, sim, dtype: int):
+    """[(reference, bound of the error)] for K and V of the merge step.  k, v: small_integers.
+    MEAN: the weights are 1 and the sums exact, which leaves the reciprocal, its product and the output's rounding: a member that
+    is lost, counted twice or taken from another slot changes the fp32 result by far more.
+    EXPSIM: fp32 sums in pieces of at most 128 members, then of at most E / 64 pieces, and weights within four units of their last
+    place, all relative to the mean magnitude of what is summed."""
+    refs = O.merge(p, k, v, ret, evi, match, sim)[:2]
+    out_rounding = 2.0 ** -8 if dtype == F.BF16 else 0.0
+    if p.merge_mode == F.MERGE_MEAN:
+        return [(r, np.abs(r) * (out_rounding + 2.0 ** -22)) for r in refs]
+    c = (128 + (p.seq_len - p.n_keep) // 64 + 16) * 2.0 ** -24
+    sizes = O.merge(p, np.abs(k), np.abs(v), ret, evi, match, sim)[:2]
+    return [(r, np.abs(r) * out_rounding + c * m) for r, m in zip(refs, sizes)]
+
+
 def oracle_params(wl, n_units: int, permille: int, **kw) -> O.OracleParams:
     base = dict(theta=wl.theta, tau=wl.tau_rel, tau_mode=O.TAU_REL)
     base.update(kw)
