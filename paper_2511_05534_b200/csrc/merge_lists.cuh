@@ -607,14 +607,17 @@ __global__ void __launch_bounds__(256) merge_pieces_kernel(const MergeArgs A, in
 constexpr int kShortList = 1024, kSoloMembers = 64;
 
 // grid = (UH, slots / (8 * kPer)), 256 threads; a warp takes kPer consecutive slots and finds the members of all of them in one
-// walk over the list (a walk per slot took 69.6 us for a call of 8 heads with 1000 entries and 1500 slots, this 61.9).
+// walk over the list (a walk per slot took 69.6 us for a call of 8 heads with 1000 entries and 1500 slots, this 61.9).  The slots'
+// counts wait in shared memory, and bf16 takes the slots one after the other: in registers and unrolled, 64 registers a thread did not
+// hold them (112 heads of 217 entries and 423 slots 23.3 -> 21.8 us, 448 of 217 and 300 87 -> 79; three blocks per SM with 75
+// registers 24.8 and 99).  fp32, two vectors per lane and row, gains from overlapping the slots (43.6 us, one after the other 47.8).
 template <typename T, int kPer>
 __global__ void __launch_bounds__(256, 4) merge_short_kernel(const MergeArgs A, const int *match, const int *evicted, const float *match_sim,
                                                              int merge_mode) {
     constexpr int V = Elem<T>::kVec, kWarps = 8;
     __shared__ int e_slot[kShortList], e_tok[kShortList];
     __shared__ float e_w[kShortList];
-    __shared__ uint16_t members[kWarps][kPer][kSoloMembers];
+    __shared__ uint16_t members[kWarps][kPer][kSoloMembers], counts[kWarps][kPer];
     __shared__ float part[kWarps][32][V + 1];
     __shared__ int popular;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -659,10 +662,15 @@ __global__ void __launch_bounds__(256, 4) merge_short_kernel(const MergeArgs A, 
             n_members[p] += __popc(hits);
         }
     }
-    __syncwarp();
+    if constexpr (kPer > 1) {
 #pragma unroll
+        for (int p = 0; p < kPer; ++p)
+            if (lane == p) counts[warp][p] = (uint16_t)n_members[p];
+    }
+    __syncwarp();
+#pragma unroll (sizeof(T) == 4 ? kPer : 1)
     for (int p = 0; p < kPer; ++p) {
-        const int slot = mine + p, count = n_members[p];
+        const int slot = mine + p, count = kPer > 1 ? counts[warp][p] : n_members[0];
         if (slot >= s1) break;
         const int r = ret[slot];
         if (count > kSoloMembers) {
