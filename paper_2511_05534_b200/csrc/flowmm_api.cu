@@ -338,7 +338,12 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
     launch(score_stats_tc_kernel<tcs::Big>, grid1, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
     FLOWMM_LAUNCHED("score_stats_tc");
     const int n_negc = UH * a.GWpad;
-    launch(score_combine_kernel, (n_negc + 63) / 64, 256, 0, st, a.row_part, 4 * a.n_chunk, a.GW, a.GWpad, UH, a.negc);
+    // Lanes per row by its parts (us with 1, 2, 4 lanes): 4 parts, 1 310 720 rows 19, 4 lanes 42, 262 144 rows 8, 10, 12, 65 536 rows
+    // 8, 8, 10; 12 parts, 655 360 rows 36, 26, 34, 50 176 rows the same; 16 parts, 65 536 rows 17, 13, 9; 24 and more, a few
+    // thousand rows 9, 8, 7
+    const int n_part = 4 * a.n_chunk, lanes = n_part < 8 ? 1 : n_part < 16 ? 2 : 4;
+    launch(lanes == 1 ? score_combine_kernel<1> : lanes == 2 ? score_combine_kernel<2> : score_combine_kernel<4>, (n_negc + 256 / lanes - 1) / (256 / lanes), 256, 0, st,
+           a.row_part, n_part, a.GW, a.GWpad, UH, a.negc);
     FLOWMM_LAUNCHED("score_combine");
     if (small2) launch(score_colsum_tc_kernel<tcs::Small>, grid2, tcs::kThreads, tcs::Small::kSmemBytes, st, k128, qb, a);
     else if (resident2) launch(score_colsum_tc_kernel<tcs::Resident>, grid2, tcs::kThreads, tcs::Resident::kSmemBytes, st, k128, qb, a);

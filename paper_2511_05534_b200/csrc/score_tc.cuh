@@ -174,22 +174,29 @@ __global__ void pack_modality_kernel(const uint8_t *modality, int L, int n_words
 
 // Row constants for pass 2: negc[r] = -(M_r + log2 Z_r) so that exp2(s + negc) is the softmax
 // probability; padding rows get a constant that makes every probability 0.
-// Four lanes share a row and read its parts together (a thread per row took 17 us for 65 536 rows of 32 parts, this 8).
+// kLanes lanes share a row and read its parts together.
+// Bound by latency while the rows are few and by issue slots when they are many: four lanes of a row of four parts spend more on
+// the row's number, the exchange of maximum and sum, and the logarithm than on its parts.
+template <int kLanes>
 __global__ void score_combine_kernel(const float2 *row_part, int n_part, int GW, int GWpad, int n_uh, float *negc) {
     predecessor_done();
-    const int i = blockIdx.x * (blockDim.x >> 2) + (threadIdx.x >> 2), sub = threadIdx.x & 3;
+    const int i = blockIdx.x * (blockDim.x / kLanes) + threadIdx.x / kLanes, sub = threadIdx.x % kLanes;
     const int uh = i / GWpad, r = i - uh * GWpad;
     const bool on = i < n_uh * GWpad && r < GW;
-    const float2 *part = row_part + ((int64_t)uh * GW + r) * n_part;       
+    const float2 *part = row_part + ((int64_t)uh * GW + r) * n_part;
     float mx = kNegBig, z = 0.f;
-    if (on)
-        for (int c = sub; c < n_part; c += 4) mx = fmaxf(mx, part[c].x);
+    if (on) {
+#pragma unroll 4
+        for (int c = sub; c < n_part; c += kLanes) mx = fmaxf(mx, part[c].x);
+    }
 #pragma unroll
-    for (int o = 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
-    if (on)
-        for (int c = sub; c < n_part; c += 4) z += part[c].y * exp2f(part[c].x - mx);
+    for (int o = kLanes / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
+    if (on) {
+#pragma unroll 4
+        for (int c = sub; c < n_part; c += kLanes) z += part[c].y * exp2f(part[c].x - mx);
+    }
 #pragma unroll
-    for (int o = 2; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
+    for (int o = kLanes / 2; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
     if (sub == 0 && i < n_uh * GWpad) negc[i] = r < GW ? -(mx + log2f(z)) : kNegBig;
 }
 

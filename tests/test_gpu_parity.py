@@ -231,3 +231,20 @@ def test_merge_steps_shared_by_clusters(heads, L, B):
     """The tensor-core merge with few heads: two or four CTAs share the steps of 128 tokens of a head's K or V (from 6 and 12
     steps on), or one takes them all; slots in uneven slices."""
     _random_case(np.random.default_rng(L + B), 1, heads, heads, 128, L, 16, B, F.BF16, tau=4.0, tau_mode=O.TAU_REL, theta=0.4)
+
+
+@pytest.mark.parametrize("L,parts", [(130, 4), (300, 8), (700, 12), (1024, 16), (1025, 20), (2500, 40)])
+@pytest.mark.parametrize("Hq,Hkv,W", [(6, 2, 32), (5, 1, 64)])
+def test_row_constants_of_few_and_many_parts(L, parts, Hq, Hkv, W):
+    """The row constants of the two-pass scoring are joined by one, two or four lanes a row, by the parts a row has (a tile of 256
+    keys gives four); rows that fill their tile and rows that do not.  A part left out would scale a row by far more than the bound:
+    the error of a logit, 128 products summed in fp32 with |q| |k| scale below 30, and 4e-6 of an exponential."""
+    assert parts == 4 * -(-L // 256)
+    rng = np.random.default_rng(L)
+    p = O.OracleParams(1, Hq, Hkv, 128, L, W, L // 4)
+    q, k = (inputs.round_to_bf16(rng.standard_normal(s).astype(np.float32)) for s in ((1, Hq, W, 128), (1, Hkv, L, 128)))
+    m = (rng.random((1, L)) < 0.5).astype(np.uint8)
+    g = run_gpu(p, q, k, k, m, F.BF16)
+    imp, cross, total = O.score(p, q, k, m)
+    assert np.all(np.abs(g["importance"] - imp) <= 2 * (30 * 128 * 2.0 ** -24 + 4e-6) * imp)
+    assert np.allclose(g["rho"], (cross / total).mean(1), rtol=5e-4)
