@@ -671,12 +671,17 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         int n_bits = 1;
         while ((p.n_keep >> n_bits) != 0) ++n_bits;
         // Few heads: a head's list is shared among 2, 4 or 8 CTAs, at least 1024 positions each, as long as every CTA has an
-        // SM (with four per SM 128 heads of 33 792 tokens took 89 instead of 68 us: the scattered writes then set the pace)
+        // SM (with four per SM 128 heads of 33 792 tokens took 89 instead of 68 us: the scattered writes then set the pace) and
+        // the counters fit it (16 heads of 33 000 positions, 3000 slots: 130 us by a CTA each, 35 by four; 5400 slots 168 and 43;
+        // 74 heads by two 131 and 59, 170 and 65).  Counters of which an SM holds one set only leave clusters of four and eight
+        // waiting for a place when they need nearly all SMs: 16 heads of 9000 by eight 28 us, by four 22, 37 heads by four 32, by
+        // two 28.
+        const size_t smem = csr_cluster_smem(p.n_keep);
+        const int sms = tc::sm_count(), room = smem <= 112 * 1024 ? sms : sms * 5 / 6;
         int ctas = 8;
-        while (ctas > 1 && (ctas * UH > tc::sm_count() || E < 1024 * ctas)) ctas >>= 1;
+        while (ctas > 1 && (ctas * UH > (ctas > 2 ? room : sms) || E < 1024 * ctas)) ctas >>= 1;
         const size_t csr_smem = csr_count_smem(E, p.n_keep, long_list ? 32 : 8);
-        if (ctas > 1 && E < 65536 && csr_cluster_smem(p.n_keep) <= 96 * 1024) {
-            const size_t smem = csr_cluster_smem(p.n_keep);
+        if (ctas > 1 && E < 65536 && smem <= 224 * 1024) {
             if (cudaFuncSetAttribute(build_csr_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
             launch_cluster(dim3(ctas), build_csr_cluster_kernel, UH * ctas, 32 * kCsrClusterWarps, smem, st, c, n_bits, ctas);
         } else if (E < 65536 && csr_smem <= 224 * 1024) {
