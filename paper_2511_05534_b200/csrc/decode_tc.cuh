@@ -66,17 +66,10 @@ __device__ __forceinline__ void sts16(uint32_t addr, unsigned short v) {
     asm volatile("st.shared.b16 [%0], %1;" ::"r"(addr), "h"(v) : "memory");
 }
 // The swizzled 128-row tile read as an MN-major operand: a 128-byte row holds 64 consecutive M
-// elements of one K index, eight K indices make a 1024-byte group, the second 64 M elements live
-// `kPanel` bytes further on.  `byte_offset` selects the 16 K indices (rows) of one instruction.
-__device__ __forceinline__ uint64_t smem_desc_sw128_mn(uint32_t tile_base, uint32_t byte_offset) {
-    uint64_t d = 0;
-    d |= (uint64_t)(((tile_base + byte_offset) & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(kPanel >> 4) << 16;                                  // between 64-element M panels
-    d |= (uint64_t)(1024u >> 4) << 32;                                   // between groups of eight K indices
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
+// elements of one K index, eight K indices make a 1024-byte group (the stride of the upper descriptor word), the second
+// 64 M elements live `kPanel` bytes further on (the leading offset, bits 16 up of the lower word).  The 16 K indices (rows)
+// of the next instruction add 2048 bytes.
+constexpr uint32_t kDescMnLead = (kPanel >> 4) << 16;
 constexpr uint32_t kIdescQK = tc::idesc_bf16(kTile, kHeads);
 constexpr uint32_t kIdescPV = tc::idesc_bf16(128, kHeads) | (1u << 15);   // A operand MN-major
 
@@ -139,7 +132,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
         // the call's status word starts at zero; here, because this warp has nothing left to do (other CTAs may have reported already)
         if (blockIdx.x == 0 && blockIdx.y == 0 && tc::elect_one()) status_write(A.status, A.call, 0);
     } else if (warp == 1) {
-        const uint32_t q_lo = tc::desc_lo(base + kSmemQ), v_lead = (kPanel >> 4) << 16;
+        const uint32_t q_lo = tc::desc_lo(base + kSmemQ);
         bool ok = tc::mbar_wait_warp(bar(kBarQ), 0, abort_flag, cta_status);
         int st = 0, phase = 0;
         auto next = [&]() { if (++st == kStages) { st = 0; phase ^= 1; } };
@@ -164,7 +157,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
                  tc::mbar_wait_warp(bar(kBarPFull + pb), (t >> 1) & 1, abort_flag, cta_status);
             if (!ok) break;
             tc::tc_fence_after();
-            const uint32_t a_lo = tc::desc_lo(base + st * kStageBytes) | v_lead, p_lo = tc::desc_lo(base + kSmemP + pb * 2 * kSmallPanel);
+            const uint32_t a_lo = tc::desc_lo(base + st * kStageBytes) | kDescMnLead, p_lo = tc::desc_lo(base + kSmemP + pb * 2 * kSmallPanel);
             if (tc::elect_one()) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j)

@@ -98,82 +98,78 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
 
     // every role walks the heads of the run: tiles [t_lo, t_hi) of head uh, hc heads before it, tile number i of the run
     if (warp == 0) {
-        {
-            bool ok = true;
-            int hc = 0;
-            for (int g = g_lo; ok && g < g_hi; ++hc) {
-                const int uh = (int)A.by_nt.div(g), u = (int)A.by_hkv.div(uh), h = uh - u * A.Hkv, hp = hc % n_bbuf;
-                ok = tc::mbar_wait_warp(bar(kBarBEmpty + hp), ((hc / n_bbuf) & 1) ^ 1, abort_flag, A.status);
+        bool ok = true;
+        int hc = 0;
+        for (int g = g_lo; ok && g < g_hi; ++hc) {
+            const int uh = (int)A.by_nt.div(g), u = (int)A.by_hkv.div(uh), h = uh - u * A.Hkv, hp = hc % n_bbuf;
+            ok = tc::mbar_wait_warp(bar(kBarBEmpty + hp), ((hc / n_bbuf) & 1) ^ 1, abort_flag, A.status);
+            if (!ok) break;
+            const uint32_t bd = base + kSmemB + hp * b_stride, md = base + kSmemMeta + hp * m_stride;
+            if (tc::elect_one()) {
+                tc::mbar_expect_tx(bar(kBarBFull + hp), b_bytes + 8u * (uint32_t)N);
+                tc::tma_load_4d(bd, &cand_map, bar(kBarBFull + hp), 0, 0, uh, 0);
+                tc::tma_load_4d(bd + b_panel, &cand_map, bar(kBarBFull + hp), 64, 0, uh, 0);
+                tc::bulk_load(md, A.cand_scale + (int64_t)uh * N, 4u * (uint32_t)N, bar(kBarBFull + hp));
+                tc::bulk_load(md + slot_off, A.cand_slot + (int64_t)uh * N, 4u * (uint32_t)N, bar(kBarBFull + hp));
+            }
+            __syncwarp();
+            for (const int end = min(g_hi, (uh + 1) * nt); ok && g < end; ++g) {
+                const int i = g - g_lo, t = g - uh * nt, st = i % kStages;
+                ok = tc::mbar_wait_warp(bar(kBarEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag, A.status);
                 if (!ok) break;
-                const uint32_t bd = base + kSmemB + hp * b_stride, md = base + kSmemMeta + hp * m_stride;
+                const uint32_t dst = base + st * kStageBytes;
                 if (tc::elect_one()) {
-                    tc::mbar_expect_tx(bar(kBarBFull + hp), b_bytes + 8u * (uint32_t)N);
-                    tc::tma_load_4d(bd, &cand_map, bar(kBarBFull + hp), 0, 0, uh, 0);
-                    tc::tma_load_4d(bd + b_panel, &cand_map, bar(kBarBFull + hp), 64, 0, uh, 0);
-                    tc::bulk_load(md, A.cand_scale + (int64_t)uh * N, 4u * (uint32_t)N, bar(kBarBFull + hp));
-                    tc::bulk_load(md + slot_off, A.cand_slot + (int64_t)uh * N, 4u * (uint32_t)N, bar(kBarBFull + hp));
+                    tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
+                    tc::tma_load_4d(dst, &k_map, bar(kBarFull + st), 0, t * kTile, h, u);
+                    tc::tma_load_4d(dst + kPanel, &k_map, bar(kBarFull + st), 64, t * kTile, h, u);
                 }
                 __syncwarp();
-                for (const int end = min(g_hi, (uh + 1) * nt); ok && g < end; ++g) {
-                    const int i = g - g_lo, t = g - uh * nt, st = i % kStages;
-                    ok = tc::mbar_wait_warp(bar(kBarEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag, A.status);
-                    if (!ok) break;
-                    const uint32_t dst = base + st * kStageBytes;
-                    if (tc::elect_one()) {
-                        tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
-                        tc::tma_load_4d(dst, &k_map, bar(kBarFull + st), 0, t * kTile, h, u);
-                        tc::tma_load_4d(dst + kPanel, &k_map, bar(kBarFull + st), 64, t * kTile, h, u);
-                    }
-                    __syncwarp();
-                }
-            }
-            if (!ok) {       // winding down after a timeout: give copies already issued a moment to land
-                for (int b = 0; b < kStages; ++b)
-                    for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + b), 0) && !tc::mbar_try_wait(bar(kBarFull + b), 1); ++s) {}
-                for (int b = 0; b < 2; ++b)
-                    for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarBFull + b), 0) && !tc::mbar_try_wait(bar(kBarBFull + b), 1); ++s) {}
             }
         }
+        if (!ok) {       // winding down after a timeout: give copies already issued a moment to land
+            for (int b = 0; b < kStages; ++b)
+                for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + b), 0) && !tc::mbar_try_wait(bar(kBarFull + b), 1); ++s) {}
+            for (int b = 0; b < 2; ++b)
+                for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarBFull + b), 0) && !tc::mbar_try_wait(bar(kBarBFull + b), 1); ++s) {}
+        }
     } else if (warp == 1) {
-        {
-            bool ok = true;
-            int hc = 0;
-            int n_text_next = A.cand_count[2 * A.by_nt.div(g_lo)], n_vis_next = A.cand_count[2 * A.by_nt.div(g_lo) + 1];   // a head ahead
-            for (int g = g_lo; ok && g < g_hi; ++hc) {
-                const int uh = (int)A.by_nt.div(g), hp = hc % n_bbuf;
-                const int n_text = n_text_next, n_vis = n_vis_next;
-                if (uh + 1 < A.n_heads) { n_text_next = A.cand_count[2 * uh + 2]; n_vis_next = A.cand_count[2 * uh + 3]; }
-                const int cols = n_vis > 0 ? ((n_text + 31) & ~31) + n_vis : n_text;         // columns up to the last candidate
-                ok = tc::mbar_wait_warp(bar(kBarBFull + hp), (hc / n_bbuf) & 1, abort_flag, A.status);
-                const uint32_t bd = base + kSmemB + hp * b_stride;
-                for (const int end = min(g_hi, (uh + 1) * nt); ok && g < end; ++g) {
-                    const int i = g - g_lo, st = i % kStages;
-                    ok = tc::mbar_wait_warp(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
-                    const uint32_t a = base + st * kStageBytes;
-                    for (int q = 0; ok && q < units; ++q) {          // unit number k goes to accumulator and team k mod 4
-                        const int k = i * units + q, set = k & (kTeams - 1), n = min(kUnitCols, cols - q * kUnitCols);
-                        ok = tc::mbar_wait_warp(bar(kBarSetFree + set), ((k / kTeams) & 1) ^ 1, abort_flag, A.status);
-                        if (!ok) break;
-                        tc::tc_fence_after();
-                        const uint32_t idesc = tc::idesc_bf16(kTile, (uint32_t)((n + 15) & ~15));
-                        const uint32_t a_lo = tc::desc_lo(a), b_lo = tc::desc_lo(bd + q * (kUnitCols * 128u));
-                        if (tc::elect_one()) {
-                            if (n > 0) {
+        bool ok = true;
+        int hc = 0;
+        int n_text_next = A.cand_count[2 * A.by_nt.div(g_lo)], n_vis_next = A.cand_count[2 * A.by_nt.div(g_lo) + 1];   // a head ahead
+        for (int g = g_lo; ok && g < g_hi; ++hc) {
+            const int uh = (int)A.by_nt.div(g), hp = hc % n_bbuf;
+            const int n_text = n_text_next, n_vis = n_vis_next;
+            if (uh + 1 < A.n_heads) { n_text_next = A.cand_count[2 * uh + 2]; n_vis_next = A.cand_count[2 * uh + 3]; }
+            const int cols = n_vis > 0 ? ((n_text + 31) & ~31) + n_vis : n_text;         // columns up to the last candidate
+            ok = tc::mbar_wait_warp(bar(kBarBFull + hp), (hc / n_bbuf) & 1, abort_flag, A.status);
+            const uint32_t bd = base + kSmemB + hp * b_stride;
+            for (const int end = min(g_hi, (uh + 1) * nt); ok && g < end; ++g) {
+                const int i = g - g_lo, st = i % kStages;
+                ok = tc::mbar_wait_warp(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
+                const uint32_t a = base + st * kStageBytes;
+                for (int q = 0; ok && q < units; ++q) {          // unit number k goes to accumulator and team k mod 4
+                    const int k = i * units + q, set = k & (kTeams - 1), n = min(kUnitCols, cols - q * kUnitCols);
+                    ok = tc::mbar_wait_warp(bar(kBarSetFree + set), ((k / kTeams) & 1) ^ 1, abort_flag, A.status);
+                    if (!ok) break;
+                    tc::tc_fence_after();
+                    const uint32_t idesc = tc::idesc_bf16(kTile, (uint32_t)((n + 15) & ~15));
+                    const uint32_t a_lo = tc::desc_lo(a), b_lo = tc::desc_lo(bd + q * (kUnitCols * 128u));
+                    if (tc::elect_one()) {
+                        if (n > 0) {
 #pragma unroll
-                                for (int j = 0; j < 8; ++j)
-                                    tc::umma_bf16(tmem + kUnitCols * set, a_lo + (j >> 2) * (kPanel >> 4) + (j & 3) * 2, tc::kDescSw128Hi,
-                                                  b_lo + (j >> 2) * (b_panel >> 4) + (j & 3) * 2, tc::kDescSw128Hi, idesc, j > 0);
-                            }
-                            tc::umma_commit(bar(kBarAccFull + set));
+                            for (int j = 0; j < 8; ++j)
+                                tc::umma_bf16(tmem + kUnitCols * set, a_lo + (j >> 2) * (kPanel >> 4) + (j & 3) * 2, tc::kDescSw128Hi,
+                                              b_lo + (j >> 2) * (b_panel >> 4) + (j & 3) * 2, tc::kDescSw128Hi, idesc, j > 0);
                         }
-                        __syncwarp();
+                        tc::umma_commit(bar(kBarAccFull + set));
                     }
-                    if (ok && tc::elect_one()) tc::umma_commit(bar(kBarEmpty + st));
                     __syncwarp();
                 }
-                if (ok && tc::elect_one()) tc::umma_commit(bar(kBarBEmpty + hp));
+                if (ok && tc::elect_one()) tc::umma_commit(bar(kBarEmpty + st));
                 __syncwarp();
             }
+            if (ok && tc::elect_one()) tc::umma_commit(bar(kBarBEmpty + hp));
+            __syncwarp();
         }
     } else {
         const int team = (warp - 2) >> 2, wq = warp & 3;

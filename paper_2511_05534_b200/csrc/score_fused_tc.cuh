@@ -100,71 +100,67 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
     const int nt = (A.L + kTile - 1) / kTile;
 
     if (warp == 0) {
-        {
-            bool ok = true;
-            int i = 0, it = 0;
-            for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x, ++it) {
-                const int u = item / A.Hkv, h = item % A.Hkv, set = it & 1;
-                ok = tc::mbar_wait_warp(bar(kBarQEmpty + set), ((it >> 1) & 1) ^ 1, abort_flag, A.status);
+        bool ok = true;
+        int i = 0, it = 0;
+        for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x, ++it) {
+            const int u = item / A.Hkv, h = item % A.Hkv, set = it & 1;
+            ok = tc::mbar_wait_warp(bar(kBarQEmpty + set), ((it >> 1) & 1) ^ 1, abort_flag, A.status);
+            if (!ok) break;
+            const uint32_t qd = base + kSmemQ + set * kQBytes;
+            if (tc::elect_one()) {
+                tc::mbar_expect_tx(bar(kBarQFull + set), kQBytes);
+                tc::tma_load_4d(qd, &qmap, bar(kBarQFull + set), 0, 0, h * A.G, u);
+                tc::tma_load_4d(qd + kQBytes / 2, &qmap, bar(kBarQFull + set), 64, 0, h * A.G, u);
+            }
+            __syncwarp();
+            for (int t = 0; ok && t < nt; ++t, ++i) {
+                const int st = i % kStages;
+                ok = tc::mbar_wait_warp(bar(kBarEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag, A.status);
                 if (!ok) break;
-                const uint32_t qd = base + kSmemQ + set * kQBytes;
+                const uint32_t dst = base + st * kStageBytes;
                 if (tc::elect_one()) {
-                    tc::mbar_expect_tx(bar(kBarQFull + set), kQBytes);
-                    tc::tma_load_4d(qd, &qmap, bar(kBarQFull + set), 0, 0, h * A.G, u);
-                    tc::tma_load_4d(qd + kQBytes / 2, &qmap, bar(kBarQFull + set), 64, 0, h * A.G, u);
+                    tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
+                    tc::tma_load_4d(dst, &kmap, bar(kBarFull + st), 0, t * kTile, h, u);
+                    tc::tma_load_4d(dst + kPanel, &kmap, bar(kBarFull + st), 64, t * kTile, h, u);
                 }
                 __syncwarp();
-                for (int t = 0; ok && t < nt; ++t, ++i) {
-                    const int st = i % kStages;
-                    ok = tc::mbar_wait_warp(bar(kBarEmpty + st), ((i / kStages) & 1) ^ 1, abort_flag, A.status);
-                    if (!ok) break;
-                    const uint32_t dst = base + st * kStageBytes;
-                    if (tc::elect_one()) {
-                        tc::mbar_expect_tx(bar(kBarFull + st), kStageBytes);
-                        tc::tma_load_4d(dst, &kmap, bar(kBarFull + st), 0, t * kTile, h, u);
-                        tc::tma_load_4d(dst + kPanel, &kmap, bar(kBarFull + st), 64, t * kTile, h, u);
-                    }
-                    __syncwarp();
-                }
-            }
-            if (!ok) {       // winding down after a timeout: give copies already issued a moment to land
-                for (int b = 0; b < kStages; ++b)
-                    for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + b), 0) && !tc::mbar_try_wait(bar(kBarFull + b), 1); ++s) {}
-                for (int b = 0; b < 2; ++b)
-                    for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarQFull + b), 0) && !tc::mbar_try_wait(bar(kBarQFull + b), 1); ++s) {}
             }
         }
+        if (!ok) {       // winding down after a timeout: give copies already issued a moment to land
+            for (int b = 0; b < kStages; ++b)
+                for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarFull + b), 0) && !tc::mbar_try_wait(bar(kBarFull + b), 1); ++s) {}
+            for (int b = 0; b < 2; ++b)
+                for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar(kBarQFull + b), 0) && !tc::mbar_try_wait(bar(kBarQFull + b), 1); ++s) {}
+        }
     } else if (warp == 1) {
-        {
-            constexpr uint32_t idesc = tc::idesc_bf16(kTile, GW);
-            bool ok = true;
-            int i = 0, it = 0;
-            for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x, ++it) {
-                const int set = it & 1, use = it >> 1;
-                ok = tc::mbar_wait_warp(bar(kBarQFull + set), use & 1, abort_flag, A.status) &&
-                     tc::mbar_wait_warp(bar(kBarSetFree + set), (use & 1) ^ 1, abort_flag, A.status);   // the half's previous head is swept
+        constexpr uint32_t idesc = tc::idesc_bf16(kTile, GW);
+        bool ok = true;
+        int i = 0, it = 0;
+        for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x, ++it) {
+            const int set = it & 1, use = it >> 1;
+            ok = tc::mbar_wait_warp(bar(kBarQFull + set), use & 1, abort_flag, A.status) &&
+                 tc::mbar_wait_warp(bar(kBarSetFree + set), (use & 1) ^ 1, abort_flag, A.status);   // the half's previous head is swept
+            tc::tc_fence_after();
+            const uint32_t qd = base + kSmemQ + set * kQBytes;
+            for (int t = 0; ok && t < nt; ++t, ++i) {
+                const int st = i % kStages;
+                ok = tc::mbar_wait_warp(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
+                if (!ok) break;
                 tc::tc_fence_after();
-                const uint32_t qd = base + kSmemQ + set * kQBytes;
-                for (int t = 0; ok && t < nt; ++t, ++i) {
-                    const int st = i % kStages;
-                    ok = tc::mbar_wait_warp(bar(kBarFull + st), (i / kStages) & 1, abort_flag, A.status);
-                    if (!ok) break;
-                    tc::tc_fence_after();
-                    const uint32_t a = base + st * kStageBytes;
-                    const uint32_t a_lo = tc::desc_lo(a), b_lo = tc::desc_lo(qd), d = tmem + 256 * set + GW * t;
-                    if (tc::elect_one()) {
+                const uint32_t a = base + st * kStageBytes;
+                const uint32_t a_lo = tc::desc_lo(a), b_lo = tc::desc_lo(qd), d = tmem + 256 * set + GW * t;
+                if (tc::elect_one()) {
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            tc::umma_bf16(d, a_lo + (j >> 2) * (kPanel >> 4) + (j & 3) * 2, tc::kDescSw128Hi,
-                                          b_lo + (j >> 2) * (kQBytes / 32) + (j & 3) * 2, tc::kDescSw128Hi, idesc, j > 0);
-                        tc::umma_commit(bar(kBarEmpty + st));
-                        tc::umma_commit(bar(kBarS + set * kMaxTiles + t));
-                    }
-                    __syncwarp();
+                    for (int j = 0; j < 8; ++j)
+                        tc::umma_bf16(d, a_lo + (j >> 2) * (kPanel >> 4) + (j & 3) * 2, tc::kDescSw128Hi,
+                                      b_lo + (j >> 2) * (kQBytes / 32) + (j & 3) * 2, tc::kDescSw128Hi, idesc, j > 0);
+                    tc::umma_commit(bar(kBarEmpty + st));
+                    tc::umma_commit(bar(kBarS + set * kMaxTiles + t));
                 }
-                if (ok && tc::elect_one()) tc::umma_commit(bar(kBarQEmpty + set));
                 __syncwarp();
             }
+            if (ok && tc::elect_one()) tc::umma_commit(bar(kBarQEmpty + set));
+            __syncwarp();
         }
     } else {
         // two sweep teams of eight warps: two warps per 32 TMEM lanes, each with half of the proxy rows (HC columns)

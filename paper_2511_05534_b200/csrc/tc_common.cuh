@@ -118,12 +118,6 @@ __device__ __forceinline__ bool mbar_wait_both_warp(uint32_t bar0, uint32_t pari
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *m) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
 }
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *m, uint32_t bar, int c0, int c1, int c2) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1), "r"(c2)
-        : "memory");
-}
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *m, uint32_t bar, int c0, int c1, int c2,
                                             int c3) {
     asm volatile(
@@ -173,17 +167,8 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {  
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, bf16 inputs, fp32 accumulate; one thread issues.
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// The same with descriptors given as their lower words, the upper words being constants of the operand's layout.
+// D[tmem] (+)= A[smem] * B[smem]^T, bf16 inputs, fp32 accumulate; one thread issues.  Descriptors are given as their lower
+// words, the upper words being constants of the operand's layout.
 __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
                                           uint32_t accumulate) {
     asm volatile(
@@ -258,25 +243,15 @@ __device__ __forceinline__ void tmem_ld_wait(uint32_t (&r)[16]) {
                  :
                  : "memory");
 }
-__device__ __forceinline__ void prefetch_l1(const void *p) {
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
 
 // ---- descriptors -------------------------------------------------------------------------------
 // K-major bf16 operand tile in shared memory, rows of 64 elements (128 bytes) with the 128-byte
 // swizzle that a TMA load with CU_TENSOR_MAP_SWIZZLE_128B produces; groups of 8 rows are 1024
-// bytes apart.  The tile base must be 1024-byte aligned; `byte_offset` selects the 32-byte K slice.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t tile_base, uint32_t byte_offset) {
-    uint64_t d = 0;
-    d |= (uint64_t)(((tile_base + byte_offset) & 0x3FFFFu) >> 4);        // start address
-    d |= (uint64_t)0 << 16;                                              // leading byte offset: unused here
-    d |= (uint64_t)(1024u >> 4) << 32;                                   // stride between 8-row groups
-    d |= (uint64_t)1 << 46;                                              // descriptor version of sm_100
-    d |= (uint64_t)2 << 61;                                              // 128-byte swizzle
-    return d;
-}
-constexpr uint32_t kDescSw128Hi = (1024u >> 4) | (1u << 14) | (2u << 29);      // upper word of smem_desc_sw128
-__device__ __forceinline__ uint32_t desc_lo(uint32_t tile_base) { return (tile_base & 0x3FFFFu) >> 4; }   // its lower word
+// bytes apart.  The tile base must be 1024-byte aligned; a K slice of 32 bytes further on adds 2 to the lower word.
+constexpr uint32_t kDescSw128Hi = (1024u >> 4)      // stride between 8-row groups
+                                | (1u << 14)        // descriptor version of sm_100
+                                | (2u << 29);       // 128-byte swizzle
+__device__ __forceinline__ uint32_t desc_lo(uint32_t tile_base) { return (tile_base & 0x3FFFFu) >> 4; }   // start address; no leading byte offset
 // kind::f16 instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, tile M x N.
 __host__ __device__ constexpr uint32_t idesc_bf16(uint32_t M, uint32_t N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((N >> 3) << 17) | ((M >> 4) << 24);

@@ -59,7 +59,7 @@ struct TilePlan {
 template <int NB, int AST, int BST>
 struct Skel {
     static constexpr int kCols = NB;                         // rows of a B tile (UMMA N)
-    static constexpr int kAStages = AST, kBStages = BST;
+    static constexpr int kBStages = BST;
     static constexpr uint32_t kBStage = NB * 128 * 2;
     static constexpr uint32_t kExtraBytes = NB * 4;          // per-column fp32 constants that travel with a B tile
     static constexpr uint32_t kSmemA = 0;                    // [stage][half]
