@@ -16,8 +16,8 @@
 // of the heads each.  With more ranges the CTA writes its record to global memory and decode_combine_kernel joins them, a
 // block per query head.  (One layer of 4 KV heads: 218 keys 12.4 us when the range that finished last joined all of them,
 // found by tickets that a memset had to clear first, 6.2 us as clusters of two.)
-// Roles: warp 0 lane 0 streams K tiles then V tiles through a three-stage TMA ring, warp 1 lane 0 issues
-// the MMAs, warps 2-5 (one thread per key of a tile / per output dim) do the softmax and the output.
+// Roles: warp 0 streams K tiles then V tiles through a three-stage TMA ring, warp 1 issues
+// the MMAs (both run whole and elect a thread at each instruction), warps 2-5 (one thread per key of a tile / per output dim) do the softmax and the output.
 // Two CTAs fit an SM (256 TMEM columns, about 109 KB of shared memory each), so one streams while the
 // other is between its phases.  Every wait is bounded.
 #pragma once

@@ -643,8 +643,12 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         FLOWMM_LAUNCHED("merge_tc");
         return FLOWMM_OK;
     }
-    // Short lists: straight from the matches.  Every slot reads its head's whole list, so beyond 256 entries this is for few
-    // slots only (28 units x 4 heads of 1270 tokens, 254 slots: 105 us sorted, 115 so; one of those units: 46 and 40).
+    // Short lists: straight from the matches.  Every block of slots reads its head's whole list.  Up to 256 entries that is the
+    // faster way at any number of slots (bf16 at head_dim 128, from 512 to 95 000 blocks: 0.4 to 1.03 of the time of the sorted
+    // lists and the staged merge).  Beyond, it is for few slots: members spread evenly take 0.5 to 0.9 of it up to 2400 blocks,
+    // the same at about 8000, 1.1 to 1.3 from 12 000 on (fp32 and head_dim 64, whose sorted lists go through merge_pieces_kernel,
+    // gain up to 33 000).  What sizes do not show: a slot with a quarter of 1000 members takes such a call 1.4 to 2.3 times as
+    // long as sorted while its blocks leave the SMs idle (512 to 2400), a quarter of 400 members 0.8 to 1.4.
     const int64_t slot_blocks = (int64_t)UH * ((p.n_keep + 7) / 8);
     // a slot per warp while the blocks fit the SMs together, else four, which share the block's copy of the list
     const int per = slot_blocks <= 4 * tc::sm_count() ? 1 : 4, grid_y = (p.n_keep + 8 * per - 1) / (8 * per);

@@ -4,10 +4,10 @@
 // Same preparation as match_tc.cuh (admissible pivots gathered into a dense matrix, text group first, visual group from
 // the next multiple of 32, NaN scales where there is no candidate).
 // The 128-token tiles of all heads form one sequence, of which every CTA (one per SM) takes an equal run, so that few long
-// heads spread over all SMs.  Per head of its run: warp 0 lane 0 loads the head's candidate tile, its reciprocal norms and
-// slots (double-buffered by head up to 128 columns) and streams the token tiles through a TMA ring; warp 1 lane 0 issues
+// heads spread over all SMs.  Per head of its run: warp 0 loads the head's candidate tile, its reciprocal norms and
+// slots (double-buffered by head up to 128 columns) and streams the token tiles through a TMA ring; warp 1 issues
 // S = K_tile C^T (tcgen05.mma, M = 128 tokens) in units of up to 128 candidate columns, one unit per tile or two, into four
-// TMEM accumulators; four teams of four warps take the units in turn: a thread owns a token, reads its key row from the A
+// TMEM accumulators (both run whole and elect a thread at each instruction); four teams of four warps take the units in turn: a thread owns a token, reads its key row from the A
 // stage for the norm, walks the blocks of 16 columns that a token of its warp may take, text group then visual group, keeps
 // the running maximum per group of 8 columns and recovers the exact column at the end.  With two units per tile the two
 // teams of a tile meet in shared memory, row by row.

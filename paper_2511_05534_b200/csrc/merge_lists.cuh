@@ -6,8 +6,8 @@ namespace flowmm {
 
 // ---------------------------------------------------------------------------------------------
 // Merge stage.  The match array maps non-pivot j to a slot (or -1).  The members of every slot
-// are needed in a fixed order, so the non-pivot positions j are sorted by slot with a stable
-// LSD radix sort (ascending j inside a slot); slot s then owns entries off[s] .. off[s+1] of the
+// are needed in a fixed order, so the non-pivot positions j are sorted by slot, stably
+// (ascending j inside a slot); slot s then owns entries off[s] .. off[s+1] of the
 // sorted order, for which the kernel writes the member's token position and Eq. 5 weight.
 // Long member lists are cut into pieces of kPiece so that many warps share a popular pivot; one
 // descriptor per piece tells its warp what to do without any search.

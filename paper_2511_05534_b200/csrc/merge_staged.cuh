@@ -10,7 +10,10 @@
 // eight warps fit an SM and each warp keeps up to 9 KB coming.
 // Pieces are drawn from a shared counter four at a time.  With few pieces per warp (kFixed) that leaves warps with four
 // pieces of one popular slot while others have none left to draw, and a draw's round trip shows: then a warp takes every
-// n-th piece (17 500 pieces of 8 heads for 3552 warps: 72 -> 58 us; with evenly spread members 37 -> 41).
+// n-th piece.  Drawn and fixed, us, at 3552 warps, members spread evenly and with a sixth of them in one slot: 1800 pieces 15, 10 and
+// 57, 25; 7200 18, 13 and 61, 33; 17 500 39, 40 and 97, 70; 28 700 30, 31 and 72, 47; 57 500 47, 52 and 92, 68; 201 000 133, 154
+// and 192, 179; 280 000 379, 412 and 487, 582.  The line of six pieces per warp (21 300) lies where even lists begin to lose;
+// popular slots would take it to fifty, but sizes do not tell the two apart.
 #pragma once
 #include "common.cuh"
 #include "merge_lists.cuh"

@@ -10,9 +10,9 @@
 //   C  per key the sum over proxy rows of exp / row sum: the importance (group mean over the G heads).
 // Lanes are keys, so the per-row reductions of A and B cross lanes (shuffles, then shared memory across
 // the warps) once per head; everything else is per thread.  K is read from HBM exactly once.
-// CTAs are persistent (one per SM) and take (unit, KV head) items in turn.  Warp 0 lane 0 streams Q and the
-// K tiles through a five-stage TMA ring and runs ahead of the arithmetic, warp 1 lane 0 issues the MMAs of
-// item i into TMEM half i mod 2, and two teams of eight warps (two warps per 32 TMEM lanes, each with
+// CTAs are persistent (one per SM) and take (unit, KV head) items in turn.  Warp 0 streams Q and the
+// K tiles through a five-stage TMA ring and runs ahead of the arithmetic, warp 1 issues the MMAs of
+// item i into TMEM half i mod 2 (both run whole and elect a thread at each instruction), and two teams of eight warps (two warps per 32 TMEM lanes, each with
 // half of the proxy rows; their partial importances meet in shared memory) take the items alternately, so
 // one head is swept while the next one streams in.
 #pragma once

@@ -1,4 +1,4 @@
-// Skeleton shared by the three tensor-core kernels (window scoring pass 1 and 2, matching).
+// Skeleton shared by four tensor-core kernels (window scoring pass 1 and 2, matching, full-prefill flow).
 //
 // Each CTA is persistent (one per SM) and walks a list of items.  An item is up to two 128-row
 // operand halves A_0, A_1 (loaded once per item) against a stream of operand tiles B_0 .. B_{n-1}

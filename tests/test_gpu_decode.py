@@ -114,8 +114,9 @@ def test_whole_stack_in_the_timed_configuration(name, permille):
 
 @pytest.mark.parametrize("U,Hq,Hkv,N", [(1, 28, 4, 128), (1, 28, 4, 129), (1, 7, 1, 1024), (1, 8, 1, 1025), (1, 6, 2, 1153), (1, 4, 4, 3000),
                                         (1, 8, 1, 15361), (1, 8, 1, 16000), (60, 5, 5, 300), (40, 64, 8, 1000)])
-def test_one_range_cluster_and_tickets(U, Hq, Hkv, N):
-    """Key counts around the switch points of how a head's ranges are joined: one range, a cluster of two to eight, tickets.
+def test_one_range_cluster_and_combine(U, Hq, Hkv, N):
+    """Key counts around the switch points of how a head's ranges are joined: one range, a cluster of two to eight, a launch
+    of its own.
     Called twice on one workspace that starts with garbage."""
     rng = np.random.default_rng(N)
     q = inputs.round_to_bf16(rng.standard_normal((U, Hq, 128)).astype(np.float32))
