@@ -1298,20 +1298,21 @@ extern "C" flowmm_status flowmm_recompress(const flowmm_params *p, const void *q
 
 // ---- bounded-wait self-test ----------------------------------------------------------------------
 namespace {
-// One CTA waits on an mbarrier phase that nothing completes, with the same bounded wait the
-// tensor-core kernels use: after the limit the first waiter records FLOWMM_ERR_TIMEOUT, raises the
-// CTA's abort flag, and every thread returns.
+// One CTA waits on an mbarrier phase that nothing completes, with the same bounded waits the
+// tensor-core kernels use, the first warp lane by lane and the second as a warp: after the limit the
+// first waiter of each records FLOWMM_ERR_TIMEOUT, raises its warp's abort flag, and every thread returns.
 __global__ void wait_timeout_selftest_kernel(int *status) {
     __shared__ __align__(8) unsigned long long bar;
-    __shared__ int abort_flag;
+    __shared__ int abort_flag[2];
     predecessor_done();
     if (threadIdx.x == 0) {
-        abort_flag = 0;
+        abort_flag[0] = abort_flag[1] = 0;
         tc::mbar_init(tc::smem_u32(&bar), 1);
         tc::mbar_init_fence();
     }
     __syncthreads();
-    tc::mbar_wait(tc::smem_u32(&bar), 0, &abort_flag, status);
+    if (threadIdx.x < 32) tc::mbar_wait(tc::smem_u32(&bar), 0, &abort_flag[0], status);
+    else tc::mbar_wait_warp(tc::smem_u32(&bar), 0, &abort_flag[1], status);
 }
 }  // namespace
 
