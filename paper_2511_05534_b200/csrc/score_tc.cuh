@@ -380,11 +380,14 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                 if ((lane & 15) == 0) cross_out[(int64_t)(up ? cur_g : held_g) * (A.n_rt * 8)] = x;
                 held_g = -1;
             };
-            for (int t = 0; ok && t < n_tiles; ++t, ++bt) {
+            // A wait that runs out changes no lane's way through the item (what follows is garbage, in bounds, and reported): the
+            // votes, shuffles and reads of tensor memory stay the whole warp's without a vote on every wait, which took 5 % (320
+            // units of 8 heads, 512 proxy rows, 33 792 tokens 16.65 ms, 17.5 with the vote).  pair_meet tells all lanes.
+            for (int t = 0; t < n_tiles; ++t, ++bt) {
                 const int ncols = min(S::kCols, A.GW - t * S::kCols);
                 if (!S::takes_part(c, ncols)) continue;
-                ok = S::quad_extra_wait(c, k++, bt, A.status);
-                if (!ok) break;
+                ok = ok && S::quad_extra_wait_lanes(c, k, bt, A.status);
+                ++k;
                 const uint32_t negc4 = c.extra(bt);
                 constexpr int kPerC = S::kCols / 64;               // 32-column chunks a warp takes of a full tile
                 const int chunk_hi = min((ncols + 31) >> 5, kPerC * c.colhalf + kPerC);
@@ -447,7 +450,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                 }
                 S::quad_release(c);
             }
-            if (ok && cur_g >= 0) {
+            if (cur_g >= 0) {
                 publish();
                 if (held_g >= 0) {
                     const float tot = warp_sum(held);

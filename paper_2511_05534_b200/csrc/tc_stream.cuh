@@ -84,7 +84,7 @@ struct Skel {
         bool ok;                   // false: shared memory was not 1024-byte aligned; nothing may run
         __device__ __forceinline__ uint32_t bar(int i) const { return bars + 8u * i; }
         // shared address of the per-column constants of the bt-th B tile this CTA streams (valid from the tile's
-        // acc_extra_wait or quad_extra_wait to its release)
+        // acc_extra_wait or quad_extra_wait_lanes to its release)
         __device__ __forceinline__ uint32_t extra(int bt) const {
             return base + kSmemExtra + (uint32_t)(bt & (kExtraSlots - 1)) * kExtraBytes;
         }
@@ -268,8 +268,8 @@ struct Skel {
         }
     }
 
-    // Epilogue side.  `k` counts the accumulator tiles this warp's half has consumed.  (All waits of the epilogue are the whole
-    // warp's: votes, shuffles and tensor-memory reads follow, which the warp must reach, or give up on, as one.)
+    // Epilogue side.  `k` counts the accumulator tiles this warp's half has consumed.  (The waits are the whole warp's: votes,
+    // shuffles and tensor-memory reads follow, which the warp must reach, or give up on, as one.)
     // Waits for the accumulator and for the per-column constants of the bt-th B tile.
     static __device__ __forceinline__ bool acc_extra_wait(const Ctx &c, int k, int bt, int *status) {
         const bool ok = tc::mbar_wait_both_warp(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1,
@@ -299,9 +299,11 @@ struct Skel {
         tc::tc_fence_after();
         return ok;
     }
-    static __device__ __forceinline__ bool quad_extra_wait(const Ctx &c, int k, int bt, int *status) {
-        const bool ok = tc::mbar_wait_both_warp(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1,
-                                                c.bar(kBarAccFull + 2 * c.group + c.colhalf), k & 1, c.abort_flag, status);
+    // Waits for the accumulator and for the per-column constants of the bt-th B tile, lane by lane: only for an epilogue whose lanes
+    // stay in step whatever their waits return, until pair_meet has told all of them.
+    static __device__ __forceinline__ bool quad_extra_wait_lanes(const Ctx &c, int k, int bt, int *status) {
+        const bool ok = tc::mbar_wait(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1, c.abort_flag, status) &&
+                        tc::mbar_wait(c.bar(kBarAccFull + 2 * c.group + c.colhalf), k & 1, c.abort_flag, status);
         tc::tc_fence_after();
         return ok;
     }

@@ -34,14 +34,16 @@ def test_every_statement_that_touches_memory_names_it():
 
 def test_waits_before_warp_wide_operations_are_the_whole_warps():
     """A wait of each lane for itself may end differently for the lanes of a warp when it runs out; votes, shuffles and
-    tensor-memory reads would then wait for lanes that have left.  Such waits are for threads that do none of these: the weight
-    builders of the tensor-core merge and the self-test."""
+    tensor-memory reads would then wait for lanes that have left.  Such waits are for threads that do none of these (the weight
+    builders of the tensor-core merge, the self-test) or whose way does not depend on what the wait returns until they have voted
+    (the second scoring pass)."""
     per_lane = {}
     for name in sorted(os.listdir(CSRC)):
         n = len(re.findall(r"(?<!bool )\bmbar_wait\(", open(os.path.join(CSRC, name)).read()))
         if n:
             per_lane[name] = n
-    assert per_lane == {"flowmm_api.cu": 1, "merge_tc.cuh": 2}, per_lane
+    assert per_lane == {"flowmm_api.cu": 1, "merge_tc.cuh": 2, "tc_stream.cuh": 2}, per_lane
+    assert {name for name in os.listdir(CSRC) if "S::quad_extra_wait_lanes(" in open(os.path.join(CSRC, name)).read()} == {"score_tc.cuh"}
 
 
 def test_no_block_leaves_or_reports_before_its_predecessor_is_done():
