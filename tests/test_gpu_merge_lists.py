@@ -1,6 +1,6 @@
 """Member lists of the gather merge at the edges of their builders: a CTA or a cluster of two, four or eight per head (2048,
 4096, 8192 non-pivots), the counting sort for many heads (short and long lists), odd and even slot counts, budgets too large for the
-clusters (5461 pivots) and those of which an SM holds one CTA (2700), lists that leave shared memory (70 000 non-pivots),
+clusters (5459 pivots) and those of which an SM holds one CTA (2729), lists that leave shared memory (70 000 non-pivots),
 everything dropped, everything in one slot.  The step
 is called on its own with hand-made matches, on values that let one lost or doubled member be seen (test_merge_reference.py)."""
 import numpy as np
@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("E,B,heads", [(1, 241, 2), (31, 242, 2), (2047, 250, 2), (2048, 251, 2), (4096, 241, 2), (8191, 300, 2), (8192, 301, 2),
                                        (9000, 1691, 2), (20000, 2501, 2), (33000, 257, 2), (9000, 2800, 2), (4096, 241, 300), (4097, 300, 300),
-                                       (9000, 2800, 16), (9000, 5500, 2), (70000, 300, 1), (38500, 300, 2)])
+                                       (9000, 2800, 16), (9000, 5459, 2), (9000, 5460, 2), (70000, 300, 1), (38500, 300, 2)])
 @pytest.mark.parametrize("kind", ["spread", "dropped", "one"])
 def test_merge_of_hand_made_matches(E, B, heads, kind):
     rng = np.random.default_rng(E + B)
