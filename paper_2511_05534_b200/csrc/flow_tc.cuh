@@ -135,8 +135,7 @@ flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
                     l = l * carry + add;
                     lc = lc * carry + addc;
                     m = mx;
-                });
-                S::quad_release(c);
+                }, [&]() { S::quad_release(c); });
             }
             // The two column halves of every row meet.  (After a wait that ran out the meeting is still kept: the vote ends the
             // loop for both warps.)

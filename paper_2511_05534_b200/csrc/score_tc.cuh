@@ -145,9 +145,8 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
                             }
                             l[h] = l[h] * tc::ex2(m[h] - mx) + add;
                             m[h] = mx;
-                        });
-                    }
-                    S::acc_release_h(c, h);
+                        }, [&]() { S::acc_release_h(c, h); });
+                    } else S::acc_release_h(c, h);
                 }
             }
             if (!ok) break;

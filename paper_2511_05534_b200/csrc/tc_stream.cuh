@@ -318,15 +318,19 @@ struct Skel {
     }
 
     // Runs f(chunk, values) over this warp's 32-column chunks of the current accumulator: the chunks of
-    // its column half, as far as they lie below n_chunks (the tile's chunk count).
-    template <class F>
-    static __device__ __forceinline__ void for_each_chunk(const Ctx &c, int n_chunks, F &&f) {
+    // its column half, as far as they lie below n_chunks (the tile's chunk count).  done() is called once, as soon as the last
+    // chunk is in registers: the accumulator is handed back before that chunk is worked on (full-prefill flow, 28 units of 28
+    // heads and 2176 tokens: 690 -> 664 us).
+    template <class F, class Done>
+    static __device__ __forceinline__ void for_each_chunk(const Ctx &c, int n_chunks, F &&f, Done &&done) {
         constexpr int kPer = NB / 64;
-        const int hi = min(n_chunks, kPer * c.colhalf + kPer);
-        for (int ch = kPer * c.colhalf; ch < hi; ++ch) {
+        const int lo = kPer * c.colhalf, hi = min(n_chunks, lo + kPer);
+        if (hi <= lo) done();
+        for (int ch = lo; ch < hi; ++ch) {
             uint32_t a[32];
             tc::tmem_ld32(acc_addr(c, ch), a);
             tc::tmem_ld_wait(a);
+            if (ch + 1 >= hi) done();
             f(ch, a);
         }
     }
@@ -342,14 +346,16 @@ struct Skel {
         __syncwarp();
         if (c.lane == 0) tc::mbar_arrive(c.bar(kBarAccEmpty + h));
     }
-    template <class F>
-    static __device__ __forceinline__ void for_each_chunk_q(const Ctx &c, int h, int colq, int n_chunks, F &&f) {
+    template <class F, class Done>
+    static __device__ __forceinline__ void for_each_chunk_q(const Ctx &c, int h, int colq, int n_chunks, F &&f, Done &&done) {
         constexpr int kPer = NB / 128;
-        const int hi = min(n_chunks, kPer * colq + kPer);
-        for (int ch = kPer * colq; ch < hi; ++ch) {
+        const int lo = kPer * colq, hi = min(n_chunks, lo + kPer);
+        if (hi <= lo) done();
+        for (int ch = lo; ch < hi; ++ch) {
             uint32_t a[32];
             tc::tmem_ld32(c.tmem_base + h * NB + ch * 32 + ((uint32_t)(c.quarter * 32) << 16), a);
             tc::tmem_ld_wait(a);
+            if (ch + 1 >= hi) done();
             f(ch, a);
         }
     }
