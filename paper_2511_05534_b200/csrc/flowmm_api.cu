@@ -96,10 +96,10 @@ constexpr int64_t kMaxHeadsPerCall = 1 << 22;
 struct Layout {
     size_t status, importance, cross_mass, rho, strategy, retained, evicted, match, match_sim;
     size_t row_part, cross_part, sort_a, sort_b, mem_tok, mem_w, piece_desc, off, piece_off, part_off, partial, ticket, slot_done;
-    size_t cand_k, cand_scale, cand_slot, cand_count, rank, tile_mod, negc;
+    size_t cand_k, cand_scale, cand_slot, cand_count, rank, tile_mod, row_all;
     size_t tokmap;             // [UH, L] (slot, weight) of every token position, for the tensor-core merge
     size_t merge_status;       // status word the merge kernels report to (the workspace's own, or one of the merge scratch)
-    int tc_n_qt, tc_n_chunk, tc_tiles_per_chunk, gw_pad;
+    int tc_n_qt, tc_n_chunk, tc_tiles_per_chunk;
     size_t total;
     int n_chunk1, chunk1, n_chunk2, chunk2, max_pieces, max_parts, csr_passes, c_tot, n_rt;
 };
@@ -171,13 +171,12 @@ Layout make_layout(const flowmm_params &p) {
             if (cost < best_cost - 1e-9) { best_cost = cost; y.tc_tiles_per_chunk = tpc; }
         }
         y.tc_n_chunk = (key_tiles + y.tc_tiles_per_chunk - 1) / y.tc_tiles_per_chunk;
-        y.gw_pad = (int)((G * W + tcs::Big::kCols - 1) / tcs::Big::kCols * tcs::Big::kCols);
     }
-    const size_t max_chunk1 = (size_t)(y.n_chunk1 > 4 * y.tc_n_chunk ? y.n_chunk1 : 4 * y.tc_n_chunk);
-    const size_t max_chunk2 = (size_t)(y.n_chunk2 > 8 * y.n_rt ? y.n_chunk2 : 8 * y.n_rt);
+    const size_t max_chunk1 = (size_t)(y.n_chunk1 > 2 * y.tc_n_chunk ? y.n_chunk1 : 2 * y.tc_n_chunk);   // records of 8 (SIMT) or 16 bytes
+    const size_t max_chunk2 = (size_t)y.n_chunk2 > W ? (size_t)y.n_chunk2 : W > 8 ? W : 8;
     y.row_part = take(U * Hq * W * max_chunk1 * 8);
     y.cross_part = take(U * Hq * max_chunk2 * 4);
-    y.negc = take(U * Hkv * (size_t)y.gw_pad * 4);
+    y.row_all = take(U * Hq * W * 16);
     layout_merge(y, p, take);
     y.merge_status = y.status;
     y.c_tot = (int)((B + 31) / 32 * 32 + 32);
@@ -294,13 +293,15 @@ bool use_tc_score(const flowmm_params &p) {
     return use_tc(p) && (p.window == 32 || p.window == 64 || p.window == 128) && gw <= 1024;
 }
 
+constexpr int kMaxRowRecords = 16;          // key chunks of the first scoring pass that the second one joins itself
+
 flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *q, const void *k, const uint8_t *mod,
                            float *importance, float *cross_mass, void *ws, cudaStream_t st, int *parts_out) {
     const int UH = p.n_units * p.n_kv_heads, G = p.n_q_heads / p.n_kv_heads, W = p.window;
     ScoreTcArgs a;
-    a.row_part = at<float2>(ws, y.row_part); a.negc = at<float>(ws, y.negc); a.modality = mod;
+    a.row_part = at<float4>(ws, y.row_part); a.modality = mod;
     a.importance = importance; a.cross_part = at<float>(ws, y.cross_part); a.status = at<int>(ws, y.status);
-    a.Hq = p.n_q_heads; a.Hkv = p.n_kv_heads; a.G = G; a.W = W; a.L = p.seq_len; a.GW = G * W; a.GWpad = y.gw_pad;
+    a.Hq = p.n_q_heads; a.Hkv = p.n_kv_heads; a.G = G; a.W = W; a.L = p.seq_len; a.GW = G * W;
     a.n_qt = y.tc_n_qt; a.n_chunk = y.tc_n_chunk; a.tiles_per_chunk = y.tc_tiles_per_chunk; a.n_rt = y.n_rt;
     a.a_heads = G < tcs::kRows / W ? G : tcs::kRows / W;        // one A half holds 128 proxy rows
     // pass 2 streams the keys as the A operand; with up to 256 proxy rows per KV head the shapes with two A stages keep
@@ -337,21 +338,21 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
         return FLOWMM_ERR_CUDA;
     launch(score_stats_tc_kernel<tcs::Big>, grid1, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
     FLOWMM_LAUNCHED("score_stats_tc");
-    const int n_negc = UH * a.GWpad;
-    // Lanes per row by its parts (us with 1, 2, 4 lanes): 4 parts, 1 310 720 rows 19, 4 lanes 42, 262 144 rows 8, 10, 12, 65 536 rows
-    // 8, 8, 10; 12 parts, 655 360 rows 36, 26, 34, 50 176 rows the same; 16 parts, 65 536 rows 17, 13, 9; 24 and more, a few
-    // thousand rows 9, 8, 7
-    const int n_part = 4 * a.n_chunk, lanes = n_part < 8 ? 1 : n_part < 16 ? 2 : 4;
-    launch(lanes == 1 ? score_combine_kernel<1> : lanes == 2 ? score_combine_kernel<2> : score_combine_kernel<4>, (n_negc + 256 / lanes - 1) / (256 / lanes), 256, 0, st,
-           a.row_part, n_part, a.GW, a.GWpad, UH, a.negc);
-    FLOWMM_LAUNCHED("score_combine");
+    a.row_rec = a.row_part; a.n_rec = a.n_chunk;
+    if (a.n_chunk > kMaxRowRecords) {
+        float4 *all = at<float4>(ws, y.row_all);
+        const int n_rows = UH * a.GW;
+        launch(score_combine_kernel<4>, (n_rows + 63) / 64, 256, 0, st, a.row_part, a.n_chunk, n_rows, all);
+        FLOWMM_LAUNCHED("score_combine");
+        a.row_rec = all; a.n_rec = 1;
+    }
     if (small2) launch(score_colsum_tc_kernel<tcs::Small>, grid2, tcs::kThreads, tcs::Small::kSmemBytes, st, k128, qb, a);
     else if (resident2) launch(score_colsum_tc_kernel<tcs::Resident>, grid2, tcs::kThreads, tcs::Resident::kSmemBytes, st, k128, qb, a);
     else launch(score_colsum_tc_kernel<tcs::Big>, grid2, tcs::kThreads, tcs::Big::kSmemBytes, st, k128, qb, a);
     FLOWMM_LAUNCHED("score_colsum_tc");
-    if (parts_out) { *parts_out = a.n_rt * 8; return FLOWMM_OK; }     // the caller reduces the partial masses itself
+    if (parts_out) { *parts_out = W; return FLOWMM_OK; }              // the caller adds the rows' shares up itself
     const int n = p.n_units * p.n_q_heads;
-    launch(cross_mass_reduce, (n + 7) / 8, 256, 0, st, a.cross_part, a.n_rt * 8, n, cross_mass);
+    launch(cross_mass_reduce, (n + 7) / 8, 256, 0, st, a.cross_part, W, n, cross_mass);
     FLOWMM_LAUNCHED("cross_mass_reduce");
     return FLOWMM_OK;
 }

@@ -5,12 +5,12 @@
 // the keys are streamed twice:
 //   pass 1  S = Q_group . K^T with the G*W proxy rows of a KV head as accumulator lanes (two
 //           halves of 128 rows per item) and 256 keys per tile: each thread keeps the running
-//           maximum and exp-sum of its own row (no cross-thread traffic);
+//           maximum and the exp-sums over text and over visual keys of its own row (no
+//           cross-thread traffic), which also give the cross-modal mass;
 //   pass 2  S^T = K . Q_group^T with keys as the lanes (two halves of 128 keys per item) and the
 //           proxy rows as columns: each thread owns one key, recomputes its logits, normalises
 //           them with the per-column constants of pass 1 and sums along its row, which is
-//           exactly the key's importance; the same probabilities, split by the modality of key
-//           and proxy token, give the cross-modal mass.
+//           exactly the key's importance.
 // Both passes run on tcgen05 with TMA-fed operands; logits never leave TMEM / registers.
 #pragma once
 #include "common.cuh"
@@ -19,13 +19,14 @@
 namespace flowmm {
 
 struct ScoreTcArgs {
-    float2 *row_part;            // [UH*GW, 4*n_chunk] (max, sum) per proxy row, key chunk and column quarter, log2 domain
-    float *negc;                 // [UH, GWpad] -(row max + log2 row sum); very negative for padding rows
+    float4 *row_part;            // [UH*GW, n_chunk] (max, exp-sum over text keys, exp-sum over visual keys, -) per proxy row and key chunk, log2 domain
+    const float4 *row_rec;       // [UH*GW, n_rec] what pass 2 reads: row_part itself, or its records joined to one per row
+    int n_rec;
     const uint8_t *modality;     // [U, L]
     float *importance;           // [UH, L]
-    float *cross_part;           // [U*Hq, n_rt * 8] partial cross-modal mass per key tile and epilogue warp
+    float *cross_part;           // [U*Hq, W] share of a proxy row's mass that falls on keys of the other modality
     int *status;
-    int Hq, Hkv, G, W, L, GW, GWpad;
+    int Hq, Hkv, G, W, L, GW;
     int n_qt;                    // 256-row tiles over the G*W proxy rows
     int n_chunk, tiles_per_chunk;   // pass 1: key chunks per row tile, 256-key tiles per chunk
     FastDiv by_grid2, by_hkv, by_rt;   // exact divisions by the second pass's grid, Hkv, n_rt
@@ -36,8 +37,10 @@ struct ScoreTcArgs {
 };
 
 // max of 32 values with three-input maxima
-__device__ __forceinline__ float max32(const float (&v)[32]) {
-    float m12[12];
+__device__ __forceinline__ float max32(const uint32_t (&a)[32]) {
+    float v[32], m12[12];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(a[i]);
 #pragma unroll
     for (int i = 0; i < 10; ++i) m12[i] = tc::max3(v[3 * i], v[3 * i + 1], v[3 * i + 2]);
     m12[10] = v[30]; m12[11] = v[31];
@@ -46,27 +49,127 @@ __device__ __forceinline__ float max32(const float (&v)[32]) {
     return fmaxf(tc::max3(a0, a1, a2), a3);
 }
 
-// Sum of 2^(raw * scale - mx) over 32 accumulator columns; every fourth exponential on the FMA pipe, two at a time.
-__device__ __forceinline__ float exp_sum32(const float (&raw)[32], float scale_log2, float mx) {
+__device__ __forceinline__ float2 pair_of(const uint32_t (&a)[32], int j) { return make_float2(__uint_as_float(a[j]), __uint_as_float(a[j + 1])); }
+// Sum of 2^(a * scale - mx) over 32 accumulator columns; every fourth exponential on the FMA pipe, two at a time.
+__device__ __forceinline__ float exp_sum32(const uint32_t (&a)[32], float scale_log2, float mx) {
     const float2 neg2 = make_float2(-mx, -mx), sc2 = make_float2(scale_log2, scale_log2);
     float2 a01 = make_float2(0.f, 0.f), a23 = make_float2(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < 32; j += 8) {
-        const float2 x01 = tc::ffma2(make_float2(raw[j], raw[j + 1]), sc2, neg2);
-        const float2 x23 = tc::ffma2(make_float2(raw[j + 2], raw[j + 3]), sc2, neg2);
-        const float2 x45 = tc::ffma2(make_float2(raw[j + 4], raw[j + 5]), sc2, neg2);
-        const float2 x67 = tc::ffma2(make_float2(raw[j + 6], raw[j + 7]), sc2, neg2);
-        const float2 pf = tc::ex2_fma2(make_float2(x23.y, x67.y));
+        const float2 x01 = tc::ffma2(pair_of(a, j), sc2, neg2), x23 = tc::ffma2(pair_of(a, j + 2), sc2, neg2);
+        const float2 x45 = tc::ffma2(pair_of(a, j + 4), sc2, neg2), x67 = tc::ffma2(pair_of(a, j + 6), sc2, neg2);
+        const float2 pf = tc::ex2_fma2(x67);
         a01 = tc::fadd2(a01, make_float2(tc::ex2(x01.x), tc::ex2(x01.y)));
-        a23 = tc::fadd2(a23, make_float2(tc::ex2(x23.x), pf.x));
+        a23 = tc::fadd2(a23, make_float2(tc::ex2(x23.x), tc::ex2(x23.y)));
         a01 = tc::fadd2(a01, make_float2(tc::ex2(x45.x), tc::ex2(x45.y)));
-        a23 = tc::fadd2(a23, make_float2(tc::ex2(x67.x), pf.y));
+        a23 = tc::fadd2(a23, pf);
     }
     return (a01.x + a01.y) + (a23.x + a23.y);
 }
 
+// The exponentials of the scoring and flow epilogues, written out in PTX so that they cost what they must and no more: 32
+// accumulator columns become probabilities in place, multiply-adds as packed pairs, every fourth exponential (two of each
+// eight, neighbours) on the FMA pipe instead of the exp2 unit, which sets these steps' pace.
+#define FLOWMM_EX_FMA(i, j, ADD)                                                           \
+    "mov.b64 x0, {%" #i ", %" #j "};\n\t"                                                  \
+    "fma.rn.f32x2 x0, x0, sc, " ADD ";\n\t"                                                \
+    "mov.b64 {%" #i ", %" #j "}, x0;\n\t"
+#define FLOWMM_EX_E(i) "ex2.approx.ftz.f32 %" #i ", %" #i ";\n\t"
+// 2^x for the pair on the FMA pipe: x clamped at -125, n = round(x) by the 1.5 * 2^23 trick, 2^f on f = x - n in [-0.5, 0.5]
+// by a degree-4 polynomial (own least-squares fit at Chebyshev nodes with the constant fixed at 1: relative error 3.6e-6), n
+// added to the exponent field.
+#define FLOWMM_EX_POLY(i, j)                                                          \
+    "max.f32 %" #i ", %" #i ", 0fC2FA0000;\n\t"                                        \
+    "max.f32 %" #j ", %" #j ", 0fC2FA0000;\n\t"                                        \
+    "mov.b64 x0, {%" #i ", %" #j "};\n\t"                                              \
+    "add.rn.f32x2 x1, x0, kmg;\n\t"          /* t = x + 1.5 * 2^23 */                  \
+    "mov.b64 {f0, f1}, x1;\n\t"                                                       \
+    "sub.rn.f32x2 x1, x1, kmg;\n\t"          /* n */                                   \
+    "sub.rn.f32x2 x0, x0, x1;\n\t"           /* f */                                   \
+    "fma.rn.f32x2 x1, kc4, x0, kc3;\n\t"                                              \
+    "fma.rn.f32x2 x1, x1, x0, kc2;\n\t"                                               \
+    "fma.rn.f32x2 x1, x1, x0, kc1;\n\t"                                               \
+    "fma.rn.f32x2 x1, x1, x0, kone;\n\t"                                              \
+    "mov.b64 {%" #i ", %" #j "}, x1;\n\t"                                              \
+    "mad.lo.s32 %" #i ", f0, 8388608, %" #i ";\n\t"                                    \
+    "mad.lo.s32 %" #j ", f1, 8388608, %" #j ";\n\t"
+#define FLOWMM_EX_DECL                                                                 \
+    ".reg .b64 x0, x1, sc, kmg, kc1, kc2, kc3, kc4, kone;\n\t"                          \
+    ".reg .b32 f0, f1;\n\t"                                                           \
+    "mov.b64 kmg, 0x4B4000004B400000;\n\t"      /* 12582912.0f twice */                \
+    "mov.b64 kone, 0x3F8000003F800000;\n\t"                                           \
+    "mov.b64 kc1, 0x3F3170613F317061;\n\t"      /* 0.69312102 */                       \
+    "mov.b64 kc2, 0x3E75FCD43E75FCD4;\n\t"      /* 0.24022228 */                       \
+    "mov.b64 kc3, 0x3D650E813D650E81;\n\t"      /* 0.05592204 */                       \
+    "mov.b64 kc4, 0x3C1E78073C1E7807;\n\t"      /* 0.00967217 */
+#define FLOWMM_EX_ALL                                                                                                             \
+    FLOWMM_EX_E(0) FLOWMM_EX_E(1) FLOWMM_EX_E(2) FLOWMM_EX_E(3) FLOWMM_EX_E(4) FLOWMM_EX_E(5) FLOWMM_EX_POLY(6, 7)                  \
+    FLOWMM_EX_E(8) FLOWMM_EX_E(9) FLOWMM_EX_E(10) FLOWMM_EX_E(11) FLOWMM_EX_E(12) FLOWMM_EX_E(13) FLOWMM_EX_POLY(14, 15)            \
+    FLOWMM_EX_E(16) FLOWMM_EX_E(17) FLOWMM_EX_E(18) FLOWMM_EX_E(19) FLOWMM_EX_E(20) FLOWMM_EX_E(21) FLOWMM_EX_POLY(22, 23)          \
+    FLOWMM_EX_E(24) FLOWMM_EX_E(25) FLOWMM_EX_E(26) FLOWMM_EX_E(27) FLOWMM_EX_E(28) FLOWMM_EX_E(29) FLOWMM_EX_POLY(30, 31)
+#define FLOWMM_EX_REGS(a)                                                                                                          \
+    "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]), "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), \
+        "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15]), "+r"(a[16]), "+r"(a[17]), "+r"(a[18]), "+r"(a[19]), "+r"(a[20]), \
+        "+r"(a[21]), "+r"(a[22]), "+r"(a[23]), "+r"(a[24]), "+r"(a[25]), "+r"(a[26]), "+r"(a[27]), "+r"(a[28]), "+r"(a[29]), "+r"(a[30]), \
+        "+r"(a[31])
+
+// a = 2^(a * scale - mx), in place (all 32 with the same mx)
+__device__ __forceinline__ void exp2_32(uint32_t (&a)[32], float scale_log2, float mx) {
+    asm volatile(
+        "{\n\t" FLOWMM_EX_DECL ".reg .b64 ng;\n\t"
+        "mov.b64 sc, {%32, %32};\n\t"
+        "mov.b64 ng, {%33, %33};\n\t"
+        FLOWMM_EX_FMA(0, 1, "ng") FLOWMM_EX_FMA(2, 3, "ng") FLOWMM_EX_FMA(4, 5, "ng") FLOWMM_EX_FMA(6, 7, "ng")
+        FLOWMM_EX_FMA(8, 9, "ng") FLOWMM_EX_FMA(10, 11, "ng") FLOWMM_EX_FMA(12, 13, "ng") FLOWMM_EX_FMA(14, 15, "ng")
+        FLOWMM_EX_FMA(16, 17, "ng") FLOWMM_EX_FMA(18, 19, "ng") FLOWMM_EX_FMA(20, 21, "ng") FLOWMM_EX_FMA(22, 23, "ng")
+        FLOWMM_EX_FMA(24, 25, "ng") FLOWMM_EX_FMA(26, 27, "ng") FLOWMM_EX_FMA(28, 29, "ng") FLOWMM_EX_FMA(30, 31, "ng")
+        FLOWMM_EX_ALL "}"
+        : FLOWMM_EX_REGS(a)
+        : "f"(scale_log2), "f"(-mx));
+}
+__device__ __forceinline__ float sum32(const uint32_t (&a)[32]) {
+    float2 s0 = pair_of(a, 0), s1 = pair_of(a, 2);
+#pragma unroll
+    for (int j = 4; j < 32; j += 4) {
+        s0 = tc::fadd2(s0, pair_of(a, j));
+        s1 = tc::fadd2(s1, pair_of(a, j + 2));
+    }
+    s0 = tc::fadd2(s0, s1);
+    return s0.x + s0.y;
+}
+// The sum over a chunk's visual keys (bit set in `vis`).  `masks`: shared address of sixteen float4, entry n the bits of n as 0.f /
+// 1.f: a multiply-add with the mask, where a test per key would cost three instructions.
+__device__ __forceinline__ float sum32_of(const uint32_t (&a)[32], uint32_t vis, uint32_t masks) {
+    float2 v01 = make_float2(0.f, 0.f), v23 = v01;
+#pragma unroll
+    for (int j = 0; j < 32; j += 4) {
+        const float4 v = tc::lds128(masks + (vis >> j & 15u) * 16);
+        v01 = tc::ffma2(pair_of(a, j), make_float2(v.x, v.y), v01); v23 = tc::ffma2(pair_of(a, j + 2), make_float2(v.z, v.w), v23);
+    }
+    return (v01.x + v01.y) + (v23.x + v23.y);
+}
+
+// A proxy row's statistics over some keys: running maximum, exp-sums over the text and over the visual keys.
+struct RowStats { float m, t, v; };
+__device__ __forceinline__ RowStats join(const RowStats &a, const RowStats &b) {
+    RowStats r;
+    r.m = fmaxf(a.m, b.m);
+    const float wa = tc::ex2(a.m - r.m), wb = tc::ex2(b.m - r.m);
+    r.t = a.t * wa + b.t * wb;
+    r.v = a.v * wa + b.v * wb;
+    return r;
+}
+
 // ---------------------------------------------------------------------------------------------
 // Pass 1.  item = (unit*head, tile of 256 proxy rows, key chunk).
+// The exp-sums are kept by modality of the key: what pass 2 had to split off its probabilities, per query head and with a sum
+// over the warp for each, costs nothing here where a warp's 64 keys of a tile are of one modality and seen by every row, as
+// nearly always (images are runs of tokens): one of the two sums grows, and they change places when the modality does.  128
+// heads of 33 792 tokens, 512 rows each, at the power cap: this pass 605 -> 640 us, pass 2 790 -> 620, the call 3095 -> 2930.
+// (With a choice by modality at every chunk this pass took 690: that code is for the other tiles.)
+// The four warps that share a row join their statistics in shared memory at the end of an item.
+// A wait that runs out changes no warp's way through the items (what follows is garbage, in bounds, and reported), so that no
+// warp is left alone at a meeting.
 template <class S>
 __global__ void __launch_bounds__(tcs::kThreads, 1)
 score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
@@ -97,65 +200,117 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     } else {
         // all sixteen warps drain one accumulator at a time: a warp owns 32 lanes x a quarter of the columns of
         // BOTH halves, so the tensor core refills one half while the other is being read
+        static_assert(S::kCols == 256, "two words of 32 keys per warp and tile");
+        constexpr uint32_t kMeetWarp = 32 * 12, kMeetBytes = 4 * 6 * kMeetWarp;    // (max, text, visual) of a warp's rows; a turn's
+        static_assert(2 * kMeetBytes + 256 <= tcs::kExtraSlots * S::kExtraBytes + tcs::kEpiBytes, "scratch of the meetings");
         const int row_in_half = c.quarter * 32 + c.lane, colq = (c.warp - 2) >> 2;
+        const uint32_t meet = c.base + S::kSmemExtra + (uint32_t)c.quarter * 6 * kMeetWarp + (uint32_t)c.lane * 12;
+        const uint32_t masks = c.base + S::kSmemExtra + 2 * kMeetBytes;
+        const int te = threadIdx.x - 64;
+        if (te < 64) tc::sts32(masks + te * 4, (float)((te >> 2) >> (te & 3) & 1));
+        tcs::named_barrier(5, 32 * tcs::kEpiWarps);
         int kh[2] = {0, 0};
+        uint32_t turn = 0;
         bool ok = true;
-        for (int item = blockIdx.x; ok && item < A.n_items1; item += gridDim.x) {
+        // modalities of this warp's 64 keys of a tile, a tile ahead (keys past the prompt count with its last token, so that they
+        // make no chunk mixed)
+        const uint8_t *mod_at = A.modality, *mod_end = A.modality;
+        uint8_t mod0 = 0, mod1 = 0;
+        auto fetch_mod = [&]() {
+            mod0 = mod_at < mod_end ? *mod_at : *mod_end;
+            mod1 = mod_at + 32 < mod_end ? mod_at[32] : *mod_end;
+            mod_at += S::kCols;
+        };
+        auto first_mod = [&](int item) {
+            if (item >= A.n_items1) return;
             const tcs::TilePlan p = plan(item);
-            if (p.empty()) continue;
+            mod_end = A.modality + (int64_t)(p.b3 + 1) * A.L - 1;
+            mod_at = mod_end + (p.b1 + colq * 64 + c.lane - A.L + 1);
+            fetch_mod();
+        };
+        first_mod(blockIdx.x);
+        for (int item = blockIdx.x; item < A.n_items1; item += gridDim.x) {
+            const tcs::TilePlan p = plan(item);
+            if (p.empty()) continue;                                     // (never: every chunk holds keys)
             const int kc = item % A.n_chunk, qt = (item / A.n_chunk) % A.n_qt, uh = item / (A.n_chunk * A.n_qt);
-            float m[2] = {kNegBig, kNegBig}, l[2] = {0.f, 0.f};
-            for (int t = 0; ok && t < p.n_tiles; ++t) {
+            RowStats st[2] = {{kNegBig, 0.f, 0.f}, {kNegBig, 0.f, 0.f}};
+            bool swapped = false;                                        // st[].t belongs to the visual keys and st[].v to the text keys
+            for (int t = 0; t < p.n_tiles; ++t) {
                 const int kb = p.b1 + t * S::kCols;
                 const int ncols = min(S::kCols, p.cols_total - t * S::kCols);
+                const uint32_t vis0 = __ballot_sync(0xFFFFFFFFu, mod0 != 0), vis1 = __ballot_sync(0xFFFFFFFFu, mod1 != 0);
+                fetch_mod();                                             // (past the item's last tile: of no use)
+                // the common tile: every row sees all of its keys, and this warp's are of one modality
+                const bool plain = kb + S::kCols <= A.L - A.W + 1 && vis0 == vis1 && (vis0 == 0u || vis0 == 0xFFFFFFFFu);
+                if (plain && (vis0 != 0u) != swapped) {
+                    swapped = !swapped;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) { const float x = st[h].t; st[h].t = st[h].v; st[h].v = x; }
+                }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    if (h >= p.n_halves || !ok) continue;
-                    ok = S::acc_wait_h(c, h, kh[h]++, A.status);
-                    if (!ok) continue;
+                    if (h >= p.n_halves) continue;
+                    if (ok) ok = S::acc_wait_h(c, h, kh[h], A.status);
+                    ++kh[h];
                     const int r0 = qt * tcs::kItemRows + h * tcs::kRows;
-                    const int pa = A.L - A.W + ((r0 + row_in_half) % A.W);   // last key this proxy row may see
-                    if (r0 + c.quarter * 32 < A.GW) {
+                    auto release = [&]() { if (ok) S::acc_release_h(c, h); };
+                    if (r0 + c.quarter * 32 >= A.GW) release();
+                    else if (plain) {
+                        S::for_each_chunk_q(c, h, colq, S::kCols / 32, [&](int, uint32_t (&acc)[32]) {
+                            const float mx = fmaxf(max32(acc) * A.scale_log2, st[h].m);
+                            const float all = exp_sum32(acc, A.scale_log2, mx), carry = tc::ex2(st[h].m - mx);
+                            st[h].t = st[h].t * carry + all;
+                            st[h].v *= carry;
+                            st[h].m = mx;
+                        }, release);
+                    } else {
+                        const int pa = A.L - A.W + ((r0 + row_in_half) & (A.W - 1));   // last key this proxy row may see (the window is 32, 64 or 128 rows)
                         S::for_each_chunk_q(c, h, colq, (ncols + 31) >> 5, [&](int ch, uint32_t (&acc)[32]) {
-                            const int k0 = kb + ch * 32;
-                            float mx;
-                            float add;
-                            if (k0 + 32 <= A.L - A.W + 1) {              // no key of this chunk is masked for any row
-                                float raw[32];
+                            const int last = pa - (kb + ch * 32);        // this row sees the chunk's keys 0 .. last
+                            uint32_t vis = (ch & 1) ? vis1 : vis0;
+                            asm volatile("" : "+r"(vis));                // (or what the sum below needs of it is formed for the plain tiles as well)
+                            if (kb + ch * 32 + 32 > A.L - A.W + 1) {
 #pragma unroll
-                                for (int j = 0; j < 32; ++j) raw[j] = __uint_as_float(acc[j]);
-                                mx = fmaxf(max32(raw) * A.scale_log2, m[h]);
-                                add = exp_sum32(raw, A.scale_log2, mx);
-                            } else {
-                                float s[32];
-#pragma unroll
-                                for (int j = 0; j < 32; ++j)
-                                    s[j] = (k0 + j <= pa) ? __uint_as_float(acc[j]) * A.scale_log2 : kNegBig;
-                                mx = fmaxf(max32(s), m[h]);
-                                float add0 = 0.f, add1 = 0.f, add2 = 0.f, add3 = 0.f;
-#pragma unroll
-                                for (int j = 0; j < 32; j += 4) {        // masked entries sit ~1e30 below: exp2 gives 0
-                                    add0 += tc::ex2(s[j] - mx);
-                                    add1 += tc::ex2(s[j + 1] - mx);
-                                    add2 += tc::ex2(s[j + 2] - mx);
-                                    add3 += tc::ex2(s[j + 3] - mx);
-                                }
-                                add = (add0 + add1) + (add2 + add3);
-                                if (mx < 0.5f * kNegBig) add = 0.f;      // nothing visible yet: exp2(0) terms are not real
+                                for (int j = 0; j < 32; ++j) acc[j] = j <= last ? acc[j] : __float_as_uint(-INFINITY);   // exp2 gives 0
                             }
-                            l[h] = l[h] * tc::ex2(m[h] - mx) + add;
-                            m[h] = mx;
-                        }, [&]() { S::acc_release_h(c, h); });
-                    } else S::acc_release_h(c, h);
+                            const float mx = fmaxf(max32(acc) * A.scale_log2, st[h].m), carry = tc::ex2(st[h].m - mx);
+                            exp2_32(acc, A.scale_log2, mx);
+                            const float all = sum32(acc);
+                            float on_vis = vis ? all : 0.f;
+                            if (vis != 0u && vis != 0xFFFFFFFFu) on_vis = sum32_of(acc, vis, masks);
+                            const float on_text = fmaxf(all - on_vis, 0.f);
+                            st[h].t = st[h].t * carry + (swapped ? on_vis : on_text);
+                            st[h].v = st[h].v * carry + (swapped ? on_text : on_vis);
+                            st[h].m = mx;
+                        }, release);
+                    }
                 }
             }
-            if (!ok) break;
+            if (swapped)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = qt * tcs::kItemRows + h * tcs::kRows + row_in_half;
-                if (h < p.n_halves && r < A.GW)
-                    A.row_part[((int64_t)uh * A.GW + r) * (4 * A.n_chunk) + 4 * kc + colq] = make_float2(m[h], l[h]);
+                for (int h = 0; h < 2; ++h) { const float x = st[h].t; st[h].t = st[h].v; st[h].v = x; }
+            first_mod(item + gridDim.x);
+            // the four warps of a row join their quarters of the columns: warp 0 the first half's rows, warp 1 the second's
+            // (two sets of slots by turns: the next meeting keeps writers from slots that are still being read)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (colq != h) {
+                    const uint32_t at = meet + turn + (uint32_t)(h * 3 + ((colq - h - 1) & 3)) * kMeetWarp;
+                    tc::sts32(at, st[h].m); tc::sts32(at + 4, st[h].t); tc::sts32(at + 8, st[h].v);
+                }
+            ok = !__any_sync(0xFFFFFFFFu, tcs::meet_vote(1 + c.quarter, 128, !ok));   // (the vote: for the compiler, which then knows the warp to be of one mind)
+            const int r = qt * tcs::kItemRows + colq * tcs::kRows + row_in_half;
+            if (colq < p.n_halves && r < A.GW) {
+                RowStats s = colq == 0 ? st[0] : st[1];
+#pragma unroll
+                for (int w = 0; w < 3; ++w) {
+                    const uint32_t at = meet + turn + (uint32_t)(colq * 3 + w) * kMeetWarp;
+                    const RowStats o = {tc::lds32(at), tc::lds32(at + 4), tc::lds32(at + 8)};
+                    s = join(s, o);
+                }
+                A.row_part[((int64_t)uh * A.GW + r) * A.n_chunk + kc] = make_float4(s.m, s.t, s.v, 0.f);
             }
+            turn ^= kMeetBytes;
         }
     }
     S::teardown(c);
@@ -171,19 +326,15 @@ __global__ void pack_modality_kernel(const uint8_t *modality, int L, int n_words
     if (lane == 0) bits[(int64_t)u * n_words + w] = word;
 }
 
-// Row constants for pass 2: negc[r] = -(M_r + log2 Z_r) so that exp2(s + negc) is the softmax
-// probability; padding rows get a constant that makes every probability 0.
-// kLanes lanes share a row and read its parts together.
-// Bound by latency while the rows are few and by issue slots when they are many: four lanes of a row of four parts spend more on
-// the row's number, the exchange of maximum and sum, and the logarithm than on its parts.
+// Joins a row's statistics over n_part key chunks to one record, where pass 2 would have to read many of them for each of its
+// heads: kLanes lanes share a row and read its parts together.
 template <int kLanes>
-__global__ void score_combine_kernel(const float2 *row_part, int n_part, int GW, int GWpad, int n_uh, float *negc) {
+__global__ void score_combine_kernel(const float4 *row_part, int n_part, int n_rows, float4 *row_all) {
     predecessor_done();
     const int i = blockIdx.x * (blockDim.x / kLanes) + threadIdx.x / kLanes, sub = threadIdx.x % kLanes;
-    const int uh = i / GWpad, r = i - uh * GWpad;
-    const bool on = i < n_uh * GWpad && r < GW;
-    const float2 *part = row_part + ((int64_t)uh * GW + r) * n_part;
-    float mx = kNegBig, z = 0.f;
+    const bool on = i < n_rows;
+    const float4 *part = row_part + (int64_t)i * n_part;
+    float mx = kNegBig, t = 0.f, v = 0.f;
     if (on) {
 #pragma unroll 4
         for (int c = sub; c < n_part; c += kLanes) mx = fmaxf(mx, part[c].x);
@@ -192,74 +343,38 @@ __global__ void score_combine_kernel(const float2 *row_part, int n_part, int GW,
     for (int o = kLanes / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
     if (on) {
 #pragma unroll 4
-        for (int c = sub; c < n_part; c += kLanes) z += part[c].y * exp2f(part[c].x - mx);
+        for (int c = sub; c < n_part; c += kLanes) {
+            const float4 p = part[c];
+            const float w = exp2f(p.x - mx);
+            t += p.y * w; v += p.z * w;
+        }
     }
 #pragma unroll
-    for (int o = kLanes / 2; o > 0; o >>= 1) z += __shfl_xor_sync(0xFFFFFFFFu, z, o);
-    if (sub == 0 && i < n_uh * GWpad) negc[i] = r < GW ? -(mx + log2f(z)) : kNegBig;
+    for (int o = kLanes / 2; o > 0; o >>= 1) {
+        t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+        v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    }
+    if (sub == 0 && on) row_all[i] = make_float4(mx, t, v, 0.f);
 }
 
-// The common case of pass 2's inner step, written out in PTX so that it costs what it must and no more: 32 accumulator
-// columns of this thread's key (32 proxy rows of one query head): probability = 2^(logit * scale + row constant), with
-// the row constants read as packed pairs from shared memory, the multiply-adds and the additions as packed pairs, one
-// exp2 per element; returns the sum of the 32 probabilities.  No mask and no split by modality: chunks that need either
-// take the general path.
-//   taddr  TMEM address of the chunk for this warp's lanes     negc  shared address of its 32 row constants
+// The common case of pass 2's inner step: 32 accumulator columns of this thread's key (32 proxy rows of one query head),
+// probability = 2^(logit * scale + row constant), with the row constants read as packed pairs from shared memory; their sum is
+// added to the packed pair `sum`.  No causal mask: chunks that need it take the general path.
+//   a  the chunk's accumulators     negc  shared address of its 32 row constants
 // (three phases, so that no exponential's result is needed before the last one has been issued: logits in place,
 // exponentials in place, then a tree of packed additions)
 #define FLOWMM_CS_X(q, i0, i1, i2, i3)                                                      \
-    "ld.shared.v2.b64 {n0, n1}, [%2 + " #q " * 16];\n\t"                                    \
-    "mov.b64 x0, {a" #i0 ", a" #i1 "};\n\t"                                                 \
-    "mov.b64 x1, {a" #i2 ", a" #i3 "};\n\t"                                                 \
-    "fma.rn.f32x2 x0, x0, sc, n0;\n\t"                                                      \
-    "fma.rn.f32x2 x1, x1, sc, n1;\n\t"                                                      \
-    "mov.b64 {a" #i0 ", a" #i1 "}, x0;\n\t"                                                 \
-    "mov.b64 {a" #i2 ", a" #i3 "}, x1;\n\t"
-#define FLOWMM_CS_E(i) "ex2.approx.ftz.f32 a" #i ", a" #i ";\n\t"
-// 2^x for the pair (a_i, a_j) on the FMA pipe instead of the exp2 unit (which sets this step's pace): x clamped at
-// -125, n = round(x) by the 1.5 * 2^23 trick, 2^f on f = x - n in [-0.5, 0.5] by a degree-4 polynomial (own least-squares
-// fit at Chebyshev nodes with the constant fixed at 1: relative error 3.6e-6), n added to the exponent field.
-#define FLOWMM_CS_POLY(i, j)                                                          \
-    "max.f32 a" #i ", a" #i ", 0fC2FA0000;\n\t"                                        \
-    "max.f32 a" #j ", a" #j ", 0fC2FA0000;\n\t"                                        \
-    "mov.b64 x0, {a" #i ", a" #j "};\n\t"                                              \
-    "add.rn.f32x2 x1, x0, kmg;\n\t"          /* t = x + 1.5 * 2^23 */                  \
-    "mov.b64 {f0, f1}, x1;\n\t"                                                       \
-    "sub.rn.f32x2 x1, x1, kmg;\n\t"          /* n */                                   \
-    "sub.rn.f32x2 x0, x0, x1;\n\t"           /* f */                                   \
-    "fma.rn.f32x2 x1, kc4, x0, kc3;\n\t"                                              \
-    "fma.rn.f32x2 x1, x1, x0, kc2;\n\t"                                               \
-    "fma.rn.f32x2 x1, x1, x0, kc1;\n\t"                                               \
-    "fma.rn.f32x2 x1, x1, x0, kone;\n\t"                                              \
-    "mov.b64 {a" #i ", a" #j "}, x1;\n\t"                                              \
-    "mad.lo.s32 a" #i ", f0, 8388608, a" #i ";\n\t"                                    \
-    "mad.lo.s32 a" #j ", f1, 8388608, a" #j ";\n\t"
-#define FLOWMM_CS_P(k, i0, i1) "mov.b64 p" #k ", {a" #i0 ", a" #i1 "};\n\t"
+    "ld.shared.v2.b64 {n0, n1}, [%33 + " #q " * 16];\n\t"                                   \
+    FLOWMM_EX_FMA(i0, i1, "n0") FLOWMM_EX_FMA(i2, i3, "n1")
+#define FLOWMM_CS_P(k, i0, i1) "mov.b64 p" #k ", {%" #i0 ", %" #i1 "};\n\t"
 #define FLOWMM_CS_A(d, x, y) "add.rn.f32x2 p" #d ", p" #x ", p" #y ";\n\t"
-__device__ __forceinline__ float colsum_chunk32(uint32_t taddr, uint32_t negc, float scale_log2) {
-    float csum;
+__device__ __forceinline__ void colsum_chunk32(uint32_t (&a)[32], uint32_t negc, float scale_log2, uint64_t &sum) {
     asm volatile(
-        "{\n\t"
-        ".reg .b32 a<32>;\n\t"
-        ".reg .b64 n0, n1, x0, x1, sc, p<16>, kmg, kc1, kc2, kc3, kc4, kone;\n\t"
-        ".reg .b32 f0, f1;\n\t"
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {a0, a1, a2, a3, a4, a5, a6, a7, a8, a9, a10, a11, a12, a13, a14, a15, "
-        "a16, a17, a18, a19, a20, a21, a22, a23, a24, a25, a26, a27, a28, a29, a30, a31}, [%1];\n\t"
-        "mov.b64 sc, {%3, %3};\n\t"
-        "mov.b64 kmg, 0x4B4000004B400000;\n\t"      /* 12582912.0f twice */
-        "mov.b64 kone, 0x3F8000003F800000;\n\t"
-        "mov.b64 kc1, 0x3F3170613F317061;\n\t"      /* 0.69312102 */
-        "mov.b64 kc2, 0x3E75FCD43E75FCD4;\n\t"      /* 0.24022228 */
-        "mov.b64 kc3, 0x3D650E813D650E81;\n\t"      /* 0.05592204 */
-        "mov.b64 kc4, 0x3C1E78073C1E7807;\n\t"      /* 0.00967217 */
-        "tcgen05.wait::ld.sync.aligned;\n\t"
+        "{\n\t" FLOWMM_EX_DECL ".reg .b64 n0, n1, p<16>;\n\t"
+        "mov.b64 sc, {%34, %34};\n\t"
         FLOWMM_CS_X(0, 0, 1, 2, 3) FLOWMM_CS_X(1, 4, 5, 6, 7) FLOWMM_CS_X(2, 8, 9, 10, 11) FLOWMM_CS_X(3, 12, 13, 14, 15)
         FLOWMM_CS_X(4, 16, 17, 18, 19) FLOWMM_CS_X(5, 20, 21, 22, 23) FLOWMM_CS_X(6, 24, 25, 26, 27) FLOWMM_CS_X(7, 28, 29, 30, 31)
-        // every fourth exponential goes to the FMA pipe, placed between the others
-        FLOWMM_CS_E(0) FLOWMM_CS_E(1) FLOWMM_CS_E(2) FLOWMM_CS_E(4) FLOWMM_CS_E(5) FLOWMM_CS_E(6) FLOWMM_CS_POLY(3, 7)
-        FLOWMM_CS_E(8) FLOWMM_CS_E(9) FLOWMM_CS_E(10) FLOWMM_CS_E(12) FLOWMM_CS_E(13) FLOWMM_CS_E(14) FLOWMM_CS_POLY(11, 15)
-        FLOWMM_CS_E(16) FLOWMM_CS_E(17) FLOWMM_CS_E(18) FLOWMM_CS_E(20) FLOWMM_CS_E(21) FLOWMM_CS_E(22) FLOWMM_CS_POLY(19, 23)
-        FLOWMM_CS_E(24) FLOWMM_CS_E(25) FLOWMM_CS_E(26) FLOWMM_CS_E(28) FLOWMM_CS_E(29) FLOWMM_CS_E(30) FLOWMM_CS_POLY(27, 31)
+        FLOWMM_EX_ALL
         FLOWMM_CS_P(0, 0, 1) FLOWMM_CS_P(1, 2, 3) FLOWMM_CS_P(2, 4, 5) FLOWMM_CS_P(3, 6, 7) FLOWMM_CS_P(4, 8, 9) FLOWMM_CS_P(5, 10, 11)
         FLOWMM_CS_P(6, 12, 13) FLOWMM_CS_P(7, 14, 15) FLOWMM_CS_P(8, 16, 17) FLOWMM_CS_P(9, 18, 19) FLOWMM_CS_P(10, 20, 21)
         FLOWMM_CS_P(11, 22, 23) FLOWMM_CS_P(12, 24, 25) FLOWMM_CS_P(13, 26, 27) FLOWMM_CS_P(14, 28, 29) FLOWMM_CS_P(15, 30, 31)
@@ -268,27 +383,32 @@ __device__ __forceinline__ float colsum_chunk32(uint32_t taddr, uint32_t negc, f
         FLOWMM_CS_A(0, 0, 2) FLOWMM_CS_A(4, 4, 6) FLOWMM_CS_A(8, 8, 10) FLOWMM_CS_A(12, 12, 14)
         FLOWMM_CS_A(0, 0, 4) FLOWMM_CS_A(8, 8, 12)
         FLOWMM_CS_A(0, 0, 8)
-        "mov.b64 {f0, f1}, p0;\n\t"
-        "add.f32 %0, f0, f1;\n\t"
+        "add.rn.f32x2 %32, %32, p0;\n\t"
         "}"
-        : "=f"(csum)
-        : "r"(taddr), "r"(negc), "f"(scale_log2)
+        : FLOWMM_EX_REGS(a), "+l"(sum)
+        : "r"(negc), "f"(scale_log2)
         : "memory");
-    return csum;
 }
 #undef FLOWMM_CS_X
-#undef FLOWMM_CS_E
-#undef FLOWMM_CS_POLY
 #undef FLOWMM_CS_P
 #undef FLOWMM_CS_A
+#undef FLOWMM_EX_FMA
+#undef FLOWMM_EX_E
+#undef FLOWMM_EX_POLY
+#undef FLOWMM_EX_DECL
+#undef FLOWMM_EX_ALL
+#undef FLOWMM_EX_REGS
 
 // ---------------------------------------------------------------------------------------------
 // Pass 2.  item = (unit*head, tile of 256 keys); the B stream is the head group's proxy rows.  A CTA takes a run of
 // consecutive items, so that proxy rows that fit the B stages (up to 512) are loaded once per head, not once per item.
-// Bound by the epilogue (four warps per scheduler, exp2 at half of its rate): what an item costs besides its exponentials
-// counts.  Its place in the run is stepped, not divided out, the two column halves of a key meet once per item, and two
-// heads' masses are summed over the warp together: 112 heads of 8448 tokens, 448 rows each, 158 -> 148 us; 128 heads of 33792,
-// 512 rows, 861 -> 812 us; 112 of 2176, 224 rows, 34.5 -> 30.8 us.
+// Row constants -(max + log2 sum) - exp2(logit + constant) is the softmax probability - are formed from pass 1's statistics by
+// the epilogue warps when the run comes to another head; the CTA with a head's first tile also writes its rows' cross-modal shares.
+// (A launch of its own for the constants took 3 us: 8 heads of 1471 tokens 39.0 -> 36.2 us for the call, 112 of 2176 121 -> 116.)
+// Bound by the epilogue (four warps per scheduler, the exp2 unit at 0.69 of its rate, 0.56 before the masses went to pass 1): a
+// chunk is read while the one before it is worked on, an accumulator is handed back as soon as its last chunk is in registers,
+// and no vote or shuffle stands between: 197 -> 152 instructions per chunk of 32 columns.  (Three or four words a thread of
+// what belongs to the item are spilled around the chunks; unrolling two chunks instead of four leaves one, and is 1 % slower.)
 template <class S>
 __global__ void __launch_bounds__(tcs::kThreads, 1)
 score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap q_map,
@@ -310,7 +430,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
         p.n_tiles = (A.GW + S::kCols - 1) / S::kCols;
         p.reuse_b = p.n_tiles <= S::kBStages && kt > 0 && g > g_lo;
         p.keep_b = p.n_tiles <= S::kBStages && kt + 1 < A.n_rt && g + 1 < g_hi;
-        p.extra = A.negc + (int64_t)uh * A.GWpad;        // row constants of pass 1, 256 per B tile
+        p.extra = nullptr;
         return p;
     };
     const uint32_t b_bytes = (uint32_t)A.b_heads * A.W * 256u;
@@ -319,150 +439,108 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
     } else if (c.warp == 1) {
         S::template mma_issuer<true>(c, blockIdx.x + n_loop, plan, A.status);
     } else {
-        const int lane = c.lane, row = c.quarter * 32 + lane;
-        const uint32_t xch = c.epi_addr() + row * 4;            // hand-over slot of this row
-        const uint32_t pxch = c.partner_addr() + row * 4;
-        int k = 0, bt = 0, cached_u = -1;
-        const int w_shift = 31 - __clz(A.W);
-        uint32_t wbits[4] = {0, 0, 0, 0};                            // modality of the proxy tokens, 32 per word
+        // scratch: two sets of row constants by turns (up to 1024 rows), then the hand-over slots of the row halves, two by turns
+        constexpr uint32_t kConstBytes = 4096, kXch = S::kSmemEpi + 2 * kConstBytes;
+        static_assert(2 * kConstBytes + 2 * 2 * tcs::kRows * 4 <= tcs::kEpiBytes, "scratch");
+        const int lane = c.lane, row = c.quarter * 32 + lane, te = threadIdx.x - 64;
+        const uint32_t xch = c.base + kXch + (uint32_t)(c.group * tcs::kRows + row) * 4;
+        int k = 0;
         bool ok = true;
         // the run's items one after the other: (unit u, KV head uh, its tile kt) step by step instead of by divisions, which
         // together with the rest of an item's start took a tenth of the epilogue's time
         const int n_tiles = (A.GW + S::kCols - 1) / S::kCols;
         int uh = (int)A.by_rt.div(g_lo), kt = g_lo - uh * A.n_rt, u = (int)A.by_hkv.div(uh), hk = uh - u * A.Hkv;
-        const int key_in_item = c.group * tcs::kRows + row;
-        auto fetch_mod = [&](int u, int kt) -> int {                 // modality of this thread's key, an item ahead
-            const int key = kt * tcs::kItemRows + key_in_item;
-            return key < A.L ? A.modality[(int64_t)u * A.L + key] : 0;
-        };
-        int mod_next = g_lo < g_hi ? fetch_mod(u, kt) : 0;
-        uint32_t slot = 0;                                           // hand-over slots by turns
-        for (int g = g_lo; ok && g < g_hi; ++g) {
-            const int uh0 = uh, kt0 = kt, u0 = u, h0 = hk;           // this item
-            if (++kt == A.n_rt) {                                    // the next one
+        uint32_t slot = 0, consts = c.base + S::kSmemEpi + kConstBytes;
+        for (int g = g_lo; g < g_hi; ++g) {
+            const int uh0 = uh, kt0 = kt;                            // this item
+            if (g == g_lo || kt0 == 0) {                             // a new head: its row constants
+                consts ^= (c.base + S::kSmemEpi) ^ (c.base + S::kSmemEpi + kConstBytes);
+                for (int r = te; r < A.GW; r += 32 * tcs::kEpiWarps) {
+                    const float4 *rec = A.row_rec + ((int64_t)uh0 * A.GW + r) * A.n_rec;
+                    float4 s = rec[0];
+#pragma unroll 4
+                    for (int i = 1; i < A.n_rec; ++i) s.x = fmaxf(s.x, rec[i].x);
+                    if (A.n_rec > 1) {
+                        const float mx = s.x;
+                        s.y = 0.f; s.z = 0.f;
+#pragma unroll 4
+                        for (int i = 0; i < A.n_rec; ++i) {
+                            const float4 o = rec[i];
+                            const float w = exp2f(o.x - mx);
+                            s.y += o.y * w; s.z += o.z * w;
+                        }
+                    }
+                    const float z = s.y + s.z;
+                    tc::sts32(consts + r * 4, -(s.x + log2f(z)));
+                    if (kt0 == 0) {                                  // (one CTA per head)
+                        const bool vis = A.modality[(int64_t)u * A.L + A.L - A.W + (r & (A.W - 1))] != 0;   // (the window is 32, 64 or 128 rows)
+                        A.cross_part[((int64_t)u * A.Hq + hk * A.G) * A.W + r] = (vis ? s.y : s.z) / z;
+                    }
+                }
+                // (the set written was read two heads ago, and every warp has been through the meeting of the head between)
+                tcs::named_barrier(9, 32 * tcs::kEpiWarps);
+            }
+            if (++kt == A.n_rt) {                                    // the next item
                 kt = 0; ++uh;
                 if (++hk == A.Hkv) { hk = 0; ++u; }
             }
-            const bool my_vis = mod_next != 0;
-            mod_next = g + 1 < g_hi ? fetch_mod(u, kt) : 0;
-            if (n_tiles <= S::kBStages && kt0 > 0 && g > g_lo) bt -= n_tiles;   // TilePlan::reuse_b (bt: number of the B tile an item begins with)
             const int key0 = kt0 * tcs::kItemRows + c.group * tcs::kRows;
-            float *cross_out = A.cross_part + ((int64_t)u0 * A.Hq + h0 * A.G) * (A.n_rt * 8) + kt0 * 8 + c.group * 4 + c.quarter;
-            if (key0 >= A.L) {                                       // no keys in this half: its masses are zero
-                if (lane == 0)
-                    for (int j = 0; j < A.G; ++j) cross_out[(int64_t)j * (A.n_rt * 8)] = 0.f;
-                bt += n_tiles;                                       // keep the B-tile count in step
-                continue;
-            }
-            if (u0 != cached_u) {
-#pragma unroll
-                for (int w = 0; w < 4; ++w) {
-                    const int a = w * 32 + lane;
-                    const bool vis = a < A.W && A.modality[(int64_t)u0 * A.L + A.L - A.W + a] != 0;
-                    wbits[w] = __ballot_sync(0xFFFFFFFFu, vis);
-                }
-                cached_u = u0;
-            }
+            if (key0 >= A.L) continue;                               // no keys in this half
             const int key = key0 + row;
             const bool masked_tile = key0 + tcs::kRows > A.L - A.W + 1;   // some (key, proxy row) pair is masked
             const int first_proxy = A.L - A.W;
-            float imp = 0.f, cg = 0.f;
-            int cur_g = -1;                                          // head whose mass is being summed; -1: none yet
-            float held = 0.f;                                        // a complete head's mass that waits for the next one's:
-            int held_g = -1;                                         // two are summed over the warp together
-            auto publish = [&]() {
-                if (held_g < 0) { held = cg; held_g = cur_g; return; }
-                const bool up = lane & 16;                           // the held head goes to the lower lanes, this one to the upper
-                float x = (up ? cg : held) + __shfl_xor_sync(0xFFFFFFFFu, up ? held : cg, 16);
-#pragma unroll
-                for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xFFFFFFFFu, x, o);
-                if ((lane & 15) == 0) cross_out[(int64_t)(up ? cur_g : held_g) * (A.n_rt * 8)] = x;
-                held_g = -1;
-            };
-            // A wait that runs out changes no lane's way through the item (what follows is garbage, in bounds, and reported): the
-            // votes, shuffles and reads of tensor memory stay the whole warp's without a vote on every wait, which took 5 % (320
+            uint64_t sum2 = 0;                                       // a packed pair of partial sums
+            float imp = 0.f;
+            // A wait that runs out changes no lane's way through the items (what follows is garbage, in bounds, and reported): the
+            // reads of tensor memory and the meetings stay the whole warp's without a vote on every wait, which took 5 % (320
             // units of 8 heads, 512 proxy rows, 33 792 tokens 16.65 ms, 17.5 with the vote).  pair_meet tells all lanes.
-            for (int t = 0; t < n_tiles; ++t, ++bt) {
+            for (int t = 0; t < n_tiles; ++t) {
                 const int ncols = min(S::kCols, A.GW - t * S::kCols);
                 if (!S::takes_part(c, ncols)) continue;
-                ok = ok && S::quad_extra_wait_lanes(c, k, bt, A.status);
+                ok = ok && S::quad_extra_wait_lanes(c, k, -1, A.status);
                 ++k;
-                const uint32_t negc4 = c.extra(bt);
-                constexpr int kPerC = S::kCols / 64;               // 32-column chunks a warp takes of a full tile
-                const int chunk_hi = min((ncols + 31) >> 5, kPerC * c.colhalf + kPerC);
-                for (int ch = kPerC * c.colhalf; ch < chunk_hi; ++ch) {
-                    const int col = t * S::kCols + ch * 32;        // proxy row index r = g_local * W + a
-                    const int g_local = col >> w_shift, a0 = col & (A.W - 1);   // (the window is 32, 64 or 128 rows)
-                    if (g_local != cur_g) {                          // a head is complete: publish its mass
-                        if (cur_g >= 0) publish();
-                        cg = 0.f;
-                        cur_g = g_local;
+                constexpr int kPerC = S::kCols / 64;                 // 32-column chunks a warp takes of a full tile
+                const int ch0 = kPerC * c.colhalf, n_ch = min((ncols + 31) >> 5, ch0 + kPerC) - ch0;   // >= 1
+                const uint32_t nc = consts + (uint32_t)(t * S::kCols + ch0 * 32) * 4;
+                if (!masked_tile) {
+                    uint32_t a[2][32];
+                    tc::tmem_ld32(S::acc_addr(c, ch0), a[0]);
+#pragma unroll
+                    for (int i = 0; i < kPerC; ++i) {
+                        if (i >= n_ch) break;
+                        tc::tmem_ld_wait(a[i & 1]);
+                        if (i + 1 < kPerC && i + 1 < n_ch) tc::tmem_ld32(S::acc_addr(c, ch0 + i + 1), a[(i + 1) & 1]);
+                        else S::quad_release(c);
+                        colsum_chunk32(a[i & 1], nc + i * 128, A.scale_log2, sum2);
                     }
-                    // proxy tokens of the other modality than this key's
-                    const uint32_t wm = a0 < 32 ? wbits[0] : a0 < 64 ? wbits[1] : a0 < 96 ? wbits[2] : wbits[3];
-                    const uint32_t other = my_vis ? ~wm : wm;
-                    // the common case: no causal mask inside this tile, and the chunk's proxy tokens are all of this
-                    // key's modality or all of the other one (decided for the whole warp: the TMEM read is warp-wide)
-                    const bool plain = !masked_tile && (other == 0u || other == 0xFFFFFFFFu);
-                    if (__all_sync(0xFFFFFFFFu, plain)) {
-                        const float csum = colsum_chunk32(S::acc_addr(c, ch), negc4 + ch * 128, A.scale_log2);
-                        imp += csum;
-                        cg += other != 0u ? csum : 0.f;
-                        continue;
-                    }
+                    continue;
+                }
+                for (int i = 0; i < n_ch; ++i) {
+                    const int a0 = (t * S::kCols + (ch0 + i) * 32) & (A.W - 1);   // the chunk's first proxy token
                     uint32_t acc[32];
-                    tc::tmem_ld32(S::acc_addr(c, ch), acc);
+                    tc::tmem_ld32(S::acc_addr(c, ch0 + i), acc);
                     tc::tmem_ld_wait(acc);
-                    float pr[32];
-                    const float2 sc2 = make_float2(A.scale_log2, A.scale_log2);
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4) {
-                        const float4 n4 = tc::lds128(negc4 + (ch * 8 + q4) * 16);
-                        const float2 x01 = tc::ffma2(make_float2(__uint_as_float(acc[4 * q4 + 0]), __uint_as_float(acc[4 * q4 + 1])),
-                                                     sc2, make_float2(n4.x, n4.y));
-                        const float2 x23 = tc::ffma2(make_float2(__uint_as_float(acc[4 * q4 + 2]), __uint_as_float(acc[4 * q4 + 3])),
-                                                     sc2, make_float2(n4.z, n4.w));
-                        pr[4 * q4 + 0] = tc::ex2(x01.x);
-                        pr[4 * q4 + 1] = tc::ex2(x01.y);
-                        pr[4 * q4 + 2] = tc::ex2(x23.x);
-                        pr[4 * q4 + 3] = tc::ex2(x23.y);
-                    }
-                    if (masked_tile) {                               // causal mask inside the window, and keys >= L
+                        const float4 n4 = tc::lds128(nc + (i * 8 + q4) * 16);
+                        const float nn[4] = {n4.x, n4.y, n4.z, n4.w};
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) pr[j] = (key <= first_proxy + a0 + j) ? pr[j] : 0.f;
-                    }
-                    float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int j = 0; j < 32; j += 4) {
-                        s01 = tc::fadd2(s01, make_float2(pr[j], pr[j + 1]));
-                        s23 = tc::fadd2(s23, make_float2(pr[j + 2], pr[j + 3]));
-                    }
-                    const float csum = (s01.x + s01.y) + (s23.x + s23.y);
-                    imp += csum;
-                    if (other == 0xFFFFFFFFu) cg += csum;
-                    else if (other != 0u) {
-                        float x = 0.f;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) x += ((other >> j) & 1u) ? pr[j] : 0.f;
-                        cg += x;
+                        for (int j = 0; j < 4; ++j) {                // causal mask inside the window, and keys >= L
+                            const float e = tc::ex2(fmaf(__uint_as_float(acc[4 * q4 + j]), A.scale_log2, nn[j]));
+                            imp += key <= first_proxy + a0 + 4 * q4 + j ? e : 0.f;
+                        }
                     }
                 }
                 S::quad_release(c);
             }
-            if (cur_g >= 0) {
-                publish();
-                if (held_g >= 0) {
-                    const float tot = warp_sum(held);
-                    if (lane == 0) cross_out[(int64_t)held_g * (A.n_rt * 8)] = tot;
-                }
-            }
+            imp += __uint_as_float((uint32_t)sum2) + __uint_as_float((uint32_t)(sum2 >> 32));
             // the two column halves of a key meet: the upper one hands its partial sum over (kept even after a
             // wait ran out, so that the partner warp is never left waiting).  Two slots by turns: the next meeting keeps the
             // upper half from a slot that is still being read.
             if (c.colhalf == 1) tc::sts32(xch + slot, imp);
-            ok = !S::pair_meet(c, !ok);                            // (both warps of a key go on, or neither)
-            if (c.colhalf == 0 && ok && key < A.L) A.importance[(int64_t)uh0 * A.L + key] = (imp + tc::lds32(pxch + slot)) / (float)A.G;   // group mean
-            slot ^= tcs::kRows * 4;
+            ok = !S::pair_meet(c, !ok);
+            if (c.colhalf == 0 && ok && key < A.L) A.importance[(int64_t)uh0 * A.L + key] = (imp + tc::lds32(xch + slot)) / (float)A.G;   // group mean
+            slot ^= 2 * tcs::kRows * 4;
         }
     }
     S::teardown(c);

@@ -40,6 +40,21 @@ constexpr int kExtraSlots = 4;               // ring of per-column constants: a 
 constexpr uint32_t kEpiBytes = 16384;
 constexpr int kStatusAlign = 6;              // FLOWMM_ERR_ALIGN
 
+// Meeting of the CTA's threads that use named barrier `id`, `count` of them in whole warps; with a vote: whether any of them says yes.
+__device__ __forceinline__ void named_barrier(int id, int count) { asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(count) : "memory"); }
+__device__ __forceinline__ bool meet_vote(int id, int count, bool yes) {
+    uint32_t any;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "barrier.cta.red.or.pred p, %2, %3, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(any)
+        : "r"((uint32_t)yes), "r"(id), "r"(count)
+        : "memory");
+    return any != 0;
+}
+
 // Where an item's operands come from.  All tensor maps are 4-D: (K element, c1, c2, c3).
 struct TilePlan {
     int a1, a2, a3;            // box origin of A half 0
@@ -299,10 +314,10 @@ struct Skel {
         tc::tc_fence_after();
         return ok;
     }
-    // Waits for the accumulator and for the per-column constants of the bt-th B tile, lane by lane: only for an epilogue whose lanes
-    // stay in step whatever their waits return, until pair_meet has told all of them.
+    // Waits for the accumulator and, where tiles carry per-column constants (bt >= 0), for those of the bt-th B tile, lane by lane:
+    // only for an epilogue whose lanes stay in step whatever their waits return, until pair_meet has told all of them.
     static __device__ __forceinline__ bool quad_extra_wait_lanes(const Ctx &c, int k, int bt, int *status) {
-        const bool ok = tc::mbar_wait(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1, c.abort_flag, status) &&
+        const bool ok = (bt < 0 || tc::mbar_wait(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1, c.abort_flag, status)) &&
                         tc::mbar_wait(c.bar(kBarAccFull + 2 * c.group + c.colhalf), k & 1, c.abort_flag, status);
         tc::tc_fence_after();
         return ok;
@@ -361,18 +376,7 @@ struct Skel {
     }
     // Meeting point of the two warps that share rows, with a vote: returns whether either warp has given up on a wait, so that both leave
     // the item loop together and neither is left alone at the next meeting.
-    static __device__ __forceinline__ bool pair_meet(const Ctx &c, bool gave_up) {
-        uint32_t any;
-        asm volatile(
-            "{\n\t.reg .pred p, q;\n\t"
-            "setp.ne.u32 q, %1, 0;\n\t"
-            "barrier.cta.red.or.pred p, %2, 64, q;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(any)
-            : "r"((uint32_t)gave_up), "r"(1 + c.group * 4 + c.quarter)
-            : "memory");
-        return any != 0;
-    }
+    static __device__ __forceinline__ bool pair_meet(const Ctx &c, bool gave_up) { return meet_vote(1 + c.group * 4 + c.quarter, 64, gave_up); }
 };
 
 using Big = Skel<256, 1, 2>;       // long B streams

@@ -1,0 +1,67 @@
+"""Scoring step on the tensor cores (two passes) against the oracle where its ways through a tile part: chunks of 32 keys of one
+modality or of both, a modality that changes inside a word, at a word or at a tile, windows of both modalities, ends of the
+prompt inside a chunk, one to four tiles of proxy rows, and row statistics of so many key chunks that a launch joins them.
+
+Tolerance: an exponential is within 4e-6 of its value (the polynomial quarter; exp2.approx is closer) and enters numerator and
+normaliser, logits of a few units in fp32 add less than 1e-6, sums of fp32 parts another 1e-6: importances within 1e-5 relative, a
+row's share of its mass within 1e-5 of the row's mass 1, a head's mass of W rows within 1e-5 W."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import flowmm_oracle as O
+from paper_2511_05534_b200 import binding as F
+from paper_2511_05534_b200 import inputs
+
+from gpu_util import gpu_params, to_dev
+
+pytestmark = pytest.mark.gpu
+
+PATTERNS = {
+    "one": lambda rng, L: np.ones(L),
+    "none": lambda rng, L: np.zeros(L),
+    "every_other": lambda rng, L: np.arange(L) % 2,
+    "random": lambda rng, L: rng.random(L) < 0.8,
+    "run_in_word": lambda rng, L: (np.arange(L) >= 41) & (np.arange(L) < L - 75),
+    "runs_of_words": lambda rng, L: np.arange(L) // 32 % 2,
+    "runs_of_tiles": lambda rng, L: np.arange(L) // 256 % 2,
+    "window_of_both": lambda rng, L: np.arange(L) >= L - 20,
+}
+
+
+def _check(rng, U, Hq, Hkv, L, W, modality):
+    p = O.OracleParams(U, Hq, Hkv, 128, L, W, 1)
+    q = inputs.round_to_bf16(rng.standard_normal((U, Hq, W, 128)).astype(np.float32))
+    k = inputs.round_to_bf16(rng.standard_normal((U, Hkv, L, 128)).astype(np.float32))
+    m = np.ascontiguousarray(modality, dtype=np.uint8)
+    imp, cross, _ = O.score(p, q, k, m)
+    fp = gpu_params(p, F.BF16)
+    g_imp = torch.full((U, Hkv, L), float("nan"), device="cuda")
+    g_cross = torch.full((U, Hq), float("nan"), device="cuda")
+    ws = F.alloc_workspace(fp)
+    F.flowmm_score(fp, to_dev(q, F.BF16), to_dev(k, F.BF16), torch.from_numpy(m).cuda(), g_imp, g_cross, ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    g_imp, g_cross = g_imp.cpu().numpy().astype(np.float64), g_cross.cpu().numpy().astype(np.float64)
+    assert np.abs(g_imp / imp - 1).max() < 1e-5
+    assert np.abs(g_cross - cross).max() < 1e-5 * W
+    if m.min() == m.max():
+        assert np.all(g_cross == 0.0)
+
+
+@pytest.mark.parametrize("pattern", sorted(PATTERNS))
+@pytest.mark.parametrize("G,W,L", [(7, 32, 1471), (7, 64, 641), (3, 128, 256), (8, 128, 289), (4, 32, 2049)])
+def test_modality_patterns(pattern, G, W, L):
+    rng = np.random.default_rng(L + G)
+    _check(rng, 2, 2 * G, 2, L, W, np.stack([PATTERNS[pattern](rng, L), rng.random(L) < 0.5]))
+
+
+@pytest.mark.parametrize("L", [64, 65, 95, 96, 97, 255, 257, 511, 513])
+def test_ends_of_the_prompt(L):
+    rng = np.random.default_rng(L)
+    _check(rng, 3, 4, 2, L, 64, rng.random((3, L)) < 0.5)
+
+
+@pytest.mark.parametrize("L", [4096, 4097, 9001])
+def test_many_key_chunks_of_one_head(L):
+    rng = np.random.default_rng(L)
+    _check(rng, 1, 8, 1, L, 64, np.arange(L)[None] // 1000 % 2)
