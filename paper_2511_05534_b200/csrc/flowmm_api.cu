@@ -92,6 +92,8 @@ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // (items = pairs x row tiles), so the bound is generous rather than a grid limit of 65535.
 constexpr int64_t kMaxHeadsPerCall = 1 << 22;
 
+constexpr int kScoreCtas = 148;             // one per SM of a B200
+
 // Where everything lives inside the caller's workspace.  One layout serves every entry point.
 struct Layout {
     size_t status, importance, cross_mass, rho, strategy, retained, evicted, match, match_sim;
@@ -99,7 +101,7 @@ struct Layout {
     size_t cand_k, cand_scale, cand_slot, cand_count, rank, tile_mod, row_all;
     size_t tokmap;             // [UH, L] (slot, weight) of every token position, for the tensor-core merge
     size_t merge_status;       // status word the merge kernels report to (the workspace's own, or one of the merge scratch)
-    int tc_n_qt, tc_n_chunk, tc_tiles_per_chunk;
+    int tc_n_qt, tc_runs, tc_n_part;
     size_t total;
     int n_chunk1, chunk1, n_chunk2, chunk2, max_pieces, max_parts, csr_passes, c_tot, n_rt;
 };
@@ -156,23 +158,15 @@ Layout make_layout(const flowmm_params &p) {
     y.match = take(U * Hkv * E * 4);
     y.match_sim = take(U * Hkv * E * 4);
     y.n_rt = (int)((L + tcs::kItemRows - 1) / tcs::kItemRows);
-    {   // pass 1 of the tensor-core scoring: key chunks of whole 256-key tiles, sized so that the
-        // persistent CTAs (one per SM, 148 on B200) finish their last round together
-        y.tc_n_qt = (int)((G * W + tcs::kItemRows - 1) / tcs::kItemRows);
-        const int key_tiles = (int)((L + tcs::Big::kCols - 1) / tcs::Big::kCols);
-        const long base_items = (long)(U * Hkv) * y.tc_n_qt;
-        double best_cost = 1e300;
-        y.tc_tiles_per_chunk = key_tiles;
-        for (int want = 1; want <= key_tiles; ++want) {
-            const int tpc = (key_tiles + want - 1) / want;
-            const int nc = (key_tiles + tpc - 1) / tpc;
-            const long rounds = (base_items * nc + 147) / 148;
-            const double cost = (double)rounds * (tpc + 0.75);     // 0.75 tile: per-item start-up
-            if (cost < best_cost - 1e-9) { best_cost = cost; y.tc_tiles_per_chunk = tpc; }
-        }
-        y.tc_n_chunk = (key_tiles + y.tc_tiles_per_chunk - 1) / y.tc_tiles_per_chunk;
+    // pass 1 of the tensor-core scoring: the key tiles of all heads in equal runs, one per SM and tile of 256 proxy rows
+    y.tc_n_qt = (int)((G * W + tcs::kItemRows - 1) / tcs::kItemRows);
+    {
+        const size_t tiles = U * Hkv * (size_t)y.n_rt, runs = kScoreCtas > y.tc_n_qt ? kScoreCtas / y.tc_n_qt : 1;
+        y.tc_runs = (int)(tiles < runs ? tiles : runs);
+        const size_t spread = (size_t)y.tc_runs / (U * Hkv) + 2;          // runs that a head's tiles can be in
+        y.tc_n_part = (int)(spread < (size_t)y.n_rt ? spread : (size_t)y.n_rt);
     }
-    const size_t max_chunk1 = (size_t)(y.n_chunk1 > 2 * y.tc_n_chunk ? y.n_chunk1 : 2 * y.tc_n_chunk);   // records of 8 (SIMT) or 16 bytes
+    const size_t max_chunk1 = (size_t)(y.n_chunk1 > 2 * y.tc_n_part ? y.n_chunk1 : 2 * y.tc_n_part);   // records of 8 (SIMT) or 16 bytes
     const size_t max_chunk2 = (size_t)y.n_chunk2 > W ? (size_t)y.n_chunk2 : W > 8 ? W : 8;
     y.row_part = take(U * Hq * W * max_chunk1 * 8);
     y.cross_part = take(U * Hq * max_chunk2 * 4);
@@ -293,7 +287,10 @@ bool use_tc_score(const flowmm_params &p) {
     return use_tc(p) && (p.window == 32 || p.window == 64 || p.window == 128) && gw <= 1024;
 }
 
-constexpr int kMaxRowRecords = 16;          // key chunks of the first scoring pass that the second one joins itself
+// Row records of a head that the CTAs of the second scoring pass join themselves when they come to it; more are joined by a launch
+// in between, which costs 2 to 3 us.  The whole call, us, without and with it: 6 records of 224 rows 36.5, 38.7; 11 of 224 86.0, 86.6;
+// 11 of 512 98.0, 96.8 and 249.5, 248.5.
+constexpr int kMaxHeadRecords = 4096;
 
 flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *q, const void *k, const uint8_t *mod,
                            float *importance, float *cross_mass, void *ws, cudaStream_t st, int *parts_out) {
@@ -302,18 +299,19 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
     a.row_part = at<float4>(ws, y.row_part); a.modality = mod;
     a.importance = importance; a.cross_part = at<float>(ws, y.cross_part); a.status = at<int>(ws, y.status);
     a.Hq = p.n_q_heads; a.Hkv = p.n_kv_heads; a.G = G; a.W = W; a.L = p.seq_len; a.GW = G * W;
-    a.n_qt = y.tc_n_qt; a.n_chunk = y.tc_n_chunk; a.tiles_per_chunk = y.tc_tiles_per_chunk; a.n_rt = y.n_rt;
+    a.n_qt = y.tc_n_qt; a.n_runs1 = y.tc_runs; a.n_part = y.tc_n_part; a.n_rt = y.n_rt;
     a.a_heads = G < tcs::kRows / W ? G : tcs::kRows / W;        // one A half holds 128 proxy rows
     // pass 2 streams the keys as the A operand; with up to 256 proxy rows per KV head the shapes with two A stages keep
     // the key loads in flight across items
     const bool small2 = a.GW <= 128 && W <= 64, resident2 = !small2 && a.GW <= 256;
     const int nb2 = small2 ? tcs::Small::kCols : tcs::Big::kCols;
     a.b_heads = G < nb2 / W ? G : nb2 / W;
-    a.n_items1 = UH * a.n_qt * a.n_chunk; a.n_items2 = UH * a.n_rt;
-    const int grid1 = a.n_items1 < tc::sm_count() ? a.n_items1 : tc::sm_count();
+    a.n_tiles1 = a.n_items2 = UH * a.n_rt;
+    const int grid1 = a.n_runs1 * a.n_qt;
     const int grid2 = a.n_items2 < tc::sm_count() ? a.n_items2 : tc::sm_count();
-    a.by_grid2 = make_fastdiv((uint32_t)grid2);
+    a.by_grid1 = make_fastdiv((uint32_t)grid1); a.by_grid2 = make_fastdiv((uint32_t)grid2);
     a.by_hkv = make_fastdiv((uint32_t)p.n_kv_heads); a.by_rt = make_fastdiv((uint32_t)a.n_rt);
+    a.by_tiles = make_fastdiv((uint32_t)a.n_tiles1);
     const float scale = p.softmax_scale != 0.f ? p.softmax_scale : 1.f / sqrtf((float)p.head_dim);
     a.scale_log2 = scale * kLog2e;
 
@@ -338,13 +336,13 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
         return FLOWMM_ERR_CUDA;
     launch(score_stats_tc_kernel<tcs::Big>, grid1, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
     FLOWMM_LAUNCHED("score_stats_tc");
-    a.row_rec = a.row_part; a.n_rec = a.n_chunk;
-    if (a.n_chunk > kMaxRowRecords) {
+    a.row_all = nullptr;
+    if (a.n_part * a.GW > kMaxHeadRecords) {
         float4 *all = at<float4>(ws, y.row_all);
         const int n_rows = UH * a.GW;
-        launch(score_combine_kernel<4>, (n_rows + 63) / 64, 256, 0, st, a.row_part, a.n_chunk, n_rows, all);
+        launch(score_combine_kernel<4>, (n_rows + 63) / 64, 256, 0, st, a, n_rows, all);
         FLOWMM_LAUNCHED("score_combine");
-        a.row_rec = all; a.n_rec = 1;
+        a.row_all = all;
     }
     if (small2) launch(score_colsum_tc_kernel<tcs::Small>, grid2, tcs::kThreads, tcs::Small::kSmemBytes, st, k128, qb, a);
     else if (resident2) launch(score_colsum_tc_kernel<tcs::Resident>, grid2, tcs::kThreads, tcs::Resident::kSmemBytes, st, k128, qb, a);

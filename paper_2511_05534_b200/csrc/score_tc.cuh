@@ -19,20 +19,20 @@
 namespace flowmm {
 
 struct ScoreTcArgs {
-    float4 *row_part;            // [UH*GW, n_chunk] (max, exp-sum over text keys, exp-sum over visual keys, -) per proxy row and key chunk, log2 domain
-    const float4 *row_rec;       // [UH*GW, n_rec] what pass 2 reads: row_part itself, or its records joined to one per row
-    int n_rec;
+    float4 *row_part;            // [UH*GW, n_part] (max, exp-sum over text keys, exp-sum over visual keys, -) per proxy row and run that its keys are in, log2 domain
+    int n_part;                  // runs a head's key tiles can be spread over
+    const float4 *row_all;       // nullptr, or [UH*GW] the records of row_part joined to one per row, which pass 2 then reads
     const uint8_t *modality;     // [U, L]
     float *importance;           // [UH, L]
     float *cross_part;           // [U*Hq, W] share of a proxy row's mass that falls on keys of the other modality
     int *status;
     int Hq, Hkv, G, W, L, GW;
     int n_qt;                    // 256-row tiles over the G*W proxy rows
-    int n_chunk, tiles_per_chunk;   // pass 1: key chunks per row tile, 256-key tiles per chunk
-    FastDiv by_grid2, by_hkv, by_rt;   // exact divisions by the second pass's grid, Hkv, n_rt
-    int n_rt;                    // pass 2: 256-key tiles
+    int n_runs1;                 // pass 1: runs that the key tiles of all heads are cut into
+    FastDiv by_grid1, by_grid2, by_hkv, by_rt, by_tiles;   // exact divisions by the passes' grids, Hkv, n_rt, n_tiles1
+    int n_rt;                    // 256-key tiles of a head
     int a_heads, b_heads;        // query heads one A box (pass 1) / B box (pass 2) delivers
-    int n_items1, n_items2;
+    int n_tiles1, n_items2;      // key tiles of all heads, for either pass
     float scale_log2;
 };
 
@@ -149,6 +149,14 @@ __device__ __forceinline__ float sum32_of(const uint32_t (&a)[32], uint32_t vis,
     return (v01.x + v01.y) + (v23.x + v23.y);
 }
 
+// Run `r` of n: tiles [run_start(r), run_start(r + 1)) of the n_tiles of all heads; and the run that holds tile x.
+__device__ __forceinline__ int run_start(int n_tiles, int n, int r) { return (int)((int64_t)n_tiles * r / n); }
+__device__ __forceinline__ int run_of(const ScoreTcArgs &A, int x) {
+    const uint64_t v = ((uint64_t)x + 1) * (uint32_t)A.n_runs1 - 1;
+    return v >> 32 ? (int)(v / (uint32_t)A.n_tiles1) : (int)A.by_tiles.div((uint32_t)v);
+}
+__device__ __forceinline__ int runs_of_head(const ScoreTcArgs &A, int uh) { return run_of(A, (uh + 1) * A.n_rt - 1) - run_of(A, uh * A.n_rt) + 1; }
+
 // A proxy row's statistics over some keys: running maximum, exp-sums over the text and over the visual keys.
 struct RowStats { float m, t, v; };
 __device__ __forceinline__ RowStats join(const RowStats &a, const RowStats &b) {
@@ -161,7 +169,11 @@ __device__ __forceinline__ RowStats join(const RowStats &a, const RowStats &b) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Pass 1.  item = (unit*head, tile of 256 proxy rows, key chunk).
+// Pass 1.  The 256-key tiles of all heads, one head's behind the other's, are cut into equal runs; a CTA takes a run for one tile
+// of 256 proxy rows (CTAs next to each other share a run, whose keys the second of them finds in L2).  item = a run's part of one
+// head.  Whole heads or equal chunks of them as items left SMs idle in the last round.  The whole call, us, so and now: 112 heads of
+// 2176 tokens, 224 rows 116.1 / 111.9; of 8448, 448 rows 867 / 851; 112 caches of 640 rows 97.9 / 95.6; 80 heads of 7906, 512
+// rows 419 / 394; 128 of 33 792 2947 / 2904.
 // The exp-sums are kept by modality of the key: what pass 2 had to split off its probabilities, per query head and with a sum
 // over the warp for each, costs nothing here where a warp's 64 keys of a tile are of one modality and seen by every row, as
 // nearly always (images are runs of tokens): one of the two sums grows, and they change places when the modality does.  128
@@ -177,26 +189,27 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const typename S::Ctx c = S::setup(smem_raw, &q_map, &k_map, A.status, 0, 16);
     if (!c.ok) return;
+    const int run = (int)blockIdx.x / A.n_qt, qt = (int)blockIdx.x - run * A.n_qt;
+    const int t_lo = run_start(A.n_tiles1, A.n_runs1, run), t_hi = run_start(A.n_tiles1, A.n_runs1, run + 1);
+    const int uh_lo = (int)A.by_rt.div(t_lo), n_loop = ((int)A.by_rt.div(t_hi - 1) - uh_lo + 1) * gridDim.x;   // the roles count items blockIdx.x, blockIdx.x + gridDim.x, ...
     auto plan = [&](int item) {
         tcs::TilePlan p;
-        const int kc = item % A.n_chunk, qt = (item / A.n_chunk) % A.n_qt, uh = item / (A.n_chunk * A.n_qt);
-        const int u = uh / A.Hkv, h = uh % A.Hkv;
-        const int key0 = kc * A.tiles_per_chunk * S::kCols;
-        const int keys = min(A.L - key0, A.tiles_per_chunk * S::kCols);
+        const int uh = uh_lo + (int)A.by_grid1.div(item), u = (int)A.by_hkv.div(uh), h = uh - u * A.Hkv, head0 = uh * A.n_rt;
+        const int t0 = max(t_lo, head0) - head0, t1 = min(t_hi, head0 + A.n_rt) - head0;
         p.a1 = 0; p.a2 = h * A.G + qt * (tcs::kItemRows / A.W); p.a3 = u;
         p.h1 = 0; p.h2 = tcs::kRows / A.W;
         p.n_halves = qt * tcs::kItemRows + tcs::kRows < A.GW ? 2 : 1;
-        p.b1 = key0; p.b2 = h; p.b3 = u; p.step1 = S::kCols; p.step2 = 0;
-        p.cols_total = keys > 0 ? keys : 0;
-        p.n_tiles = (p.cols_total + S::kCols - 1) / S::kCols;
+        p.b1 = t0 * S::kCols; p.b2 = h; p.b3 = u; p.step1 = S::kCols; p.step2 = 0;
+        p.cols_total = min(A.L, t1 * S::kCols) - p.b1;
+        p.n_tiles = t1 - t0;
         p.extra = nullptr;
         return p;
     };
     const uint32_t a_bytes = (uint32_t)A.a_heads * A.W * 256u;
     if (c.warp == 0) {
-        S::producer(c, &q_map, &k_map, A.n_items1, a_bytes, S::kBStage, plan, A.status);
+        S::producer(c, &q_map, &k_map, blockIdx.x + n_loop, a_bytes, S::kBStage, plan, A.status);
     } else if (c.warp == 1) {
-        S::template mma_issuer<false>(c, A.n_items1, plan, A.status);
+        S::template mma_issuer<false>(c, blockIdx.x + n_loop, plan, A.status);
     } else {
         // all sixteen warps drain one accumulator at a time: a warp owns 32 lanes x a quarter of the columns of
         // BOTH halves, so the tensor core refills one half while the other is being read
@@ -222,17 +235,17 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
             mod_at += S::kCols;
         };
         auto first_mod = [&](int item) {
-            if (item >= A.n_items1) return;
+            if (item >= (int)blockIdx.x + n_loop) return;
             const tcs::TilePlan p = plan(item);
             mod_end = A.modality + (int64_t)(p.b3 + 1) * A.L - 1;
             mod_at = mod_end + (p.b1 + colq * 64 + c.lane - A.L + 1);
             fetch_mod();
         };
         first_mod(blockIdx.x);
-        for (int item = blockIdx.x; item < A.n_items1; item += gridDim.x) {
+        // runs of a head before this CTA's: none, unless it begins inside the head
+        int part = run - run_of(A, uh_lo * A.n_rt), uh = uh_lo;
+        for (int item = blockIdx.x; item < (int)blockIdx.x + n_loop; item += gridDim.x, ++uh, part = 0) {
             const tcs::TilePlan p = plan(item);
-            if (p.empty()) continue;                                     // (never: every chunk holds keys)
-            const int kc = item % A.n_chunk, qt = (item / A.n_chunk) % A.n_qt, uh = item / (A.n_chunk * A.n_qt);
             RowStats st[2] = {{kNegBig, 0.f, 0.f}, {kNegBig, 0.f, 0.f}};
             bool swapped = false;                                        // st[].t belongs to the visual keys and st[].v to the text keys
             for (int t = 0; t < p.n_tiles; ++t) {
@@ -308,7 +321,7 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
                     const RowStats o = {tc::lds32(at), tc::lds32(at + 4), tc::lds32(at + 8)};
                     s = join(s, o);
                 }
-                A.row_part[((int64_t)uh * A.GW + r) * A.n_chunk + kc] = make_float4(s.m, s.t, s.v, 0.f);
+                A.row_part[((int64_t)uh * A.GW + r) * A.n_part + part] = make_float4(s.m, s.t, s.v, 0.f);
             }
             turn ^= kMeetBytes;
         }
@@ -326,24 +339,25 @@ __global__ void pack_modality_kernel(const uint8_t *modality, int L, int n_words
     if (lane == 0) bits[(int64_t)u * n_words + w] = word;
 }
 
-// Joins a row's statistics over n_part key chunks to one record, where pass 2 would have to read many of them for each of its
-// heads: kLanes lanes share a row and read its parts together.
+// Joins the records of a row to one, where pass 2 would have to read many of them for each of its heads: kLanes lanes share a row
+// and read its records together.
 template <int kLanes>
-__global__ void score_combine_kernel(const float4 *row_part, int n_part, int n_rows, float4 *row_all) {
+__global__ void score_combine_kernel(const ScoreTcArgs A, int n_rows, float4 *row_all) {
     predecessor_done();
     const int i = blockIdx.x * (blockDim.x / kLanes) + threadIdx.x / kLanes, sub = threadIdx.x % kLanes;
     const bool on = i < n_rows;
-    const float4 *part = row_part + (int64_t)i * n_part;
+    const int n = runs_of_head(A, on ? i / A.GW : 0);
+    const float4 *part = A.row_part + (int64_t)i * A.n_part;
     float mx = kNegBig, t = 0.f, v = 0.f;
     if (on) {
 #pragma unroll 4
-        for (int c = sub; c < n_part; c += kLanes) mx = fmaxf(mx, part[c].x);
+        for (int c = sub; c < n; c += kLanes) mx = fmaxf(mx, part[c].x);
     }
 #pragma unroll
     for (int o = kLanes / 2; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
     if (on) {
 #pragma unroll 4
-        for (int c = sub; c < n_part; c += kLanes) {
+        for (int c = sub; c < n; c += kLanes) {
             const float4 p = part[c];
             const float w = exp2f(p.x - mx);
             t += p.y * w; v += p.z * w;
@@ -404,7 +418,6 @@ __device__ __forceinline__ void colsum_chunk32(uint32_t (&a)[32], uint32_t negc,
 // consecutive items, so that proxy rows that fit the B stages (up to 512) are loaded once per head, not once per item.
 // Row constants -(max + log2 sum) - exp2(logit + constant) is the softmax probability - are formed from pass 1's statistics by
 // the epilogue warps when the run comes to another head; the CTA with a head's first tile also writes its rows' cross-modal shares.
-// (A launch of its own for the constants took 3 us: 8 heads of 1471 tokens 39.0 -> 36.2 us for the call, 112 of 2176 121 -> 116.)
 // Bound by the epilogue (four warps per scheduler, the exp2 unit at 0.69 of its rate, 0.56 before the masses went to pass 1): a
 // chunk is read while the one before it is worked on, an accumulator is handed back as soon as its last chunk is in registers,
 // and no vote or shuffle stands between: 197 -> 152 instructions per chunk of 32 columns.  (Three or four words a thread of
@@ -455,26 +468,31 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
             const int uh0 = uh, kt0 = kt;                            // this item
             if (g == g_lo || kt0 == 0) {                             // a new head: its row constants
                 consts ^= (c.base + S::kSmemEpi) ^ (c.base + S::kSmemEpi + kConstBytes);
+                const int n_rec = A.row_all ? 1 : runs_of_head(A, uh0);
                 for (int r = te; r < A.GW; r += 32 * tcs::kEpiWarps) {
-                    const float4 *rec = A.row_rec + ((int64_t)uh0 * A.GW + r) * A.n_rec;
-                    float4 s = rec[0];
-#pragma unroll 4
-                    for (int i = 1; i < A.n_rec; ++i) s.x = fmaxf(s.x, rec[i].x);
-                    if (A.n_rec > 1) {
-                        const float mx = s.x;
-                        s.y = 0.f; s.z = 0.f;
-#pragma unroll 4
-                        for (int i = 0; i < A.n_rec; ++i) {
-                            const float4 o = rec[i];
-                            const float w = exp2f(o.x - mx);
-                            s.y += o.y * w; s.z += o.z * w;
+                    const int64_t i0 = (int64_t)uh0 * A.GW + r;
+                    const float4 *rec = A.row_all ? A.row_all + i0 : A.row_part + i0 * A.n_part;
+                    RowStats s = {kNegBig, 0.f, 0.f};
+                    for (int i = 0; i < n_rec; i += 8) {             // eight records on their way together
+                        float4 o[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) o[e] = i + e < n_rec ? rec[i + e] : make_float4(kNegBig, 0.f, 0.f, 0.f);
+                        const float m0 = s.m;
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) s.m = fmaxf(s.m, o[e].x);
+                        const float w0 = exp2f(m0 - s.m);
+                        s.t *= w0; s.v *= w0;
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const float w = exp2f(o[e].x - s.m);
+                            s.t += o[e].y * w; s.v += o[e].z * w;
                         }
                     }
-                    const float z = s.y + s.z;
-                    tc::sts32(consts + r * 4, -(s.x + log2f(z)));
+                    const float z = s.t + s.v;
+                    tc::sts32(consts + r * 4, -(s.m + log2f(z)));
                     if (kt0 == 0) {                                  // (one CTA per head)
                         const bool vis = A.modality[(int64_t)u * A.L + A.L - A.W + (r & (A.W - 1))] != 0;   // (the window is 32, 64 or 128 rows)
-                        A.cross_part[((int64_t)u * A.Hq + hk * A.G) * A.W + r] = (vis ? s.y : s.z) / z;
+                        A.cross_part[((int64_t)u * A.Hq + hk * A.G) * A.W + r] = (vis ? s.t : s.v) / z;
                     }
                 }
                 // (the set written was read two heads ago, and every warp has been through the meeting of the head between)

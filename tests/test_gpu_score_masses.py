@@ -61,6 +61,13 @@ def test_ends_of_the_prompt(L):
     _check(rng, 3, 4, 2, L, 64, rng.random((3, L)) < 0.5)
 
 
+@pytest.mark.parametrize("U,G,W,L", [(37, 12, 64, 600), (150, 3, 32, 200), (299, 2, 64, 257), (5, 4, 64, 2600), (1, 7, 32, 5000)])
+def test_runs_of_tiles_across_heads(U, G, W, L):
+    """Runs that hold many heads, end inside heads, and heads spread over many runs, with one to three tiles of proxy rows."""
+    rng = np.random.default_rng(U)
+    _check(rng, U, G, 1, L, W, np.arange(L)[None] // 100 % 2 ^ rng.integers(0, 2, (U, 1)))
+
+
 @pytest.mark.parametrize("L", [4096, 4097, 9001])
 def test_many_key_chunks_of_one_head(L):
     rng = np.random.default_rng(L)
