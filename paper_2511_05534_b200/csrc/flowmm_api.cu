@@ -98,12 +98,12 @@ constexpr int kScoreCtas = 148;             // one per SM of a B200
 struct Layout {
     size_t status, importance, cross_mass, rho, strategy, retained, evicted, match, match_sim;
     size_t row_part, cross_part, sort_a, sort_b, mem_tok, mem_w, piece_desc, off, piece_off, part_off, partial, ticket, slot_done;
-    size_t cand_k, cand_scale, cand_slot, cand_count, rank, tile_mod, row_all;
+    size_t cand_k, cand_scale, cand_slot, cand_count, rank, evi_mod, tile_mod, row_all;
     size_t tokmap;             // [UH, L] (slot, weight) of every token position, for the tensor-core merge
     size_t merge_status;       // status word the merge kernels report to (the workspace's own, or one of the merge scratch)
     int tc_n_qt, tc_runs, tc_n_part;
     size_t total;
-    int n_chunk1, chunk1, n_chunk2, chunk2, max_pieces, max_parts, csr_passes, c_tot, n_rt;
+    int n_chunk1, chunk1, n_chunk2, chunk2, max_pieces, max_parts, csr_passes, c_tot, n_rt, n_et;
 };
 
 int chunks_for(int L, int other_ctas, int &chunk) {
@@ -179,7 +179,9 @@ Layout make_layout(const flowmm_params &p) {
     y.cand_slot = take(U * Hkv * (size_t)y.c_tot * 4);
     y.cand_count = take(U * Hkv * 2 * 4);
     y.rank = take(U * Hkv * L * 4);
-    y.tile_mod = take(U * (size_t)y.n_rt);
+    y.evi_mod = take(U * Hkv * E);
+    y.n_et = (int)((E + kMtItemRows - 1) / kMtItemRows);
+    y.tile_mod = take(U * Hkv * (size_t)y.n_et);
     y.total = o;
     return y;
 }
@@ -452,8 +454,8 @@ MatchPrepArgs match_prep_args(const flowmm_params &p, const Layout &y, const voi
     g.retained = retained; g.evicted = evicted;
     g.cand_k = at<__nv_bfloat16>(ws, y.cand_k); g.cand_scale = at<float>(ws, y.cand_scale);
     g.cand_slot = at<int>(ws, y.cand_slot); g.cand_count = at<int>(ws, y.cand_count);
-    g.rank = at<int>(ws, y.rank); g.tile_mod = at<uint8_t>(ws, y.tile_mod);
-    g.Hkv = p.n_kv_heads; g.L = p.seq_len; g.B = p.n_keep; g.E = p.seq_len - p.n_keep; g.Ctot = y.c_tot; g.n_rt = y.n_rt;
+    g.rank = at<int>(ws, y.rank); g.evi_mod = at<uint8_t>(ws, y.evi_mod); g.tile_mod = at<uint8_t>(ws, y.tile_mod);
+    g.Hkv = p.n_kv_heads; g.L = p.seq_len; g.B = p.n_keep; g.E = p.seq_len - p.n_keep; g.Ctot = y.c_tot; g.n_rt = y.n_et;
     g.tau_eff = tau_effective(p);
     for (int i = 0; i < 3; ++i) g.ks[i] = p.k_stride[i];
     g.copy_here = y.c_tot <= 256;
@@ -542,21 +544,21 @@ flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *
         FLOWMM_LAUNCHED("match_small_tc");
         return FLOWMM_OK;
     }
-    const uint32_t box_a[4] = {64, kMtRows, 1, 1};
     const uint32_t box_b[4] = {64, tcs::Big::kCols, 1, 1};
-    if (!tc::make_bf16_map(&k_map, k, 4, kd, ks, box_a) || !tc::make_bf16_map(&cand_map, g.cand_k, 4, cd, cs, box_b))
-        return FLOWMM_ERR_CUDA;
+    if (!tc::make_bf16_map(&cand_map, g.cand_k, 4, cd, cs, box_b)) return FLOWMM_ERR_CUDA;
     MatchTcArgs a;
-    a.cand_count = g.cand_count; a.cand_slot = g.cand_slot; a.rank = g.rank; a.strategy = strategy;
-    a.cand_scale = g.cand_scale; a.modality = mod; a.tile_mod = g.tile_mod;
+    a.cand_count = g.cand_count; a.cand_slot = g.cand_slot; a.evicted = evicted; a.strategy = strategy;
+    a.cand_scale = g.cand_scale; a.evi_mod = g.evi_mod; a.tile_mod = g.tile_mod;
     a.match = match; a.match_sim = match_sim; a.status = at<int>(ws, y.status);
-    a.Hkv = p.n_kv_heads; a.L = p.seq_len; a.E = E; a.Ctot = y.c_tot; a.n_rt = y.n_rt; a.n_items = UH * y.n_rt;
-    a.by_nrt = make_fastdiv((uint32_t)y.n_rt); a.by_hkv = make_fastdiv((uint32_t)p.n_kv_heads);
+    a.Hkv = p.n_kv_heads; a.L = p.seq_len; a.E = E; a.Ctot = y.c_tot; a.n_rt = y.n_et; a.n_items = UH * y.n_et;
+    a.k = static_cast<const __nv_bfloat16 *>(k);
+    a.k_unit = p.k_stride[0]; a.k_head = p.k_stride[1]; a.row_bytes = (uint32_t)(p.k_stride[2] * 2);
+    a.by_nrt = make_fastdiv((uint32_t)y.n_et); a.by_hkv = make_fastdiv((uint32_t)p.n_kv_heads);
     if (cudaFuncSetAttribute(match_tc_kernel<tcs::Big>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)tcs::Big::kSmemBytes) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
     const int grid = a.n_items < tc::sm_count() ? a.n_items : tc::sm_count();
-    launch(match_tc_kernel<tcs::Big>, grid, tcs::kThreads, tcs::Big::kSmemBytes, st, k_map, cand_map, a);
+    launch(match_tc_kernel<tcs::Big>, grid, kMtThreads, tcs::Big::kSmemBytes, st, cand_map, a);
     FLOWMM_LAUNCHED("match_tc");
     return FLOWMM_OK;
 }

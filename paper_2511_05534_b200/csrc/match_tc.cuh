@@ -3,11 +3,14 @@
 // Per (unit, KV head) the admissible pivots (importance <= tau) are gathered into a dense
 // candidate matrix, text candidates first and visual candidates from the next multiple of 32.
 // The similarity contraction then runs as  S[128 tokens x 256 candidates] = K_tile . C_tile^T
-// (two such 128-token halves per candidate tile) on tcgen05 with the token rows taken straight from the caller's K by TMA (every token of the
-// head in prompt order; rows that are pivots are computed and dropped), fp32 accumulators in
-// TMEM, and an epilogue that scales each column by the candidate's reciprocal norm and keeps a
-// running row maximum.  Raw bf16 keys feed the MMA (their products are exact in fp32); the
-// norms enter in fp32 afterwards, so no precision is lost before the argmax.
+// (two such 128-token halves per candidate tile) on tcgen05, fp32 accumulators in TMEM, and an epilogue that scales each column
+// by the candidate's reciprocal norm and keeps a running row maximum.  Raw bf16 keys feed the MMA (their products are exact in
+// fp32); the norms enter in fp32 afterwards, so no precision is lost before the argmax.
+// The token rows are the non-pivots alone, gathered from the caller's K by two warps of their own.  (Tiles of consecutive tokens,
+// which the TMA unit can load, computed the pivots as well, only to drop them.  The whole call, us, so and now: 112 heads of 8448
+// tokens with 1690 pivots 843 / 771, 112 of 640 with 423 95.2 / 87.5, 64 of 2407 with 1441 166 / 134; 128 of 33 792 with 1690
+// 2860 / 2839.  Gathered copies by the TMA unit, four rows to one, are bit for bit the same and slower with few pivots: 256 rows took
+// 3 us more than the two warps, which these hide behind the item before.)
 // An intra-modal layer visits only the candidate group of the row tile's modality.
 #pragma once
 #include <type_traits>
@@ -29,8 +32,11 @@ struct MatchPrepArgs {
     float *cand_scale;           // [UH, Ctot]
     int *cand_slot;              // [UH, Ctot]
     int *cand_count;             // [UH, 2]  admissible text / visual pivots
+    // what the matching kernel reads per token: the one for short candidate lists (copy_here) the rank of every token,
     int *rank;                   // [UH, L]  position in the non-pivot list, or -(s + 2) for the pivot of slot s
-    uint8_t *tile_mod;           // [U, n_rt] per tile of 256 tokens; bit 0: holds text tokens, bit 1: visual tokens
+    // the general one, by position in the non-pivot list,
+    uint8_t *evi_mod;            // [UH, E]  the token's modality
+    uint8_t *tile_mod;           // [UH, n_rt] per tile of 256 positions; bit 0: holds text tokens, bit 1: visual tokens
     int Hkv, L, B, E, Ctot, n_rt;
     int *status;                 // device status word (index checks of the debug build report here)
     int copy_here;               // 1: this kernel also gathers the candidate rows; 0: match_gather_kernel does
@@ -131,9 +137,10 @@ __device__ __forceinline__ void match_lay_out_candidates(const MatchPrepArgs &A,
 
 // The preparation of flowmm_match, which is handed the index lists (inside flowmm_compress_layer and flowmm_recompress the
 // selection kernel lays everything out itself).  grid = (U*Hkv, 1 + parts), block = 512: blocks y = 0 lay out a head's
-// candidates, the others write the rank of every token and the tiles' modalities, a slice each.
+// candidates, the others write what the matching kernel reads per token, a slice each.
 constexpr int kPrepThreads = 512;
-constexpr int kPrepSlice = 8 * kPrepThreads;                   // list entries of a rank block: eight loads in flight per thread
+constexpr int kPrepSlice = 8 * kPrepThreads;                   // list entries of such a block: eight loads in flight per thread
+static_assert(kPrepSlice % kMtItemRows == 0 && kPrepThreads % kMtItemRows == 0, "a slice is whole tiles, a step as well");
 __global__ void __launch_bounds__(kPrepThreads) match_prepare_kernel(const MatchPrepArgs A) {
     __shared__ int scratch[33];
     predecessor_done();
@@ -142,33 +149,50 @@ __global__ void __launch_bounds__(kPrepThreads) match_prepare_kernel(const Match
     const int part = blockIdx.y - 1, parts = gridDim.y - 1;
     const int *ret = A.retained + (int64_t)uh * A.B;
     const int *evi = A.evicted + (int64_t)uh * A.E;
-    int *rank = A.rank + (int64_t)uh * A.L;
-    for (int i0 = part * kPrepSlice; i0 < A.L; i0 += parts * kPrepSlice) {   // entries of the two lists, pivots first
-        int tok[8];
+    if (A.copy_here) {
+        int *rank = A.rank + (int64_t)uh * A.L;
+        for (int i0 = part * kPrepSlice; i0 < A.L; i0 += parts * kPrepSlice) {   // entries of the two lists, pivots first
+            int tok[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int i = i0 + e * kPrepThreads + tid;
-            tok[e] = i < A.B ? ret[i] : i < A.L ? evi[i - A.B] : -1;
-        }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int i = i0 + e * kPrepThreads + tid;
-            if (i < A.L && index_ok(tok[e], A.L, A.status)) rank[tok[e]] = i < A.B ? -(i + 2) : i - A.B;
-        }
-    }
-    if (uh % A.Hkv == 0) {
-        const int u = uh / A.Hkv, lane = tid & 31, n_warps = kPrepThreads / 32;
-        const uint8_t *mod = A.modality + (int64_t)u * A.L;
-        for (int t = part * n_warps + (tid >> 5); t < A.n_rt; t += parts * n_warps) {
-            bool any_t = false, any_v = false;
-#pragma unroll
-            for (int q = 0; q < kMtItemRows / 32; ++q) {
-                const int i = t * kMtItemRows + q * 32 + lane;
-                if (i < A.L) { if (mod[i]) any_v = true; else any_t = true; }
+            for (int e = 0; e < 8; ++e) {
+                const int i = i0 + e * kPrepThreads + tid;
+                tok[e] = i < A.B ? ret[i] : i < A.L ? evi[i - A.B] : -1;
             }
-            any_t = __any_sync(0xFFFFFFFFu, any_t); any_v = __any_sync(0xFFFFFFFFu, any_v);
-            if (lane == 0) A.tile_mod[(int64_t)u * A.n_rt + t] = (uint8_t)((any_t ? 1 : 0) | (any_v ? 2 : 0));
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int i = i0 + e * kPrepThreads + tid;
+                if (i < A.L && index_ok(tok[e], A.L, A.status)) rank[tok[e]] = i < A.B ? -(i + 2) : i - A.B;
+            }
         }
+        return;
+    }
+    const uint8_t *mod = A.modality + (int64_t)(uh / A.Hkv) * A.L;
+    for (int j0 = part * kPrepSlice; j0 < A.E; j0 += parts * kPrepSlice) {
+        int tok[8];
+        uint8_t m[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int j = j0 + e * kPrepThreads + tid;
+            tok[e] = j < A.E ? evi[j] : -1;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) m[e] = tok[e] >= 0 && index_ok(tok[e], A.L, A.status) ? mod[tok[e]] : 0;
+        if (tid < 2 * kPrepSlice / kMtItemRows) scratch[tid] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int j = j0 + e * kPrepThreads + tid, t = (j - j0) / kMtItemRows;
+            if (j < A.E) A.evi_mod[(int64_t)uh * A.E + j] = m[e] != 0;
+            const bool any_t = __any_sync(0xFFFFFFFFu, j < A.E && m[e] == 0), any_v = __any_sync(0xFFFFFFFFu, j < A.E && m[e] != 0);
+            if ((tid & 31) == 0) {
+                if (any_t) scratch[2 * t] = 1;
+                if (any_v) scratch[2 * t + 1] = 1;
+            }
+        }
+        __syncthreads();
+        const int t = j0 / kMtItemRows + tid;
+        if (tid < kPrepSlice / kMtItemRows && t < A.n_rt) A.tile_mod[(int64_t)uh * A.n_rt + t] = (uint8_t)(scratch[2 * tid] | scratch[2 * tid + 1] << 1);
+        __syncthreads();
     }
 }
 
@@ -181,13 +205,16 @@ __global__ void __launch_bounds__(256) match_gather_kernel(const MatchPrepArgs A
 }
 
 struct MatchTcArgs {
-    const int *cand_count, *cand_slot, *rank, *strategy;
+    const int *cand_count, *cand_slot, *evicted, *strategy;
     const float *cand_scale;
-    const uint8_t *modality, *tile_mod;
+    const uint8_t *evi_mod, *tile_mod;
     int *match;
     float *match_sim;
     int *status;
     int Hkv, L, E, Ctot, n_rt, n_items;
+    const __nv_bfloat16 *k;
+    int64_t k_unit, k_head;      // strides in elements
+    uint32_t row_bytes;          // stride of the tokens (32 bits: more than 224 rows of 4 GB each are no GPU's)
     FastDiv by_nrt, by_hkv;      // exact division of item numbers by n_rt and of head numbers by Hkv
 };
 
@@ -207,7 +234,7 @@ __device__ __forceinline__ MatchRaw match_raw(const MatchTcArgs &A, int item) {
     r.uh = (int)A.by_nrt.div(item); r.rt = item - r.uh * A.n_rt; r.u = (int)A.by_hkv.div(r.uh);
     r.n_text = A.cand_count[2 * r.uh]; r.n_vis = A.cand_count[2 * r.uh + 1];
     r.strategy = A.strategy[r.u];
-    r.tile_mod = A.tile_mod[(int64_t)r.u * A.n_rt + r.rt];
+    r.tile_mod = A.tile_mod[item];
     return r;
 }
 
@@ -228,9 +255,8 @@ __device__ __forceinline__ MatchItem match_plan(const MatchTcArgs &A, const Matc
     else if (tm == 1) { p.lo = 0; p.hi = p.n_text; }
     else { p.lo = p.t0; p.hi = p.t0 + p.n_vis; }
     const int cols = p.hi > p.lo ? p.hi - p.lo : 0;
-    p.tp.a1 = p.rt * kMtItemRows; p.tp.a2 = p.h; p.tp.a3 = p.u;
-    p.tp.h1 = kMtRows; p.tp.h2 = 0;
-    p.tp.n_halves = p.tp.a1 + kMtRows < A.L ? 2 : 1;
+    p.tp.a1 = p.rt * kMtItemRows;                                // first position in the non-pivot list
+    p.tp.n_halves = p.tp.a1 + kMtRows < A.E ? 2 : 1;
     p.tp.b1 = p.lo; p.tp.b2 = p.uh; p.tp.b3 = 0;
     p.tp.step1 = kMtCols; p.tp.step2 = 0;
     p.tp.n_tiles = (cols + kMtCols - 1) / kMtCols;
@@ -378,19 +404,60 @@ __device__ __forceinline__ float row_half_ssq(uint32_t row_addr, int row) {
     return acc.x + acc.y;
 }
 
-// Persistent kernel, one CTA per SM; item = (unit, head, tile of 256 tokens).
+// Persistent kernel, one CTA per SM; item = (unit, head, tile of 256 non-pivots).
+constexpr int kMtThreads = tcs::kThreads + 64;
 template <class S>
-__global__ void __launch_bounds__(tcs::kThreads, 1)
-match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap cand_map,
-                const MatchTcArgs A) {
+__global__ void __launch_bounds__(kMtThreads, 1)
+match_tc_kernel(const __grid_constant__ CUtensorMap cand_map, const MatchTcArgs A) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     constexpr int kMtCols = S::kCols;
     constexpr int kPer = kMtCols / 32;                           // blocks of 16 columns a warp takes of a full tile
-    const typename S::Ctx c = S::setup(smem_raw, &k_map, &cand_map, A.status, 8);
+    const typename S::Ctx c = S::setup(smem_raw, &cand_map, &cand_map, A.status, 8);
     if (!c.ok) return;
     auto plan = [&](int item) { return match_plan<S>(A, item).tp; };
     if (c.warp == 0) {
-        S::producer(c, &k_map, &cand_map, A.n_items, tcs::kAHalf, S::kBStage, plan, A.status);
+        S::template producer<false>(c, nullptr, &cand_map, A.n_items, 0, S::kBStage, plan, A.status);
+    } else if (c.warp >= tcs::kThreads / 32) {
+        // A warp per half gathers its 128 rows, two to an instruction: lanes 0-15 and 16-31 take 16 bytes each of a row, to where the
+        // 128-byte swizzle puts them.  The rows' tokens are fetched an item ahead (rows past the list's end repeat its last).
+        const int h = c.warp - tcs::kThreads / 32, odd = c.lane >> 4, unit = c.lane & 15;
+        const uint32_t dst = c.a_addr_of(h) + (uint32_t)(unit >> 3) * (tcs::kAHalf / 2) + (uint32_t)odd * 128;
+        uint32_t at[4];                                              // rows 2 i + odd, i = 0 .. 3, of a group of eight
+#pragma unroll
+        for (int i = 0; i < 4; ++i) at[i] = dst + (uint32_t)i * 256 + (uint32_t)(((unit & 7) ^ (2 * i + odd)) << 4);
+        int tok[4] = {0, 0, 0, 0}, n = 0;
+        auto fetch_tokens = [&](int item) {
+            if (item >= A.n_items) return;
+            const int uh = (int)A.by_nrt.div(item), j0 = (item - uh * A.n_rt) * kMtItemRows + h * kMtRows + c.lane;
+            const int *evi = A.evicted + (int64_t)uh * A.E;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                tok[q] = evi[min(j0 + 32 * q, A.E - 1)];
+                if (!index_ok(tok[q], A.L, A.status)) tok[q] = 0;
+            }
+        };
+        fetch_tokens(blockIdx.x);
+        bool ok = true;
+        for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x) {
+            const MatchItem p = match_plan<S>(A, item);
+            if (!p.tp.empty() && h < p.tp.n_halves) {
+                const char *src = reinterpret_cast<const char *>(A.k + p.u * A.k_unit + p.h * A.k_head + unit * 8);
+                ok = tc::mbar_wait_warp(c.bar(S::kBarAEmpty + h), (n & 1) ^ 1, c.abort_flag, A.status);
+                if (!ok) break;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const int t = __shfl_sync(0xFFFFFFFFu, tok[q], 2 * i + odd);
+                        tc::copy16_async(at[i & 3] + (uint32_t)(q * 32 + (i >> 2) * 8) * 128, src + (uint64_t)((uint32_t)t) * A.row_bytes);
+                    }
+                fetch_tokens(item + gridDim.x);
+                tc::copies_landed();
+                __syncwarp();
+                if (c.lane == 0) tc::mbar_arrive(c.bar(S::kBarAFull + h));
+                ++n;
+            } else fetch_tokens(item + gridDim.x);
+        }
     } else if (c.warp == 1) {
         S::template mma_issuer<false>(c, A.n_items, plan, A.status);
     } else {
@@ -402,28 +469,21 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
         const uint32_t t_lane = c.tmem_base + c.group * kMtCols + b0 * 16 + ((uint32_t)(c.quarter * 32) << 16);
         int k = 0, bt = 0, n_mine = 0;
         bool ok = true;
-        // what an item needs from global memory is fetched one item ahead: its plan values, the token's
-        // modality and its place in the non-pivot list
+        // what an item needs from global memory is fetched one item ahead: its plan values and the token's modality
         auto fetch_mod = [&](const MatchRaw &r, int item) -> int {
-            const int token = r.rt * kMtItemRows + c.group * kMtRows + row;
-            return item < A.n_items && token < A.L ? A.modality[(int64_t)r.u * A.L + token] : 0;
-        };
-        auto fetch_rank = [&](const MatchRaw &r, int item) -> int {
-            const int token = r.rt * kMtItemRows + c.group * kMtRows + row;
-            return item < A.n_items && token < A.L ? A.rank[(int64_t)r.uh * A.L + token] : -1;
+            const int j = r.rt * kMtItemRows + c.group * kMtRows + row;
+            return item < A.n_items && j < A.E ? A.evi_mod[(int64_t)r.uh * A.E + j] : 0;
         };
         MatchRaw raw_next = match_raw(A, blockIdx.x);
-        int mod_next = fetch_mod(raw_next, blockIdx.x), rank_next = fetch_rank(raw_next, blockIdx.x);
+        int mod_next = fetch_mod(raw_next, blockIdx.x);
         for (int item = blockIdx.x; ok && item < A.n_items; item += gridDim.x) {
             const MatchRaw raw = raw_next;
-            const int my_mod = mod_next, my_rank = rank_next;
+            const int my_mod = mod_next;
             raw_next = match_raw(A, item + gridDim.x);
             mod_next = fetch_mod(raw_next, item + gridDim.x);
-            rank_next = fetch_rank(raw_next, item + gridDim.x);
             const MatchItem p = match_plan<S>(A, raw);
             const bool active = !p.tp.empty() && c.group < p.tp.n_halves;
-            const int token = p.rt * kMtItemRows + c.group * kMtRows + row;
-            const bool in_range = token < A.L;
+            const int j = p.rt * kMtItemRows + c.group * kMtRows + row;      // position in the non-pivot list
             const bool row_masked = p.intra && p.mixed;
             const int *slots = A.cand_slot + (int64_t)p.uh * A.Ctot;
             // Running winner of this row among the warp's columns: its similarity (still times the row's norm, four
@@ -522,14 +582,11 @@ match_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant
                 const float4 other = tc::lds128(prow + turn);
                 if (match_better(other.x, __float_as_int(other.y), best, slot)) { best = other.x; slot = __float_as_int(other.y); }
                 ssq += other.z;
-                if (in_range) {
-                    const int j = my_rank;
-                    if (j >= 0 && index_ok(j, A.E, A.status)) {      // a non-pivot: report its match
-                        float sim = 0.f;
-                        if (slot >= 0 && ssq > 0.f) sim = best * rsqrtf(ssq);
-                        A.match[(int64_t)p.uh * A.E + j] = slot;
-                        A.match_sim[(int64_t)p.uh * A.E + j] = sim;
-                    }
+                if (j < A.E) {
+                    float sim = 0.f;
+                    if (slot >= 0 && ssq > 0.f) sim = best * rsqrtf(ssq);
+                    A.match[(int64_t)p.uh * A.E + j] = slot;
+                    A.match_sim[(int64_t)p.uh * A.E + j] = sim;
                 }
             }
             turn ^= kMtRows * 16;                                  // (the next meeting keeps the upper half from a slot that is still being read)

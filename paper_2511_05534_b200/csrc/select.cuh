@@ -212,10 +212,16 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
     int *ret = A.retained + (int64_t)head * A.B;
     int *evi = A.evicted + (int64_t)head * (A.L - A.B) + i0;
     int *rank = P.rank + (int64_t)head * A.L + i0;
+    uint8_t *evi_mod = P.evi_mod + (int64_t)head * (A.L - A.B) + i0;
     int *cand_tok = hist;                                            // token of every candidate column (copy_here: up to 256)
     int *slot_out = P.cand_slot + (int64_t)head * P.Ctot;
     float *scale_out = P.cand_scale + (int64_t)head * P.Ctot;
-    const bool copy_here = with_prepare && P.copy_here;
+    const bool copy_here = with_prepare && P.copy_here, by_list = with_prepare && !P.copy_here;
+    // modalities in every tile of 256 non-pivots (by_list; the counters' place, as far as it goes)
+    uint32_t *tiles = reinterpret_cast<uint32_t *>(hist);
+    const bool tiles_here = by_list && P.n_rt <= 2 * kSelBins;
+    if (kCtas == 1 && tiles_here)
+        for (int t = tid; t < P.n_rt; t += kThreads) tiles[t] = 0;
     auto block_sum = [&](unsigned long long v, unsigned long long &total) -> unsigned long long {   // exclusive prefix sum
         unsigned long long incl_v = v;
 #pragma unroll
@@ -318,7 +324,10 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
             if (kCtas > 1) {                                         // (from here on `all` is the head's)
                 const unsigned long long ahead = cluster_sum(all, all);
                 seen = (int)(ahead & 0xFFFFFF); seen_t = (int)(ahead >> 24) & 0xFFFFF; seen_v = (int)(ahead >> 44);
-                if (!copy_here) cluster_arrive();                    // the other CTAs' words have been read
+                if (tiles_here) {                                    // (every CTA of the cluster has read the counters)
+                    for (int t = tid; t < P.n_rt; t += kThreads) tiles[t] = 0;
+                    __syncthreads();
+                }
             }
             const int n_text = (int)(all >> 24) & 0xFFFFF, n_vis = (int)(all >> 44);
             if (kOneChunk) t0 = (n_text + 31) & ~31;                 // text group first, visual group from the next multiple of 32
@@ -334,16 +343,23 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
                 for (int w = warp; w < n_w; w += kWarps) {           // the lists, a word per warp and step: coalesced
                     const uint32_t keep = keep_w[w];
                     const int i = c0 + 32 * w + lane, sl = pos_w[w] + __popc(keep & lt);
+                    bool is_vis = false;
+                    if (by_list) {
+                        is_vis = i < L && word(i) >> 31;
+                        const uint32_t m = __ballot_sync(0xFFFFFFFFu, is_vis);
+                        if (lane == 0) words[32 * w] = m;                // (nobody reads these keys any more)
+                    }
                     if (i >= L) continue;
                     if (!((keep >> lane) & 1u)) {
                         evi[i - sl] = i0 + i;
-                        if (with_prepare) rank[i] = i0 + i - sl;
+                        if (copy_here) rank[i] = i0 + i - sl;
+                        if (by_list) evi_mod[i - sl] = is_vis;
                         continue;
                     }
                     ret[sl] = i0 + i;
                     if (A.row_mod_out) A.row_mod_out[(int64_t)head * A.B + sl] = mod[i];
                     if (with_prepare) {
-                        rank[i] = -(sl + 2);
+                        if (copy_here) rank[i] = -(sl + 2);
                         const uint32_t text = text_w[w], vis = vis_w[w];
                         const int c = ((text >> lane) & 1u) ? pt_w[w] + __popc(text & lt) : ((vis >> lane) & 1u) ? pv_w[w] + __popc(vis & lt) : -1;
                         if (c >= 0 && index_ok(c, P.Ctot, P.status)) {
@@ -356,6 +372,20 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
                                 } else cand_tok[c] = i;
                             }
                         }
+                    }
+                }
+                if (tiles_here) {
+                    // A word's non-pivots are neighbours in the list, of one tile or of two (a word of both modalities at a tile's
+                    // edge may claim both for each: such a tile is then visited as a mixed one, with the same result).
+                    __syncthreads();
+                    for (int w = tid; w < n_w; w += kThreads) {
+                        const int left = L - c0 - 32 * w;
+                        const uint32_t out = ~keep_w[w] & (left < 32 ? (1u << left) - 1u : 0xFFFFFFFFu), m = words[32 * w];
+                        if (out == 0u) continue;
+                        const uint32_t what = (out & ~m ? 1u : 0u) | (out & m ? 2u : 0u);
+                        const int e = i0 + c0 + 32 * w - pos_w[w];
+                        atomicOr(&tiles[e / kMtItemRows], what);
+                        if (e % kMtItemRows + __popc(out) > kMtItemRows) atomicOr(&tiles[e / kMtItemRows + 1], what);
                     }
                 }
                 if (!kOneChunk) __syncthreads();                     // (the next chunk's words go into the same place)
@@ -377,25 +407,24 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
             if (tid == 0 && rank_c == 0) { P.cand_count[2 * head] = seen_t; P.cand_count[2 * head + 1] = seen_v; }
         }
     }
-    if (with_prepare && head % P.Hkv == 0) {                         // modalities in every tile of 256 tokens
-        const int u = head / P.Hkv, n_tiles = (L + kMtItemRows - 1) / kMtItemRows;
-        for (int tl = warp; tl < n_tiles; tl += kWarps) {
-            uint32_t any_v = 0, any_t = 0;
+    if (by_list) {
+        if (kCtas > 1) cluster_sync(); else __syncthreads();         // every CTA's tiles are marked
+        if (rank_c == 0)
+            for (int t = tid; t < P.n_rt; t += kThreads) {
+                uint32_t m = tiles_here ? tiles[t] : 3u;
+                if (kCtas > 1 && tiles_here) {
+                    const uint32_t at = (uint32_t)__cvta_generic_to_shared(tiles + t);
 #pragma unroll
-            for (int q = 0; q < kMtItemRows / 32; ++q) {
-                const int i = tl * kMtItemRows + q * 32 + lane;
-                const bool in = i < L, vis = in && word(i) >> 31;
-                any_v |= vis; any_t |= in && !vis;
+                    for (int q = 1; q < kCtas; ++q) m |= ld_cluster_u32(at, q);
+                }
+                P.tile_mod[(int64_t)head * P.n_rt + t] = (uint8_t)m;
             }
-            any_v = __any_sync(0xFFFFFFFFu, any_v); any_t = __any_sync(0xFFFFFFFFu, any_t);
-            if (lane == 0) P.tile_mod[(int64_t)u * P.n_rt + i0 / kMtItemRows + tl] = (uint8_t)((any_t ? 1 : 0) | (any_v ? 2 : 0));
-        }
     }
     if (copy_here) {
         if (kCtas > 1) cluster_sync(); else __syncthreads();         // every candidate's token is in place, in every CTA
         const int lo = P.Ctot / 32 * rank_c / kCtas * 32, hi = P.Ctot / 32 * (rank_c + 1) / kCtas * 32;
         match_gather_rows<8>(P, head, cand_tok, lo, hi, tid, kThreads);
-    } else if (kCtas > 1) cluster_wait();                            // nobody's words go away while they are read
+    } else if (kCtas > 1) cluster_sync();                            // nobody's words go away while they are read
 }
 
 }  // namespace flowmm

@@ -126,6 +126,16 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *m, 
         : "memory");
 }
 
+// 16 bytes global -> shared by this thread, the wait for all of its copies so far, and the fence that lets asynchronous readers (tensor
+// core) see what it has written.
+__device__ __forceinline__ void copy16_async(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(src)) : "memory");
+}
+__device__ __forceinline__ void copies_landed() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
 // Untiled bulk copy global -> shared (both addresses 16-byte aligned, size a multiple of 16 bytes);
 // completes `bytes` on the mbarrier like a tensor load.
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {

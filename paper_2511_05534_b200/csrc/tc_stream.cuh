@@ -5,7 +5,7 @@
 // of up to NB rows; every B tile is used by both halves, which halves the operand traffic per
 // multiply-add, and yields one 128 x NB fp32 accumulator per half in TMEM (half h owns TMEM
 // columns [NB h, NB h + NB)).
-// Roles: warp 0 issues the TMA loads, warp 1 issues tcgen05.mma, warps 2-17 run the kernel's
+// Roles: warp 0 issues the TMA loads (the matching kernel has two more warps that gather its A halves), warp 1 issues tcgen05.mma, warps 2-17 run the kernel's
 // epilogue: a quad of warps (one per 32 TMEM lanes) per (A half, column half), i.e. four epilogue
 // warps per SM sub-partition, so that TMEM reads, shared-memory reads and dependent arithmetic of
 // one warp are covered by the other three.  The two quads of a half split each accumulator's
@@ -108,6 +108,8 @@ struct Skel {
         __device__ __forceinline__ uint32_t partner_addr() const {
             return base + kSmemEpi + (uint32_t)(group * 2 + (colhalf ^ 1)) * (kEpiBytes / 4);
         }
+        // shared address of A half h (one A stage)
+        __device__ __forceinline__ uint32_t a_addr_of(int h) const { return base + kSmemA + (uint32_t)h * kAHalf; }
         // shared address of A half `group` of the n-th item this group takes part in
         __device__ __forceinline__ uint32_t a_addr(int n) const {
             return base + kSmemA + (uint32_t)((n % AST) * 2 + group) * kAHalf;
@@ -164,7 +166,8 @@ struct Skel {
     }
 
     // Call from a whole warp.  a_bytes / b_bytes: bytes one A-half / B box pair delivers (both K halves).
-    template <class PlanFn>
+    // kLoadsA: false where warps of the kernel's own bring the A halves (they wait for kBarAEmpty and arrive at kBarAFull).
+    template <bool kLoadsA = true, class PlanFn>
     static __device__ __forceinline__ void producer(const Ctx &c, const CUtensorMap *ma, const CUtensorMap *mb, int n_items,
                                                     uint32_t a_bytes, uint32_t b_bytes, PlanFn plan, int *status) {
         int ia[2] = {0, 0}, bt = 0;
@@ -195,7 +198,7 @@ struct Skel {
                     __syncwarp();
                     ++bt;
                 }
-                if (t == 0) {                  // the item's A halves go out right after its first B tile
+                if (kLoadsA && t == 0) {       // the item's A halves go out right after its first B tile
                     for (int h = 0; ok && h < p.n_halves; ++h) {
                         const int st = ia[h] % AST, full = kBarAFull + st * 2 + h;
                         ok = tc::mbar_wait_warp(c.bar(kBarAEmpty + st * 2 + h), ((ia[h] / AST) & 1) ^ 1, c.abort_flag, status);
@@ -213,7 +216,7 @@ struct Skel {
             }
         }
         if (!ok) {          // winding down after a timeout: give copies already issued a moment to land
-            for (int i = 0; i < 2 * AST; ++i)
+            for (int i = 0; kLoadsA && i < 2 * AST; ++i)
                 for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(c.bar(kBarAFull + i), 0) && !tc::mbar_try_wait(c.bar(kBarAFull + i), 1); ++s) {}
             for (int i = 0; i < BST; ++i)
                 for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(c.bar(kBarBFull + i), 0) && !tc::mbar_try_wait(c.bar(kBarBFull + i), 1); ++s) {}
