@@ -1,13 +1,14 @@
 // Weighted merge (Eq. 5) + compaction, gather form, for rows of 256 bytes (bf16 at head_dim 128): the same
 // pieces, order of accumulation and results as merge_pieces_kernel, with the member rows brought into shared
-// memory by asynchronous bulk copies instead of register loads.
+// memory by asynchronous copies instead of register loads.
 //
 // merge_pieces_kernel is bound by latency: a warp has one batch of row loads in flight, then computes, then
-// stores, and only then starts the next piece.  Here every warp owns two row buffers in shared memory and a
-// pair of mbarriers; while it accumulates one batch (pivot row + up to 8 member rows, K and V side by side)
-// the next batch - of the same piece or already of the next piece - is on its way (cp.async.bulk, 256 bytes
-// per row and tensor, one copy per lane).  The rows cost no registers while in flight, so three CTAs of
-// eight warps fit an SM and each warp keeps up to 9 KB coming.
+// stores, and only then starts the next piece.  Here every warp owns two row buffers in shared memory; while it
+// accumulates one batch (pivot row + up to 8 member rows, K and V side by side) the next batch - of the same piece or
+// already of the next piece - is on its way (cp.async, 16 bytes of each row per lane, which that lane alone reads back).
+// The rows cost no registers while in flight, so three CTAs of eight warps fit an SM and each warp keeps up to 9 KB coming.
+// Bulk copies of 256 bytes, one per row and tensor, kept the TMA unit busy: it takes one every 10 clocks or so, 20 bytes per
+// clock and SM.  128 heads of 33 792 tokens with 1690 pivots 473 -> 421 us, 112 of 8448 137 -> 126, 8 of 33 792 the call 249.8 -> 240.5.
 // Pieces are drawn from a shared counter four at a time.  With few pieces per warp (kFixed) that leaves warps with four
 // pieces of one popular slot while others have none left to draw, and a draw's round trip shows: then a warp takes every
 // n-th piece.  Drawn and fixed, us, at 3552 warps, members spread evenly and with a sixth of them in one slot: 1800 pieces 15, 10 and
@@ -27,7 +28,7 @@ constexpr int kBatch = 8;                                    // member rows per 
 constexpr uint32_t kRowBytes = 512;                          // a token's K row and V row
 constexpr uint32_t kBufBytes = (kBatch + 1) * kRowBytes;     // + the pivot row
 constexpr uint32_t kWarpBytes = 2 * kBufBytes;
-constexpr uint32_t kSmemBytes = (kThreads / 32) * kWarpBytes + (kThreads / 32) * 16 + 16;
+constexpr uint32_t kSmemBytes = (kThreads / 32) * kWarpBytes;
 
 template <typename T, bool kFixed>
 __global__ void __launch_bounds__(kThreads, 3) merge_staged_kernel(const MergeArgs A, int n_uh, int *status,
@@ -37,15 +38,6 @@ __global__ void __launch_bounds__(kThreads, 3) merge_staged_kernel(const MergeAr
     extern __shared__ __align__(128) uint8_t mstg_smem[];
     const int lane = lane_id(), warp = threadIdx.x >> 5;
     const uint32_t bufs = tc::smem_u32(mstg_smem) + warp * kWarpBytes;
-    const uint32_t bar0 = tc::smem_u32(mstg_smem) + (kThreads / 32) * kWarpBytes + warp * 16;
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(mstg_smem + (kThreads / 32) * (kWarpBytes + 16));
-    if (threadIdx.x == 0) *abort_flag = 0;
-    if (lane == 0) {
-        tc::mbar_init(bar0, 1);
-        tc::mbar_init(bar0 + 8, 1);
-        tc::mbar_init_fence();
-    }
-    __syncthreads();
     predecessor_done();
     const unsigned total = (unsigned)n_uh * (unsigned)A.max_pieces;
     const bool is_v = lane >= 16;                             // lanes 0-15: the K row, 16-31: the V row, 16 bytes each
@@ -84,38 +76,34 @@ __global__ void __launch_bounds__(kThreads, 3) merge_staged_kernel(const MergeAr
         return drawn++;
     };
     // Starts the copies of batch `b` of a piece into buffer `j & 1` (j = batches this warp has started so far):
-    // row slot 0 = the pivot (first batch of a single-piece slot only), slots 1.. = members 8 b .. 8 b + 7.
+    // row slot 0 = the pivot (first batch of a single-piece slot only), slots 1.. = members 8 b .. 8 b + 7.  A lane copies, and
+    // later reads, its own 16 bytes of each row: nothing has to be told to the other lanes.
     // this lane's source rows (K for lanes 0-15, V for 16-31) and output rows of one (unit, head), kept until the head changes
     int src_uh = -1, dst_uh = -1;
-    const T *src_base = nullptr;
+    const char *src_base = nullptr;
     T *dst_base = nullptr;
-    const int64_t tstride = is_v ? A.vs[2] : A.ks[2], ostride = is_v ? A.vos[2] : A.kos[2];
+    const int64_t ostride = is_v ? A.vos[2] : A.kos[2];
+    const uint32_t row_bytes = (uint32_t)((is_v ? A.vs[2] : A.ks[2]) * sizeof(T));   // (32 bits: hundreds of rows of 4 GB each are no GPU's)
     auto issue = [&](const Piece &pc, unsigned g, int b, int j) {
         const int uh = (int)by_pieces.div(g);
         if (uh != src_uh) {
             const int u = (int)by_hkv.div(uh), h = uh - u * A.Hkv;
-            src_base = is_v ? static_cast<const T *>(A.v) + u * A.vs[0] + h * A.vs[1]
-                            : static_cast<const T *>(A.k) + u * A.ks[0] + h * A.ks[1];
+            src_base = reinterpret_cast<const char *>((is_v ? static_cast<const T *>(A.v) + u * A.vs[0] + h * A.vs[1]
+                                                            : static_cast<const T *>(A.k) + u * A.ks[0] + h * A.ks[1]) + c0);
             src_uh = uh;
         }
         const int n_mem = min(kBatch, pc.d.z - b * kBatch);
-        const bool pivot = b == 0 && pc.d.w < 0;
-        const uint32_t buf = bufs + (j & 1) * kBufBytes, bar = bar0 + (j & 1) * 8;
-        // (the buffer was read by this warp two batches ago; order those reads before the copies' writes)
-        __syncwarp();
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        if (lane == 0) tc::mbar_expect_tx(bar, (uint32_t)(n_mem + (pivot ? 1 : 0)) * kRowBytes);
-        __syncwarp();
-        // lane l < 16 copies a row's K part, lane 16 + l its V part: rows l = 0 .. 8 (0 = pivot)
-        const int rowslot = lane & 15;
-        const int t = b * kBatch + rowslot - 1;               // member index of this lane's row
-        // (every lane asks for another member, so both halves of the list are offered and the asker picks)
-        const int tok_a = __shfl_sync(0xFFFFFFFFu, pc.tok_lo, t & 31), tok_b = __shfl_sync(0xFFFFFFFFu, pc.tok_hi, t & 31);
-        int tok = t < 32 ? tok_a : tok_b;
-        bool go = rowslot >= 1 && rowslot <= n_mem;
-        if (rowslot == 0) { tok = pc.r; go = pivot; }
-        if (go && !index_ok(tok, A.L, status)) tok = 0;     // (debug build: a bad row number is recorded; row 0 stands in so that the byte count still arrives)
-        if (go) tc::bulk_load(buf + rowslot * kRowBytes + (is_v ? 256u : 0u), src_base + (int64_t)tok * tstride, 256u, bar);
+        const uint32_t buf = bufs + (j & 1) * kBufBytes + lane * 16;
+        auto copy = [&](int rowslot, int tok) {
+            if (!index_ok(tok, A.L, status)) tok = 0;
+            tc::copy16_async(buf + rowslot * kRowBytes, src_base + (uint64_t)(uint32_t)tok * row_bytes);
+        };
+        if (b == 0 && pc.d.w < 0) copy(0, pc.r);
+        const int toks = b * kBatch < 32 ? pc.tok_lo : pc.tok_hi;
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q)
+            if (q < n_mem) copy(q + 1, __shfl_sync(0xFFFFFFFFu, toks, (b * kBatch + q) & 31));
+        tc::copies_commit();
     };
 
     unsigned g = next_piece(), g_nxt = next_piece();
@@ -125,8 +113,7 @@ __global__ void __launch_bounds__(kThreads, 3) merge_staged_kernel(const MergeAr
     fetch_members(g, cur);
     int j = 0, jc = 0;                                        // batches started / taken so far
     bool started = false;                                     // the first batch of `cur` is already on its way
-    bool ok = true;
-    while (ok && g < total) {
+    while (g < total) {
         const unsigned g_d2 = next_piece();
         const int4 d2 = fetch_desc(g_d2);                     // two pieces ahead
         fetch_members(g_nxt, nxt);                            // one piece ahead
@@ -141,12 +128,11 @@ __global__ void __launch_bounds__(kThreads, 3) merge_staged_kernel(const MergeAr
             for (int e = 0; e < V; ++e) acc[e] = 0.f;
             float wsum = 0.f;
             uint4 xr = make_uint4(0, 0, 0, 0);
-            for (int b = 0; ok && b < nb; ++b) {
+            for (int b = 0; b < nb; ++b) {
                 // the next batch starts before this one is worked on: of this piece, else the next piece's first
                 if (b + 1 < nb) { issue(cur, g, b + 1, j); ++j; }
                 else if (g_nxt < total && nxt.d.z >= 0) { issue(nxt, g_nxt, 0, j); ++j; next_started = true; }
-                ok = tc::mbar_wait_warp(bar0 + (jc & 1) * 8, (jc >> 1) & 1, abort_flag, status);
-                if (!ok) break;
+                if (j - jc > 1) tc::copies_wait<1>(); else tc::copies_wait<0>();
                 const uint32_t buf = bufs + (jc & 1) * kBufBytes + lane * 16;
                 ++jc;
                 if (b == 0 && part < 0) {
@@ -168,7 +154,6 @@ __global__ void __launch_bounds__(kThreads, 3) merge_staged_kernel(const MergeAr
                     }
                 }
             }
-            if (!ok) break;
             if (part < 0) {
                 if (uh != dst_uh) {
                     const int u = (int)by_hkv.div(uh), h = uh - u * A.Hkv;
@@ -210,10 +195,6 @@ __global__ void __launch_bounds__(kThreads, 3) merge_staged_kernel(const MergeAr
         nxt.d = d2;
         g_nxt = g_d2;
         started = next_started;
-    }
-    if (!ok) {               // winding down after a timeout: give copies already started a moment to land
-        for (int b = 0; b < 2; ++b)
-            for (int s = 0; s < (1 << 16) && !tc::mbar_try_wait(bar0 + b * 8, 0) && !tc::mbar_try_wait(bar0 + b * 8, 1); ++s) {}
     }
 }
 

@@ -126,11 +126,15 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *m, 
         : "memory");
 }
 
-// 16 bytes global -> shared by this thread, the wait for all of its copies so far, and the fence that lets asynchronous readers (tensor
+// 16 bytes global -> shared by this thread; its copies so far as a group, and the wait until at most kLater groups are on their way;
+// the wait for all of its copies so far, and the fence that lets asynchronous readers (tensor
 // core) see what it has written.
 __device__ __forceinline__ void copy16_async(uint32_t dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(reinterpret_cast<uint64_t>(src)) : "memory");
 }
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kLater>
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(kLater) : "memory"); }
 __device__ __forceinline__ void copies_landed() {
     asm volatile("cp.async.wait_all;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
