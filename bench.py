@@ -161,7 +161,7 @@ def kernel_model(wl, B, dsize):
         "score_stats": (score_flops, score_bytes),
         "score_colsum": (score_flops, score_bytes + 4.0 * Hkv * L),
         "match": (2.0 * Hkv * E * B * D, Hkv * L * D * dsize + 8.0 * Hkv * E),
-        "merge_pieces": (4.0 * Hkv * L * D, 2.0 * Hkv * (L + B) * D * dsize),
+        "merge_rows": (4.0 * Hkv * L * D, 2.0 * Hkv * (L + B) * D * dsize),
         "select_topb": (0.0, 4.0 * Hkv * L * 2),
         "build_csr": (0.0, 4.0 * Hkv * E * 3),
     }
@@ -198,8 +198,8 @@ def ncu_traffic(workload, permille, units, kernel):
 KERNEL_MODEL = {   # kernel name -> entry of kernel_model()
     "score_stats_simt": "score_stats", "score_stats_tc": "score_stats", "score_fused_tc": "score_colsum",
     "score_colsum_simt": "score_colsum", "score_colsum_tc": "score_colsum",
-    "score_cluster_simt": "score_colsum", "merge_short": "merge_pieces", "match_simt": "match", "match_tc": "match", "match_small_tc": "match", "merge_pieces": "merge_pieces",
-    "merge_tc": "merge_pieces", "merge_staged": "merge_pieces",
+    "score_cluster_simt": "score_colsum", "merge_short": "merge_rows", "match_simt": "match", "match_tc": "match", "match_small_tc": "match", "merge_rows": "merge_rows",
+    "merge_tc": "merge_rows",
     "select_topb": "select_topb", "build_csr": "build_csr",
 }
 

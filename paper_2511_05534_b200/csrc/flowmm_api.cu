@@ -14,7 +14,7 @@
 #include "decode_tc.cuh"
 #include "flow_tc.cuh"
 #include "match_small_tc.cuh"
-#include "merge_staged.cuh"
+#include "merge_rows.cuh"
 #include "merge_tc.cuh"
 #include "score_fused_tc.cuh"
 #include "match_tc.cuh"
@@ -97,13 +97,13 @@ constexpr int kScoreCtas = 148;             // one per SM of a B200
 // Where everything lives inside the caller's workspace.  One layout serves every entry point.
 struct Layout {
     size_t status, importance, cross_mass, rho, strategy, retained, evicted, match, match_sim;
-    size_t row_part, cross_part, sort_a, sort_b, mem_tok, mem_w, piece_desc, off, piece_off, part_off, partial, ticket, slot_done;
+    size_t row_part, cross_part, sort_a, sort_b, rows, row_count, off, first_slot, part_off, pieces, partial, ticket, slot_done;
     size_t cand_k, cand_scale, cand_slot, cand_count, rank, evi_mod, tile_mod, row_all;
     size_t tokmap;             // [UH, L] (slot, weight) of every token position, for the tensor-core merge
     size_t merge_status;       // status word the merge kernels report to (the workspace's own, or one of the merge scratch)
     int tc_n_qt, tc_runs, tc_n_part;
     size_t total;
-    int n_chunk1, chunk1, n_chunk2, chunk2, max_pieces, max_parts, csr_passes, c_tot, n_rt, n_et;
+    int n_chunk1, chunk1, n_chunk2, chunk2, max_parts, csr_passes, merge_win, n_win, c_tot, n_rt, n_et;
 };
 
 int chunks_for(int L, int other_ctas, int &chunk) {
@@ -116,27 +116,39 @@ int chunks_for(int L, int other_ctas, int &chunk) {
     return (L + chunk - 1) / chunk;
 }
 
-// The part of the workspace that the merge step uses (CSR of the match, piece table, partial sums).
+// Rows of a window of the merge kernel (merge_rows.cuh).  Long windows cost less per row, short ones give every warp one: 1.2 million
+// rows at most leave 3552 warps five windows of 64.  34 000 rows by 32 and 16: 77.7 and 76.4 us for the call, 43 000 84.3 and 87.3,
+// 270 000 231.5 and 240.6.
+// From kManyRows on warps draw their windows from a counter and a slot may have 128 members before it is cut, else windows are taken with a
+// stride and a slot is cut beyond 64 (270 000 rows 252 and 236 us; 4.5 million rows the merge 410 and 460).
+constexpr int64_t kManyRows = 1300000;
+int merge_window(const flowmm_params &p) {
+    const int64_t rows = (int64_t)p.n_units * p.n_kv_heads * p.seq_len;
+    return rows >= kManyRows ? 64 : rows >= 40000 ? 32 : 16;
+}
+
+// The part of the workspace that the merge step uses (rows in slot order, windows, pieces, partial sums).
 template <class Take>
 void layout_merge(Layout &y, const flowmm_params &p, Take take) {
-    const size_t UH = (size_t)p.n_units * p.n_kv_heads, B = p.n_keep, E = (size_t)p.seq_len - B, D = p.head_dim;
-    y.max_pieces = (int)(B + E / kPiece + 1);
+    const size_t UH = (size_t)p.n_units * p.n_kv_heads, B = p.n_keep, L = p.seq_len, E = L - B, D = p.head_dim;
     y.max_parts = (int)(2 * (E / kPiece) + 2);
     y.csr_passes = 1;                                        // digits of kCsrBits bits over the keys 0 .. B
     while (y.csr_passes < 6 && (B >> (kCsrBits * y.csr_passes)) != 0) ++y.csr_passes;
+    y.merge_win = merge_window(p);
+    y.n_win = (int)((L + y.merge_win - 1) / y.merge_win);
     y.sort_a = take(UH * E * 4);
     y.sort_b = take(UH * E * 4);
-    y.mem_tok = take(UH * E * 4);
-    y.mem_w = take(UH * E * 4);
-    y.piece_desc = take(UH * (size_t)y.max_pieces * 16);
+    y.rows = take(UH * L * 8);
+    y.row_count = take(UH * 8);
     y.off = take(UH * (B + 1) * 4);
-    y.piece_off = take(UH * (B + 1) * 4);
+    y.first_slot = take(UH * (size_t)y.n_win * 4);
     y.part_off = take(UH * (B + 1) * 4);
+    y.pieces = take(UH * (size_t)y.max_parts * 16);
     y.partial = take(UH * (size_t)y.max_parts * (2 * D + 4) * 4);
     y.ticket = take(256);
     y.slot_done = take(UH * B * 4);
     y.merge_status = take(256);
-    y.tokmap = take(UH * (size_t)p.seq_len * 8);
+    y.tokmap = take(UH * L * 8);
 }
 
 Layout make_layout(const flowmm_params &p) {
@@ -591,8 +603,6 @@ bool merge_is_tc(const flowmm_params &p) {
            p.seq_len < 65536 && p.path != FLOWMM_PATH_SIMT;
 }
 
-constexpr int kFixedPieces = 6;             // merge_staged_kernel: fixed assignment below this many pieces per warp
-
 // map_ready: the (slot, weight) table of the tensor-core merge has been written already (by the matching kernel)
 flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, const void *v,
                         const int32_t *retained, const int32_t *evicted, const int32_t *match, const float *match_sim,
@@ -600,10 +610,10 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
     const int E = p.seq_len - p.n_keep, UH = p.n_units * p.n_kv_heads;
     MergeArgs m;
     m.k = k; m.v = v; m.k_out = k_out; m.v_out = v_out; m.retained = retained;
-    m.mem_tok = nullptr; m.mem_w = nullptr; m.piece_desc = nullptr; m.piece_off = nullptr; m.part_off = nullptr;
+    m.rows = nullptr; m.row_count = nullptr; m.first_slot = nullptr; m.pieces = nullptr; m.part_off = nullptr;
     m.partial = at<float>(ws, y.partial); m.ticket = nullptr; m.slot_done = nullptr;
     m.Hkv = p.n_kv_heads; m.D = p.head_dim; m.L = p.seq_len; m.B = p.n_keep; m.E = E;
-    m.max_pieces = E == 0 ? p.n_keep : y.max_pieces; m.max_parts = y.max_parts;
+    m.max_parts = y.max_parts; m.win = y.merge_win; m.n_win = y.n_win;
     for (int i = 0; i < 3; ++i) {
         m.ks[i] = p.k_stride[i]; m.vs[i] = p.v_stride[i]; m.kos[i] = p.ko_stride[i]; m.vos[i] = p.vo_stride[i];
     }
@@ -644,17 +654,16 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         FLOWMM_LAUNCHED("merge_tc");
         return FLOWMM_OK;
     }
-    // Short lists: straight from the matches.  Every block of slots reads its head's whole list.  Up to 256 entries that is the
-    // faster way at any number of slots (bf16 at head_dim 128, from 512 to 95 000 blocks: 0.4 to 1.03 of the time of the sorted
-    // lists and the staged merge).  Beyond, it is for few slots: members spread evenly take 0.5 to 0.9 of it up to 2400 blocks,
-    // the same at about 8000, 1.1 to 1.3 from 12 000 on (fp32 and head_dim 64, whose sorted lists go through merge_pieces_kernel,
-    // gain up to 33 000).  What sizes do not show: a slot with a quarter of 1000 members takes such a call 1.4 to 2.3 times as
-    // long as sorted while its blocks leave the SMs idle (512 to 2400), a quarter of 400 members 0.8 to 1.4.
+    // Short lists: straight from the matches.  Every block of slots reads its head's whole list, where the sorted way is two launches
+    // and streams.  Time of the one over the other's, members spread evenly (with 15 % of them in one slot): up to 2048 blocks 0.4 to
+    // 0.9 for up to 1000 members (500 0.6 to 1.6, 1000 1.0 to 2.3); about 3600 blocks 0.98 to 1.13 up to 256 members, 1.17 beyond;
+    // 5600 blocks of 32 heads 0.70 to 0.87 up to 256 members, 1.0 to 1.1 beyond, 5900 of 112 heads 1.05 to 1.24 and 1.3 to 1.5;
+    // 14 000 and more 1.3 to 2.0.
     const int64_t slot_blocks = (int64_t)UH * ((p.n_keep + 7) / 8);
     // a slot per warp while the blocks fit the SMs together, else four, which share the block's copy of the list
     const int per = slot_blocks <= 4 * tc::sm_count() ? 1 : 4, grid_y = (p.n_keep + 8 * per - 1) / (8 * per);
     // (more slots than a grid has room for: the persistent kernels below take any number)
-    if (E > 0 && grid_y <= 65535 && (E <= 256 || (E <= kShortList && slot_blocks <= 2048))) {
+    if (E > 0 && grid_y <= 65535 && (E <= 256 ? slot_blocks <= (UH <= 32 ? 6000 : 3600) : E <= kShortList && slot_blocks <= 2048)) {
         const dim3 grid(UH, grid_y);
         auto kernel = p.dtype == FLOWMM_BF16 ? (per == 1 ? merge_short_kernel<__nv_bfloat16, 1> : merge_short_kernel<__nv_bfloat16, 4>)
                                              : (per == 1 ? merge_short_kernel<float, 1> : merge_short_kernel<float, 4>);
@@ -666,10 +675,11 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         CsrArgs c;
         c.match = match; c.evicted = evicted; c.match_sim = match_sim;
         c.sort_a = at<int>(ws, y.sort_a); c.sort_b = at<int>(ws, y.sort_b);
-        c.mem_tok = at<int>(ws, y.mem_tok); c.mem_w = at<float>(ws, y.mem_w);
-        c.off = at<int>(ws, y.off); c.piece_off = at<int>(ws, y.piece_off); c.part_off = at<int>(ws, y.part_off);
-        c.piece_desc = at<int4>(ws, y.piece_desc); c.ticket = at<unsigned>(ws, y.ticket); c.slot_done = at<int>(ws, y.slot_done);
-        c.B = p.n_keep; c.E = E; c.n_pass = y.csr_passes; c.max_pieces = y.max_pieces; c.merge_mode = p.merge_mode;
+        c.retained = retained; c.rows = at<int2>(ws, y.rows); c.row_count = at<int2>(ws, y.row_count);
+        c.off = at<int>(ws, y.off); c.first_slot = at<int>(ws, y.first_slot); c.part_off = at<int>(ws, y.part_off);
+        c.pieces = at<int4>(ws, y.pieces); c.ticket = at<unsigned>(ws, y.ticket); c.slot_done = at<int>(ws, y.slot_done);
+        c.B = p.n_keep; c.E = E; c.n_pass = y.csr_passes; c.max_parts = y.max_parts; c.merge_mode = p.merge_mode;
+        c.win = y.merge_win; c.n_win = y.n_win; c.longest = (int64_t)UH * p.seq_len < kManyRows ? kPiece : 128;
         // Warps per head by the length of its list: 8 walk up to 4096 positions in 16 steps each, which ends before 32 warps
         // are through their barriers.  Sorted in shared memory when positions and counters fit, else through global memory.
         const bool long_list = E > 4096;
@@ -696,28 +706,25 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         } else if (!long_list) launch(build_csr_kernel<8>, UH, 256, 0, st, c);
         else launch(build_csr_kernel<32>, UH, 1024, 0, st, c);
         FLOWMM_LAUNCHED("build_csr");
-        m.mem_tok = c.mem_tok; m.mem_w = c.mem_w; m.piece_desc = c.piece_desc;
-        m.piece_off = c.piece_off; m.part_off = c.part_off; m.ticket = c.ticket; m.slot_done = c.slot_done;
+        m.rows = c.rows; m.row_count = c.row_count; m.first_slot = c.first_slot; m.pieces = c.pieces;
+        m.part_off = c.part_off; m.ticket = c.ticket; m.slot_done = c.slot_done;
     }
-    const int64_t total_pieces = (int64_t)UH * m.max_pieces;
-    if (total_pieces > 0xFFFF0000ll) return FLOWMM_ERR_SHAPE;           // the piece table is indexed with 32 bits
-    const int64_t want_blocks = (total_pieces + 7) / 8;
-    const int gp = (int)(want_blocks < 2 * tc::sm_count() ? want_blocks : 2 * tc::sm_count());   // persistent warps
-    if (p.dtype == FLOWMM_BF16 && p.head_dim == 128 && E > 0 && p.path != FLOWMM_PATH_SIMT) {
-        // rows of 256 bytes: member rows staged through shared memory by asynchronous copies, three CTAs per SM
-        const int gs = (int)(want_blocks < 3 * tc::sm_count() ? want_blocks : 3 * tc::sm_count());
-        auto kernel = total_pieces < kFixedPieces * 8 * gs ? mstg::merge_staged_kernel<__nv_bfloat16, true> : mstg::merge_staged_kernel<__nv_bfloat16, false>;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mstg::kSmemBytes) != cudaSuccess) return FLOWMM_ERR_CUDA;
-        launch(kernel, gs, mstg::kThreads, mstg::kSmemBytes, st, m, UH, at<int>(ws, y.merge_status), make_fastdiv((uint32_t)m.max_pieces),
-               make_fastdiv((uint32_t)p.n_kv_heads));
-        FLOWMM_LAUNCHED("merge_staged");
-    } else if (p.dtype == FLOWMM_BF16) {
-        launch(merge_pieces_kernel<__nv_bfloat16>, gp, 256, 0, st, m, UH);
-        FLOWMM_LAUNCHED("merge_pieces");
-    } else {
-        launch(merge_pieces_kernel<float>, gp, 256, 0, st, m, UH);
-        FLOWMM_LAUNCHED("merge_pieces");
-    }
+    const int64_t items = (int64_t)UH * y.n_win;
+    if ((int64_t)UH * p.seq_len < kManyRows) m.ticket = nullptr;
+    if ((int64_t)UH * (E == 0 ? p.n_keep : (int64_t)p.n_keep + E / kPiece + 1) > 0xFFFF0000ll) return FLOWMM_ERR_SHAPE;   // (window numbers fit 32 bits long before)
+    const int bytes = p.head_dim * (p.dtype == FLOWMM_BF16 ? 2 : 4) / 16;     // of a row per lane
+    auto kernel = p.dtype == FLOWMM_BF16 ? (bytes == 16 ? mrow::merge_rows_kernel<__nv_bfloat16, 16> : mrow::merge_rows_kernel<__nv_bfloat16, 8>)
+                                         : (bytes == 16 ? mrow::merge_rows_kernel<float, 16> : mrow::merge_rows_kernel<float, 32>);
+    const size_t smem = mrow::kWarps * mrow::warp_bytes(bytes);
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
+    // Few windows: the pieces of long slots are items of their own behind them, on warps that would be idle (one head of 33 792
+    // tokens 105 -> 99 us for the call); else they are spread over the windows, as most of a head's possible pieces are none (8 such
+    // heads 237 us, as items of their own 245).
+    const int64_t most = 3 * tc::sm_count(), apart = E > 0 && items + (int64_t)UH * y.max_parts <= 2 * mrow::kWarps * most ? (int64_t)UH * y.max_parts : 0;
+    const int64_t blocks = (items + apart + mrow::kWarps - 1) / mrow::kWarps;
+    launch(kernel, (int)(blocks < most ? blocks : most), mrow::kThreads, smem, st, m, (unsigned)items, (unsigned)apart, at<int>(ws, y.merge_status),
+           make_fastdiv((uint32_t)y.n_win), make_fastdiv((uint32_t)y.max_parts), make_fastdiv((uint32_t)p.n_kv_heads));
+    FLOWMM_LAUNCHED("merge_rows");
     return FLOWMM_OK;
 }
 
@@ -1329,7 +1336,9 @@ extern "C" flowmm_status flowmm_selftest_wait_timeout(void *ws, void *cuda_strea
 
 // ---- merge without caller scratch --------------------------------------------------------------
 // Scratch of flowmm_merge_static: lives in the library image, one copy per GPU that loads it.
-static __device__ __align__(256) unsigned char g_merge_static_scratch[FLOWMM_MERGE_STATIC_BYTES];
+// (A little more than the size that callers know: merge_static_need.)
+constexpr size_t kStaticScratch = FLOWMM_MERGE_STATIC_BYTES + FLOWMM_MERGE_STATIC_BYTES / 32;
+static __device__ __align__(256) unsigned char g_merge_static_scratch[kStaticScratch];
 
 namespace {
 
@@ -1364,6 +1373,15 @@ Layout make_merge_layout(const flowmm_params &p) {
     return y;
 }
 
+// The sum that decides whether a problem is small enough: 16 bytes and a table entry per member, which is what callers have been
+// held to.  The layout above comes to less, or to 1 % more where slots are few.
+size_t merge_static_need(const flowmm_params &p) {
+    const size_t UH = (size_t)p.n_units * p.n_kv_heads, B = p.n_keep, E = (size_t)p.seq_len - B;
+    return 256 + 4 * align256(UH * E * 4) + align256(UH * (B + E / kPiece + 1) * 16) + 3 * align256(UH * (B + 1) * 4) +
+           align256(UH * (2 * (E / kPiece) + 2) * (2 * (size_t)p.head_dim + 4) * 4) + 256 + align256(UH * B * 4) + 256 +
+           align256(UH * (size_t)p.seq_len * 8);
+}
+
 }  // namespace
 
 extern "C" flowmm_status flowmm_merge_static(const flowmm_params *p, const void *k, const void *v,
@@ -1380,12 +1398,12 @@ extern "C" flowmm_status flowmm_merge_static(const flowmm_params *p, const void 
         !strides_ok(p->ko_stride, p->head_dim) || !strides_ok(p->vo_stride, p->head_dim))
         return FLOWMM_ERR_ALIGN;
     const Layout y = make_merge_layout(*p);
-    if (y.total > (size_t)FLOWMM_MERGE_STATIC_BYTES) return FLOWMM_ERR_WORKSPACE;   // problem too large for the array
+    if (merge_static_need(*p) > (size_t)FLOWMM_MERGE_STATIC_BYTES || y.total > kStaticScratch) return FLOWMM_ERR_WORKSPACE;   // problem too large for the array
     FLOWMM_TRY(check_device());
     void *base = nullptr;
     FLOWMM_TRY(merge_static_base(&base));
     FLOWMM_DEBUG_LISTS(*p, retained_idx, evicted_idx, match, static_cast<int *>(base), static_cast<cudaStream_t>(cuda_stream));
-    // Nothing in this scratch has to start at zero: the slot lists, the piece table, the work counter and
+    // Nothing in this scratch has to start at zero: the rows, windows and pieces, the work counter and
     // the arrival counters are written (or cleared) by this call's first kernel before they are read, a
     // partial-sum record is only read for pieces that wrote it in the same call, and the status word is
     // sticky on purpose (the loader zero-fills the array; flowmm_merge_static_status clears the word).

@@ -7,10 +7,10 @@ namespace flowmm {
 // ---------------------------------------------------------------------------------------------
 // Merge stage.  The match array maps non-pivot j to a slot (or -1).  The members of every slot
 // are needed in a fixed order, so the non-pivot positions j are sorted by slot, stably
-// (ascending j inside a slot); slot s then owns entries off[s] .. off[s+1] of the
-// sorted order, for which the kernel writes the member's token position and Eq. 5 weight.
-// Long member lists are cut into pieces of kPiece so that many warps share a popular pivot; one
-// descriptor per piece tells its warp what to do without any search.
+// (ascending j inside a slot).  What comes out is the sequence of a head's rows in slot order: each slot's
+// pivot, then its members, with token position and Eq. 5 weight; slot s begins at row off[s] + s, off[s] being the
+// number of members of the slots before it.  The merge kernel (merge_rows.cuh) takes the sequence a window of rows at a time.
+// A slot of more than `longest` members is left out there: it is cut into pieces of kPiece, so that many warps share it.
 // ---------------------------------------------------------------------------------------------
 constexpr int kPiece = 64;
 
@@ -19,16 +19,18 @@ struct CsrArgs {
     const int *evicted;      // [UH, E]
     const float *match_sim;  // [UH, E]
     int *sort_a, *sort_b;    // [UH, E] ping-pong buffers of non-pivot positions
-    int *mem_tok;            // [UH, E] token position of the i-th member in slot order
-    float *mem_w;            // [UH, E] its merge weight
+    const int *retained;     // [UH, B]
+    int2 *rows;              // [UH, B + E] (token, weight bits) of the head's rows in slot order; pivots with kRowPivot, of a long slot with kRowLong
+    int2 *row_count;         // [UH] (rows, pieces of long slots)
     int *off;                // [UH, B+1] first member of each slot in the sorted order
-    int *piece_off;          // [UH, B+1] first piece of each slot
-    int *part_off;           // [UH, B+1] first partial-sum record of each slot (multi-piece slots only)
-    int4 *piece_desc;        // [UH, max_pieces] (slot, first member, members, partial record or -1)
+    int *first_slot;         // [UH, n_win] first slot that begins in a window of `win` rows, for windows in which one does
+    int *part_off;           // [UH, B+1] first piece of each slot (long slots only)
+    int4 *pieces;            // [UH, max_parts] (slot, first row, rows, number of the piece)
     unsigned *ticket;        // work counter of the merge kernel, cleared here
     int *slot_done;          // [UH, B] pieces of a slot that have stored their partial sums, cleared here
-    int B, E, n_pass, max_pieces, merge_mode;
+    int B, E, n_pass, max_parts, merge_mode, win, n_win, longest;
 };
+constexpr int kRowPivot = (int)0x80000000u, kRowLong = 1 << 30, kRowToken = kRowLong - 1;
 
 __device__ __forceinline__ int csr_key(int m, int B) { return m < 0 ? B : m; }   // dropped tokens sort last
 
@@ -46,33 +48,38 @@ __device__ __forceinline__ uint32_t digit_peers(int digit, bool valid) {
     return mine;
 }
 
-// Pieces per slot and partial records per slot, exclusive scans over the slots; off[s] = first member of slot s (s <= B).
+// What the merge kernel needs beside the members' rows: the pivots' rows, the windows' first slots, the pieces of long slots.
+// off[s] = first member of slot s (s <= B).
 template <int kThreads>
-__device__ __forceinline__ void csr_write_pieces(const CsrArgs &A, int uh, const int *off, int *scratch) {
+__device__ __forceinline__ void csr_write_slots(const CsrArgs &A, int uh, const int *off, int *scratch) {
     const int tid = threadIdx.x;
-    int *piece_off = A.piece_off + (int64_t)uh * (A.B + 1);
+    const int *ret = A.retained + (int64_t)uh * A.B;
+    int2 *rows = A.rows + (int64_t)uh * (A.B + A.E);
+    int *first_slot = A.first_slot + (int64_t)uh * A.n_win;
     int *part_off = A.part_off + (int64_t)uh * (A.B + 1);
-    int4 *desc = A.piece_desc + (int64_t)uh * A.max_pieces;
-    int piece_seen = 0, part_seen = 0;
+    int4 *pieces = A.pieces + (int64_t)uh * A.max_parts;
+    int seen = 0;
     for (int base = 0; base <= A.B; base += kThreads) {
         const int s = base + tid;
-        int n = 0, np = 0, npart = 0;
+        int n = 0, np = 0;
         if (s < A.B) {
             n = off[s + 1] - off[s];
-            np = n > kPiece ? (n + kPiece - 1) / kPiece : 1;
-            npart = np > 1 ? np : 0;
+            np = n > A.longest ? (n + kPiece - 1) / kPiece : 0;
         }
-        int tot_p, tot_q;
-        const int pp = piece_seen + block_exclusive_scan(np, scratch, tot_p);
-        const int qq = part_seen + block_exclusive_scan(npart, scratch, tot_q);
-        if (s <= A.B) { piece_off[s] = pp; part_off[s] = qq; }
-        if (s < A.B) A.slot_done[(int64_t)uh * A.B + s] = 0;
-        for (int q = 0; q < np; ++q)
-            desc[pp + q] = make_int4(s, off[s] + q * kPiece, min(kPiece, n - q * kPiece), np > 1 ? qq + q : -1);
-        piece_seen += tot_p;
-        part_seen += tot_q;
+        int total;
+        const int part = seen + block_exclusive_scan(np, scratch, total);
+        if (s <= A.B) part_off[s] = part;
+        if (s < A.B) {
+            const int row = off[s] + s;
+            rows[row] = make_int2(ret[s] | kRowPivot | (np ? kRowLong : 0), 0);
+            for (int w = s == 0 ? 0 : (off[s - 1] + s - 1) / A.win + 1; w <= row / A.win; ++w) first_slot[w] = s;
+            for (int q = 0; q < np; ++q) pieces[part + q] = make_int4(s, row + 1 + q * kPiece, min(kPiece, n - q * kPiece), part + q);
+            A.slot_done[(int64_t)uh * A.B + s] = 0;
+        }
+        seen += total;
     }
-    for (int i = piece_seen + tid; i < A.max_pieces; i += kThreads) desc[i] = make_int4(0, 0, -1, -1);   // unused entries
+    if (tid == 0) A.row_count[uh] = make_int2(off[A.B] + A.B, seen);
+    if (uh == 0 && tid == 0) *A.ticket = 0u;
 }
 
 // grid = U*Hkv, block = 32 * NW threads (warp w owns a contiguous range of the input).  n_pass passes of kCsrBits bits.
@@ -87,7 +94,6 @@ __global__ void __launch_bounds__(32 * NW) build_csr_kernel(const CsrArgs A) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int uh = blockIdx.x;
     predecessor_done();
-    if (uh == 0 && tid == 0) *A.ticket = 0u;
     const int *match = A.match + (int64_t)uh * A.E;
     int *bufs[2] = {A.sort_a + (int64_t)uh * A.E, A.sort_b + (int64_t)uh * A.E};
     auto key_of = [&](int j) -> int { return csr_key(match[j], A.B); };
@@ -166,23 +172,21 @@ __global__ void __launch_bounds__(32 * NW) build_csr_kernel(const CsrArgs A) {
     {
         const int *evi = A.evicted + (int64_t)uh * A.E;
         const float *sim = A.match_sim + (int64_t)uh * A.E;
-        int *mem_tok = A.mem_tok + (int64_t)uh * A.E;
-        float *mem_w = A.mem_w + (int64_t)uh * A.E;
+        int2 *rows = A.rows + (int64_t)uh * (A.B + A.E);
         // ... and off[s] = number of sorted entries with key < s: entry i starts every slot above its predecessor's
         // key up to its own, the last entry also ends the slots above its key (E > 0: the kernel is not launched otherwise)
         for (int i = tid; i < A.E; i += kThreads) {
             const int j = sorted[i];
             const int key = key_of(j);
             const int prev = i > 0 ? key_of(sorted[i - 1]) : -1;
-            mem_tok[i] = evi[j];
-            mem_w[i] = A.merge_mode == 1 ? 1.f : __expf(sim[j] - 1.f);
+            if (key < A.B) rows[i + key + 1] = make_int2(evi[j], __float_as_int(A.merge_mode == 1 ? 1.f : __expf(sim[j] - 1.f)));
             for (int s2 = prev + 1; s2 <= key; ++s2) off[s2] = i;
             if (i == A.E - 1)
                 for (int s2 = key + 1; s2 <= A.B; ++s2) off[s2] = A.E;
         }
     }
     __syncthreads();
-    csr_write_pieces<kThreads>(A, uh, off, scratch);
+    csr_write_slots<kThreads>(A, uh, off, scratch);
 }
 
 // The same lists for heads whose sort fits in shared memory: one counting pass over the whole slot number instead of a
@@ -190,13 +194,13 @@ __global__ void __launch_bounds__(32 * NW) build_csr_kernel(const CsrArgs A) {
 //   1. warps count their ranges;  2. a thread per pair of slots turns the counts into every warp's start inside the slot,
 //   one prefix sum over the slots gives the slots' starts;  3. warps walk their ranges again, in order, and place the
 //   positions (lanes of the same slot rank themselves by votes);  4. token positions and similarities are staged in the
-//   counters' place and written out in slot order;  5. the piece table.
+//   counters' place and written out in slot order;  5. what csr_write_slots adds.
 // Bound by issue slots and shared-memory latency of one CTA per head (two walks of E positions, 11 votes per step at
 // B = 1690): 8 heads of 32 102 positions 77 us with two 6-bit digits in shared memory, 58 us so; 112 heads of 6 758 32 and
 // 25 us.  Dynamic shared memory: csr_count_smem().
 __host__ __device__ constexpr size_t csr_count_smem(int E, int B, int n_warps) {
-    const size_t Ep = ((size_t)E + 7) & ~(size_t)7, cnt = (size_t)n_warps * (((size_t)B + 2) & ~(size_t)1) * 2;
-    return 2 * Ep + 4 * (((size_t)B + 4) & ~(size_t)3) + (4 * Ep > cnt ? 4 * Ep : cnt) + 16;
+    const size_t Ep = ((size_t)E + 7) & ~(size_t)7, Lp = ((size_t)E + B + 7) & ~(size_t)7, cnt = (size_t)n_warps * (((size_t)B + 2) & ~(size_t)1) * 2;
+    return 2 * Lp + 4 * (((size_t)B + 4) & ~(size_t)3) + (4 * Ep > cnt ? 4 * Ep : cnt) + 16;
 }
 template <int NW>
 __global__ void __launch_bounds__(32 * NW) build_csr_count_kernel(const CsrArgs A, int n_bits) {
@@ -204,16 +208,15 @@ __global__ void __launch_bounds__(32 * NW) build_csr_count_kernel(const CsrArgs 
     extern __shared__ __align__(16) uint8_t csr_raw[];
     __shared__ int scratch[33];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, uh = blockIdx.x, E = A.E, B = A.B;
-    const size_t Ep = ((size_t)E + 7) & ~(size_t)7;
-    uint16_t *sorted = reinterpret_cast<uint16_t *>(csr_raw);                        // [Ep] positions in slot order
-    int *off = reinterpret_cast<int *>(csr_raw + 2 * Ep);                            // [B + 1] first member of every slot
-    uint8_t *region = csr_raw + 2 * Ep + 4 * (((size_t)B + 4) & ~(size_t)3);
+    const size_t Lp = ((size_t)E + B + 7) & ~(size_t)7;
+    uint16_t *sorted = reinterpret_cast<uint16_t *>(csr_raw);                        // [Lp] positions in slot order, a place before each slot's for its pivot
+    int *off = reinterpret_cast<int *>(csr_raw + 2 * Lp);                            // [B + 1] first member of every slot
+    uint8_t *region = csr_raw + 2 * Lp + 4 * (((size_t)B + 4) & ~(size_t)3);
     const int pitch = (B + 2) & ~1;                                                  // counters of a warp, an even number
     uint16_t *cnt = reinterpret_cast<uint16_t *>(region) + warp * pitch;
     for (int i = tid; i < NW * pitch / 2; i += kThreads) reinterpret_cast<uint32_t *>(region)[i] = 0u;
     __syncthreads();
     predecessor_done();
-    if (uh == 0 && tid == 0) *A.ticket = 0u;
     const int *match = A.match + (int64_t)uh * E;
     const int per_warp = ((E + NW - 1) / NW + 31) / 32 * 32, lo = min(E, warp * per_warp), hi = min(E, lo + per_warp);
     auto fetch = [&](int t0, int (&key)[kBatch]) {                                   // -1: no such position
@@ -262,35 +265,38 @@ __global__ void __launch_bounds__(32 * NW) build_csr_count_kernel(const CsrArgs 
                 const uint32_t vote = __ballot_sync(0xFFFFFFFFu, (key[b] >> q) & 1);
                 mine &= ((key[b] >> q) & 1) ? vote : ~vote;
             }
-            if (valid) sorted[off[key[b]] + cnt[key[b]] + __popc(mine & lanemask_lt())] = (uint16_t)(t0 + 32 * b + lane);
+            if (valid && key[b] < B) sorted[off[key[b]] + key[b] + 1 + cnt[key[b]] + __popc(mine & lanemask_lt())] = (uint16_t)(t0 + 32 * b + lane);
             __syncwarp();
             if (valid && lane == __ffs(mine) - 1) cnt[key[b]] += (uint16_t)__popc(mine);
             __syncwarp();
         }
     }
+    for (int s = tid; s < B; s += kThreads) sorted[off[s] + s] = 0xFFFF;             // the pivots' places (E < 65536: no position is that)
     __syncthreads();
-    // (entries past off[B] are the dropped tokens: nobody reads them)
-    const int n_mem = off[B];
-    int *mem_tok = A.mem_tok + (int64_t)uh * E;
-    float *mem_w = A.mem_w + (int64_t)uh * E;
+    const int n_rows = off[B] + B;
+    int2 *rows = A.rows + (int64_t)uh * (B + E);
     {
         const int *evi = A.evicted + (int64_t)uh * E;
+        const float *sim = A.match_sim + (int64_t)uh * E;
         int *stage = reinterpret_cast<int *>(region);
         for (int i = tid; i < E; i += kThreads) stage[i] = evi[i];
         __syncthreads();
-        for (int i = tid; i < n_mem; i += kThreads) mem_tok[i] = stage[sorted[i]];
-        if (A.merge_mode == 1) {
-            for (int i = tid; i < n_mem; i += kThreads) mem_w[i] = 1.f;
-        } else {
-            const float *sim = A.match_sim + (int64_t)uh * E;
-            float *stage_f = reinterpret_cast<float *>(region);
+        for (int i = tid; i < n_rows; i += kThreads) {
+            const int j = sorted[i];
+            if (j != 0xFFFF) rows[i].x = stage[j];
+        }
+        float *stage_f = reinterpret_cast<float *>(region);
+        if (A.merge_mode != 1) {
             __syncthreads();
             for (int i = tid; i < E; i += kThreads) stage_f[i] = sim[i];
             __syncthreads();
-            for (int i = tid; i < n_mem; i += kThreads) mem_w[i] = __expf(stage_f[sorted[i]] - 1.f);
+        }
+        for (int i = tid; i < n_rows; i += kThreads) {
+            const int j = sorted[i];
+            if (j != 0xFFFF) rows[i].y = __float_as_int(A.merge_mode == 1 ? 1.f : __expf(stage_f[j] - 1.f));
         }
     }
-    csr_write_pieces<kThreads>(A, uh, off, scratch);
+    csr_write_slots<kThreads>(A, uh, off, scratch);
 }
 
 // The counting sort with a head's positions shared among the CTAs of a cluster, for calls whose heads do not fill the GPU.
@@ -318,7 +324,6 @@ __global__ void __launch_bounds__(32 * kCsrClusterWarps) build_csr_cluster_kerne
     for (int i = tid; i < NW * pitch / 2; i += kThreads) words[i] = 0u;
     __syncthreads();
     predecessor_done();
-    if (blockIdx.x == 0 && tid == 0) *A.ticket = 0u;
     const int *match = A.match + (int64_t)uh * E;
     const int per_warp = ((E + ctas * NW - 1) / (ctas * NW) + 31) / 32 * 32;
     const int lo = min(E, (rank * NW + warp) * per_warp), hi = min(E, lo + per_warp);
@@ -362,8 +367,7 @@ __global__ void __launch_bounds__(32 * kCsrClusterWarps) build_csr_cluster_kerne
     cluster_arrive();                                                                // the other CTAs' totals have been read
     const int *evi = A.evicted + (int64_t)uh * E;
     const float *sim = A.match_sim + (int64_t)uh * E;
-    int *mem_tok = A.mem_tok + (int64_t)uh * E;
-    float *mem_w = A.mem_w + (int64_t)uh * E;
+    int2 *rows = A.rows + (int64_t)uh * (B + E);
     for (int t0 = lo; t0 < hi; t0 += 32 * kBatch) {
         int key[kBatch], tok[kBatch];
         float w[kBatch];
@@ -385,15 +389,14 @@ __global__ void __launch_bounds__(32 * kCsrClusterWarps) build_csr_cluster_kerne
             }
             if (valid && key[b] < B) {                                               // (dropped tokens have no place)
                 const int at = base[key[b]] + cnt[key[b]] + __popc(mine & lanemask_lt());
-                mem_tok[at] = tok[b];
-                mem_w[at] = A.merge_mode == 1 ? 1.f : __expf(w[b] - 1.f);
+                rows[at + key[b] + 1] = make_int2(tok[b], __float_as_int(A.merge_mode == 1 ? 1.f : __expf(w[b] - 1.f)));
             }
             __syncwarp();
             if (valid && lane == __ffs(mine) - 1) cnt[key[b]] += (uint16_t)__popc(mine);
             __syncwarp();
         }
     }
-    if (rank == ctas - 1) csr_write_pieces<kThreads>(A, uh, off, scratch);           // (the last CTA has the fewest positions)
+    if (rank == ctas - 1) csr_write_slots<kThreads>(A, uh, off, scratch);           // (the last CTA has the fewest positions)
     __syncwarp();
     cluster_wait();                                                                  // nobody's totals go away while they are read
 }
@@ -402,14 +405,15 @@ struct MergeArgs {
     const void *k, *v;
     void *k_out, *v_out;
     const int *retained;              // [UH, B]
-    const int *mem_tok;               // [UH, E] member token positions in slot order; nullptr when E == 0
-    const float *mem_w;               // [UH, E] member weights
-    const int4 *piece_desc;           // [UH, max_pieces]
-    const int *piece_off, *part_off;  // [UH, B+1]
+    const int2 *rows;                 // [UH, L] as in CsrArgs; nullptr when E == 0: the pivots alone
+    const int2 *row_count;            // [UH]
+    const int *first_slot;            // [UH, n_win]
+    const int4 *pieces;               // [UH, max_parts]
+    const int *part_off;              // [UH, B+1]
     float *partial;                   // [UH, max_parts, 2*D + 4] fp32 partial sums
-    unsigned *ticket;                 // shared work counter (pieces are handed out in table order); nullptr: fixed stride
-    int *slot_done;                   // [UH, B] arrival counters of multi-piece slots
-    int Hkv, D, L, B, E, max_pieces, max_parts;
+    unsigned *ticket;                 // shared work counter; nullptr: windows are taken with a stride
+    int *slot_done;                   // [UH, B] arrival counters of long slots
+    int Hkv, D, L, B, E, max_parts, win, n_win;
     int64_t ks[3], vs[3], kos[3], vos[3];
 };
 
@@ -420,9 +424,8 @@ template <typename T>
 __device__ __forceinline__ void merge_finish_slot(const MergeArgs &A, int uh, int slot, int lane) {
     constexpr int V = Elem<T>::kVec;
     const int u = uh / A.Hkv, h = uh % A.Hkv;
-    const int *poff = A.piece_off + (int64_t)uh * (A.B + 1);
-    const int n_pieces = poff[slot + 1] - poff[slot];
-    const int part_base = A.part_off[(int64_t)uh * (A.B + 1) + slot];
+    const int *poff = A.part_off + (int64_t)uh * (A.B + 1);
+    const int part_base = poff[slot], n_pieces = poff[slot + 1] - part_base;
     const float *rec0 = A.partial + ((int64_t)uh * A.max_parts + part_base) * (2 * A.D + 4);
     const int rv = A.D / V;
     const int r = A.retained[(int64_t)uh * A.B + slot];
@@ -454,153 +457,9 @@ __device__ __forceinline__ void merge_finish_slot(const MergeArgs &A, int uh, in
 
 constexpr int kMergeBatch = 8;        // member rows a warp keeps in flight
 
-// One warp per piece of a slot, persistent: a warp walks the flat piece table with a stride and
-// fetches the next piece's descriptor, member list and pivot index while it streams the rows of
-// the current one, so the row loads never wait on index loads.  A 16-byte vector of a K row or V
-// row per lane: with D*sizeof(T) = 256 bytes lanes 0-15 carry the K row and lanes 16-31 the V
-// row.  A single-piece slot is finished here (pivot row with weight 1, Eq. 5 weights, normalise,
-// round once); a piece of a multi-piece slot stores its fp32 partial sums, and the piece that arrives
-// last adds them up in piece order (so the result does not depend on which piece that was).
-template <typename T>
-__global__ void __launch_bounds__(256) merge_pieces_kernel(const MergeArgs A, int n_uh) {
-    constexpr int V = Elem<T>::kVec;
-    predecessor_done();
-    const int lane = lane_id();
-    const unsigned n_warps = gridDim.x * (blockDim.x >> 5);
-    const unsigned total = (unsigned)n_uh * (unsigned)A.max_pieces;
-    const int rv = A.D / V;                                   // 16-byte vectors per row
-    const int n_vec = 2 * rv;
-
-    struct Piece { int4 d; int tok_lo, tok_hi, r; float w_lo, w_hi; };
-    auto fetch_desc = [&](unsigned g) -> int4 {              // (slot, first, count, part); count < 0: no such piece
-        if (g >= total) return make_int4(0, 0, -1, -1);
-        if (!A.piece_desc) return make_int4((int)(g % (unsigned)A.max_pieces), 0, 0, -1);   // E == 0: plain copy of the pivots
-        return A.piece_desc[g];
-    };
-    auto fetch_members = [&](unsigned g, Piece &pc) {        // needs pc.d
-        pc.tok_lo = pc.tok_hi = pc.r = 0; pc.w_lo = pc.w_hi = 0.f;
-        if (pc.d.z < 0) return;
-        const int64_t uh = g / (unsigned)A.max_pieces;
-        if (pc.d.z > 0) {
-            const int *mt = A.mem_tok + uh * A.E + pc.d.y;
-            const float *mw = A.mem_w + uh * A.E + pc.d.y;
-            if (lane < pc.d.z) { pc.tok_lo = mt[lane]; pc.w_lo = mw[lane]; }
-            if (lane + 32 < pc.d.z) { pc.tok_hi = mt[lane + 32]; pc.w_hi = mw[lane + 32]; }
-        }
-        if (pc.d.w < 0) pc.r = A.retained[uh * A.B + pc.d.x];
-    };
-    // the next piece of this warp: from the shared counter (warps that drew light pieces come back sooner, so
-    // the last pieces end together), or with a fixed stride when there is no counter
-    unsigned stride_next = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    unsigned drawn = 0, drawn_left = 0;                       // pieces are drawn kDraw at a time
-    constexpr unsigned kDraw = 4;
-    auto next_piece = [&]() -> unsigned {
-        if (!A.ticket) { const unsigned g = stride_next; stride_next = g + n_warps < g ? 0xFFFFFFFFu : g + n_warps; return g; }
-        if (drawn_left == 0) {
-            unsigned g = 0;
-            if (lane == 0) g = atomicAdd(A.ticket, kDraw);
-            drawn = __shfl_sync(0xFFFFFFFFu, g, 0);
-            drawn_left = kDraw;
-        }
-        --drawn_left;
-        return drawn++;
-    };
-
-    unsigned g = next_piece(), g_nxt = next_piece();
-    Piece cur, nxt;
-    cur.d = fetch_desc(g);
-    nxt.d = fetch_desc(g_nxt);
-    fetch_members(g, cur);
-    while (g < total) {
-        const unsigned g_d2 = next_piece();
-        const int4 d2 = fetch_desc(g_d2);                     // two pieces ahead
-        fetch_members(g_nxt, nxt);                            // one piece ahead
-        const int slot = cur.d.x, count = cur.d.z, part = cur.d.w;
-        if (count >= 0) {
-            const int uh = (int)(g / (unsigned)A.max_pieces), u = uh / A.Hkv, h = uh % A.Hkv;
-            const T *kb = static_cast<const T *>(A.k) + u * A.ks[0] + h * A.ks[1];
-            const T *vb = static_cast<const T *>(A.v) + u * A.vs[0] + h * A.vs[1];
-            for (int vec0 = 0; vec0 < n_vec; vec0 += 32) {    // which vector of the (K row, V row) pair
-                const int vec = vec0 + lane;
-                const bool on = vec < n_vec;
-                const bool is_v = vec >= rv;
-                const int c0 = on ? (is_v ? vec - rv : vec) * V : 0;
-                const T *src = is_v ? vb : kb;
-                const int64_t tstride = is_v ? A.vs[2] : A.ks[2];
-                float acc[V];
-#pragma unroll
-                for (int e = 0; e < V; ++e) acc[e] = 0.f;
-                float wsum = 0.f;
-                uint4 xr = make_uint4(0, 0, 0, 0);
-                if (on && part < 0) xr = load_raw16(src + (int64_t)cur.r * tstride + c0);    // the pivot row, early
-                for (int t0 = 0; t0 < count; t0 += kMergeBatch) {
-                    uint4 x[kMergeBatch];
-                    int tok[kMergeBatch];
-                    float w[kMergeBatch];
-#pragma unroll
-                    for (int q = 0; q < kMergeBatch; ++q) {   // this batch's positions and weights from the lanes that hold them
-                        const int t = t0 + q;
-                        tok[q] = __shfl_sync(0xFFFFFFFFu, t < 32 ? cur.tok_lo : cur.tok_hi, t & 31);
-                        w[q] = __shfl_sync(0xFFFFFFFFu, t < 32 ? cur.w_lo : cur.w_hi, t & 31);
-                    }
-#pragma unroll
-                    for (int q = 0; q < kMergeBatch; ++q)     // the batch's row loads, back to back
-                        x[q] = (t0 + q < count && on) ? load_raw16(src + (int64_t)tok[q] * tstride + c0) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-                    for (int q = 0; q < kMergeBatch; ++q) {   // fixed order: ascending member index
-                        if (t0 + q < count) {
-                            float xf[V];
-                            Elem<T>::unpack(x[q], xf);
-                            wsum += w[q];
-#pragma unroll
-                            for (int e = 0; e < V; ++e) acc[e] = fmaf(w[q], xf[e], acc[e]);
-                        }
-                    }
-                }
-                if (!on) continue;
-                if (part < 0) {
-                    T *dst = is_v ? static_cast<T *>(A.v_out) + u * A.vos[0] + h * A.vos[1] + (int64_t)slot * A.vos[2]
-                                  : static_cast<T *>(A.k_out) + u * A.kos[0] + h * A.kos[1] + (int64_t)slot * A.kos[2];
-                    if (count == 0) {
-                        *reinterpret_cast<uint4 *>(dst + c0) = xr;   // nothing merged in: the pivot row, bit for bit
-                    } else {
-                        const float inv = 1.f / (1.f + wsum);
-                        float xf[V], o[V];
-                        Elem<T>::unpack(xr, xf);
-#pragma unroll
-                        for (int e = 0; e < V; ++e) o[e] = (xf[e] + acc[e]) * inv;
-                        Elem<T>::store16(dst + c0, o);
-                    }
-                } else {
-                    float *rec = A.partial + ((int64_t)uh * A.max_parts + part) * (2 * A.D + 4);
-#pragma unroll
-                    for (int e = 0; e < V; ++e) rec[(is_v ? A.D : 0) + c0 + e] = acc[e];
-                    if (vec == 0) rec[2 * A.D] = wsum;
-                }
-            }
-            if (part >= 0) {                                  // multi-piece slot: was this the last piece to arrive?
-                __threadfence();
-                __syncwarp();
-                int prev = 0;
-                if (lane == 0) prev = atomicAdd(&A.slot_done[(int64_t)uh * A.B + slot], 1);
-                prev = __shfl_sync(0xFFFFFFFFu, prev, 0);
-                const int *poff = A.piece_off + (int64_t)uh * (A.B + 1);
-                if (prev == poff[slot + 1] - poff[slot] - 1) {
-                    __threadfence();
-                    merge_finish_slot<T>(A, uh, slot, lane);
-                }
-            }
-        }
-        cur = nxt;
-        g = g_nxt;
-        nxt.d = d2;
-        g_nxt = g_d2;
-    }
-}
-
-// Short lists (up to kShortList non-pivots per head): no member lists and no piece table.  A block holds the head's matches,
+// Short lists (up to kShortList non-pivots per head): no member lists.  A block holds the head's matches,
 // tokens and weights in shared memory, a warp finds the members of its slot by ballots over them, in ascending order, and
-// sums their rows as merge_pieces_kernel sums a piece (8 on their way at a time).  A slot of more than kSoloMembers is shared
+// sums their rows, 8 on their way at a time.  A slot of more than kSoloMembers is shared
 // by the block's warps, each with an eighth of the members; the parts are added in order.
 // Bound by latency: a chain of three loads, where the sort of the lists and the tables around it took a launch of its own.  The
 // call of 4 heads of 192 tokens (fp32) 40.6 -> 31.4 us, 8 of 950 62 -> 50, 112 of 640 with 423 slots (bf16) 110 -> 102.

@@ -1,0 +1,92 @@
+"""Merge of sorted lists by windows of rows: slots of chosen numbers of members (none, the most that stay whole, one more, several
+chunks of 128 rows) at chosen places of a window, windows of 16, 32 and 64 rows, taken with a stride or drawn from the counter,
+pieces of long slots as items of their own and spread over the windows, every row width, and output layouts with gaps.
+The values let one lost or doubled member be seen (test_merge_reference.py)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import flowmm_oracle as O
+from paper_2511_05534_b200 import binding as F
+
+from gpu_util import gpu_params, merge_reference, small_integers, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _members(pattern, B, rng):
+    """Members of each slot."""
+    n = rng.integers(0, 4, B)
+    edges = [63, 64, 65, 127, 128, 129, 130, 191, 192, 193, 257, 640]
+    if pattern == "edges_first":
+        n[: len(edges)] = edges
+    elif pattern == "edges_apart":                                  # every one at another place of its window
+        n[7:7 + 17 * len(edges):17] = edges
+    elif pattern == "edges_last":
+        n[B - len(edges):] = edges
+    elif pattern == "alternate":
+        n[:] = 0
+        n[5:65:2] = np.tile([65, 15, 64, 129, 1], 6)
+    return n
+
+
+@pytest.mark.parametrize("dtype,D", [(F.BF16, 128), (F.BF16, 64), (F.F32, 64), (F.F32, 128)])
+@pytest.mark.parametrize("heads", [1, 12, 90])                     # windows of 16, of 32 with pieces of their own, of 32 with pieces spread
+@pytest.mark.parametrize("pattern", ["edges_first", "edges_apart", "edges_last", "alternate"])
+def test_slots_of_chosen_sizes(pattern, heads, dtype, D):
+    rng = np.random.default_rng(D + heads)
+    B = 700
+    n = _members(pattern, B, rng)
+    dropped = 150
+    E = int(n.sum()) + dropped
+    L = E + B
+    if E <= 1024:
+        pytest.skip("short list")
+    k, v = (small_integers(rng, (1, 1, L, D)) for _ in range(2))
+    ret = np.sort(rng.choice(L, B, replace=False))
+    evi = np.setdiff1d(np.arange(L), ret)
+    match = np.concatenate([np.repeat(np.arange(B), n), np.full(dropped, -1)])
+    rng.shuffle(match)
+    sim = np.where(match >= 0, rng.random(E), 0).astype(np.float32)
+    ret, evi, match = (x.astype(np.int32)[None, None] for x in (ret, evi, match))
+    sim = sim[None, None]
+    rep = lambda x: torch.from_numpy(np.ascontiguousarray(np.repeat(x, heads, 1))).cuda()
+    lists = [rep(x) for x in (ret, evi, match, sim)]
+    kd, vd = (rep(x).to(F.torch_dtype(dtype)) for x in (k, v))
+    for mode in (F.MERGE_MEAN, F.MERGE_EXPSIM):
+        refs = merge_reference(O.OracleParams(1, 1, 1, D, L, 1, B, merge_mode=mode), k, v, ret, evi, match, sim.astype(np.float64), dtype)
+        fp = gpu_params(O.OracleParams(1, heads, heads, D, L, 1, B, merge_mode=mode), dtype)
+        ws = F.alloc_workspace(fp)
+        out = [torch.full((1, heads, B, D + 8), float("nan"), dtype=F.torch_dtype(dtype), device="cuda")[..., :D] for _ in range(2)]
+        F.flowmm_merge(fp, kd, vd, *lists, out[0], out[1], ws)
+        assert F.flowmm_last_device_status(ws) == 0
+        for got, (ref, bound) in zip(out, refs):
+            assert np.all(np.abs(got[:, :1].double().cpu().numpy() - ref) <= bound), mode
+            assert torch.equal(got, got[:, :1].expand(-1, heads, -1, -1))
+
+
+def test_many_rows_draw_their_windows():
+    """1.6 million rows of 160 heads: windows of 64 from the counter, slots of up to 128 members whole."""
+    rng = np.random.default_rng(3)
+    heads, B, D = 160, 1000, 64
+    n = _members("edges_apart", B, rng)
+    n[300:340] = rng.integers(100, 160, 40)
+    E = int(n.sum())
+    L = E + B
+    assert heads * L >= 1300000
+    k, v = (small_integers(rng, (1, 1, L, D)) for _ in range(2))
+    ret = np.sort(rng.choice(L, B, replace=False))
+    evi = np.setdiff1d(np.arange(L), ret)
+    match = rng.permutation(np.repeat(np.arange(B), n))
+    ret, evi, match = (x.astype(np.int32)[None, None] for x in (ret, evi, match))
+    sim = rng.random((1, 1, E)).astype(np.float32)
+    refs = merge_reference(O.OracleParams(1, 1, 1, D, L, 1, B, merge_mode=F.MERGE_MEAN), k, v, ret, evi, match, sim.astype(np.float64), F.BF16)
+    rep = lambda x: torch.from_numpy(np.ascontiguousarray(np.repeat(x, heads, 1))).cuda()
+    fp = gpu_params(O.OracleParams(1, heads, heads, D, L, 1, B, merge_mode=F.MERGE_MEAN), F.BF16)
+    out = [torch.full((1, heads, B, D), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    ws = F.alloc_workspace(fp)
+    F.flowmm_merge(fp, rep(k).bfloat16(), rep(v).bfloat16(), *(rep(x) for x in (ret, evi, match, sim)), out[0], out[1], ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    for got, (ref, bound) in zip(out, refs):
+        assert np.all(np.abs(got[:, :1].double().cpu().numpy() - ref) <= bound)
+        assert torch.equal(got, got[:, :1].expand(-1, heads, -1, -1))
