@@ -50,17 +50,18 @@ struct MatchPrepArgs {
 // cand_tok: the positions' tokens (-1: no candidate), or nullptr: found through the slots and the pivot list.
 // kRows rows per lane are in flight together: a row is one dependent chain of loads.
 template <int kRows>
-__device__ __forceinline__ void match_gather_rows(const MatchPrepArgs &A, int uh, const int *cand_tok, int lo, int hi, int tid, int nthreads) {
-    const int u = uh / A.Hkv, h = uh % A.Hkv;
-    const int *ret = A.retained + (int64_t)uh * A.B;
-    const int *slot_out = A.cand_slot + (int64_t)uh * A.Ctot;
-    float *scale_out = A.cand_scale + (int64_t)uh * A.Ctot;
-    const __nv_bfloat16 *kb = static_cast<const __nv_bfloat16 *>(A.k) + u * A.ks[0] + h * A.ks[1];
-    uint4 *dst = reinterpret_cast<uint4 *>(A.cand_k + (int64_t)uh * A.Ctot * 128);
-    const int sub = tid & 15, stride = nthreads >> 4;
-    for (int p0 = lo + (tid >> 4); p0 < hi; p0 += kRows * stride) {         // uniform trip count within a warp
-        int tok[kRows];
-        uint4 val[kRows];
+struct MatchGather {
+    const MatchPrepArgs &A;
+    const __nv_bfloat16 *kb;
+    int uh, sub, stride, tok[kRows];
+    uint4 val[kRows];
+    __device__ __forceinline__ MatchGather(const MatchPrepArgs &a, int uh_, int tid, int nthreads) : A(a), uh(uh_), sub(tid & 15), stride(nthreads >> 4) {
+        const int u = uh / A.Hkv, h = uh % A.Hkv;
+        kb = static_cast<const __nv_bfloat16 *>(A.k) + u * A.ks[0] + h * A.ks[1];
+    }
+    // Positions p0, p0 + stride, ... below hi: their rows start to come.
+    __device__ __forceinline__ void start(const int *cand_tok, int p0, int hi) {
+        const int *ret = A.retained + (int64_t)uh * A.B, *slot_out = A.cand_slot + (int64_t)uh * A.Ctot;
 #pragma unroll
         for (int q = 0; q < kRows; ++q) {
             const int pos = p0 + q * stride;
@@ -79,6 +80,10 @@ __device__ __forceinline__ void match_gather_rows(const MatchPrepArgs &A, int uh
             if (tok[q] >= 0 && index_ok(tok[q], A.L, A.status))
                 val[q] = *reinterpret_cast<const uint4 *>(kb + (int64_t)tok[q] * A.ks[2] + sub * 8);
         }
+    }
+    __device__ __forceinline__ void finish(int p0, int hi) {
+        float *scale_out = A.cand_scale + (int64_t)uh * A.Ctot;
+        uint4 *dst = reinterpret_cast<uint4 *>(A.cand_k + (int64_t)uh * A.Ctot * 128);
 #pragma unroll
         for (int q = 0; q < kRows; ++q) {
             const int pos = p0 + q * stride;
@@ -92,6 +97,14 @@ __device__ __forceinline__ void match_gather_rows(const MatchPrepArgs &A, int uh
             for (int o = 8; o > 0; o >>= 1) ssq += __shfl_xor_sync(0xFFFFFFFFu, ssq, o);
             if (sub == 0 && tok[q] >= 0) scale_out[pos] = ssq > 0.f ? rsqrtf(ssq) : 0.f;
         }
+    }
+};
+template <int kRows>
+__device__ __forceinline__ void match_gather_rows(const MatchPrepArgs &A, int uh, const int *cand_tok, int lo, int hi, int tid, int nthreads) {
+    MatchGather<kRows> g(A, uh, tid, nthreads);
+    for (int p0 = lo + (tid >> 4); p0 < hi; p0 += kRows * g.stride) {       // uniform trip count within a warp
+        g.start(cand_tok, p0, hi);
+        g.finish(p0, hi);
     }
 }
 

@@ -89,10 +89,11 @@ static_assert(select_smem(kSelMaxChunk) <= 232448 - 1024, "shared memory budget"
 // added up through distributed shared memory in every pass, their totals before the lists are written.  For calls of few
 // heads, whose blocks would leave most SMs idle: 8 heads of 33 792 tokens 31 -> 18 us, 4 heads of 8448 14 -> 12.
 template <int kThreads, bool kOneChunk, int kCtas>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, kThreads == 256 ? 4 : kThreads == 512 && kCtas == 1 ? 2 : 1)
 select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P, int with_prepare) {
     static_assert(kCtas == 1 || (kOneChunk && kThreads == 512), "a CTA's part is one chunk; four counters per thread");
     constexpr int kWarps = kThreads / 32, kPer = kSelBins / kThreads;
+    constexpr bool kFew = kOneChunk && kCtas == 1 && kThreads <= 512;   // (launched for up to 1024 or 4096 positions)
     extern __shared__ __align__(16) int sel_smem[];
     __shared__ int wtot[kWarps], res[3];
     __shared__ unsigned long long wsum[kWarps];
@@ -222,6 +223,126 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
     const bool tiles_here = by_list && P.n_rt <= 2 * kSelBins;
     if (kCtas == 1 && tiles_here)
         for (int t = tid; t < P.n_rt; t += kThreads) tiles[t] = 0;
+    // Up to 4096 positions: a warp's words, one run of them, stay in registers, and what comes before them is added up over the warps'
+    // totals behind one barrier; the candidates' key rows are fetched while the lists are written.  (With marks in shared memory and
+    // a prefix sum over all words, which every warp took for itself, the block of 1471 positions spent 1900 clocks on the marks, 2800 on
+    // the sum, 2400 on the lists and 3600 on the rows, of 15 600.  The whole call, us: 4 heads of 192 positions 22.3 -> 21.3, 32 of 640
+    // 26.4 -> 25.7, 8 of 1471 36.0 -> 35.0, 112 of 2176 112.7 -> 111.0, 1024 of 640 156.3 -> 153.4.)  Four blocks of 256 threads to an
+    // SM: with five or six a thread has too few registers for four rows, with more rows too many.
+    if constexpr (kFew) {
+        constexpr int kE = kThreads == 256 ? 4 : 8;
+        const int n_w = (L + 31) >> 5, per = (n_w + kWarps - 1) / kWarps, w0 = warp * per;
+        uint32_t wd[kE], keep[kE], text[kE], vis[kE];
+#pragma unroll
+        for (int e = 0; e < kE; ++e) {
+            const int i = 32 * (w0 + e) + lane;
+            wd[e] = e < per && i < L ? words[i] : 0u;
+        }
+        int ties = 0;                                                // equal keys before this warp's: the lower positions are taken
+        if (!all_eq) {
+            int n = 0;
+#pragma unroll
+            for (int e = 0; e < kE; ++e)
+                if (e < per) n += __popc(__ballot_sync(0xFFFFFFFFu, 32 * (w0 + e) + lane < L && (wd[e] & kKeyMask) == prefix));
+            if (lane == 0) wtot[warp] = n;
+            __syncthreads();
+            ties = (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? (unsigned)wtot[lane] : 0u);
+        }
+        uint32_t n_keep_text = 0, n_vis = 0;                         // pivots, and admissible text ones from bit 16 on; admissible visual ones
+#pragma unroll
+        for (int e = 0; e < kE; ++e) {
+            keep[e] = text[e] = vis[e] = 0;
+            if (e >= per) continue;
+            const int i = 32 * (w0 + e) + lane;
+            const uint32_t mk = wd[e] & kKeyMask & mask;
+            bool take = i < L && mk >= prefix;
+            if (!all_eq) {
+                const bool eq = i < L && mk == prefix;
+                const uint32_t m = __ballot_sync(0xFFFFFFFFu, eq);
+                if (eq) take = ties + __popc(m & lt) < need;
+                ties += __popc(m);
+            }
+            keep[e] = __ballot_sync(0xFFFFFFFFu, take);
+            n_keep_text += __popc(keep[e]);
+            if (with_prepare) {                                      // Eq. 10: pivots above tau are kept out of merging
+                const bool adm = take && (i < first_forced ? __uint_as_float(wd[e] & kKeyMask) : imp[i]) <= P.tau_eff;
+                const uint32_t cand = __ballot_sync(0xFFFFFFFFu, adm), seen_vis = __ballot_sync(0xFFFFFFFFu, wd[e] >> 31);
+                text[e] = cand & ~seen_vis; vis[e] = cand & seen_vis;
+                n_keep_text += __popc(text[e]) << 16;
+                n_vis += __popc(vis[e]);
+            }
+        }
+        if (lane == 0) wsum[warp] = n_keep_text | (unsigned long long)n_vis << 32;
+        __syncthreads();
+        const unsigned long long mine = lane < kWarps ? wsum[lane] : 0ull;
+        const uint32_t kt_all = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)mine), v_all = __reduce_add_sync(0xFFFFFFFFu, (uint32_t)(mine >> 32));
+        const uint32_t kt = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? (uint32_t)mine : 0u);
+        const int n_text = (int)(kt_all >> 16), n_vis_all = (int)v_all, t0 = (n_text + 31) & ~31;   // text group first, visual group from the next multiple of 32
+        int s = (int)(kt & 0xFFFF), pt = (int)(kt >> 16), pv = t0 + (int)__reduce_add_sync(0xFFFFFFFFu, lane < warp ? (uint32_t)(mine >> 32) : 0u);
+        if (with_prepare) {                                          // the candidates, and the columns without one
+            int s1 = s;
+#pragma unroll
+            for (int e = 0; e < kE; ++e) {
+                const uint32_t bit = 1u << lane;
+                const int c = text[e] & bit ? pt + __popc(text[e] & lt) : vis[e] & bit ? pv + __popc(vis[e] & lt) : -1;
+                if (c >= 0 && index_ok(c, P.Ctot, P.status)) {
+                    slot_out[c] = s1 + __popc(keep[e] & lt);
+                    if (copy_here) cand_tok[c] = 32 * (w0 + e) + lane;
+                }
+                s1 += __popc(keep[e]); pt += __popc(text[e]); pv += __popc(vis[e]);
+            }
+            for (int c = n_text + tid; c < P.Ctot; c += kThreads)
+                if (c < t0 || c >= t0 + n_vis_all) {
+                    slot_out[c] = -1;
+                    scale_out[c] = __int_as_float(0x7FC00000);       // NaN: no candidate here
+                    if (copy_here) cand_tok[c] = -1;
+                }
+            if (tid == 0) { P.cand_count[2 * head] = n_text; P.cand_count[2 * head + 1] = n_vis_all; }
+        }
+        if (copy_here) __syncthreads();                              // every candidate's token is in place
+        constexpr int kRows = 4;                          // candidates' rows per thread on their way together
+        MatchGather<kRows> gather(P, head, tid, kThreads);
+        int p0 = tid >> 4;
+        if (copy_here) gather.start(cand_tok, p0, P.Ctot);
+#pragma unroll
+        for (int e = 0; e < kE; ++e) {
+            if (e >= per) break;
+            const int i = 32 * (w0 + e) + lane, sl = s + __popc(keep[e] & lt);
+            const bool out = i < L && !((keep[e] >> lane) & 1u), seen = by_list && i < L && words[i] >> 31;
+            if (out) {
+                evi[i - sl] = i;
+                if (copy_here) rank[i] = i - sl;
+                else if (by_list) evi_mod[i - sl] = seen;
+            } else if (i < L) {
+                ret[sl] = i;
+                if (A.row_mod_out) A.row_mod_out[(int64_t)head * A.B + sl] = mod[i];
+                if (copy_here) rank[i] = -(sl + 2);
+            }
+            if (by_list) {
+                // A word's non-pivots are neighbours in the list, of one tile or of two (a word of both modalities at a tile's
+                // edge may claim both for each: such a tile is then visited as a mixed one, with the same result).
+                const uint32_t o = __ballot_sync(0xFFFFFFFFu, out), m = __ballot_sync(0xFFFFFFFFu, seen);
+                const int first = 32 * (w0 + e) - s;
+                if (lane == 0 && o) {
+                    const uint32_t what = (o & ~m ? 1u : 0u) | (o & m ? 2u : 0u);
+                    atomicOr(&tiles[first / kMtItemRows], what);
+                    if (first % kMtItemRows + __popc(o) > kMtItemRows) atomicOr(&tiles[first / kMtItemRows + 1], what);
+                }
+            }
+            s += __popc(keep[e]);
+        }
+        if (copy_here) {
+            gather.finish(p0, P.Ctot);
+            for (p0 += kRows * gather.stride; p0 < P.Ctot; p0 += kRows * gather.stride) {   // (uniform trip count within a warp)
+                gather.start(cand_tok, p0, P.Ctot);
+                gather.finish(p0, P.Ctot);
+            }
+        } else if (by_list) {
+            __syncthreads();
+            for (int t = tid; t < P.n_rt; t += kThreads) P.tile_mod[(int64_t)head * P.n_rt + t] = (uint8_t)tiles[t];
+        }
+        return;
+    }
     auto block_sum = [&](unsigned long long v, unsigned long long &total) -> unsigned long long {   // exclusive prefix sum
         unsigned long long incl_v = v;
 #pragma unroll
@@ -303,24 +424,14 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
             }
             __syncthreads();
             // Pivots (24 bits), admissible text pivots (20) and admissible visual ones (20) before each word: one prefix sum
-            // for all three.  Up to 128 words every warp takes it for itself, four words to a lane, without a barrier.
+            // for all three.
             auto counts = [&](int w) -> unsigned long long {
                 return (unsigned long long)__popc(keep_w[w]) | (unsigned long long)__popc(text_w[w]) << 24 | (unsigned long long)__popc(vis_w[w]) << 44;
             };
-            const bool few = kOneChunk && n_w <= 128;
-            const int w_lo = min(n_w, few ? 4 * lane : tid * per), w_hi = min(n_w, w_lo + (few ? 4 : per));
-            unsigned long long mine = 0, all, before;
+            const int w_lo = min(n_w, tid * per), w_hi = min(n_w, w_lo + per);
+            unsigned long long mine = 0, all;
             for (int w = w_lo; w < w_hi; ++w) mine += counts(w);
-            if (few) {
-                before = mine;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned long long t = __shfl_up_sync(0xFFFFFFFFu, before, o);
-                    if (lane >= o) before += t;
-                }
-                all = __shfl_sync(0xFFFFFFFFu, before, 31);
-                before -= mine;
-            } else before = block_sum(mine, all);
+            const unsigned long long before = block_sum(mine, all);
             if (kCtas > 1) {                                         // (from here on `all` is the head's)
                 const unsigned long long ahead = cluster_sum(all, all);
                 seen = (int)(ahead & 0xFFFFFF); seen_t = (int)(ahead >> 24) & 0xFFFFF; seen_v = (int)(ahead >> 44);
@@ -333,12 +444,12 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
             if (kOneChunk) t0 = (n_text + 31) & ~31;                 // text group first, visual group from the next multiple of 32
             if (walk == 1) {
                 int s = seen + (int)(before & 0xFFFFFF), pt = seen_t + ((int)(before >> 24) & 0xFFFFF), pv = t0 + seen_v + (int)(before >> 44);
-                for (int w = w_lo; w < w_hi; ++w) {                  // (few: every warp writes the same values, and reads its own)
+                for (int w = w_lo; w < w_hi; ++w) {
                     pos_w[w] = s; pt_w[w] = pt; pv_w[w] = pv;
                     const unsigned long long c = counts(w);
                     s += (int)(c & 0xFFFFFF); pt += (int)(c >> 24) & 0xFFFFF; pv += (int)(c >> 44);
                 }
-                if (few) __syncwarp(); else __syncthreads();
+                __syncthreads();
 #pragma unroll 4
                 for (int w = warp; w < n_w; w += kWarps) {           // the lists, a word per warp and step: coalesced
                     const uint32_t keep = keep_w[w];

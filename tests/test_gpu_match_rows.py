@@ -74,9 +74,10 @@ def test_lists_of_any_length(E, layout):
     _check(k.astype(np.float64), m, ret, evi, strat, imp, 0.8, match.cpu().numpy(), sim.cpu().numpy().astype(np.float64))
 
 
-@pytest.mark.parametrize("U,H,L,B", [(2, 2, 700, 423), (1, 3, 4200, 2100), (3, 1, 9000, 900), (1, 1, 6144, 5000), (40, 1, 6200, 300), (1, 1, 46000, 230)])
+@pytest.mark.parametrize("U,H,L,B", [(2, 2, 700, 423), (2, 2, 1024, 300), (2, 1, 4096, 1000), (3, 2, 97, 40), (2, 2, 1024, 100), (2, 1, 4096, 224), (2, 1, 1025, 33), (1, 3, 4200, 2100), (3, 1, 9000, 900), (1, 1, 6144, 5000), (40, 1, 6200, 300), (1, 1, 46000, 230)])
 def test_selection_lays_the_rows_out(U, H, L, B):
-    """One and several words per thread, a cluster per head, contexts past one chunk; runs of a modality and tokens by turns."""
+    """One to eight words of 32 positions per warp, more of them in shared memory, a cluster per head, contexts past one chunk, short and
+    long candidate lists; runs of a modality and tokens by turns."""
     rng = np.random.default_rng(L)
     q = inputs.round_to_bf16(rng.standard_normal((U, H, 32, 128)).astype(np.float32))
     k = inputs.round_to_bf16(rng.standard_normal((U, H, L, 128)).astype(np.float32))
