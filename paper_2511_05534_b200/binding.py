@@ -104,8 +104,8 @@ class Params:
 
 
 # A call's C struct depends on the parameter fields and the tensors' strides alone, so the structs of the last few
-# hundred distinct calls are kept: building one takes about 8 us of Python, as long as the kernels of a small call run,
-# finding it again 1 us.  The library only reads them.
+# hundred distinct calls are kept, as the references that the calls pass: building one takes about 8 us of Python, as
+# long as the kernels of a small call run, finding it again 1 us.  The library only reads them.
 _FIELDS = operator.attrgetter("n_units", "n_q_heads", "n_kv_heads", "head_dim", "seq_len", "window", "n_keep", "dtype",
                               "softmax_scale", "theta", "tau", "tau_mode", "flow_mode", "merge_mode", "keep_window", "path")
 _MAX_STRUCTS = 512
@@ -115,16 +115,16 @@ _structs = {}
 def _keep_struct(key, cp):
     if len(_structs) >= _MAX_STRUCTS:
         _structs.clear()
-    _structs[key] = cp
-    return cp
+    _structs[key] = ref = ctypes.byref(cp)       # (holds on to the struct)
+    return ref
 
 
-def _params(p: Params, q=None, k=None, v=None, ko=None, vo=None) -> _CParams:
-    """p.c(...), out of the kept structs where the same fields and strides have been seen."""
+def _params(p: Params, q=None, k=None, v=None, ko=None, vo=None):
+    """A reference to p.c(...), out of the kept structs where the same fields and strides have been seen."""
     key = (_FIELDS(p), q is None or q.stride(), k is None or k.stride(), v is None or v.stride(), ko is None or ko.stride(),
            vo is None or vo.stride())
-    cp = _structs.get(key)
-    return cp if cp is not None else _keep_struct(key, p.c(q=q, k=k, v=v, ko=ko, vo=vo))
+    ref = _structs.get(key)
+    return ref if ref is not None else _keep_struct(key, p.c(q=q, k=k, v=v, ko=ko, vo=vo))
 
 
 _lib = None
@@ -213,7 +213,7 @@ def alloc_workspace(p: Params, device="cuda") -> torch.Tensor:
 
 def flowmm_score(p: Params, q_win, k, modality, importance, cross_mass, ws):
     cp = _params(p, q=q_win, k=k)
-    _check(load().flowmm_score(ctypes.byref(cp), _p(q_win), _p(k), _p(modality), _p(importance), _p(cross_mass),
+    _check(load().flowmm_score(cp, _p(q_win), _p(k), _p(modality), _p(importance), _p(cross_mass),
                                _p(ws), ws.numel(), _stream()), "flowmm_score")
 
 
@@ -230,32 +230,32 @@ def flowmm_full_flow(p: Params, q_full, k, modality, cross_mass, rho, strategy, 
         raise ValueError("expected a [units, heads, tokens, head_dim] tensor with contiguous head_dim")
     cp = _params(p, k=k)
     qs = (ctypes.c_int64 * 3)(q_full.stride(0), q_full.stride(1), q_full.stride(2))
-    _check(load().flowmm_full_flow(ctypes.byref(cp), _p(q_full), ctypes.byref(qs), _p(k), _p(modality), _p(cross_mass), _p(rho),
+    _check(load().flowmm_full_flow(cp, _p(q_full), ctypes.byref(qs), _p(k), _p(modality), _p(cross_mass), _p(rho),
                                    _p(strategy), _p(ws), ws.numel(), _stream()), "flowmm_full_flow")
 
 
 def flowmm_layer_flow(p: Params, cross_mass, rho, strategy):
     cp = _params(p)
-    _check(load().flowmm_layer_flow(ctypes.byref(cp), _p(cross_mass), _p(rho), _p(strategy), _stream()),
+    _check(load().flowmm_layer_flow(cp, _p(cross_mass), _p(rho), _p(strategy), _stream()),
            "flowmm_layer_flow")
 
 
 def flowmm_select(p: Params, importance, retained_idx, evicted_idx, ws):
     cp = _params(p)
-    _check(load().flowmm_select(ctypes.byref(cp), _p(importance), _p(retained_idx), _p(evicted_idx), _p(ws),
+    _check(load().flowmm_select(cp, _p(importance), _p(retained_idx), _p(evicted_idx), _p(ws),
                                 ws.numel(), _stream()), "flowmm_select")
 
 
 def flowmm_match(p: Params, k, importance, modality, retained_idx, evicted_idx, strategy, match, match_sim, ws):
     cp = _params(p, k=k)
-    _check(load().flowmm_match(ctypes.byref(cp), _p(k), _p(importance), _p(modality), _p(retained_idx),
+    _check(load().flowmm_match(cp, _p(k), _p(importance), _p(modality), _p(retained_idx),
                                _p(evicted_idx), _p(strategy), _p(match), _p(match_sim), _p(ws),
                                ws.numel(), _stream()), "flowmm_match")
 
 
 def flowmm_merge(p: Params, k, v, retained_idx, evicted_idx, match, match_sim, k_out, v_out, ws):
     cp = _params(p, k=k, v=v, ko=k_out, vo=v_out)
-    _check(load().flowmm_merge(ctypes.byref(cp), _p(k), _p(v), _p(retained_idx), _p(evicted_idx), _p(match),
+    _check(load().flowmm_merge(cp, _p(k), _p(v), _p(retained_idx), _p(evicted_idx), _p(match),
                                _p(match_sim), _p(k_out), _p(v_out), _p(ws), ws.numel(), _stream()),
            "flowmm_merge")
 
@@ -264,7 +264,7 @@ def flowmm_merge_static(p: Params, k, v, retained_idx, evicted_idx, match, match
     """flowmm_merge for callers that cannot allocate: no workspace argument, the scratch is a
     fixed array inside the library (see include/flowmm.h for its size limit and sharing rules)."""
     cp = _params(p, k=k, v=v, ko=k_out, vo=v_out)
-    _check(load().flowmm_merge_static(ctypes.byref(cp), _p(k), _p(v), _p(retained_idx), _p(evicted_idx), _p(match),
+    _check(load().flowmm_merge_static(cp, _p(k), _p(v), _p(retained_idx), _p(evicted_idx), _p(match),
                                       _p(match_sim), _p(k_out), _p(v_out), _stream()), "flowmm_merge_static")
 
 
@@ -280,7 +280,7 @@ def flowmm_merge_static_poke_status(word: int):
 def flowmm_compress_layer(p: Params, q_win, k, v, modality, k_out, v_out, ws, importance=None, rho=None,
                           strategy=None, retained_idx=None, evicted_idx=None, match=None, match_sim=None):
     cp = _params(p, q=q_win, k=k, v=v, ko=k_out, vo=v_out)
-    _check(load().flowmm_compress_layer(ctypes.byref(cp), _p(q_win), _p(k), _p(v), _p(modality), _p(k_out),
+    _check(load().flowmm_compress_layer(cp, _p(q_win), _p(k), _p(v), _p(modality), _p(k_out),
                                         _p(v_out), _p(importance), _p(rho), _p(strategy), _p(retained_idx),
                                         _p(evicted_idx), _p(match), _p(match_sim), _p(ws),
                                         ws.numel(), _stream()), "flowmm_compress_layer")
@@ -298,7 +298,7 @@ def flowmm_recompress(p: Params, q_win, k_cache, v_cache, row_modality, k_out, v
                       match_sim=None):
     """Section 3.3 again on a cache that grew during decoding; row_modality [units, kv_heads, rows] uint8."""
     cp = _params(p, q=q_win, k=k_cache, v=v_cache, ko=k_out, vo=v_out)
-    _check(load().flowmm_recompress(ctypes.byref(cp), _p(q_win), _p(k_cache), _p(v_cache), _p(row_modality), _p(k_out),
+    _check(load().flowmm_recompress(cp, _p(q_win), _p(k_cache), _p(v_cache), _p(row_modality), _p(k_out),
                                     _p(v_out), _p(row_modality_out), _p(importance), _p(rho), _p(strategy),
                                     _p(retained_idx), _p(evicted_idx), _p(match), _p(match_sim), _p(ws),
                                     ws.numel(), _stream()), "flowmm_recompress")
@@ -336,15 +336,21 @@ def _decode_params(q, k, v, softmax_scale: float, path: int) -> _CDecodeParams:
 def flowmm_decode_workspace_bytes(q, k, v, softmax_scale: float = 0.0, path: int = PATH_AUTO) -> int:
     n = ctypes.c_size_t(0)
     cp = _decode_params(q, k, v, softmax_scale, path)
-    _check(load().flowmm_decode_workspace_bytes(ctypes.byref(cp), ctypes.byref(n)), "flowmm_decode_workspace_bytes")
+    _check(load().flowmm_decode_workspace_bytes(cp, ctypes.byref(n)), "flowmm_decode_workspace_bytes")
     return int(n.value)
 
 
 def flowmm_decode_attention(q, k, v, out, ws, softmax_scale: float = 0.0, path: int = PATH_AUTO):
     """Eq. 4 for one new query per head over the cache rows of k, v; out [units, q_heads, head_dim] float32."""
-    cp = _decode_params(q, k, v, softmax_scale, path)
-    _check(load().flowmm_decode_attention(ctypes.byref(cp), _p(q), _p(k), _p(v), _p(out), _p(ws),
-                                          ws.numel(), _stream()), "flowmm_decode_attention")
+    # One launch of 5 us on a short cache, so Python sets the pace of its calls: _p() and _stream() are written out (the
+    # tensors are on a GPU, so CUDA is up and the device need not be asked for through torch.cuda).
+    ref = _decode_params(q, k, v, softmax_scale, path)
+    if not (q.is_cuda and k.is_cuda and v.is_cuda and ws.is_cuda):
+        raise ValueError("flowmm takes CUDA tensors")
+    code = (_lib or load()).flowmm_decode_attention(ref, q.data_ptr(), k.data_ptr(), v.data_ptr(), _p(out), ws.data_ptr(), ws.numel(),
+                                                    torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+    if code != 0:
+        raise FlowmmError(code, "flowmm_decode_attention")
 
 
 def flowmm_selftest_wait_timeout(ws):
