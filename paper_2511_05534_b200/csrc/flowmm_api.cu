@@ -101,7 +101,7 @@ struct Layout {
     size_t cand_k, cand_scale, cand_slot, cand_count, rank, evi_mod, tile_mod, row_all;
     size_t tokmap;             // [UH, L] (slot, weight) of every token position, for the tensor-core merge
     size_t merge_status;       // status word the merge kernels report to (the workspace's own, or one of the merge scratch)
-    int tc_n_qt, tc_runs, tc_n_part;
+    int tc_q_rows, tc_keys2, tc_n_qt, tc_runs, tc_n_part;
     size_t total;
     int n_chunk1, chunk1, n_chunk2, chunk2, max_parts, csr_passes, merge_win, n_win, c_tot, n_rt, n_et;
 };
@@ -170,8 +170,15 @@ Layout make_layout(const flowmm_params &p) {
     y.match = take(U * Hkv * E * 4);
     y.match_sim = take(U * Hkv * E * 4);
     y.n_rt = (int)((L + tcs::kItemRows - 1) / tcs::kItemRows);
-    // pass 1 of the tensor-core scoring: the key tiles of all heads in equal runs, one per SM and tile of 256 proxy rows
-    y.tc_n_qt = (int)((G * W + tcs::kItemRows - 1) / tcs::kItemRows);
+    // Items of 256 proxy rows (pass 1) or keys (pass 2) take two halves of 128 against every operand tile.  Where that leaves SMs
+    // idle and items of one half still have an SM each, they are of one half: their products and exponentials then take half as
+    // long.  The whole call, us, 256 and 128: 8 heads of 1471 tokens, 224 rows 34.8, 32.8; 4 of 500 30.6, 28.1; 4 of 2300 45.1, 43.4;
+    // 4 of 4500 51.8, 50.1; 8 of 1000, 512 rows 35.7, 32.8; 4 caches of 640 rows 37.2, 34.8; where pass 2 alone is cut finer 8 of
+    // 2300 42.2, 41.1.  With more items than SMs the second round costs what the finer cut gains.
+    y.tc_q_rows = G * W > tcs::kRows && U * Hkv * (size_t)y.n_rt * ((G * W + tcs::kRows - 1) / tcs::kRows) <= kScoreCtas ? tcs::kRows : tcs::kItemRows;
+    y.tc_keys2 = U * Hkv * ((L + tcs::kRows - 1) / tcs::kRows) <= kScoreCtas ? tcs::kRows : tcs::kItemRows;
+    // pass 1 of the tensor-core scoring: the key tiles of all heads in equal runs, one per SM and tile of proxy rows
+    y.tc_n_qt = (int)((G * W + y.tc_q_rows - 1) / y.tc_q_rows);
     {
         const size_t tiles = U * Hkv * (size_t)y.n_rt, runs = kScoreCtas > y.tc_n_qt ? kScoreCtas / y.tc_n_qt : 1;
         y.tc_runs = (int)(tiles < runs ? tiles : runs);
@@ -313,18 +320,19 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
     a.row_part = at<float4>(ws, y.row_part); a.modality = mod;
     a.importance = importance; a.cross_part = at<float>(ws, y.cross_part); a.status = at<int>(ws, y.status);
     a.Hq = p.n_q_heads; a.Hkv = p.n_kv_heads; a.G = G; a.W = W; a.L = p.seq_len; a.GW = G * W;
-    a.n_qt = y.tc_n_qt; a.n_runs1 = y.tc_runs; a.n_part = y.tc_n_part; a.n_rt = y.n_rt;
+    a.q_rows = y.tc_q_rows; a.n_qt = y.tc_n_qt; a.n_runs1 = y.tc_runs; a.n_part = y.tc_n_part; a.n_rt = y.n_rt;
     a.a_heads = G < tcs::kRows / W ? G : tcs::kRows / W;        // one A half holds 128 proxy rows
     // pass 2 streams the keys as the A operand; with up to 256 proxy rows per KV head the shapes with two A stages keep
     // the key loads in flight across items
     const bool small2 = a.GW <= 128 && W <= 64, resident2 = !small2 && a.GW <= 256;
     const int nb2 = small2 ? tcs::Small::kCols : tcs::Big::kCols;
     a.b_heads = G < nb2 / W ? G : nb2 / W;
-    a.n_tiles1 = a.n_items2 = UH * a.n_rt;
+    a.n_tiles1 = UH * a.n_rt;
+    a.keys2 = y.tc_keys2; a.n_rt2 = (p.seq_len + a.keys2 - 1) / a.keys2; a.n_items2 = UH * a.n_rt2;
     const int grid1 = a.n_runs1 * a.n_qt;
     const int grid2 = a.n_items2 < tc::sm_count() ? a.n_items2 : tc::sm_count();
     a.by_grid1 = make_fastdiv((uint32_t)grid1); a.by_grid2 = make_fastdiv((uint32_t)grid2);
-    a.by_hkv = make_fastdiv((uint32_t)p.n_kv_heads); a.by_rt = make_fastdiv((uint32_t)a.n_rt);
+    a.by_hkv = make_fastdiv((uint32_t)p.n_kv_heads); a.by_rt = make_fastdiv((uint32_t)a.n_rt); a.by_rt2 = make_fastdiv((uint32_t)a.n_rt2);
     a.by_tiles = make_fastdiv((uint32_t)a.n_tiles1);
     const float scale = p.softmax_scale != 0.f ? p.softmax_scale : 1.f / sqrtf((float)p.head_dim);
     a.scale_log2 = scale * kLog2e;

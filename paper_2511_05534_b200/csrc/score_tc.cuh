@@ -27,12 +27,13 @@ struct ScoreTcArgs {
     float *cross_part;           // [U*Hq, W] share of a proxy row's mass that falls on keys of the other modality
     int *status;
     int Hq, Hkv, G, W, L, GW;
-    int n_qt;                    // 256-row tiles over the G*W proxy rows
+    int q_rows, n_qt;            // pass 1: proxy rows of an item (256, or 128: one half), tiles of so many over the G*W rows
     int n_runs1;                 // pass 1: runs that the key tiles of all heads are cut into
-    FastDiv by_grid1, by_grid2, by_hkv, by_rt, by_tiles;   // exact divisions by the passes' grids, Hkv, n_rt, n_tiles1
+    FastDiv by_grid1, by_grid2, by_hkv, by_rt, by_rt2, by_tiles;   // exact divisions by the passes' grids, Hkv, n_rt, n_rt2, n_tiles1
     int n_rt;                    // 256-key tiles of a head
+    int keys2, n_rt2;            // pass 2: keys of an item (256, or 128: one half), items of a head
     int a_heads, b_heads;        // query heads one A box (pass 1) / B box (pass 2) delivers
-    int n_tiles1, n_items2;      // key tiles of all heads, for either pass
+    int n_tiles1, n_items2;      // key tiles and items of all heads
     float scale_log2;
 };
 
@@ -170,7 +171,7 @@ __device__ __forceinline__ RowStats join(const RowStats &a, const RowStats &b) {
 
 // ---------------------------------------------------------------------------------------------
 // Pass 1.  The 256-key tiles of all heads, one head's behind the other's, are cut into equal runs; a CTA takes a run for one tile
-// of 256 proxy rows (CTAs next to each other share a run, whose keys the second of them finds in L2).  item = a run's part of one
+// of 256 proxy rows, or of 128 (CTAs next to each other share a run, whose keys the second of them finds in L2).  item = a run's part of one
 // head.  Whole heads or equal chunks of them as items left SMs idle in the last round.  The whole call, us, so and now: 112 heads of
 // 2176 tokens, 224 rows 116.1 / 111.9; of 8448, 448 rows 867 / 851; 112 caches of 640 rows 97.9 / 95.6; 80 heads of 7906, 512
 // rows 419 / 394; 128 of 33 792 2947 / 2904.
@@ -196,9 +197,9 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
         tcs::TilePlan p;
         const int uh = uh_lo + (int)A.by_grid1.div(item), u = (int)A.by_hkv.div(uh), h = uh - u * A.Hkv, head0 = uh * A.n_rt;
         const int t0 = max(t_lo, head0) - head0, t1 = min(t_hi, head0 + A.n_rt) - head0;
-        p.a1 = 0; p.a2 = h * A.G + qt * (tcs::kItemRows / A.W); p.a3 = u;
+        p.a1 = 0; p.a2 = h * A.G + qt * (A.q_rows / A.W); p.a3 = u;
         p.h1 = 0; p.h2 = tcs::kRows / A.W;
-        p.n_halves = qt * tcs::kItemRows + tcs::kRows < A.GW ? 2 : 1;
+        p.n_halves = A.q_rows > tcs::kRows && qt * A.q_rows + tcs::kRows < A.GW ? 2 : 1;
         p.b1 = t0 * S::kCols; p.b2 = h; p.b3 = u; p.step1 = S::kCols; p.step2 = 0;
         p.cols_total = min(A.L, t1 * S::kCols) - p.b1;
         p.n_tiles = t1 - t0;
@@ -265,7 +266,7 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
                     if (h >= p.n_halves) continue;
                     if (ok) ok = S::acc_wait_h(c, h, kh[h], A.status);
                     ++kh[h];
-                    const int r0 = qt * tcs::kItemRows + h * tcs::kRows;
+                    const int r0 = qt * A.q_rows + h * tcs::kRows;
                     auto release = [&]() { if (ok) S::acc_release_h(c, h); };
                     if (r0 + c.quarter * 32 >= A.GW) release();
                     else if (plain) {
@@ -312,7 +313,7 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
                     tc::sts32(at, st[h].m); tc::sts32(at + 4, st[h].t); tc::sts32(at + 8, st[h].v);
                 }
             ok = !__any_sync(0xFFFFFFFFu, tcs::meet_vote(1 + c.quarter, 128, !ok));   // (the vote: for the compiler, which then knows the warp to be of one mind)
-            const int r = qt * tcs::kItemRows + colq * tcs::kRows + row_in_half;
+            const int r = qt * A.q_rows + colq * tcs::kRows + row_in_half;
             if (colq < p.n_halves && r < A.GW) {
                 RowStats s = colq == 0 ? st[0] : st[1];
 #pragma unroll
@@ -414,7 +415,7 @@ __device__ __forceinline__ void colsum_chunk32(uint32_t (&a)[32], uint32_t negc,
 #undef FLOWMM_EX_REGS
 
 // ---------------------------------------------------------------------------------------------
-// Pass 2.  item = (unit*head, tile of 256 keys); the B stream is the head group's proxy rows.  A CTA takes a run of
+// Pass 2.  item = (unit*head, tile of 256 keys, or of 128 where few items leave SMs idle); the B stream is the head group's proxy rows.  A CTA takes a run of
 // consecutive items, so that proxy rows that fit the B stages (up to 512) are loaded once per head, not once per item.
 // Row constants -(max + log2 sum) - exp2(logit + constant) is the softmax probability - are formed from pass 1's statistics by
 // the epilogue warps when the run comes to another head; the CTA with a head's first tile also writes its rows' cross-modal shares.
@@ -433,16 +434,16 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
     const int n_loop = (g_hi - g_lo) * gridDim.x;                   // the roles count items blockIdx.x, blockIdx.x + gridDim.x, ...
     auto plan = [&](int item) {
         tcs::TilePlan p;
-        const int g = g_lo + (int)A.by_grid2.div(item), uh = (int)A.by_rt.div(g), kt = g - uh * A.n_rt;
+        const int g = g_lo + (int)A.by_grid2.div(item), uh = (int)A.by_rt2.div(g), kt = g - uh * A.n_rt2;
         const int u = (int)A.by_hkv.div(uh), h = uh - u * A.Hkv;
-        p.a1 = kt * tcs::kItemRows; p.a2 = h; p.a3 = u;
+        p.a1 = kt * A.keys2; p.a2 = h; p.a3 = u;
         p.h1 = tcs::kRows; p.h2 = 0;
-        p.n_halves = p.a1 + tcs::kRows < A.L ? 2 : 1;
+        p.n_halves = A.keys2 > tcs::kRows && p.a1 + tcs::kRows < A.L ? 2 : 1;
         p.b1 = 0; p.b2 = h * A.G; p.b3 = u; p.step1 = 0; p.step2 = S::kCols / A.W;
         p.cols_total = A.GW;
         p.n_tiles = (A.GW + S::kCols - 1) / S::kCols;
         p.reuse_b = p.n_tiles <= S::kBStages && kt > 0 && g > g_lo;
-        p.keep_b = p.n_tiles <= S::kBStages && kt + 1 < A.n_rt && g + 1 < g_hi;
+        p.keep_b = p.n_tiles <= S::kBStages && kt + 1 < A.n_rt2 && g + 1 < g_hi;
         p.extra = nullptr;
         return p;
     };
@@ -462,7 +463,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
         // the run's items one after the other: (unit u, KV head uh, its tile kt) step by step instead of by divisions, which
         // together with the rest of an item's start took a tenth of the epilogue's time
         const int n_tiles = (A.GW + S::kCols - 1) / S::kCols;
-        int uh = (int)A.by_rt.div(g_lo), kt = g_lo - uh * A.n_rt, u = (int)A.by_hkv.div(uh), hk = uh - u * A.Hkv;
+        int uh = (int)A.by_rt2.div(g_lo), kt = g_lo - uh * A.n_rt2, u = (int)A.by_hkv.div(uh), hk = uh - u * A.Hkv;
         uint32_t slot = 0, consts = c.base + S::kSmemEpi + kConstBytes;
         for (int g = g_lo; g < g_hi; ++g) {
             const int uh0 = uh, kt0 = kt;                            // this item
@@ -498,12 +499,12 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                 // (the set written was read two heads ago, and every warp has been through the meeting of the head between)
                 tcs::named_barrier(9, 32 * tcs::kEpiWarps);
             }
-            if (++kt == A.n_rt) {                                    // the next item
+            if (++kt == A.n_rt2) {                                    // the next item
                 kt = 0; ++uh;
                 if (++hk == A.Hkv) { hk = 0; ++u; }
             }
-            const int key0 = kt0 * tcs::kItemRows + c.group * tcs::kRows;
-            if (key0 >= A.L) continue;                               // no keys in this half
+            const int key0 = kt0 * A.keys2 + c.group * tcs::kRows;
+            if (key0 >= A.L || c.group * tcs::kRows >= A.keys2) continue;   // no keys in this half
             const int key = key0 + row;
             const bool masked_tile = key0 + tcs::kRows > A.L - A.W + 1;   // some (key, proxy row) pair is masked
             const int first_proxy = A.L - A.W;

@@ -72,3 +72,11 @@ def test_runs_of_tiles_across_heads(U, G, W, L):
 def test_many_key_chunks_of_one_head(L):
     rng = np.random.default_rng(L)
     _check(rng, 1, 8, 1, L, 64, np.arange(L)[None] // 1000 % 2)
+
+
+@pytest.mark.parametrize("U,G,W,L", [(74, 2, 128, 256), (75, 2, 128, 256), (74, 2, 128, 257), (18, 8, 128, 200), (19, 8, 128, 200),
+                                     (148, 5, 32, 128), (149, 5, 32, 128), (49, 5, 32, 384), (50, 5, 32, 385), (2, 5, 32, 129)])
+def test_items_of_one_half_and_of_two(U, G, W, L):
+    """Both sides of the lines at which either pass goes from items of 128 proxy rows or keys to items of 256."""
+    rng = np.random.default_rng(U * L)
+    _check(rng, U, G, 1, L, W, np.arange(L)[None] // 50 % 2 ^ rng.integers(0, 2, (U, 1)))
