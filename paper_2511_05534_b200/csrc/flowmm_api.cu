@@ -960,6 +960,8 @@ flowmm_status run_flow_tc(const flowmm_params &p, const void *q, const int64_t q
     a.Hq = p.n_q_heads; a.Hkv = p.n_kv_heads; a.G = p.n_q_heads / p.n_kv_heads; a.L = p.seq_len;
     a.n_rp = (p.seq_len + tcs::kItemRows - 1) / tcs::kItemRows; a.n_heads = p.n_units * p.n_q_heads; a.mod_words = mod_words;
     a.n_items = a.n_heads * a.n_rp;
+    const int sms = tc::sm_count(), grid = a.n_items < sms ? a.n_items : sms;
+    a.by_grid = make_fastdiv((uint32_t)grid); a.n_rounds = (a.n_items + grid - 1) / grid;
     const float scale = p.softmax_scale != 0.f ? p.softmax_scale : 1.f / sqrtf((float)p.head_dim);
     a.scale_log2 = scale * kLog2e;
     // every block of rows reads its head's keys again: the keys of a group of heads take at most 48 MB of the 126 MB L2
@@ -978,8 +980,7 @@ flowmm_status run_flow_tc(const flowmm_params &p, const void *q, const int64_t q
     if (!tc::make_bf16_map(&qa, q, 4, qd, qs, bqa) || !tc::make_bf16_map(&k256, k, 4, kd, ks, bk256)) return FLOWMM_ERR_CUDA;
     if (cudaFuncSetAttribute(flow_stats_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcs::Big::kSmemBytes) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
-    const int sms = tc::sm_count();
-    launch(flow_stats_tc_kernel, a.n_items < sms ? a.n_items : sms, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
+    launch(flow_stats_tc_kernel, grid, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
     FLOWMM_LAUNCHED("flow_stats_tc");
     return FLOWMM_OK;
 }

@@ -116,3 +116,16 @@ def test_heads_in_several_groups_equal_the_units_alone(L):
     for u in (0, 10, 11, 12):
         c1, r1 = run(u, u + 1)
         assert torch.equal(cross[u], c1[0]) and torch.equal(rho[u], r1[0])
+
+
+@pytest.mark.parametrize("U,Hq,Hkv,L", [(149, 1, 1, 200), (37, 4, 2, 257), (5, 28, 4, 300), (75, 2, 1, 520), (12, 37, 1, 260)])
+def test_rounds_of_items(U, Hq, Hkv, L):
+    """More items than SMs: two to six rounds, the last of them full, nearly full or of one item.  Tolerance: exponentials within 4e-6
+    and sums of fp32 parts within 1e-6 of their values, so a row's share within 1e-5 of the row's mass 1."""
+    rng = np.random.default_rng(U)
+    q = inputs.round_to_bf16(rng.standard_normal((U, Hq, L, 128)).astype(np.float32))
+    k = inputs.round_to_bf16(rng.standard_normal((U, Hkv, L, 128)).astype(np.float32))
+    m = (np.arange(L)[None] // 90 % 2 ^ rng.integers(0, 2, (U, 1))).astype(np.uint8)
+    cross, rho, _ = _oracle(U, Hq, Hkv, 128, L, q, k, m, 0.35)
+    g_cross, g_rho, _ = _gpu(U, Hq, Hkv, 128, L, q, k, m, 0.35, F.BF16)
+    assert np.abs(g_cross - cross).max() < 1e-5 * L and np.abs(g_rho - rho).max() < 1e-5
