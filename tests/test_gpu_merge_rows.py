@@ -90,3 +90,29 @@ def test_many_rows_draw_their_windows():
     for got, (ref, bound) in zip(out, refs):
         assert np.all(np.abs(got[:, :1].double().cpu().numpy() - ref) <= bound)
         assert torch.equal(got, got[:, :1].expand(-1, heads, -1, -1))
+
+
+@pytest.mark.parametrize("E", [1, 33, 300, 2047, 2048, 2049, 4096])
+def test_lists_of_many_heads(E):
+    """150 heads, so a block per head: positions kept from the first walk (up to 2048) and staged, a sixth of them dropped."""
+    rng = np.random.default_rng(E)
+    heads, B, D = 150, 700, 128
+    L = E + B
+    k, v = (small_integers(rng, (1, 1, L, D)) for _ in range(2))
+    ret = np.sort(rng.choice(L, B, replace=False))
+    evi = np.setdiff1d(np.arange(L), ret)
+    match = np.where(rng.random(E) < 1 / 6, -1, np.minimum(rng.integers(0, B, E), rng.integers(0, 2 * B, E)))   # (some slots popular)
+    sim = np.where(match >= 0, rng.random(E), 0).astype(np.float32)[None, None]
+    ret, evi, match = (x.astype(np.int32)[None, None] for x in (ret, evi, match))
+    rep = lambda x: torch.from_numpy(np.ascontiguousarray(np.repeat(x, heads, 1))).cuda()
+    lists = [rep(x) for x in (ret, evi, match, sim)]
+    for mode in (F.MERGE_MEAN, F.MERGE_EXPSIM):
+        refs = merge_reference(O.OracleParams(1, 1, 1, D, L, 1, B, merge_mode=mode), k, v, ret, evi, match, sim.astype(np.float64), F.BF16)
+        fp = gpu_params(O.OracleParams(1, heads, heads, D, L, 1, B, merge_mode=mode), F.BF16)
+        out = [torch.full((1, heads, B, D), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        ws = F.alloc_workspace(fp)
+        F.flowmm_merge(fp, rep(k).bfloat16(), rep(v).bfloat16(), *lists, out[0], out[1], ws)
+        assert F.flowmm_last_device_status(ws) == 0
+        for got, (ref, bound) in zip(out, refs):
+            assert np.all(np.abs(got[:, :1].double().cpu().numpy() - ref) <= bound), mode
+            assert torch.equal(got, got[:, :1].expand(-1, heads, -1, -1))
