@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
     predecessor_done();
     const bool is_v = lane >= 16;
     const int c0 = (lane & 15) * V;
-    const uint32_t row_bytes = (uint32_t)((is_v ? A.vs[2] : A.ks[2]) * sizeof(T));   // (32 bits: hundreds of rows of 4 GB each are no GPU's)
+    const int64_t row_bytes = (is_v ? A.vs[2] : A.ks[2]) * (int64_t)sizeof(T);   // (two rows may be more than 4 GB apart)
     const unsigned n_warps = gridDim.x * kWarps;
 
     // what an item needs from global memory, a word of 32 rows per register
@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
                     int tok = __float_as_int(tc::lds32(ents + (lo + q) * 8)) & kRowToken;
                     if (!index_ok(tok, A.L, status)) tok = 0;
                     const uint32_t dst = bufs + (gi & (kStages - 1)) * kStage + q * kRow;
-                    const char *from = src + (uint64_t)(uint32_t)tok * row_bytes;
+                    const char *from = src + tok * row_bytes;
                     if constexpr (kBytes == 8) tc::copy8_async(dst, from);
                     else tc::copy16_async(dst, from);
                     if constexpr (kBytes == 32) tc::copy16_async(dst + 16, from + 16);

@@ -116,3 +116,26 @@ def test_lists_of_many_heads(E):
         for got, (ref, bound) in zip(out, refs):
             assert np.all(np.abs(got[:, :1].double().cpu().numpy() - ref) <= bound), mode
             assert torch.equal(got, got[:, :1].expand(-1, heads, -1, -1))
+
+
+@pytest.mark.parametrize("dtype,D,E", [(F.BF16, 128, 0), (F.BF16, 64, 0), (F.BF16, 64, 1), (F.F32, 64, 0), (F.F32, 128, 1)])
+def test_rows_gigabytes_apart(dtype, D, E):
+    """Two or three rows, 4 GiB between one and the next (a byte offset that 32 bits do not hold): pivots alone, and a merged row of
+    each of so many heads, all on the same rows, that their lists are sorted."""
+    B, heads = 2, 1 if E == 0 else 20000
+    L, apart = B + E, 2 ** 32 // torch.empty((), dtype=F.torch_dtype(dtype)).element_size()
+    rows = torch.arange(1, 1 + L * D, device="cuda").reshape(L, D).remainder(50).to(F.torch_dtype(dtype))
+    k, v = (torch.zeros((L - 1) * apart + D, dtype=F.torch_dtype(dtype), device="cuda").as_strided((1, heads, L, D), (0, 0, apart, 1)) for _ in range(2))
+    k[0, 0], v[0, 0] = rows, rows.flip(0)
+    fp = F.Params(1, heads, heads, D, L, 1, B, dtype=dtype, merge_mode=F.MERGE_MEAN)
+    ret = torch.tensor([0, L - 1], dtype=torch.int32, device="cuda").expand(1, heads, B).contiguous()
+    evi, match = (torch.full((1, heads, E), x, dtype=torch.int32, device="cuda") for x in (1, 0))
+    out = [torch.full((1, heads, B, D), float("nan"), dtype=F.torch_dtype(dtype), device="cuda") for _ in range(2)]
+    ws = F.alloc_workspace(fp)
+    F.flowmm_merge(fp, k, v, ret, evi, match, torch.zeros((1, heads, E), device="cuda"), out[0], out[1], ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    for got, src in zip(out, (rows, rows.flip(0))):
+        want = src[[0, L - 1]].clone()
+        if E:
+            want[0] = ((src[0].float() + src[1].float()) / 2).to(want.dtype)     # (exact: halves of small integers)
+        assert torch.equal(got, want.expand(1, heads, B, D))
