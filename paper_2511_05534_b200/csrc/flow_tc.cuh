@@ -9,7 +9,7 @@
 //
 // Bound by the epilogue: Hq L^2 / 2 exponentials per unit, a quarter of them as a polynomial on the FMA pipe, with four
 // warps per scheduler to cover the latencies (half of the issue slots used; TMA and MMA alone take half the time).  A chunk
-// becomes exponentials in place, whatever is masked or mixed in it (28 x 28 heads x 2176 tokens 664 -> 641 us at the power
+// becomes exponentials in place (28 x 28 heads x 2176 tokens 664 -> 641 us at the power
 // cap; reading the next chunk ahead, which costs another 32 registers, gives that back).  The
 // form before launched the statistics once per 128 query rows, with a join of all partial statistics after each: launches
 // of a few hundred items in one to three uneven rounds, 1190 us for 28 layers of 28 heads and 2176 tokens against 595 us.
@@ -110,17 +110,25 @@ flow_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_con
                 const int ncols = min(S::kCols, min(r0 + 32, A.L) - kb);
                 S::for_each_chunk(c, (ncols + 31) >> 5, [&](int ch, uint32_t (&acc)[32]) {
                     const int k0 = kb + ch * 32;
-                    uint32_t other = bits[k0 >> 5] ^ flip;               // keys of the other modality than the row's token
-                    if (k0 >= r0) {                                  // the chunk on the diagonal: exp2 of what is masked gives 0 (or 2^-125)
-                        other &= 0xFFFFFFFFu >> (31 - c.lane);
+                    const uint32_t word = bits[k0 >> 5];
+                    uint32_t other = word ^ flip;                        // keys of the other modality than the row's token
+                    float mx, add, addc;
+                    // Where a few keys can make up a share - on the diagonal and in words of both modalities - all exponentials are
+                    // the exp2 unit's: with the polynomial in a quarter of them a share was off by up to 7e-7 instead of 2e-7.
+                    if (k0 < r0 && (word == 0u || word == 0xFFFFFFFFu)) {
+                        mx = fmaxf(max32(acc) * A.scale_log2, m);
+                        exp2_32(acc, A.scale_log2, mx);
+                        add = sum32(acc);
+                        addc = other != 0u ? add : 0.f;
+                    } else {
+                        if (k0 >= r0) {                              // the chunk on the diagonal: exp2 of what is masked gives 0
+                            other &= 0xFFFFFFFFu >> (31 - c.lane);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) acc[j] = j <= c.lane ? acc[j] : __float_as_uint(-INFINITY);
-                    }
-                    const float mx = fmaxf(max32(acc) * A.scale_log2, m);
-                    exp2_32(acc, A.scale_log2, mx);
-                    const float add = sum32(acc);
-                    float addc = other == 0xFFFFFFFFu ? add : 0.f;
-                    if (other != 0u && other != 0xFFFFFFFFu) {
+                            for (int j = 0; j < 32; ++j) acc[j] = j <= c.lane ? acc[j] : __float_as_uint(-INFINITY);
+                        }
+                        mx = fmaxf(max32(acc) * A.scale_log2, m);
+                        exp2_32_exact(acc, A.scale_log2, mx);
+                        add = sum32(acc);
                         float x[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                         for (int j = 0; j < 32; ++j) x[j & 3] += ((other >> j) & 1u) ? __uint_as_float(acc[j]) : 0.f;

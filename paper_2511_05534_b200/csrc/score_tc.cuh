@@ -108,26 +108,33 @@ __device__ __forceinline__ float exp_sum32(const uint32_t (&a)[32], float scale_
     FLOWMM_EX_E(8) FLOWMM_EX_E(9) FLOWMM_EX_E(10) FLOWMM_EX_E(11) FLOWMM_EX_E(12) FLOWMM_EX_E(13) FLOWMM_EX_POLY(14, 15)            \
     FLOWMM_EX_E(16) FLOWMM_EX_E(17) FLOWMM_EX_E(18) FLOWMM_EX_E(19) FLOWMM_EX_E(20) FLOWMM_EX_E(21) FLOWMM_EX_POLY(22, 23)          \
     FLOWMM_EX_E(24) FLOWMM_EX_E(25) FLOWMM_EX_E(26) FLOWMM_EX_E(27) FLOWMM_EX_E(28) FLOWMM_EX_E(29) FLOWMM_EX_POLY(30, 31)
+#define FLOWMM_EX_HW                                                                                                              \
+    FLOWMM_EX_E(0) FLOWMM_EX_E(1) FLOWMM_EX_E(2) FLOWMM_EX_E(3) FLOWMM_EX_E(4) FLOWMM_EX_E(5) FLOWMM_EX_E(6) FLOWMM_EX_E(7)          \
+    FLOWMM_EX_E(8) FLOWMM_EX_E(9) FLOWMM_EX_E(10) FLOWMM_EX_E(11) FLOWMM_EX_E(12) FLOWMM_EX_E(13) FLOWMM_EX_E(14) FLOWMM_EX_E(15)    \
+    FLOWMM_EX_E(16) FLOWMM_EX_E(17) FLOWMM_EX_E(18) FLOWMM_EX_E(19) FLOWMM_EX_E(20) FLOWMM_EX_E(21) FLOWMM_EX_E(22) FLOWMM_EX_E(23)  \
+    FLOWMM_EX_E(24) FLOWMM_EX_E(25) FLOWMM_EX_E(26) FLOWMM_EX_E(27) FLOWMM_EX_E(28) FLOWMM_EX_E(29) FLOWMM_EX_E(30) FLOWMM_EX_E(31)
 #define FLOWMM_EX_REGS(a)                                                                                                          \
     "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]), "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), \
         "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15]), "+r"(a[16]), "+r"(a[17]), "+r"(a[18]), "+r"(a[19]), "+r"(a[20]), \
         "+r"(a[21]), "+r"(a[22]), "+r"(a[23]), "+r"(a[24]), "+r"(a[25]), "+r"(a[26]), "+r"(a[27]), "+r"(a[28]), "+r"(a[29]), "+r"(a[30]), \
         "+r"(a[31])
 
-// a = 2^(a * scale - mx), in place (all 32 with the same mx)
-__device__ __forceinline__ void exp2_32(uint32_t (&a)[32], float scale_log2, float mx) {
-    asm volatile(
-        "{\n\t" FLOWMM_EX_DECL ".reg .b64 ng;\n\t"
-        "mov.b64 sc, {%32, %32};\n\t"
-        "mov.b64 ng, {%33, %33};\n\t"
-        FLOWMM_EX_FMA(0, 1, "ng") FLOWMM_EX_FMA(2, 3, "ng") FLOWMM_EX_FMA(4, 5, "ng") FLOWMM_EX_FMA(6, 7, "ng")
-        FLOWMM_EX_FMA(8, 9, "ng") FLOWMM_EX_FMA(10, 11, "ng") FLOWMM_EX_FMA(12, 13, "ng") FLOWMM_EX_FMA(14, 15, "ng")
-        FLOWMM_EX_FMA(16, 17, "ng") FLOWMM_EX_FMA(18, 19, "ng") FLOWMM_EX_FMA(20, 21, "ng") FLOWMM_EX_FMA(22, 23, "ng")
-        FLOWMM_EX_FMA(24, 25, "ng") FLOWMM_EX_FMA(26, 27, "ng") FLOWMM_EX_FMA(28, 29, "ng") FLOWMM_EX_FMA(30, 31, "ng")
-        FLOWMM_EX_ALL "}"
-        : FLOWMM_EX_REGS(a)
-        : "f"(scale_log2), "f"(-mx));
-}
+// a = 2^(a * scale - mx), in place (all 32 with the same mx).  exp2_32_exact: by the exp2 unit alone, within 2^-22 of the value.
+#define FLOWMM_EX2_32(EXPS)                                                                                                       \
+    asm volatile(                                                                                                                 \
+        "{\n\t" FLOWMM_EX_DECL ".reg .b64 ng;\n\t"                                                                                 \
+        "mov.b64 sc, {%32, %32};\n\t"                                                                                             \
+        "mov.b64 ng, {%33, %33};\n\t"                                                                                             \
+        FLOWMM_EX_FMA(0, 1, "ng") FLOWMM_EX_FMA(2, 3, "ng") FLOWMM_EX_FMA(4, 5, "ng") FLOWMM_EX_FMA(6, 7, "ng")                     \
+        FLOWMM_EX_FMA(8, 9, "ng") FLOWMM_EX_FMA(10, 11, "ng") FLOWMM_EX_FMA(12, 13, "ng") FLOWMM_EX_FMA(14, 15, "ng")               \
+        FLOWMM_EX_FMA(16, 17, "ng") FLOWMM_EX_FMA(18, 19, "ng") FLOWMM_EX_FMA(20, 21, "ng") FLOWMM_EX_FMA(22, 23, "ng")             \
+        FLOWMM_EX_FMA(24, 25, "ng") FLOWMM_EX_FMA(26, 27, "ng") FLOWMM_EX_FMA(28, 29, "ng") FLOWMM_EX_FMA(30, 31, "ng")             \
+        EXPS "}"                                                                                                                  \
+        : FLOWMM_EX_REGS(a)                                                                                                       \
+        : "f"(scale_log2), "f"(-mx))
+__device__ __forceinline__ void exp2_32(uint32_t (&a)[32], float scale_log2, float mx) { FLOWMM_EX2_32(FLOWMM_EX_ALL); }
+__device__ __forceinline__ void exp2_32_exact(uint32_t (&a)[32], float scale_log2, float mx) { FLOWMM_EX2_32(FLOWMM_EX_HW); }
+#undef FLOWMM_EX2_32
 __device__ __forceinline__ float sum32(const uint32_t (&a)[32]) {
     float2 s0 = pair_of(a, 0), s1 = pair_of(a, 2);
 #pragma unroll
@@ -412,6 +419,7 @@ __device__ __forceinline__ void colsum_chunk32(uint32_t (&a)[32], uint32_t negc,
 #undef FLOWMM_EX_POLY
 #undef FLOWMM_EX_DECL
 #undef FLOWMM_EX_ALL
+#undef FLOWMM_EX_HW
 #undef FLOWMM_EX_REGS
 
 // ---------------------------------------------------------------------------------------------

@@ -1,0 +1,45 @@
+"""Exponentials of the flow epilogue where they are exp2 of the hardware in every column: chunks of 32 keys under the causal mask or
+of both modalities.  Logits are chosen so that one key's, or one row's, exponential is
+the whole of a result's error, over the residues of its position and over the fractions that exp2 sees.
+
+Tolerance: exp2.approx is within 2^-22 of its value, its argument (below 2 in magnitude, a product of two rounded factors) within
+2^-22, which is 1.7e-7 of the value; sums of at most 64 equal terms in at least four chains, the normaliser's logarithm and the
+quotient round at 2^-24 a dozen times at most: 1.2e-6 together.  A polynomial with an error of 3.6e-6 in some columns does not pass."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import flowmm_oracle as O
+from paper_2511_05534_b200 import binding as F
+from paper_2511_05534_b200 import inputs
+
+from gpu_util import to_dev
+
+pytestmark = pytest.mark.gpu
+D, ROOT = 128, 128.0 ** 0.5
+C = np.linspace(0.35, 1.04, 64)                                      # minus the logit: its exp2 argument runs over [-1.5, -0.5]
+
+
+def _bf16(x):
+    return inputs.round_to_bf16(np.ascontiguousarray(x, dtype=np.float32))
+
+
+@pytest.mark.parametrize("L", [32, 64])
+def test_flow_of_one_visual_token(L):
+    """Rows after the one visual token see it in the chunk on the diagonal (L = 32), or in an earlier one of both modalities as well.  Its
+    own row is all but blind to the text."""
+    U, H = 8, len(C)
+    q, k = np.zeros((U, H, L, D)), np.zeros((U, H, L, D))
+    m = np.zeros((U, L), np.uint8)
+    q[..., 0] = C[:, None] * ROOT
+    k[:, :, 1:, 0] = -1
+    for u in range(U):
+        q[u, :, 8 + u, 0], q[u, :, 8 + u, 1], k[u, :, 8 + u, 1], m[u, 8 + u] = 0, 40 * ROOT, 1, 1
+    q, k = _bf16(q), _bf16(k)
+    cross = O.score(O.OracleParams(U, H, H, D, L, L, 1), q, k, m)[1]
+    fp = F.Params(U, H, H, D, L, 1, 1)
+    g_cross, rho, strat = torch.zeros((U, H), device="cuda"), torch.zeros(U, device="cuda"), torch.zeros(U, dtype=torch.int32, device="cuda")
+    ws = torch.zeros(F.flowmm_full_flow_workspace_bytes(fp), dtype=torch.uint8, device="cuda")
+    F.flowmm_full_flow(fp, to_dev(q, F.BF16), to_dev(k, F.BF16), torch.from_numpy(m).cuda(), g_cross, rho, strat, ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    assert np.abs(g_cross.double().cpu().numpy() / cross - 1).max() < 1.2e-6
