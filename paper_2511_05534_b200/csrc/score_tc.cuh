@@ -290,12 +290,17 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
                             const int last = pa - (kb + ch * 32);        // this row sees the chunk's keys 0 .. last
                             uint32_t vis = (ch & 1) ? vis1 : vis0;
                             asm volatile("" : "+r"(vis));                // (or what the sum below needs of it is formed for the plain tiles as well)
+                            float mx;
                             if (kb + ch * 32 + 32 > A.L - A.W + 1) {
 #pragma unroll
-                                for (int j = 0; j < 32; ++j) acc[j] = j <= last ? acc[j] : __float_as_uint(-INFINITY);   // exp2 gives 0
+                                for (int j = 0; j < 32; ++j) acc[j] = j <= last ? acc[j] : __float_as_uint(-INFINITY);
+                                mx = fmaxf(max32(acc) * A.scale_log2, st[h].m);
+                                exp2_32_exact(acc, A.scale_log2, mx);           // (0 where masked; the polynomial would leave 2^-125)
+                            } else {
+                                mx = fmaxf(max32(acc) * A.scale_log2, st[h].m);
+                                exp2_32(acc, A.scale_log2, mx);
                             }
-                            const float mx = fmaxf(max32(acc) * A.scale_log2, st[h].m), carry = tc::ex2(st[h].m - mx);
-                            exp2_32(acc, A.scale_log2, mx);
+                            const float carry = tc::ex2(st[h].m - mx);
                             const float all = sum32(acc);
                             float on_vis = vis ? all : 0.f;
                             if (vis != 0u && vis != 0xFFFFFFFFu) on_vis = sum32_of(acc, vis, masks);

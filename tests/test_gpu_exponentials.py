@@ -1,4 +1,4 @@
-"""Exponentials of the flow epilogue where they are exp2 of the hardware in every column: chunks of 32 keys under the causal mask or
+"""Exponentials of the scoring and flow epilogues where they are exp2 of the hardware in every column: chunks of 32 keys under the causal mask or
 of both modalities.  Logits are chosen so that one key's, or one row's, exponential is
 the whole of a result's error, over the residues of its position and over the fractions that exp2 sees.
 
@@ -13,7 +13,7 @@ from oracle import flowmm_oracle as O
 from paper_2511_05534_b200 import binding as F
 from paper_2511_05534_b200 import inputs
 
-from gpu_util import to_dev
+from gpu_util import gpu_params, to_dev
 
 pytestmark = pytest.mark.gpu
 D, ROOT = 128, 128.0 ** 0.5
@@ -22,6 +22,15 @@ C = np.linspace(0.35, 1.04, 64)                                      # minus the
 
 def _bf16(x):
     return inputs.round_to_bf16(np.ascontiguousarray(x, dtype=np.float32))
+
+
+def _score(p, q, k, m):
+    imp, cross, _ = O.score(p, q, k, m)
+    g_imp, g_cross = torch.full(imp.shape, float("nan"), device="cuda"), torch.full(cross.shape, float("nan"), device="cuda")
+    ws = F.alloc_workspace(gpu_params(p, F.BF16))
+    F.flowmm_score(gpu_params(p, F.BF16), to_dev(q, F.BF16), to_dev(k, F.BF16), torch.from_numpy(m).cuda(), g_imp, g_cross, ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    return imp, cross, g_imp.double().cpu().numpy(), g_cross.double().cpu().numpy()
 
 
 @pytest.mark.parametrize("L", [32, 64])
@@ -43,3 +52,16 @@ def test_flow_of_one_visual_token(L):
     F.flowmm_full_flow(fp, to_dev(q, F.BF16), to_dev(k, F.BF16), torch.from_numpy(m).cuda(), g_cross, rho, strat, ws)
     assert F.flowmm_last_device_status(ws) == 0
     assert np.abs(g_cross.double().cpu().numpy() / cross - 1).max() < 1.2e-6
+
+
+def test_normalisers_of_masked_chunks():
+    """All of a proxy row's mass is on the first key and on the window's keys of one residue (mod 8)."""
+    U, H, W, L = 8, len(C) // 2, 32, 320
+    q, k = np.zeros((U, 2 * H, W, D)), np.zeros((U, H, L, D))
+    q[..., 0], q[..., 1] = C[:, None] * ROOT, ROOT
+    k[:, :, 1:, 1] = -60
+    for u in range(U):
+        k[u, :, L - W + u::8, 0], k[u, :, L - W + u::8, 1] = -1, 0
+    imp, _, g_imp, _ = _score(O.OracleParams(U, 2 * H, H, D, L, W, 1), _bf16(q), _bf16(k), np.zeros((U, L), np.uint8))
+    on = imp > 1e-3
+    assert on.sum() == U * H * 5 and np.abs(g_imp[on] / imp[on] - 1).max() < 1.2e-6
