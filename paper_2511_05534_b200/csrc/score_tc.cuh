@@ -552,6 +552,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                     uint32_t acc[32];
                     tc::tmem_ld32(S::acc_addr(c, ch0 + i), acc);
                     tc::tmem_ld_wait(acc);
+                    float s4[4] = {0.f, 0.f, 0.f, 0.f};              // (one sum over all rows would lose the small ones)
 #pragma unroll
                     for (int q4 = 0; q4 < 8; ++q4) {
                         const float4 n4 = tc::lds128(nc + (i * 8 + q4) * 16);
@@ -559,9 +560,10 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {                // causal mask inside the window, and keys >= L
                             const float e = tc::ex2(fmaf(__uint_as_float(acc[4 * q4 + j]), A.scale_log2, nn[j]));
-                            imp += key <= first_proxy + a0 + 4 * q4 + j ? e : 0.f;
+                            s4[j] += key <= first_proxy + a0 + 4 * q4 + j ? e : 0.f;
                         }
                     }
+                    imp += (s4[0] + s4[1]) + (s4[2] + s4[3]);
                 }
                 S::quad_release(c);
             }

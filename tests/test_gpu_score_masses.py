@@ -80,3 +80,25 @@ def test_items_of_one_half_and_of_two(U, G, W, L):
     """Both sides of the lines at which either pass goes from items of 128 proxy rows or keys to items of 256."""
     rng = np.random.default_rng(U * L)
     _check(rng, U, G, 1, L, W, np.arange(L)[None] // 50 % 2 ^ rng.integers(0, 2, (U, 1)))
+
+
+def test_sums_over_many_proxy_rows():
+    """A key of the window that one proxy row gives all of its mass and 1023 others 2.5e-8 each: added to the one, one by one, they would
+    vanish (half of them share its sum: 1.3e-5).  Exponentials within 2^-22, their arguments (up to 26) within 2e-6, sums of 32 by fours."""
+    L, W, G = 300, 128, 8
+    q, k = np.zeros((1, G, W, 128), np.float32), np.zeros((1, 1, L, 128), np.float32)
+    q[..., 0], q[..., 2] = 1, 1
+    q[0, 0, 0, 0], q[0, 0, 0, 1] = 0, 1
+    k[0, 0, 1:, 2] = -1024                                          # (logit -90)
+    k[0, 0, L - W, 0], k[0, 0, L - W, 2] = -198, 0                  # (logit -17.5)
+    k[0, 0, 0, 1], k[0, 0, L - W, 1] = -1024, 0
+    q, k = inputs.round_to_bf16(q), inputs.round_to_bf16(k)
+    p = O.OracleParams(1, G, 1, 128, L, W, 1)
+    m = np.zeros((1, L), np.uint8)
+    imp = O.score(p, q, k, m)[0][0, 0, L - W]
+    fp = gpu_params(p, F.BF16)
+    g_imp, g_cross = torch.zeros((1, 1, L), device="cuda"), torch.zeros((1, G), device="cuda")
+    ws = F.alloc_workspace(fp)
+    F.flowmm_score(fp, to_dev(q, F.BF16), to_dev(k, F.BF16), torch.from_numpy(m).cuda(), g_imp, g_cross, ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    assert imp > 0.125 * (1 + 2e-5) and abs(float(g_imp[0, 0, L - W]) / imp - 1) < 1e-6
