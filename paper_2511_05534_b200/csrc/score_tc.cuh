@@ -395,27 +395,31 @@ __global__ void score_combine_kernel(const ScoreTcArgs A, int n_rows, float4 *ro
     FLOWMM_EX_FMA(i0, i1, "n0") FLOWMM_EX_FMA(i2, i3, "n1")
 #define FLOWMM_CS_P(k, i0, i1) "mov.b64 p" #k ", {%" #i0 ", %" #i1 "};\n\t"
 #define FLOWMM_CS_A(d, x, y) "add.rn.f32x2 p" #d ", p" #x ", p" #y ";\n\t"
-__device__ __forceinline__ void colsum_chunk32(uint32_t (&a)[32], uint32_t negc, float scale_log2, uint64_t &sum) {
-    asm volatile(
-        "{\n\t" FLOWMM_EX_DECL ".reg .b64 n0, n1, p<16>;\n\t"
-        "mov.b64 sc, {%34, %34};\n\t"
-        FLOWMM_CS_X(0, 0, 1, 2, 3) FLOWMM_CS_X(1, 4, 5, 6, 7) FLOWMM_CS_X(2, 8, 9, 10, 11) FLOWMM_CS_X(3, 12, 13, 14, 15)
-        FLOWMM_CS_X(4, 16, 17, 18, 19) FLOWMM_CS_X(5, 20, 21, 22, 23) FLOWMM_CS_X(6, 24, 25, 26, 27) FLOWMM_CS_X(7, 28, 29, 30, 31)
-        FLOWMM_EX_ALL
-        FLOWMM_CS_P(0, 0, 1) FLOWMM_CS_P(1, 2, 3) FLOWMM_CS_P(2, 4, 5) FLOWMM_CS_P(3, 6, 7) FLOWMM_CS_P(4, 8, 9) FLOWMM_CS_P(5, 10, 11)
-        FLOWMM_CS_P(6, 12, 13) FLOWMM_CS_P(7, 14, 15) FLOWMM_CS_P(8, 16, 17) FLOWMM_CS_P(9, 18, 19) FLOWMM_CS_P(10, 20, 21)
-        FLOWMM_CS_P(11, 22, 23) FLOWMM_CS_P(12, 24, 25) FLOWMM_CS_P(13, 26, 27) FLOWMM_CS_P(14, 28, 29) FLOWMM_CS_P(15, 30, 31)
-        FLOWMM_CS_A(0, 0, 1) FLOWMM_CS_A(2, 2, 3) FLOWMM_CS_A(4, 4, 5) FLOWMM_CS_A(6, 6, 7) FLOWMM_CS_A(8, 8, 9) FLOWMM_CS_A(10, 10, 11)
-        FLOWMM_CS_A(12, 12, 13) FLOWMM_CS_A(14, 14, 15)
-        FLOWMM_CS_A(0, 0, 2) FLOWMM_CS_A(4, 4, 6) FLOWMM_CS_A(8, 8, 10) FLOWMM_CS_A(12, 12, 14)
-        FLOWMM_CS_A(0, 0, 4) FLOWMM_CS_A(8, 8, 12)
-        FLOWMM_CS_A(0, 0, 8)
-        "add.rn.f32x2 %32, %32, p0;\n\t"
-        "}"
-        : FLOWMM_EX_REGS(a), "+l"(sum)
-        : "r"(negc), "f"(scale_log2)
-        : "memory");
-}
+#define FLOWMM_CS(EXPS)                                                                                                            \
+    asm volatile(                                                                                                                 \
+        "{\n\t" FLOWMM_EX_DECL ".reg .b64 n0, n1, p<16>;\n\t"                                                                      \
+        "mov.b64 sc, {%34, %34};\n\t"                                                                                             \
+        FLOWMM_CS_X(0, 0, 1, 2, 3) FLOWMM_CS_X(1, 4, 5, 6, 7) FLOWMM_CS_X(2, 8, 9, 10, 11) FLOWMM_CS_X(3, 12, 13, 14, 15)           \
+        FLOWMM_CS_X(4, 16, 17, 18, 19) FLOWMM_CS_X(5, 20, 21, 22, 23) FLOWMM_CS_X(6, 24, 25, 26, 27) FLOWMM_CS_X(7, 28, 29, 30, 31) \
+        EXPS                                                                                                                      \
+        FLOWMM_CS_P(0, 0, 1) FLOWMM_CS_P(1, 2, 3) FLOWMM_CS_P(2, 4, 5) FLOWMM_CS_P(3, 6, 7) FLOWMM_CS_P(4, 8, 9)                    \
+        FLOWMM_CS_P(5, 10, 11) FLOWMM_CS_P(6, 12, 13) FLOWMM_CS_P(7, 14, 15) FLOWMM_CS_P(8, 16, 17) FLOWMM_CS_P(9, 18, 19)          \
+        FLOWMM_CS_P(10, 20, 21) FLOWMM_CS_P(11, 22, 23) FLOWMM_CS_P(12, 24, 25) FLOWMM_CS_P(13, 26, 27) FLOWMM_CS_P(14, 28, 29)     \
+        FLOWMM_CS_P(15, 30, 31)                                                                                                   \
+        FLOWMM_CS_A(0, 0, 1) FLOWMM_CS_A(2, 2, 3) FLOWMM_CS_A(4, 4, 5) FLOWMM_CS_A(6, 6, 7) FLOWMM_CS_A(8, 8, 9)                    \
+        FLOWMM_CS_A(10, 10, 11) FLOWMM_CS_A(12, 12, 13) FLOWMM_CS_A(14, 14, 15)                                                   \
+        FLOWMM_CS_A(0, 0, 2) FLOWMM_CS_A(4, 4, 6) FLOWMM_CS_A(8, 8, 10) FLOWMM_CS_A(12, 12, 14)                                   \
+        FLOWMM_CS_A(0, 0, 4) FLOWMM_CS_A(8, 8, 12)                                                                                \
+        FLOWMM_CS_A(0, 0, 8)                                                                                                      \
+        "add.rn.f32x2 %32, %32, p0;\n\t"                                                                                          \
+        "}"                                                                                                                       \
+        : FLOWMM_EX_REGS(a), "+l"(sum)                                                                                            \
+        : "r"(negc), "f"(scale_log2)                                                                                              \
+        : "memory")
+__device__ __forceinline__ void colsum_chunk32(uint32_t (&a)[32], uint32_t negc, float scale_log2, uint64_t &sum) { FLOWMM_CS(FLOWMM_EX_ALL); }
+// (all exponentials by the exp2 unit)
+__device__ __forceinline__ void colsum_chunk32_exact(uint32_t (&a)[32], uint32_t negc, float scale_log2, uint64_t &sum) { FLOWMM_CS(FLOWMM_EX_HW); }
+#undef FLOWMM_CS
 #undef FLOWMM_CS_X
 #undef FLOWMM_CS_P
 #undef FLOWMM_CS_A
@@ -478,11 +482,16 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
         const int n_tiles = (A.GW + S::kCols - 1) / S::kCols;
         int uh = (int)A.by_rt2.div(g_lo), kt = g_lo - uh * A.n_rt2, u = (int)A.by_hkv.div(uh), hk = uh - u * A.Hkv;
         uint32_t slot = 0, consts = c.base + S::kSmemEpi + kConstBytes;
+        uint32_t both = 0;                                           // which words of 32 proxy tokens are of both modalities
         for (int g = g_lo; g < g_hi; ++g) {
             const int uh0 = uh, kt0 = kt;                            // this item
             if (g == g_lo || kt0 == 0) {                             // a new head: its row constants
                 consts ^= (c.base + S::kSmemEpi) ^ (c.base + S::kSmemEpi + kConstBytes);
                 const int n_rec = A.row_all ? 1 : runs_of_head(A, uh0);
+                const uint8_t *proxy_mod = A.modality + (int64_t)(u + 1) * A.L - A.W;
+                uint8_t of_lane[4];
+#pragma unroll
+                for (int w = 0; w < 4; ++w) of_lane[w] = proxy_mod[min(32 * w, A.W - 32) + lane];   // (the window is 32, 64 or 128 rows)
                 for (int r = te; r < A.GW; r += 32 * tcs::kEpiWarps) {
                     const int64_t i0 = (int64_t)uh0 * A.GW + r;
                     const float4 *rec = A.row_all ? A.row_all + i0 : A.row_part + i0 * A.n_part;
@@ -505,9 +514,15 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                     const float z = s.t + s.v;
                     tc::sts32(consts + r * 4, -(s.m + log2f(z)));
                     if (kt0 == 0) {                                  // (one CTA per head)
-                        const bool vis = A.modality[(int64_t)u * A.L + A.L - A.W + (r & (A.W - 1))] != 0;   // (the window is 32, 64 or 128 rows)
+                        const bool vis = proxy_mod[r & (A.W - 1)] != 0;
                         A.cross_part[((int64_t)u * A.Hq + hk * A.G) * A.W + r] = (vis ? s.t : s.v) / z;
                     }
+                }
+                both = 0;
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    const uint32_t vis = __ballot_sync(0xFFFFFFFFu, of_lane[w] != 0);
+                    if (vis != 0u && vis != 0xFFFFFFFFu) both |= 1u << w;
                 }
                 // (the set written was read two heads ago, and every warp has been through the meeting of the head between)
                 tcs::named_barrier(9, 32 * tcs::kEpiWarps);
@@ -534,7 +549,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                 constexpr int kPerC = S::kCols / 64;                 // 32-column chunks a warp takes of a full tile
                 const int ch0 = kPerC * c.colhalf, n_ch = min((ncols + 31) >> 5, ch0 + kPerC) - ch0;   // >= 1
                 const uint32_t nc = consts + (uint32_t)(t * S::kCols + ch0 * 32) * 4;
-                if (!masked_tile) {
+                if (!masked_tile && both == 0u) {
                     uint32_t a[2][32];
                     tc::tmem_ld32(S::acc_addr(c, ch0), a[0]);
 #pragma unroll
@@ -544,6 +559,20 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                         if (i + 1 < kPerC && i + 1 < n_ch) tc::tmem_ld32(S::acc_addr(c, ch0 + i + 1), a[(i + 1) & 1]);
                         else S::quad_release(c);
                         colsum_chunk32(a[i & 1], nc + i * 128, A.scale_log2, sum2);
+                    }
+                    continue;
+                }
+                if (!masked_tile) {
+                    // proxy tokens of both modalities, whose share a few rows can make up: by the exp2 unit alone (asking for it at every
+                    // chunk of every call costs 4 % of the pass)
+#pragma unroll 1
+                    for (int i = 0; i < n_ch; ++i) {
+                        uint32_t acc[32];
+                        tc::tmem_ld32(S::acc_addr(c, ch0 + i), acc);
+                        tc::tmem_ld_wait(acc);
+                        if (i + 1 == n_ch) S::quad_release(c);
+                        if (both >> (((ch0 + i) * 32 & (A.W - 1)) >> 5) & 1u) colsum_chunk32_exact(acc, nc + i * 128, A.scale_log2, sum2);
+                        else colsum_chunk32(acc, nc + i * 128, A.scale_log2, sum2);
                     }
                     continue;
                 }

@@ -1,5 +1,5 @@
-"""Exponentials of the scoring and flow epilogues where they are exp2 of the hardware in every column: chunks of 32 keys under the causal mask or
-of both modalities.  Logits are chosen so that one key's, or one row's, exponential is
+"""Exponentials of the scoring and flow epilogues where they are exp2 of the hardware in every column: chunks of 32 keys under the
+causal mask or of both modalities, proxy rows of both modalities.  Logits are chosen so that one key's, or one row's, exponential is
 the whole of a result's error, over the residues of its position and over the fractions that exp2 sees.
 
 Tolerance: exp2.approx is within 2^-22 of its value, its argument (below 2 in magnitude, a product of two rounded factors) within
@@ -65,3 +65,19 @@ def test_normalisers_of_masked_chunks():
     imp, _, g_imp, _ = _score(O.OracleParams(U, 2 * H, H, D, L, W, 1), _bf16(q), _bf16(k), np.zeros((U, L), np.uint8))
     on = imp > 1e-3
     assert on.sum() == U * H * 5 and np.abs(g_imp[on] / imp[on] - 1).max() < 1.2e-6
+
+
+@pytest.mark.parametrize("W", [32, 64, 128])
+def test_importances_from_a_window_of_both_modalities(W):
+    """Keys that the window's rows of one residue (mod 8) alone see; every word of 32 rows has both modalities."""
+    U, H, L = 8, len(C) // 2, 512
+    q, k = np.zeros((U, 2 * H, W, D)), np.zeros((U, H, L, D))
+    q[..., 1] = ROOT
+    q[..., 2] = ROOT
+    for u in range(U):
+        q[u, :, u::8, 0], q[u, :, u::8, 2] = C[:, None] * ROOT, 0
+    k[:, :, 1:, 1] = -60
+    k[:, :, 8:128:8, 0], k[:, :, 8:128:8, 1], k[:, :, 8:128:8, 2] = -1, 0, -60
+    m = np.ascontiguousarray(np.broadcast_to(np.arange(L) // 16 % 2, (U, L)), dtype=np.uint8)
+    imp, _, g_imp, _ = _score(O.OracleParams(U, 2 * H, H, D, L, W, 1), _bf16(q), _bf16(k), m)
+    assert np.abs(g_imp[:, :, 8:128:8] / imp[:, :, 8:128:8] - 1).max() < 1.2e-6
