@@ -145,16 +145,20 @@ __device__ __forceinline__ float sum32(const uint32_t (&a)[32]) {
     s0 = tc::fadd2(s0, s1);
     return s0.x + s0.y;
 }
-// The sum over a chunk's visual keys (bit set in `vis`).  `masks`: shared address of sixteen float4, entry n the bits of n as 0.f /
-// 1.f: a multiply-add with the mask, where a test per key would cost three instructions.
-__device__ __forceinline__ float sum32_of(const uint32_t (&a)[32], uint32_t vis, uint32_t masks) {
-    float2 v01 = make_float2(0.f, 0.f), v23 = v01;
+// The sums over a chunk's text keys and over its visual keys (bit set in `vis`), each a sum of its own: as the difference of all and the
+// others a small one would lose its digits.  `masks`: shared address of sixteen float4, entry n the bits of n as 0.f / -1.f: two
+// multiply-adds with the mask, where tests per key would cost three instructions each.
+__device__ __forceinline__ void sums32_by(const uint32_t (&a)[32], uint32_t vis, uint32_t masks, float &on_text, float &on_vis) {
+    float2 t01 = make_float2(0.f, 0.f), t23 = t01, v01 = t01, v23 = t01;
 #pragma unroll
     for (int j = 0; j < 32; j += 4) {
         const float4 v = tc::lds128(masks + (vis >> j & 15u) * 16);
-        v01 = tc::ffma2(pair_of(a, j), make_float2(v.x, v.y), v01); v23 = tc::ffma2(pair_of(a, j + 2), make_float2(v.z, v.w), v23);
+        const float2 x01 = pair_of(a, j), x23 = pair_of(a, j + 2), m01 = make_float2(v.x, v.y), m23 = make_float2(v.z, v.w);
+        t01 = tc::fadd2(t01, tc::ffma2(x01, m01, x01)); t23 = tc::fadd2(t23, tc::ffma2(x23, m23, x23));   // (x or 0)
+        v01 = tc::ffma2(x01, m01, v01); v23 = tc::ffma2(x23, m23, v23);
     }
-    return (v01.x + v01.y) + (v23.x + v23.y);
+    on_text = (t01.x + t01.y) + (t23.x + t23.y);
+    on_vis = -((v01.x + v01.y) + (v23.x + v23.y));
 }
 
 // Run `r` of n: tiles [run_start(r), run_start(r + 1)) of the n_tiles of all heads; and the run that holds tile x.
@@ -228,7 +232,7 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
         const uint32_t meet = c.base + S::kSmemExtra + (uint32_t)c.quarter * 6 * kMeetWarp + (uint32_t)c.lane * 12;
         const uint32_t masks = c.base + S::kSmemExtra + 2 * kMeetBytes;
         const int te = threadIdx.x - 64;
-        if (te < 64) tc::sts32(masks + te * 4, (float)((te >> 2) >> (te & 3) & 1));
+        if (te < 64) tc::sts32(masks + te * 4, (te >> 2) >> (te & 3) & 1 ? -1.f : 0.f);
         tcs::named_barrier(5, 32 * tcs::kEpiWarps);
         int kh[2] = {0, 0};
         uint32_t turn = 0;
@@ -301,10 +305,10 @@ score_stats_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
                                 exp2_32(acc, A.scale_log2, mx);
                             }
                             const float carry = tc::ex2(st[h].m - mx);
-                            const float all = sum32(acc);
-                            float on_vis = vis ? all : 0.f;
-                            if (vis != 0u && vis != 0xFFFFFFFFu) on_vis = sum32_of(acc, vis, masks);
-                            const float on_text = fmaxf(all - on_vis, 0.f);
+                            float on_text = 0.f, on_vis = 0.f;
+                            if (vis == 0u) on_text = sum32(acc);
+                            else if (vis == 0xFFFFFFFFu) on_vis = sum32(acc);
+                            else sums32_by(acc, vis, masks, on_text, on_vis);
                             st[h].t = st[h].t * carry + (swapped ? on_vis : on_text);
                             st[h].v = st[h].v * carry + (swapped ? on_text : on_vis);
                             st[h].m = mx;

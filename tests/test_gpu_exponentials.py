@@ -81,3 +81,19 @@ def test_importances_from_a_window_of_both_modalities(W):
     m = np.ascontiguousarray(np.broadcast_to(np.arange(L) // 16 % 2, (U, L)), dtype=np.uint8)
     imp, _, g_imp, _ = _score(O.OracleParams(U, 2 * H, H, D, L, W, 1), _bf16(q), _bf16(k), m)
     assert np.abs(g_imp[:, :, 8:128:8] / imp[:, :, 8:128:8] - 1).max() < 1.2e-6
+
+
+@pytest.mark.parametrize("few", [0, 1])
+@pytest.mark.parametrize("logit", [-10, -14, -17, -25, -60])
+def test_small_masses_in_chunks_of_both_modalities(few, logit):
+    """Chunks in which one modality has a share of 1e-4 to 1e-26, and a window of the other one, whose cross-modal mass it is.  Tolerance: the
+    polynomial's 3.6e-6 in numerator and normaliser, and the exp2 argument, which is as large as 87 (1e-5 of the value)."""
+    U, H, W, L = 2, 4, 32, 513
+    rng = np.random.default_rng(1)
+    m = (rng.random((U, L)) < 0.5).astype(np.uint8)
+    m[:, L - W:] = 1 - few
+    q, k = np.zeros((U, 2 * H, W, D)), 0.25 * rng.standard_normal((U, H, L, D))
+    q[..., 0] = ROOT
+    k[..., 0] = np.where(m == few, logit, 0)[:, None]
+    _, cross, _, g_cross = _score(O.OracleParams(U, 2 * H, H, D, L, W, 1), _bf16(q), _bf16(k), m)
+    assert np.abs(g_cross / cross - 1).max() < 2e-5
