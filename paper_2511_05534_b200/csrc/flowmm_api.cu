@@ -119,12 +119,13 @@ int chunks_for(int L, int other_ctas, int &chunk) {
 // Rows of a window of the merge kernel (merge_rows.cuh).  Long windows cost less per row, short ones give every warp one: 1.2 million
 // rows at most leave 3552 warps five windows of 64.  34 000 rows by 32 and 16: 77.7 and 76.4 us for the call, 43 000 84.3 and 87.3,
 // 270 000 231.5 and 240.6.
-// From kManyRows on warps draw their windows from a counter and a slot may have 128 members before it is cut, else windows are taken with a
-// stride and a slot is cut beyond 64 (270 000 rows 252 and 236 us; 4.5 million rows the merge 410 and 460).
+// From kManyRows on warps draw their windows from a counter, else windows are taken with a stride.  The merge by windows of 32 with a
+// stride, and of 64 from the counter, us: 300 000 rows 44 to 53, 53 to 64; 0.8 million 83, 86; 1.0 million 109 to 123, 113 to 124;
+// 1.3 million 154, 156; 1.6 million 165, 164; 2.5 million 257, 248; 4.3 million 422, 392 (fp32 rows of 64 within 1 %, equal from 0.8 million on).
 constexpr int64_t kManyRows = 1300000;
 int merge_window(const flowmm_params &p) {
     const int64_t rows = (int64_t)p.n_units * p.n_kv_heads * p.seq_len;
-    return rows >= kManyRows ? 64 : rows >= 40000 ? 32 : 16;
+    return rows >= kManyRows ? mrow::kMaxWin : rows >= 40000 ? 32 : 16;
 }
 
 // The part of the workspace that the merge step uses (rows in slot order, windows, pieces, partial sums).
@@ -687,7 +688,7 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         c.off = at<int>(ws, y.off); c.first_slot = at<int>(ws, y.first_slot); c.part_off = at<int>(ws, y.part_off);
         c.pieces = at<int4>(ws, y.pieces); c.ticket = at<unsigned>(ws, y.ticket); c.slot_done = at<int>(ws, y.slot_done);
         c.B = p.n_keep; c.E = E; c.n_pass = y.csr_passes; c.max_parts = y.max_parts; c.merge_mode = p.merge_mode;
-        c.win = y.merge_win; c.n_win = y.n_win; c.longest = (int64_t)UH * p.seq_len < kManyRows ? kPiece : 128;
+        c.win = y.merge_win; c.n_win = y.n_win;
         // Warps per head by the length of its list: 8 walk up to 4096 positions in 16 steps each, which ends before 32 warps
         // are through their barriers.  Sorted in shared memory when positions and counters fit, else through global memory.
         const bool long_list = E > 4096;

@@ -10,7 +10,8 @@ namespace flowmm {
 // (ascending j inside a slot).  What comes out is the sequence of a head's rows in slot order: each slot's
 // pivot, then its members, with token position and Eq. 5 weight; slot s begins at row off[s] + s, off[s] being the
 // number of members of the slots before it.  The merge kernel (merge_rows.cuh) takes the sequence a window of rows at a time.
-// A slot of more than `longest` members is left out there: it is cut into pieces of kPiece, so that many warps share it.
+// A slot of more than kPiece members is left out there: it is cut into pieces of kPiece, so that many warps share it and no sum is
+// a longer chain than that.
 // ---------------------------------------------------------------------------------------------
 constexpr int kPiece = 64;
 
@@ -28,7 +29,7 @@ struct CsrArgs {
     int4 *pieces;            // [UH, max_parts] (slot, first row, rows, number of the piece)
     unsigned *ticket;        // work counter of the merge kernel, cleared here
     int *slot_done;          // [UH, B] pieces of a slot that have stored their partial sums, cleared here
-    int B, E, n_pass, max_parts, merge_mode, win, n_win, longest;
+    int B, E, n_pass, max_parts, merge_mode, win, n_win;
 };
 constexpr int kRowPivot = (int)0x80000000u, kRowLong = 1 << 30, kRowToken = kRowLong - 1;
 
@@ -64,7 +65,7 @@ __device__ __forceinline__ void csr_write_slots(const CsrArgs &A, int uh, const 
         int n = 0, np = 0;
         if (s < A.B) {
             n = off[s + 1] - off[s];
-            np = n > A.longest ? (n + kPiece - 1) / kPiece : 0;
+            np = n > kPiece ? (n + kPiece - 1) / kPiece : 0;
         }
         int total;
         const int part = seen + block_exclusive_scan(np, scratch, total);

@@ -21,6 +21,8 @@ namespace mrow {
 
 constexpr int kThreads = 256, kWarps = kThreads / 32;
 constexpr int kChunk = 128;                                  // rows whose tokens and weights wait in shared memory
+constexpr int kMaxWin = 64;                                  // rows of a window at most
+static_assert(kChunk >= kMaxWin + kPiece, "the last slot that begins in a window ends among them");
 constexpr int kStages = 4;
 constexpr uint32_t kEntryBytes = kChunk * 8;
 __host__ __device__ constexpr int group_rows(int bytes) { return bytes == 32 ? 2 : 4; }
@@ -183,23 +185,21 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
         const int u = (int)by_hkv.div(uh), h = uh - u * A.Hkv;
         const int left = is_window ? it.count.x - w * A.win : 0, n_pieces = is_window && n_piece_items != 0 ? 0 : it.count.y;   // left: rows from the window's first on
         int slot = it.first;
-        const int uh_row = w * A.win;
         // the rows of a chunk go to shared memory; which of them begin a slot, or lie past the last row
         unsigned long long lo, hi;
-        auto take = [&](int base, const int (&x)[4], const int (&y)[4]) {
+        {
             uint32_t begins[4];
             __syncwarp();                                            // (the rows before have been read)
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const int r = 32 * k + lane, v = base + r < left ? x[k] : kRowPivot;
+                const int r = 32 * k + lane, v = r < left ? it.x[k] : kRowPivot;
                 begins[k] = __ballot_sync(0xFFFFFFFFu, v < 0);
-                tc::sts64(ents + r * 8, (uint32_t)v, (uint32_t)y[k]);
+                tc::sts64(ents + r * 8, (uint32_t)v, (uint32_t)it.y[k]);
             }
             __syncwarp();
             lo = begins[0] | (unsigned long long)begins[1] << 32;
             hi = begins[2] | (unsigned long long)begins[3] << 32;
-        };
-        take(0, it.x, it.y);
+        }
         fetch(g_next, it);
         const char *src = reinterpret_cast<const char *>((is_v ? static_cast<const T *>(A.v) + u * A.vs[0] + h * A.vs[1]
                                                                : static_cast<const T *>(A.k) + u * A.ks[0] + h * A.ks[1]) + c0);
@@ -207,13 +207,12 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
         const unsigned long long own = n_own <= 0 ? 0ull : lo & (~0ull >> (64 - n_own));
         if (own) {
             const int last = 63 - __clzll((long long)own);
-            int r0 = __ffsll((long long)own) - 1, r1 = last;         // a long slot, which is the window's last, is left to its pieces
-            bool more = false;
-            auto end_from = [&](unsigned long long a, unsigned long long b) {
-                more = a == 0ull && b == 0ull;
-                r1 = a ? __ffsll((long long)a) - 1 : b ? 64 + __ffsll((long long)b) - 1 : kChunk;
-            };
-            if (!(__float_as_int(tc::lds32(ents + last * 8)) & kRowLong)) end_from(last == 63 ? 0ull : lo & (~0ull << (last + 1)), hi);
+            const int r0 = __ffsll((long long)own) - 1;
+            int r1 = last;         // a long slot, which is the window's last, is left to its pieces
+            if (!(__float_as_int(tc::lds32(ents + last * 8)) & kRowLong)) {
+                const unsigned long long next = last == 63 ? 0ull : lo & (~0ull << (last + 1));
+                r1 = next ? __ffsll((long long)next) - 1 : hi ? 64 + __ffsll((long long)hi) - 1 : kChunk;
+            }
             T *out = is_v ? static_cast<T *>(A.v_out) + u * A.vos[0] + h * A.vos[1] : static_cast<T *>(A.k_out) + u * A.kos[0] + h * A.kos[1];
             const int64_t ostride = is_v ? A.vos[2] : A.kos[2];
             out += c0 + (slot - 1) * ostride;                        // (the first pivot steps to the first slot)
@@ -243,20 +242,7 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
                 open = true;
                 out += ostride;
             };
-            for (int base = kChunk;; base += kChunk) {
-                walk(src, r0, r1, lo, hi, begin);
-                if (!more) break;
-                int x[4], y[4];                                      // the last slot's other members
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int r = uh_row + base + 32 * k + lane;
-                    x[k] = kRowPivot; y[k] = 0;
-                    if (r < A.L && A.rows) { const int2 e = A.rows[(int64_t)uh * A.L + r]; x[k] = e.x; y[k] = e.y; }
-                }
-                take(base, x, y);
-                end_from(lo, hi);
-                r0 = 0;
-            }
+            walk(src, r0, r1, lo, hi, begin);
             if (open) finish();
         }
         for (int p = w; p < n_pieces; p += is_window ? A.n_win : A.max_parts) {   // this window's share of the head's pieces, or the piece

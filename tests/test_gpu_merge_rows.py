@@ -1,5 +1,5 @@
 """Merge of sorted lists by windows of rows: slots of chosen numbers of members (none, the most that stay whole, one more, several
-chunks of 128 rows) at chosen places of a window, windows of 16, 32 and 64 rows, taken with a stride or drawn from the counter,
+pieces) at chosen places of a window, windows of 16, 32 and 64 rows, taken with a stride or drawn from the counter,
 pieces of long slots as items of their own and spread over the windows, every row width, and output layouts with gaps.
 The values let one lost or doubled member be seen (test_merge_reference.py)."""
 import numpy as np
@@ -66,7 +66,7 @@ def test_slots_of_chosen_sizes(pattern, heads, dtype, D):
 
 
 def test_many_rows_draw_their_windows():
-    """1.6 million rows of 160 heads: windows of 64 from the counter, slots of up to 128 members whole."""
+    """1.6 million rows of 160 heads: windows of 64 from the counter."""
     rng = np.random.default_rng(3)
     heads, B, D = 160, 1000, 64
     n = _members("edges_apart", B, rng)
@@ -139,3 +139,33 @@ def test_rows_gigabytes_apart(dtype, D, E):
         if E:
             want[0] = ((src[0].float() + src[1].float()) / 2).to(want.dtype)     # (exact: halves of small integers)
         assert torch.equal(got, want.expand(1, heads, B, D))
+
+
+@pytest.mark.parametrize("n", [100, 128])
+def test_many_rows_sum_long_slots_in_parts_of_64(n):
+    """1.3 million rows, whose windows are drawn from the counter: a slot's first 64 members add up to 2^24, the others are ones, which
+    vanish if they are added to that one by one.  With the parts added up on their own only the last sum and the mean round:
+    2^-22 relative covers both; all ones lost would be 64 / 2^24."""
+    heads, B, D = 160, 300, 64
+    E = 30 * n
+    L = E + B
+    heads = -(-1310000 // L)
+    ret = np.arange(B)                                              # (every tenth slot is long, the others have no members)
+    evi = np.arange(B, L)
+    match = np.repeat(np.arange(0, B, 10), n)
+    k = np.ones((L, D), np.float32)
+    k[B:][np.arange(E) % n < 64] = 2.0 ** 18
+    k *= np.arange(1, D + 1) % 3 + 1
+    kd = torch.from_numpy(k).cuda().expand(1, heads, L, D)
+    rep = lambda x, t: torch.from_numpy(np.ascontiguousarray(np.broadcast_to(x.astype(t), (1, heads, x.size)))).cuda()
+    fp = F.Params(1, heads, heads, D, L, 1, B, dtype=F.F32, merge_mode=F.MERGE_MEAN)
+    ws = F.alloc_workspace(fp)
+    out = [torch.full((1, heads, B, D), float("nan"), device="cuda") for _ in range(2)]
+    F.flowmm_merge(fp, kd, kd, rep(ret, np.int32), rep(evi, np.int32), rep(match, np.int32), rep(np.zeros(E), np.float32), out[0], out[1], ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    k64 = k.astype(np.float64)
+    want = k64[:B].copy()
+    want[::10] = (k64[:B:10] + k64[B:].reshape(30, n, D).sum(1)) / (n + 1)
+    for got in out:
+        assert torch.equal(got, got[:, :1].expand(-1, heads, -1, -1))
+        assert np.abs(got[0, 0].double().cpu().numpy() / want - 1).max() < 2.0 ** -22
