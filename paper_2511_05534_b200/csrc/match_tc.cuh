@@ -553,9 +553,10 @@ match_tc_kernel(const __grid_constant__ CUtensorMap cand_map, const MatchTcArgs 
                         uint32_t a[32];
                         tc::tmem_ld32(tl + 16 * (kPer - 2), a);
                         tc::tmem_ld_wait(a);
-                        S::acc_release(c);
+                        if (t + 1 < p.tp.n_tiles) S::acc_release(c);
                         match_block16<kPer - 2>(a, sc + 64 * (kPer - 2), best, win);
                         match_block16<kPer - 1>(a + 16, sc + 64 * (kPer - 1), best, win);
+                        if (t + 1 == p.tp.n_tiles) S::acc_release(c);   // (the norms are safe until the item's last release: Ctx::extra)
                     } else {
                         // (the group boundary is a multiple of 32 columns, the warp's share starts at one: pairs of blocks)
 #pragma unroll

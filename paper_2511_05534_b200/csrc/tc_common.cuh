@@ -106,7 +106,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
     }
 }
 
-// Two of them, both looked at before the one vote.
+// Two of them, the second one looked at after the first, both before the one vote.
 __device__ __forceinline__ bool mbar_wait_both_warp(uint32_t bar0, uint32_t parity0, uint32_t bar1, uint32_t parity1, volatile int *abort_flag,
                                                     int *status_word) {
     const bool there = mbar_try_wait(bar0, parity0), too = mbar_try_wait(bar1, parity1);

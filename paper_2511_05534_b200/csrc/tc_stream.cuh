@@ -98,8 +98,9 @@ struct Skel {
         int colhalf;               // ... and which half of each accumulator's columns
         bool ok;                   // false: shared memory was not 1024-byte aligned; nothing may run
         __device__ __forceinline__ uint32_t bar(int i) const { return bars + 8u * i; }
-        // shared address of the per-column constants of the bt-th B tile this CTA streams (valid from the tile's
-        // acc_extra_wait or quad_extra_wait_lanes to its release)
+        // shared address of the per-column constants of the bt-th B tile this CTA streams.  Valid from the tile's acc_extra_wait to
+        // the release of the item's tile after it, or, for an item's last tile, to its own release: until then the half may sit out
+        // an item, and what the issuer goes by is the last release.
         __device__ __forceinline__ uint32_t extra(int bt) const {
             return base + kSmemExtra + (uint32_t)(bt & (kExtraSlots - 1)) * kExtraBytes;
         }
@@ -179,7 +180,9 @@ struct Skel {
                 const int sb = bt % BST;
                 if (!p.reuse_b) ok = tc::mbar_wait_warp(c.bar(kBarBEmpty + sb), ((bt / BST) & 1) ^ 1, c.abort_flag, status);
                 if (!ok) break;
-                if (p.extra && !p.reuse_b) {   // slot reuse is safe: every epilogue released tile bt-4 before the stage of bt-2 was released
+                // The slot's readers are through with tile bt - 4: the stage just waited for was handed back after the products of tile
+                // bt - 2, which each half's wait for the release of its tile before, bt - 3 or older (mma_issuer).
+                if (p.extra && !p.reuse_b) {
                     const int xs = bt & (kExtraSlots - 1);
                     if (tc::elect_one()) {
                         tc::mbar_expect_tx(c.bar(kBarXFull + xs), kExtraBytes);
@@ -273,10 +276,10 @@ struct Skel {
                     }
                 }
                 if (!ok) break;
-                if constexpr (kQuads) {
-                    // accumulators without a part in this tile: their quads must be through with the tiles before it as well,
-                    // so that a tile's release tells the producer that nobody reads the constants of the tile before any more
-                    for (int q = 0; ok && q < 4; ++q)
+                if (kQuads || p.extra) {
+                    // accumulators without a part in this tile: their warps must be through with the tiles before it as well,
+                    // so that the stage's release tells the producer that nobody reads the constants of those tiles any more
+                    for (int q = 0; ok && q < 2 * kParts; ++q)
                         if (!(took & (1u << q))) ok = tc::mbar_wait_warp(c.bar(kBarAccEmpty + q), (ta[q] & 1) ^ 1, c.abort_flag, status);
                     if (!ok) break;
                 }
@@ -288,10 +291,13 @@ struct Skel {
 
     // Epilogue side.  `k` counts the accumulator tiles this warp's half has consumed.  (The waits are the whole warp's: votes,
     // shuffles and tensor-memory reads follow, which the warp must reach, or give up on, as one.)
-    // Waits for the accumulator and for the per-column constants of the bt-th B tile.
+    // Waits for the accumulator and then for the per-column constants of the bt-th B tile.  In this order: the products of tile bt
+    // come after half 0, which has a part in every tile, has seen the constants of tile bt - 4, so that the slot's barrier is in the
+    // phase of tile bt or just past it.  A half that sat out an item may come here while the barrier is two phases behind, where its
+    // parity is that of the phase waited for.
     static __device__ __forceinline__ bool acc_extra_wait(const Ctx &c, int k, int bt, int *status) {
-        const bool ok = tc::mbar_wait_both_warp(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1,
-                                                c.bar(kBarAccFull + c.group), k & 1, c.abort_flag, status);
+        const bool ok = tc::mbar_wait_both_warp(c.bar(kBarAccFull + c.group), k & 1, c.bar(kBarXFull + (bt & (kExtraSlots - 1))),
+                                                (bt / kExtraSlots) & 1, c.abort_flag, status);
         tc::tc_fence_after();
         return ok;
     }

@@ -88,3 +88,24 @@ def test_selection_lays_the_rows_out(U, H, L, B):
     tau = 2.0 * 32 / L
     _check(k[:n_units].astype(np.float64), m, g["retained"].reshape(U, H, B), g["evicted"].reshape(U, H, L - B), g["strategy"],
            g["importance"].reshape(U, H, L), np.float32(tau), g["match"].reshape(U, H, L - B), g["match_sim"].reshape(U, H, L - B))
+
+
+@pytest.mark.parametrize("H,B,E", [(40, 1300, 1892), (75, 2300, 600), (150, 1100, 300)])
+def test_halves_that_sit_items_out(H, B, E):
+    """More items than SMs, the last one of a head of one half of 128 rows: the other half's warps are tiles behind or ahead when the
+    CTA goes on, with five to nine tiles of candidates and their norms to an item."""
+    rng = np.random.default_rng(E)
+    U, L = 2, B + E
+    k = inputs.round_to_bf16(rng.standard_normal((U, H, L, 128)).astype(np.float32) * np.exp(rng.uniform(-2, 2, (U, H, L, 1))).astype(np.float32))
+    m = np.stack([np.arange(L) // 300 % 2, rng.random(L) < 0.3]).astype(np.uint8)
+    imp = rng.random((U, H, L)).astype(np.float32)
+    strat = np.array([0, 1], np.int32)
+    perm = np.argsort(rng.random((U, H, L)), axis=-1)
+    ret, evi = np.sort(perm[..., :B], -1).astype(np.int32), np.sort(perm[..., B:], -1).astype(np.int32)
+    fp = gpu_params(O.OracleParams(U, H, H, 128, L, 1, B, tau=1.0, tau_mode=O.TAU_ABS), F.BF16)
+    ws = F.alloc_workspace(fp)
+    match, sim = torch.full((U, H, E), -7, dtype=torch.int32, device="cuda"), torch.full((U, H, E), float("nan"), device="cuda")
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    F.flowmm_match(fp, to_dev(k, F.BF16), dev(imp), dev(m), dev(ret), dev(evi), dev(strat), match, sim, ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    _check(k, m, ret, evi, strat, imp, 1.0, match.cpu().numpy(), sim.cpu().numpy().astype(np.float64))
