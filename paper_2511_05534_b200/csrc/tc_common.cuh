@@ -286,24 +286,6 @@ __device__ __forceinline__ float ex2(float x) {        // 2^x, hardware approxim
     return y;
 }
 
-// 2^x on the FMA pipe (relative error 2.2e-7 for x in [-125, 127]; smaller x give 2^-125): round x to
-// the nearest integer n with the 1.5 * 2^23 trick, a degree-5 polynomial for 2^f on f = x - n in
-// [-0.5, 0.5] (own least-squares fit at Chebyshev nodes), then n is added to the exponent field.
-// The exp2 unit does 16 results per clock per SM; the row-statistics pass of the scoring step, which
-// is bound by that unit, sends a quarter of its exponentials here.
-__device__ __forceinline__ float ex2_fma(float x) {
-    x = fmaxf(x, -125.f);
-    const float t = x + 12582912.f;
-    const float f = x - (t - 12582912.f);
-    float p = 0.0013266971f;
-    p = fmaf(p, f, 0.0096754599f);
-    p = fmaf(p, f, 0.055507425f);
-    p = fmaf(p, f, 0.24022122f);
-    p = fmaf(p, f, 0.69314694f);
-    p = fmaf(p, f, 1.0000001f);
-    return __int_as_float(__float_as_int(p) + (__float_as_int(t) << 23));
-}
-
 // Packed fp32 pairs (sm_100): one instruction does two fused multiply-adds / two additions, which
 // halves the issue slots the scoring epilogues spend around their exponentials.
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
@@ -326,7 +308,8 @@ __device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
     return d;
 }
 
-// 2^x for a pair on the FMA pipe with packed operations (half the issue slots of two ex2_fma): x clamped at -125,
+// 2^x for a pair on the FMA pipe with packed operations.  The exp2 unit does 16 results per clock per SM; the row statistics of the
+// scoring step, which that unit bounds, send a quarter of their exponentials here: x clamped at -125,
 // n = round(x) by the 1.5 * 2^23 trick, 2^f on f = x - n in [-0.5, 0.5] by a degree-4 polynomial (own least-squares fit at
 // Chebyshev nodes with the constant fixed at 1: relative error 3.6e-6), n added to the exponent field.
 __device__ __forceinline__ float2 ex2_fma2(float2 x) {

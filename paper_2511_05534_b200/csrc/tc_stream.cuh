@@ -243,7 +243,7 @@ struct Skel {
                 const int ncols = min(NB, p.cols_total - t * NB);
                 const int ncols0 = p.cols_first ? min(NB, p.cols_first - t * NB) : ncols;
                 const uint32_t b_base = c.base + kSmemB + sb * kBStage;
-                uint32_t took = 0;
+                uint32_t took = 0;                                       // accumulators with a part in this tile
                 for (int h = 0; ok && h < p.n_halves; ++h) {
                     const int st = ia[h] % AST;
                     if (t == 0) ok = tc::mbar_wait_warp(c.bar(kBarAFull + st * 2 + h), (ia[h] / AST) & 1, c.abort_flag, status);
@@ -276,7 +276,7 @@ struct Skel {
                     }
                 }
                 if (!ok) break;
-                if (kQuads || p.extra) {
+                if (p.extra) {
                     // accumulators without a part in this tile: their warps must be through with the tiles before it as well,
                     // so that the stage's release tells the producer that nobody reads the constants of those tiles any more
                     for (int q = 0; ok && q < 2 * kParts; ++q)
@@ -323,11 +323,12 @@ struct Skel {
         tc::tc_fence_after();
         return ok;
     }
-    // Waits for the accumulator and, where tiles carry per-column constants (bt >= 0), for those of the bt-th B tile, lane by lane:
-    // only for an epilogue whose lanes stay in step whatever their waits return, until pair_meet has told all of them.
+    // Waits for the accumulator and, where tiles carry per-column constants (bt >= 0; the second scoring pass forms its own), then for
+    // those of the bt-th B tile, lane by lane: only for an epilogue whose lanes stay in step whatever their waits return, until
+    // pair_meet has told all of them.
     static __device__ __forceinline__ bool quad_extra_wait_lanes(const Ctx &c, int k, int bt, int *status) {
-        const bool ok = (bt < 0 || tc::mbar_wait(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1, c.abort_flag, status)) &&
-                        tc::mbar_wait(c.bar(kBarAccFull + 2 * c.group + c.colhalf), k & 1, c.abort_flag, status);
+        const bool ok = tc::mbar_wait(c.bar(kBarAccFull + 2 * c.group + c.colhalf), k & 1, c.abort_flag, status) &&
+                        (bt < 0 || tc::mbar_wait(c.bar(kBarXFull + (bt & (kExtraSlots - 1))), (bt / kExtraSlots) & 1, c.abort_flag, status));
         tc::tc_fence_after();
         return ok;
     }
