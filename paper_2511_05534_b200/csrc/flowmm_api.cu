@@ -663,16 +663,19 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         FLOWMM_LAUNCHED("merge_tc");
         return FLOWMM_OK;
     }
-    // Short lists: straight from the matches.  Every block of slots reads its head's whole list, where the sorted way is two launches
-    // and streams.  Time of the one over the other's, members spread evenly (with 15 % of them in one slot): up to 2048 blocks 0.4 to
-    // 0.9 for up to 1000 members (500 0.6 to 1.6, 1000 1.0 to 2.3); about 3600 blocks 0.98 to 1.13 up to 256 members, 1.17 beyond;
-    // 5600 blocks of 32 heads 0.70 to 0.87 up to 256 members, 1.0 to 1.1 beyond, 5900 of 112 heads 1.05 to 1.24 and 1.3 to 1.5;
-    // 14 000 and more 1.3 to 2.0.
+    // Short lists: straight from the matches.  Every block of slots reads its head's whole list, where the sorted way is two launches,
+    // the first of them a block per head that walks all of the head's slots, and streams.  Up to 256 members the number of heads
+    // decides, as that block's time grows with the slots of a head and the short way's with the slots of all heads; the second
+    // launch counts while both are small.  Time of the short way over the sorted one, members spread evenly or 15 % of them in one slot,
+    // 100 to 256 members, bf16 of 64 and 128 and fp32: 2 heads 0.09 to 0.14 at any number of slots, 8 heads 0.30 to 0.58, 24 heads
+    // 0.70 to 0.95, 32 heads 0.72 to 1.04 up to 8000 blocks and 0.79 to 1.11 at 20 000 and 60 000, 40 heads 0.74 to 1.20 and 0.90 to
+    // 1.27, 48 heads 0.85 to 1.23 and 1.06 to 1.56, 96 heads 0.97 to 1.24 at 3600 blocks and 0.99 to 1.58 beyond, 160 heads 1.03 to 1.39
+    // and 1.15 to 1.84.  For up to 1000 members (500 0.6 to 1.6, 1000 1.0 to 2.3 with 15 % in one slot) 0.4 to 0.9 up to 2048 blocks.
     const int64_t slot_blocks = (int64_t)UH * ((p.n_keep + 7) / 8);
     // a slot per warp while the blocks fit the SMs together, else four, which share the block's copy of the list
     const int per = slot_blocks <= 4 * tc::sm_count() ? 1 : 4, grid_y = (p.n_keep + 8 * per - 1) / (8 * per);
     // (more slots than a grid has room for: the persistent kernels below take any number)
-    if (E > 0 && grid_y <= 65535 && (E <= 256 ? slot_blocks <= (UH <= 32 ? 6000 : 3600) : E <= kShortList && slot_blocks <= 2048)) {
+    if (E > 0 && grid_y <= 65535 && (E <= 256 ? UH <= 32 || slot_blocks <= 3600 : E <= kShortList && slot_blocks <= 2048)) {
         const dim3 grid(UH, grid_y);
         auto kernel = p.dtype == FLOWMM_BF16 ? (per == 1 ? merge_short_kernel<__nv_bfloat16, 1> : merge_short_kernel<__nv_bfloat16, 4>)
                                              : (per == 1 ? merge_short_kernel<float, 1> : merge_short_kernel<float, 4>);

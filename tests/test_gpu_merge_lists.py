@@ -116,3 +116,27 @@ def test_short_list_with_more_slots_than_a_grid_has_rows(B):
         # the output's rounding to bf16 (8 bits: 2^-8 of the value), and below it fp32 sums of up to 69 members: (69 + 16) 2^-24
         # of the mean magnitude, which is below 8
         assert torch.all((got[0, 0][slots].double() - ref).abs() <= ref.abs() * 2 ** -8 + 2 ** -14)
+
+
+@pytest.mark.parametrize("E,B,heads,launches", [(100, 40000, 2, 1), (256, 20000, 3, 1), (256, 2100, 32, 1), (257, 20000, 3, 2), (200, 1000, 33, 2), (200, 800, 33, 1)])
+def test_few_heads_of_many_slots(E, B, heads, launches):
+    """Up to 256 members of up to 32 heads go straight from the matches however many slots there are: a list builder of a block per
+    head walks the slots one round after the other (2 heads of 30 000 slots took ten times as long)."""
+    rng = np.random.default_rng(E + B)
+    D, L = 64, E + B
+    k, v = (small_integers(rng, (1, heads, L, D)) for _ in range(2))
+    ret = np.sort(np.argsort(rng.random((1, heads, L)), -1)[..., :B], -1).astype(np.int32)
+    evi = np.stack([np.setdiff1d(np.arange(L), r) for r in ret[0]])[None].astype(np.int32)
+    match = rng.integers(-1, B, (1, heads, E)).astype(np.int32)
+    sim = np.where(match >= 0, rng.random((1, heads, E)), 0).astype(np.float32)
+    p = O.OracleParams(1, heads, heads, D, L, 1, B, merge_mode=F.MERGE_MEAN)
+    refs = merge_reference(p, k, v, ret, evi, match, sim.astype(np.float64), F.BF16)
+    fp = gpu_params(p, F.BF16)
+    t = lambda x: torch.from_numpy(x).cuda()
+    g = [torch.full((1, heads, B, D), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    ws = F.alloc_workspace(fp)
+    F.flowmm_merge(fp, to_dev(k, F.BF16), to_dev(v, F.BF16), *(t(x) for x in (ret, evi, match, sim)), g[0], g[1], ws)
+    assert F.flowmm_last_launch_count() == launches
+    assert F.flowmm_last_device_status(ws) == 0
+    for got, (ref, bound) in zip(g, refs):
+        assert np.all(np.abs(got.double().cpu().numpy() - ref) <= bound)
