@@ -103,7 +103,8 @@ typedef struct {
 } flowmm_params;
 
 /* Scratch size in bytes that any entry point below needs for these params.  Host only; makes
- * no CUDA call.  Fails with the same validation errors as the compute entry points. */
+ * no CUDA call.  Fails with the same validation errors as the compute entry points.  Never smaller
+ * for more units or a longer context with all other fields alike, so a workspace serves those calls too. */
 flowmm_status flowmm_workspace_bytes(const flowmm_params *p, size_t *bytes);
 
 /*

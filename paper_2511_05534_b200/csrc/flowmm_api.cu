@@ -6,6 +6,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
@@ -92,7 +93,9 @@ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // (items = pairs x row tiles), so the bound is generous rather than a grid limit of 65535.
 constexpr int64_t kMaxHeadsPerCall = 1 << 22;
 
-constexpr int kScoreCtas = 148;             // one per SM of a B200
+// Blocks that the scoring is cut for: one per SM of a B200, and about two of the SIMT kernels.  (By hand: the size of a workspace is
+// asked for without a GPU.)
+constexpr int kScoreCtas = 148, kSimtCtas = 2 * kScoreCtas;
 
 // Where everything lives inside the caller's workspace.  One layout serves every entry point.
 struct Layout {
@@ -108,7 +111,7 @@ struct Layout {
 
 int chunks_for(int L, int other_ctas, int &chunk) {
     // enough CTAs to fill the GPU about twice, at least 64 keys per chunk
-    int want = (2 * 148 + other_ctas - 1) / other_ctas;
+    int want = (kSimtCtas + other_ctas - 1) / other_ctas;
     const int max_chunks = (L + kTile - 1) / kTile;
     if (want < 1) want = 1;
     if (want > max_chunks) want = max_chunks;
@@ -123,9 +126,10 @@ int chunks_for(int L, int other_ctas, int &chunk) {
 // stride, and of 64 from the counter, us: 300 000 rows 44 to 53, 53 to 64; 0.8 million 83, 86; 1.0 million 109 to 123, 113 to 124;
 // 1.3 million 154, 156; 1.6 million 165, 164; 2.5 million 257, 248; 4.3 million 422, 392 (fp32 rows of 64 within 1 %, equal from 0.8 million on).
 constexpr int64_t kManyRows = 1300000;
+constexpr int kMinWin = 16;
 int merge_window(const flowmm_params &p) {
     const int64_t rows = (int64_t)p.n_units * p.n_kv_heads * p.seq_len;
-    return rows >= kManyRows ? mrow::kMaxWin : rows >= 40000 ? 32 : 16;
+    return rows >= kManyRows ? mrow::kMaxWin : rows >= 40000 ? 32 : kMinWin;
 }
 
 // The part of the workspace that the merge step uses (rows in slot order, windows, pieces, partial sums).
@@ -142,7 +146,7 @@ void layout_merge(Layout &y, const flowmm_params &p, Take take) {
     y.rows = take(UH * L * 8);
     y.row_count = take(UH * 8);
     y.off = take(UH * (B + 1) * 4);
-    y.first_slot = take(UH * (size_t)y.n_win * 4);
+    y.first_slot = take(UH * ((L + kMinWin - 1) / kMinWin) * 4);   // (of the shortest windows, so that more rows never need less room)
     y.part_off = take(UH * (B + 1) * 4);
     y.pieces = take(UH * (size_t)y.max_parts * 16);
     y.partial = take(UH * (size_t)y.max_parts * (2 * D + 4) * 4);
@@ -186,10 +190,13 @@ Layout make_layout(const flowmm_params &p) {
         const size_t spread = (size_t)y.tc_runs / (U * Hkv) + 2;          // runs that a head's tiles can be in
         y.tc_n_part = (int)(spread < (size_t)y.n_rt ? spread : (size_t)y.n_rt);
     }
-    const size_t max_chunk1 = (size_t)(y.n_chunk1 > 2 * y.tc_n_part ? y.n_chunk1 : 2 * y.tc_n_part);   // records of 8 (SIMT) or 16 bytes
-    const size_t max_chunk2 = (size_t)y.n_chunk2 > W ? (size_t)y.n_chunk2 : W > 8 ? W : 8;
-    y.row_part = take(U * Hq * W * max_chunk1 * 8);
-    y.cross_part = take(U * Hq * max_chunk2 * 4);
+    // Row statistics and partial masses: bounds of what the cuts above come to for all heads (records of 16 bytes, of the SIMT kernels of
+    // 8, per proxy row) that, unlike those, never fall when units or tokens are added.
+    const size_t UH = U * Hkv, key_tiles = (L + kTile - 1) / kTile, qt = (G * W + tcs::kItemRows - 1) / tcs::kItemRows;
+    const size_t parts = std::min(UH * (size_t)y.n_rt, std::max<size_t>(kScoreCtas / qt, 1) + 2 * UH);
+    const size_t simt1 = std::min(UH * key_tiles, kSimtCtas / row_tiles + 1 + UH), simt2 = std::min(UH * key_tiles, kSimtCtas + UH);
+    y.row_part = take(G * W * std::max(16 * parts, 8 * simt1));
+    y.cross_part = take(G * std::max(simt2, UH * std::max<size_t>(W, 8)) * 4);
     y.row_all = take(U * Hq * W * 16);
     layout_merge(y, p, take);
     y.merge_status = y.status;

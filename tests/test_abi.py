@@ -59,3 +59,20 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(F, "LIB_PATH", str(tmp_path / "libflowmm.so"))
     with pytest.raises(FileNotFoundError):
         F.load()
+
+
+@pytest.mark.parametrize("Hkv,G,W,D,dtype", [(4, 7, 32, 128, F.BF16), (8, 8, 64, 128, F.BF16), (32, 1, 32, 128, F.BF16), (1, 8, 128, 128, F.BF16),
+                                             (3, 5, 32, 128, F.BF16), (4, 4, 16, 64, F.F32), (1, 4, 100, 128, F.F32)])
+def test_workspace_never_shrinks_with_the_problem(lib, Hkv, G, W, D, dtype):
+    """A workspace kept for the most units and the longest context serves the smaller calls of the same budget, across the lines at which
+    windows, chunks and items change size."""
+    size = lambda U, L, B: F.flowmm_workspace_bytes(F.Params(U, G * Hkv, Hkv, D, L, W, B, dtype=dtype))
+    for U in (1, 2, 5, 28):
+        for B in (16, 500):
+            lengths = sorted({max(B, W) + i for i in range(900)} | set(range(max(B, W), 45000, 37)) | {40000 // (U * Hkv) + i for i in range(-300, 300)} |
+                             {1300000 // (U * Hkv) + i for i in range(-300, 300)})
+            sizes = [size(U, L, B) for L in lengths if L >= max(B, W)]
+            assert sizes == sorted(sizes), (U, B)
+    for L, B in ((200, 50), (640, 64), (2176, 217), (33792, 1690)):
+        sizes = [size(U, L, B) for U in range(1, 320)]
+        assert sizes == sorted(sizes), (L, B)
