@@ -435,6 +435,7 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
             if (kCtas > 1) {                                         // (from here on `all` is the head's)
                 const unsigned long long ahead = cluster_sum(all, all);
                 seen = (int)(ahead & 0xFFFFFF); seen_t = (int)(ahead >> 24) & 0xFFFFF; seen_v = (int)(ahead >> 44);
+                if (!with_prepare) cluster_arrive();                 // the other CTAs' totals have been read
                 if (tiles_here) {                                    // (every CTA of the cluster has read the counters)
                     for (int t = tid; t < P.n_rt; t += kThreads) tiles[t] = 0;
                     __syncthreads();
@@ -450,8 +451,21 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
                     s += (int)(c & 0xFFFFFF); pt += (int)(c >> 24) & 0xFFFFF; pv += (int)(c >> 44);
                 }
                 __syncthreads();
+                // The lists, a word per warp and step: coalesced.  A selection alone has a loop of its own: the other's stores to shared
+                // memory keep its steps apart.
+                if (!with_prepare) {
 #pragma unroll 4
-                for (int w = warp; w < n_w; w += kWarps) {           // the lists, a word per warp and step: coalesced
+                    for (int w = warp; w < n_w; w += kWarps) {
+                        const uint32_t keep = keep_w[w];
+                        const int i = c0 + 32 * w + lane, sl = pos_w[w] + __popc(keep & lt);
+                        if (i >= L) continue;
+                        if (!((keep >> lane) & 1u)) { evi[i - sl] = i0 + i; continue; }
+                        ret[sl] = i0 + i;
+                        if (A.row_mod_out) A.row_mod_out[(int64_t)head * A.B + sl] = mod[i];
+                    }
+                } else
+#pragma unroll 4
+                for (int w = warp; w < n_w; w += kWarps) {
                     const uint32_t keep = keep_w[w];
                     const int i = c0 + 32 * w + lane, sl = pos_w[w] + __popc(keep & lt);
                     bool is_vis = false;
@@ -469,19 +483,17 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
                     }
                     ret[sl] = i0 + i;
                     if (A.row_mod_out) A.row_mod_out[(int64_t)head * A.B + sl] = mod[i];
-                    if (with_prepare) {
-                        if (copy_here) rank[i] = -(sl + 2);
-                        const uint32_t text = text_w[w], vis = vis_w[w];
-                        const int c = ((text >> lane) & 1u) ? pt_w[w] + __popc(text & lt) : ((vis >> lane) & 1u) ? pv_w[w] + __popc(vis & lt) : -1;
-                        if (c >= 0 && index_ok(c, P.Ctot, P.status)) {
-                            slot_out[c] = sl;
-                            if (copy_here) {
-                                if (kCtas > 1) {
-                                    const uint32_t at = (uint32_t)__cvta_generic_to_shared(cand_tok + c);
+                    if (copy_here) rank[i] = -(sl + 2);
+                    const uint32_t text = text_w[w], vis = vis_w[w];
+                    const int c = ((text >> lane) & 1u) ? pt_w[w] + __popc(text & lt) : ((vis >> lane) & 1u) ? pv_w[w] + __popc(vis & lt) : -1;
+                    if (c >= 0 && index_ok(c, P.Ctot, P.status)) {
+                        slot_out[c] = sl;
+                        if (copy_here) {
+                            if (kCtas > 1) {
+                                const uint32_t at = (uint32_t)__cvta_generic_to_shared(cand_tok + c);
 #pragma unroll
-                                    for (int q = 0; q < kCtas; ++q) st_cluster_u32(at, q, (uint32_t)(i0 + i));
-                                } else cand_tok[c] = i;
-                            }
+                                for (int q = 0; q < kCtas; ++q) st_cluster_u32(at, q, (uint32_t)(i0 + i));
+                            } else cand_tok[c] = i;
                         }
                     }
                 }
@@ -535,7 +547,10 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
         if (kCtas > 1) cluster_sync(); else __syncthreads();         // every candidate's token is in place, in every CTA
         const int lo = P.Ctot / 32 * rank_c / kCtas * 32, hi = P.Ctot / 32 * (rank_c + 1) / kCtas * 32;
         match_gather_rows<8>(P, head, cand_tok, lo, hi, tid, kThreads);
-    } else if (kCtas > 1) cluster_sync();                            // nobody's words go away while they are read
+    } else if (kCtas > 1) {                                          // nobody's totals and tiles go away while they are read
+        if (with_prepare) cluster_arrive();
+        cluster_wait();
+    }
 }
 
 }  // namespace flowmm
