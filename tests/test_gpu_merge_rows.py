@@ -1,6 +1,7 @@
 """Merge of sorted lists by windows of rows: slots of chosen numbers of members (none, the most that stay whole, one more, several
 pieces) at chosen places of a window, windows of 16, 32 and 64 rows, taken with a stride or drawn from the counter,
-pieces of long slots as items of their own and spread over the windows, every row width, and output layouts with gaps.
+pieces of long slots as items of their own and spread over the windows, every row width, heads and units that differ, and layouts of
+all tensors with gaps or other strides.
 The values let one lost or doubled member be seen (test_merge_reference.py)."""
 import numpy as np
 import pytest
@@ -9,7 +10,7 @@ import torch
 from oracle import flowmm_oracle as O
 from paper_2511_05534_b200 import binding as F
 
-from gpu_util import gpu_params, merge_reference, small_integers, to_dev
+from gpu_util import gpu_params, merge_reference, small_integers
 
 pytestmark = pytest.mark.gpu
 
@@ -30,92 +31,84 @@ def _members(pattern, B, rng):
     return n
 
 
+def _lists(rng, B, E, counts):
+    """Pivots, non-pivots and matches of heads whose slots have these numbers of members, [variants, .]; what is left of E is dropped."""
+    L = B + E
+    ret = np.stack([np.sort(rng.choice(L, B, replace=False)) for _ in counts])
+    evi = np.stack([np.setdiff1d(np.arange(L), r) for r in ret])
+    match = np.stack([rng.permutation(np.concatenate([np.repeat(np.arange(B), n), np.full(E - n.sum(), -1)])) for n in counts])
+    sim = np.where(match >= 0, rng.random(match.shape), 0)
+    return ret.astype(np.int32), evi.astype(np.int32), match.astype(np.int32), sim.astype(np.float32)
+
+
+def _heads(x, U, H, roll=False):
+    """[variants, ...] as [U, H, ...] on the GPU: the heads have the variants by turns, their rows' columns rolled by the head's number,
+    so that a row or a list of another head shows."""
+    x = torch.from_numpy(x).cuda()
+    return torch.stack([x[i % len(x)].roll(i, -1) if roll else x[i % len(x)] for i in range(U * H)]).reshape(U, H, *x.shape[1:])
+
+
+def _gaps(x):
+    """The same values with NaN between rows, heads and units (gaps of 16 bytes' multiples)."""
+    U, H, L, D = x.shape
+    row, head = D + 8, L * (D + 8) + 24
+    return torch.full((U * H * head + U * 8,), float("nan"), device="cuda", dtype=x.dtype).as_strided((U, H, L, D), (H * head + 8, head, row, 1)).copy_(x)
+
+
+def _check_merge(rng, U, H, B, E, D, dtype, mode, counts):
+    """K by tokens first, V and the outputs with gaps, against the oracle for each of the variants."""
+    L = B + E
+    k, v = (small_integers(rng, (1, len(counts), L, D)) for _ in range(2))
+    lists = _lists(rng, B, E, counts)
+    ref_p = O.OracleParams(1, len(counts), len(counts), D, L, 1, B, merge_mode=mode)
+    refs = merge_reference(ref_p, k, v, *(x[None] for x in lists[:3]), lists[3][None].astype(np.float64), dtype)
+    kd, vd = (_heads(x[0], U, H, roll=True).to(F.torch_dtype(dtype)) for x in (k, v))
+    kd = kd.transpose(1, 2).contiguous().transpose(1, 2)
+    fp = gpu_params(O.OracleParams(U, H, H, D, L, 1, B, merge_mode=mode), dtype)
+    ws = F.alloc_workspace(fp)
+    out = [torch.full((U, H, B, D + 8), float("nan"), dtype=F.torch_dtype(dtype), device="cuda")[..., :D] for _ in range(2)]
+    F.flowmm_merge(fp, kd, _gaps(vd), *(_heads(x, U, H) for x in lists), out[0], out[1], ws)
+    assert F.flowmm_last_device_status(ws) == 0
+    for got, (ref, bound) in zip(out, refs):
+        assert torch.all((got.double() - _heads(ref[0], U, H, roll=True)).abs() <= _heads(bound[0], U, H, roll=True))
+
+
 @pytest.mark.parametrize("dtype,D", [(F.BF16, 128), (F.BF16, 64), (F.F32, 64), (F.F32, 128)])
-@pytest.mark.parametrize("heads", [1, 12, 90])                     # windows of 16, of 32 with pieces of their own, of 32 with pieces spread
+@pytest.mark.parametrize("U,H", [(1, 1), (4, 5), (2, 45)])          # windows of 16, of 32 with pieces of their own, of 32 with pieces spread
 @pytest.mark.parametrize("pattern", ["edges_first", "edges_apart", "edges_last", "alternate"])
-def test_slots_of_chosen_sizes(pattern, heads, dtype, D):
-    rng = np.random.default_rng(D + heads)
+def test_slots_of_chosen_sizes(pattern, U, H, dtype, D):
+    rng = np.random.default_rng(D + U * H)
     B = 700
-    n = _members(pattern, B, rng)
-    dropped = 150
-    E = int(n.sum()) + dropped
-    L = E + B
-    if E <= 1024:
-        pytest.skip("short list")
-    k, v = (small_integers(rng, (1, 1, L, D)) for _ in range(2))
-    ret = np.sort(rng.choice(L, B, replace=False))
-    evi = np.setdiff1d(np.arange(L), ret)
-    match = np.concatenate([np.repeat(np.arange(B), n), np.full(dropped, -1)])
-    rng.shuffle(match)
-    sim = np.where(match >= 0, rng.random(E), 0).astype(np.float32)
-    ret, evi, match = (x.astype(np.int32)[None, None] for x in (ret, evi, match))
-    sim = sim[None, None]
-    rep = lambda x: torch.from_numpy(np.ascontiguousarray(np.repeat(x, heads, 1))).cuda()
-    lists = [rep(x) for x in (ret, evi, match, sim)]
-    kd, vd = (rep(x).to(F.torch_dtype(dtype)) for x in (k, v))
+    counts = [_members(pattern, B, rng) for _ in range(min(U * H, 7))]
+    E = max(int(n.sum()) for n in counts) + 150
+    assert E > 1024 and (U * H == 1 or U * H * (E + B) >= 40000)    # (no short list)
     for mode in (F.MERGE_MEAN, F.MERGE_EXPSIM):
-        refs = merge_reference(O.OracleParams(1, 1, 1, D, L, 1, B, merge_mode=mode), k, v, ret, evi, match, sim.astype(np.float64), dtype)
-        fp = gpu_params(O.OracleParams(1, heads, heads, D, L, 1, B, merge_mode=mode), dtype)
-        ws = F.alloc_workspace(fp)
-        out = [torch.full((1, heads, B, D + 8), float("nan"), dtype=F.torch_dtype(dtype), device="cuda")[..., :D] for _ in range(2)]
-        F.flowmm_merge(fp, kd, vd, *lists, out[0], out[1], ws)
-        assert F.flowmm_last_device_status(ws) == 0
-        for got, (ref, bound) in zip(out, refs):
-            assert np.all(np.abs(got[:, :1].double().cpu().numpy() - ref) <= bound), mode
-            assert torch.equal(got, got[:, :1].expand(-1, heads, -1, -1))
+        _check_merge(rng, U, H, B, E, D, dtype, mode, counts)
 
 
 def test_many_rows_draw_their_windows():
     """1.6 million rows of 160 heads: windows of 64 from the counter."""
     rng = np.random.default_rng(3)
-    heads, B, D = 160, 1000, 64
-    n = _members("edges_apart", B, rng)
-    n[300:340] = rng.integers(100, 160, 40)
-    E = int(n.sum())
-    L = E + B
-    assert heads * L >= 1300000
-    k, v = (small_integers(rng, (1, 1, L, D)) for _ in range(2))
-    ret = np.sort(rng.choice(L, B, replace=False))
-    evi = np.setdiff1d(np.arange(L), ret)
-    match = rng.permutation(np.repeat(np.arange(B), n))
-    ret, evi, match = (x.astype(np.int32)[None, None] for x in (ret, evi, match))
-    sim = rng.random((1, 1, E)).astype(np.float32)
-    refs = merge_reference(O.OracleParams(1, 1, 1, D, L, 1, B, merge_mode=F.MERGE_MEAN), k, v, ret, evi, match, sim.astype(np.float64), F.BF16)
-    rep = lambda x: torch.from_numpy(np.ascontiguousarray(np.repeat(x, heads, 1))).cuda()
-    fp = gpu_params(O.OracleParams(1, heads, heads, D, L, 1, B, merge_mode=F.MERGE_MEAN), F.BF16)
-    out = [torch.full((1, heads, B, D), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
-    ws = F.alloc_workspace(fp)
-    F.flowmm_merge(fp, rep(k).bfloat16(), rep(v).bfloat16(), *(rep(x) for x in (ret, evi, match, sim)), out[0], out[1], ws)
-    assert F.flowmm_last_device_status(ws) == 0
-    for got, (ref, bound) in zip(out, refs):
-        assert np.all(np.abs(got[:, :1].double().cpu().numpy() - ref) <= bound)
-        assert torch.equal(got, got[:, :1].expand(-1, heads, -1, -1))
+    B = 1000
+    counts = [_members("edges_apart", B, rng) for _ in range(7)]
+    for n in counts:
+        n[300:340] = rng.integers(100, 160, 40)
+    E = max(int(n.sum()) for n in counts)
+    assert 160 * (E + B) >= 1300000
+    _check_merge(rng, 2, 80, B, E, 64, F.BF16, F.MERGE_MEAN, counts)
 
 
 @pytest.mark.parametrize("E", [1, 33, 300, 2047, 2048, 2049, 4096])
 def test_lists_of_many_heads(E):
-    """150 heads, so a block per head: positions kept from the first walk (up to 2048) and staged, a sixth of them dropped."""
+    """150 heads, so a block per head: positions kept from the first walk (up to 2048) and staged, about a sixth of them dropped."""
     rng = np.random.default_rng(E)
-    heads, B, D = 150, 700, 128
-    L = E + B
-    k, v = (small_integers(rng, (1, 1, L, D)) for _ in range(2))
-    ret = np.sort(rng.choice(L, B, replace=False))
-    evi = np.setdiff1d(np.arange(L), ret)
-    match = np.where(rng.random(E) < 1 / 6, -1, np.minimum(rng.integers(0, B, E), rng.integers(0, 2 * B, E)))   # (some slots popular)
-    sim = np.where(match >= 0, rng.random(E), 0).astype(np.float32)[None, None]
-    ret, evi, match = (x.astype(np.int32)[None, None] for x in (ret, evi, match))
-    rep = lambda x: torch.from_numpy(np.ascontiguousarray(np.repeat(x, heads, 1))).cuda()
-    lists = [rep(x) for x in (ret, evi, match, sim)]
+    B = 700
+    counts = []
+    for _ in range(7):                                              # (some slots popular)
+        match = np.where(rng.random(E) < 1 / 6, -1, np.minimum(rng.integers(0, B, E), rng.integers(0, 2 * B, E)))
+        counts.append(np.bincount(match[match >= 0], minlength=B))
     for mode in (F.MERGE_MEAN, F.MERGE_EXPSIM):
-        refs = merge_reference(O.OracleParams(1, 1, 1, D, L, 1, B, merge_mode=mode), k, v, ret, evi, match, sim.astype(np.float64), F.BF16)
-        fp = gpu_params(O.OracleParams(1, heads, heads, D, L, 1, B, merge_mode=mode), F.BF16)
-        out = [torch.full((1, heads, B, D), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
-        ws = F.alloc_workspace(fp)
-        F.flowmm_merge(fp, rep(k).bfloat16(), rep(v).bfloat16(), *lists, out[0], out[1], ws)
-        assert F.flowmm_last_device_status(ws) == 0
-        for got, (ref, bound) in zip(out, refs):
-            assert np.all(np.abs(got[:, :1].double().cpu().numpy() - ref) <= bound), mode
-            assert torch.equal(got, got[:, :1].expand(-1, heads, -1, -1))
+        _check_merge(rng, 2, 75, B, E, 128, F.BF16, mode, counts)
 
 
 @pytest.mark.parametrize("dtype,D,E", [(F.BF16, 128, 0), (F.BF16, 64, 0), (F.BF16, 64, 1), (F.F32, 64, 0), (F.F32, 128, 1)])
