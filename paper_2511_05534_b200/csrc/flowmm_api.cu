@@ -125,11 +125,18 @@ int chunks_for(int L, int other_ctas, int &chunk) {
 // From kManyRows on warps draw their windows from a counter, else windows are taken with a stride.  The merge by windows of 32 with a
 // stride, and of 64 from the counter, us: 300 000 rows 44 to 53, 53 to 64; 0.8 million 83, 86; 1.0 million 109 to 123, 113 to 124;
 // 1.3 million 154, 156; 1.6 million 165, 164; 2.5 million 257, 248; 4.3 million 422, 392 (fp32 rows of 64 within 1 %, equal from 0.8 million on).
+// While every warp has one window at most, the windows are as short as leaves it so, by groups of four rows (other lengths misalign the
+// reads of the list: 64 heads of 1688 rows by 31 were 1.3 % slower): 112 caches of 640 rows by 24 instead of 32 80.7 -> 78.8 us for the call,
+// 16 heads of 3972 by 20 75.4 -> 72.9.  (Equal numbers of longer windows, 39 rows for 270 000, 232 -> 243.)
 constexpr int64_t kManyRows = 1300000;
-constexpr int kMinWin = 16;
+constexpr int kMinWin = 16, kMergeCtas = 3 * kScoreCtas;
 int merge_window(const flowmm_params &p) {
-    const int64_t rows = (int64_t)p.n_units * p.n_kv_heads * p.seq_len;
-    return rows >= kManyRows ? mrow::kMaxWin : rows >= 40000 ? 32 : kMinWin;
+    const int64_t heads = (int64_t)p.n_units * p.n_kv_heads, rows = heads * p.seq_len;
+    if (rows >= kManyRows) return mrow::kMaxWin;
+    if (rows < 40000) return kMinWin;
+    int win = kMinWin;
+    while (win < 32 && heads * ((p.seq_len + win - 1) / win) > kMergeCtas * mrow::kWarps) win += 4;
+    return win;
 }
 
 // The part of the workspace that the merge step uses (rows in slot order, windows, pieces, partial sums).

@@ -1,5 +1,5 @@
 """Merge of sorted lists by windows of rows: slots of chosen numbers of members (none, the most that stay whole, one more, several
-pieces) at chosen places of a window, windows of 16, 32 and 64 rows, taken with a stride or drawn from the counter,
+pieces) at chosen places of a window, windows of 16 to 32 and of 64 rows, taken with a stride or drawn from the counter,
 pieces of long slots as items of their own and spread over the windows, every row width, heads and units that differ, and layouts of
 all tensors with gaps or other strides.
 The values let one lost or doubled member be seen (test_merge_reference.py)."""
@@ -84,6 +84,18 @@ def test_slots_of_chosen_sizes(pattern, U, H, dtype, D):
     assert E > 1024 and (U * H == 1 or U * H * (E + B) >= 40000)    # (no short list)
     for mode in (F.MERGE_MEAN, F.MERGE_EXPSIM):
         _check_merge(rng, U, H, B, E, D, dtype, mode, counts)
+
+
+@pytest.mark.parametrize("H,win", [(16, 20), (20, 24), (23, 28)])
+@pytest.mark.parametrize("dtype,D", [(F.BF16, 128), (F.F32, 64)])
+def test_windows_in_between(H, win, dtype, D):
+    """Windows of 20, 24 and 28 rows: the shortest that give each of 3552 warps one at most."""
+    rng = np.random.default_rng(H + D)
+    B = 700
+    counts = [_members(p, B, rng) for p in ("edges_apart", "edges_last", "alternate")]
+    E = 4000 - B
+    assert min(w for w in range(16, 36, 4) if H * -(-4000 // w) <= 3552) == win and max(n.sum() for n in counts) < E
+    _check_merge(rng, 1, H, B, E, D, dtype, F.MERGE_EXPSIM, counts)
 
 
 def test_many_rows_draw_their_windows():
