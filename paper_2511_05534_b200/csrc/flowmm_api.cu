@@ -532,6 +532,9 @@ flowmm_status run_select(const flowmm_params &p, const float *importance, int32_
         a.chunk = part;
         return launch_select<512, true, 4>(a, f, g, prep != nullptr, st);
     }
+    // More heads than four blocks of 256 threads per SM would be in two rounds; of 128 threads an SM holds eight.  (1024 heads of 640
+    // positions 151.4 -> 149.5 us for the call, of 1000 222.7 -> 221.4; of 400, where a block's rounds are short, 110.4 -> 111.5.)
+    if (p.seq_len > 512 && p.seq_len <= 1024 && a.n_heads > 4 * tc::sm_count()) return launch_select<128, true>(a, f, g, prep != nullptr, st);
     if (p.seq_len <= 1024) return launch_select<256, true>(a, f, g, prep != nullptr, st);
     if (p.seq_len <= 4096) return launch_select<512, true>(a, f, g, prep != nullptr, st);
     if (p.seq_len <= kSelMaxChunk) return launch_select<1024, true>(a, f, g, prep != nullptr, st);

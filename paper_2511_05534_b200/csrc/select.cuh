@@ -4,6 +4,8 @@
 #include "common.cuh"
 #include "match_tc.cuh"
 
+#include <type_traits>
+
 namespace flowmm {
 
 // Order-preserving integer key of an importance (a non-negative float); window tokens forced
@@ -89,7 +91,7 @@ static_assert(select_smem(kSelMaxChunk) <= 232448 - 1024, "shared memory budget"
 // added up through distributed shared memory in every pass, their totals before the lists are written.  For calls of few
 // heads, whose blocks would leave most SMs idle: 8 heads of 33 792 tokens 31 -> 18 us, 4 heads of 8448 14 -> 12.
 template <int kThreads, bool kOneChunk, int kCtas>
-__global__ void __launch_bounds__(kThreads, kThreads == 256 ? 4 : kThreads == 512 && kCtas == 1 ? 2 : 1)
+__global__ void __launch_bounds__(kThreads, kThreads <= 256 ? 1024 / kThreads : kThreads == 512 && kCtas == 1 ? 2 : 1)
 select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P, int with_prepare) {
     static_assert(kCtas == 1 || (kOneChunk && kThreads == 512), "a CTA's part is one chunk; four counters per thread");
     constexpr int kWarps = kThreads / 32, kPer = kSelBins / kThreads;
@@ -166,8 +168,17 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
             for (int q = 0; q < kCtas; ++q) { c[0] += (int)part[q].w; c[1] += (int)part[q].z; c[2] += (int)part[q].y; c[3] += (int)part[q].x; }
             sum = (c[0] + c[1]) + (c[2] + c[3]);
         } else {
+            // (16 bytes at a time: word by word, lanes kPer words apart are kPer deep in a bank)
+            constexpr int kVec = kPer < 4 ? kPer : 4;
+            using Vec = std::conditional_t<kVec == 4, int4, int2>;
 #pragma unroll
-            for (int e = 0; e < kPer; ++e) { c[e] = h[hi - e]; sum += c[e]; }
+            for (int e = 0; e < kPer; e += kVec) {
+                const Vec v = *reinterpret_cast<const Vec *>(h + hi - e - (kVec - 1));
+                c[e + kVec - 1] = v.x; c[e + kVec - 2] = v.y;
+                if constexpr (kVec == 4) { c[e + 1] = v.z; c[e] = v.w; }
+            }
+#pragma unroll
+            for (int e = 0; e < kPer; ++e) sum += c[e];
         }
         int incl = sum;
 #pragma unroll

@@ -33,6 +33,34 @@ def test_select_against_oracle(L, B, kind):
     assert np.array_equal(e.cpu().numpy(), ref_e)
 
 
+@pytest.mark.parametrize("L,B", [(512, 60), (513, 60), (640, 64), (1001, 1000), (1024, 200)])
+@pytest.mark.parametrize("kind", ["spread", "ties", "equal", "window"])
+def test_many_heads_of_up_to_1024_positions(L, B, kind):
+    """More heads than four blocks per SM (blocks of 128 threads between 512 and 1024 positions), and, with the candidates laid out
+    by the same launch, the matches of the separate step."""
+    heads, W = 600, 32
+    gen = torch.Generator(device="cuda").manual_seed(L + B)
+    imp = torch.exp(torch.randn((1, heads, L), generator=gen, device="cuda") * 2)
+    if kind == "ties":
+        imp = (imp * 2).round() / 2
+    elif kind == "equal":
+        imp[:] = 0.125
+    p = O.OracleParams(1, heads, heads, 128, L, W, B, keep_window=int(kind == "window"), theta=0.3, tau=2.0, tau_mode=O.TAU_REL)
+    ref_r, ref_e = O.select(p, imp.cpu().numpy().astype(np.float64))
+    fp = gpu_params(p, F.BF16)
+    r = torch.full((1, heads, B), -9, dtype=torch.int32, device="cuda")
+    e = torch.full((1, heads, L - B), -9, dtype=torch.int32, device="cuda")
+    F.flowmm_select(fp, imp, r, e, F.alloc_workspace(fp))
+    assert np.array_equal(r.cpu().numpy(), ref_r)
+    assert np.array_equal(e.cpu().numpy(), ref_e)
+    q, k = (torch.randn((1, heads, n, 128), generator=gen, device="cuda").bfloat16() for n in (W, L))
+    m = (torch.arange(L, device="cuda") % 70 < 50).to(torch.uint8)[None]
+    out = F.compress_layer_alloc(fp, q, k, k, m)
+    match, sim = torch.full_like(out["match"], -9), torch.zeros_like(out["match_sim"])
+    F.flowmm_match(fp, k, out["importance"], m, out["retained"], out["evicted"], out["strategy"], match, sim, F.alloc_workspace(fp))
+    assert torch.equal(match, out["match"]) and torch.equal(sim, out["match_sim"])
+
+
 @pytest.mark.parametrize("L,B", [(6143, 600), (6144, 600), (6145, 601), (8192, 8000), (33792, 1690), (45249, 77)])
 @pytest.mark.parametrize("U", [1, 18, 20])
 @pytest.mark.parametrize("kind", ["spread", "ties"])
