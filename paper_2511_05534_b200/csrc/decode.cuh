@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(kCombineParts * D) decode_combine_kernel(const
     const int64_t step = (int64_t)A.G * (D + 2);
     const float *rec = A.part + (((int64_t)u * A.Hkv + h) * A.n_split * A.G + g) * (D + 2);
     predecessor_done();
+    successor_may_start();
     float mx = kNegBig;
     for (int sp = threadIdx.x; sp < A.n_split; sp += kCombineParts * D) mx = fmaxf(mx, rec[sp * step + D]);
 #pragma unroll

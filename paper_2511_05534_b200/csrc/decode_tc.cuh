@@ -103,6 +103,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     predecessor_done();
+    if (A.n_split == 1 || A.clustered) successor_may_start();        // (not the small blocks that join many ranges)
 
     const int uh = blockIdx.x, u = uh / A.Hkv, h = uh % A.Hkv, split = blockIdx.y;
     const int tiles_total = (A.N + kTile - 1) / kTile;

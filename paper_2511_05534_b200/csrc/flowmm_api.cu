@@ -519,6 +519,8 @@ flowmm_status run_select(const flowmm_params &p, const float *importance, int32_
     a.n_heads = p.n_units * p.n_kv_heads; a.L = p.seq_len; a.B = p.n_keep; a.W = p.window; a.keep_window = p.keep_window;
     a.chunk = p.seq_len <= kSelMaxChunk ? (p.seq_len + 31) / 32 * 32 : kSelMaxChunk;
     const SelectFlow no_flow = {};
+    // (few heads: 112 of 2176 tokens would be 2 % slower)
+    a.lets_in = prep && 3 * (a.n_heads + p.n_units) <= 2 * tc::sm_count();
     MatchPrepArgs g = {};
     g.Hkv = 1; g.modality = row_mod;
     if (prep) g = *prep;

@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(kPrepThreads) match_prepare_kernel(const Match
 // CTAs share a head's rows.  grid = (U*Hkv, ceil(Ctot / 64)), block = 256.
 __global__ void __launch_bounds__(256) match_gather_kernel(const MatchPrepArgs A) {
     predecessor_done();
+    successor_may_start();
     const int lo = blockIdx.y * 64;
     match_gather_rows<4>(A, blockIdx.x, nullptr, lo, min(A.Ctot, lo + 64), threadIdx.x, blockDim.x);
 }

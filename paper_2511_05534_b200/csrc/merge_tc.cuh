@@ -152,6 +152,7 @@ merge_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     predecessor_done();
+    successor_may_start();
     const int ctas = A.ctas, rank = ctas > 1 ? (int)(blockIdx.x % (unsigned)ctas) : 0;
     const int first_item = ctas > 1 ? (int)(blockIdx.x / (unsigned)ctas) : (int)blockIdx.x, item_step = ctas > 1 ? A.n_items : (int)gridDim.x;
     const int n_steps = (A.L + kTile - 1) / kTile, c_lo = n_steps * rank / ctas, n_chunk = n_steps * (rank + 1) / ctas;   // steps c_lo .. n_chunk - 1

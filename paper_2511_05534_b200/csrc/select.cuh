@@ -35,6 +35,7 @@ struct SelectArgs {
     int *retained, *evicted;     // [n_heads, B], [n_heads, L - B]
     uint8_t *row_mod_out;        // nullptr, or [n_heads, B]: the pivots' modalities (one modality map per head: P.Hkv == 1)
     int n_heads, L, B, W, keep_window;
+    int lets_in;                 // the successor may be set up beside this kernel
     int chunk;                   // positions handled at a time, a multiple of 32: the whole context if it fits in shared memory, or a CTA's part of it
 };
 
@@ -109,6 +110,7 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
     for (int i = tid; i < 2 * kSelBins / 4; i += kThreads) reinterpret_cast<int4 *>(hist)[i] = make_int4(0, 0, 0, 0);
     __syncthreads();
     predecessor_done();
+    if (A.lets_in) successor_may_start();
     if (head >= A.n_heads) {
         if (rank_c == 0) select_flow_block(F, head - A.n_heads, A.W, reinterpret_cast<float *>(hist));
         return;
