@@ -371,17 +371,17 @@ struct Skel {
         __syncwarp();
         if (c.lane == 0) tc::mbar_arrive(c.bar(kBarAccEmpty + h));
     }
+    // (n of them: first, first + step, ...; f(which of them, chunk, values))
     template <class F, class Done>
-    static __device__ __forceinline__ void for_each_chunk_q(const Ctx &c, int h, int colq, int n_chunks, F &&f, Done &&done) {
-        constexpr int kPer = NB / 128;
-        const int lo = kPer * colq, hi = min(n_chunks, lo + kPer);
-        if (hi <= lo) done();
-        for (int ch = lo; ch < hi; ++ch) {
+    static __device__ __forceinline__ void for_each_chunk_h(const Ctx &c, int h, int first, int step, int n, F &&f, Done &&done) {
+        if (n <= 0) done();
+#pragma unroll 1
+        for (int i = 0, ch = first; i < n; ++i, ch += step) {
             uint32_t a[32];
             tc::tmem_ld32(c.tmem_base + h * NB + ch * 32 + ((uint32_t)(c.quarter * 32) << 16), a);
             tc::tmem_ld_wait(a);
-            if (ch + 1 >= hi) done();
-            f(ch, a);
+            if (i + 1 >= n) done();
+            f(i, ch, a);
         }
     }
     // Meeting point of the two warps that share rows, with a vote: returns whether either warp has given up on a wait, so that both leave
