@@ -14,6 +14,7 @@
 #include "decode.cuh"
 #include "decode_tc.cuh"
 #include "flow_tc.cuh"
+#include "match_merge_tc.cuh"
 #include "match_small_tc.cuh"
 #include "merge_rows.cuh"
 #include "merge_tc.cuh"
@@ -759,6 +760,45 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
     return FLOWMM_OK;
 }
 
+// Whether the matching and the merge of a call go into one launch (match_merge_tc.cuh): heads that fill the GPU, few slots (see there).
+// With several heads to an SM up to three steps a head are too few to hide its ends (1024 heads of 300 tokens 81.5 us by two launches, 82.9
+// by one; of 384 the same), and a second round of few heads leaves SMs without any, where the matching alone spreads tiles (160 heads of
+// 1200 tokens 85.0, 85.6; 256 of 640 42.9, 39.7).
+bool use_match_merge(const flowmm_params &p) {
+    const int UH = p.n_units * p.n_kv_heads, sms = tc::sm_count();
+    if (!use_tc(p) || !merge_is_tc(p) || p.n_keep > mmt::kMaxSlots) return false;
+    if (UH <= sms) return 2 * UH > sms;
+    return p.seq_len > 3 * mmt::kTile && 5 * UH >= 6 * sms;
+}
+
+// Matching and merge behind a selection that has laid out the candidates.  match, match_sim: nullptr where nobody asks for them.
+flowmm_status run_match_merge(const flowmm_params &p, const Layout &y, const void *k, const void *v, const uint8_t *mod,
+                              const int32_t *strategy, int32_t *match, float *match_sim, void *k_out, void *v_out, void *ws, cudaStream_t st) {
+    const int UH = p.n_units * p.n_kv_heads;
+    CUtensorMap kmap, vmap, cand_map;
+    const uint64_t dims[4] = {128, (uint64_t)p.seq_len, (uint64_t)p.n_kv_heads, (uint64_t)p.n_units};
+    const uint64_t ksb[3] = {(uint64_t)p.k_stride[2] * 2, (uint64_t)p.k_stride[1] * 2, (uint64_t)p.k_stride[0] * 2};
+    const uint64_t vsb[3] = {(uint64_t)p.v_stride[2] * 2, (uint64_t)p.v_stride[1] * 2, (uint64_t)p.v_stride[0] * 2};
+    const uint64_t cd[4] = {128, (uint64_t)y.c_tot, (uint64_t)UH, 1};
+    const uint64_t cs[3] = {256, (uint64_t)y.c_tot * 256, (uint64_t)y.c_tot * 256 * (uint64_t)UH};
+    const uint32_t box[4] = {64, mmt::kTile, 1, 1}, box_c[4] = {64, (uint32_t)y.c_tot, 1, 1};
+    if (!tc::make_bf16_map(&kmap, k, 4, dims, ksb, box) || !tc::make_bf16_map(&vmap, v, 4, dims, vsb, box) ||
+        !tc::make_bf16_map(&cand_map, at<__nv_bfloat16>(ws, y.cand_k), 4, cd, cs, box_c))
+        return FLOWMM_ERR_CUDA;
+    mmt::Args a;
+    a.cand_count = at<int>(ws, y.cand_count); a.cand_slot = at<int>(ws, y.cand_slot); a.cand_scale = at<float>(ws, y.cand_scale);
+    a.rank = at<int>(ws, y.rank); a.strategy = strategy; a.modality = mod; a.match = match; a.match_sim = match_sim;
+    a.k_out = k_out; a.v_out = v_out; a.status = at<int>(ws, y.status);
+    a.Hkv = p.n_kv_heads; a.L = p.seq_len; a.E = p.seq_len - p.n_keep; a.B = p.n_keep; a.Ctot = y.c_tot; a.merge_mode = p.merge_mode;
+    a.n_items = UH; a.at = mmt::smem_plan(p.n_keep, y.c_tot);
+    for (int i = 0; i < 3; ++i) { a.kos[i] = p.ko_stride[i]; a.vos[i] = p.vo_stride[i]; }
+    if (cudaFuncSetAttribute(mmt::match_merge_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.at.total) != cudaSuccess)
+        return FLOWMM_ERR_CUDA;
+    launch(mmt::match_merge_tc_kernel, std::min(UH, tc::sm_count()), mmt::kThreads, a.at.total, st, kmap, vmap, cand_map, a);
+    FLOWMM_LAUNCHED("match_merge_tc");
+    return FLOWMM_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -862,6 +902,7 @@ flowmm_status flowmm_compress_layer(const flowmm_params *p, const void *q_win, c
     if (!strategy) strategy = at<int32_t>(ws, y.strategy);
     if (!retained_idx) retained_idx = at<int32_t>(ws, y.retained);
     if (!evicted_idx) evicted_idx = at<int32_t>(ws, y.evicted);
+    const bool matches_wanted = match || match_sim;
     if (!match) match = at<int32_t>(ws, y.match);
     if (!match_sim) match_sim = at<float>(ws, y.match_sim);
     float *cross_mass = at<float>(ws, y.cross_mass);
@@ -876,6 +917,8 @@ flowmm_status flowmm_compress_layer(const flowmm_params *p, const void *q_win, c
     flow.rho = rho; flow.strategy = strategy; flow.n_units = p->n_units; flow.Hq = p->n_q_heads;
     flow.theta = p->theta; flow.flow_mode = p->flow_mode;
     FLOWMM_TRY(run_select(*p, importance, retained_idx, evicted_idx, st, &flow, prep_in_select ? &prep : nullptr));
+    if (use_match_merge(*p))
+        return run_match_merge(*p, y, k, v, modality, strategy, matches_wanted ? match : nullptr, match_sim, k_out, v_out, ws, st);
     // when both the short-list matching kernel and the tensor-core merge apply, the former writes the latter's table
     const bool map_in_match = p->seq_len > p->n_keep && use_tc(*p) && y.c_tot <= mst::kMaxCols && merge_is_tc(*p);
     FLOWMM_TRY(run_match(*p, y, k, importance, modality, retained_idx, evicted_idx, strategy, match, match_sim, ws, st,
@@ -1314,6 +1357,7 @@ extern "C" flowmm_status flowmm_recompress(const flowmm_params *p, const void *q
     if (!strategy) strategy = at<int32_t>(ws, y.strategy);
     if (!retained_idx) retained_idx = at<int32_t>(ws, y.retained);
     if (!evicted_idx) evicted_idx = at<int32_t>(ws, y.evicted);
+    const bool matches_wanted = match || match_sim;
     if (!match) match = at<int32_t>(ws, y.match);
     if (!match_sim) match_sim = at<float>(ws, y.match_sim);
     float *cross_mass = at<float>(ws, y.cross_mass);             // [U * Hkv, G] = [U, Hq]
@@ -1330,6 +1374,9 @@ extern "C" flowmm_status flowmm_recompress(const flowmm_params *p, const void *q
     flow.n_rep = p->n_kv_heads; flow.theta = p->theta; flow.flow_mode = p->flow_mode;
     FLOWMM_TRY(run_select(ph, importance, retained_idx, evicted_idx, st, &flow, prep_in_select ? &prep : nullptr, row_modality,
                           row_modality_out));
+    if (use_match_merge(ph))
+        return run_match_merge(ph, y, k_cache, v_cache, row_modality, strategy_h, matches_wanted ? match : nullptr, match_sim, k_out, v_out,
+                               ws, st);
     const bool map_in_match = prep_in_select && y.c_tot <= mst::kMaxCols && merge_is_tc(ph);
     FLOWMM_TRY(run_match(ph, y, k_cache, importance, row_modality, retained_idx, evicted_idx, strategy_h, match, match_sim, ws, st,
                          map_in_match ? at<int2>(ws, y.tokmap) : nullptr, prep_in_select));

@@ -57,6 +57,88 @@ __device__ __forceinline__ void pair_sync(int pair, int wq) { asm volatile("bar.
 // group of 8 columns is; the 8 values are in the thread's stash.
 struct Winner { float best; int col; };
 
+// The winner of a thread's token among the candidate columns of a unit: its similarity (still times the row's norm) and pivot slot
+// (-1: none).  trow: TMEM address of the unit's columns for the warp's lanes; md, slot_off: the head's scales in shared memory and how
+// far behind them its slots are; wrow: the thread's stash; blocks of 16 columns, numbered from the head's first column: the unit's first
+// one blk0, the text group's [blk0, tb) and the visual group's [vb, ve).  Call with the whole warp; release() as soon as the
+// accumulator has been read (whatever the waits returned: !ok).
+template <class Release>
+__device__ __forceinline__ void match_unit(uint32_t trow, uint32_t md, uint32_t slot_off, uint32_t wrow, int blk0, int tb, int vb, int ve,
+                                           bool want_text, bool want_vis, int N, bool ok, int *status, float &best, int &slot,
+                                           Release &&release) {
+    // Candidates are laid out text group first, each group by ascending slot, so the first maximum of a group is
+    // its lowest slot; the groups' winners meet by (similarity, slot), so that equal similarities go to the lower.
+    auto slot_of = [&](const Winner &w) -> int {         // lowest column of the winning 8 that holds the maximum
+        if (w.col < 0) return -1;
+        int idx = 0;
+#pragma unroll
+        for (int q4 = 1; q4 >= 0; --q4) {
+            const float4 v = tc::lds128(wrow + q4 * 16);
+            if (v.w == w.best) idx = 4 * q4 + 3;
+            if (v.z == w.best) idx = 4 * q4 + 2;
+            if (v.y == w.best) idx = 4 * q4 + 1;
+            if (v.x == w.best) idx = 4 * q4;
+        }
+        return index_ok(w.col + idx, N, status) ? __float_as_int(tc::lds32(md + slot_off + (w.col + idx) * 4)) : -1;
+    };
+    auto block = [&](int blk, const uint32_t *acc, bool want, Winner &w) {
+        float v[16];
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) {                 // a column that is no candidate has scale NaN and never wins
+            const float4 s4 = tc::lds128(md + (blk * 4 + q4) * 16);
+            v[4 * q4 + 0] = __uint_as_float(acc[4 * q4 + 0]) * s4.x;
+            v[4 * q4 + 1] = __uint_as_float(acc[4 * q4 + 1]) * s4.y;
+            v[4 * q4 + 2] = __uint_as_float(acc[4 * q4 + 2]) * s4.z;
+            v[4 * q4 + 3] = __uint_as_float(acc[4 * q4 + 3]) * s4.w;
+        }
+#pragma unroll
+        for (int h8 = 0; h8 < 2; ++h8) {                 // two groups of 8 columns, in column order
+            const float q8 = tc::max3(tc::max3(v[8 * h8], v[8 * h8 + 1], v[8 * h8 + 2]),
+                                      tc::max3(v[8 * h8 + 3], v[8 * h8 + 4], v[8 * h8 + 5]), fmaxf(v[8 * h8 + 6], v[8 * h8 + 7]));
+            if (want && q8 > w.best) {                   // strict: an earlier group keeps a tie (false for NaN)
+                w.best = q8;
+                w.col = blk * 16 + 8 * h8;
+                tc::sts128(wrow, v[8 * h8], v[8 * h8 + 1], v[8 * h8 + 2], v[8 * h8 + 3]);
+                tc::sts128(wrow + 16, v[8 * h8 + 4], v[8 * h8 + 5], v[8 * h8 + 6], v[8 * h8 + 7]);
+            }
+        }
+    };
+    auto walk = [&](int lo, int hi, bool want) -> Winner {    // blocks [lo, hi); pairs of blocks per read
+        Winner w = {-INFINITY, -1};
+        if (!__any_sync(0xFFFFFFFFu, want)) return w;
+        int blk = lo;
+#pragma unroll 1
+        for (; blk + 1 < hi; blk += 2) {
+            uint32_t acc[32];
+            tc::tmem_ld32(trow + (blk - blk0) * 16, acc);
+            tc::tmem_ld_wait(acc);
+            block(blk, acc, want, w);
+            block(blk + 1, acc + 16, want, w);
+        }
+        if (blk < hi) {
+            uint32_t acc[16];
+            tc::tmem_ld16(trow + (blk - blk0) * 16, acc);
+            tc::tmem_ld_wait(acc);
+            block(blk, acc, want, w);
+        }
+        return w;
+    };
+    best = -INFINITY;
+    slot = -1;
+    Winner wv = {-INFINITY, -1};
+    if (ok) {
+        const Winner wt = walk(blk0, tb, want_text);
+        best = wt.best;
+        slot = slot_of(wt);
+        wv = walk(vb, ve, want_vis);
+    }
+    release();
+    if (ok) {
+        const int slot_v = slot_of(wv);
+        if (match_better(wv.best, slot_v, best, slot)) { best = wv.best; slot = slot_v; }
+    }
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
 match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap cand_map, const Args A) {
     extern __shared__ __align__(1024) uint8_t mst_smem[];
@@ -234,79 +316,13 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
                 }
                 ok = ok && tc::mbar_wait_warp(bar(kBarAccFull + team), (k / kTeams) & 1, abort_flag, A.status);
                 tc::tc_fence_after();
-                // Candidates are laid out text group first, each group by ascending slot, so the first maximum of a group is
-                // its lowest slot; the groups' winners meet by (similarity, slot), so that equal similarities go to the lower.
-                auto slot_of = [&](const Winner &w) -> int {         // lowest column of the winning 8 that holds the maximum
-                    if (w.col < 0) return -1;
-                    int idx = 0;
-#pragma unroll
-                    for (int q4 = 1; q4 >= 0; --q4) {
-                        const float4 v = tc::lds128(wrow + q4 * 16);
-                        if (v.w == w.best) idx = 4 * q4 + 3;
-                        if (v.z == w.best) idx = 4 * q4 + 2;
-                        if (v.y == w.best) idx = 4 * q4 + 1;
-                        if (v.x == w.best) idx = 4 * q4;
-                    }
-                    return index_ok(w.col + idx, N, A.status) ? __float_as_int(tc::lds32(md + slot_off + (w.col + idx) * 4)) : -1;
-                };
-                auto block = [&](int blk, const uint32_t *acc, bool want, Winner &w) {
-                    float v[16];
-#pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {                 // a column that is no candidate has scale NaN and never wins
-                        const float4 s4 = tc::lds128(md + (blk * 4 + q4) * 16);
-                        v[4 * q4 + 0] = __uint_as_float(acc[4 * q4 + 0]) * s4.x;
-                        v[4 * q4 + 1] = __uint_as_float(acc[4 * q4 + 1]) * s4.y;
-                        v[4 * q4 + 2] = __uint_as_float(acc[4 * q4 + 2]) * s4.z;
-                        v[4 * q4 + 3] = __uint_as_float(acc[4 * q4 + 3]) * s4.w;
-                    }
-#pragma unroll
-                    for (int h8 = 0; h8 < 2; ++h8) {                 // two groups of 8 columns, in column order
-                        const float q8 = tc::max3(tc::max3(v[8 * h8], v[8 * h8 + 1], v[8 * h8 + 2]),
-                                                  tc::max3(v[8 * h8 + 3], v[8 * h8 + 4], v[8 * h8 + 5]), fmaxf(v[8 * h8 + 6], v[8 * h8 + 7]));
-                        if (want && q8 > w.best) {                   // strict: an earlier group keeps a tie (false for NaN)
-                            w.best = q8;
-                            w.col = blk * 16 + 8 * h8;
-                            tc::sts128(wrow, v[8 * h8], v[8 * h8 + 1], v[8 * h8 + 2], v[8 * h8 + 3]);
-                            tc::sts128(wrow + 16, v[8 * h8 + 4], v[8 * h8 + 5], v[8 * h8 + 6], v[8 * h8 + 7]);
-                        }
-                    }
-                };
-                auto walk = [&](int lo, int hi, bool want) -> Winner {    // blocks [lo, hi); pairs of blocks per read
-                    Winner w = {-INFINITY, -1};
-                    if (!__any_sync(0xFFFFFFFFu, want)) return w;
-                    int blk = lo;
-#pragma unroll 1
-                    for (; blk + 1 < hi; blk += 2) {
-                        uint32_t acc[32];
-                        tc::tmem_ld32(trow + (blk - blk0) * 16, acc);
-                        tc::tmem_ld_wait(acc);
-                        block(blk, acc, want, w);
-                        block(blk + 1, acc + 16, want, w);
-                    }
-                    if (blk < hi) {
-                        uint32_t acc[16];
-                        tc::tmem_ld16(trow + (blk - blk0) * 16, acc);
-                        tc::tmem_ld_wait(acc);
-                        block(blk, acc, want, w);
-                    }
-                    return w;
-                };
-                float best = -INFINITY;
-                int slot = -1;
-                Winner wv = {-INFINITY, -1};
-                if (ok) {
-                    const Winner wt = walk(blk0, tb, want_text);
-                    best = wt.best;
-                    slot = slot_of(wt);
-                    wv = walk(vb, ve, want_vis);
-                }
-                tc::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(bar(kBarSetFree + team));   // this warp has read the accumulator
-                if (ok) {
-                    const int slot_v = slot_of(wv);
-                    if (match_better(wv.best, slot_v, best, slot)) { best = wv.best; slot = slot_v; }
-                }
+                float best;
+                int slot;
+                match_unit(trow, md, slot_off, wrow, blk0, tb, vb, ve, want_text, want_vis, N, ok, A.status, best, slot, [&]() {
+                    tc::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(bar(kBarSetFree + team));   // this warp has read the accumulator
+                });
                 if (units == 2) {
                     // the upper unit hands its result and its half of the norm to the lower one, which owns the row's output;
                     // (kept also after a wait that ran out, so that the partner warp is never left waiting)
