@@ -49,38 +49,61 @@ __device__ __forceinline__ uint32_t digit_peers(int digit, bool valid) {
     return mine;
 }
 
-// What the merge kernel needs beside the members' rows: the pivots' rows, the windows' first slots, the pieces of long slots.
+// What the merge kernel needs beside the members' rows: the pivots' rows and the windows' first slots, of the slots [s_lo, s_hi) ...
 // off[s] = first member of slot s (s <= B).
 template <int kThreads>
-__device__ __forceinline__ void csr_write_slots(const CsrArgs &A, int uh, const int *off, int *scratch) {
-    const int tid = threadIdx.x;
+__device__ __forceinline__ void csr_write_pivots(const CsrArgs &A, int uh, const int *off, int s_lo, int s_hi) {
     const int *ret = A.retained + (int64_t)uh * A.B;
     int2 *rows = A.rows + (int64_t)uh * (A.B + A.E);
     int *first_slot = A.first_slot + (int64_t)uh * A.n_win;
+    for (int s = s_lo + threadIdx.x; s < s_hi; s += kThreads) {
+        const int row = off[s] + s;
+        rows[row] = make_int2(ret[s] | kRowPivot | (off[s + 1] - off[s] > kPiece ? kRowLong : 0), 0);
+        for (int w = s == 0 ? 0 : (off[s - 1] + s - 1) / A.win + 1; w <= row / A.win; ++w) first_slot[w] = s;
+        A.slot_done[(int64_t)uh * A.B + s] = 0;
+    }
+}
+// ... and the head's pieces of long slots.
+template <int kThreads>
+__device__ __forceinline__ void csr_write_pieces(const CsrArgs &A, int uh, const int *off, int *scratch) {
+    const int tid = threadIdx.x;
     int *part_off = A.part_off + (int64_t)uh * (A.B + 1);
     int4 *pieces = A.pieces + (int64_t)uh * A.max_parts;
-    int seen = 0;
+    int longest = 0, seen = 0;
+    for (int s = tid; s < A.B; s += kThreads) longest = max(longest, off[s + 1] - off[s]);
+    const bool any = __syncthreads_or(longest > kPiece);             // (mostly none: then there is nothing to add up)
     for (int base = 0; base <= A.B; base += kThreads) {
         const int s = base + tid;
-        int n = 0, np = 0;
+        int n = 0, np = 0, total = 0, part = 0;
         if (s < A.B) {
             n = off[s + 1] - off[s];
             np = n > kPiece ? (n + kPiece - 1) / kPiece : 0;
         }
-        int total;
-        const int part = seen + block_exclusive_scan(np, scratch, total);
+        if (any) part = seen + block_exclusive_scan(np, scratch, total);
         if (s <= A.B) part_off[s] = part;
-        if (s < A.B) {
-            const int row = off[s] + s;
-            rows[row] = make_int2(ret[s] | kRowPivot | (np ? kRowLong : 0), 0);
-            for (int w = s == 0 ? 0 : (off[s - 1] + s - 1) / A.win + 1; w <= row / A.win; ++w) first_slot[w] = s;
-            for (int q = 0; q < np; ++q) pieces[part + q] = make_int4(s, row + 1 + q * kPiece, min(kPiece, n - q * kPiece), part + q);
-            A.slot_done[(int64_t)uh * A.B + s] = 0;
-        }
+        for (int q = 0; q < np; ++q) pieces[part + q] = make_int4(s, off[s] + s + 1 + q * kPiece, min(kPiece, n - q * kPiece), part + q);
         seen += total;
     }
     if (tid == 0) A.row_count[uh] = make_int2(off[A.B] + A.B, seen);
     if (uh == 0 && tid == 0) *A.ticket = 0u;
+}
+template <int kThreads>
+__device__ __forceinline__ void csr_write_slots(const CsrArgs &A, int uh, const int *off, int *scratch) {
+    csr_write_pivots<kThreads>(A, uh, off, 0, A.B);
+    csr_write_pieces<kThreads>(A, uh, off, scratch);
+}
+
+// n words from global to shared memory, eight per thread on their way together.
+template <int kThreads, typename T>
+__device__ __forceinline__ void copy_batched(T *dst, const T *src, int n) {
+    for (int i = threadIdx.x; i < n; i += 8 * kThreads) {
+        T v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = i + e * kThreads < n ? src[i + e * kThreads] : T(0);
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (i + e * kThreads < n) dst[i + e * kThreads] = v[e];
+    }
 }
 
 // grid = U*Hkv, block = 32 * NW threads (warp w owns a contiguous range of the input).  n_pass passes of kCsrBits bits.
@@ -304,7 +327,7 @@ __global__ void __launch_bounds__(32 * NW) build_csr_count_kernel(const CsrArgs 
         __syncthreads();
         const int n_rows = off[B] + B;
         int *stage = reinterpret_cast<int *>(region);
-        for (int i = tid; i < E; i += kThreads) stage[i] = evi[i];
+        copy_batched<kThreads>(stage, evi, E);
         __syncthreads();
         for (int i = tid; i < n_rows; i += kThreads) {
             const int j = sorted[i];
@@ -313,7 +336,7 @@ __global__ void __launch_bounds__(32 * NW) build_csr_count_kernel(const CsrArgs 
         float *stage_f = reinterpret_cast<float *>(region);
         if (A.merge_mode != 1) {
             __syncthreads();
-            for (int i = tid; i < E; i += kThreads) stage_f[i] = sim[i];
+            copy_batched<kThreads>(stage_f, sim, E);
             __syncthreads();
         }
         for (int i = tid; i < n_rows; i += kThreads) {
@@ -327,9 +350,11 @@ __global__ void __launch_bounds__(32 * NW) build_csr_count_kernel(const CsrArgs 
 // The counting sort with a head's positions shared among the CTAs of a cluster, for calls whose heads do not fill the GPU.
 // As above, but every CTA counts its part of the positions, reads the other CTAs' totals per slot out of their shared
 // memory, and writes its members' token positions and weights straight to their places (8 heads of 32 102 positions:
-// 59 -> 22 us).
+// 59 -> 22 us).  Bound by its chain of loads: where a warp's positions are one batch, all that is needed of them is fetched at the
+// start, the other CTAs' totals are read together, and every CTA writes its share of the slots (the whole call: 8 heads of 33 792 tokens
+// 231 -> 227 us, of 12 000 102.3 -> 101.1, 4 of 10 800 with 2160 pivots 88.6 -> 85.6).
 // grid = (U*Hkv * ctas), cluster = ctas along x.  Dynamic shared memory: csr_cluster_smem().
-constexpr int kCsrClusterWarps = 16;
+constexpr int kCsrClusterWarps = 16, kMaxCsrCtas = 8;
 __host__ __device__ constexpr size_t csr_cluster_smem(int B) {
     const size_t pitch = ((size_t)B + 2) & ~(size_t)1;
     return kCsrClusterWarps * pitch * 2 + pitch * 2 + 2 * pitch * 4 + 16;
@@ -349,13 +374,25 @@ __global__ void __launch_bounds__(32 * kCsrClusterWarps) build_csr_cluster_kerne
     for (int i = tid; i < NW * pitch / 2; i += kThreads) words[i] = 0u;
     __syncthreads();
     predecessor_done();
-    const int *match = A.match + (int64_t)uh * E;
+    const int *match = A.match + (int64_t)uh * E, *evi = A.evicted + (int64_t)uh * E;
+    const float *sim = A.match_sim + (int64_t)uh * E;
     const int per_warp = ((E + ctas * NW - 1) / (ctas * NW) + 31) / 32 * 32;
     const int lo = min(E, (rank * NW + warp) * per_warp), hi = min(E, lo + per_warp);
-    for (int t0 = lo; t0 < hi; t0 += 32 * kBatch) {
-        int key[kBatch];
+    // a batch of the warp's positions (key -1: no such position); what its rows need comes along
+    auto fetch = [&](int t0, int (&key)[kBatch], int (&tok)[kBatch], float (&w)[kBatch], bool rows_too) {
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b) key[b] = t0 + 32 * b + lane < hi ? csr_key(match[t0 + 32 * b + lane], B) : -1;
+        for (int b = 0; b < kBatch; ++b) {
+            const int j = t0 + 32 * b + lane;
+            key[b] = j < hi ? csr_key(match[j], B) : -1;
+            tok[b] = rows_too && j < hi ? evi[j] : 0;
+            w[b] = rows_too && j < hi ? sim[j] : 0.f;
+        }
+    };
+    const bool one = per_warp <= 32 * kBatch;                                        // the first batch is the only one, and stays in registers
+    int key[kBatch], tok[kBatch];
+    float w[kBatch];
+    for (int t0 = lo; t0 < hi || t0 == lo; t0 += 32 * kBatch) {
+        fetch(t0, key, tok, w, one);
 #pragma unroll
         for (int b = 0; b < kBatch; ++b)
             if (key[b] >= 0) atomicAdd(reinterpret_cast<uint32_t *>(cnt) + (key[b] >> 1), (key[b] & 1) ? 0x10000u : 1u);
@@ -364,9 +401,9 @@ __global__ void __launch_bounds__(32 * kCsrClusterWarps) build_csr_cluster_kerne
     for (int i = tid; i < pitch / 2; i += kThreads) {                                // two slots at a time, no carry between them: E < 65536
         uint32_t run = 0;
 #pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const uint32_t x = words[w * (pitch / 2) + i];
-            words[w * (pitch / 2) + i] = run;
+        for (int q = 0; q < NW; ++q) {
+            const uint32_t x = words[q * (pitch / 2) + i];
+            words[q * (pitch / 2) + i] = run;
             run += x;
         }
         totals[i] = run;
@@ -375,12 +412,14 @@ __global__ void __launch_bounds__(32 * kCsrClusterWarps) build_csr_cluster_kerne
     const uint32_t totals_at = (uint32_t)__cvta_generic_to_shared(totals);
     for (int i0 = 0, seen = 0; i0 < pitch / 2; i0 += kThreads) {
         const int i = i0 + tid;
-        uint32_t all = 0, before = 0;
-        if (i < pitch / 2)
-            for (int r = 0; r < ctas; ++r) {
-                if (r == rank) before = all;
-                all += ld_cluster_u32(totals_at + 4 * i, r);
-            }
+        uint32_t part[kMaxCsrCtas], all = 0, before = 0;
+#pragma unroll
+        for (int r = 0; r < kMaxCsrCtas; ++r) part[r] = r < ctas && i < pitch / 2 ? ld_cluster_u32(totals_at + 4 * i, r) : 0u;   // (on their way together)
+#pragma unroll
+        for (int r = 0; r < kMaxCsrCtas; ++r) {
+            before = r == rank ? all : before;
+            all += part[r];
+        }
         int total;
         const int first = seen + block_exclusive_scan((int)(all & 0xFFFFu) + (int)(all >> 16), scratch, total);
         const int second = first + (int)(all & 0xFFFFu);
@@ -390,19 +429,9 @@ __global__ void __launch_bounds__(32 * kCsrClusterWarps) build_csr_cluster_kerne
     }
     __syncthreads();
     cluster_arrive();                                                                // the other CTAs' totals have been read
-    const int *evi = A.evicted + (int64_t)uh * E;
-    const float *sim = A.match_sim + (int64_t)uh * E;
     int2 *rows = A.rows + (int64_t)uh * (B + E);
     for (int t0 = lo; t0 < hi; t0 += 32 * kBatch) {
-        int key[kBatch], tok[kBatch];
-        float w[kBatch];
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            const int j = t0 + 32 * b + lane;
-            key[b] = j < hi ? csr_key(match[j], B) : -1;
-            tok[b] = j < hi ? evi[j] : 0;
-            w[b] = j < hi ? sim[j] : 0.f;
-        }
+        if (!one) fetch(t0, key, tok, w, true);
 #pragma unroll
         for (int b = 0; b < kBatch; ++b) {
             const bool valid = key[b] >= 0;
@@ -421,7 +450,9 @@ __global__ void __launch_bounds__(32 * kCsrClusterWarps) build_csr_cluster_kerne
             __syncwarp();
         }
     }
-    if (rank == ctas - 1) csr_write_slots<kThreads>(A, uh, off, scratch);           // (the last CTA has the fewest positions)
+    // the slots in even shares, the pieces by the last CTA, which has the fewest positions
+    csr_write_pivots<kThreads>(A, uh, off, B * rank / ctas, B * (rank + 1) / ctas);
+    if (rank == ctas - 1) csr_write_pieces<kThreads>(A, uh, off, scratch);
     __syncwarp();
     cluster_wait();                                                                  // nobody's totals go away while they are read
 }
