@@ -1162,7 +1162,7 @@ struct DecodePlan {
     size_t part_off, bytes;
 };
 
-constexpr int kMaxDecodeCluster = 8;         // ranges of a head that are joined as one cluster (the portable cluster size)
+constexpr int kMaxDecodeCluster = dtc::kMaxRanges;         // ranges of a head that are joined as one cluster (the portable cluster size)
 
 DecodePlan decode_plan(const flowmm_decode_params &p) {
     DecodePlan d;
