@@ -128,7 +128,8 @@ int chunks_for(int L, int other_ctas, int &chunk) {
 // 1.3 million 154, 156; 1.6 million 165, 164; 2.5 million 257, 248; 4.3 million 422, 392 (fp32 rows of 64 within 1 %, equal from 0.8 million on).
 // While every warp has one window at most, the windows are as short as leaves it so, by groups of four rows (other lengths misalign the
 // reads of the list: 64 heads of 1688 rows by 31 were 1.3 % slower): 112 caches of 640 rows by 24 instead of 32 80.7 -> 78.8 us for the call,
-// 16 heads of 3972 by 20 75.4 -> 72.9.  (Equal numbers of longer windows, 39 rows for 270 000, 232 -> 243.)
+// 16 heads of 3972 by 20 75.4 -> 72.9.  Windows shorter than two slots would often be empty: 4 heads of 10 822 rows with 542 slots by 16
+// instead of 32 81.8 -> 85.2.  (Equal numbers of longer windows, 39 rows for 270 000, 232 -> 243.)
 constexpr int64_t kManyRows = 1300000;
 constexpr int kMinWin = 16, kMergeCtas = 3 * kScoreCtas;
 int merge_window(const flowmm_params &p) {
@@ -136,7 +137,7 @@ int merge_window(const flowmm_params &p) {
     if (rows >= kManyRows) return mrow::kMaxWin;
     if (rows < 40000) return kMinWin;
     int win = kMinWin;
-    while (win < 32 && heads * ((p.seq_len + win - 1) / win) > kMergeCtas * mrow::kWarps) win += 4;
+    while (win < 32 && (win * (int64_t)p.n_keep < 2 * (int64_t)p.seq_len || heads * ((p.seq_len + win - 1) / win) > kMergeCtas * mrow::kWarps)) win += 4;
     return win;
 }
 
@@ -520,8 +521,9 @@ flowmm_status run_select(const flowmm_params &p, const float *importance, int32_
     a.n_heads = p.n_units * p.n_kv_heads; a.L = p.seq_len; a.B = p.n_keep; a.W = p.window; a.keep_window = p.keep_window;
     a.chunk = p.seq_len <= kSelMaxChunk ? (p.seq_len + 31) / 32 * 32 : kSelMaxChunk;
     const SelectFlow no_flow = {};
-    // (few heads: 112 of 2176 tokens would be 2 % slower)
-    a.lets_in = prep && 3 * (a.n_heads + p.n_units) <= 2 * tc::sm_count();
+    // (few heads, 112 of 2176 tokens would be 2 % slower, and one block per SM behind them, not the small blocks that gather long candidate
+    // lists)
+    a.lets_in = prep && prep->copy_here && 3 * (a.n_heads + p.n_units) <= 2 * tc::sm_count();
     MatchPrepArgs g = {};
     g.Hkv = 1; g.modality = row_mod;
     if (prep) g = *prep;
