@@ -108,38 +108,66 @@ __device__ __forceinline__ void match_gather_rows(const MatchPrepArgs &A, int uh
     }
 }
 
-// The candidate layout of one head from its pivot list, by a whole block (`scratch`: 33 ints of shared memory).
+// The candidate layout of one head from its pivot list, by a whole block (`scratch`: 33 ints of shared memory).  A thread takes eight
+// pivots in a row, whose loads are on their way together; one prefix sum numbers the candidates of both groups.  (The steps one by one,
+// 8 heads of 33 792 tokens with 1690 pivots: 235.8 -> 228.6 us, where rounds of a pivot per thread loaded twice and summed each time.)
 __device__ __forceinline__ void match_lay_out_candidates(const MatchPrepArgs &A, int uh, int *scratch) {
-    const int tid = threadIdx.x, u = uh / A.Hkv;
+    constexpr int kPer = 8;
+    const int tid = threadIdx.x, u = uh / A.Hkv, chunk = kPer * blockDim.x;
     const int *ret = A.retained + (int64_t)uh * A.B;
     const float *imp = A.importance + (int64_t)uh * A.L;
     const uint8_t *mod = A.modality + (int64_t)u * A.L;
     int *slot_out = A.cand_slot + (int64_t)uh * A.Ctot;
     float *scale_out = A.cand_scale + (int64_t)uh * A.Ctot;
     for (int i = tid; i < A.Ctot; i += blockDim.x) { slot_out[i] = -1; scale_out[i] = __int_as_float(0x7FC00000); }   // NaN: no candidate here
-    // admissible text pivots first: count them to know where the visual group starts
-    int n_text = 0;
-    for (int s = tid; s < A.B; s += blockDim.x) {
-        const int r = index_ok(ret[s], A.L, A.status) ? ret[s] : 0;
-        n_text += (imp[r] <= A.tau_eff && mod[r] == 0) ? 1 : 0;
-    }
-    int total;
-    block_exclusive_scan(n_text, scratch, total);
-    const int t0 = (total + 31) & ~31;
-    int seen_t = 0, seen_v = 0;
-    for (int base = 0; base < A.B; base += blockDim.x) {
-        const int s = base + tid;
-        int ft = 0, fv = 0, r = 0;
-        if (s < A.B) {
-            r = index_ok(ret[s], A.L, A.status) ? ret[s] : 0;
-            const bool adm = imp[r] <= A.tau_eff;              // Eq. 10: pivots above tau are kept out of merging
-            ft = adm && mod[r] == 0;
-            fv = adm && mod[r] != 0;
+    // which of the thread's pivots are admissible text ones, which visual ones
+    uint32_t text = 0, vis = 0;
+    auto look = [&](int base) {
+        int r[kPer];
+        float v[kPer];
+        uint8_t m[kPer];
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            const int s = base + tid * kPer + e;
+            r[e] = s < A.B ? ret[s] : -1;
+            if (r[e] >= 0 && !index_ok(r[e], A.L, A.status)) r[e] = 0;
         }
-        int tot;                                               // (both counts in one scan: text in the low half, at most 1024 each)
-        const int both = block_exclusive_scan(ft | fv << 16, scratch, tot);
-        if (ft) slot_out[seen_t + (both & 0xFFFF)] = s;
-        if (fv) slot_out[t0 + seen_v + (both >> 16)] = s;
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            v[e] = r[e] >= 0 ? imp[r[e]] : 0.f;
+            m[e] = r[e] >= 0 ? mod[r[e]] : 0;
+        }
+        text = vis = 0;
+#pragma unroll
+        for (int e = 0; e < kPer; ++e)
+            if (r[e] >= 0 && v[e] <= A.tau_eff) {              // Eq. 10: pivots above tau are kept out of merging
+                if (m[e] == 0) text |= 1u << e;
+                else vis |= 1u << e;
+            }
+    };
+    // the text group comes first: where it ends is needed before the visual group is written
+    int n_text = 0, seen_t = 0, seen_v = 0;
+    if (A.B > chunk) {
+        for (int base = 0; base < A.B; base += chunk) {
+            look(base);
+            n_text += __popc(text);
+        }
+        int total;
+        block_exclusive_scan(n_text, scratch, total);
+        n_text = total;
+    }
+    for (int base = 0; base < A.B; base += chunk) {
+        look(base);
+        int tot;                                               // (both counts in one sum: text in the low half, a chunk's at most)
+        const int both = block_exclusive_scan(__popc(text) | __popc(vis) << 16, scratch, tot);
+        if (A.B <= chunk) n_text = tot & 0xFFFF;
+        int pt = seen_t + (both & 0xFFFF), pv = ((n_text + 31) & ~31) + seen_v + (both >> 16);
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            const int s = base + tid * kPer + e;
+            if (text >> e & 1u) slot_out[pt++] = s;
+            if (vis >> e & 1u) slot_out[pv++] = s;
+        }
         seen_t += tot & 0xFFFF;
         seen_v += tot >> 16;
     }
