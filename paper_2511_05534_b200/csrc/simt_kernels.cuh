@@ -17,21 +17,23 @@ struct SimtTiles {
     float norm_a[kTile], norm_b[kTile];      // kNorms: reciprocal norms of the tile's rows (0 for a zero row)
 };
 
-// acc[i][j] = sum_d A[ty*4+i][d] * B[tx*4+j][d] for a 64x64 tile; rowA(r) / rowB(r) give the
+// acc[i][j] = sum_d A[ty*kR+i][d] * B[tx*4+j][d] for a tile of 16 kR x 64, kR = 4 or 1; rowA(r) / rowB(r) give the
 // address of tile row r (nullptr: a row of zeros).  All 256 threads of the CTA take part.
 // Small calls wait for their loads more than they compute: a slice of the head dimension is fetched while the one before it
 // is multiplied, and with kNorms the threads that bring the rows in take their norms on the way (left in sm.norm_a / norm_b
 // at the function's end, behind a barrier).
-template <typename T, bool kNorms = false, typename FA, typename FB>
-__device__ __forceinline__ void simt_tile_dot(SimtTiles &sm, int D, FA rowA, FB rowB, float (&acc)[4][4]) {
+template <typename T, bool kNorms = false, int kR, typename FA, typename FB>
+__device__ __forceinline__ void simt_tile_dot(SimtTiles &sm, int D, FA rowA, FB rowB, float (&acc)[kR][4]) {
+    static_assert(kR == 4 || kR == 1, "a thread's rows are read 16 bytes at a time, or it has one");
     constexpr int V = Elem<T>::kVec;
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < kR; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
     const int lr = tid >> 2, ld = (tid & 3) * V;       // this thread loads 8 elements of row lr, 16 bytes at a time
-    const T *pa = rowA(lr);
+    const bool has_a = lr < 16 * kR;
+    const T *pa = has_a ? rowA(lr) : nullptr;
     const T *pb = rowB(lr);
     float va[8 / V][V], vb[8 / V][V], na = 0.f, nb = 0.f;
     auto fetch = [&](int d0) {
@@ -50,7 +52,7 @@ __device__ __forceinline__ void simt_tile_dot(SimtTiles &sm, int D, FA rowA, FB 
         for (int half = 0; half < 8 / V; ++half) {
 #pragma unroll
             for (int e = 0; e < V; ++e) {
-                sm.a[ld + half * 4 * V + e][lr] = va[half][e];
+                if (has_a) sm.a[ld + half * 4 * V + e][lr] = va[half][e];
                 sm.b[ld + half * 4 * V + e][lr] = vb[half][e];
                 if (kNorms) {
                     na = fmaf(va[half][e], va[half][e], na);
@@ -62,12 +64,15 @@ __device__ __forceinline__ void simt_tile_dot(SimtTiles &sm, int D, FA rowA, FB 
         if (d0 + kDChunk < D) fetch(d0 + kDChunk);
 #pragma unroll 8
         for (int d = 0; d < kDChunk; ++d) {
-            const float4 a4 = *reinterpret_cast<const float4 *>(&sm.a[d][ty * 4]);
+            float a[kR];
+            if constexpr (kR == 4) {
+                const float4 a4 = *reinterpret_cast<const float4 *>(&sm.a[d][ty * 4]);
+                a[0] = a4.x; a[1] = a4.y; a[2] = a4.z; a[3] = a4.w;
+            } else a[0] = sm.a[d][ty];
             const float4 b4 = *reinterpret_cast<const float4 *>(&sm.b[d][tx * 4]);
-            const float a[4] = {a4.x, a4.y, a4.z, a4.w};
             const float b[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < kR; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
@@ -272,8 +277,10 @@ __global__ void __launch_bounds__(kSimtThreads) score_colsum_simt(const ScoreArg
 // shared memory and go on with the probabilities.  grid = (U*Hkv * ctas), cluster = ctas <= 8, kTiles key tiles per CTA.
 // Bound by latency: against two launches that compute the logits twice, 4 heads of 192 tokens 29.8 -> 23.2 us for the call, 8 of
 // 950 46.6 -> 43.0.
+// With up to 16 proxy rows a thread has one row (kR = 1), as tiles of 64 would be zeros for three quarters: with the same in the matching, 4
+// heads of 192 tokens 21.5 -> 17.9 us for the call, of 1000 59.4 -> 56.2.
 constexpr int kClusterScoreTiles = 16;
-template <typename T, int kTiles>
+template <typename T, int kTiles, int kR>
 __global__ void __launch_bounds__(kSimtThreads) score_cluster_simt(const ScoreArgs A, int ctas) {
     __shared__ SimtTiles sm;
     __shared__ float colpart[16][kTile];
@@ -286,13 +293,13 @@ __global__ void __launch_bounds__(kSimtThreads) score_cluster_simt(const ScoreAr
     const T *k = static_cast<const T *>(A.k) + u * A.ks[0] + h * A.ks[1];
     const uint8_t *mod = A.modality + (int64_t)u * A.L;
 
-    float acc[kTiles][4][4], m[4], l[4];
-    int pa[4];
-    uint8_t mq[4], mk[kTiles][4];
+    float acc[kTiles][kR][4], m[kR], l[kR];
+    int pa[kR];
+    uint8_t mq[kR], mk[kTiles][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kR; ++i) {
         m[i] = kNegBig; l[i] = 0.f;
-        const int r = ty * 4 + i;
+        const int r = ty * kR + i;
         pa[i] = r < GW ? A.L - A.W + (r % A.W) : -1;
         mq[i] = r < GW ? mod[pa[i]] : 0;
     }
@@ -308,7 +315,7 @@ __global__ void __launch_bounds__(kSimtThreads) score_cluster_simt(const ScoreAr
         auto rowB = [&](int lr) -> const T * { return kt + lr < A.L ? k + (int64_t)(kt + lr) * A.ks[2] : nullptr; };
         simt_tile_dot<T>(sm, A.D, rowA, rowB, acc[t]);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < kR; ++i) {
             float mx = m[i], add = 0.f;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -323,7 +330,7 @@ __global__ void __launch_bounds__(kSimtThreads) score_cluster_simt(const ScoreAr
         }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {                                // the 16 threads that share a row sit in one half-warp
+    for (int i = 0; i < kR; ++i) {                                // the 16 threads that share a row sit in one half-warp
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) {
             const float mo = __shfl_xor_sync(0xFFFFFFFFu, m[i], o);
@@ -332,7 +339,7 @@ __global__ void __launch_bounds__(kSimtThreads) score_cluster_simt(const ScoreAr
             l[i] = l[i] * exp2f(m[i] - mx) + lo * exp2f(mo - mx);
             m[i] = mx;
         }
-        if (tx == 0) { stat_m[ty * 4 + i] = m[i]; stat_l[ty * 4 + i] = l[i]; }
+        if (tx == 0) { stat_m[ty * kR + i] = m[i]; stat_l[ty * kR + i] = l[i]; }
     }
     cluster_sync();
     if (tid < GW) {
@@ -351,15 +358,15 @@ __global__ void __launch_bounds__(kSimtThreads) score_cluster_simt(const ScoreAr
     }
     cluster_arrive();                                            // the other CTAs' statistics have been read
     __syncthreads();
-    float cross[4] = {0.f, 0.f, 0.f, 0.f};
+    float cross[kR] = {};
 #pragma unroll
     for (int t = 0; t < kTiles; ++t) {
         const int kt = (rank + t * ctas) * kTile;
         if (kt >= A.L) break;
         float colacc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = ty * 4 + i;
+        for (int i = 0; i < kR; ++i) {
+            const int r = ty * kR + i;
             if (r >= GW) break;
             const float mx = row_max[r], inv = row_inv[r];
 #pragma unroll
@@ -381,10 +388,10 @@ __global__ void __launch_bounds__(kSimtThreads) score_cluster_simt(const ScoreAr
         }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kR; ++i) {
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) cross[i] += __shfl_xor_sync(0xFFFFFFFFu, cross[i], o);
-        if (tx == 0) row_cross[ty * 4 + i] = cross[i];
+        if (tx == 0) row_cross[ty * kR + i] = cross[i];
     }
     __syncthreads();
     for (int g = tid; g < A.G; g += kSimtThreads) {
@@ -453,9 +460,9 @@ struct MatchArgs {
     int64_t ks[3];
 };
 
-// Eq. 9 and Eq. 10: cosine similarity of 64 non-pivots against every pivot, gated argmax per row.
-// grid = (U*Hkv, ceil(E / 64)).
-template <typename T>
+// Eq. 9 and Eq. 10: cosine similarity of 16 kR non-pivots against every pivot, gated argmax per row.
+// grid = (U*Hkv, ceil(E / (16 kR))).
+template <typename T, int kR>
 __global__ void __launch_bounds__(kSimtThreads) match_simt(const MatchArgs A) {
     predecessor_done();
     __shared__ SimtTiles sm;
@@ -467,14 +474,14 @@ __global__ void __launch_bounds__(kSimtThreads) match_simt(const MatchArgs A) {
     const float *imp = A.importance + (int64_t)uh * A.L;
     const uint8_t *mod = A.modality + (int64_t)u * A.L;
     const bool intra = A.strategy[u] == 0;
-    const int j0 = blockIdx.y * kTile;
+    const int j0 = blockIdx.y * (16 * kR);
 
-    float best[4];
-    int bests[4];
-    uint8_t me[4];
+    float best[kR];
+    int bests[kR];
+    uint8_t me[kR];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int j = j0 + ty * 4 + i;
+    for (int i = 0; i < kR; ++i) {
+        const int j = j0 + ty * kR + i;
         const int e = j < A.E ? evi[j] : -1;
         me[i] = e >= 0 ? mod[e] : 0;
         best[i] = -INFINITY;
@@ -497,7 +504,7 @@ __global__ void __launch_bounds__(kSimtThreads) match_simt(const MatchArgs A) {
             adm[j] = r >= 0 && imp[r] <= A.tau_eff;          // a highly sensitive pivot is never a merge target
             mr[j] = r >= 0 ? mod[r] : 0;
         }
-        float acc[4][4];
+        float acc[kR][4];
         simt_tile_dot<T, true>(sm, A.D, rowA, rowB, acc);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -505,22 +512,22 @@ __global__ void __launch_bounds__(kSimtThreads) match_simt(const MatchArgs A) {
             if (!adm[j]) continue;
             const float rnr = sm.norm_b[tx * 4 + j];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
+            for (int i = 0; i < kR; ++i) {
                 if (intra && mr[j] != me[i]) continue;
-                const float uval = acc[i][j] * sm.norm_a[ty * 4 + i] * rnr;
+                const float uval = acc[i][j] * sm.norm_a[ty * kR + i] * rnr;
                 if (uval > best[i] || (uval == best[i] && s < bests[i])) { best[i] = uval; bests[i] = s; }
             }
         }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < kR; ++i) {
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1) {
             const float bo = __shfl_xor_sync(0xFFFFFFFFu, best[i], o);
             const int so = __shfl_xor_sync(0xFFFFFFFFu, bests[i], o);
             if (bo > best[i] || (bo == best[i] && so < bests[i])) { best[i] = bo; bests[i] = so; }
         }
-        const int j = j0 + ty * 4 + i;
+        const int j = j0 + ty * kR + i;
         if (tx == 0 && j < A.E) {
             const bool none = bests[i] == 0x7FFFFFFF;
             A.match[(int64_t)uh * A.E + j] = none ? -1 : bests[i];
