@@ -7,7 +7,8 @@
 // keeps every tile of the head in TMEM, and a team of eight warps sweeps them three times:
 //   A  per proxy row the maximum over all keys (running while the K tiles still stream),
 //   B  per proxy row the sum of exponentials, in total and over the keys of the other modality (Eq. 7),
-//   C  per key the sum over proxy rows of exp / row sum: the importance (group mean over the G heads).
+//   C  per key the sum over proxy rows of exp / row sum: the importance (group mean over the G heads); the exponentials are those of
+//      sweep B, which leaves them in TMEM (1024 heads of 640 tokens 132 -> 122 us for the whole call, 32 of 640 24.7 -> 23.7).
 // Lanes are keys, so the per-row reductions of A and B cross lanes (shuffles, then shared memory across
 // the warps) once per head; everything else is per thread.  K is read from HBM exactly once.
 // CTAs are persistent (one per SM) and take (unit, KV head) items in turn.  Warp 0 streams Q and the
@@ -253,6 +254,7 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
 #pragma unroll
                     for (int q = 0; q < HC; ++q) p[q] = key > lim[cb + q] ? 0.f : p[q];
                 }
+                tc::tmem_st16(trow + GW * t, p);                     // in the logits' place, for sweep C
                 if (one_kind) {
                     const float o = (oth & 1u) ? 1.f : 0.f;
 #pragma unroll
@@ -262,6 +264,7 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
                     for (int q = 0; q < HC; ++q) { lt[q] += p[q]; lc[q] += ((oth >> q) & 1u) ? p[q] : 0.f; }
                 }
             }
+            tc::tmem_st_wait();
             warp_reduce16(lt, [](float a, float b) { return a + b; });
             warp_reduce16(lc, [](float a, float b) { return a + b; });
             if (!(lane & 1)) {
@@ -287,20 +290,10 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
             for (int t = 0; t < kMaxTiles; ++t) {
                 imp[t] = 0.f;
                 if (t < nt) {
-                    const int key = t * kTile + row;
                     uint32_t r[HC];
                     load(t, r);
-                    if (t < n_plain) {
 #pragma unroll
-                        for (int q = 0; q < HC; ++q)
-                            imp[t] = fmaf(tc::ex2(fmaf(__uint_as_float(r[q]), A.scale_log2, -mx[q])), lt[q], imp[t]);
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < HC; ++q) {
-                            const float p = tc::ex2(fmaf(__uint_as_float(r[q]), A.scale_log2, -mx[q])) * lt[q];
-                            imp[t] += key <= lim[cb + q] ? p : 0.f;
-                        }
-                    }
+                    for (int q = 0; q < HC; ++q) imp[t] = fmaf(__uint_as_float(r[q]), lt[q], imp[t]);
                     if (half == 1) impx[t * kTile + row] = imp[t];
                 }
             }
