@@ -198,7 +198,7 @@ def ncu_traffic(workload, permille, units, kernel):
 KERNEL_MODEL = {   # kernel name -> entry of kernel_model()
     "score_stats_simt": "score_stats", "score_stats_tc": "score_stats", "score_fused_tc": "score_colsum",
     "score_colsum_simt": "score_colsum", "score_colsum_tc": "score_colsum",
-    "score_cluster_simt": "score_colsum", "merge_short": "merge_rows", "match_simt": "match", "match_tc": "match", "match_small_tc": "match", "merge_rows": "merge_rows",
+    "score_cluster_simt": "score_colsum", "score_cluster_tc": "score_colsum", "merge_short": "merge_rows", "match_simt": "match", "match_tc": "match", "match_small_tc": "match", "merge_rows": "merge_rows",
     "merge_tc": "merge_rows", "match_merge_tc": "merge_rows",
     "select_topb": "select_topb", "build_csr": "build_csr",
 }

@@ -18,6 +18,7 @@
 #include "match_small_tc.cuh"
 #include "merge_rows.cuh"
 #include "merge_tc.cuh"
+#include "score_cluster_tc.cuh"
 #include "score_fused_tc.cuh"
 #include "match_tc.cuh"
 #include "merge_lists.cuh"
@@ -424,6 +425,46 @@ flowmm_status run_score_fused(const flowmm_params &p, const Layout &y, const voi
     return FLOWMM_OK;
 }
 
+// One pass by clusters (score_cluster_tc.cuh) where all of its CTAs run at once: a cluster's CTAs take 9 us one after the other what the two
+// passes take side by side (112 heads of 640 tokens, 448 rows, whole call 77.9 us by two passes, 96.8 by clusters; 16 of 1471 36.8, 33.5).
+// Few proxy rows would leave lanes without one (32 heads of 2000 tokens, 32 rows, 45.2, 51.8).  Key tiles per CTA: the fewest that fit;
+// returns the CTAs per head (0: not so).
+constexpr int kClusterScoreCtas = 112;
+int cluster_score_split(const flowmm_params &p, int &kt) {
+    const int gw = p.n_q_heads / p.n_kv_heads * p.window, rt = (gw + sct::kTile - 1) / sct::kTile, nt = (p.seq_len + sct::kTile - 1) / sct::kTile;
+    if (!use_tc_score(p) || gw < 96 || rt > sct::kMaxAcc) return 0;
+    for (kt = 1; rt * kt <= sct::kMaxAcc; kt *= 2) {
+        const int ctas = (nt + kt - 1) / kt;
+        if (ctas <= sct::kMaxCtas && (int64_t)p.n_units * p.n_kv_heads * ctas <= kClusterScoreCtas) return ctas;
+    }
+    return 0;
+}
+
+flowmm_status run_score_cluster(const flowmm_params &p, const Layout &y, const void *q, const void *k, const uint8_t *mod, float *importance, int kt,
+                                int ctas, void *ws, cudaStream_t st) {
+    const int UH = p.n_units * p.n_kv_heads, G = p.n_q_heads / p.n_kv_heads, W = p.window;
+    sct::Args a;
+    a.modality = mod; a.importance = importance; a.cross_part = at<float>(ws, y.cross_part); a.status = at<int>(ws, y.status);
+    a.Hq = p.n_q_heads; a.Hkv = p.n_kv_heads; a.G = G; a.W = W; a.L = p.seq_len; a.GW = G * W;
+    a.rt = (a.GW + sct::kTile - 1) / sct::kTile; a.kt = kt; a.ctas = ctas;
+    const int q_heads = G < sct::kTile / W ? G : sct::kTile / W;      // of a tile of proxy rows
+    a.q_bytes = (uint32_t)(q_heads * W) * 256u;
+    const float scale = p.softmax_scale != 0.f ? p.softmax_scale : 1.f / sqrtf((float)p.head_dim);
+    a.scale_log2 = scale * kLog2e;
+    CUtensorMap qmap, kmap;
+    const uint64_t qd[4] = {128, (uint64_t)W, (uint64_t)p.n_q_heads, (uint64_t)p.n_units};
+    const uint64_t qs[3] = {(uint64_t)p.q_stride[2] * 2, (uint64_t)p.q_stride[1] * 2, (uint64_t)p.q_stride[0] * 2};
+    const uint64_t kd[4] = {128, (uint64_t)p.seq_len, (uint64_t)p.n_kv_heads, (uint64_t)p.n_units};
+    const uint64_t ks[3] = {(uint64_t)p.k_stride[2] * 2, (uint64_t)p.k_stride[1] * 2, (uint64_t)p.k_stride[0] * 2};
+    const uint32_t bq[4] = {64, (uint32_t)W, (uint32_t)q_heads, 1}, bk[4] = {64, sct::kTile, 1, 1};
+    if (!tc::make_bf16_map(&qmap, q, 4, qd, qs, bq) || !tc::make_bf16_map(&kmap, k, 4, kd, ks, bk)) return FLOWMM_ERR_CUDA;
+    const uint32_t smem = sct::smem_bytes(a.rt, kt);
+    if (cudaFuncSetAttribute(sct::score_cluster_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
+    launch_cluster(dim3(ctas), sct::score_cluster_tc_kernel, UH * ctas, sct::kThreads, smem, st, qmap, kmap, a);
+    FLOWMM_LAUNCHED("score_cluster_tc");
+    return FLOWMM_OK;
+}
+
 // The scoring of short contexts in one launch: a key tile per CTA or two, a row per thread or four.
 template <typename T>
 auto cluster_score_kernel(bool one_tile, bool one_row) {
@@ -436,6 +477,15 @@ flowmm_status run_score(const flowmm_params &p, const Layout &y, const void *q, 
     if (use_fused_score(p)) {
         if (parts_out) *parts_out = 0;
         return run_score_fused(p, y, q, k, mod, importance, cross_mass, ws, st);
+    }
+    int kt = 0;
+    if (const int ctas = cluster_score_split(p, kt)) {
+        FLOWMM_TRY(run_score_cluster(p, y, q, k, mod, importance, kt, ctas, ws, st));
+        if (parts_out) { *parts_out = p.window; return FLOWMM_OK; }  // the caller adds the rows' shares up itself
+        const int n = p.n_units * p.n_q_heads;
+        launch(cross_mass_reduce, (n + 7) / 8, 256, 0, st, at<float>(ws, y.cross_part), p.window, n, cross_mass);
+        FLOWMM_LAUNCHED("cross_mass_reduce");
+        return FLOWMM_OK;
     }
     if (use_tc_score(p)) return run_score_tc(p, y, q, k, mod, importance, cross_mass, ws, st, parts_out);
     ScoreArgs a;

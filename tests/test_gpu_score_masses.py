@@ -102,3 +102,27 @@ def test_sums_over_many_proxy_rows():
     F.flowmm_score(fp, to_dev(q, F.BF16), to_dev(k, F.BF16), torch.from_numpy(m).cuda(), g_imp, g_cross, ws)
     assert F.flowmm_last_device_status(ws) == 0
     assert imp > 0.125 * (1 + 2e-5) and abs(float(g_imp[0, 0, L - W]) / imp - 1) < 1e-6
+
+
+@pytest.mark.parametrize("pattern", ["random", "run_in_word", "window_of_both"])
+@pytest.mark.parametrize("G,W,L", [(3, 32, 97), (4, 32, 1024), (4, 32, 1025), (4, 32, 4096), (4, 32, 4097), (7, 32, 1471), (8, 32, 2048), (8, 32, 2049),
+                                   (3, 128, 256), (7, 64, 641), (8, 64, 1024), (8, 64, 1025)])
+def test_few_heads_and_many_of_the_same(G, W, L, pattern):
+    """One unit, whose heads are shared by clusters of one to eight CTAs of one, two or four key tiles (up to the longest prompt that
+    one to four tiles of proxy rows leave room for), and sixty times that unit, which takes the two passes."""
+    rng = np.random.default_rng(L + G)
+    modality = PATTERNS[pattern](rng, L)[None]
+    p = O.OracleParams(1, 2 * G, 2, 128, L, W, 1)
+    q, k = (inputs.round_to_bf16(rng.standard_normal(s).astype(np.float32)) for s in ((1, 2 * G, W, 128), (1, 2, L, 128)))
+    m = np.ascontiguousarray(modality, dtype=np.uint8)
+    imp, cross, _ = O.score(p, q, k, m)
+    qd, kd, md = to_dev(q, F.BF16), to_dev(k, F.BF16), torch.from_numpy(m).cuda()
+    for U in (1, 60):
+        fp = F.Params(U, 2 * G, 2, 128, L, W, 1)
+        g_imp, g_cross = torch.full((U, 2, L), float("nan"), device="cuda"), torch.full((U, 2 * G), float("nan"), device="cuda")
+        ws = F.alloc_workspace(fp)
+        F.flowmm_score(fp, qd.repeat(U, 1, 1, 1), kd.repeat(U, 1, 1, 1), md.repeat(U, 1), g_imp, g_cross, ws)
+        assert F.flowmm_last_device_status(ws) == 0
+        for u in (0, U - 1):
+            assert np.abs(g_imp[u].double().cpu().numpy() / imp[0] - 1).max() < 1e-5
+            assert np.abs(g_cross[u].double().cpu().numpy() - cross[0]).max() < 1e-5 * W
