@@ -1226,25 +1226,40 @@ struct DecodePlan {
 
 constexpr int kMaxDecodeCluster = dtc::kMaxRanges;         // ranges of a head that are joined as one cluster (the portable cluster size)
 
+// Records that are set aside for the ranges of all heads whatever the plan, so that a workspace for more keys or heads is never smaller: four
+// per SM, and for every head eight, or as many as its ranges of kMaxTiles are.  A head is cut into its share of them at most.
+int64_t decode_records(int uh, int tiles) {
+    const int longest = (tiles + dtc::kMaxTiles - 1) / dtc::kMaxTiles;
+    return std::min((int64_t)uh * tiles, std::max((int64_t)uh * std::max(kMaxDecodeCluster, longest), (int64_t)4 * kScoreCtas + uh));
+}
+
 DecodePlan decode_plan(const flowmm_decode_params &p) {
     DecodePlan d;
     const int uh = p.n_units * p.n_kv_heads, g = p.n_q_heads / p.n_kv_heads;
     d.tc = p.dtype == FLOWMM_BF16 && p.head_dim == 128 && p.path != FLOWMM_PATH_SIMT;
     if (d.tc) {
-        // Two CTAs share an SM.  Of the range lengths TMEM allows, take the one with the least work per CTA slot: rounds of
-        // CTAs (a last one that is nearly empty counts half when there are several) times a CTA's tiles and its fixed cost
-        // (set-up, the pause between its two phases: like a tile and a half), and for joining the ranges a tile and a half
-        // as a cluster or two and a half as a launch of its own.  Measured over 16 shapes from 4 heads of 218 keys to 640
-        // of 1690 the choice is within 11 % of the best length.
-        const int tiles = (p.n_keys + dtc::kTile - 1) / dtc::kTile;
-        const double slots = 2.0 * tc::sm_count();
+        // Two CTAs share an SM.  Of the range lengths TMEM allows, the one whose call is the shortest by this account, in us: all tiles of K
+        // and V at the memory's rate, or the one CTA's, 0.9 a tile, where that is longer; when the CTAs do not fit at once, 1 per further
+        // round, and part of what the last ones take with the memory mostly idle; for joining the ranges 2 as a cluster, 3 as a launch of
+        // its own.  Clusters find room for 0.88 of the CTAs (96 of three, 12 tiles each, ran two after the other: 47 us, by five of 7 tiles
+        // 40).  Measured with every length on 18 shapes, 16 to 554 MB of 4 to 1024 heads: 1 % on average, 10 % at most above the best
+        // length (4 and 18 % by rounds of CTAs times their tiles and a fixed cost each).
+        const int tiles = (p.n_keys + dtc::kTile - 1) / dtc::kTile, most = (int)(decode_records(uh, tiles) / uh);
         double best = 0.0;
-        d.per_split = 1;
+        d.per_split = 0;
         for (int per = 1; per <= dtc::kMaxTiles && per <= tiles; ++per) {
-            const int64_t splits = (tiles + per - 1) / per;
-            const double full = (double)(uh * splits) / slots, rounds = fmax(1.0, fmin(ceil(full), full + 0.5));
-            const double cost = rounds * (per + 1.5) + (splits == 1 ? 0.0 : splits <= kMaxDecodeCluster ? 1.5 : 2.5);
-            if (per == 1 || cost < best) { best = cost; d.per_split = per; }
+            const int splits = (tiles + per - 1) / per;
+            if (splits > most) continue;
+            const bool cluster = splits > 1 && splits <= kMaxDecodeCluster;
+            const double slots = 2.0 * kScoreCtas * (cluster ? 0.88 : 1.0), ctas = (double)uh * splits, rounds = ctas / slots;
+            const double tile_us = 0.00985, all = uh * (double)tiles * tile_us, lone = 0.9 * per;
+            double cost = all > lone ? all : lone;
+            if (rounds > 1.0) {
+                const double last = ctas - floor(rounds) * slots, gap = lone + 3.0 - last * per * tile_us;
+                cost = all + (last > 0.0 && gap > 0.0 ? gap * (cluster ? 0.5 : 0.1) : 0.0) + (rounds - 1.0);
+            }
+            cost += (splits == 1 ? 0.0 : cluster ? 2.0 : 3.0) + 0.15 * per;
+            if (d.per_split == 0 || cost < best) { best = cost; d.per_split = per; }
         }
         d.n_split = (tiles + d.per_split - 1) / d.per_split;
     }
@@ -1257,7 +1272,8 @@ DecodePlan decode_plan(const flowmm_decode_params &p) {
         d.n_split = (p.n_keys + d.per_split - 1) / d.per_split;
     }
     d.part_off = 256;
-    d.bytes = d.part_off + align256((size_t)uh * d.n_split * g * (p.head_dim + 2) * sizeof(float));
+    const size_t n_rec = d.tc ? (size_t)decode_records(uh, (p.n_keys + dtc::kTile - 1) / dtc::kTile) : (size_t)uh * d.n_split;
+    d.bytes = d.part_off + align256(n_rec * g * (p.head_dim + 2) * sizeof(float));
     return d;
 }
 
