@@ -86,10 +86,9 @@ __device__ __forceinline__ void match_unit(uint32_t trow, uint32_t md, uint32_t 
 #pragma unroll
         for (int q4 = 0; q4 < 4; ++q4) {                 // a column that is no candidate has scale NaN and never wins
             const float4 s4 = tc::lds128(md + (blk * 4 + q4) * 16);
-            v[4 * q4 + 0] = __uint_as_float(acc[4 * q4 + 0]) * s4.x;
-            v[4 * q4 + 1] = __uint_as_float(acc[4 * q4 + 1]) * s4.y;
-            v[4 * q4 + 2] = __uint_as_float(acc[4 * q4 + 2]) * s4.z;
-            v[4 * q4 + 3] = __uint_as_float(acc[4 * q4 + 3]) * s4.w;
+            const float2 p01 = tc::fmul2(make_float2(__uint_as_float(acc[4 * q4]), __uint_as_float(acc[4 * q4 + 1])), make_float2(s4.x, s4.y));
+            const float2 p23 = tc::fmul2(make_float2(__uint_as_float(acc[4 * q4 + 2]), __uint_as_float(acc[4 * q4 + 3])), make_float2(s4.z, s4.w));
+            v[4 * q4] = p01.x; v[4 * q4 + 1] = p01.y; v[4 * q4 + 2] = p23.x; v[4 * q4 + 3] = p23.y;
         }
 #pragma unroll
         for (int h8 = 0; h8 < 2; ++h8) {                 // two groups of 8 columns, in column order
