@@ -246,9 +246,12 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
                 const unsigned oth = ((vis_bits >> t) & 1u) ? ~qvis : qvis;   // proxy rows of the other modality than this key's
                 uint32_t r[HC];
                 load(t, r);
-                float p[HC];
+                float p[HC];                                         // (multiply-adds as packed pairs: half the issue slots)
 #pragma unroll
-                for (int q = 0; q < HC; ++q) p[q] = tc::ex2(fmaf(__uint_as_float(r[q]), A.scale_log2, -mx[q]));
+                for (int q = 0; q < HC; q += 2) {
+                    const float2 x = tc::ffma2(make_float2(__uint_as_float(r[q]), __uint_as_float(r[q + 1])), make_float2(A.scale_log2, A.scale_log2), make_float2(-mx[q], -mx[q + 1]));
+                    p[q] = tc::ex2(x.x); p[q + 1] = tc::ex2(x.y);
+                }
                 if (t >= n_plain) {
                     const int key = t * kTile + row;
 #pragma unroll
@@ -258,7 +261,11 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
                 if (one_kind) {
                     const float o = (oth & 1u) ? 1.f : 0.f;
 #pragma unroll
-                    for (int q = 0; q < HC; ++q) { lt[q] += p[q]; lc[q] = fmaf(o, p[q], lc[q]); }
+                    for (int q = 0; q < HC; q += 2) {
+                        const float2 p2 = make_float2(p[q], p[q + 1]);
+                        const float2 t2 = tc::fadd2(make_float2(lt[q], lt[q + 1]), p2), c2 = tc::ffma2(make_float2(o, o), p2, make_float2(lc[q], lc[q + 1]));
+                        lt[q] = t2.x; lt[q + 1] = t2.y; lc[q] = c2.x; lc[q + 1] = c2.y;
+                    }
                 } else {
 #pragma unroll
                     for (int q = 0; q < HC; ++q) { lt[q] += p[q]; lc[q] += ((oth >> q) & 1u) ? p[q] : 0.f; }
@@ -292,8 +299,10 @@ score_fused_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_con
                 if (t < nt) {
                     uint32_t r[HC];
                     load(t, r);
+                    float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
-                    for (int q = 0; q < HC; ++q) imp[t] = fmaf(__uint_as_float(r[q]), lt[q], imp[t]);
+                    for (int q = 0; q < HC; q += 2) s2 = tc::ffma2(make_float2(__uint_as_float(r[q]), __uint_as_float(r[q + 1])), make_float2(lt[q], lt[q + 1]), s2);
+                    imp[t] = s2.x + s2.y;
                     if (half == 1) impx[t * kTile + row] = imp[t];
                 }
             }
