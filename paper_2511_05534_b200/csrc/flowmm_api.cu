@@ -191,7 +191,11 @@ Layout make_layout(const flowmm_params &p) {
     // 4 of 4500 51.8, 50.1; 8 of 1000, 512 rows 35.7, 32.8; 4 caches of 640 rows 37.2, 34.8; where pass 2 alone is cut finer 8 of
     // 2300 42.2, 41.1.  With more items than SMs the second round costs what the finer cut gains.
     y.tc_q_rows = G * W > tcs::kRows && U * Hkv * (size_t)y.n_rt * ((G * W + tcs::kRows - 1) / tcs::kRows) <= kScoreCtas ? tcs::kRows : tcs::kItemRows;
-    y.tc_keys2 = U * Hkv * ((L + tcs::kRows - 1) / tcs::kRows) <= kScoreCtas ? tcs::kRows : tcs::kItemRows;
+    // Pass 2 by items of 128 as well, on which all warps of a CTA work, where the longest run of items of 256 is a good deal more than the longest
+    // of 128: heads that end in half an item, few items per CTA (112 caches of 640 rows, 448 proxy rows: the call 77.7 -> 75.9 us).
+    const size_t halves2 = U * Hkv * ((L + tcs::kRows - 1) / tcs::kRows), items2 = U * Hkv * (size_t)y.n_rt;
+    const size_t run_items = (items2 + kScoreCtas - 1) / kScoreCtas, run_halves = (halves2 + kScoreCtas - 1) / kScoreCtas;
+    y.tc_keys2 = halves2 <= kScoreCtas || 50 * run_halves * items2 <= 41 * run_items * halves2 ? tcs::kRows : tcs::kItemRows;
     // pass 1 of the tensor-core scoring: the key tiles of all heads in equal runs, one per SM and tile of proxy rows
     y.tc_n_qt = (int)((G * W + y.tc_q_rows - 1) / y.tc_q_rows);
     {
@@ -365,14 +369,14 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
     if (!tc::make_bf16_map(&qa, q, 4, qd, qs, bqa) || !tc::make_bf16_map(&qb, q, 4, qd, qs, bqb) ||
         !tc::make_bf16_map(&k128, k, 4, kd, ks, bk128) || !tc::make_bf16_map(&k256, k, 4, kd, ks, bk256))
         return FLOWMM_ERR_CUDA;
+    const bool split2 = a.keys2 == tcs::kRows;
+    auto pass2 = small2 ? (split2 ? score_colsum_tc_kernel<tcs::Small, true> : score_colsum_tc_kernel<tcs::Small, false>)
+                 : resident2 ? (split2 ? score_colsum_tc_kernel<tcs::Resident, true> : score_colsum_tc_kernel<tcs::Resident, false>)
+                             : (split2 ? score_colsum_tc_kernel<tcs::Big, true> : score_colsum_tc_kernel<tcs::Big, false>);
+    const uint32_t smem2 = small2 ? tcs::Small::kSmemBytes : resident2 ? tcs::Resident::kSmemBytes : tcs::Big::kSmemBytes;
     if (cudaFuncSetAttribute(score_stats_tc_kernel<tcs::Big>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)tcs::Big::kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(score_colsum_tc_kernel<tcs::Big>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tcs::Big::kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(score_colsum_tc_kernel<tcs::Resident>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tcs::Resident::kSmemBytes) != cudaSuccess ||
-        cudaFuncSetAttribute(score_colsum_tc_kernel<tcs::Small>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)tcs::Small::kSmemBytes) != cudaSuccess)
+        cudaFuncSetAttribute(pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
     launch(score_stats_tc_kernel<tcs::Big>, grid1, tcs::kThreads, tcs::Big::kSmemBytes, st, qa, k256, a);
     FLOWMM_LAUNCHED("score_stats_tc");
@@ -384,9 +388,7 @@ flowmm_status run_score_tc(const flowmm_params &p, const Layout &y, const void *
         FLOWMM_LAUNCHED("score_combine");
         a.row_all = all;
     }
-    if (small2) launch(score_colsum_tc_kernel<tcs::Small>, grid2, tcs::kThreads, tcs::Small::kSmemBytes, st, k128, qb, a);
-    else if (resident2) launch(score_colsum_tc_kernel<tcs::Resident>, grid2, tcs::kThreads, tcs::Resident::kSmemBytes, st, k128, qb, a);
-    else launch(score_colsum_tc_kernel<tcs::Big>, grid2, tcs::kThreads, tcs::Big::kSmemBytes, st, k128, qb, a);
+    launch(pass2, grid2, tcs::kThreads, smem2, st, k128, qb, a);
     FLOWMM_LAUNCHED("score_colsum_tc");
     if (parts_out) { *parts_out = W; return FLOWMM_OK; }              // the caller adds the rows' shares up itself
     const int n = p.n_units * p.n_q_heads;

@@ -440,7 +440,7 @@ __device__ __forceinline__ void colsum_chunk32_exact(uint32_t (&a)[32], uint32_t
 #undef FLOWMM_EX_REGS
 
 // ---------------------------------------------------------------------------------------------
-// Pass 2.  item = (unit*head, tile of 256 keys, or of 128 where few items leave SMs idle); the B stream is the head group's proxy rows.  A CTA takes a run of
+// Pass 2.  item = (unit*head, tile of 256 keys, or of 128, on which all sixteen epilogue warps work, where items are few); the B stream is the head group's proxy rows.  A CTA takes a run of
 // consecutive items, so that proxy rows that fit the B stages (up to 512) are loaded once per head, not once per item.
 // Row constants -(max + log2 sum) - exp2(logit + constant) is the softmax probability - are formed from pass 1's statistics by
 // the epilogue warps when the run comes to another head; the CTA with a head's first tile also writes its rows' cross-modal shares.
@@ -448,13 +448,16 @@ __device__ __forceinline__ void colsum_chunk32_exact(uint32_t (&a)[32], uint32_t
 // chunk is read while the one before it is worked on, an accumulator is handed back as soon as its last chunk is in registers,
 // and no vote or shuffle stands between: 197 -> 152 instructions per chunk of 32 columns.  (Three or four words a thread of
 // what belongs to the item are spilled around the chunks; unrolling two chunks instead of four leaves one, and is 1 % slower.)
-template <class S>
+template <class S, bool kSplit>
 __global__ void __launch_bounds__(tcs::kThreads, 1)
 score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_constant__ CUtensorMap q_map,
                        const ScoreTcArgs A) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    const typename S::Ctx c = S::setup(smem_raw, &k_map, &q_map, A.status, 0, 4);
+    // kSplit (A.keys2 == 128): one half per item, whose columns the two groups of warps share
+    typename S::Ctx c = S::setup(smem_raw, &k_map, &q_map, A.status, 0, kSplit ? 8 : 4);
     if (!c.ok) return;
+    const int share = kSplit ? c.group : 0, part_of = c.group * 2 + c.colhalf;   // which of a column half's chunks; which of a key's partial sums
+    if (kSplit) c.group = 0;
     const int g_lo = (int)((int64_t)A.n_items2 * blockIdx.x / gridDim.x), g_hi = (int)((int64_t)A.n_items2 * (blockIdx.x + 1) / gridDim.x);
     const int n_loop = (g_hi - g_lo) * gridDim.x;                   // the roles count items blockIdx.x, blockIdx.x + gridDim.x, ...
     auto plan = [&](int item) {
@@ -479,10 +482,10 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
         S::template mma_issuer<true>(c, blockIdx.x + n_loop, plan, A.status);
     } else {
         // scratch: two sets of row constants by turns (up to 1024 rows), then the hand-over slots of the row halves, two by turns
-        constexpr uint32_t kConstBytes = 4096, kXch = S::kSmemEpi + 2 * kConstBytes;
-        static_assert(2 * kConstBytes + 2 * 2 * tcs::kRows * 4 <= tcs::kEpiBytes, "scratch");
+        constexpr uint32_t kConstBytes = 4096, kXch = S::kSmemEpi + 2 * kConstBytes, kXchPart = tcs::kRows * 4;
+        static_assert(2 * kConstBytes + 2 * 4 * kXchPart <= tcs::kEpiBytes, "scratch");
         const int lane = c.lane, row = c.quarter * 32 + lane, te = threadIdx.x - 64;
-        const uint32_t xch = c.base + kXch + (uint32_t)(c.group * tcs::kRows + row) * 4;
+        const uint32_t xch = c.base + kXch + (uint32_t)part_of * kXchPart + (uint32_t)row * 4;
         int k = 0;
         bool ok = true;
         // the run's items one after the other: (unit u, KV head uh, its tile kt) step by step instead of by divisions, which
@@ -540,7 +543,7 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                 if (++hk == A.Hkv) { hk = 0; ++u; }
             }
             const int key0 = kt0 * A.keys2 + c.group * tcs::kRows;
-            if (key0 >= A.L || c.group * tcs::kRows >= A.keys2) continue;   // no keys in this half
+            if (key0 >= A.L) continue;                               // no keys in this half
             const int key = key0 + row;
             const bool masked_tile = key0 + tcs::kRows > A.L - A.W + 1;   // some (key, proxy row) pair is masked
             const int first_proxy = A.L - A.W;
@@ -555,7 +558,12 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                 ok = ok && S::quad_extra_wait_lanes(c, k, -1, A.status);
                 ++k;
                 constexpr int kPerC = S::kCols / 64;                 // 32-column chunks a warp takes of a full tile
-                const int ch0 = kPerC * c.colhalf, n_ch = min((ncols + 31) >> 5, ch0 + kPerC) - ch0;   // >= 1
+                int ch0 = kPerC * c.colhalf, n_ch = min((ncols + 31) >> 5, ch0 + kPerC) - ch0;   // >= 1
+                if (kSplit) {
+                    ch0 += share * (kPerC / 2);
+                    n_ch = min(n_ch - share * (kPerC / 2), kPerC / 2);
+                    if (n_ch <= 0) { S::quad_release(c); continue; }
+                }
                 const uint32_t nc = consts + (uint32_t)(t * S::kCols + ch0 * 32) * 4;
                 if (!masked_tile && both == 0u) {
                     uint32_t a[2][32];
@@ -605,13 +613,18 @@ score_colsum_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_c
                 S::quad_release(c);
             }
             imp += __uint_as_float((uint32_t)sum2) + __uint_as_float((uint32_t)(sum2 >> 32));
-            // the two column halves of a key meet: the upper one hands its partial sum over (kept even after a
-            // wait ran out, so that the partner warp is never left waiting).  Two slots by turns: the next meeting keeps the
-            // upper half from a slot that is still being read.
-            if (c.colhalf == 1) tc::sts32(xch + slot, imp);
-            ok = !S::pair_meet(c, !ok);
-            if (c.colhalf == 0 && ok && key < A.L) A.importance[(int64_t)uh0 * A.L + key] = (imp + tc::lds32(xch + slot)) / (float)A.G;   // group mean
-            slot ^= 2 * tcs::kRows * 4;
+            // the two column halves of a key meet (or their four shares): the others hand their partial sums to the first (kept even
+            // after a wait ran out, so that no partner warp is left waiting).  Two sets of slots by turns: the next meeting keeps the
+            // others from slots that are still being read.
+            const bool owner = c.colhalf == 0 && share == 0;
+            if (!owner) tc::sts32(xch + slot, imp);
+            ok = !(kSplit ? tcs::meet_vote(1 + c.quarter, 128, !ok) : S::pair_meet(c, !ok));
+            if (owner && ok && key < A.L) {
+                float sum = imp + tc::lds32(xch + slot + kXchPart);
+                if (kSplit) sum += tc::lds32(xch + slot + 2 * kXchPart) + tc::lds32(xch + slot + 3 * kXchPart);
+                A.importance[(int64_t)uh0 * A.L + key] = sum / (float)A.G;   // group mean
+            }
+            slot ^= 4 * kXchPart;
         }
     }
     S::teardown(c);

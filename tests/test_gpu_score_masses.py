@@ -82,6 +82,15 @@ def test_items_of_one_half_and_of_two(U, G, W, L):
     _check(rng, U, G, 1, L, W, np.arange(L)[None] // 50 % 2 ^ rng.integers(0, 2, (U, 1)))
 
 
+@pytest.mark.parametrize("G,W", [(2, 64), (7, 32), (7, 64)])
+@pytest.mark.parametrize("L", [513, 640])
+def test_runs_of_half_items(G, W, L):
+    """112 heads of five halves of an item: the second pass gives all warps of a CTA one half at a time, four to a CTA, in each of its
+    three shapes."""
+    rng = np.random.default_rng(G * W + L)
+    _check(rng, 112, G, 1, L, W, np.arange(L)[None] // 50 % 2 ^ rng.integers(0, 2, (112, 1)))
+
+
 def test_sums_over_many_proxy_rows():
     """A key of the window that one proxy row gives all of its mass and 1023 others 2.5e-8 each: added to the one, one by one, they would
     vanish (half of them share its sum: 1.3e-5).  Exponentials within 2^-22, their arguments (up to 26) within 2e-6, sums of 32 by fours."""
