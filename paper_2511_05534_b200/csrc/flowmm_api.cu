@@ -557,12 +557,12 @@ MatchPrepArgs match_prep_args(const flowmm_params &p, const Layout &y, const voi
     return g;
 }
 
-template <int kThreads, bool kOneChunk, int kCtas = 1>
+template <int kThreads, bool kOneChunk, int kCtas = 1, bool kFew = false>
 flowmm_status launch_select(const SelectArgs &a, const SelectFlow &f, const MatchPrepArgs &g, int with_prepare, cudaStream_t st) {
     const size_t smem = select_smem(a.chunk);
-    if (cudaFuncSetAttribute(select_topb_kernel<kThreads, kOneChunk, kCtas>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(select_topb_kernel<kThreads, kOneChunk, kCtas, kFew>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return FLOWMM_ERR_CUDA;
-    launch_cluster(dim3(kCtas), select_topb_kernel<kThreads, kOneChunk, kCtas>, (a.n_heads + f.n_units) * kCtas, kThreads, smem, st, a, f, g, with_prepare);
+    launch_cluster(dim3(kCtas), select_topb_kernel<kThreads, kOneChunk, kCtas, kFew>, (a.n_heads + f.n_units) * kCtas, kThreads, smem, st, a, f, g, with_prepare);
     FLOWMM_LAUNCHED("select_topb");
     return FLOWMM_OK;
 }
@@ -596,9 +596,13 @@ flowmm_status run_select(const flowmm_params &p, const float *importance, int32_
     }
     // More heads than four blocks of 256 threads per SM would be in two rounds; of 128 threads an SM holds eight.  (1024 heads of 640
     // positions 151.4 -> 149.5 us for the call, of 1000 222.7 -> 221.4; of 400, where a block's rounds are short, 110.4 -> 111.5.)
-    if (p.seq_len > 512 && p.seq_len <= 1024 && a.n_heads > 4 * tc::sm_count()) return launch_select<128, true>(a, f, g, prep != nullptr, st);
-    if (p.seq_len <= 1024) return launch_select<256, true>(a, f, g, prep != nullptr, st);
-    if (p.seq_len <= 4096) return launch_select<512, true>(a, f, g, prep != nullptr, st);
+    if (p.seq_len > 512 && p.seq_len <= 1024 && a.n_heads > 4 * tc::sm_count()) return launch_select<128, true, 1, true>(a, f, g, prep != nullptr, st);
+    // A block that has an SM for itself takes twice the warps: 32 heads of 640 positions 23.5 -> 23.0 us for the call, 4 of 3000 42.5 -> 41.7, 112
+    // of 900 67.1 -> 65.4, of 2176 110.6 -> 109.5; of 4 heads of 192 17.9 -> 18.3, so from 257 positions on.
+    const bool alone = a.n_heads + p.n_units <= tc::sm_count();
+    if (p.seq_len <= (alone ? 256 : 1024)) return launch_select<256, true, 1, true>(a, f, g, prep != nullptr, st);
+    if (p.seq_len <= (alone ? 1024 : 4096)) return launch_select<512, true, 1, true>(a, f, g, prep != nullptr, st);
+    if (p.seq_len <= 4096) return launch_select<1024, true, 1, true>(a, f, g, prep != nullptr, st);
     if (p.seq_len <= kSelMaxChunk) return launch_select<1024, true>(a, f, g, prep != nullptr, st);
     return launch_select<1024, false>(a, f, g, prep != nullptr, st);
 }

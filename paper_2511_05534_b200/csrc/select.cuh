@@ -91,12 +91,12 @@ static_assert(select_smem(kSelMaxChunk) <= 232448 - 1024, "shared memory budget"
 // kCtas > 1: the CTAs of a cluster share a head, A.chunk positions each (a multiple of 256).  The counts of all of them are
 // added up through distributed shared memory in every pass, their totals before the lists are written.  For calls of few
 // heads, whose blocks would leave most SMs idle: 8 heads of 33 792 tokens 31 -> 18 us, 4 heads of 8448 14 -> 12.
-template <int kThreads, bool kOneChunk, int kCtas>
+template <int kThreads, bool kOneChunk, int kCtas, bool kFew>
 __global__ void __launch_bounds__(kThreads, kThreads <= 256 ? 1024 / kThreads : kThreads == 512 && kCtas == 1 ? 2 : 1)
 select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P, int with_prepare) {
     static_assert(kCtas == 1 || (kOneChunk && kThreads == 512), "a CTA's part is one chunk; four counters per thread");
     constexpr int kWarps = kThreads / 32, kPer = kSelBins / kThreads;
-    constexpr bool kFew = kOneChunk && kCtas == 1 && kThreads <= 512;   // (launched for up to 1024 or 4096 positions)
+    static_assert(!kFew || (kOneChunk && kCtas == 1), "a warp's words in registers");   // (kFew: launched for up to 1024 or 4096 positions)
     extern __shared__ __align__(16) int sel_smem[];
     __shared__ int wtot[kWarps], res[3];
     __shared__ unsigned long long wsum[kWarps];
@@ -243,7 +243,7 @@ select_topb_kernel(const SelectArgs A, const SelectFlow F, const MatchPrepArgs P
     // 26.4 -> 25.7, 8 of 1471 36.0 -> 35.0, 112 of 2176 112.7 -> 111.0, 1024 of 640 156.3 -> 153.4.)  Four blocks of 256 threads to an
     // SM: with five or six a thread has too few registers for four rows, with more rows too many.
     if constexpr (kFew) {
-        constexpr int kE = kThreads == 256 ? 4 : 8;
+        constexpr int kE = kThreads == 256 || kThreads == 1024 ? 4 : 8;   // words of a warp: 1024 positions by up to 256 threads, else 4096
         const int n_w = (L + 31) >> 5, per = (n_w + kWarps - 1) / kWarps, w0 = warp * per;
         uint32_t wd[kE], keep[kE], text[kE], vis[kE];
 #pragma unroll

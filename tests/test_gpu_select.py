@@ -33,12 +33,13 @@ def test_select_against_oracle(L, B, kind):
     assert np.array_equal(e.cpu().numpy(), ref_e)
 
 
-@pytest.mark.parametrize("L,B", [(512, 60), (513, 60), (640, 64), (1001, 1000), (1024, 200)])
+@pytest.mark.parametrize("heads,L,B", [(600, 512, 60), (600, 513, 60), (600, 640, 64), (600, 1001, 1000), (600, 1024, 200), (160, 257, 30), (160, 1024, 100),
+                                       (160, 1025, 100), (160, 4096, 300), (147, 256, 30), (147, 257, 30), (147, 1025, 100), (147, 4096, 300)])
 @pytest.mark.parametrize("kind", ["spread", "ties", "equal", "window"])
-def test_many_heads_of_up_to_1024_positions(L, B, kind):
-    """More heads than four blocks per SM (blocks of 128 threads between 512 and 1024 positions), and, with the candidates laid out
-    by the same launch, the matches of the separate step."""
-    heads, W = 600, 32
+def test_many_heads(heads, L, B, kind):
+    """More heads than four blocks per SM (blocks of 128 threads between 512 and 1024 positions), than one per SM, and one fewer than
+    SMs (twice the warps from 257 positions on); and, with the candidates laid out by the same launch, the matches of the separate step."""
+    W = 32
     gen = torch.Generator(device="cuda").manual_seed(L + B)
     imp = torch.exp(torch.randn((1, heads, L), generator=gen, device="cuda") * 2)
     if kind == "ties":
