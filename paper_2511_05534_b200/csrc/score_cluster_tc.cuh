@@ -16,6 +16,7 @@
 // 32 keys of every accumulator).
 #pragma once
 #include "common.cuh"
+#include "decode_tc.cuh"
 #include "score_fused_tc.cuh"
 #include "score_tc.cuh"
 #include "tc_common.cuh"
@@ -31,7 +32,15 @@ constexpr int kBarQ = 0, kBarK = kMaxAcc, kBarAcc = 2 * kMaxAcc, kNumBars = 3 * 
 // Shared memory behind the operand tiles: records of the warps and of the CTA, row constants, a table for sums by modality, partial sums.
 constexpr uint32_t kRows = kMaxAcc * kTile;
 constexpr uint32_t kStat = 0, kRec = kStat + 4 * kRows * 12, kConst = kRec + kRows * 16, kMasks = kConst + kRows * 4, kPart = kMasks + 256;
-inline __host__ __device__ uint32_t smem_bytes(int rt, int kt) { return (uint32_t)(rt + kt) * kTileBytes + kPart + 4u * kt * kTile * 4u + 8 * kNumBars + 16; }
+// At least so much that no other block with tensor memory fits beside it on an SM (decode attention's are the smallest, 109 KB): a cluster's
+// blocks wait for one another, and two clusters of different streams, each with a block that waits for the tensor memory of one of the
+// other's, would wait forever.
+constexpr uint32_t kMinSmem = 120 * 1024;
+static_assert(kMinSmem + dtc::kSmemBytes > 227 * 1024, "no room beside it");
+inline __host__ uint32_t smem_bytes(int rt, int kt) {
+    const uint32_t n = (uint32_t)(rt + kt) * kTileBytes + kPart + 4u * kt * kTile * 4u + 8 * kNumBars + 16;
+    return n > kMinSmem ? n : kMinSmem;
+}
 
 struct Args {
     const uint8_t *modality;     // [U, L]
