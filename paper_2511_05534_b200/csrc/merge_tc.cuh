@@ -20,8 +20,8 @@
 // When SMs are left over even so, a cluster of two or four CTAs shares the steps: each leaves its part of out^T in fp32 in its
 // shared memory (where W was) and they add the parts up in a fixed order through distributed shared memory, a slice of the
 // slots each: calls of 8 heads of 1471 tokens 42.0 -> 39.8 us, 4 of 2176 47.4 -> 43.0, 4 of 4528 65.6 -> 52.5.
-// Bound by the products: a step of 128 tokens takes the tensor core about 1000 clocks per tensor whatever the slots (the X
-// operand is read MN-major).  With four readers storing two bytes per lane the readout took 9 000 (64 slots) to 30 000
+// Bound by HBM with few slots and by the products with many: a step of 128 tokens takes the tensor core 384 clocks per tensor with 64
+// slots, 512 with 128, 896 with 224 (that X is read MN-major costs nothing).  With four readers storing two bytes per lane the readout took 9 000 (64 slots) to 30 000
 // clocks (218) per head on top: 8 heads of 1471 tokens, 148 slots 32 -> 18 us, 112 of 2176, 218 slots 47 -> 36 us, 32 of 640,
 // 64 slots 18 -> 12 us, 1024 of 640 68 -> 63 us.
 // The weights enter rounded to bf16 (relative error <= 2^-9) in numerator and denominator alike, so every

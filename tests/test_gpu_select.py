@@ -33,8 +33,8 @@ def test_select_against_oracle(L, B, kind):
     assert np.array_equal(e.cpu().numpy(), ref_e)
 
 
-@pytest.mark.parametrize("heads,L,B", [(600, 512, 60), (600, 513, 60), (600, 640, 64), (600, 1001, 1000), (600, 1024, 200), (160, 257, 30), (160, 1024, 100),
-                                       (160, 1025, 100), (160, 4096, 300), (147, 256, 30), (147, 257, 30), (147, 1025, 100), (147, 4096, 300)])
+@pytest.mark.parametrize("heads,L,B", [(600, 512, 60), (600, 513, 60), (600, 640, 64), (600, 1001, 1000), (600, 1024, 200), (160, 257, 40), (160, 1024, 100),
+                                       (160, 1025, 100), (160, 4096, 300), (147, 256, 40), (147, 257, 40), (147, 1025, 100), (147, 4096, 300)])
 @pytest.mark.parametrize("kind", ["spread", "ties", "equal", "window"])
 def test_many_heads(heads, L, B, kind):
     """More heads than four blocks per SM (blocks of 128 threads between 512 and 1024 positions), than one per SM, and one fewer than
