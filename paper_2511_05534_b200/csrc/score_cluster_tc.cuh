@@ -169,8 +169,9 @@ score_cluster_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_c
                 for (int j = 0; j < 32; ++j) a[j] = j <= last ? a[j] : __float_as_uint(-INFINITY);
             }
             const float mx = fmaxf(max32(a) * A.scale_log2, kNegBig);
-            // (by the exp2 unit alone where few keys or rows can make up a result)
-            if (masked || (vis != 0u && vis != 0xFFFFFFFFu) || (rows != 0u && rows != 0xFFFFFFFFu)) exp2_32_exact(a, A.scale_log2, mx);
+            // By the exp2 unit alone where few keys or rows can make up a result, and in the window's whole tile, whose keys the second of two
+            // passes gives to that unit as well.
+            if ((tile0 + k + 1) * kTile > A.L - A.W + 1 || (vis != 0u && vis != 0xFFFFFFFFu) || (rows != 0u && rows != 0xFFFFFFFFu)) exp2_32_exact(a, A.scale_log2, mx);
             else exp2_32(a, A.scale_log2, mx);
             tc::tmem_st32(trow + i * kTile, a);
             float on_text = 0.f, on_vis = 0.f;

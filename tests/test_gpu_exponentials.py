@@ -54,33 +54,53 @@ def test_flow_of_one_visual_token(L):
     assert np.abs(g_cross.double().cpu().numpy() / cross - 1).max() < 1.2e-6
 
 
-def test_normalisers_of_masked_chunks():
+@pytest.mark.parametrize("H,G", [(32, 2), (7, 3)])                   # two passes; few heads: one pass by clusters
+def test_normalisers_of_masked_chunks(H, G):
     """All of a proxy row's mass is on the first key and on the window's keys of one residue (mod 8)."""
-    U, H, W, L = 8, len(C) // 2, 32, 320
-    q, k = np.zeros((U, 2 * H, W, D)), np.zeros((U, H, L, D))
-    q[..., 0], q[..., 1] = C[:, None] * ROOT, ROOT
+    U, W, L = 8, 32, 320
+    q, k = np.zeros((U, G * H, W, D)), np.zeros((U, H, L, D))
+    q[..., 0], q[..., 1] = C[:G * H, None] * ROOT, ROOT
     k[:, :, 1:, 1] = -60
     for u in range(U):
         k[u, :, L - W + u::8, 0], k[u, :, L - W + u::8, 1] = -1, 0
-    imp, _, g_imp, _ = _score(O.OracleParams(U, 2 * H, H, D, L, W, 1), _bf16(q), _bf16(k), np.zeros((U, L), np.uint8))
+    imp, _, g_imp, _ = _score(O.OracleParams(U, G * H, H, D, L, W, 1), _bf16(q), _bf16(k), np.zeros((U, L), np.uint8))
     on = imp > 1e-3
     assert on.sum() == U * H * 5 and np.abs(g_imp[on] / imp[on] - 1).max() < 1.2e-6
 
 
-@pytest.mark.parametrize("W", [32, 64, 128])
-def test_importances_from_a_window_of_both_modalities(W):
+@pytest.mark.parametrize("W,H,G", [(32, 32, 2), (64, 32, 2), (128, 32, 2), (32, 7, 3), (64, 7, 2), (128, 7, 1)])
+def test_importances_from_a_window_of_both_modalities(W, H, G):
     """Keys that the window's rows of one residue (mod 8) alone see; every word of 32 rows has both modalities."""
-    U, H, L = 8, len(C) // 2, 512
-    q, k = np.zeros((U, 2 * H, W, D)), np.zeros((U, H, L, D))
+    U, L = 8, 512
+    q, k = np.zeros((U, G * H, W, D)), np.zeros((U, H, L, D))
     q[..., 1] = ROOT
     q[..., 2] = ROOT
     for u in range(U):
-        q[u, :, u::8, 0], q[u, :, u::8, 2] = C[:, None] * ROOT, 0
+        q[u, :, u::8, 0], q[u, :, u::8, 2] = C[:G * H, None] * ROOT, 0
     k[:, :, 1:, 1] = -60
     k[:, :, 8:128:8, 0], k[:, :, 8:128:8, 1], k[:, :, 8:128:8, 2] = -1, 0, -60
     m = np.ascontiguousarray(np.broadcast_to(np.arange(L) // 16 % 2, (U, L)), dtype=np.uint8)
-    imp, _, g_imp, _ = _score(O.OracleParams(U, 2 * H, H, D, L, W, 1), _bf16(q), _bf16(k), m)
+    imp, _, g_imp, _ = _score(O.OracleParams(U, G * H, H, D, L, W, 1), _bf16(q), _bf16(k), m)
     assert np.abs(g_imp[:, :, 8:128:8] / imp[:, :, 8:128:8] - 1).max() < 1.2e-6
+
+
+@pytest.mark.parametrize("W,G", [(32, 3), (32, 4), (64, 2), (64, 3)])
+@pytest.mark.parametrize("H", [7, 32])                               # one pass by clusters; two passes
+def test_importances_in_front_of_the_window(W, G, H):
+    """Keys in front of the window in its tile of 128: one per chunk of 32, of residue u (mod 8), that all proxy rows see with one logit, against
+    one that has the chunk's maximum."""
+    U, L = 8, 256
+    q, k = np.zeros((U, H * G, W, D)), np.zeros((U, H, L, D))
+    q[..., 0], q[..., 1] = np.repeat(np.resize(C, U * H).reshape(U, H), G, 1)[:, :, None] * ROOT, ROOT
+    k[:, :, 1:, 1] = -60
+    for u in range(U):
+        k[u, :, 144 + u:L - W:32, 0] = -1
+        for first in (144 + u, 128 + (u + 4) % 8):
+            k[u, :, first:L - W:32, 1] = 0
+    imp, _, g_imp, _ = _score(O.OracleParams(U, H * G, H, D, L, W, 1), _bf16(q), _bf16(k), np.zeros((U, L), np.uint8))
+    for u in range(U):
+        ref, got = (x[u, :, 144 + u:L - W:32] / x[u, :, 128 + (u + 4) % 8:L - W:32] for x in (imp, g_imp))
+        assert ref.min() > 0.3 and np.abs(got / ref - 1).max() < 1.2e-6
 
 
 @pytest.mark.parametrize("few", [0, 1])
