@@ -1227,22 +1227,35 @@ flowmm_status validate_decode(const flowmm_decode_params *p) {
 struct DecodePlan {
     bool tc;                 // tensor-core kernel (bf16, head_dim 128) or the SIMT one
     int n_split, per_split;  // ranges per (unit, KV head); keys (SIMT) or 128-key tiles (tensor core) per range
-    size_t part_off, bytes;
+    size_t least;            // bytes of workspace below which the call is refused
 };
 
+constexpr size_t kDecodePartOff = 256;
 constexpr int kMaxDecodeCluster = dtc::kMaxRanges;         // ranges of a head that are joined as one cluster (the portable cluster size)
 
-// Records that are set aside for the ranges of all heads whatever the plan, so that a workspace for more keys or heads is never smaller: four
-// per SM, and for every head eight, or as many as its ranges of kMaxTiles are.  A head is cut into its share of them at most.
-int64_t decode_records(int uh, int tiles) {
-    const int longest = (tiles + dtc::kMaxTiles - 1) / dtc::kMaxTiles;
-    return std::min((int64_t)uh * tiles, std::max((int64_t)uh * std::max(kMaxDecodeCluster, longest), (int64_t)4 * kScoreCtas + uh));
+// Partial records of the ranges of all heads: `fewest`, as many as the longest tensor-core ranges make, without which a call is refused, and
+// `most`, that a workspace is asked to hold.  Both never fall when keys or heads are added, so that a workspace kept for the largest call serves
+// the smaller ones.  Ranges that a cluster joins write none, so a plan needs room for more than eight ranges of a head alone: of these up to
+// four per SM and one more per head (2560 heads of 1690 keys, 8 query heads each, 11 MB; eight records for every head were 85).  SIMT
+// ranges, of 64 keys and more: four per SM in whole numbers per head.
+struct DecodeRecords { int64_t fewest, most; };
+DecodeRecords decode_records(bool tensor_cores, int uh, int keys) {
+    constexpr int64_t few = 4 * kScoreCtas;
+    if (!tensor_cores) return {0, std::min((int64_t)uh * ((keys + 63) / 64), few + uh - 1)};
+    const int tiles = (keys + dtc::kTile - 1) / dtc::kTile;
+    const int64_t fewest = (int64_t)uh * ((tiles + dtc::kMaxTiles - 1) / dtc::kMaxTiles);
+    return {fewest, std::max(fewest, std::min((int64_t)uh * tiles, few + std::min<int64_t>(uh, few / kMaxDecodeCluster)))};
+}
+size_t decode_bytes(const flowmm_decode_params &p, int64_t records) {
+    return kDecodePartOff + align256((size_t)records * (p.n_q_heads / p.n_kv_heads) * (p.head_dim + 2) * sizeof(float));
 }
 
-DecodePlan decode_plan(const flowmm_decode_params &p) {
+bool decode_use_tc(const flowmm_decode_params &p) { return p.dtype == FLOWMM_BF16 && p.head_dim == 128 && p.path != FLOWMM_PATH_SIMT; }
+
+DecodePlan decode_plan(const flowmm_decode_params &p, size_t ws_bytes) {
     DecodePlan d;
-    const int uh = p.n_units * p.n_kv_heads, g = p.n_q_heads / p.n_kv_heads;
-    d.tc = p.dtype == FLOWMM_BF16 && p.head_dim == 128 && p.path != FLOWMM_PATH_SIMT;
+    const int uh = p.n_units * p.n_kv_heads;
+    d.tc = decode_use_tc(p);
     if (d.tc) {
         // Two CTAs share an SM.  Of the range lengths TMEM allows, the one whose call is the shortest by this account, in us: all tiles of K
         // and V at the memory's rate, or the one CTA's, 0.9 a tile, where that is longer; when the CTAs do not fit at once, 1 per further
@@ -1250,14 +1263,19 @@ DecodePlan decode_plan(const flowmm_decode_params &p) {
         // its own.  Clusters find room for 0.88 of the CTAs (96 of three, 12 tiles each, ran two after the other: 47 us, by five of 7 tiles
         // 40).  Measured with every length on 18 shapes, 16 to 554 MB of 4 to 1024 heads: 1 % on average, 10 % at most above the best
         // length (4 and 18 % by rounds of CTAs times their tiles and a fixed cost each).
-        const int tiles = (p.n_keys + dtc::kTile - 1) / dtc::kTile, most = (int)(decode_records(uh, tiles) / uh);
+        // (A smaller workspace than is asked for has room for fewer ranges.)
+        const int tiles = (p.n_keys + dtc::kTile - 1) / dtc::kTile;
+        const DecodeRecords records = decode_records(true, uh, p.n_keys);
+        d.least = decode_bytes(p, records.fewest);
+        const bool all_fit = ws_bytes >= decode_bytes(p, records.most);
         double best = 0.0;
         d.per_split = 0;
         for (int per = 1; per <= dtc::kMaxTiles && per <= tiles; ++per) {
             const int splits = (tiles + per - 1) / per;
-            if (splits > most) continue;
             const bool cluster = splits > 1 && splits <= kMaxDecodeCluster;
-            const double slots = 2.0 * kScoreCtas * (cluster ? 0.88 : 1.0), ctas = (double)uh * splits, rounds = ctas / slots;
+            const int64_t n = (int64_t)uh * splits;
+            if (splits > kMaxDecodeCluster && n != records.fewest && (n > records.most || (!all_fit && decode_bytes(p, n) > ws_bytes))) continue;
+            const double slots = 2.0 * kScoreCtas * (cluster ? 0.88 : 1.0), ctas = (double)n, rounds = ctas / slots;
             const double tile_us = 0.00985, all = uh * (double)tiles * tile_us, lone = 0.9 * per;
             double cost = all > lone ? all : lone;
             if (rounds > 1.0) {
@@ -1271,15 +1289,13 @@ DecodePlan decode_plan(const flowmm_decode_params &p) {
     }
     if (!d.tc) {
         // enough CTAs for about four per SM, at least 64 keys each
-        int want = (4 * 148 + uh - 1) / uh;
+        int want = (4 * kScoreCtas + uh - 1) / uh;
         const int max_split = (p.n_keys + 63) / 64;
         want = want < 1 ? 1 : (want > max_split ? max_split : want);
         d.per_split = (p.n_keys + want - 1) / want;
         d.n_split = (p.n_keys + d.per_split - 1) / d.per_split;
+        d.least = decode_bytes(p, (int64_t)uh * d.n_split);
     }
-    d.part_off = 256;
-    const size_t n_rec = d.tc ? (size_t)decode_records(uh, (p.n_keys + dtc::kTile - 1) / dtc::kTile) : (size_t)uh * d.n_split;
-    d.bytes = d.part_off + align256(n_rec * g * (p.head_dim + 2) * sizeof(float));
     return d;
 }
 
@@ -1342,7 +1358,7 @@ flowmm_status launch_decode_tc(const flowmm_decode_params &p, const DecodeArgs &
 extern "C" flowmm_status flowmm_decode_workspace_bytes(const flowmm_decode_params *p, size_t *bytes) {
     if (!bytes) return FLOWMM_ERR_NULL;
     FLOWMM_TRY(validate_decode(p));
-    *bytes = decode_plan(*p).bytes;
+    *bytes = decode_bytes(*p, decode_records(decode_use_tc(*p), p->n_units * p->n_kv_heads, p->n_keys).most);
     return FLOWMM_OK;
 }
 
@@ -1356,12 +1372,12 @@ extern "C" flowmm_status flowmm_decode_attention(const flowmm_decode_params *p, 
     if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !strides_ok(p->k_stride, p->head_dim) ||
         !strides_ok(p->v_stride, p->head_dim) || (reinterpret_cast<uintptr_t>(ws) & 255))
         return FLOWMM_ERR_ALIGN;
-    const DecodePlan plan = decode_plan(*p);
-    if (ws_bytes < plan.bytes) return FLOWMM_ERR_WORKSPACE;
+    const DecodePlan plan = decode_plan(*p, ws_bytes);
+    if (ws_bytes < plan.least) return FLOWMM_ERR_WORKSPACE;
     FLOWMM_TRY(check_device());
     DecodeArgs a;
     a.status = static_cast<int *>(ws);                               // (cleared by the kernel)
-    a.q = q; a.k = k; a.v = v; a.part = reinterpret_cast<float *>(static_cast<char *>(ws) + plan.part_off); a.out = out;
+    a.q = q; a.k = k; a.v = v; a.part = reinterpret_cast<float *>(static_cast<char *>(ws) + kDecodePartOff); a.out = out;
     a.Hq = p->n_q_heads; a.Hkv = p->n_kv_heads; a.G = p->n_q_heads / p->n_kv_heads; a.N = p->n_keys;
     a.n_split = plan.n_split; a.keys_per_split = plan.per_split;
     const float scale = p->softmax_scale != 0.f ? p->softmax_scale : 1.f / sqrtf((float)p->head_dim);

@@ -76,3 +76,22 @@ def test_workspace_never_shrinks_with_the_problem(lib, Hkv, G, W, D, dtype):
     for L, B in ((200, 50), (640, 64), (2176, 217), (33792, 1690)):
         sizes = [size(U, L, B) for U in range(1, 320)]
         assert sizes == sorted(sizes), (L, B)
+
+
+@pytest.mark.parametrize("D,dtype", [(128, F.BF16), (64, F.BF16), (128, F.F32)])
+def test_decode_workspace_never_shrinks_and_stays_small(lib, D, dtype):
+    """More keys or heads never ask for less; a head is given room for eight records, or as many as its ranges of 1920 keys, only
+    while four ranges per SM of a B200 come to that many."""
+    def size(uh, keys, G):
+        n, cp = ctypes.c_size_t(0), F._CDecodeParams(uh, G, 1, D, keys, dtype, 0.0, F.PATH_AUTO)
+        assert lib.flowmm_decode_workspace_bytes(ctypes.byref(cp), ctypes.byref(n)) == 0
+        return n.value
+    for uh in (1, 4, 33, 74, 75, 296, 591, 592, 2560):
+        sizes = [size(uh, keys, 4) for keys in sorted(set(range(1, 40000, 61)) | set(range(37880, 37900)) | set(range(15300, 15400)))]
+        assert sizes == sorted(sizes), uh
+    for keys in (1, 128, 129, 1690, 15361, 33792):
+        sizes = [size(uh, keys, 4) for uh in range(1, 1300)]
+        assert sizes == sorted(sizes), keys
+    for uh, keys, G in ((2560, 1690, 8), (296, 1690, 8), (8, 33792, 8), (1, 100, 1)):
+        ranges = -(-keys // 1920)
+        assert size(uh, keys, G) <= 512 + max(uh * ranges, 592 + (min(uh, 74) if (D, dtype) == (128, F.BF16) else uh)) * G * (D + 2) * 4

@@ -131,3 +131,26 @@ def test_one_range_cluster_and_combine(U, Hq, Hkv, N):
         assert F.flowmm_last_device_status(ws) == 0
         got = out.cpu().numpy().astype(np.float64)
         assert np.allclose(got, ref, rtol=RTOL, atol=ATOL), np.abs(got - ref).max()
+
+
+@pytest.mark.parametrize("U,Hq,Hkv,N", [(1, 28, 4, 15361), (1, 8, 1, 33792), (2, 16, 2, 20000), (1, 8, 1, 1690)])
+def test_workspace_of_the_fewest_ranges(U, Hq, Hkv, N):
+    """A workspace with room for ranges of 1920 keys is enough, whatever is asked for; nothing behind it is written.  Without that room the
+    call is refused."""
+    gen = torch.Generator(device="cuda").manual_seed(N)
+    q = torch.randn((U, Hq, 128), generator=gen, device="cuda").bfloat16()
+    k, v = (torch.randn((U, Hkv, N, 128), generator=gen, device="cuda").bfloat16() for _ in range(2))
+    least = 256 + -(-(U * Hq * -(-N // 1920) * 130 * 4) // 256) * 256
+    full = F.flowmm_decode_workspace_bytes(q, k, v)
+    assert least <= full
+    outs = []
+    for n in (full, least):
+        buf = torch.full((n + 4096,), 77, dtype=torch.uint8, device="cuda")
+        out = torch.full((U, Hq, 128), float("nan"), device="cuda")
+        F.flowmm_decode_attention(q, k, v, out, buf[:n])
+        assert F.flowmm_last_device_status(buf) == 0 and bool((buf[n:] == 77).all())
+        outs.append(out.double().cpu().numpy())
+        with pytest.raises(F.FlowmmError) as e:
+            F.flowmm_decode_attention(q, k, v, out, buf[:least - 256])
+        assert e.value.code == 5
+    assert np.allclose(outs[0], outs[1], rtol=RTOL, atol=ATOL)
