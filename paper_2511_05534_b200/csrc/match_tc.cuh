@@ -108,11 +108,12 @@ __device__ __forceinline__ void match_gather_rows(const MatchPrepArgs &A, int uh
     }
 }
 
-// The candidate layout of one head from its pivot list, by a whole block (`scratch`: 33 ints of shared memory).  A thread takes eight
-// pivots in a row, whose loads are on their way together; one prefix sum numbers the candidates of both groups.  (The steps one by one,
-// 8 heads of 33 792 tokens with 1690 pivots: 235.8 -> 228.6 us, where rounds of a pivot per thread loaded twice and summed each time.)
-__device__ __forceinline__ void match_lay_out_candidates(const MatchPrepArgs &A, int uh, int *scratch) {
-    constexpr int kPer = 8;
+// The candidate layout of one head from its pivot list, by a whole block (`scratch`: 33 ints of shared memory).  A thread takes kPer
+// pivots in a row, whose loads are on their way together; one prefix sum numbers the candidates of both groups.  One pivot while the block
+// has a thread for each, else eight: the steps one by one, 8 heads of 33 792 tokens with 1690 pivots, 235.8 -> 228.6 us, where rounds of a
+// pivot per thread loaded twice and summed each time; flowmm_match of 56 heads of 1200 tokens with 120 pivots by eight 14.2, by one 12.4.
+template <int kPer>
+__device__ __forceinline__ void match_number_candidates(const MatchPrepArgs &A, int uh, int *scratch) {
     const int tid = threadIdx.x, u = uh / A.Hkv, chunk = kPer * blockDim.x;
     const int *ret = A.retained + (int64_t)uh * A.B;
     const float *imp = A.importance + (int64_t)uh * A.L;
@@ -172,8 +173,13 @@ __device__ __forceinline__ void match_lay_out_candidates(const MatchPrepArgs &A,
         seen_v += tot >> 16;
     }
     if (tid == 0) { A.cand_count[2 * uh] = seen_t; A.cand_count[2 * uh + 1] = seen_v; }
+}
+
+__device__ __forceinline__ void match_lay_out_candidates(const MatchPrepArgs &A, int uh, int *scratch) {
+    if (A.B <= (int)blockDim.x) match_number_candidates<1>(A, uh, scratch);
+    else match_number_candidates<8>(A, uh, scratch);
     __syncthreads();
-    if (A.copy_here) match_gather_rows<4>(A, uh, nullptr, 0, A.Ctot, tid, blockDim.x);
+    if (A.copy_here) match_gather_rows<4>(A, uh, nullptr, 0, A.Ctot, threadIdx.x, blockDim.x);
 }
 
 // The preparation of flowmm_match, which is handed the index lists (inside flowmm_compress_layer and flowmm_recompress the

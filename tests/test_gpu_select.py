@@ -81,7 +81,8 @@ def test_select_by_clusters_and_by_blocks(L, B, U, kind):
     assert np.array_equal(e.cpu().numpy(), ref_e)
 
 
-@pytest.mark.parametrize("L,B", [(290, 193), (7000, 130), (9000, 700), (2000, 225), (46000, 300), (6000, 4096), (6000, 4097), (12000, 9000)])
+@pytest.mark.parametrize("L,B", [(290, 193), (7000, 130), (9000, 700), (2000, 225), (46000, 300), (6000, 4096), (6000, 4097), (12000, 9000),
+                                 (3000, 512), (3000, 513)])
 def test_fused_preparation_equals_the_steps(L, B):
     """The candidate layout written by the selection launch of flowmm_compress_layer against the one flowmm_match makes
     from the lists: same matches, bit for bit (short lists, long lists, a context of more than one chunk)."""
