@@ -176,7 +176,7 @@ match_small_tc_kernel(const __grid_constant__ CUtensorMap k_map, const __grid_co
     tc::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     predecessor_done();
-    successor_may_start();
+    if (A.tokmap) successor_may_start();   // (the merge, a block per SM; the small blocks that come behind the step alone: 56 heads of 1200, 10.6 -> 12.4)
 
     // every role walks the heads of the run: tiles [t_lo, t_hi) of head uh, hc heads before it, tile number i of the run
     if (warp == 0) {
