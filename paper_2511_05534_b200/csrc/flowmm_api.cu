@@ -570,6 +570,8 @@ flowmm_status launch_select(const SelectArgs &a, const SelectFlow &f, const Matc
 // flow != nullptr: the launch also applies Eq. 6 and the theta rule (SelectFlow's comments).
 // prep != nullptr: each block goes on to prepare its head's matching candidates (tensor-core matching).
 // row_mod, row_mod_out: the pivots' modalities are written as well, from one modality map per head.
+bool use_match_merge(const flowmm_params &p);
+
 flowmm_status run_select(const flowmm_params &p, const float *importance, int32_t *retained, int32_t *evicted,
                          cudaStream_t st, const SelectFlow *flow = nullptr, const MatchPrepArgs *prep = nullptr,
                          const uint8_t *row_mod = nullptr, uint8_t *row_mod_out = nullptr) {
@@ -578,9 +580,13 @@ flowmm_status run_select(const flowmm_params &p, const float *importance, int32_
     a.n_heads = p.n_units * p.n_kv_heads; a.L = p.seq_len; a.B = p.n_keep; a.W = p.window; a.keep_window = p.keep_window;
     a.chunk = p.seq_len <= kSelMaxChunk ? (p.seq_len + 31) / 32 * 32 : kSelMaxChunk;
     const SelectFlow no_flow = {};
-    // (few heads, 112 of 2176 tokens would be 2 % slower, and one block per SM behind them, not the small blocks that gather long candidate
-    // lists)
-    a.lets_in = prep && prep->copy_here && 3 * (a.n_heads + p.n_units) <= 2 * tc::sm_count();
+    // Heads that leave SMs free, the short-list matching behind them (a block per SM; not the small blocks that gather long lists) and up to
+    // five tiles of 128 tokens per SM for it.  The whole call, with and without: 32 heads of 640 tokens 23.1, 23.5 us; 16 of 2000 36.1, 36.4, with
+    // 7 query heads each 41.6, 42.4; but 4 of 400 23.3, 22.4; 72 of 1500 49.3, 45.9; 52 of 2500 54.4, 51.5; 40 of 3500 61.5, 58.6; with the
+    // matching and the merge in one launch 76 of 640 25.0, 23.6, of 2600 66.7, 62.8.
+    const int64_t tiles = (int64_t)a.n_heads * ((p.seq_len + mst::kTile - 1) / mst::kTile);
+    a.lets_in = prep && prep->copy_here && !use_match_merge(p) && a.n_heads >= 8 && 3 * (a.n_heads + p.n_units) <= 2 * tc::sm_count() &&
+                tiles <= 5 * tc::sm_count();
     MatchPrepArgs g = {};
     g.Hkv = 1; g.modality = row_mod;
     if (prep) g = *prep;
