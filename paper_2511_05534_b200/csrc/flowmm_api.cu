@@ -687,10 +687,11 @@ flowmm_status run_match(const flowmm_params &p, const Layout &y, const void *k, 
     a.Hkv = p.n_kv_heads; a.D = p.head_dim; a.L = p.seq_len; a.B = p.n_keep; a.E = E;
     a.tau_eff = tau_effective(p);
     for (int i = 0; i < 3; ++i) a.ks[i] = p.k_stride[i];
-    // A row per thread where blocks of 16 rows still find room together, four of them to an SM: a block's products then take a quarter of the
-    // time.  fp32, the whole call: 4 heads of 600 tokens and 32 proxy rows, where only this changes, 30.0 -> 27.0 us.
+    // A row per thread where all blocks of 16 rows get an SM: a block's products then take a quarter of the time, but every block goes through
+    // all pivots' rows.  fp32, head_dim 64, us, by 64 rows and by 16: 4 heads of 400 rows and 150 pivots 18.0, 12.3; 1 of 1200 and 300 24.9, 19.0;
+    // with 1 to 1.3 blocks per SM 2 heads of 1200 and 150 15.9, 16.9, 4 of 600 and 300 28.8, 26.8; with 2 8 of 600 and 150 16.0, 21.8.
     const int UH = p.n_units * p.n_kv_heads;
-    const bool one_row = (int64_t)UH * ((E + 15) / 16) <= 4 * tc::sm_count();
+    const bool one_row = (int64_t)UH * ((E + 15) / 16) <= tc::sm_count();
     const dim3 grid(UH, one_row ? (E + 15) / 16 : (E + kTile - 1) / kTile);
     auto kernel = p.dtype == FLOWMM_BF16 ? (one_row ? match_simt<__nv_bfloat16, 1> : match_simt<__nv_bfloat16, 4>)
                                          : (one_row ? match_simt<float, 1> : match_simt<float, 4>);
