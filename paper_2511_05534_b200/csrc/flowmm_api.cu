@@ -189,13 +189,15 @@ Layout make_layout(const flowmm_params &p) {
     // idle and items of one half still have an SM each, they are of one half: their products and exponentials then take half as
     // long.  The whole call, us, 256 and 128: 8 heads of 1471 tokens, 224 rows 34.8, 32.8; 4 of 500 30.6, 28.1; 4 of 2300 45.1, 43.4;
     // 4 of 4500 51.8, 50.1; 8 of 1000, 512 rows 35.7, 32.8; 4 caches of 640 rows 37.2, 34.8; where pass 2 alone is cut finer 8 of
-    // 2300 42.2, 41.1.  With more items than SMs the second round costs what the finer cut gains.
+    // 2300 42.2, 41.1.
     y.tc_q_rows = G * W > tcs::kRows && U * Hkv * (size_t)y.n_rt * ((G * W + tcs::kRows - 1) / tcs::kRows) <= kScoreCtas ? tcs::kRows : tcs::kItemRows;
-    // Pass 2 by items of 128 as well, on which all warps of a CTA work, where the longest run of items of 256 is a good deal more than the longest
-    // of 128: heads that end in half an item, few items per CTA (112 caches of 640 rows, 448 proxy rows: the call 77.7 -> 75.9 us).
+    // Pass 2 by items of 128 as well, on which all warps of a CTA work, where the longest run of them is at most two thirds of the longest of
+    // items of 256: heads that end in half an item, few items per CTA.  The scoring, us, by 256 and by 128, 224 rows: runs of half the length
+    // 56 heads of 640 tokens 21.7, 20.1, 96 of 300 21.0, 19.6; of two thirds 112 of 640 26.9, 25.7, 64 of 1150 27.0, 25.6, 168 of 300 25.5, 25.5; of
+    // three quarters 16 of 2312 21.6, 23.2, 40 of 900 20.9, 21.8, 64 of 1664 29.8, 31.6, 32 of 1400 21.7, 21.6, 24 of 2000 24.0, 23.5.
     const size_t halves2 = U * Hkv * ((L + tcs::kRows - 1) / tcs::kRows), items2 = U * Hkv * (size_t)y.n_rt;
     const size_t run_items = (items2 + kScoreCtas - 1) / kScoreCtas, run_halves = (halves2 + kScoreCtas - 1) / kScoreCtas;
-    y.tc_keys2 = halves2 <= kScoreCtas || 50 * run_halves * items2 <= 41 * run_items * halves2 ? tcs::kRows : tcs::kItemRows;
+    y.tc_keys2 = halves2 <= kScoreCtas || 3 * run_halves <= 4 * run_items ? tcs::kRows : tcs::kItemRows;
     // pass 1 of the tensor-core scoring: the key tiles of all heads in equal runs, one per SM and tile of proxy rows
     y.tc_n_qt = (int)((G * W + y.tc_q_rows - 1) / y.tc_q_rows);
     {
@@ -567,11 +569,11 @@ flowmm_status launch_select(const SelectArgs &a, const SelectFlow &f, const Matc
     return FLOWMM_OK;
 }
 
+bool use_match_merge(const flowmm_params &p);
+
 // flow != nullptr: the launch also applies Eq. 6 and the theta rule (SelectFlow's comments).
 // prep != nullptr: each block goes on to prepare its head's matching candidates (tensor-core matching).
 // row_mod, row_mod_out: the pivots' modalities are written as well, from one modality map per head.
-bool use_match_merge(const flowmm_params &p);
-
 flowmm_status run_select(const flowmm_params &p, const float *importance, int32_t *retained, int32_t *evicted,
                          cudaStream_t st, const SelectFlow *flow = nullptr, const MatchPrepArgs *prep = nullptr,
                          const uint8_t *row_mod = nullptr, uint8_t *row_mod_out = nullptr) {
