@@ -429,17 +429,41 @@ flowmm_status run_score_fused(const flowmm_params &p, const Layout &y, const voi
     return FLOWMM_OK;
 }
 
-// One pass by clusters (score_cluster_tc.cuh) where all of its CTAs run at once: a cluster's CTAs take 9 us one after the other what the two
-// passes take side by side (112 heads of 640 tokens, 448 rows, whole call 77.9 us by two passes, 96.8 by clusters; 16 of 1471 36.8, 33.5).
-// Few proxy rows would leave lanes without one (32 heads of 2000 tokens, 32 rows, 45.2, 51.8).  Key tiles per CTA: the fewest that fit;
-// returns the CTAs per head (0: not so).
-constexpr int kClusterScoreCtas = 112;
+// Clusters of `ctas` CTAs of the one-pass scoring that run at once on the current device, an SM for each CTA (score_cluster_tc.cuh asks for too
+// much shared memory for two).  A cluster's CTAs are in one group of SMs, so by fours 132 of 148 find room, by sevens 105.  Asked for once per
+// device and size (a benign race: every thread would store the same value).
+int score_clusters_at_once(int ctas) {
+    constexpr int kSlots = 64;
+    static std::atomic<int> known[kSlots][sct::kMaxCtas + 1];            // one more than the answer; 0: not asked for yet
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+    if (dev < kSlots && (n = known[dev][ctas].load(std::memory_order_relaxed)) != 0) return n - 1;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = ctas; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(sct::kThreads); cfg.dynamicSmemBytes = sct::kMinSmem; cfg.attrs = &attr; cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(sct::score_cluster_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sct::kMinSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, sct::score_cluster_tc_kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    if (dev < kSlots) known[dev][ctas].store(n + 1, std::memory_order_relaxed);
+    return n;
+}
+
+// One pass by clusters (score_cluster_tc.cuh) where all of them run at once: a cluster's CTAs take 9 us one after the other what the two passes
+// take side by side.  The scoring, us, by two passes and so: 20 heads of 709 tokens, 128 rows, by sixes 12.0, 9.1; 28 of 986, 224 rows, by
+// fours 15.9, 12.4; where some clusters come second 16 of 791, 128 rows, by sevens 11.9, 14.9; 48 of 306, 96 rows, by threes 11.9, 13.6.
+// Few proxy rows would leave lanes without one (32 heads of 2000 tokens, 32 rows, whole call 45.2, 51.8).  Key tiles per CTA: the fewest that
+// fit; returns the CTAs per head (0: not so).
 int cluster_score_split(const flowmm_params &p, int &kt) {
     const int gw = p.n_q_heads / p.n_kv_heads * p.window, rt = (gw + sct::kTile - 1) / sct::kTile, nt = (p.seq_len + sct::kTile - 1) / sct::kTile;
-    if (!use_tc_score(p) || gw < 96 || rt > sct::kMaxAcc) return 0;
+    const int64_t heads = (int64_t)p.n_units * p.n_kv_heads;
+    if (!use_tc_score(p) || gw < 96 || rt > sct::kMaxAcc || heads > kScoreCtas) return 0;
     for (kt = 1; rt * kt <= sct::kMaxAcc; kt *= 2) {
         const int ctas = (nt + kt - 1) / kt;
-        if (ctas <= sct::kMaxCtas && (int64_t)p.n_units * p.n_kv_heads * ctas <= kClusterScoreCtas) return ctas;
+        if (ctas <= sct::kMaxCtas && heads <= score_clusters_at_once(ctas)) return ctas;
     }
     return 0;
 }

@@ -115,10 +115,11 @@ def test_sums_over_many_proxy_rows():
 
 @pytest.mark.parametrize("pattern", ["random", "run_in_word", "window_of_both"])
 @pytest.mark.parametrize("G,W,L", [(3, 32, 97), (4, 32, 1024), (4, 32, 1025), (4, 32, 4096), (4, 32, 4097), (7, 32, 1471), (8, 32, 2048), (8, 32, 2049),
-                                   (3, 128, 256), (7, 64, 641), (8, 64, 1024), (8, 64, 1025)])
+                                   (3, 128, 256), (7, 64, 641), (8, 64, 1024), (8, 64, 1025), (4, 32, 791)])
 def test_few_heads_and_many_of_the_same(G, W, L, pattern):
     """One unit, whose heads are shared by clusters of one to eight CTAs of one, two or four key tiles (up to the longest prompt that
-    one to four tiles of proxy rows leave room for), and sixty times that unit, which takes the two passes."""
+    one to four tiles of proxy rows leave room for); eight of it, for which some sizes of clusters do not find room; and sixty and eighty
+    times that unit, which take the two passes (sixty with more than one CTA to a head)."""
     rng = np.random.default_rng(L + G)
     modality = PATTERNS[pattern](rng, L)[None]
     p = O.OracleParams(1, 2 * G, 2, 128, L, W, 1)
@@ -126,7 +127,7 @@ def test_few_heads_and_many_of_the_same(G, W, L, pattern):
     m = np.ascontiguousarray(modality, dtype=np.uint8)
     imp, cross, _ = O.score(p, q, k, m)
     qd, kd, md = to_dev(q, F.BF16), to_dev(k, F.BF16), torch.from_numpy(m).cuda()
-    for U in (1, 60):
+    for U in (1, 8, 60, 80):
         fp = F.Params(U, 2 * G, 2, 128, L, W, 1)
         g_imp, g_cross = torch.full((U, 2, L), float("nan"), device="cuda"), torch.full((U, 2 * G), float("nan"), device="cuda")
         ws = F.alloc_workspace(fp)
