@@ -455,13 +455,14 @@ int score_clusters_at_once(int ctas) {
 // One pass by clusters (score_cluster_tc.cuh) where all of them run at once: a cluster's CTAs take 9 us one after the other what the two passes
 // take side by side.  The scoring, us, by two passes and so: 20 heads of 709 tokens, 128 rows, by sixes 12.0, 9.1; 28 of 986, 224 rows, by
 // fours 15.9, 12.4; where some clusters come second 16 of 791, 128 rows, by sevens 11.9, 14.9; 48 of 306, 96 rows, by threes 11.9, 13.6.
-// Few proxy rows would leave lanes without one (32 heads of 2000 tokens, 32 rows, whole call 45.2, 51.8).  Key tiles per CTA: the fewest that
-// fit; returns the CTAs per head (0: not so).
+// Rows short of a tile leave lanes without one.  64 rows: 4 heads of 640 tokens 11.3, 8.6, 28 of 2000 17.6, 12.9; by four key tiles to a CTA, beyond
+// 2048 tokens, 4 of 3000 11.9, 12.4, so not there.  32 rows: 4 of 1500 11.0, 9.5, of 3000 11.5, 11.7, 32 of 2000, whole call, 45.2, 51.8.  Key tiles
+// per CTA: the fewest that fit; returns the CTAs per head (0: not so).
 int cluster_score_split(const flowmm_params &p, int &kt) {
     const int gw = p.n_q_heads / p.n_kv_heads * p.window, rt = (gw + sct::kTile - 1) / sct::kTile, nt = (p.seq_len + sct::kTile - 1) / sct::kTile;
     const int64_t heads = (int64_t)p.n_units * p.n_kv_heads;
-    if (!use_tc_score(p) || gw < 96 || rt > sct::kMaxAcc || heads > kScoreCtas) return 0;
-    for (kt = 1; rt * kt <= sct::kMaxAcc; kt *= 2) {
+    if (!use_tc_score(p) || gw < 64 || rt > sct::kMaxAcc || heads > kScoreCtas) return 0;
+    for (kt = 1; rt * kt <= sct::kMaxAcc && (gw >= 96 || kt <= 2); kt *= 2) {
         const int ctas = (nt + kt - 1) / kt;
         if (ctas <= sct::kMaxCtas && heads <= score_clusters_at_once(ctas)) return ctas;
     }

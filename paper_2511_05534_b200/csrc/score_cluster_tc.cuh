@@ -1,4 +1,4 @@
-// Window scoring (Eq. 8 with the softmax of Eq. 4, and the masses of Eq. 7) in one pass over K for contexts of a few key tiles and up to
+// Window scoring (Eq. 8 with the softmax of Eq. 4, and the masses of Eq. 7) in one pass over K for contexts of a few key tiles and 64 to
 // 512 proxy rows per KV head (bf16, head_dim 128): the CTAs of a cluster share a head's keys, every logit of a CTA's keys stays in its
 // TMEM, and only the rows' statistics are exchanged.
 //

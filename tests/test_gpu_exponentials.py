@@ -84,7 +84,7 @@ def test_importances_from_a_window_of_both_modalities(W, H, G):
     assert np.abs(g_imp[:, :, 8:128:8] / imp[:, :, 8:128:8] - 1).max() < 1.2e-6
 
 
-@pytest.mark.parametrize("W,G", [(32, 3), (32, 4), (64, 2), (64, 3)])
+@pytest.mark.parametrize("W,G", [(32, 2), (32, 3), (32, 4), (64, 1), (64, 2), (64, 3)])
 @pytest.mark.parametrize("H", [7, 32])                               # one pass by clusters; two passes
 def test_importances_in_front_of_the_window(W, G, H):
     """Keys in front of the window in its tile of 128: one per chunk of 32, of residue u (mod 8), that all proxy rows see with one logit, against

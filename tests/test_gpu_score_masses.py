@@ -115,7 +115,8 @@ def test_sums_over_many_proxy_rows():
 
 @pytest.mark.parametrize("pattern", ["random", "run_in_word", "window_of_both"])
 @pytest.mark.parametrize("G,W,L", [(3, 32, 97), (4, 32, 1024), (4, 32, 1025), (4, 32, 4096), (4, 32, 4097), (7, 32, 1471), (8, 32, 2048), (8, 32, 2049),
-                                   (3, 128, 256), (7, 64, 641), (8, 64, 1024), (8, 64, 1025), (4, 32, 791)])
+                                   (3, 128, 256), (7, 64, 641), (8, 64, 1024), (8, 64, 1025), (4, 32, 791),
+                                   (2, 32, 97), (2, 32, 2048), (2, 32, 2049), (1, 64, 641)])
 def test_few_heads_and_many_of_the_same(G, W, L, pattern):
     """One unit, whose heads are shared by clusters of one to eight CTAs of one, two or four key tiles (up to the longest prompt that
     one to four tiles of proxy rows leave room for); eight of it, for which some sizes of clusters do not find room; and sixty and eighty
