@@ -226,10 +226,10 @@ __host__ __device__ constexpr size_t csr_count_smem(int E, int B, int n_warps) {
     const size_t Ep = ((size_t)E + 7) & ~(size_t)7, Lp = ((size_t)E + B + 7) & ~(size_t)7, cnt = (size_t)n_warps * (((size_t)B + 2) & ~(size_t)1) * 2;
     return 2 * Lp + 4 * (((size_t)B + 4) & ~(size_t)3) + (4 * Ep > cnt ? 4 * Ep : cnt) + 16;
 }
-// (Two blocks of 32 warps to an SM, of 32 registers, or five of 8 warps, of 48: 284 heads of 9000 tokens with 37 registers 104.9 us for the step, so
-// 97.0; 576 heads of 4300 with 80 117.5, so 107.7.)
+// (Two blocks of 32 warps to an SM, of 32 registers: 284 heads of 9000 tokens with 37 registers 104.9 us for the step, so 97.0.  Blocks of 8 warps
+// are left to the compiler's 48 registers: with 80 registers 576 heads of 4300 117.5 us instead of 107.7; held to 48, it spills.)
 template <int NW>
-__global__ void __launch_bounds__(32 * NW, NW == 32 ? 2 : 5) build_csr_count_kernel(const CsrArgs A, int n_bits) {
+__global__ void __launch_bounds__(32 * NW, NW == 32 ? 2 : 0) build_csr_count_kernel(const CsrArgs A, int n_bits) {
     constexpr int kThreads = 32 * NW, kBatch = 8;
     extern __shared__ __align__(16) uint8_t csr_raw[];
     __shared__ int scratch[33];
