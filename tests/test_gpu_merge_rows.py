@@ -31,6 +31,17 @@ def _members(pattern, B, rng):
     return n
 
 
+def _window(heads, L, B):
+    """Rows of a window, and whether the pieces of long slots are items of their own, by the library's rule: the shortest windows by which
+    each of 3552 warps has one window or piece at most."""
+    parts = 2 * ((L - B) // 64) + 2
+    if heads * L >= 1300000:
+        return 64, False
+    win = 16 if heads * L < 40000 else next(w for w in range(16, 36, 4) if w == 32 or (
+        w * B >= 2 * L and heads * (-(-L // w) + (parts if L - B > B else 0)) <= 3552))
+    return win, heads * (-(-L // win) + parts) <= 2 * 3552
+
+
 def _lists(rng, B, E, counts):
     """Pivots, non-pivots and matches of heads whose slots have these numbers of members, [variants, .]; what is left of E is dropped."""
     L = B + E
@@ -81,20 +92,22 @@ def test_slots_of_chosen_sizes(pattern, U, H, dtype, D):
     B = 700
     counts = [_members(pattern, B, rng) for _ in range(min(U * H, 7))]
     E = max(int(n.sum()) for n in counts) + 150
-    assert E > 1024 and (U * H == 1 or U * H * (E + B) >= 40000)    # (no short list)
+    assert E > 1024                                                 # (no short list)
+    assert _window(U * H, E + B, B) == {1: (16, True), 20: (24 if pattern == "alternate" else 32, True), 90: (32, False)}[U * H]
     for mode in (F.MERGE_MEAN, F.MERGE_EXPSIM):
         _check_merge(rng, U, H, B, E, D, dtype, mode, counts)
 
 
-@pytest.mark.parametrize("H,win", [(16, 20), (20, 24), (23, 28)])
+@pytest.mark.parametrize("H,B,win", [(16, 700, 32), (20, 700, 32), (23, 700, 32), (11, 700, 20), (12, 700, 24), (14, 700, 28), (16, 2000, 20), (20, 2000, 24),
+                                     (23, 2000, 28), (12, 250, 32)])
 @pytest.mark.parametrize("dtype,D", [(F.BF16, 128), (F.F32, 64)])
-def test_windows_in_between(H, win, dtype, D):
-    """Windows of 20, 24 and 28 rows: the shortest that give each of 3552 warps one at most."""
+def test_windows_in_between(H, B, win, dtype, D):
+    """Windows of 20, 24 and 28 rows: the shortest that give each of 3552 warps one at most, with the possible pieces of long slots where slots
+    have more than one member on average; and few slots, where windows are not shorter than two of them."""
     rng = np.random.default_rng(H + D)
-    B = 700
-    counts = [_members(p, B, rng) for p in ("edges_apart", "edges_last", "alternate")]
+    counts = [_members(p, B, rng) for p in (("edges_apart", "edges_last", "alternate") if B < 2000 else ("alternate",))]
     E = 4000 - B
-    assert min(w for w in range(16, 36, 4) if H * -(-4000 // w) <= 3552) == win and max(n.sum() for n in counts) < E
+    assert _window(H, 4000, B) == (win, True) and max(n.sum() for n in counts) < E
     _check_merge(rng, 1, H, B, E, D, dtype, F.MERGE_EXPSIM, counts)
 
 
