@@ -35,9 +35,16 @@ inline bool make_bf16_map(CUtensorMap *map, const void *base, int rank, const ui
     cuuint32_t box[5], estr[5];
     for (int i = 0; i < rank; ++i) { gdim[i] = dims[i]; box[i] = box_dims[i]; estr[i] = 1; }
     for (int i = 0; i + 1 < rank; ++i) gstride[i] = strides_bytes[i];
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(base), gdim, gstride, box,
-              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    auto encode = [&]() {
+        return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(base), gdim, gstride, box,
+                  estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    CUresult r = encode();
+    int dev = 0;
+    if (r == CUDA_ERROR_INVALID_CONTEXT && cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess)
+        r = encode();                    // (the thread's first call: the driver wants a context, which the runtime binds as late as it can)
+    return r == CUDA_SUCCESS;
 }
 
 // SM count of the current device (a benign race: every thread would store the same value).
