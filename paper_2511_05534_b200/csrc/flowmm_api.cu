@@ -89,6 +89,14 @@ void launch(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaS
         if (_s != FLOWMM_OK) return _s;          \
     } while (0)
 
+// Lets a kernel have all of a block's shared memory beside `static_bytes` of its own.  The same for every call: function attributes are the
+// device's, and a call's own size could be lowered by another thread's between here and the launch.
+constexpr int kBlockSmem = 227 * 1024;
+template <typename... Params>
+bool allow_smem(void (*kernel)(Params...), int static_bytes = 0) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kBlockSmem - static_bytes) == cudaSuccess;
+}
+
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // (unit, head) pairs per call: they index grid.x of several launches and 32-bit item counters
@@ -450,7 +458,7 @@ int score_clusters_at_once(int ctas) {
     attr.val.clusterDim.x = ctas; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(sct::kThreads); cfg.dynamicSmemBytes = sct::kMinSmem; cfg.attrs = &attr; cfg.numAttrs = 1;
-    if (cudaFuncSetAttribute(sct::score_cluster_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sct::kMinSmem) != cudaSuccess ||
+    if (!allow_smem(sct::score_cluster_tc_kernel) ||
         cudaOccupancyMaxActiveClusters(&n, sct::score_cluster_tc_kernel, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -495,7 +503,7 @@ flowmm_status run_score_cluster(const flowmm_params &p, const Layout &y, const v
     const uint32_t bq[4] = {64, (uint32_t)W, (uint32_t)q_heads, 1}, bk[4] = {64, sct::kTile, 1, 1};
     if (!tc::make_bf16_map(&qmap, q, 4, qd, qs, bq) || !tc::make_bf16_map(&kmap, k, 4, kd, ks, bk)) return FLOWMM_ERR_CUDA;
     const uint32_t smem = sct::smem_bytes(a.rt, kt);
-    if (cudaFuncSetAttribute(sct::score_cluster_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
+    if (!allow_smem(sct::score_cluster_tc_kernel)) return FLOWMM_ERR_CUDA;
     launch_cluster(dim3(ctas), sct::score_cluster_tc_kernel, UH * ctas, sct::kThreads, smem, st, qmap, kmap, a);
     FLOWMM_LAUNCHED("score_cluster_tc");
     return FLOWMM_OK;
@@ -594,8 +602,7 @@ MatchPrepArgs match_prep_args(const flowmm_params &p, const Layout &y, const voi
 template <int kThreads, bool kOneChunk, int kCtas = 1, bool kFew = false>
 flowmm_status launch_select(const SelectArgs &a, const SelectFlow &f, const MatchPrepArgs &g, int with_prepare, cudaStream_t st) {
     const size_t smem = select_smem(a.chunk);
-    if (cudaFuncSetAttribute(select_topb_kernel<kThreads, kOneChunk, kCtas, kFew>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return FLOWMM_ERR_CUDA;
+    if (!allow_smem(select_topb_kernel<kThreads, kOneChunk, kCtas, kFew>, 1024)) return FLOWMM_ERR_CUDA;
     launch_cluster(dim3(kCtas), select_topb_kernel<kThreads, kOneChunk, kCtas, kFew>, (a.n_heads + f.n_units) * kCtas, kThreads, smem, st, a, f, g, with_prepare);
     FLOWMM_LAUNCHED("select_topb");
     return FLOWMM_OK;
@@ -780,8 +787,7 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         a.n_items = a.per_item == 1 ? 2 * UH : UH;
         for (int i = 0; i < 3; ++i) { a.kos[i] = p.ko_stride[i]; a.vos[i] = p.vo_stride[i]; }
         const uint32_t smem = mtc::smem_bytes(p.n_keep, a.n_stages);
-        if (cudaFuncSetAttribute(mtc::merge_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return FLOWMM_ERR_CUDA;
+        if (!allow_smem(mtc::merge_tc_kernel)) return FLOWMM_ERR_CUDA;
         // ... and, while SMs are left, the steps of such an item on two or four (three steps each, or adding the parts up costs
         // what the split saves: 5 steps of 32 heads took 12 instead of 10 us; clusters of eight with this much shared memory start late)
         const int steps = (p.seq_len + mtc::kTile - 1) / mtc::kTile;
@@ -838,11 +844,11 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
         while (ctas > 1 && (ctas * UH > (ctas > 2 ? room : sms) || E < 1024 * ctas)) ctas >>= 1;
         const size_t csr_smem = csr_count_smem(E, p.n_keep, long_list ? 32 : 8);
         if (ctas > 1 && E < 65536 && smem <= 224 * 1024) {
-            if (cudaFuncSetAttribute(build_csr_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
+            if (!allow_smem(build_csr_cluster_kernel, 1024)) return FLOWMM_ERR_CUDA;
             launch_cluster(dim3(ctas), build_csr_cluster_kernel, UH * ctas, 32 * kCsrClusterWarps, smem, st, c, n_bits, ctas);
         } else if (E < 65536 && csr_smem <= 224 * 1024) {
             auto kernel = long_list ? build_csr_count_kernel<32> : build_csr_count_kernel<8>;
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csr_smem) != cudaSuccess) return FLOWMM_ERR_CUDA;
+            if (!allow_smem(kernel, 1024)) return FLOWMM_ERR_CUDA;
             launch(kernel, UH, long_list ? 1024 : 256, csr_smem, st, c, n_bits);
         } else if (!long_list) launch(build_csr_kernel<8>, UH, 256, 0, st, c);
         else launch(build_csr_kernel<32>, UH, 1024, 0, st, c);
@@ -901,8 +907,7 @@ flowmm_status run_match_merge(const flowmm_params &p, const Layout &y, const voi
     a.Hkv = p.n_kv_heads; a.L = p.seq_len; a.E = p.seq_len - p.n_keep; a.B = p.n_keep; a.Ctot = y.c_tot; a.merge_mode = p.merge_mode;
     a.n_items = UH; a.at = mmt::smem_plan(p.n_keep, y.c_tot);
     for (int i = 0; i < 3; ++i) { a.kos[i] = p.ko_stride[i]; a.vos[i] = p.vo_stride[i]; }
-    if (cudaFuncSetAttribute(mmt::match_merge_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)a.at.total) != cudaSuccess)
-        return FLOWMM_ERR_CUDA;
+    if (!allow_smem(mmt::match_merge_tc_kernel)) return FLOWMM_ERR_CUDA;
     launch(mmt::match_merge_tc_kernel, std::min(UH, tc::sm_count()), mmt::kThreads, a.at.total, st, kmap, vmap, cand_map, a);
     FLOWMM_LAUNCHED("match_merge_tc");
     return FLOWMM_OK;
