@@ -77,7 +77,9 @@ def test_small_fp32_workload_with_guards(debug_lib):
     C.compare(p, data["q"], data["k"], data["v"], data["modality"], g, bf16_out=False)
 
 
-@pytest.mark.parametrize("shape", [(2, 6, 2, 128, 333, 21, 37), (1, 4, 2, 128, 1031, 32, 300), (1, 8, 1, 128, 2600, 64, 500)])
+# (the second line: scoring by clusters, with one tile of proxy rows, with half of one, with four; matching and merge in one launch)
+@pytest.mark.parametrize("shape", [(2, 6, 2, 128, 333, 21, 37), (1, 4, 2, 128, 1031, 32, 300), (1, 8, 1, 128, 2600, 64, 500),
+                                   (1, 8, 2, 128, 333, 32, 37), (2, 4, 2, 128, 1031, 32, 40), (1, 8, 1, 128, 701, 64, 65), (20, 4, 4, 128, 203, 32, 33)])
 def test_ragged_bf16_cases_with_guards(debug_lib, shape):
     U, Hq, Hkv, D, L, W, B = shape
     rng = np.random.default_rng(L)

@@ -40,3 +40,31 @@ def test_one_launch_equals_the_steps(heads, L, B, kw, flow):
     assert torch.equal(k2[..., :128], k_out) and torch.equal(v2[..., :128], v_out)
     assert not k2[..., 128:].any() and not v2[..., 128:].any()
     assert F.flowmm_last_device_status(ws) == 0
+
+
+@pytest.mark.parametrize("U,Hkv,G,L,B", [(20, 4, 2, 300, 48), (40, 8, 1, 400, 33), (3, 32, 1, 700, 64)])
+def test_units_of_both_strategies_and_matches_alone(U, Hkv, G, L, B):
+    """Several units, whose modalities and strategies differ; of the matches' two tensors both, either or none asked for."""
+    W = 32
+    gen = torch.Generator(device="cuda").manual_seed(U * L)
+    draw = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    q, k, v = draw(U, Hkv * G, W, 128), draw(U, Hkv, L, 128), draw(U, Hkv, L, 128)
+    share = torch.linspace(0.05, 0.95, U, device="cuda")[:, None]
+    m = (torch.rand((U, L), generator=gen, device="cuda") < share).to(torch.uint8)
+    p = F.Params(U, Hkv * G, Hkv, 128, L, W, B, theta=0.4, tau=1.5, tau_mode=F.TAU_REL)
+    rho = F.compress_layer_alloc(p, q, k, v, m)["rho"]
+    p = F.Params(U, Hkv * G, Hkv, 128, L, W, B, theta=float(rho.sort().values[U // 2 - 1:U // 2 + 1].mean()), tau=1.5, tau_mode=F.TAU_REL)
+    full = F.compress_layer_alloc(p, q, k, v, m)
+    assert F.flowmm_last_device_status(full["ws"]) == 0 and 0 < int(full["strategy"].sum()) < U
+    match, sim = torch.full_like(full["match"], -9), torch.zeros_like(full["match_sim"])
+    ws = F.alloc_workspace(p)
+    F.flowmm_match(p, k, full["importance"], m, full["retained"], full["evicted"], full["strategy"], match, sim, ws)
+    k_out, v_out = torch.zeros_like(full["k_out"]), torch.zeros_like(full["v_out"])
+    F.flowmm_merge(p, k, v, full["retained"], full["evicted"], match, sim, k_out, v_out, ws)
+    assert torch.equal(match, full["match"]) and torch.equal(sim, full["match_sim"])
+    assert torch.equal(k_out, full["k_out"]) and torch.equal(v_out, full["v_out"])
+    for asked in ((), ("match",), ("match_sim",)):
+        out = {key: torch.full_like(full[key], -9) for key in ("k_out", "v_out") + asked}
+        F.flowmm_compress_layer(p, q, k, v, m, out["k_out"], out["v_out"], ws, **{key: out[key] for key in asked})
+        assert F.flowmm_last_device_status(ws) == 0
+        assert all(torch.equal(out[key], full[key]) for key in out)

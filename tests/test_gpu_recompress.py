@@ -102,6 +102,20 @@ def test_long_cache_on_the_general_tensor_core_kernels():
     _check(p, q2, k_cache, v_cache, rm, F.BF16)
 
 
+def test_many_heads_of_few_rows_in_one_launch():
+    # 80 heads, 48 rows kept of 300: matching and merge in one launch, with row modalities that differ between the heads of a unit and
+    # units of both strategies
+    rng = np.random.default_rng(91)
+    U, H, W, n = 20, 4, 32, 300
+    q2, k_cache, v_cache, rm = _grown_cache(rng, U, H, H, 128, 500, W, 240, 60, F.BF16)
+    for u in range(U):                                              # (shares of visual rows between 0.05 and 0.95, so that rho differs)
+        rm[u, :, :240] = rng.random((H, 240)) < 0.05 + 0.9 * u / (U - 1)
+    p = O.OracleParams(U, H, H, 128, n, W, 48, tau=3.0, tau_mode=O.TAU_REL)
+    p = dataclasses.replace(p, theta=float(np.median(O.recompress(p, q2, k_cache, v_cache, rm)["rho"])) + 1e-4)
+    g = _check(p, q2, k_cache, v_cache, rm, F.BF16)
+    assert 0 < (g["strategy"] == O.CROSS).sum() < U and not np.array_equal(rm[5, 0], rm[5, 1])
+
+
 def test_full_budget_returns_the_cache_with_its_appended_rows():
     rng = np.random.default_rng(5)
     q2, k_cache, v_cache, rm = _grown_cache(rng, 2, 4, 2, 128, 200, 8, 30, 10, F.BF16)
