@@ -14,8 +14,8 @@
 // A head with one range is normalised and written at once.  Two to eight ranges are a cluster: every CTA leaves its
 // unnormalised output, maximum and sum of weights in its shared memory, and after a cluster barrier the CTAs join a share
 // of the heads each.  With more ranges the CTA writes its record to global memory and decode_combine_kernel joins them, a
-// block per query head.  (One layer of 4 KV heads: 218 keys 12.4 us when the range that finished last joined all of them,
-// found by tickets that a memset had to clear first, 6.2 us as clusters of two.)
+// block per query head.  (One layer of 4 KV heads of 218 keys, as two ranges 12.4 us when the range that finished last
+// joined them, found by tickets that a memset had to clear first, 6.2 us as clusters of two, and as long as one range.)
 // Roles: warp 0 streams K tiles then V tiles through a three-stage TMA ring, warp 1 issues
 // the MMAs (both run whole and elect a thread at each instruction), warps 2-5 (one thread per key of a tile / per output dim) do the softmax and the output.
 // Two CTAs fit an SM (256 TMEM columns, about 109 KB of shared memory each), so one streams while the

@@ -876,6 +876,10 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
 }
 
 // Whether the matching and the merge of a call go into one launch (match_merge_tc.cuh): heads that fill the GPU, few slots (see there).
+// Up to a head per SM the line is half the SMs, whatever the length: K from memory twice costs the two launches as much as its heads' steps
+// in a row cost the one.  The whole call, us, by two and by one, 64 slots: 76 heads of 300 tokens 24.2, 22.1, of 1280 46.8, 44.4, of 2000 57.6,
+// 58.1, of 4000 89.7, 88.1, of 12 000 229, 212; 112 of 640 29.8, 27.2, of 2000 68.8, 66.0, of 12 000 309, 264; 144 of 4000 148, 130; but 72 of
+// 640 25.9, 25.4, of 2000 49.5, 55.8, of 4000 79.9, 85.3, of 12 000 213, 207, and 48 of 640 24.8, 24.6, of 4000 63.6, 76.7.
 // With several heads to an SM up to three steps a head are too few to hide its ends (1024 heads of 300 tokens 81.5 us by two launches, 82.9
 // by one; of 384 the same), and a second round of few heads leaves SMs without any, where the matching alone spreads tiles (160 heads of
 // 1200 tokens 85.0, 85.6; 256 of 640 42.9, 39.7).
@@ -1307,8 +1311,10 @@ DecodePlan decode_plan(const flowmm_decode_params &p, size_t ws_bytes) {
         // and V at the memory's rate, or the one CTA's, 0.9 a tile, where that is longer; when the CTAs do not fit at once, 1 per further
         // round, and part of what the last ones take with the memory mostly idle; for joining the ranges 2 as a cluster, 3 as a launch of
         // its own.  Clusters find room for 0.88 of the CTAs (96 of three, 12 tiles each, ran two after the other: 47 us, by five of 7 tiles
-        // 40).  Measured with every length on 18 shapes, 16 to 554 MB of 4 to 1024 heads: 1 % on average, 10 % at most above the best
-        // length (4 and 18 % by rounds of CTAs times their tiles and a fixed cost each).
+        // 40).  Measured with every length on the 18 shapes the constants are from, 16 to 554 MB of 4 to 1024 heads: 1 % on average, 10 % at
+        // most above the best length (4 and 18 % by rounds of CTAs times their tiles and a fixed cost each); on 31 others of 7 us and more, K
+        // and V from memory, 2 and 13 % (9 and 54 %); one head alone of 24 306 keys 45 % (48 %).  Where 80 MB stay in L2 from the call before,
+        // 56 heads of 2795 keys 12.2 us, 11.6 by rounds; from memory 16.4, 17.2.
         // (A smaller workspace than is asked for has room for fewer ranges.)
         const int tiles = (p.n_keys + dtc::kTile - 1) / dtc::kTile;
         const DecodeRecords records = decode_records(true, uh, p.n_keys);
