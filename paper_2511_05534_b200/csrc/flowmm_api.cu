@@ -135,23 +135,20 @@ int chunks_for(int L, int other_ctas, int &chunk) {
 // From kManyRows on warps draw their windows from a counter, else windows are taken with a stride.  The merge by windows of 32 with a
 // stride, and of 64 from the counter, us: 300 000 rows 44 to 53, 53 to 64; 0.8 million 83, 86; 1.0 million 109 to 123, 113 to 124;
 // 1.3 million 154, 156; 1.6 million 165, 164; 2.5 million 257, 248; 4.3 million 422, 392 (fp32 rows of 64 within 1 %, equal from 0.8 million on).
-// While every warp has one window or possible piece of a long slot at most, the windows are as short as leaves it so, by groups of four rows
-// (other lengths misalign the reads of the list: 64 heads of 1688 rows by 31 were 1.3 % slower).  The merge step, us, by windows of 32 and so:
-// 32 heads of 1500 with 300 slots 15.7, 14.1; 16 of 2500 with 250 15.9, 14.6; 12 of 4300 with 860 17.1, 16.0.  A warp with a window and a piece
-// sets the pace: with windows that leave the pieces out of account 32 of 2500 with 250 19.9 -> 23.7, 16 of 3500 with 350 18.7 -> 21.3, 32 of
-// 1500 with 300, 64 of them long, 19.5 -> 23.9 (and 12 of 6000 with 1200, none of them long, 19.8 -> 18.3); pieces by turns on the warps
-// without a window, up to four each, 32 of 2500 with 500, 97 of them long, 26.0 -> 31.9.  Windows shorter than two slots would often be empty: 4
-// heads of 10 822 rows with 542 slots by 16 instead of 32 81.8 -> 85.2 for the call.  Slots of up to one member on average are not expected to be
-// long: 112 caches of 640 rows with 423 slots by 28 79.3, by 24 78.3 for the call.  (Equal numbers of longer windows, 39 rows for 270 000,
-// 232 -> 243.)
+// While every warp has one window at most and warps are left for the pieces of long slots, one per 256 members (members seldom make more; the
+// first ones of all heads get them, merge_rows.cuh), the windows are as short as leaves it so, by groups of four rows (other lengths misalign the
+// reads of the list: 64 heads of 1688 rows by 31 were 1.3 % slower).  The merge step, us, by windows of 32, so, and with the pieces left out of
+// account, head by head behind the windows, so that a warp with a window and a piece set the pace: 32 heads of 2500 with 250 slots, one of
+// them long, 19.9, 19.3, 23.7; 16 of 3500 with 350 18.7, 19.2, 21.2; 24 of 4296 with 430 26.5, 21.5, 25.3; 32 of 1500 with 300, 64 of them long,
+// 19.5, 20.6, 23.8; none long 12 of 6000 with 1200 19.7, 18.3, 18.2.  Windows shorter than two slots would often be empty: 4 heads of 10 822
+// rows with 542 slots by 16 instead of 32 81.8 -> 85.2 for the call.  (Equal numbers of longer windows, 39 rows for 270 000, 232 -> 243.)
 constexpr int64_t kManyRows = 1300000;
 constexpr int kMinWin = 16, kMergeCtas = 3 * kScoreCtas;
-int max_parts(int E) { return 2 * (E / kPiece) + 2; }              // pieces of a head's long slots at most
 int merge_window(const flowmm_params &p) {
     const int64_t heads = (int64_t)p.n_units * p.n_kv_heads, rows = heads * p.seq_len;
     if (rows >= kManyRows) return mrow::kMaxWin;
     if (rows < 40000) return kMinWin;
-    const int E = p.seq_len - p.n_keep, parts = E > p.n_keep ? max_parts(E) : 0;
+    const int parts = (p.seq_len - p.n_keep) / 256;
     int win = kMinWin;
     while (win < 32 && (win * (int64_t)p.n_keep < 2 * (int64_t)p.seq_len || heads * ((p.seq_len + win - 1) / win + parts) > kMergeCtas * mrow::kWarps)) win += 4;
     return win;
@@ -161,7 +158,7 @@ int merge_window(const flowmm_params &p) {
 template <class Take>
 void layout_merge(Layout &y, const flowmm_params &p, Take take) {
     const size_t UH = (size_t)p.n_units * p.n_kv_heads, B = p.n_keep, L = p.seq_len, E = L - B, D = p.head_dim;
-    y.max_parts = max_parts((int)E);
+    y.max_parts = (int)(2 * (E / kPiece) + 2);
     y.csr_passes = 1;                                        // digits of kCsrBits bits over the keys 0 .. B
     while (y.csr_passes < 6 && (B >> (kCsrBits * y.csr_passes)) != 0) ++y.csr_passes;
     y.merge_win = merge_window(p);
@@ -870,7 +867,7 @@ flowmm_status run_merge(const flowmm_params &p, const Layout &y, const void *k, 
     const int64_t most = 3 * tc::sm_count(), apart = E > 0 && items + (int64_t)UH * y.max_parts <= 2 * mrow::kWarps * most ? (int64_t)UH * y.max_parts : 0;
     const int64_t blocks = (items + apart + mrow::kWarps - 1) / mrow::kWarps;
     launch(kernel, (int)(blocks < most ? blocks : most), mrow::kThreads, smem, st, m, (unsigned)items, (unsigned)apart, at<int>(ws, y.merge_status),
-           make_fastdiv((uint32_t)y.n_win), make_fastdiv((uint32_t)y.max_parts), make_fastdiv((uint32_t)p.n_kv_heads));
+           make_fastdiv((uint32_t)y.n_win), make_fastdiv((uint32_t)UH), make_fastdiv((uint32_t)p.n_kv_heads));
     FLOWMM_LAUNCHED("merge_rows");
     return FLOWMM_OK;
 }

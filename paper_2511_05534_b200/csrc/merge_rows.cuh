@@ -30,7 +30,7 @@ __host__ __device__ constexpr uint32_t warp_bytes(int bytes) { return kEntryByte
 
 // kBytes: of a K row (a V row) per lane.
 template <typename T, int kBytes>
-__global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs A, unsigned n_items, unsigned n_piece_items, int *status, const FastDiv by_win, const FastDiv by_parts, const FastDiv by_hkv) {
+__global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs A, unsigned n_items, unsigned n_piece_items, int *status, const FastDiv by_win, const FastDiv by_heads, const FastDiv by_hkv) {
     constexpr int V = kBytes / (int)sizeof(T), kWords = kBytes / 4, kGroup = group_rows(kBytes);
     constexpr uint32_t kRow = 32 * kBytes, kStage = kGroup * kRow;
     extern __shared__ __align__(128) uint8_t mrow_smem[];
@@ -40,13 +40,19 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
     const bool is_v = lane >= 16;
     const int c0 = (lane & 15) * V;
     const int64_t row_bytes = (is_v ? A.vs[2] : A.ks[2]) * (int64_t)sizeof(T);   // (two rows may be more than 4 GB apart)
-    const unsigned n_warps = gridDim.x * kWarps;
+    const unsigned n_warps = gridDim.x * kWarps, n_heads = n_piece_items / (unsigned)A.max_parts;
 
+    // (head, number) of a piece that is an item: all heads' first ones, then all heads' second ones, ...  Most possible pieces are none, and the
+    // ones that are find warps without a window so (merge_window() leaves some).
+    auto piece_of = [&](unsigned g) {
+        const unsigned p = by_heads.div(g - n_items);
+        return make_int2((int)(g - n_items - p * n_heads), (int)p);
+    };
     // what an item needs from global memory, a word of 32 rows per register
     struct Item { int2 count; int first, x[4], y[4]; };
     auto fetch = [&](unsigned g, Item &it) {
         if (g >= n_items) {
-            if (g - n_items < n_piece_items) it.count = A.row_count[by_parts.div(g - n_items)];
+            if (g - n_items < n_piece_items) it.count = A.row_count[piece_of(g).x];
             return;
         }
         const int uh = (int)by_win.div(g), w = (int)(g - (unsigned)uh * (unsigned)A.n_win);
@@ -180,8 +186,8 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
     for (; g < n_items + n_piece_items; g = g_next, g_next = __shfl_sync(0xFFFFFFFFu, g_after, 0)) {
         g_after = draw(g_next);
         const bool is_window = g < n_items;
-        const int uh = (int)(is_window ? by_win.div(g) : by_parts.div(g - n_items));
-        const int w = (int)(is_window ? g - (unsigned)uh * (unsigned)A.n_win : g - n_items - (unsigned)uh * (unsigned)A.max_parts);   // window, or piece
+        const int2 piece = is_window ? make_int2(0, 0) : piece_of(g);
+        const int uh = is_window ? (int)by_win.div(g) : piece.x, w = is_window ? (int)(g - (unsigned)uh * (unsigned)A.n_win) : piece.y;   // window, or piece
         const int u = (int)by_hkv.div(uh), h = uh - u * A.Hkv;
         const int left = is_window ? it.count.x - w * A.win : 0, n_pieces = is_window && n_piece_items != 0 ? 0 : it.count.y;   // left: rows from the window's first on
         int slot = it.first;
