@@ -639,8 +639,11 @@ flowmm_status run_select(const flowmm_params &p, const float *importance, int32_
         return launch_select<512, true, 4>(a, f, g, prep != nullptr, st);
     }
     // More heads than four blocks of 256 threads per SM would be in two rounds; of 128 threads an SM holds eight.  (1024 heads of 640
-    // positions 151.4 -> 149.5 us for the call, of 1000 222.7 -> 221.4; of 400, where a block's rounds are short, 110.4 -> 111.5.)
-    if (p.seq_len > 512 && p.seq_len <= 1024 && a.n_heads > 4 * tc::sm_count()) return launch_select<128, true, 1, true>(a, f, g, prep != nullptr, st);
+    // positions 151.4 -> 149.5 us for the call, of 1000 222.7 -> 221.4; of 400, where a block's rounds are short, 110.4 -> 111.5.)  Not beyond
+    // 64 query heads a unit, which its own block takes by warps, one chain of loads after the other: 864 heads of 600 positions with 64, 128 and
+    // 256 query heads a unit 142.1, 159.8, 205.2 us by 256 threads, 140.2, 162.4, 218.7 by 128.
+    if (p.seq_len > 512 && p.seq_len <= 1024 && a.n_heads > 4 * tc::sm_count() && (f.n_units == 0 || f.Hq <= 64))
+        return launch_select<128, true, 1, true>(a, f, g, prep != nullptr, st);
     // A block that has an SM for itself takes twice the warps: 32 heads of 640 positions 23.5 -> 23.0 us for the call, 4 of 3000 42.5 -> 41.7, 112
     // of 900 67.1 -> 65.4, of 2176 110.6 -> 109.5; of 4 heads of 192 17.9 -> 18.3, so from 257 positions on.
     const bool alone = a.n_heads + p.n_units <= tc::sm_count();
