@@ -623,10 +623,11 @@ flowmm_status run_select(const flowmm_params &p, const float *importance, int32_
     const SelectFlow no_flow = {};
     // Heads that leave SMs free, the short-list matching behind them (a block per SM; not the small blocks that gather long lists) and up to
     // five tiles of 128 tokens per SM for it.  The whole call, with and without: 32 heads of 640 tokens 23.1, 23.5 us; 16 of 2000 36.1, 36.4, with
-    // 7 query heads each 41.6, 42.4; but 4 of 400 23.3, 22.4; 72 of 1500 49.3, 45.9; 52 of 2500 54.4, 51.5; 40 of 3500 61.5, 58.6; with the
-    // matching and the merge in one launch 76 of 640 25.0, 23.6, of 2600 66.7, 62.8.
+    // 7 query heads each 41.6, 42.4; one of 206 16.4, 16.8; but 72 of 1500 49.3, 45.9; 52 of 2500 54.4, 51.5; 40 of 3500 61.5, 58.6; with the
+    // matching and the merge in one launch 76 of 640 25.0, 23.6, of 2600 66.7, 62.8.  (4 heads whose keys and queries are still in L2 from the call
+    // before: of 400 23.3, 22.4.)
     const int64_t tiles = (int64_t)a.n_heads * ((p.seq_len + mst::kTile - 1) / mst::kTile);
-    a.lets_in = prep && prep->copy_here && !use_match_merge(p) && a.n_heads >= 8 && 3 * (a.n_heads + p.n_units) <= 2 * tc::sm_count() &&
+    a.lets_in = prep && prep->copy_here && !use_match_merge(p) && 3 * (a.n_heads + p.n_units) <= 2 * tc::sm_count() &&
                 tiles <= 5 * tc::sm_count();
     MatchPrepArgs g = {};
     g.Hkv = 1; g.modality = row_mod;
