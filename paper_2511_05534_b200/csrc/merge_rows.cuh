@@ -40,13 +40,13 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
     const bool is_v = lane >= 16;
     const int c0 = (lane & 15) * V;
     const int64_t row_bytes = (is_v ? A.vs[2] : A.ks[2]) * (int64_t)sizeof(T);   // (two rows may be more than 4 GB apart)
-    const unsigned n_warps = gridDim.x * kWarps, n_heads = n_piece_items / (unsigned)A.max_parts;
+    const unsigned n_warps = gridDim.x * kWarps;
 
     // (head, number) of a piece that is an item: all heads' first ones, then all heads' second ones, ...  Most possible pieces are none, and the
     // ones that are find warps without a window so (merge_window() leaves some).
     auto piece_of = [&](unsigned g) {
         const unsigned p = by_heads.div(g - n_items);
-        return make_int2((int)(g - n_items - p * n_heads), (int)p);
+        return make_int2((int)(g - n_items - p * by_heads.d), (int)p);
     };
     // what an item needs from global memory, a word of 32 rows per register
     struct Item { int2 count; int first, x[4], y[4]; };
