@@ -666,7 +666,7 @@ flowmm_status run_match_tc(const flowmm_params &p, const Layout &y, const void *
     const MatchPrepArgs g = match_prep_args(p, y, k, importance, mod, retained, evicted, ws);
     if (!prepared) {                                 // (the fused call's selection launch has done it already)
         const int slices = (p.seq_len + kPrepSlice - 1) / kPrepSlice;
-        launch(match_prepare_kernel, dim3(UH, 1 + (slices < 64 ? slices : 64)), kPrepThreads, 0, st, g);
+        launch(p.n_keep <= kPrepThreads ? match_prepare_kernel<1> : match_prepare_kernel<8>, dim3(UH, 1 + (slices < 64 ? slices : 64)), kPrepThreads, 0, st, g);
         FLOWMM_LAUNCHED("match_prepare");
     }
     if (!g.copy_here) {

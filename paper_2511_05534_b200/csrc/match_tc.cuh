@@ -113,7 +113,7 @@ __device__ __forceinline__ void match_gather_rows(const MatchPrepArgs &A, int uh
 // has a thread for each, else eight: the steps one by one, 8 heads of 33 792 tokens with 1690 pivots, 235.8 -> 228.6 us, where rounds of a
 // pivot per thread loaded twice and summed each time; flowmm_match of 56 heads of 1200 tokens with 120 pivots by eight 14.2, by one 12.4.
 template <int kPer>
-__device__ __forceinline__ void match_number_candidates(const MatchPrepArgs &A, int uh, int *scratch) {
+__device__ __forceinline__ void match_lay_out_candidates(const MatchPrepArgs &A, int uh, int *scratch) {
     const int tid = threadIdx.x, u = uh / A.Hkv, chunk = kPer * blockDim.x;
     const int *ret = A.retained + (int64_t)uh * A.B;
     const float *imp = A.importance + (int64_t)uh * A.L;
@@ -173,13 +173,8 @@ __device__ __forceinline__ void match_number_candidates(const MatchPrepArgs &A, 
         seen_v += tot >> 16;
     }
     if (tid == 0) { A.cand_count[2 * uh] = seen_t; A.cand_count[2 * uh + 1] = seen_v; }
-}
-
-__device__ __forceinline__ void match_lay_out_candidates(const MatchPrepArgs &A, int uh, int *scratch) {
-    if (A.B <= (int)blockDim.x) match_number_candidates<1>(A, uh, scratch);
-    else match_number_candidates<8>(A, uh, scratch);
     __syncthreads();
-    if (A.copy_here) match_gather_rows<4>(A, uh, nullptr, 0, A.Ctot, threadIdx.x, blockDim.x);
+    if (A.copy_here) match_gather_rows<4>(A, uh, nullptr, 0, A.Ctot, tid, blockDim.x);
 }
 
 // The preparation of flowmm_match, which is handed the index lists (inside flowmm_compress_layer and flowmm_recompress the
@@ -188,11 +183,13 @@ __device__ __forceinline__ void match_lay_out_candidates(const MatchPrepArgs &A,
 constexpr int kPrepThreads = 512;
 constexpr int kPrepSlice = 8 * kPrepThreads;                   // list entries of such a block: eight loads in flight per thread
 static_assert(kPrepSlice % kMtItemRows == 0 && kPrepThreads % kMtItemRows == 0, "a slice is whole tiles, a step as well");
+// kPer: pivots of a thread that lays out candidates.
+template <int kPer>
 __global__ void __launch_bounds__(kPrepThreads) match_prepare_kernel(const MatchPrepArgs A) {
     __shared__ int scratch[33];
     predecessor_done();
     const int uh = blockIdx.x, tid = threadIdx.x;
-    if (blockIdx.y == 0) { match_lay_out_candidates(A, uh, scratch); return; }
+    if (blockIdx.y == 0) { match_lay_out_candidates<kPer>(A, uh, scratch); return; }
     const int part = blockIdx.y - 1, parts = gridDim.y - 1;
     const int *ret = A.retained + (int64_t)uh * A.B;
     const int *evi = A.evicted + (int64_t)uh * A.E;
