@@ -139,8 +139,8 @@ int chunks_for(int L, int other_ctas, int &chunk) {
 // first ones of all heads get them, merge_rows.cuh), the windows are as short as leaves it so, by groups of four rows (other lengths misalign the
 // reads of the list: 64 heads of 1688 rows by 31 were 1.3 % slower).  The merge step, us, by windows of 32, so, and with the pieces left out of
 // account, head by head behind the windows, so that a warp with a window and a piece set the pace: 32 heads of 2500 with 250 slots, one of
-// them long, 19.9, 19.3, 23.7; 16 of 3500 with 350 18.7, 19.2, 21.2; 24 of 4296 with 430 26.5, 21.5, 25.3; 32 of 1500 with 300, 64 of them long,
-// 19.5, 20.6, 23.8; none long 12 of 6000 with 1200 19.7, 18.3, 18.2.  Windows shorter than two slots would often be empty: 4 heads of 10 822
+// them long, 19.8, 19.5, 23.1; 16 of 3500 with 350 18.6, 19.0, 22.0; 24 of 4296 with 430 26.6, 21.5, 26.5; 32 of 1500 with 300, 64 of them long,
+// 19.5, 18.9, 23.6; none long 12 of 6000 with 1200 19.8, 18.3, 18.3.  Windows shorter than two slots would often be empty: 4 heads of 10 822
 // rows with 542 slots by 16 instead of 32 81.8 -> 85.2 for the call.  (Equal numbers of longer windows, 39 rows for 270 000, 232 -> 243.)
 constexpr int64_t kManyRows = 1300000;
 constexpr int kMinWin = 16, kMergeCtas = 3 * kScoreCtas;
