@@ -43,12 +43,10 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
     const unsigned n_warps = gridDim.x * kWarps;
 
     // (head, number) of a piece that is an item: all heads' first ones, then all heads' second ones, ...  Most possible pieces are none, and the
-    // ones that are find warps without a window so (merge_window() leaves some), of one block after the other: with eight of them on the
-    // warps of one block 32 heads of 1500 rows with 64 long slots 20.4 us, so 18.9; 12 of 4992 with 249 slots 18.6, 17.5.
-    const unsigned piece_blocks = (n_items < n_warps ? min(n_piece_items, n_warps - n_items) : 0u) / kWarps;
+    // ones that are find warps without a window so (merge_window() leaves some).
     auto piece_of = [&](unsigned g) {
-        const unsigned o = g - n_items, k = o < piece_blocks * kWarps ? o % kWarps * piece_blocks + o / kWarps : o, p = by_heads.div(k);
-        return make_int2((int)(k - p * by_heads.d), (int)p);
+        const unsigned p = by_heads.div(g - n_items);
+        return make_int2((int)(g - n_items - p * by_heads.d), (int)p);
     };
     // what an item needs from global memory, a word of 32 rows per register
     struct Item { int2 count; int first, x[4], y[4]; };
@@ -182,6 +180,12 @@ __global__ void __launch_bounds__(kThreads, 3) merge_rows_kernel(const MergeArgs
     // A warp's first window is given, the others are drawn from a shared counter, two ahead (or taken with a stride, without one).
     Item it;
     unsigned g = blockIdx.x * kWarps + warp, g_next, g_after;
+    // Pieces in a row go to the warps of one block after the other: with eight real ones on the warps of one block 32 heads of 1500 rows with
+    // 64 long slots took 20.4 us, so 18.9; 12 of 4992 with 249 slots 18.6, 17.5.
+    if (g >= n_items) {
+        const unsigned blocks = min(n_piece_items, n_warps - n_items) / kWarps, o = g - n_items;
+        if (o < blocks * kWarps) g = n_items + o % kWarps * blocks + o / kWarps;
+    }
     auto draw = [&](unsigned from) { return A.ticket ? (lane == 0 ? n_warps + atomicAdd(A.ticket, 1u) : 0u) : from + n_warps; };
     fetch(g, it);
     g_next = __shfl_sync(0xFFFFFFFFu, draw(g), 0);
